@@ -291,16 +291,15 @@ int spec_attention_static(const void *q, const void *k_pool, const void *v_pool,
  * product, only one dot product per step).  One call = the attention of one simulated step for one sequence:
  *   out[i][h] = softmax over { q[i][h].K0[p][g] : p <= i } U { q[i][h].Kd[s][i][g] : s < n_steps } (scale hd^-1/2) applied
  *   to the matching rows of V0 / Vd, with g = h / (n_heads / n_kv_heads).
- * q, out: bf16 [T rounded up to a multiple of 128][n_heads][128] (rows >= T are padding: read, never used; out rows >= T
- * are not written).  Pool positions T .. (T rounded up to 128) - 1 that fall in a mapped page are read with weight zero
+ * q, out: bf16 [T][n_heads][128].  Pool positions T .. (T rounded up to 128) - 1 that fall in a mapped page are read with weight zero
  * and must hold finite values.  K0 / V0 (the native step's keys and values, RoPE already applied): a paged pool
  * [num_pages][n_kv_heads][page_size][128] bf16 with page_table int32 [pages_per_seq] (position p lives in page
  * page_table[p / page_size]); page_size 16, 32 or 64.  k_diag / v_diag: bf16 [n_steps][T][n_kv_heads][128], the keys and
  * values each simulated step produced at every position (may be NULL when n_steps is 0: plain causal attention);
  * n_steps <= 8.  lse: optional float [T * n_heads], the natural-log normaliser of every row (what a backward pass needs).
- * scratch: spec_ttt_attention_scratch_bytes(...) bytes of device memory.  head_dim must be 128 (SPEC_ERR_UNSUPPORTED
- * otherwise).  The dense causal part runs on the tcgen05 tile kernel of the tree attention; the backward pass is not
- * part of this library. */
+ * scratch: spec_ttt_attention_scratch_bytes(...) bytes of device memory (not written any more).  head_dim must be 128
+ * (SPEC_ERR_UNSUPPORTED otherwise).  One launch of the causal tcgen05 kernel, which the prefill runs as well; the backward
+ * pass is not part of this library. */
 size_t spec_ttt_attention_scratch_bytes(int32_t T, int32_t n_heads, int32_t n_kv_heads, int32_t head_dim);
 int spec_ttt_attention(const void *q, const void *k_pool, const void *v_pool, const int32_t *page_table, int32_t pages_per_seq,
                        int32_t page_size, const void *k_diag, const void *v_diag, int32_t n_steps, void *out, float *lse,

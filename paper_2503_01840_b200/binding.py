@@ -399,19 +399,19 @@ def ttt_attention(q: torch.Tensor, k_pool: torch.Tensor, v_pool: torch.Tensor, p
     Returns out bf16 [T][H][128] (and the float32 [T][H] log-normaliser when want_lse)."""
     T, H, hd = q.shape
     G, ps = k_pool.shape[1], k_pool.shape[2]
-    rows = (T + 127) // 128 * 128
-    qp = torch.zeros(rows, H, hd, dtype=torch.bfloat16, device=q.device)
-    qp[:T] = q
-    out = torch.zeros_like(qp)
+    q = q.to(torch.bfloat16).contiguous()
+    if q.data_ptr() % 16:
+        q = q.clone()
+    out = torch.empty_like(q)
     J = 0 if k_diag is None else k_diag.shape[0]
     lse = torch.empty(T, H, dtype=torch.float32, device=q.device) if want_lse else None
     scratch = torch.empty(max(64, lib().spec_ttt_attention_scratch_bytes(T, H, G, hd)), dtype=torch.uint8, device=q.device)
-    rc = lib().spec_ttt_attention(qp.data_ptr(), k_pool.data_ptr(), v_pool.data_ptr(), page_table.data_ptr(), page_table.numel(), ps,
+    rc = lib().spec_ttt_attention(q.data_ptr(), k_pool.data_ptr(), v_pool.data_ptr(), page_table.data_ptr(), page_table.numel(), ps,
                                   k_diag.data_ptr() if J else None, v_diag.data_ptr() if J else None, J, out.data_ptr(),
                                   lse.data_ptr() if want_lse else None, T, H, G, hd, scratch.data_ptr(), _stream_ptr(None))
     if rc:
         raise SpecError(rc, "spec_ttt_attention")
-    return (out[:T], lse) if want_lse else out[:T]
+    return (out, lse) if want_lse else out
 
 
 def gemm_swiglu(x: torch.Tensor, w_gate: torch.Tensor, w_up: torch.Tensor) -> torch.Tensor:

@@ -1,0 +1,505 @@
+// Causal paged attention on the fifth-generation tensor cores, head_dim 128 (sm_100a): the prefill's attention and the
+// dense part of training-time-test attention.
+//
+// A query at position i attends keys 0..i of its sequence, read from the paged cache.  4 hd flops and one exponential per
+// (query, key, head): the tensor pipe (512 cycles for each of the two 128 x 128 x 128 contractions) and the special-function
+// unit (16 ex2 per cycle and SM: 1024 cycles per 128 x 128 scores) take the same time, so both have to run all the time:
+//
+//  * a CTA owns TWO query tiles of 128 positions that share every K and V tile: two heads of the same KV head (even
+//    groups, same positions, so both tiles have the same key range), or two consecutive blocks of positions (odd groups);
+//  * S = Q K^T of a tile goes to 128 columns of tensor memory; the tile's softmax warpgroup (thread = query row) reads it,
+//    writes P (bf16) over the first 64 of these columns, and O += P V takes P straight from tensor memory.  While one
+//    warpgroup is in its softmax the tensor pipe works for the other tile: P V of step j, then S of step j + 1;
+//  * the P V of step j is issued before the S of step j + 1, so seeing S complete also means that O is up to date: a row
+//    whose reference maximum moves (by more than 2^8, rare after the first steps) rescales its O without a further wait;
+//  * only the tiles that cross the diagonal are masked.
+//
+// Measured (one B200, T = 8192, 32 / 8 heads, 3 diagonal entries per row): 0.67 ms = 826 TFLOP/s of causal flops; with one
+// 128-row tile per CTA, P in shared memory, partial results through memory and a merge kernel: 1.27 ms.
+//
+// Every wait is bounded; a time-out is recorded in the status words and the CTA winds down.
+#include <math.h>
+#include <string.h>
+
+#include "../../include/spec_b200.h"
+#include "attn_causal.cuh"
+#include "tcgen05_ptx.cuh"
+#include "attn_fast.cuh"
+#include "attn_maps.cuh"
+
+namespace spec {
+
+namespace {
+
+using tc::elect_one;
+using tc::mbar_expect_tx;
+using tc::mbar_init;
+using tc::mbar_wait;
+using tc::mbar_wait_warp;
+using tc::smem_u32;
+
+constexpr int CA_HD = 128, CA_T = CAUSAL_TILE;
+constexpr int CA_TILE = CA_T * CA_HD * 2;          // 32 KB: a Q, K or V tile
+constexpr int CA_HALF = CA_T * 128;                // 16 KB: 64 of the 128 dimensions of a tile
+constexpr int CA_STAGES = 2;                       // K tiles and V tiles in flight (each)
+constexpr int CA_CTRL = 256;
+constexpr int CA_SMEM = (2 + 2 * CA_STAGES) * CA_TILE + CA_CTRL + 1024;
+// Two softmax warpgroups and one with the TMA warp and the MMA warp.  384 threads start with 168 registers each (64512 in
+// all); the softmax holds a row's 128 scores, so its 256 threads take 208 and the other 128 go down to 88 (64512 again).
+constexpr int CA_THREADS = 384, CA_REGS_SOFTMAX = 208, CA_REGS_ISSUE = 88;
+static_assert(256 * CA_REGS_SOFTMAX + 128 * CA_REGS_ISSUE <= CA_THREADS * 168, "register shares must fit what the block is launched with");
+constexpr int CA_MAX_DIAG = 8;
+
+struct CausalParams {
+  PageMap pm;
+  bf16 *out;
+  int H, G, T, J;
+  const CausalBlock *blocks;
+  const bf16 *kd, *vd;
+  float *lse;
+  int narrow;                      // out / kd / vd are only 8-byte aligned
+  int32_t *status;
+};
+
+__device__ __forceinline__ uint4 ld_row16(const bf16 *p, int narrow) {
+  if (!narrow) return *(const uint4 *)p;
+  const uint2 a = *(const uint2 *)p, b = *(const uint2 *)(p + 4);
+  return make_uint4(a.x, a.y, b.x, b.y);
+}
+__device__ __forceinline__ float ex2(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ uint32_t pack2(float lo, float hi) {
+  __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+  return *(uint32_t *)&v;
+}
+__device__ __forceinline__ void load_3d(void *dst, const CUtensorMap *map, int c0, int c1, int c2, uint64_t *bar) {
+  asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];" ::"r"(smem_u32(dst)),
+               "l"(map), "r"(smem_u32(bar)), "r"(c0), "r"(c1), "r"(c2)
+               : "memory");
+}
+// D += A B with A (128 x 16 bf16, two elements per column) in tensor memory
+__device__ __forceinline__ void umma_ts(uint32_t tmem_d, uint32_t tmem_a, uint64_t db, uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(tmem_d),
+      "r"(tmem_a), "l"(db), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+__device__ __forceinline__ uint64_t desc_mn(uint32_t saddr, uint32_t lbo) {      // MN-major operand, 128-byte swizzle
+  return (uint64_t)((saddr & 0x3FFFF) >> 4) | ((uint64_t)(lbo >> 4) << 16) | ((uint64_t)(1024 >> 4) << 32) | ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
+}
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float *f) {     // no wait
+  uint32_t *v = (uint32_t *)f;
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, "
+      "%19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]), "=r"(v[9]),
+        "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]), "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]),
+        "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]),
+        "=r"(v[30]), "=r"(v[31])
+      : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t *v) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, "
+      "%19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};" ::"r"(taddr),
+      "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(v[8]), "r"(v[9]), "r"(v[10]),
+      "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]), "r"(v[16]), "r"(v[17]), "r"(v[18]), "r"(v[19]), "r"(v[20]), "r"(v[21]),
+      "r"(v[22]), "r"(v[23]), "r"(v[24]), "r"(v[25]), "r"(v[26]), "r"(v[27]), "r"(v[28]), "r"(v[29]), "r"(v[30]), "r"(v[31])
+      : "memory");
+}
+__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ float2 bf2(uint32_t u) { return __bfloat1622float2(*(const __nv_bfloat162 *)&u); }
+
+// DIAG: the diagonal keys of training-time test are folded in (J may be 0) and the log-normaliser is written
+template <bool DIAG>
+__global__ void __launch_bounds__(CA_THREADS, 1) attn_causal_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
+                                                           const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CausalParams p) {
+  pdl_trigger();
+  pdl_wait();
+  extern __shared__ unsigned char smem_raw[];
+  unsigned char *sQ = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);   // two tiles [hd half][128 rows][128 B]
+  unsigned char *sK = sQ + 2 * CA_TILE, *sV = sK + CA_STAGES * CA_TILE;
+  uint64_t *kfull = (uint64_t *)(sV + CA_STAGES * CA_TILE), *kempty = kfull + CA_STAGES, *vfull = kempty + CA_STAGES, *vempty = vfull + CA_STAGES;
+  uint64_t *q_bar = vempty + CA_STAGES, *s_bar = q_bar + 1, *p_bar = s_bar + 2, *o_bar = p_bar + 2;     // the last three: one per tile
+  uint32_t *tmem_slot = (uint32_t *)(o_bar + 2);
+  volatile uint32_t *abort_flag = tmem_slot + 1;
+  volatile int *n_filled = (volatile int *)(tmem_slot + 2);     // [0] K tiles, [1] V tiles requested
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int grp = p.H / p.G;
+  const bool two_heads = (grp & 1) == 0;
+  int row0, nrows, seq, pos0;
+  if (p.blocks) {
+    const CausalBlock b = p.blocks[blockIdx.y];
+    row0 = b.row0; nrows = b.nrows; seq = b.seq; pos0 = b.pos0;
+  } else {                                          // one sequence of T rows; the longest key ranges first
+    const int br = two_heads ? CA_T : 2 * CA_T;
+    row0 = ((int)gridDim.y - 1 - (int)blockIdx.y) * br;
+    nrows = min(br, p.T - row0); seq = 0; pos0 = row0;
+  }
+  const int head0 = two_heads ? 2 * blockIdx.x : blockIdx.x;
+  const int g = head0 / grp;
+  // tile t of the CTA: rows, first position, key tiles
+  const int rows_0 = min(nrows, CA_T), rows_1 = two_heads ? rows_0 : max(0, nrows - CA_T);
+  const int off_1 = two_heads ? 0 : CA_T;
+  const int n0 = (pos0 + rows_0 + CA_T - 1) / CA_T, n1 = rows_1 > 0 ? (pos0 + off_1 + rows_1 + CA_T - 1) / CA_T : 0;
+  const int n = max(n0, n1);
+
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < CA_STAGES; i++) { mbar_init(&kfull[i], 1); mbar_init(&kempty[i], 1); mbar_init(&vfull[i], 1); mbar_init(&vempty[i], 1); }
+    mbar_init(q_bar, 1);
+    for (int i = 0; i < 2; i++) { mbar_init(&s_bar[i], 1); mbar_init(&p_bar[i], 128); mbar_init(&o_bar[i], 1); }
+    *abort_flag = 0;
+    n_filled[0] = n_filled[1] = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 9) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(512) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem_base = *tmem_slot;            // S / P of tile t at column 128 t, O at 256 + 128 t
+
+  if (warp >= 8) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(CA_REGS_ISSUE));
+    if (warp == 8) {
+      // ================================================================ TMA warp
+      const int ps = p.pm.page_size, ppt = CA_T / ps;          // pages per key tile: 8, 4 or 2
+      const int32_t *tbl = p.pm.table + (size_t)seq * p.pm.pages_per_seq;
+      const int fallback = tbl[0];                             // keys past the last page are masked; they still need a valid source
+      if (elect_one()) {
+        mbar_expect_tx(q_bar, 2 * CA_TILE);
+#pragma unroll
+        for (int t = 0; t < 2; t++)
+#pragma unroll
+          for (int h = 0; h < 2; h++)
+            load_3d(sQ + t * CA_TILE + h * CA_HALF, &map_q, 64 * h, two_heads ? head0 + t : head0, row0 + (two_heads ? 0 : t * CA_T), q_bar);
+      }
+      __syncwarp();
+      auto page_of = [&](int j) {                              // lane's page of key tile j
+        const int ip = j * ppt + lane;
+        int page = (lane < ppt && ip < p.pm.pages_per_seq) ? tbl[ip] : -1;
+        if (page < 0 || page >= p.pm.num_pages) page = fallback;
+        return (page * p.G + g) * ps;
+      };
+      int cur = page_of(0);
+      for (int j = 0; j < n; j++) {
+        const int nxt = j + 1 < n ? page_of(j + 1) : 0;
+        const int st = j % CA_STAGES;
+        const uint32_t ph = (uint32_t)((j / CA_STAGES) & 1);
+        int row[8];
+#pragma unroll
+        for (int i = 0; i < 8; i++) row[i] = __shfl_sync(0xffffffffu, cur, i);
+#pragma unroll
+        for (int kv = 0; kv < 2; kv++) {
+          uint64_t *fb = kv ? &vfull[st] : &kfull[st], *eb = kv ? &vempty[st] : &kempty[st];
+          if (!mbar_wait_warp(eb, ph ^ 1u)) { *abort_flag = 1; if (p.status) set_status(p.status, ST_TIMEOUT, 430 + kv, blockIdx.y, j); break; }
+          if (elect_one()) {
+            unsigned char *d = (kv ? sV : sK) + st * CA_TILE;
+            mbar_expect_tx(fb, CA_TILE);
+#pragma unroll
+            for (int i = 0; i < 8; i++) {
+              if (i >= ppt) break;
+#pragma unroll
+              for (int h = 0; h < 2; h++) load_3d(d + h * CA_HALF + i * ps * 128, kv ? &map_v : &map_k, 0, row[i], h, fb);
+            }
+            n_filled[kv] = j + 1;
+          }
+          __syncwarp();
+        }
+        if (*abort_flag) break;
+        cur = nxt;
+      }
+    } else if (warp == 9) {
+      // ================================================================ MMA warp
+      constexpr uint32_t idesc_s = tc::umma_idesc(CA_T);                    // both operands K-major, N = 128 keys
+      constexpr uint32_t idesc_o = tc::umma_idesc(CA_HD) | (1u << 16);      // B (the V tile) MN-major, N = 128 dimensions
+      const uint64_t dq = tc::umma_desc_sw128(smem_u32(sQ)), dk = tc::umma_desc_sw128(smem_u32(sK));
+      const uint64_t dv = desc_mn(smem_u32(sV), CA_HALF);
+      auto issue_s = [&](int t, int st) {
+#pragma unroll
+        for (int kk = 0; kk < 8; kk++) {
+          const uint64_t o = (uint64_t)(((kk >> 2) * CA_HALF + (kk & 3) * 32) >> 4);
+          tc::umma_bf16(tmem_base + t * 128, dq + (uint64_t)((t * CA_TILE) >> 4) + o, dk + (uint64_t)((st * CA_TILE) >> 4) + o, idesc_s, kk ? 1u : 0u);
+        }
+        tc::umma_commit(&s_bar[t]);
+      };
+      bool ok = mbar_wait_warp(q_bar, 0) && mbar_wait_warp(&kfull[0], 0);
+      if (!ok) { *abort_flag = 1; if (p.status) set_status(p.status, ST_TIMEOUT, 432, blockIdx.y, 0); }
+      if (ok) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        if (elect_one()) {
+          issue_s(0, 0);
+          if (n1 > 0) issue_s(1, 0);
+          tc::umma_commit(&kempty[0]);
+        }
+        __syncwarp();
+        for (int j = 0; j < n && ok; j++) {
+          const int st = j % CA_STAGES, st1 = (j + 1) % CA_STAGES;
+          bool have_v = false, have_k = false;
+#pragma unroll
+          for (int t = 0; t < 2; t++) {
+            const int nt = t ? n1 : n0;
+            if (j >= nt) continue;
+            ok = mbar_wait_warp(&p_bar[t], (uint32_t)(j & 1));
+            if (ok && !have_v) { ok = mbar_wait_warp(&vfull[st], (uint32_t)((j / CA_STAGES) & 1)); have_v = true; }
+            if (!ok || *abort_flag) { ok = false; *abort_flag = 1; if (p.status) set_status(p.status, ST_TIMEOUT, 433, blockIdx.y, j); break; }
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            if (elect_one()) {
+#pragma unroll
+              for (int kk = 0; kk < 8; kk++)         // 16 keys: 8 columns of P, 16 rows of V
+                umma_ts(tmem_base + 256 + t * 128, tmem_base + t * 128 + kk * 8, dv + (uint64_t)((st * CA_TILE + kk * 16 * 128) >> 4), idesc_o, (j | kk) ? 1u : 0u);
+              if (j + 1 == nt) tc::umma_commit(&o_bar[t]);
+            }
+            __syncwarp();
+            if (j + 1 < nt) {
+              if (!have_k) { ok = mbar_wait_warp(&kfull[st1], (uint32_t)(((j + 1) / CA_STAGES) & 1)); have_k = true; }
+              if (!ok) { *abort_flag = 1; if (p.status) set_status(p.status, ST_TIMEOUT, 434, blockIdx.y, j); break; }
+              asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+              if (elect_one()) issue_s(t, st1);
+              __syncwarp();
+            }
+          }
+          if (!ok) break;
+          if (elect_one()) {
+            tc::umma_commit(&vempty[st]);
+            if (j + 1 < n) tc::umma_commit(&kempty[st1]);
+          }
+          __syncwarp();
+        }
+      }
+    }
+  } else {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(CA_REGS_SOFTMAX));
+    // ================================================================ softmax: thread = query row = tensor-memory lane
+    const int t = warp >> 2, lr = threadIdx.x & 127;
+    const int nt = t ? n1 : n0, nr = t ? rows_1 : rows_0;
+    const int head = two_heads ? head0 + t : head0;
+    const int trow = row0 + (t ? off_1 : 0), pos = pos0 + (t ? off_1 : 0) + lr;      // first row of the tile, this thread's position
+    const uint32_t lanes = (uint32_t)((warp & 3) * 32) << 16;
+    const uint32_t my_s = tmem_base + lanes + (uint32_t)(t * 128), my_o = tmem_base + lanes + 256u + (uint32_t)(t * 128);
+    const float sc = rsqrtf((float)CA_HD) * 1.4426950408889634f;                     // softmax scale folded into exp2
+    float mx = -INFINITY, l = 0.0f;
+    bool alive = true;
+    for (int j = 0; j < nt; j++) {
+      bool ok = mbar_wait_warp(&s_bar[t], (uint32_t)(j & 1));
+      if (!ok || *abort_flag) { if (lane == 0) { *abort_flag = 1; if (p.status) set_status(p.status, ST_TIMEOUT, 435, blockIdx.y, j); } alive = false; break; }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      float s[CA_T];
+#pragma unroll
+      for (int c = 0; c < 4; c++) tmem_ld32(my_s + c * 32, s + c * 32);
+      tmem_ld_wait();
+      const int k0 = j * CA_T;
+      if (k0 + CA_T - 1 > pos - (int)(threadIdx.x & 31)) {       // uniform over the warp: its first row does not see the whole tile
+        const int lim = pos - k0;                                // keys 0..lim of the tile
+#pragma unroll
+        for (int e = 0; e < CA_T; e++) s[e] = e <= lim ? s[e] : -INFINITY;
+      }
+      float m4[4] = {s[0], s[1], s[2], s[3]};
+#pragma unroll
+      for (int e = 4; e < CA_T; e += 4) {
+#pragma unroll
+        for (int z = 0; z < 4; z++) m4[z] = fmaxf(m4[z], s[e + z]);
+      }
+      const float tm = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
+      // the reference maximum moves only when the tile's exceeds it by more than 2^8 in the exponent
+      float f = 1.0f;
+      if (tm > mx && (mx == -INFINITY || (tm - mx) * sc > 8.0f)) {
+        f = (mx == -INFINITY) ? 1.0f : ex2((mx - tm) * sc);
+        mx = tm;
+      }
+      if (j > 0 && __any_sync(0xffffffffu, f != 1.0f)) {         // S of this step is complete, hence the P V of the last one
+#pragma unroll 1
+        for (int c = 0; c < 4; c++) {
+          float o[32];
+          tmem_ld32(my_o + c * 32, o);
+          tmem_ld_wait();
+#pragma unroll
+          for (int e = 0; e < 32; e++) o[e] *= f;
+          tmem_st32(my_o + c * 32, (uint32_t *)o);
+        }
+      }
+      const float nb = (mx == -INFINITY) ? 0.0f : mx * sc;
+      float rs[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+      for (int c = 0; c < 2; c++) {
+        uint32_t pk[32];
+#pragma unroll
+        for (int e = 0; e < 32; e++) {
+          const float p0 = ex2(fmaf(s[c * 64 + 2 * e], sc, -nb)), p1 = ex2(fmaf(s[c * 64 + 2 * e + 1], sc, -nb));
+          rs[(2 * e) & 3] += p0; rs[(2 * e + 1) & 3] += p1;
+          pk[e] = pack2(p0, p1);
+        }
+        tmem_st32(my_s + c * 32, pk);
+      }
+      l = l * f + ((rs[0] + rs[1]) + (rs[2] + rs[3]));
+      tmem_st_wait();
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&p_bar[t])) : "memory");
+    }
+    if (alive && nt > 0) {
+      bool ok = mbar_wait_warp(&o_bar[t], 0);
+      if (!ok || *abort_flag) { if (lane == 0) { *abort_flag = 1; if (p.status) set_status(p.status, ST_TIMEOUT, 436, blockIdx.y, nt); } alive = false; }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    }
+    if (alive && nt > 0) {
+      unsigned char *qt = sQ + t * CA_TILE;                      // this row's 16-byte chunk c: half c / 8, row lr, chunk (c % 8) ^ (lr % 8)
+      auto chunk = [&](int r, int c) { return (uint4 *)(qt + (c >> 3) * CA_HALF + r * 128 + (((c & 7) ^ (r & 7)) << 4)); };
+      const bool rv = lr < nr;
+      float fo = 1.0f, wd[CA_MAX_DIAG];
+      size_t doff = 0;
+      if (DIAG) {
+        doff = ((size_t)(rv ? trow + lr : 0) * p.G + g) * CA_HD;
+        const size_t dstep = (size_t)p.T * p.G * CA_HD;
+        float d[CA_MAX_DIAG];
+#pragma unroll
+        for (int s = 0; s < CA_MAX_DIAG; s++) d[s] = 0.0f;
+        if (p.J > 0) {
+#pragma unroll 2
+          for (int c = 0; c < 16; c++) {
+            const uint4 qv = *chunk(lr, c);
+            const float2 q0 = bf2(qv.x), q1 = bf2(qv.y), q2 = bf2(qv.z), q3 = bf2(qv.w);
+#pragma unroll
+            for (int s = 0; s < CA_MAX_DIAG; s++)
+              if (s < p.J) {
+                const uint4 kv = ld_row16(p.kd + s * dstep + doff + c * 8, p.narrow);
+                const float2 k0 = bf2(kv.x), k1 = bf2(kv.y), k2 = bf2(kv.z), k3 = bf2(kv.w);
+                d[s] += ((q0.x * k0.x + q0.y * k0.y) + (q1.x * k1.x + q1.y * k1.y)) + ((q2.x * k2.x + q2.y * k2.y) + (q3.x * k3.x + q3.y * k3.y));
+              }
+          }
+        }
+        float M = mx;
+#pragma unroll
+        for (int s = 0; s < CA_MAX_DIAG; s++)
+          if (s < p.J) M = fmaxf(M, d[s]);
+        fo = ex2((mx - M) * sc);
+        l *= fo;
+#pragma unroll
+        for (int s = 0; s < CA_MAX_DIAG; s++) {
+          wd[s] = s < p.J ? exp2f((d[s] - M) * sc) : 0.0f;
+          l += wd[s];
+        }
+        if (p.lse && rv) p.lse[(size_t)(trow + lr) * p.H + head] = logf(l) + M * rsqrtf((float)CA_HD);
+      }
+      const float inv = l > 0.0f ? 1.0f / l : 0.0f;
+      __syncwarp();                                              // every lane has read its q row: the tile becomes the output staging
+#pragma unroll 1
+      for (int c = 0; c < 4; c++) {
+        float o[32];
+        tmem_ld32(my_o + c * 32, o);
+        tmem_ld_wait();
+        if (DIAG) {
+          const size_t dstep = (size_t)p.T * p.G * CA_HD;
+#pragma unroll
+          for (int e = 0; e < 32; e++) o[e] *= fo;
+#pragma unroll
+          for (int s = 0; s < CA_MAX_DIAG; s++)
+            if (s < p.J) {
+#pragma unroll
+              for (int u = 0; u < 4; u++) {
+                const uint4 vv = ld_row16(p.vd + s * dstep + doff + c * 32 + u * 8, p.narrow);
+                const float2 v0 = bf2(vv.x), v1 = bf2(vv.y), v2 = bf2(vv.z), v3 = bf2(vv.w);
+                o[u * 8 + 0] += wd[s] * v0.x; o[u * 8 + 1] += wd[s] * v0.y; o[u * 8 + 2] += wd[s] * v1.x; o[u * 8 + 3] += wd[s] * v1.y;
+                o[u * 8 + 4] += wd[s] * v2.x; o[u * 8 + 5] += wd[s] * v2.y; o[u * 8 + 6] += wd[s] * v3.x; o[u * 8 + 7] += wd[s] * v3.y;
+              }
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; u++)
+          *chunk(lr, c * 4 + u) = make_uint4(pack2(o[u * 8] * inv, o[u * 8 + 1] * inv), pack2(o[u * 8 + 2] * inv, o[u * 8 + 3] * inv),
+                                             pack2(o[u * 8 + 4] * inv, o[u * 8 + 5] * inv), pack2(o[u * 8 + 6] * inv, o[u * 8 + 7] * inv));
+      }
+      __syncwarp();
+      // a warp's 32 rows, two whole rows (256 bytes each) per instruction
+      const int rw = (warp & 3) * 32;
+#pragma unroll 4
+      for (int i = 0; i < 16; i++) {
+        const int r = rw + 2 * i + (lane >> 4), c = lane & 15;
+        if (r < nr) {
+          bf16 *dst = p.out + ((size_t)(trow + r) * p.H + head) * CA_HD + c * 8;
+          const uint4 v = *chunk(r, c);
+          if (DIAG && p.narrow) { *(uint2 *)dst = make_uint2(v.x, v.y); *(uint2 *)(dst + 4) = make_uint2(v.z, v.w); }
+          else *(uint4 *)dst = v;
+        }
+      }
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (*abort_flag && threadIdx.x == 0) {            // no copy may still be landing when the CTA exits
+    mbar_wait(q_bar, 0);
+    for (int kv = 0; kv < 2; kv++)
+      for (int j = max(0, n_filled[kv] - CA_STAGES); j < n_filled[kv]; j++) mbar_wait(kv ? &vfull[j % CA_STAGES] : &kfull[j % CA_STAGES], (uint32_t)((j / CA_STAGES) & 1));
+  }
+  if (warp == 9) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512) : "memory");
+}
+
+}  // namespace
+
+bool causal_attn_supported(int head_dim, int page_size) { return head_dim == CA_HD && (page_size == 16 || page_size == 32 || page_size == 64); }
+
+int launch_causal_attn(const CausalArgs &a, cudaStream_t s) {
+  if (a.J > CA_MAX_DIAG || a.H % a.G) return -1;
+  const int grp = a.H / a.G;
+  const CUtensorMap *mk = kv_map(a.pool.k, a.pm.num_pages, a.G, a.pm.page_size, CA_HD, 1), *mv = kv_map(a.pool.v, a.pm.num_pages, a.G, a.pm.page_size, CA_HD, 1);
+  CUtensorMap mq;
+  if (!mk || !mv || !q_map(&mq, a.q, a.q_rows, a.H, CA_T)) return -6;
+  CausalParams p;
+  memset(&p, 0, sizeof p);
+  p.pm = a.pm; p.out = a.out; p.H = a.H; p.G = a.G; p.T = a.T; p.J = a.J; p.blocks = a.blocks; p.kd = a.kd; p.vd = a.vd; p.lse = a.lse;
+  p.narrow = (((uintptr_t)a.out | (uintptr_t)a.kd | (uintptr_t)a.vd) & 15) ? 1 : 0;
+  p.status = a.status;
+  const int br = causal_block_rows(grp);
+  dim3 grid(grp % 2 == 0 ? a.H / 2 : a.H, a.blocks ? a.n_blocks : (a.T + br - 1) / br);
+  static SmemLimit limit[2];
+  const bool diag = !a.blocks;
+  if (diag) {
+    if (!limit[1].ensure(attn_causal_kernel<true>, CA_SMEM)) return -6;
+    launch_k(attn_causal_kernel<true>, grid, dim3(CA_THREADS), (size_t)CA_SMEM, s, mq, *mk, *mv, p);
+  } else {
+    if (!limit[0].ensure(attn_causal_kernel<false>, CA_SMEM)) return -6;
+    launch_k(attn_causal_kernel<false>, grid, dim3(CA_THREADS), (size_t)CA_SMEM, s, mq, *mk, *mv, p);
+  }
+  return 0;
+}
+
+}  // namespace spec
+
+// ------------------------------------------------------------------------------------------------
+// Training-time-test attention (Section 3.2, the figure of the attention masks during training-time test).
+//
+// While the draft model is trained, its own outputs are fed back for further simulated steps.  At simulated step j a
+// query at slot i sees the ORIGINAL sequence causally (keys 0..i of the native step: an ordinary lower-triangular mask)
+// and, of every earlier simulated step s = 1..j, only the entry at its own slot i (a diagonal mask).  The diagonal part is
+// j dot products per (slot, head): the causal kernel computes them as such after the key loop, when the row's statistics
+// and its O are at hand, and folds them into the same softmax.  Nothing passes through global memory in between, so the
+// call needs no scratch; the parameter stays in the interface.
+extern "C" size_t spec_ttt_attention_scratch_bytes(int32_t T, int32_t n_heads, int32_t n_kv_heads, int32_t head_dim) {
+  if (T < 1 || n_heads < 1 || n_kv_heads < 1 || n_heads % n_kv_heads || head_dim != 128) return 0;
+  return 256;
+}
+
+extern "C" int spec_ttt_attention(const void *q, const void *k_pool, const void *v_pool, const int32_t *page_table,
+                                  int32_t pages_per_seq, int32_t page_size, const void *k_diag, const void *v_diag, int32_t n_steps,
+                                  void *out, float *lse, int32_t T, int32_t H, int32_t G, int32_t hd, void *scratch, void *stream) {
+  using namespace spec;
+  if (!q || !k_pool || !v_pool || !page_table || !out || !scratch || (n_steps > 0 && (!k_diag || !v_diag))) return SPEC_ERR_NULL;
+  if (T < 1 || H < 1 || G < 1 || H % G || n_steps < 0 || n_steps > CA_MAX_DIAG) return SPEC_ERR_INVALID_CFG;
+  if (!causal_attn_supported(hd, page_size) || (long long)pages_per_seq * page_size < T) return SPEC_ERR_UNSUPPORTED;
+  CausalArgs a;
+  a.q = (const bf16 *)q; a.q_rows = T;
+  a.pool = KvPool{(void *)k_pool, (void *)v_pool};
+  a.pm = PageMap{page_table, pages_per_seq, page_size, 1 << 20};
+  a.out = (bf16 *)out; a.H = H; a.G = G; a.T = T;
+  a.kd = n_steps ? (const bf16 *)k_diag : nullptr; a.vd = n_steps ? (const bf16 *)v_diag : nullptr; a.J = n_steps; a.lse = lse;
+  if (launch_causal_attn(a, (cudaStream_t)stream)) return SPEC_ERR_CUDA;
+  attn_fast_forget_maps();
+  return cudaGetLastError() == cudaSuccess ? SPEC_OK : SPEC_ERR_CUDA;
+}

@@ -43,7 +43,7 @@ def main():
     ms = e0.elapsed_time(e1) / a.iters
     flops = 4.0 * hd * H * T * (T + 1) / 2
     line = {"op": "ttt_attention", "T": T, "heads": H, "kv_heads": G, "simulated_steps": J, "ms": round(ms, 4),
-            "tflops": round(flops / ms / 1e9, 2), "note": "includes the binding's padding copies and the merge kernel"}
+            "tflops": round(flops / ms / 1e9, 2), "note": "through the binding"}
     if a.peak_tflops > 0:
         line["frac_of_measured_bf16_peak"] = round(flops / ms / 1e9 / a.peak_tflops, 4)
     print(json.dumps(line))
