@@ -12,7 +12,9 @@
 #include "../../include/spec_b200.h"
 #include "tma_maps.cuh"
 #include "gemm_fused.cuh"
+#include "gemm_wide.cuh"
 #include "attn_fast.cuh"
+#include "attn_causal.cuh"
 #include "state.cuh"
 
 using namespace spec;
@@ -103,6 +105,8 @@ struct spec_ctx {
   int dbg_withhold_spin = 0;    // test hook: > 0 makes one CTA of the verify LM-head GEMM run a bounded wait out after that many polls
   void *attn_scratch;
   size_t attn_scratch_bytes;
+  char *wide_base;             // the step's own buffers, free during a prefill (see WideBufs)
+  size_t wide_bytes;
   // partial-sum bookkeeping of the plain (fp32 / debug) schedule: its GEMMs write one slice
   int np_proj = 1, np_qkv = 1, np_gu = 1;
   size_t ps_proj = 0, ps_qkv = 0, ps_gu = 0;
@@ -189,9 +193,7 @@ static size_t carve(spec_ctx *c, void *base) {
   Carver cv(base);
   c->x = cv.take<float>((size_t)R * k);
   c->proj = cv.take<float>((size_t)R * k);
-  c->qkv = cv.take<float>((size_t)R * qkvd);
-  c->gu = cv.take<float>((size_t)R * 2 * c->F);
-  c->logits = cv.take<float>((size_t)R * std::max(c->V, c->Vd));
+  if (g.flags & SPEC_FLAG_CAPTURE) c->logits = cv.take<float>((size_t)R * std::max(c->V, c->Vd));
   c->h = cv.take_bytes((size_t)R * k * e);
   c->q = cv.take_bytes((size_t)R * qd * e);
   c->ao = cv.take_bytes((size_t)R * qd * e);
@@ -244,6 +246,7 @@ static size_t carve(spec_ctx *c, void *base) {
   c->ssq = cv.take<float>((size_t)c->ktiles * R);
   c->best_val = cv.take<float>((size_t)c->vtiles * R);
   c->best_idx = cv.take<int32_t>((size_t)c->vtiles * R);
+  c->stamps = (g.flags & SPEC_FLAG_STAMPS) ? cv.take<unsigned long long>((size_t)MAX_STAMPS * 2) : nullptr;
   c->topk_scratch = cv.take_bytes(topk_scratch_bytes(R, c->Vd, c->K));
   c->dtiles = (c->Vd + 127) / 128;
   const size_t cld = (size_t)draft_tree_cand_ld(c->dtiles);
@@ -251,9 +254,16 @@ static size_t carve(spec_ctx *c, void *base) {
   c->cand_idx = cv.take<int32_t>(cld * R * c->K);
   c->cand_max = cv.take<float>(cld * R);
   c->cand_sum = cv.take<float>(cld * R);
-  c->stamps = (g.flags & SPEC_FLAG_STAMPS) ? cv.take<unsigned long long>((size_t)MAX_STAMPS * 2) : nullptr;
+  // What only a step (or only the fp32 schedule) uses, in one run: the packed prefill lays its wide passes over it.
+  // (No buffer of indices is among them: a step that gave up on a wait may leave one unwritten and read it.)
+  const size_t wide0 = (cv.off + 255) & ~(size_t)255;
+  c->qkv = cv.take<float>((size_t)R * qkvd);
+  c->gu = cv.take<float>((size_t)R * 2 * c->F);
+  if (!(g.flags & SPEC_FLAG_CAPTURE)) c->logits = cv.take<float>((size_t)R * std::max(c->V, c->Vd));
   c->attn_scratch_bytes = attn_fast_scratch_bytes(R, c->H, c->hd, g.max_ctx);
   c->attn_scratch = cv.take_bytes(c->attn_scratch_bytes);
+  c->wide_base = base ? (char *)base + wide0 : nullptr;
+  c->wide_bytes = cv.off - wide0;
   return (cv.off + 255) & ~(size_t)255;
 }
 
@@ -350,6 +360,36 @@ extern "C" int spec_free(spec_ctx *c) {
   return SPEC_OK;
 }
 
+// Buffers of the packed prefill's passes, laid over the step's own (spec_ctx::wide_base): a workspace of the size the
+// steps need anyway holds passes of about 3000 rows of the 8B shapes.
+struct WideBufs {
+  int cap = 0;                 // rows
+  float *x, *ssq;
+  bf16 *h, *q, *ao, *act, *cat, *taps;
+  float2 *cs;
+  PackMeta m;
+  CausalBlock *blocks;         // of all passes
+  int2 *fin;                   // {row of its pass, sequence} of every prompt's last position
+};
+static size_t wide_carve(const spec_ctx *c, WideBufs &w, void *base, int rows, size_t n_blocks, size_t n_fin) {
+  Carver cv(base);
+  const size_t R = rows, k = c->k, qd = (size_t)c->H * c->hd;
+  w.cap = rows;
+  w.x = cv.take<float>(R * k);
+  w.ssq = cv.take<float>(R * c->ktiles);
+  w.h = cv.take<bf16>(R * k);
+  w.q = cv.take<bf16>(R * qd);
+  w.ao = cv.take<bf16>(R * qd);
+  w.act = cv.take<bf16>(R * std::max((size_t)c->F, 2 * k));
+  w.cat = w.act;               // the FC2 input is built when the last layer's activations are done with
+  w.taps = cv.take<bf16>(R * 3 * k);
+  w.cs = cv.take<float2>(R * (c->hd / 2));
+  for (int32_t **p : {&w.m.seq, &w.m.seq_d, &w.m.pos, &w.m.tok, &w.m.tok_next, &w.m.slot, &w.m.slot_d}) *p = cv.take<int32_t>(R);
+  w.blocks = cv.take<CausalBlock>(n_blocks);
+  w.fin = cv.take<int2>(n_fin);
+  return cv.off;
+}
+
 // ------------------------------------------------------------------------------------------ schedule
 template <typename T> struct Sched {
   spec_ctx *c;
@@ -443,16 +483,18 @@ template <typename T> struct Sched {
     tick();
     for (int l = 0; l < c->L; l++)
       block_fused(c->tl[l], c->pools[l], rows, tail_len, l + 1 < c->L ? c->tl[l + 1].attn_norm : c->final_norm, tap_mask_of(l));
-    if (want_logits) {
-      FusedGemmArgs a = fargs(c->h, rows, c->k);
-      a.w[0] = (const bf16 *)c->lm_head; a.O[0] = c->V; a.nw = 1;
-      with_norm_scale(a);
-      a.best_val = c->best_val; a.best_idx = c->best_idx; a.best_ld = c->Ralloc;
-      if (c->cap_logits || c->sampled) { a.out_f32 = c->logits; a.ldo = c->V; }
-      if (c->dbg_withhold_spin > 0) { a.withhold = true; a.spin_limit = (unsigned)c->dbg_withhold_spin; }
-      fgemm(EPI_ARGMAX, a);
-      mark(SPEC_PROF_ARGMAX); launch_argmax_merge(c->best_val, c->best_idx, c->vtiles, c->Ralloc, rows, c->tb.y, s); tick();
-    }
+    if (want_logits) lm_head_fused(rows);
+  }
+  // argmax (and, where they are wanted, logits) of the rows whose normed hidden states are in c->h
+  void lm_head_fused(int rows) {
+    FusedGemmArgs a = fargs(c->h, rows, c->k);
+    a.w[0] = (const bf16 *)c->lm_head; a.O[0] = c->V; a.nw = 1;
+    with_norm_scale(a);
+    a.best_val = c->best_val; a.best_idx = c->best_idx; a.best_ld = c->Ralloc;
+    if (c->cap_logits || c->sampled) { a.out_f32 = c->logits; a.ldo = c->V; }
+    if (c->dbg_withhold_spin > 0) { a.withhold = true; a.spin_limit = (unsigned)c->dbg_withhold_spin; }
+    fgemm(EPI_ARGMAX, a);
+    mark(SPEC_PROF_ARGMAX); launch_argmax_merge(c->best_val, c->best_idx, c->vtiles, c->Ralloc, rows, c->tb.y, s); tick();
   }
   void fuse_fused(const void *taps, int rows) {
     FusedGemmArgs a = fargs(taps, rows, 3 * c->k);
@@ -615,6 +657,137 @@ template <typename T> struct Sched {
     tick(2);
   }
 
+  // ---- packed prefill: one pass over the rows of several prompts (see do_prefill_packed) ------------------------------
+  WideGemmArgs wargs(const WideBufs &w, const void *x, int rows, int I) const {
+    WideGemmArgs a;
+    a.x = (const bf16 *)x; a.rows = rows; a.x_rows = w.cap; a.I = I; a.status = c->status; a.pdl = tl_pdl;
+    return a;
+  }
+  void wgemm(WideEpi epi, WideGemmArgs a) {
+    int rc = wide_gemm_launch(c->fg, epi, a, s);
+    if (rc && !c->sched_err) c->sched_err = rc;
+    tick();
+  }
+  // The passes of up to 256 rows stay on the weight-streaming kernel (its launches split K, so a short pass still spreads
+  // over the chip: 139 us per layer of the 8B shapes at 256 rows, against 128 us plus a longer epilogue for a single row
+  // tile of the wide kernel); above, the wide kernel takes the pass in one sweep over the weights.
+  bool narrow(int rows) const { return rows <= 256; }
+  void pass_qkv(const WideBufs &w, const LayerW &lw, KvPool pool, int rows, bool draft) {
+    const int qd = c->H * c->hd, kvd = c->G * c->hd;
+    const PageMap pm{c->page_table, c->pps, c->cfg.page_size, c->cfg.num_pages};
+    if (narrow(rows)) {
+      FusedGemmArgs a = fargs(w.h, rows, c->k);
+      a.w[0] = (const bf16 *)lw.wq; a.w[1] = (const bf16 *)lw.wk; a.w[2] = (const bf16 *)lw.wv;
+      a.O[0] = qd; a.O[1] = kvd; a.O[2] = kvd; a.nw = 3;
+      a.ssq_in = w.ssq; a.ssq_in_tiles = c->ktiles; a.ssq_ld = w.cap; a.k_in = c->k; a.eps = c->cfg.rms_eps;
+      a.cs = w.cs; a.q = w.q; a.pool = pool; a.pm = pm;
+      a.m.seq = draft ? w.m.seq_d : w.m.seq; a.m.kvpos = w.m.pos;
+      a.H = c->H; a.G = c->G; a.hd = c->hd;
+      fgemm(EPI_QKV, a);
+      return;
+    }
+    WideGemmArgs a = wargs(w, w.h, rows, c->k);
+    int n = 0;
+    if (!draft) { a.w[n] = (const bf16 *)lw.wq; a.O[n++] = qd; }
+    a.w[n] = (const bf16 *)lw.wk; a.O[n++] = kvd;
+    a.w[n] = (const bf16 *)lw.wv; a.O[n++] = kvd;
+    a.nw = n;
+    a.ssq_in = w.ssq; a.ssq_in_tiles = c->ktiles; a.ssq_ld = w.cap; a.k_in = c->k; a.eps = c->cfg.rms_eps;
+    a.cs = w.cs; a.slot = draft ? w.m.slot_d : w.m.slot; a.q = w.q; a.pool = pool; a.H = c->H; a.G = c->G; a.page_size = c->cfg.page_size;
+    wgemm(WIDE_QKV, a);
+  }
+  void pass_resid(const WideBufs &w, const void *in, int I, const void *wt, int rows, bool add, const void *gain, int tap_mask) {
+    if (narrow(rows)) {
+      FusedGemmArgs a = fargs(in, rows, I);
+      a.w[0] = (const bf16 *)wt; a.O[0] = c->k; a.nw = 1;
+      a.xres = w.x; a.gain = (const bf16 *)gain; a.hb = w.h; a.ssq_out = w.ssq; a.ssq_ld = w.cap;
+      a.taps = w.taps; a.tap_mask = tap_mask; a.resid_add = add ? 1 : 0;
+      fgemm(EPI_RESID, a);
+      return;
+    }
+    WideGemmArgs a = wargs(w, in, rows, I);
+    a.w[0] = (const bf16 *)wt; a.O[0] = c->k; a.nw = 1;
+    a.xres = w.x; a.gain = (const bf16 *)gain; a.hb = w.h; a.ssq_out = w.ssq; a.ssq_ld = w.cap;
+    a.taps = w.taps; a.tap_mask = tap_mask; a.resid_add = add ? 1 : 0;
+    wgemm(WIDE_RESID, a);
+  }
+  void pass_swiglu(const WideBufs &w, const LayerW &lw, int rows) {
+    if (narrow(rows)) {
+      FusedGemmArgs a = fargs(w.h, rows, c->k);
+      a.w[0] = (const bf16 *)lw.w_gate; a.w[1] = (const bf16 *)lw.w_up; a.O[0] = c->F; a.O[1] = c->F; a.nw = 2;
+      a.ssq_in = w.ssq; a.ssq_in_tiles = c->ktiles; a.ssq_ld = w.cap; a.k_in = c->k; a.eps = c->cfg.rms_eps;
+      a.act = w.act;
+      fgemm(EPI_SWIGLU, a);
+      return;
+    }
+    WideGemmArgs a = wargs(w, w.h, rows, c->k);
+    a.w[0] = (const bf16 *)lw.w_gate; a.w[1] = (const bf16 *)lw.w_up; a.O[0] = c->F; a.O[1] = c->F; a.nw = 2;
+    a.ssq_in = w.ssq; a.ssq_in_tiles = c->ktiles; a.ssq_ld = w.cap; a.k_in = c->k; a.eps = c->cfg.rms_eps;
+    a.act = w.act;
+    wgemm(WIDE_SWIGLU, a);
+  }
+  // Nothing reads the last layer's hidden states but the prompts' last positions (for their first token), unless that
+  // layer is tapped for the draft; and of the draft layer the prefill needs only the cached K/V: the rest is not computed.
+  bool last_layer_on_last_rows() const { return tap_mask_of(c->L - 1) == 0; }
+  void prefill_pass(const WideBufs &w, int rows, const CausalBlock *blocks, int n_blocks, const int2 *fin, int nfin) {
+    const PageMap pm{c->page_table, c->pps, c->cfg.page_size, c->cfg.num_pages};
+    const int qd = c->H * c->hd;
+    launch_pack_meta(blocks, n_blocks, c->prompt_dev, w.m, pm, c->G, c->status, s); tick();
+    launch_rope_table(w.m.pos, rows, c->hd / 2, c->inv_freq, w.cs, s); tick();
+    launch_embed_norm((const bf16 *)c->embed, w.m.tok, (const bf16 *)c->tl[0].attn_norm, w.x, w.h, w.ssq, rows, c->k, w.cap, s); tick();
+    const bool prune = last_layer_on_last_rows();
+    for (int l = 0; l < c->L; l++) {
+      const LayerW &lw = c->tl[l];
+      pass_qkv(w, lw, c->pools[l], rows, false);
+      CausalArgs a;
+      a.q = w.q; a.q_rows = w.cap; a.pool = c->pools[l]; a.pm = pm; a.out = w.ao; a.H = c->H; a.G = c->G;
+      a.blocks = blocks; a.n_blocks = n_blocks; a.status = c->status;
+      int rc = launch_causal_attn(a, s);
+      if (rc && !c->sched_err) c->sched_err = rc;
+      tick();
+      if (prune && l == c->L - 1) break;
+      pass_resid(w, w.ao, qd, lw.wo, rows, true, lw.mlp_norm, 0);
+      pass_swiglu(w, lw, rows);
+      pass_resid(w, w.act, c->F, lw.w_down, rows, true, l + 1 < c->L ? c->tl[l + 1].attn_norm : c->final_norm, tap_mask_of(l));
+    }
+    if (nfin > 0) {
+      launch_gather_last(fin, nfin, w.taps, (bf16 *)c->pend_taps, c->Pmax, w.x, c->x, c->k, prune ? w.ao : nullptr, (bf16 *)c->ao, qd, s);
+      tick();
+    }
+    if (rows == nfin) return;               // prompts of one token: the draft has no entry yet
+    if (narrow(rows)) {
+      FusedGemmArgs a = fargs(w.taps, rows, 3 * c->k);
+      a.w[0] = (const bf16 *)c->fc3; a.O[0] = c->k; a.nw = 1;
+      a.out_f32 = c->proj; a.ldo = c->k;
+      fgemm(EPI_F32, a);
+      launch_build_cat<bf16>(c->proj, 1, 0, nullptr, (const bf16 *)c->embed, w.m.tok_next, w.m.seq_d, w.cat, rows, c->k, s); tick();
+    } else {
+      launch_embed_half((const bf16 *)c->embed, w.m.tok_next, w.cat, rows, c->k, s); tick();
+      WideGemmArgs a = wargs(w, w.taps, rows, 3 * c->k);
+      a.w[0] = (const bf16 *)c->fc3; a.O[0] = c->k; a.nw = 1;
+      a.out_b = w.cat; a.ldo = 2 * c->k;
+      wgemm(WIDE_BF16, a);
+    }
+    pass_resid(w, w.cat, 2 * c->k, c->fc2, rows, false, c->dl.attn_norm, 0);
+    pass_qkv(w, c->dl, c->pools[c->L], rows, true);
+  }
+  // the first tokens of all sequences, from the rows the passes gathered
+  void prefill_finish() {
+    if (last_layer_on_last_rows()) {
+      const LayerW &lw = c->tl[c->L - 1];
+      fgemm_resid(c->ao, c->H * c->hd, lw.wo, c->B, true, lw.mlp_norm, 0);
+      FusedGemmArgs g = fargs(c->h, c->B, c->k);
+      g.w[0] = (const bf16 *)lw.w_gate; g.w[1] = (const bf16 *)lw.w_up; g.O[0] = c->F; g.O[1] = c->F; g.nw = 2;
+      with_norm_scale(g);
+      g.act = (bf16 *)c->act;
+      fgemm(EPI_SWIGLU, g);
+      fgemm_resid(c->act, c->F, lw.w_down, c->B, true, c->final_norm, 0);
+    } else {
+      launch_residual_norm(c->x, (const bf16 *)c->final_norm, (bf16 *)c->h, c->ssq, c->B, c->k, c->Ralloc, s); tick();
+    }
+    lm_head_fused(c->B);
+  }
+
   void step(bool plain) {
     int rows = plain ? c->B : c->Tv, rps = plain ? 1 : c->N;
     tl_launch_budget = c->dbg_launch_budget;
@@ -686,6 +859,128 @@ static int read_status(spec_ctx *c) {
   return SPEC_OK;
 }
 
+// ---- prefill, one prompt after the other in passes of PREFILL_CHUNK rows: the fp32 model, head dimensions other than 128
+// and the page sizes without tensor maps
+template <typename T> static int prefill_blocks(spec_ctx *c, const int32_t *lens, int32_t *root_host) {
+  cudaStream_t s = c->stream;
+  Sched<T> sc(c);
+  const int B = c->B, CH = PREFILL_CHUNK;
+  auto upload_meta = [&](int nvalid, int b, int start, const int32_t *toks_dev) -> cudaError_t {
+    launch_prefill_meta(c->meta, toks_dev, b, start, nvalid, CH, PREFILL_BLOCK, s);
+    sc.tick();
+    return cudaGetLastError();
+  };
+  size_t off = 0;
+  for (int b = 0; b < B; b++) {
+    int n = lens[b];
+    for (int start = 0; start < n; start += CH) {
+      int nv = std::min(CH, n - start);
+      bool last = start + nv == n;
+      CUDA_TRY(c, upload_meta(nv, b, start, c->prompt_dev + off + start));
+      c->cur_rps = PREFILL_BLOCK;
+      c->ctx_hint = start + CH - PREFILL_BLOCK;
+      sc.target_forward(CH, PREFILL_BLOCK, last);
+      if (last) {
+        // the last position stays pending: its taps become pending entry 0
+        CUDA_TRY(c, cudaMemcpyAsync((char *)c->pend_taps + (size_t)b * c->Pmax * 3 * c->k * c->esz,
+                                    (char *)c->node_taps + (size_t)(nv - 1) * 3 * c->k * c->esz, (size_t)3 * c->k * c->esz,
+                                    cudaMemcpyDeviceToDevice, s));
+        CUDA_TRY(c, cudaMemcpyAsync(&root_host[b], c->tb.y + (nv - 1), 4, cudaMemcpyDeviceToHost, s));
+      }
+      int nd = last ? nv - 1 : nv;        // draft entries j use token j+1; the last position waits for the root
+      if (nd > 0) {
+        sc.fuse(c->node_taps, CH);
+        CUDA_TRY(c, upload_meta(nd, b, start, c->prompt_dev + off + start + 1));
+        sc.draft_forward(c->proj, c->np_proj, c->ps_proj, nullptr, CH, PREFILL_BLOCK);
+      }
+    }
+    CUDA_TRY(c, cudaStreamSynchronize(s));
+    c->ctx_hint = -1;
+    off += n;
+  }
+  return SPEC_OK;
+}
+
+// ---- prefill, packed: the prompts' positions are laid out one after the other and cut into passes of up to ~3000 rows
+// whatever prompt they belong to, so every weight is read once per pass and not once per prompt and 256 positions, and the
+// GEMMs run at the tensor pipe's rate (64 prompts of 64..768 tokens: 26.6k rows are 9 passes instead of 132).
+constexpr int WIDE_MAX_TILES = 16;       // row tiles (256 rows) of a pass: the waves of a launch are full enough by then
+constexpr int WIDE_LAYER_COST = 64;      // what a layer's launches cost beside their waves, in k-blocks (0.27 us each)
+static int prefill_packed(spec_ctx *c, const int32_t *lens, size_t total, int32_t *root_host, bool &done) {
+  done = false;
+  const spec_cfg &g = c->cfg;
+  if (!c->fused || !causal_attn_supported(c->hd, g.page_size) || (g.flags & (SPEC_FLAG_REF_ATTN | SPEC_FLAG_NO_TMA_ATTN))) return SPEC_OK;
+  if (total > (size_t)1 << 30) return SPEC_OK;
+  const int B = c->B, blk = causal_block_rows(c->H / c->G);
+  const int ntiles = (int)((total + WIDE_ROWS - 1) / WIDE_ROWS);
+  // The layout follows from the context alone, not from this call's prompts: tensor maps are cached by address.  A block
+  // ends at a multiple of `blk` positions, at a prompt's end or at a pass boundary.
+  const size_t most = (size_t)B * g.max_ctx, most_tiles = (most + WIDE_ROWS - 1) / WIDE_ROWS;
+  const size_t max_blocks = most / blk + B + 2 * most_tiles + 2;
+  WideBufs w;
+  int cap = (int)std::min<size_t>(WIDE_MAX_TILES, most_tiles);
+  while (cap > 0 && wide_carve(c, w, nullptr, cap * WIDE_ROWS, max_blocks, B) > c->wide_bytes) cap--;
+  if (cap < 1) return SPEC_OK;
+  // ---- row tiles per pass: the split whose launches take the fewest waves
+  const int qd = c->H * c->hd, kvd = c->G * c->hd;
+  const int Oqkv[3] = {qd, kvd, kvd}, Ok[1] = {c->k}, Of[2] = {c->F, c->F};
+  std::vector<long long> cost(cap + 1, 0);
+  for (int m = 1; m <= cap; m++) {
+    const long long layer = wide_gemm_cost(WIDE_QKV, Oqkv, 3, c->k, m) + wide_gemm_cost(WIDE_RESID, Ok, 1, qd, m) +
+                            wide_gemm_cost(WIDE_SWIGLU, Of, 2, c->k, m) + wide_gemm_cost(WIDE_RESID, Ok, 1, c->F, m) + WIDE_LAYER_COST;
+    cost[m] = layer * c->L + wide_gemm_cost(WIDE_BF16, Ok, 1, 3 * c->k, m) + wide_gemm_cost(WIDE_RESID, Ok, 1, 2 * c->k, m) + WIDE_LAYER_COST;
+  }
+  std::vector<long long> best(ntiles + 1, 0);
+  std::vector<int> pick(ntiles + 1, 0);
+  for (int n = 1; n <= ntiles; n++)
+    for (int m = 1; m <= std::min(cap, n); m++)
+      if (!pick[n] || best[n - m] + cost[m] < best[n]) { best[n] = best[n - m] + cost[m]; pick[n] = m; }
+  std::vector<int> pass_tiles;
+  for (int n = ntiles; n > 0; n -= pick[n]) pass_tiles.push_back(pick[n]);
+  std::sort(pass_tiles.rbegin(), pass_tiles.rend());       // the ragged end falls into the smallest pass
+  // ---- the blocks of each pass
+  struct Pass { int rows; size_t blk0, nblk, fin0, nfin; };
+  std::vector<Pass> passes;
+  std::vector<CausalBlock> blocks;
+  std::vector<int2> fin;
+  int b = 0, at = 0;
+  size_t off = 0, left = total;
+  for (int m : pass_tiles) {
+    Pass ps = {(int)std::min<size_t>(left, (size_t)m * WIDE_ROWS), blocks.size(), 0, fin.size(), 0};
+    for (int row = 0; row < ps.rows;) {
+      const int take = std::min(ps.rows - row, lens[b] - at);
+      for (int j = 0; j < take;) {        // blocks end at multiples of blk, so that their key range ends with a key tile
+        const int n = std::min(take - j, blk - (at + j) % blk);
+        blocks.push_back(CausalBlock{row + j, n, b, at + j, (int32_t)off, lens[b], 0, 0});
+        j += n;
+      }
+      row += take; at += take;
+      if (at == lens[b]) { fin.push_back(make_int2(row - 1, b)); off += lens[b]; at = 0; b++; }
+    }
+    left -= ps.rows;
+    ps.nblk = blocks.size() - ps.blk0; ps.nfin = fin.size() - ps.fin0;
+    // the attention CTAs are issued longest key range first
+    std::stable_sort(blocks.begin() + ps.blk0, blocks.end(), [](const CausalBlock &x, const CausalBlock &y) { return x.pos0 + x.nrows > y.pos0 + y.nrows; });
+    passes.push_back(ps);
+  }
+  if (blocks.size() > max_blocks || passes[0].rows > cap * WIDE_ROWS) return fail(c, SPEC_ERR_STATE, "spec_prefill: pass plan out of bounds");
+  cudaStream_t s = c->stream;
+  wide_carve(c, w, c->wide_base, cap * WIDE_ROWS, max_blocks, B);
+  CUDA_TRY(c, cudaMemcpyAsync(w.blocks, blocks.data(), blocks.size() * sizeof(CausalBlock), cudaMemcpyHostToDevice, s));
+  CUDA_TRY(c, cudaMemcpyAsync(w.fin, fin.data(), fin.size() * sizeof(int2), cudaMemcpyHostToDevice, s));
+  {
+    Sched<bf16> sc(c);
+    for (const Pass &ps : passes) sc.prefill_pass(w, ps.rows, w.blocks + ps.blk0, (int)ps.nblk, w.fin + ps.fin0, (int)ps.nfin);
+    sc.prefill_finish();
+  }
+  CUDA_TRY(c, cudaGetLastError());
+  if (c->sched_err) return fail(c, SPEC_ERR_CUDA, "a prefill launch was rejected (code %d)", c->sched_err);
+  CUDA_TRY(c, cudaMemcpyAsync(root_host, c->tb.y, B * 4, cudaMemcpyDeviceToHost, s));
+  CUDA_TRY(c, cudaStreamSynchronize(s));
+  done = true;
+  return SPEC_OK;
+}
+
 template <typename T> static int do_prefill(spec_ctx *c, const int32_t *ids, const int32_t *lens, int32_t reserve, int32_t *first) {
   const spec_cfg &g = c->cfg;
   cudaStream_t s = c->stream;
@@ -719,51 +1014,21 @@ template <typename T> static int do_prefill(spec_ctx *c, const int32_t *ids, con
   CUDA_TRY(c, cudaMemcpyAsync(c->st.cap, cap.data(), B * 4, cudaMemcpyHostToDevice, s));
   CUDA_TRY(c, cudaStreamSynchronize(s));
 
-  Sched<T> sc(c);
-  const int CH = PREFILL_CHUNK;
-  // the prompts go to the device once; each pass's row metadata is then built by a small kernel, so the host never
-  // waits inside the loop over passes
   size_t total_ids = 0;
-  for (int b = 0; b < B; b++) total_ids += (size_t)lens[b];
-  CUDA_TRY(c, cudaMemcpyAsync(c->prompt_dev, ids, total_ids * 4, cudaMemcpyHostToDevice, s));
-  auto upload_meta = [&](int nvalid, int b, int start, const int32_t *toks_dev) -> cudaError_t {
-    launch_prefill_meta(c->meta, toks_dev, b, start, nvalid, CH, PREFILL_BLOCK, s);
-    sc.tick();
-    return cudaGetLastError();
-  };
-  size_t off = 0;
-  std::vector<int32_t> n_host(B), P_host(B, 1), root_host(B);
   for (int b = 0; b < B; b++) {
-    const int32_t *p = ids + off;
-    int n = lens[b];
-    for (int i = 0; i < n; i++)
+    const int32_t *p = ids + total_ids;
+    for (int i = 0; i < lens[b]; i++)
       if (p[i] < 0 || p[i] >= g.vocab) return fail(c, SPEC_ERR_INVALID_CFG, "spec_prefill: token id out of range in prompt %d", b);
-    for (int start = 0; start < n; start += CH) {
-      int nv = std::min(CH, n - start);
-      bool last = start + nv == n;
-      CUDA_TRY(c, upload_meta(nv, b, start, c->prompt_dev + off + start));
-      c->cur_rps = PREFILL_BLOCK;
-      c->ctx_hint = start + CH - PREFILL_BLOCK;
-      sc.target_forward(CH, PREFILL_BLOCK, last);
-      if (last) {
-        // the last position stays pending: its taps become pending entry 0
-        CUDA_TRY(c, cudaMemcpyAsync((char *)c->pend_taps + (size_t)b * c->Pmax * 3 * c->k * c->esz,
-                                    (char *)c->node_taps + (size_t)(nv - 1) * 3 * c->k * c->esz, (size_t)3 * c->k * c->esz,
-                                    cudaMemcpyDeviceToDevice, s));
-        CUDA_TRY(c, cudaMemcpyAsync(&root_host[b], c->tb.y + (nv - 1), 4, cudaMemcpyDeviceToHost, s));
-      }
-      int nd = last ? nv - 1 : nv;        // draft entries j use token j+1; the last position waits for the root
-      if (nd > 0) {
-        sc.fuse(c->node_taps, CH);
-        CUDA_TRY(c, upload_meta(nd, b, start, c->prompt_dev + off + start + 1));
-        sc.draft_forward(c->proj, c->np_proj, c->ps_proj, nullptr, CH, PREFILL_BLOCK);
-      }
-    }
-    CUDA_TRY(c, cudaStreamSynchronize(s));
-    c->ctx_hint = -1;
-    n_host[b] = n;
-    off += n;
+    total_ids += (size_t)lens[b];
   }
+  // the prompts go to the device once; the row metadata of each pass is then built by a small kernel, so the host never
+  // waits inside the loop over passes
+  CUDA_TRY(c, cudaMemcpyAsync(c->prompt_dev, ids, total_ids * 4, cudaMemcpyHostToDevice, s));
+  std::vector<int32_t> n_host(lens, lens + B), P_host(B, 1), root_host(B);
+  bool packed = false;
+  if (int rc = prefill_packed(c, lens, total_ids, root_host.data(), packed)) return rc;
+  if (!packed)
+    if (int rc = prefill_blocks<T>(c, lens, root_host.data())) return rc;
   CUDA_TRY(c, cudaMemcpyAsync(c->st.n, n_host.data(), B * 4, cudaMemcpyHostToDevice, s));
   CUDA_TRY(c, cudaMemcpyAsync(c->st.n_prev, n_host.data(), B * 4, cudaMemcpyHostToDevice, s));
   CUDA_TRY(c, cudaMemcpyAsync(c->st.P, P_host.data(), B * 4, cudaMemcpyHostToDevice, s));

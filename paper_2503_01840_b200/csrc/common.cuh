@@ -155,6 +155,21 @@ void launch_add_norm(float *x, const float *parts, int nparts, size_t part_strid
 // tokens toks[0..nvalid) (device), causal blocks of `block` positions
 void launch_prefill_meta(RowMeta m, const int32_t *toks, int b, int start, int nvalid, int rows, int block, cudaStream_t s);
 
+// ---- packed prefill: rows of several prompts in one pass, described block by block (CausalBlock, attn_causal.cuh)
+struct CausalBlock;
+struct PackMeta {
+  int32_t *seq, *seq_d;        // sequence of the row; seq_d: the same, -1 where the draft has no entry (a prompt's last position)
+  int32_t *pos;                // position (RoPE and cache)
+  int32_t *tok, *tok_next;     // the row's token and the one after it
+  int32_t *slot, *slot_d;      // cache row page * G * page_size + offset of its K/V; slot_d: -1 where the draft has no entry
+};
+void launch_pack_meta(const CausalBlock *blocks, int n_blocks, const int32_t *prompt, PackMeta m, PageMap pm, int G, int32_t *status,
+                      cudaStream_t s);
+void launch_gather_last(const int2 *fin, int nfin, const bf16 *taps, bf16 *pend_taps, int Pmax, const float *x, float *cx, int k,
+                        const bf16 *ao, bf16 *cao, int qd, cudaStream_t s);
+void launch_embed_half(const bf16 *embed, const int32_t *tok, bf16 *cat, int rows, int k, cudaStream_t s);
+void launch_residual_norm(const float *x, const bf16 *gain, bf16 *hb, float *ssq, int rows, int k, int ssq_ld, cudaStream_t s);
+
 void launch_rope_table(const int32_t *pos, int rows, int half, const double *inv_freq, float2 *cs, cudaStream_t s);
 
 // qkv partial sums [nparts][rows][(H+2G)hd] fp32 -> q (T, [rows][H][hd], rotated) and K/V written into the

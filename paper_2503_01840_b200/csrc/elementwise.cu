@@ -1,6 +1,7 @@
 // Elementwise / per-row kernels between the GEMMs: embedding gather, split-K reduction fused with
 // residual add + RMSNorm (+ feature taps), RoPE + paged K/V write, SiLU*up, FC2 input assembly.
 // All statistics and the residual stream are fp32; T is the storage type (fp32 or bf16).
+#include "attn_causal.cuh"
 #include "common.cuh"
 
 namespace spec {
@@ -147,6 +148,87 @@ __global__ void prefill_meta_kernel(RowMeta m, const int32_t *__restrict__ toks,
 }
 void launch_prefill_meta(RowMeta m, const int32_t *toks, int b, int start, int nvalid, int rows, int block, cudaStream_t s) {
   launch_k(prefill_meta_kernel, dim3(rows / 64), dim3(64), 0, s, m, toks, b, start, nvalid, block);
+}
+
+// ---------------------------------------------------------------- packed prefill: several prompts in one pass
+// One CTA per block of query rows: what every row is (sequence, position, tokens) and where its K/V go.  Draft entry j is
+// fed with token j + 1, so the last position of a prompt has none yet (seq_d / slot_d -1).
+__global__ void pack_meta_kernel(const CausalBlock *__restrict__ blocks, const int32_t *__restrict__ prompt, PackMeta m, PageMap pm, int G,
+                                 int32_t *status) {
+  pdl_wait();
+  pdl_trigger();
+  const CausalBlock b = blocks[blockIdx.x];
+  for (int j = threadIdx.x; j < b.nrows; j += blockDim.x) {
+    const int r = b.row0 + j, pos = b.pos0 + j;
+    const bool last = pos + 1 >= b.len;
+    int slot = -1;
+    const int page = pos / pm.page_size < pm.pages_per_seq ? pm.table[(size_t)b.seq * pm.pages_per_seq + pos / pm.page_size] : -1;
+    if (page < 0 || page >= pm.num_pages) set_status(status, ST_BOUNDS, 2, r, page);
+    else slot = page * G * pm.page_size + pos % pm.page_size;
+    m.seq[r] = b.seq; m.seq_d[r] = last ? -1 : b.seq;
+    m.pos[r] = pos;
+    m.tok[r] = prompt[b.tok0 + pos]; m.tok_next[r] = last ? 0 : prompt[b.tok0 + pos + 1];
+    m.slot[r] = slot; m.slot_d[r] = last ? -1 : slot;
+  }
+}
+void launch_pack_meta(const CausalBlock *blocks, int n_blocks, const int32_t *prompt, PackMeta m, PageMap pm, int G, int32_t *status,
+                      cudaStream_t s) {
+  launch_k(pack_meta_kernel, dim3(n_blocks), dim3(128), 0, s, blocks, prompt, m, pm, G, status);
+}
+
+// What is kept of a prompt's last position (fin[i] = {row of the pass, sequence}): its feature taps become pending entry 0,
+// its residual (and, when the last layer's second half runs on these rows only, its attention output) row `sequence` of
+// the compact buffers.
+__global__ void gather_last_kernel(const int2 *__restrict__ fin, const uint4 *__restrict__ taps, uint4 *__restrict__ pend_taps, int tap_vecs,
+                                   int pend_stride, const uint4 *__restrict__ x, uint4 *__restrict__ cx, int x_vecs,
+                                   const uint4 *__restrict__ ao, uint4 *__restrict__ cao, int ao_vecs) {
+  pdl_wait();
+  pdl_trigger();
+  const int2 f = fin[blockIdx.x];
+  for (int i = threadIdx.x; i < tap_vecs; i += blockDim.x) pend_taps[(size_t)f.y * pend_stride + i] = taps[(size_t)f.x * tap_vecs + i];
+  for (int i = threadIdx.x; i < x_vecs; i += blockDim.x) cx[(size_t)f.y * x_vecs + i] = x[(size_t)f.x * x_vecs + i];
+  for (int i = threadIdx.x; i < ao_vecs; i += blockDim.x) cao[(size_t)f.y * ao_vecs + i] = ao[(size_t)f.x * ao_vecs + i];
+}
+void launch_gather_last(const int2 *fin, int nfin, const bf16 *taps, bf16 *pend_taps, int Pmax, const float *x, float *cx, int k,
+                        const bf16 *ao, bf16 *cao, int qd, cudaStream_t s) {
+  launch_k(gather_last_kernel, dim3(nfin), dim3(512), 0, s, fin, (const uint4 *)taps, (uint4 *)pend_taps, 3 * k / 8, Pmax * 3 * k / 8,
+           (const uint4 *)x, (uint4 *)cx, k / 4, (const uint4 *)ao, (uint4 *)cao, ao ? qd / 8 : 0);
+}
+
+// the embedding half of the FC2 input: cat[r][k ..] = E[tok[r]]
+__global__ void embed_half_kernel(const bf16 *__restrict__ embed, const int32_t *__restrict__ tok, bf16 *__restrict__ cat, int k, int vec) {
+  pdl_wait();
+  pdl_trigger();
+  const int r = blockIdx.x;
+  const bf16 *src = embed + (size_t)tok[r] * k;
+  bf16 *dst = cat + (size_t)r * 2 * k + k;
+  if (vec) for (int i = threadIdx.x; i < k / 8; i += blockDim.x) ((uint4 *)dst)[i] = ((const uint4 *)src)[i];
+  else for (int i = threadIdx.x; i < k; i += blockDim.x) dst[i] = src[i];
+}
+void launch_embed_half(const bf16 *embed, const int32_t *tok, bf16 *cat, int rows, int k, cudaStream_t s) {
+  launch_k(embed_half_kernel, dim3(rows), dim3(256), 0, s, embed, tok, cat, k, ((uintptr_t)embed & 15) == 0 ? 1 : 0);
+}
+
+// h = bf16(x * gain) and the per-128-feature sums of squares of residual rows that come from a copy (cf. embed_norm_kernel)
+__global__ void residual_norm_kernel(const float *__restrict__ x, const bf16 *__restrict__ gain, bf16 *__restrict__ hb, float *__restrict__ ssq,
+                                     int k, int ssq_ld) {
+  pdl_wait();
+  pdl_trigger();
+  __shared__ float sh[4];
+  const int r = blockIdx.x, tile = blockIdx.y, o = tile * 128 + threadIdx.x;
+  float v = 0.0f;
+  if (o < k) {
+    v = x[(size_t)r * k + o];
+    hb[(size_t)r * k + o] = __float2bfloat16_rn(v * __bfloat162float(gain[o]));
+  }
+  float sq = v * v;
+  for (int off = 16; off > 0; off >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, off);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = sq;
+  __syncthreads();
+  if (threadIdx.x == 0) ssq[(size_t)tile * ssq_ld + r] = ((sh[0] + sh[1]) + sh[2]) + sh[3];
+}
+void launch_residual_norm(const float *x, const bf16 *gain, bf16 *hb, float *ssq, int rows, int k, int ssq_ld, cudaStream_t s) {
+  launch_k(residual_norm_kernel, dim3(rows, (k + 127) / 128), dim3(128), 0, s, x, gain, hb, ssq, k, ssq_ld);
 }
 
 // ---------------------------------------------------------------- RoPE + q store + paged K/V write

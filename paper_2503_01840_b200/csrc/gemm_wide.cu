@@ -1,0 +1,504 @@
+// bf16 GEMM with fused epilogues for many token rows (prefill), sm_100a.
+//
+//   out[r][o] = sum_i x[r][i] * w[o][i],  hundreds to thousands of rows
+//
+// From about 215 rows on the contraction is bound by the tensor pipe, no longer by the weight stream, so this kernel is
+// the mirror image of the weight-streaming one (gemm_fused.cu): token rows are the UMMA M side, features the N side.
+//
+//  * a CTA pair (cta_group::2) owns a tile of 256 rows x 256 features: each CTA stages its own 128 rows and half of the
+//    features per 64-element k-block (32 KB, six stages), so a k-block costs 64 bytes of shared-memory fill per tensor
+//    cycle, which the L2 can deliver; one M = 256, N = 256 MMA per 16 elements;
+//  * the kernel is persistent (one pair per two SMs, tiles dealt out in order, row tiles fastest so that the pairs that
+//    run together share their weights in L2), and the 512 tensor-memory columns hold two accumulators: the epilogue of a
+//    tile runs under the main loop of the next one;
+//  * a thread of the epilogue owns one token row (tensor-memory lane), so the RMSNorm factor, the cache slot and the RoPE
+//    row are one value per thread; the values cross to row-contiguous order through 4 KB of shared memory per warp, so
+//    that every global access of the epilogue moves whole 64- or 128-byte runs.
+//
+// Measured with the packing of prompts into passes (one B200, whole requests, before: one prompt at a time in passes of 256
+// rows on the weight-streaming kernel): 64 prompts of 64..768 tokens, 8 layers of the 8B shapes, 24 chain steps 306 -> 156 ms;
+// 56 prompts of 16..96 tokens, 16 layers 268 -> 104 ms; 16384 tokens, 32 layers 535 -> 292 ms.
+//
+// Every mbarrier wait is bounded; on a time-out the CTA records it, stops, waits (bounded) for the copies in flight, keeps
+// its cluster barriers and frees its tensor memory.
+#include <cuda.h>
+#include <string.h>
+
+#include <algorithm>
+
+#include "gemm_wide.cuh"
+#include "tcgen05_ptx.cuh"
+
+namespace spec {
+
+namespace {
+
+using namespace tc;
+
+constexpr int W_HALF = 128;                               // rows of a CTA / features of a half tile
+constexpr int W_A_BYTES = W_HALF * TILE_K * 2;            // 16 KB: the CTA's rows of a k-block
+constexpr int W_STAGE = 2 * W_A_BYTES;                    // + its half of the features
+constexpr int W_STAGES = 6;
+constexpr int W_EPI_WARPS = 8;                            // two per quarter of the tensor-memory lanes: one per half tile
+constexpr int W_THREADS = (W_EPI_WARPS + 2) * 32;
+constexpr int W_STG = 32 * 128;                           // staging bytes per epilogue warp: 32 rows x 128 B
+constexpr int W_CTRL = 256;
+constexpr int W_SMEM = W_STAGES * W_STAGE + W_EPI_WARPS * W_STG + W_CTRL + 1024 /*alignment slack*/;
+constexpr int W_PAIRS = 74;                               // 148 SMs
+
+struct alignas(64) WideParams {
+  CUtensorMap map_x, map_w[3];
+  int rows, KB, m_tiles, n_tiles;
+  int h0, h1;                    // half tiles [0,h0) belong to w0, [h0,h1) to w1, the rest to w2
+  int O[3];
+  int kind0;                     // WIDE_QKV: what w0 is (0 q, 1 k)
+  const float *ssq_in; int ssq_in_tiles, ssq_ld; float inv_k_in, eps;
+  float *xres; const bf16 *gain; bf16 *hb; float *ssq_out; bf16 *taps; int tap_mask, resid_add;
+  const float2 *cs; const int32_t *slot; bf16 *q; bf16 *kp, *vp; int H, page_size;
+  bf16 *act;
+  bf16 *out_b; int ldo;
+  int32_t *status;
+};
+
+__device__ __forceinline__ void cluster_sync_all() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// one arrival on an mbarrier of the cluster (shared::cluster address), releasing this thread's earlier work
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t addr) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
+}
+// bounded wait for arrivals that come from both CTAs of the pair (cluster-scope acquire)
+__device__ __forceinline__ bool mbar_wait_cluster(uint64_t *bar, uint32_t parity) {
+  const uint32_t addr = smem_u32(bar);
+  for (uint32_t it = 0; it < SPIN_LIMIT; it++) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(addr), "r"(parity)
+        : "memory");
+    if (ok) return true;
+  }
+  return false;
+}
+// 32 consecutive columns of this thread's tensor-memory lane; tmem_ld_wait() before the values are used
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, "
+      "%19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]), "=r"(v[9]),
+        "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]), "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]),
+        "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]),
+        "=r"(v[30]), "=r"(v[31])
+      : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t pack2(float a, float b) {
+  __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
+  return *(uint32_t *)&v;
+}
+__device__ __forceinline__ uint2 pack4(float4 v) { return make_uint2(pack2(v.x, v.y), pack2(v.z, v.w)); }
+
+// 32 values of every lane's own row -> row-contiguous order: afterwards lane l holds, in t[i], columns 4 (l % 8) .. + 3 of
+// row 4 i + l / 8.  stg: the warp's 4 KB, 16-byte chunks swizzled by the row.
+__device__ __forceinline__ void transpose32(unsigned char *stg, int lane, const uint32_t (&v)[32], float4 (&t)[8]) {
+#pragma unroll
+  for (int j = 0; j < 8; j++)
+    *(uint4 *)(stg + lane * 128 + ((j ^ (lane & 7)) << 4)) = make_uint4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+  __syncwarp();
+#pragma unroll
+  for (int i = 0; i < 8; i++) {
+    const int r = i * 4 + (lane >> 3);
+    t[i] = *(const float4 *)(stg + r * 128 + (((lane & 7) ^ (r & 7)) << 4));
+  }
+  __syncwarp();
+}
+
+template <int EPI>
+__global__ void __launch_bounds__(W_THREADS, 1) gemm_wide_kernel(const __grid_constant__ WideParams p) {
+  extern __shared__ unsigned char smem_raw[];
+  unsigned char *ring = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  unsigned char *stg_all = ring + W_STAGES * W_STAGE;
+  uint64_t *full = (uint64_t *)(stg_all + W_EPI_WARPS * W_STG);
+  uint64_t *empty = full + W_STAGES;
+  uint64_t *tfull = empty + W_STAGES, *tempty = tfull + 2;
+  uint32_t *tmem_slot = (uint32_t *)(tempty + 2);
+  volatile uint32_t *abort_flag = tmem_slot + 1;
+  volatile int *n_issued = (volatile int *)(tmem_slot + 2), *n_consumed = (volatile int *)(tmem_slot + 3);
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  uint32_t crank;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(crank));
+  const int xr = (int)(crank & 1u);
+  const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
+  const int ntiles = p.m_tiles * p.n_tiles, KB = p.KB;
+
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < W_STAGES; i++) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
+    for (int i = 0; i < 2; i++) { mbar_init(&tfull[i], 1); mbar_init(&tempty[i], 2 * W_EPI_WARPS); }
+    *abort_flag = 0;
+    *n_issued = 0; *n_consumed = 0;
+    // the pair is (even, odd) blocks with ranks 0, 1: checked, never assumed
+    if (crank != (blockIdx.x & 1u)) { *abort_flag = 1; set_status(p.status, ST_TIMEOUT, 244, blockIdx.x, (int)crank); }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == W_EPI_WARPS + 1) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(512) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  cluster_sync_all();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem_base = *tmem_slot;        // 512 columns: the whole tensor memory, so both CTAs start at column 0
+  pdl_trigger();
+
+  if (warp == W_EPI_WARPS) {
+    // ================================================================ producer (converged warp, the elected lane issues)
+    const uint64_t pol = l2_policy_evict_first();
+    int issued = 0, st = 0;
+    uint32_t ph = 1;                             // a stage's first use needs no wait: the preceding phase counts as complete
+    bool ok = !*abort_flag, first = true;
+    for (int t = pair; t < ntiles && ok; t += n_pairs) {
+      const int mt = t % p.m_tiles, nt = t / p.m_tiles;
+      int mi = 0, tm = nt;
+      if (EPI == WIDE_SWIGLU) mi = xr;
+      else {
+        tm = 2 * nt + xr;
+        if (tm >= p.h1) { mi = 2; tm -= p.h1; }
+        else if (tm >= p.h0) { mi = 1; tm -= p.h0; }
+      }
+      const CUtensorMap *mw = &p.map_w[mi];
+      const int wrow = tm * W_HALF, xrow = mt * WIDE_ROWS + xr * W_HALF;
+      int kb = 0;
+      if (first) {
+        // the weights do not depend on the previous kernel: fill the ring with them, then wait for the activations
+        first = false;
+        const int npre = KB < W_STAGES ? KB : W_STAGES;
+        if (elect_one())
+          for (int i = 0; i < npre; i++) {
+            if (xr == 0) mbar_expect_tx(&full[i], 2 * W_STAGE);
+            tma_load_2d_pair_hint(ring + i * W_STAGE + W_A_BYTES, mw, i * TILE_K, wrow, mapa_u32(smem_u32(&full[i]), 0u), pol);
+          }
+        __syncwarp();
+        pdl_wait();
+        if (elect_one())
+          for (int i = 0; i < npre; i++) tma_load_2d_pair(ring + i * W_STAGE, &p.map_x, i * TILE_K, xrow, mapa_u32(smem_u32(&full[i]), 0u));
+        __syncwarp();
+        kb = npre; issued = npre;
+        if (npre == W_STAGES) ph = 0; else st = npre;
+      }
+      for (; kb < KB; kb++) {
+        if (!mbar_wait_warp(&empty[st], ph)) { *abort_flag = 1; set_status(p.status, ST_TIMEOUT, 240, blockIdx.x, t); ok = false; break; }
+        if (elect_one()) {
+          unsigned char *a = ring + st * W_STAGE;
+          const uint32_t fb = mapa_u32(smem_u32(&full[st]), 0u);
+          if (xr == 0) mbar_expect_tx(&full[st], 2 * W_STAGE);
+          tma_load_2d_pair_hint(a + W_A_BYTES, mw, kb * TILE_K, wrow, fb, pol);
+          tma_load_2d_pair(a, &p.map_x, kb * TILE_K, xrow, fb);
+        }
+        __syncwarp();
+        issued++;
+        if (++st == W_STAGES) { st = 0; ph ^= 1u; }
+      }
+    }
+    if (first) pdl_wait();
+    if (lane == 0) *n_issued = issued;
+  } else if (warp == W_EPI_WARPS + 1) {
+    // ================================================================ MMA issuer (even CTA only)
+    pdl_wait();
+    if (xr == 0 && !*abort_flag) {
+      constexpr uint32_t idesc = umma_idesc_m(256, 256);
+      const uint64_t desc0 = umma_desc_sw128(smem_u32(ring));
+      int consumed = 0, st = 0, it = 0;
+      uint32_t ph = 0, ready = 0;
+      bool ok = true;
+      for (int t = pair; t < ntiles && ok; t += n_pairs, it++) {
+        const int acc = it & 1, use = it >> 1;
+        if (use > 0) {                           // both CTAs' epilogues have emptied this accumulator
+          const bool w = mbar_wait_cluster(&tempty[acc], (uint32_t)((use - 1) & 1));
+          if (!__all_sync(0xffffffffu, w)) { *abort_flag = 1; set_status(p.status, ST_TIMEOUT, 241, blockIdx.x, t); break; }
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        }
+        const uint32_t d = tmem_base + (uint32_t)(acc * 256);
+        for (int kb = 0; kb < KB; kb++) {
+          if (!ready && !mbar_wait_warp(&full[st], ph)) { *abort_flag = 1; set_status(p.status, ST_TIMEOUT, 242, blockIdx.x, t); ok = false; break; }
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const uint64_t da = desc0 + (uint64_t)((st * W_STAGE) >> 4), db = da + (W_A_BYTES >> 4);
+          int nst = st + 1;
+          uint32_t nph = ph;
+          if (nst == W_STAGES) { nst = 0; nph ^= 1u; }
+          if (elect_one()) {
+#pragma unroll
+            for (int j = 0; j < TILE_K / UMMA_K; j++) umma_bf16_pair(d, da + 2 * j, db + 2 * j, idesc, (kb | j) ? 1u : 0u);
+            umma_commit_pair(&empty[st], 0u);    // frees the stage in both CTAs
+            if (kb == KB - 1) umma_commit_pair(&tfull[acc], 0u);
+          }
+          __syncwarp();
+          consumed++;
+          ready = mbar_test_warp(&full[nst], nph) ? 1u : 0u;
+          st = nst; ph = nph;
+        }
+      }
+      if (lane == 0) *n_consumed = consumed;
+    }
+  } else {
+    // ================================================================ epilogue: thread = token row, warp / 4 = half tile
+    pdl_wait();
+    unsigned char *stg = stg_all + warp * W_STG;
+    const int quarter = warp & 3, half = warp >> 2;
+    const int sub = lane >> 3, c4 = (lane & 7) * 4;              // place in row-contiguous order: rows 4 i + sub, columns c4 ..
+    int it = 0;
+    for (int t = pair; t < ntiles; t += n_pairs, it++) {
+      const int acc = it & 1, use = it >> 1;
+      const int mt = t % p.m_tiles, nt = t / p.m_tiles;
+      const int row_w = mt * WIDE_ROWS + xr * W_HALF + quarter * 32;        // first row of the warp
+      const int row = row_w + lane;
+      const bool any_row = row_w < p.rows;
+      float inv = 1.0f;
+      if (p.ssq_in && row < p.rows) {
+        float ss = 0.0f;
+#pragma unroll 8
+        for (int u = 0; u < p.ssq_in_tiles; u++) ss += p.ssq_in[(size_t)u * p.ssq_ld + row];
+        inv = 1.0f / sqrtf(ss * p.inv_k_in + p.eps);
+      }
+      int slot = -1;
+      if (EPI == WIDE_QKV && row < p.rows) slot = p.slot[row];
+      // everything that does not depend on the accumulator is requested before the wait for it
+      float4 xin[8];
+      const int fo0 = nt * 256 + half * 128;                     // WIDE_RESID / WIDE_BF16: first feature of the warp
+      if (EPI == WIDE_RESID && p.resid_add && any_row) {
+#pragma unroll
+        for (int i = 0; i < 8; i++) {
+          const int gr = row_w + i * 4 + sub, f = fo0 + c4;
+          xin[i] = (gr < p.rows && f < p.O[0]) ? *(const float4 *)(p.xres + (size_t)gr * p.O[0] + f) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+      }
+      bool ok = mbar_wait_warp(&tfull[acc], (uint32_t)(use & 1));
+      if (!ok || *abort_flag) {
+        if (!ok && lane == 0) { *abort_flag = 1; set_status(p.status, ST_TIMEOUT, 243, blockIdx.x, t); }
+        break;
+      }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t ta = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * 256);
+      if (EPI == WIDE_RESID || EPI == WIDE_BF16) {
+        float sq[8];
+#pragma unroll
+        for (int i = 0; i < 8; i++) sq[i] = 0.0f;
+#pragma unroll
+        for (int c = 0; c < 4; c++) {
+          uint32_t v[32];
+          tmem_ld32(ta + half * 128 + c * 32, v);
+          float4 a[8];
+          transpose32(stg, lane, v, a);
+          const int f = fo0 + c * 32 + c4;
+          const bool fok = f < p.O[0];
+          if (EPI == WIDE_BF16) {
+#pragma unroll
+            for (int i = 0; i < 8; i++) {
+              const int gr = row_w + i * 4 + sub;
+              if (gr < p.rows && fok) *(uint2 *)(p.out_b + (size_t)gr * p.ldo + f) = pack4(a[i]);
+            }
+          } else {
+            float4 xn[8];                         // the next 32 columns of the residual, in flight during this round
+            if (c < 3 && p.resid_add && any_row) {
+#pragma unroll
+              for (int i = 0; i < 8; i++) {
+                const int gr = row_w + i * 4 + sub;
+                xn[i] = (gr < p.rows && f + 32 < p.O[0]) ? *(const float4 *)(p.xres + (size_t)gr * p.O[0] + f + 32) : make_float4(0.f, 0.f, 0.f, 0.f);
+              }
+            }
+            float4 gn = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (fok) {
+              const uint2 g = *(const uint2 *)(p.gain + f);
+              const float2 g01 = __bfloat1622float2(*(const __nv_bfloat162 *)&g.x), g23 = __bfloat1622float2(*(const __nv_bfloat162 *)&g.y);
+              gn = make_float4(g01.x, g01.y, g23.x, g23.y);
+            }
+#pragma unroll
+            for (int i = 0; i < 8; i++) {
+              const int gr = row_w + i * 4 + sub;
+              float4 o = a[i];
+              if (p.resid_add) { o.x += xin[i].x; o.y += xin[i].y; o.z += xin[i].z; o.w += xin[i].w; }
+              if (gr < p.rows && fok) {
+                const size_t xi = (size_t)gr * p.O[0] + f;
+                *(float4 *)(p.xres + xi) = o;
+                *(uint2 *)(p.hb + xi) = pack4(make_float4(o.x * gn.x, o.y * gn.y, o.z * gn.z, o.w * gn.w));
+                if (p.tap_mask) {
+                  const uint2 tb = pack4(o);
+#pragma unroll
+                  for (int s = 0; s < 3; s++)
+                    if ((p.tap_mask >> s) & 1) *(uint2 *)(p.taps + (size_t)gr * 3 * p.O[0] + (size_t)s * p.O[0] + f) = tb;
+                }
+                sq[i] += (o.x * o.x + o.y * o.y) + (o.z * o.z + o.w * o.w);
+              }
+              if (c < 3) xin[i] = xn[i];
+            }
+          }
+        }
+        if (EPI == WIDE_RESID) {
+#pragma unroll
+          for (int i = 0; i < 8; i++) {
+            float s = sq[i];
+            for (int off = 4; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+            const int gr = row_w + i * 4 + sub;
+            if ((lane & 7) == 0 && gr < p.rows && fo0 < p.O[0]) p.ssq_out[(size_t)(fo0 >> 7) * p.ssq_ld + gr] = s;
+          }
+        }
+      } else if (EPI == WIDE_SWIGLU) {
+        // this warp: gate columns 64 half .. + 63, up columns 128 + the same, of features 128 nt + 64 half ..
+        const int f0 = nt * 128 + half * 64;
+#pragma unroll
+        for (int c = 0; c < 2; c++) {
+          uint32_t g[32], u[32];
+          tmem_ld32(ta + half * 64 + c * 32, g);
+          tmem_ld32(ta + 128 + half * 64 + c * 32, u);
+#pragma unroll
+          for (int j = 0; j < 4; j++) {
+            uint32_t w[4];
+#pragma unroll
+            for (int e = 0; e < 4; e++) {
+              float r[2];
+#pragma unroll
+              for (int z = 0; z < 2; z++) {
+                const float gv = __uint_as_float(g[8 * j + 2 * e + z]) * inv, uv = __uint_as_float(u[8 * j + 2 * e + z]) * inv;
+                r[z] = (gv / (1.0f + expf(-gv))) * uv;
+              }
+              w[e] = pack2(r[0], r[1]);
+            }
+            *(uint4 *)(stg + lane * 128 + (((c * 4 + j) ^ (lane & 7)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
+          }
+        }
+        __syncwarp();
+        const int f = f0 + (lane & 7) * 8;
+#pragma unroll
+        for (int i = 0; i < 8; i++) {
+          const int r = i * 4 + sub, gr = row_w + r;
+          if (gr < p.rows && f < p.O[0])
+            *(uint4 *)(p.act + (size_t)gr * p.O[0] + f) = *(const uint4 *)(stg + r * 128 + (((lane & 7) ^ (r & 7)) << 4));
+        }
+        __syncwarp();
+      } else {   // WIDE_QKV: the half tile is one head of q, k or v
+        int mi = 0, tm = 2 * nt + half;
+        if (tm >= p.h1) { mi = 2; tm -= p.h1; }
+        else if (tm >= p.h0) { mi = 1; tm -= p.h0; }
+        const int kind = mi + p.kind0;
+        const bool head_ok = tm * 128 < p.O[mi];
+        bf16 *kv = kind == 1 ? p.kp : p.vp;
+#pragma unroll
+        for (int c = 0; c < 2; c++) {
+          float4 a[8], b[8];
+          {
+            uint32_t v[32];
+            tmem_ld32(ta + half * 128 + c * 32, v);
+            transpose32(stg, lane, v, a);
+            tmem_ld32(ta + half * 128 + 64 + c * 32, v);
+            transpose32(stg, lane, v, b);
+          }
+#pragma unroll
+          for (int i = 0; i < 8; i++) {
+            const int r = i * 4 + sub, gr = row_w + r;
+            const float sc = __shfl_sync(0xffffffffu, inv, r);
+            const int sl = __shfl_sync(0xffffffffu, slot, r);
+            if (gr >= p.rows || !head_ok) continue;
+            float4 lo = make_float4(a[i].x * sc, a[i].y * sc, a[i].z * sc, a[i].w * sc);
+            float4 hi = make_float4(b[i].x * sc, b[i].y * sc, b[i].z * sc, b[i].w * sc);
+            if (kind < 2) {                       // rotate-half RoPE: feature j pairs with j + 64
+              const float4 c0 = *(const float4 *)(p.cs + (size_t)gr * 64 + c * 32 + c4), c1 = *(const float4 *)(p.cs + (size_t)gr * 64 + c * 32 + c4 + 2);
+              const float4 l = lo, h = hi;
+              lo = make_float4(l.x * c0.x - h.x * c0.y, l.y * c0.z - h.y * c0.w, l.z * c1.x - h.z * c1.y, l.w * c1.z - h.w * c1.w);
+              hi = make_float4(h.x * c0.x + l.x * c0.y, h.y * c0.z + l.y * c0.w, h.z * c1.x + l.z * c1.y, h.w * c1.z + l.w * c1.w);
+            }
+            bf16 *dst = nullptr;
+            if (kind == 0) dst = p.q + ((size_t)gr * p.H + tm) * 128;
+            else if (sl >= 0) dst = kv + ((size_t)sl + (size_t)tm * p.page_size) * 128;
+            if (dst) {
+              *(uint2 *)(dst + c * 32 + c4) = pack4(lo);
+              *(uint2 *)(dst + 64 + c * 32 + c4) = pack4(hi);
+            }
+          }
+        }
+      }
+      // the accumulator may be overwritten: one arrival per warp on the even CTA's barrier
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive_cluster(mapa_u32(smem_u32(&tempty[acc]), 0u));
+    }
+  }
+  __syncthreads();
+  if (*abort_flag && threadIdx.x == 0 && xr == 0) {
+    // no bulk copy may still be landing when the pair exits (the even CTA's barriers count both CTAs' bytes)
+    for (int i = *n_consumed; i < *n_issued; i++) mbar_wait(&full[i % W_STAGES], (uint32_t)((i / W_STAGES) & 1));
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  cluster_sync_all();
+  if (warp == W_EPI_WARPS + 1) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512) : "memory");
+}
+
+int n_tiles_of(WideEpi epi, const int *O, int nw) {
+  if (epi == WIDE_SWIGLU) return (O[0] + 127) / 128;
+  int h = 0;
+  for (int j = 0; j < nw; j++) h += (O[j] + 127) / 128;
+  return (h + 1) / 2;
+}
+
+template <int EPI>
+int launch_wide(const WideParams &p, bool pdl, cudaStream_t s) {
+  static SmemLimit limit;
+  if (!limit.ensure(gemm_wide_kernel<EPI>, W_SMEM)) return -6;
+  if (!launch_allowed()) return 0;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(2 * std::min(W_PAIRS, p.m_tiles * p.n_tiles), 1, 1);
+  cfg.blockDim = dim3(W_THREADS, 1, 1);
+  cfg.dynamicSmemBytes = W_SMEM;
+  cfg.stream = s;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = 2; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = pdl ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, gemm_wide_kernel<EPI>, p) == cudaSuccess ? 0 : -6;
+}
+
+}  // namespace
+
+long long wide_gemm_cost(WideEpi epi, const int *O, int nw, int I, int row_tiles) {
+  const long long tiles = (long long)n_tiles_of(epi, O, nw) * row_tiles;
+  return (tiles + W_PAIRS - 1) / W_PAIRS * ((I + TILE_K - 1) / TILE_K);
+}
+
+int wide_gemm_launch(TmaMaps *g, WideEpi epi, const WideGemmArgs &a, cudaStream_t s) {
+  if (!g || a.rows < 1 || a.rows > a.x_rows || a.I < 8 || (a.I % 8) || ((uintptr_t)a.x & 15)) return -1;
+  if (a.nw < 1 || a.nw > 3 || (epi == WIDE_SWIGLU && (a.nw != 2 || a.O[0] != a.O[1])) || (epi == WIDE_QKV && a.nw < 2)) return -1;
+  WideParams p;
+  memset(&p, 0, sizeof p);
+  for (int j = 0; j < a.nw; j++) {
+    if (!a.w[j] || ((uintptr_t)a.w[j] & 15) || a.O[j] < 8 || (a.O[j] % 8)) return -1;
+    const CUtensorMap *mw = tma_maps_get(g, a.w[j], a.O[j], a.I, W_HALF);
+    if (!mw) return -6;
+    p.map_w[j] = *mw;
+    p.O[j] = a.O[j];
+  }
+  const CUtensorMap *mx = tma_maps_get(g, a.x, a.x_rows, a.I, W_HALF);
+  if (!mx) return -6;
+  p.map_x = *mx;
+  p.rows = a.rows; p.KB = (a.I + TILE_K - 1) / TILE_K;
+  p.m_tiles = (a.rows + WIDE_ROWS - 1) / WIDE_ROWS; p.n_tiles = n_tiles_of(epi, a.O, a.nw);
+  p.h0 = a.nw > 1 ? (a.O[0] + 127) / 128 : 1 << 30;
+  p.h1 = a.nw > 2 ? p.h0 + (a.O[1] + 127) / 128 : 1 << 30;
+  p.kind0 = a.nw == 3 ? 0 : 1;
+  p.ssq_in = a.ssq_in; p.ssq_in_tiles = a.ssq_in_tiles; p.ssq_ld = a.ssq_ld; p.inv_k_in = 1.0f / (float)a.k_in; p.eps = a.eps;
+  p.xres = a.xres; p.gain = a.gain; p.hb = a.hb; p.ssq_out = a.ssq_out; p.taps = a.taps; p.tap_mask = a.taps ? a.tap_mask : 0; p.resid_add = a.resid_add;
+  p.cs = a.cs; p.slot = a.slot; p.q = a.q; p.kp = (bf16 *)a.pool.k; p.vp = (bf16 *)a.pool.v; p.H = a.H; p.page_size = a.page_size;
+  p.act = a.act; p.out_b = a.out_b; p.ldo = a.ldo; p.status = a.status;
+  switch (epi) {
+    case WIDE_RESID: return launch_wide<WIDE_RESID>(p, a.pdl, s);
+    case WIDE_QKV: return launch_wide<WIDE_QKV>(p, a.pdl, s);
+    case WIDE_SWIGLU: return launch_wide<WIDE_SWIGLU>(p, a.pdl, s);
+    default: return launch_wide<WIDE_BF16>(p, a.pdl, s);
+  }
+}
+
+}  // namespace spec

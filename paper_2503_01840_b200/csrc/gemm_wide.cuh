@@ -1,0 +1,55 @@
+// GEMM for passes of hundreds to thousands of token rows (the prefill): host-side interface.
+#pragma once
+#include "tma_maps.cuh"
+
+namespace spec {
+
+enum WideEpi {
+  WIDE_RESID = 0,    // x[r][o] (+)= acc; hb = bf16(x * gain[o]); per-128-feature sums of squares; optional taps
+  WIDE_QKV = 1,      // scale, rotate q and k by the row's position, store q, write K/V into the paged cache (head_dim 128)
+  WIDE_SWIGLU = 2,   // two weights (gate, up): act = bf16(silu(scale*g) * scale*u)
+  WIDE_BF16 = 3      // out_b[r][o] = bf16(acc)
+};
+
+struct WideGemmArgs {
+  // out[r][o] = sum_i x[r][i] * w[o][i]; x has x_rows allocated rows of which the first `rows` are computed
+  const bf16 *x = nullptr;
+  int rows = 0, x_rows = 0, I = 0;
+  const bf16 *w[3] = {nullptr, nullptr, nullptr};   // [O[j]][I]
+  int O[3] = {0, 0, 0};
+  int nw = 1;
+  // per-row scale of the input: rsqrt(sum_t ssq_in[t * ssq_ld + r] / k_in + eps); nullptr: 1
+  const float *ssq_in = nullptr;
+  int ssq_in_tiles = 0, ssq_ld = 0, k_in = 1;
+  float eps = 0.0f;
+  // WIDE_RESID (O[0] = width of the residual stream)
+  float *xres = nullptr;
+  const bf16 *gain = nullptr;
+  bf16 *hb = nullptr;
+  float *ssq_out = nullptr;     // [ceil(O/128)][ssq_ld]
+  bf16 *taps = nullptr;         // [rows][3*O], slot s written when bit s of tap_mask is set
+  int tap_mask = 0;
+  int resid_add = 1;
+  // WIDE_QKV: w = {wq, wk, wv}, or {wk, wv} when only the cache is to be written (nw = 2)
+  const float2 *cs = nullptr;   // [rows][64] (cos, sin)
+  const int32_t *slot = nullptr;   // [rows] cache row page * G * page_size + offset of the row's K/V; -1: none is written
+  bf16 *q = nullptr;            // [rows][H][128]
+  KvPool pool = {nullptr, nullptr};
+  int H = 0, G = 0, page_size = 0;
+  // WIDE_SWIGLU
+  bf16 *act = nullptr;          // [rows][O[0]]
+  // WIDE_BF16
+  bf16 *out_b = nullptr;
+  int ldo = 0;
+  // launch
+  int32_t *status = nullptr;
+  bool pdl = false;
+};
+
+constexpr int WIDE_ROWS = 256;      // token rows per tile
+// waves of the launch on this chip times its k-blocks (64 elements): what the launch's time goes with
+long long wide_gemm_cost(WideEpi epi, const int *O, int nw, int I, int row_tiles);
+// Returns 0 or a negative code (-1: the shape does not fit).
+int wide_gemm_launch(TmaMaps *g, WideEpi epi, const WideGemmArgs &a, cudaStream_t s);
+
+}  // namespace spec
