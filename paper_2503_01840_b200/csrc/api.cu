@@ -394,7 +394,7 @@ static size_t wide_carve(const spec_ctx *c, WideBufs &w, void *base, int rows, s
 template <typename T> struct Sched {
   spec_ctx *c;
   cudaStream_t s;
-  explicit Sched(spec_ctx *ctx) : c(ctx), s(ctx->stream) { tl_pdl = c->fused && !(c->cfg.flags & SPEC_FLAG_NO_PDL); }
+  explicit Sched(spec_ctx *ctx) : c(ctx), s(ctx->stream) { tl_pdl = !(c->cfg.flags & SPEC_FLAG_NO_PDL); }
   ~Sched() { tl_pdl = false; }
   Sched(const Sched &) = delete;
   void tick(int n = 1) { c->launches += n; }
@@ -429,6 +429,13 @@ template <typename T> struct Sched {
     (void)S;
     launch_gemm_ref<T>((const T *)x, (const T *)w, out + col0, rows, O, I, ldo, s);
     tick();
+  }
+  // the same for weights that share their input, outputs side by side
+  void gemm_cat(const void *x, const void *w0, int O0, const void *w1, int O1, const void *w2, int O2, int nw, float *out, int rows, int I, int ldo) {
+    mark(SPEC_PROF_GEMM);
+    const T *const w[3] = {(const T *)w0, (const T *)w1, (const T *)w2};
+    const int O[3] = {O0, O1, O2};
+    tick(launch_gemm_ref_cat<T>((const T *)x, w, O, nw, out, rows, I, ldo, s));
   }
 
   // ---- fused bf16 path -----------------------------------------------------------------------
@@ -573,9 +580,7 @@ template <typename T> struct Sched {
                        c->cfg.rms_eps, (T *)c->h, nullptr, rows, rows, k, s);
     tick();
     c->np_qkv = pick(qd, k, 1); c->ps_qkv = pstride(qkvd);
-    gemm(c->h, w.wq, c->qkv, rows, qd, k, qkvd, 0, c->np_qkv);
-    gemm(c->h, w.wk, c->qkv, rows, kvd, k, qkvd, qd, c->np_qkv);
-    gemm(c->h, w.wv, c->qkv, rows, kvd, k, qkvd, qd + kvd, c->np_qkv);
+    gemm_cat(c->h, w.wq, qd, w.wk, kvd, w.wv, kvd, 3, c->qkv, rows, k, qkvd);
     mark(SPEC_PROF_ROPE_KV); launch_rope_kv<T>(c->qkv, c->np_qkv, c->ps_qkv, c->cs, c->meta, (T *)c->q, pool, pm, rows, c->H, c->G, c->hd, c->status, s);
     tick();
     attention(pool, rows, tail_len);
@@ -585,8 +590,7 @@ template <typename T> struct Sched {
                        (T *)c->h, nullptr, rows, rows, k, s);
     tick();
     c->np_gu = pick(F, k, 1); c->ps_gu = pstride(2 * F);
-    gemm(c->h, w.w_gate, c->gu, rows, F, k, 2 * F, 0, c->np_gu);
-    gemm(c->h, w.w_up, c->gu, rows, F, k, 2 * F, F, c->np_gu);
+    gemm_cat(c->h, w.w_gate, F, w.w_up, F, nullptr, 0, 2, c->gu, rows, k, 2 * F);
     mark(SPEC_PROF_ACT); launch_silu_mul<T>(c->gu, c->np_gu, c->ps_gu, (T *)c->act, rows, F, s);
     tick();
     c->np_proj = pick(k, F, 1); c->ps_proj = pstride(k);
@@ -599,8 +603,9 @@ template <typename T> struct Sched {
     return m;
   }
 
-  // target forward over the rows of c->meta: taps -> node_taps, argmax -> tb.y
-  void target_forward(int rows, int tail_len, bool want_logits) {
+  // target forward over the rows of c->meta: taps -> node_taps, argmax -> tb.y (only_row >= 0: of that row alone, where the
+  // plain schedule can leave the others out)
+  void target_forward(int rows, int tail_len, bool want_logits, int only_row = -1) {
     if (c->fused) return target_forward_fused(rows, tail_len, want_logits);
     mark(SPEC_PROF_MISC); launch_rope_table(c->meta.pos, rows, c->hd / 2, c->inv_freq, c->cs, s); tick();
     mark(SPEC_PROF_MISC); launch_embed<T>((const T *)c->embed, c->meta.tok, c->x, rows, c->k, s); tick();
@@ -610,8 +615,10 @@ template <typename T> struct Sched {
                        (const T *)c->final_norm, c->cfg.rms_eps, (T *)c->h, nullptr, rows, rows, c->k, s);
     tick();
     if (want_logits) {
-      gemm(c->h, c->lm_head, c->logits, rows, c->V, c->k, c->V, 0, 1);
-      mark(SPEC_PROF_ARGMAX); launch_argmax(c->logits, rows, c->V, c->tb.y, s); tick();
+      const int r0 = only_row >= 0 ? only_row : 0, nr = only_row >= 0 ? 1 : rows;
+      float *lg = c->logits + (size_t)r0 * c->V;
+      gemm((const T *)c->h + (size_t)r0 * c->k, c->lm_head, lg, nr, c->V, c->k, c->V, 0, 1);
+      mark(SPEC_PROF_ARGMAX); launch_argmax(lg, nr, c->V, c->tb.y + r0, s); tick();
     }
   }
 
@@ -864,7 +871,8 @@ static int read_status(spec_ctx *c) {
 template <typename T> static int prefill_blocks(spec_ctx *c, const int32_t *lens, int32_t *root_host) {
   cudaStream_t s = c->stream;
   Sched<T> sc(c);
-  const int B = c->B, CH = PREFILL_CHUNK;
+  const int B = c->B;
+  int CH = PREFILL_CHUNK;                  // rows of the pass
   auto upload_meta = [&](int nvalid, int b, int start, const int32_t *toks_dev) -> cudaError_t {
     launch_prefill_meta(c->meta, toks_dev, b, start, nvalid, CH, PREFILL_BLOCK, s);
     sc.tick();
@@ -873,13 +881,16 @@ template <typename T> static int prefill_blocks(spec_ctx *c, const int32_t *lens
   size_t off = 0;
   for (int b = 0; b < B; b++) {
     int n = lens[b];
-    for (int start = 0; start < n; start += CH) {
-      int nv = std::min(CH, n - start);
+    for (int start = 0; start < n; start += PREFILL_CHUNK) {
+      int nv = std::min(PREFILL_CHUNK, n - start);
       bool last = start + nv == n;
+      // the fp32 schedule takes any number of rows (the metadata comes in 64s), the tile kernels whole blocks
+      const int unit = c->cfg.dtype == SPEC_F32 ? 64 : PREFILL_BLOCK;
+      CH = (nv + unit - 1) / unit * unit;
       CUDA_TRY(c, upload_meta(nv, b, start, c->prompt_dev + off + start));
       c->cur_rps = PREFILL_BLOCK;
       c->ctx_hint = start + CH - PREFILL_BLOCK;
-      sc.target_forward(CH, PREFILL_BLOCK, last);
+      sc.target_forward(CH, PREFILL_BLOCK, last, nv - 1);
       if (last) {
         // the last position stays pending: its taps become pending entry 0
         CUDA_TRY(c, cudaMemcpyAsync((char *)c->pend_taps + (size_t)b * c->Pmax * 3 * c->k * c->esz,

@@ -189,6 +189,11 @@ void launch_build_cat(const float *feat, int nparts, size_t part_stride, const i
 // ---------------------------------------------------------------- launchers (gemm_ref.cu)
 template <typename T>
 void launch_gemm_ref(const T *x, const T *w, float *out, int rows, int O, int I, int ldo, cudaStream_t s);
+template <> void launch_gemm_ref<float>(const float *x, const float *w, float *out, int rows, int O, int I, int ldo, cudaStream_t s);
+template <> void launch_gemm_ref<bf16>(const bf16 *x, const bf16 *w, float *out, int rows, int O, int I, int ldo, cudaStream_t s);
+// nw (2 or 3) weights that share the input, their outputs side by side in `out`; returns the number of kernels launched
+template <typename T>
+int launch_gemm_ref_cat(const T *x, const T *const (&w)[3], const int (&O)[3], int nw, float *out, int rows, int I, int ldo, cudaStream_t s);
 
 // ---------------------------------------------------------------- launchers (attn_ref.cu)
 template <typename T>

@@ -1,0 +1,56 @@
+"""The fp32 model's GEMM and attention kernels at the edges of their row groups, against fp64."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2503_01840_b200 import binding as sb
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("rows,O,I,shift", [(1, 1, 4, 0), (3, 31, 128, 0), (4, 256, 256, 0), (5, 33, 688, 0), (8, 8, 12, 0), (9, 1000, 260, 0),
+                                            (16, 100, 768, 0), (17, 65, 132, 0), (32, 7, 512, 0), (33, 300, 256, 0), (256, 64, 128, 0),
+                                            (257, 64, 128, 0), (64, 2049, 2052, 0), (4, 50, 30, 0), (4, 50, 32, 1)])
+def test_fp32_gemm_row_groups(rows, O, I, shift):
+    """Every row group of the warp-per-feature kernel, its remainders, and the shapes that stay on the tile kernel (a
+    contraction that is no multiple of four, operands off a 16-byte boundary, many rows of a large weight)."""
+    g = torch.Generator().manual_seed(rows * 1000 + O + I)
+    x, w = torch.randn(rows, I, generator=g), torch.randn(O, I, generator=g)
+
+    def dev(t):
+        buf = torch.empty(t.numel() + shift, device="cuda")
+        buf[shift:] = t.flatten().cuda()
+        return buf[shift:].view(t.shape)
+
+    out = sb.gemm(dev(x), dev(w), impl=1).cpu().double().numpy()
+    ref = x.double().numpy() @ w.double().numpy().T
+    bound = 2.0 ** -23 * (8 + I / 32) * (np.abs(x.double().numpy()) @ np.abs(w.double().numpy()).T)     # 32 partial sums of I / 32 products
+    assert (np.abs(out - ref) <= bound + 1e-30).all(), np.abs(out - ref).max()
+
+
+@pytest.mark.parametrize("H,G,hd,ctx,tail,ps", [(4, 2, 64, 0, 1, 16), (4, 2, 64, 70, 5, 16), (2, 2, 16, 31, 33, 8), (3, 1, 128, 129, 70, 32), (2, 1, 240, 40, 128, 16)])
+def test_fp32_attention_vs_fp64(H, G, hd, ctx, tail, ps):
+    rows = 5
+    g = torch.Generator().manual_seed(hd + ctx)
+    n = ctx + tail
+    pages = (n + ps - 1) // ps
+    q, k, v = torch.randn(rows, H, hd, generator=g), torch.randn(n, G, hd, generator=g), torch.randn(n, G, hd, generator=g)
+    perm = torch.randperm(pages + 1, generator=g)[:pages].to(torch.int32)
+    kp, vp = torch.zeros(pages + 1, G, ps, hd), torch.zeros(pages + 1, G, ps, hd)
+    for p in range(n):
+        kp[perm[p // ps], :, p % ps], vp[perm[p // ps], :, p % ps] = k[p], v[p]
+    bits = [int(b) for b in torch.randint(0, 2, (rows, 128), generator=g).flatten()]
+    mask = np.array(bits, bool).reshape(rows, 128)
+    mask[:, 0] = True
+    words = [[int(sum(1 << i for i in range(64) if mask[r, 64 * w + i])) for r in range(rows)] for w in (0, 1)]
+    lo, hi = (torch.tensor(np.array(w, np.uint64).view(np.int64)).cuda() for w in words)
+    full = lambda c: torch.full((rows,), c, dtype=torch.int32, device="cuda")
+    out = sb.attention(q.cuda(), kp.cuda(), vp.cuda(), perm.view(1, -1).cuda(), ps, full(0), full(ctx), full(ctx), lo, hi, tail, G, ctx + tail, impl=1)
+    vis = np.concatenate([np.ones((rows, ctx), bool), mask[:, :tail]], 1)
+    qd, kd, vd = q.double().numpy(), k.double().numpy(), v.double().numpy()
+    for h in range(H):
+        s = qd[:, h] @ kd[:, h // (H // G)].T / np.sqrt(hd)
+        s[~vis] = -np.inf
+        p = np.exp(s - s.max(1, keepdims=True))
+        ref = (p / p.sum(1, keepdims=True)) @ vd[:, h // (H // G)]
+        assert np.abs(out[:, h].cpu().double().numpy() - ref).max() < 5e-6          # scores of order 1 .. 3 in fp32, sums of ~200 terms
