@@ -448,10 +448,30 @@ template <typename T> struct Sched {
   void with_norm_scale(FusedGemmArgs &a) const {
     a.ssq_in = c->ssq; a.ssq_in_tiles = c->ktiles; a.ssq_ld = c->Ralloc; a.k_in = c->k; a.eps = c->cfg.rms_eps;
   }
+  // From 129 rows on (up to 256: batches, and whole trees at a small batch) a weight byte meets more flops than the
+  // weight-streaming kernel's tiles feed the tensor pipe with: it re-reads the 32 KB activation k-block for every 128
+  // features and spends as long in its 256-row epilogues as in its loops.  These passes take the row-major kernel.
+  bool row_major(FusedEpi epi, const FusedGemmArgs &a) const {
+    return a.rows > (epi == EPI_SWIGLU ? 192 : 128) && !a.withhold && !fused_gemm_pairs() && epi != EPI_TOPK && (epi != EPI_QKV || a.hd == 128);
+  }
+  static WideEpi wide_epi(FusedEpi e) {
+    return e == EPI_RESID ? WIDE_RESID : e == EPI_QKV ? WIDE_QKV : e == EPI_SWIGLU ? WIDE_SWIGLU : e == EPI_ARGMAX ? WIDE_ARGMAX : WIDE_F32;
+  }
+  static WideGemmArgs widened(const FusedGemmArgs &a) {
+    WideGemmArgs w;
+    w.x = a.x; w.rows = w.x_rows = a.rows; w.I = a.I; w.nw = a.nw;
+    for (int j = 0; j < 3; j++) { w.w[j] = a.w[j]; w.O[j] = a.O[j]; }
+    w.ssq_in = a.ssq_in; w.ssq_in_tiles = a.ssq_in_tiles; w.ssq_ld = a.ssq_ld; w.k_in = a.k_in; w.eps = a.eps;
+    w.xres = a.xres; w.gain = a.gain; w.hb = a.hb; w.ssq_out = a.ssq_out; w.taps = a.taps; w.tap_mask = a.tap_mask; w.resid_add = a.resid_add;
+    w.cs = a.cs; w.seq = a.m.seq; w.kvpos = a.m.kvpos; w.pm = a.pm; w.q = a.q; w.pool = a.pool; w.H = a.H; w.G = a.G; w.page_size = a.pm.page_size;
+    w.act = a.act; w.out_f32 = a.out_f32; w.ldo = a.ldo; w.best_val = a.best_val; w.best_idx = a.best_idx; w.best_ld = a.best_ld;
+    w.status = a.status; w.pdl = a.pdl; w.stamp = a.stamp;
+    return w;
+  }
   void fgemm(FusedEpi epi, FusedGemmArgs a) {
     prof_mark(SPEC_PROF_GEMM);
     a.stamp = next_stamp(SPEC_PROF_GEMM);
-    int rc = fused_gemm_launch(c->fg, epi, a, s);
+    int rc = row_major(epi, a) ? wide_gemm_launch(c->fg, wide_epi(epi), widened(a), s) : fused_gemm_launch(c->fg, epi, a, s);
     if (rc && !c->sched_err) c->sched_err = rc;
     tick();
   }
@@ -675,10 +695,7 @@ template <typename T> struct Sched {
     if (rc && !c->sched_err) c->sched_err = rc;
     tick();
   }
-  // The passes of up to 256 rows stay on the weight-streaming kernel (its launches split K, so a short pass still spreads
-  // over the chip: 139 us per layer of the 8B shapes at 256 rows, against 128 us plus a longer epilogue for a single row
-  // tile of the wide kernel); above, the wide kernel takes the pass in one sweep over the weights.
-  bool narrow(int rows) const { return rows <= 256; }
+  bool narrow(int rows) const { return rows <= 128; }      // see row_major()
   void pass_qkv(const WideBufs &w, const LayerW &lw, KvPool pool, int rows, bool draft) {
     const int qd = c->H * c->hd, kvd = c->G * c->hd;
     const PageMap pm{c->page_table, c->pps, c->cfg.page_size, c->cfg.num_pages};
@@ -704,7 +721,7 @@ template <typename T> struct Sched {
     wgemm(WIDE_QKV, a);
   }
   void pass_resid(const WideBufs &w, const void *in, int I, const void *wt, int rows, bool add, const void *gain, int tap_mask) {
-    if (narrow(rows)) {
+    if (rows <= 256) {          // fgemm chooses
       FusedGemmArgs a = fargs(in, rows, I);
       a.w[0] = (const bf16 *)wt; a.O[0] = c->k; a.nw = 1;
       a.xres = w.x; a.gain = (const bf16 *)gain; a.hb = w.h; a.ssq_out = w.ssq; a.ssq_ld = w.cap;
@@ -719,7 +736,7 @@ template <typename T> struct Sched {
     wgemm(WIDE_RESID, a);
   }
   void pass_swiglu(const WideBufs &w, const LayerW &lw, int rows) {
-    if (narrow(rows)) {
+    if (rows <= 256) {          // fgemm chooses
       FusedGemmArgs a = fargs(w.h, rows, c->k);
       a.w[0] = (const bf16 *)lw.w_gate; a.w[1] = (const bf16 *)lw.w_up; a.O[0] = c->F; a.O[1] = c->F; a.nw = 2;
       a.ssq_in = w.ssq; a.ssq_in_tiles = c->ktiles; a.ssq_ld = w.cap; a.k_in = c->k; a.eps = c->cfg.rms_eps;

@@ -1031,6 +1031,7 @@ void fused_gemm_set_target_ctas(int n) { g_target_ctas = n; }
 // 256-row tiles of neighbouring feature tiles as CTA pairs.  Bit 0: the split-K kernel (measured no faster: off); bit 1: the
 // gate/up kernel (gate/up launch -1 %, C3 step -0.6 %: on)
 namespace { int g_pairs = 0, g_pairs_swiglu = 1; }
+int fused_gemm_pairs() { return g_pairs; }
 void fused_gemm_set_pairs(int on) { g_pairs = on & 1; g_pairs_swiglu = (on >> 1) & 1; }
 
 int fused_gemm_tiles(FusedEpi epi, const FusedGemmArgs &a) {

@@ -54,11 +54,34 @@ struct alignas(64) WideParams {
   int kind0;                     // WIDE_QKV: what w0 is (0 q, 1 k)
   const float *ssq_in; int ssq_in_tiles, ssq_ld; float inv_k_in, eps;
   float *xres; const bf16 *gain; bf16 *hb; float *ssq_out; bf16 *taps; int tap_mask, resid_add;
-  const float2 *cs; const int32_t *slot; bf16 *q; bf16 *kp, *vp; int H, page_size;
+  const float2 *cs; const int32_t *slot, *seq, *kvpos; PageMap pm; bf16 *q; bf16 *kp, *vp; int H, G, page_size;
   bf16 *act;
   bf16 *out_b; int ldo;
+  float *out_f32;
+  float *best_val; int32_t *best_idx; int best_ld;
+  int fpt, stages;               // gate/up kernel with tiles of a chosen width: features per tile, ring stages
   int32_t *status;
+  unsigned long long *stamp;
 };
+
+// cache row of a row's K/V (-1: none); seq: the row's sequence, negative for padding (1 where the caller gave slots: a real row)
+__device__ __forceinline__ int row_slot(const WideParams &p, int row, int *seq) {
+  if (p.slot) { *seq = 1; return p.slot[row]; }
+  *seq = p.seq[row];
+  if (*seq < 0) return -1;
+  const int kvpos = p.kvpos[row];
+  if (kvpos < 0 || kvpos / p.pm.page_size >= p.pm.pages_per_seq) { set_status(p.status, ST_BOUNDS, 1, row, kvpos); return -1; }
+  const int page = p.pm.table[(size_t)*seq * p.pm.pages_per_seq + kvpos / p.pm.page_size];
+  if (page < 0 || page >= p.pm.num_pages) { set_status(p.status, ST_BOUNDS, 2, row, page); return -1; }
+  return page * p.G * p.pm.page_size + kvpos % p.pm.page_size;
+}
+__device__ __forceinline__ float row_scale(const WideParams &p, int row) {
+  if (!p.ssq_in) return 1.0f;
+  float ss = 0.0f;
+#pragma unroll 8
+  for (int u = 0; u < p.ssq_in_tiles; u++) ss += p.ssq_in[(size_t)u * p.ssq_ld + row];
+  return 1.0f / sqrtf(ss * p.inv_k_in + p.eps);
+}
 
 __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -195,8 +218,9 @@ __global__ void __launch_bounds__(W_THREADS, 1) gemm_wide_kernel(const __grid_co
           unsigned char *a = ring + st * W_STAGE;
           const uint32_t fb = mapa_u32(smem_u32(&full[st]), 0u);
           if (xr == 0) mbar_expect_tx(&full[st], 2 * W_STAGE);
-          tma_load_2d_pair_hint(a + W_A_BYTES, mw, kb * TILE_K, wrow, fb, pol);
-          tma_load_2d_pair(a, &p.map_x, kb * TILE_K, xrow, fb);
+          const int kx = kb * TILE_K;
+          tma_load_2d_pair_hint(a + W_A_BYTES, mw, kx, wrow, fb, pol);
+          tma_load_2d_pair(a, &p.map_x, kx, xrow, fb);
         }
         __syncwarp();
         issued++;
@@ -246,6 +270,7 @@ __global__ void __launch_bounds__(W_THREADS, 1) gemm_wide_kernel(const __grid_co
   } else {
     // ================================================================ epilogue: thread = token row, warp / 4 = half tile
     pdl_wait();
+    if (p.stamp && threadIdx.x == 0) atomicMin(p.stamp, global_ns());
     unsigned char *stg = stg_all + warp * W_STG;
     const int quarter = warp & 3, half = warp >> 2;
     const int sub = lane >> 3, c4 = (lane & 7) * 4;              // place in row-contiguous order: rows 4 i + sub, columns c4 ..
@@ -256,15 +281,9 @@ __global__ void __launch_bounds__(W_THREADS, 1) gemm_wide_kernel(const __grid_co
       const int row_w = mt * WIDE_ROWS + xr * W_HALF + quarter * 32;        // first row of the warp
       const int row = row_w + lane;
       const bool any_row = row_w < p.rows;
-      float inv = 1.0f;
-      if (p.ssq_in && row < p.rows) {
-        float ss = 0.0f;
-#pragma unroll 8
-        for (int u = 0; u < p.ssq_in_tiles; u++) ss += p.ssq_in[(size_t)u * p.ssq_ld + row];
-        inv = 1.0f / sqrtf(ss * p.inv_k_in + p.eps);
-      }
-      int slot = -1;
-      if (EPI == WIDE_QKV && row < p.rows) slot = p.slot[row];
+      const float inv = row < p.rows ? row_scale(p, row) : 1.0f;
+      int slot = -1, seq = -1;
+      if (EPI == WIDE_QKV && row < p.rows) slot = row_slot(p, row, &seq);
       // everything that does not depend on the accumulator is requested before the wait for it
       float4 xin[8];
       const int fo0 = nt * 256 + half * 128;                     // WIDE_RESID / WIDE_BF16: first feature of the warp
@@ -282,7 +301,7 @@ __global__ void __launch_bounds__(W_THREADS, 1) gemm_wide_kernel(const __grid_co
       }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t ta = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * 256);
-      if (EPI == WIDE_RESID || EPI == WIDE_BF16) {
+      if (EPI == WIDE_RESID || EPI == WIDE_BF16 || EPI == WIDE_F32) {
         float sq[8];
 #pragma unroll
         for (int i = 0; i < 8; i++) sq[i] = 0.0f;
@@ -294,7 +313,14 @@ __global__ void __launch_bounds__(W_THREADS, 1) gemm_wide_kernel(const __grid_co
           transpose32(stg, lane, v, a);
           const int f = fo0 + c * 32 + c4;
           const bool fok = f < p.O[0];
-          if (EPI == WIDE_BF16) {
+          if (EPI == WIDE_F32) {
+#pragma unroll
+            for (int i = 0; i < 8; i++) {
+              const int r = i * 4 + sub, gr = row_w + r;
+              const float sc = __shfl_sync(0xffffffffu, inv, r);
+              if (gr < p.rows && fok) *(float4 *)(p.out_f32 + (size_t)gr * p.ldo + f) = make_float4(a[i].x * sc, a[i].y * sc, a[i].z * sc, a[i].w * sc);
+            }
+          } else if (EPI == WIDE_BF16) {
 #pragma unroll
             for (int i = 0; i < 8; i++) {
               const int gr = row_w + i * 4 + sub;
@@ -378,6 +404,44 @@ __global__ void __launch_bounds__(W_THREADS, 1) gemm_wide_kernel(const __grid_co
             *(uint4 *)(p.act + (size_t)gr * p.O[0] + f) = *(const uint4 *)(stg + r * 128 + (((lane & 7) ^ (r & 7)) << 4));
         }
         __syncwarp();
+      } else if (EPI == WIDE_ARGMAX) {
+        // the thread scans its row's 128 features in order: the first of equal values wins (lowest index)
+        const int f0 = nt * 256 + half * 128;
+        float bv = 0.0f;
+        int bi = -1;
+#pragma unroll
+        for (int c = 0; c < 4; c++) {
+          uint32_t v[32];
+          tmem_ld32(ta + half * 128 + c * 32, v);
+#pragma unroll
+          for (int e = 0; e < 32; e++) {
+            const float x = __uint_as_float(v[e]);
+            const bool better = f0 + c * 32 + e < p.O[0] && (bi < 0 || x > bv);
+            bv = better ? x : bv;
+            bi = better ? f0 + c * 32 + e : bi;
+          }
+          if (p.out_f32) {
+            float4 a[8];
+            transpose32(stg, lane, v, a);
+            const int f = f0 + c * 32 + c4;
+#pragma unroll
+            for (int i = 0; i < 8; i++) {
+              const int r = i * 4 + sub, gr = row_w + r;
+              const float sc = __shfl_sync(0xffffffffu, inv, r);
+              if (gr < p.rows && f < p.O[0]) {
+                float *dst = p.out_f32 + (size_t)gr * p.ldo + f;
+                const float o[4] = {a[i].x * sc, a[i].y * sc, a[i].z * sc, a[i].w * sc};
+#pragma unroll
+                for (int z = 0; z < 4; z++)
+                  if (f + z < p.O[0]) dst[z] = o[z];
+              }
+            }
+          }
+        }
+        if (row < p.rows && f0 < p.O[0]) {
+          p.best_val[(size_t)(f0 >> 7) * p.best_ld + row] = bv;
+          p.best_idx[(size_t)(f0 >> 7) * p.best_ld + row] = bi;
+        }
       } else {   // WIDE_QKV: the half tile is one head of q, k or v
         int mi = 0, tm = 2 * nt + half;
         if (tm >= p.h1) { mi = 2; tm -= p.h1; }
@@ -399,7 +463,7 @@ __global__ void __launch_bounds__(W_THREADS, 1) gemm_wide_kernel(const __grid_co
           for (int i = 0; i < 8; i++) {
             const int r = i * 4 + sub, gr = row_w + r;
             const float sc = __shfl_sync(0xffffffffu, inv, r);
-            const int sl = __shfl_sync(0xffffffffu, slot, r);
+            const int sl = __shfl_sync(0xffffffffu, slot, r), sq = __shfl_sync(0xffffffffu, seq, r);
             if (gr >= p.rows || !head_ok) continue;
             float4 lo = make_float4(a[i].x * sc, a[i].y * sc, a[i].z * sc, a[i].w * sc);
             float4 hi = make_float4(b[i].x * sc, b[i].y * sc, b[i].z * sc, b[i].w * sc);
@@ -410,8 +474,10 @@ __global__ void __launch_bounds__(W_THREADS, 1) gemm_wide_kernel(const __grid_co
               hi = make_float4(h.x * c0.x + l.x * c0.y, h.y * c0.z + l.y * c0.w, h.z * c1.x + l.z * c1.y, h.w * c1.z + l.w * c1.w);
             }
             bf16 *dst = nullptr;
-            if (kind == 0) dst = p.q + ((size_t)gr * p.H + tm) * 128;
-            else if (sl >= 0) dst = kv + ((size_t)sl + (size_t)tm * p.page_size) * 128;
+            if (kind == 0) {
+              dst = p.q + ((size_t)gr * p.H + tm) * 128;
+              if (sq < 0) lo = hi = make_float4(0.f, 0.f, 0.f, 0.f);      // padding row
+            } else if (sl >= 0) dst = kv + ((size_t)sl + (size_t)tm * p.page_size) * 128;
             if (dst) {
               *(uint2 *)(dst + c * 32 + c4) = pack4(lo);
               *(uint2 *)(dst + 64 + c * 32 + c4) = pack4(hi);
@@ -433,6 +499,438 @@ __global__ void __launch_bounds__(W_THREADS, 1) gemm_wide_kernel(const __grid_co
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   cluster_sync_all();
   if (warp == W_EPI_WARPS + 1) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512) : "memory");
+  if (p.stamp && threadIdx.x == 0) atomicMin(p.stamp + 1, ~global_ns());
+}
+
+// ------------------------------------------------------------------------------------------------
+// The same contraction with the K range split over S CTA pairs, for launches that have fewer tiles than the chip has pairs
+// (16 tiles of a 4096-wide residual at 256 rows): the 2 S CTAs of a tile are one cluster (rank = position in the pair + 2 x
+// slice).  Every CTA parks its accumulator (128 rows x 256 features, fp32, 128 KB) in its own shared memory, which the ring
+// no longer needs, and takes an S-th of its ROWS from all slices through distributed shared memory, in slice order
+// (deterministic); a warp handles one row of a half tile per step, a lane four consecutive features, so the epilogue's
+// global accesses are whole rows of 256 or 512 bytes, the row's sum of squares is one warp sum, and RoPE's partner feature
+// is sixteen lanes away.
+constexpr int WS_DUMP = 2 * W_HALF * W_HALF * 4;               // 128 KB
+constexpr int WS_SMEM = W_STAGES * W_STAGE + 2 * W_HALF * 4 + W_HALF * 4 + W_CTRL + 1024;
+constexpr int WS_EPI_WARPS = 16, WS_THREADS = (WS_EPI_WARPS + 2) * 32;      // parking and reduction are latency chains: 16 warps, not 8
+static_assert(WS_DUMP <= W_STAGES * W_STAGE, "the accumulator is parked in the ring");
+
+__device__ __forceinline__ float4 ld_peer4(uint32_t local_addr, uint32_t rank) {      // several may be in flight (no memory clobber)
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(mapa_u32(local_addr, rank)));
+  return v;
+}
+
+template <int EPI, int S>
+__global__ void __launch_bounds__(WS_THREADS, 1) gemm_wide_split_kernel(const __grid_constant__ WideParams p) {
+  extern __shared__ unsigned char smem_raw[];
+  unsigned char *ring = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  float *inv_s = (float *)(ring + W_STAGES * W_STAGE);         // [128] scale of this CTA's rows
+  int *slot_s = (int *)(inv_s + W_HALF), *seq_s = slot_s + W_HALF;
+  uint64_t *full = (uint64_t *)(seq_s + W_HALF);
+  uint64_t *empty = full + W_STAGES;
+  uint64_t *acc_bar = empty + W_STAGES;
+  uint32_t *tmem_slot = (uint32_t *)(acc_bar + 1);
+  volatile uint32_t *abort_flag = tmem_slot + 1;
+  volatile int *n_issued = (volatile int *)(tmem_slot + 2), *n_consumed = (volatile int *)(tmem_slot + 3);
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  uint32_t crank;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(crank));
+  const int xr = (int)(crank & 1u), slice = (int)(crank >> 1);
+  const uint32_t lead = crank & ~1u;
+  const int t = blockIdx.x / (2 * S), mt = t % p.m_tiles, nt = t / p.m_tiles;
+  const int kb0 = (int)(((long long)slice * p.KB) / S), kb1 = (int)(((long long)(slice + 1) * p.KB) / S), nkb = kb1 - kb0;
+  const int row_c = mt * WIDE_ROWS + xr * W_HALF;              // first row of this CTA
+  const int nrow = min(max(p.rows - row_c, 0), W_HALF);
+
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < W_STAGES; i++) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
+    mbar_init(acc_bar, 1);
+    *abort_flag = 0;
+    *n_issued = 0; *n_consumed = 0;
+    if ((int)crank != (int)(blockIdx.x % (2u * (unsigned)S))) { *abort_flag = 1; set_status(p.status, ST_TIMEOUT, 254, blockIdx.x, (int)crank); }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == WS_EPI_WARPS + 1) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(256) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  cluster_sync_all();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem_base = *tmem_slot;
+  pdl_trigger();
+
+  if (warp == WS_EPI_WARPS) {
+    // ---- producer: own rows and own half of the features; all bytes are counted on the even CTA's barrier
+    int mi = 0, tm = 2 * nt + xr;
+    if (tm >= p.h1) { mi = 2; tm -= p.h1; }
+    else if (tm >= p.h0) { mi = 1; tm -= p.h0; }
+    const CUtensorMap *mw = &p.map_w[mi];
+    const uint64_t pol = l2_policy_evict_first();
+    const int npre = *abort_flag ? 0 : nkb < W_STAGES ? nkb : W_STAGES;
+    if (elect_one())
+      for (int i = 0; i < npre; i++) {
+        if (xr == 0) mbar_expect_tx(&full[i], 2 * W_STAGE);
+        tma_load_2d_pair_hint(ring + i * W_STAGE + W_A_BYTES, mw, (kb0 + i) * TILE_K, tm * W_HALF, mapa_u32(smem_u32(&full[i]), lead), pol);
+      }
+    __syncwarp();
+    pdl_wait();
+    if (elect_one()) {
+      if (p.stamp) atomicMin(p.stamp, global_ns());
+      for (int i = 0; i < npre; i++) tma_load_2d_pair(ring + i * W_STAGE, &p.map_x, (kb0 + i) * TILE_K, row_c, mapa_u32(smem_u32(&full[i]), lead));
+    }
+    __syncwarp();
+    int i = npre, st = 0;
+    uint32_t ph = 0;
+    if (!*abort_flag)
+      for (; i < nkb; i++) {
+        if (!mbar_wait_warp(&empty[st], ph)) { *abort_flag = 1; set_status(p.status, ST_TIMEOUT, 250, blockIdx.x, i); break; }
+        if (elect_one()) {
+          unsigned char *a = ring + st * W_STAGE;
+          const uint32_t fb = mapa_u32(smem_u32(&full[st]), lead);
+          if (xr == 0) mbar_expect_tx(&full[st], 2 * W_STAGE);
+          const int kx = (kb0 + i) * TILE_K;
+          tma_load_2d_pair_hint(a + W_A_BYTES, mw, kx, tm * W_HALF, fb, pol);
+          tma_load_2d_pair(a, &p.map_x, kx, row_c, fb);
+        }
+        __syncwarp();
+        if (++st == W_STAGES) { st = 0; ph ^= 1u; }
+      }
+    if (lane == 0) *n_issued = i;
+  } else if (warp == WS_EPI_WARPS + 1) {
+    pdl_wait();
+    if (xr == 0 && !*abort_flag) {
+      constexpr uint32_t idesc = umma_idesc_m(256, 256);
+      uint32_t partner_base;
+      asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(partner_base) : "r"(mapa_u32(smem_u32(tmem_slot), crank | 1u)) : "memory");
+      bool ok = partner_base == tmem_base;
+      if (!ok) { *abort_flag = 1; set_status(p.status, ST_TIMEOUT, 253, blockIdx.x, (int)partner_base); }
+      const uint64_t desc0 = umma_desc_sw128(smem_u32(ring));
+      int i = 0, st = 0;
+      uint32_t ph = 0, ready = 0;
+      for (; ok && i < nkb; i++) {
+        if (!ready && !mbar_wait_warp(&full[st], ph)) { *abort_flag = 1; set_status(p.status, ST_TIMEOUT, 251, blockIdx.x, i); ok = false; break; }
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint64_t da = desc0 + (uint64_t)((st * W_STAGE) >> 4), db = da + (W_A_BYTES >> 4);
+        int nst = st + 1;
+        uint32_t nph = ph;
+        if (nst == W_STAGES) { nst = 0; nph ^= 1u; }
+        if (elect_one()) {
+#pragma unroll
+          for (int j = 0; j < TILE_K / UMMA_K; j++) umma_bf16_pair(tmem_base, da + 2 * j, db + 2 * j, idesc, (i | j) ? 1u : 0u);
+          umma_commit_pair(&empty[st], lead);
+        }
+        __syncwarp();
+        ready = mbar_test_warp(&full[nst], nph) ? 1u : 0u;
+        st = nst; ph = nph;
+      }
+      if (lane == 0) *n_consumed = i;
+      __syncwarp();
+      if (ok && elect_one()) umma_commit_pair(acc_bar, lead);
+    }
+  } else {
+    pdl_wait();
+    if ((int)threadIdx.x < nrow) {                             // per-row values of this CTA's rows
+      inv_s[threadIdx.x] = row_scale(p, row_c + threadIdx.x);
+      if (EPI == WIDE_QKV) {
+        int seq;
+        slot_s[threadIdx.x] = row_slot(p, row_c + threadIdx.x, &seq);
+        seq_s[threadIdx.x] = seq;
+      }
+    }
+    // ---- accumulator -> shared memory: [half][row][128 floats], 16-byte chunks swizzled by the row
+    const bool ok = mbar_wait_warp(acc_bar, 0) && !*abort_flag;
+    if (!ok) {
+      if (lane == 0 && !*abort_flag) set_status(p.status, ST_TIMEOUT, 252, blockIdx.x, slice);
+      *abort_flag = 1;
+    } else {
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const int r = (warp & 3) * 32 + lane, half = warp >> 3, c0 = (warp >> 2 & 1) * 2;      // four warps per quarter: 64 columns each
+      unsigned char *dst = ring + (half * W_HALF + r) * 512;
+#pragma unroll
+      for (int c = 0; c < 2; c++) {
+        uint32_t v[32];
+        tmem_ld32(tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + half * 128 + (c0 + c) * 32, v);
+#pragma unroll
+        for (int j = 0; j < 8; j++)
+          *(uint4 *)(dst + ((((c0 + c) * 8 + j) ^ (r & 7)) << 4)) = make_uint4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+      }
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  cluster_sync_all();
+  const bool good = !*abort_flag;                              // (a CTA that gave up stores nothing; its peers read stale sums, the status says so)
+
+  if (warp < WS_EPI_WARPS) {
+    const int per = (nrow + S - 1) / S, r0 = min(slice * per, nrow), r1 = min(r0 + per, nrow);
+    const int half = warp & 1, sub = warp >> 1;                // eight warps per half tile, every eighth row each
+    const int fo = nt * 256 + half * 128 + lane * 4;           // WIDE_RESID / WIDE_F32: first of the lane's features
+    int mi = 0, tm = 2 * nt + half;
+    if (EPI == WIDE_QKV) {
+      if (tm >= p.h1) { mi = 2; tm -= p.h1; }
+      else if (tm >= p.h0) { mi = 1; tm -= p.h0; }
+    }
+    const int kind = mi + p.kind0;
+    const bool fok = good && (EPI == WIDE_QKV ? tm * 128 < p.O[mi] : fo < p.O[0]);
+    float4 gn = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (EPI == WIDE_RESID && fok) {
+      const uint2 g = *(const uint2 *)(p.gain + fo);
+      const float2 g01 = __bfloat1622float2(*(const __nv_bfloat162 *)&g.x), g23 = __bfloat1622float2(*(const __nv_bfloat162 *)&g.y);
+      gn = make_float4(g01.x, g01.y, g23.x, g23.y);
+    }
+    constexpr int RB = S == 3 ? 6 : 4;                         // rows in flight per warp: a full tile's share in one or two batches
+    for (int rb = r0 + sub; rb < r1; rb += 8 * RB) {
+      float4 xin[RB];
+#pragma unroll
+      for (int j = 0; j < RB; j++) {
+        const int r = rb + 8 * j;
+        xin[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (EPI == WIDE_RESID && p.resid_add && fok && r < r1) xin[j] = *(const float4 *)(p.xres + (size_t)(row_c + r) * p.O[0] + fo);
+      }
+      float4 v[S][RB];                                         // every remote load of the batch is in flight before the first sum
+#pragma unroll
+      for (int s = 0; s < S; s++)
+#pragma unroll
+        for (int j = 0; j < RB; j++) {
+          const int r = min(rb + 8 * j, r1 - 1);
+          v[s][j] = ld_peer4(smem_u32(ring + (half * W_HALF + r) * 512 + ((lane ^ (r & 7)) << 4)), (uint32_t)(xr + 2 * s));
+        }
+#pragma unroll
+      for (int s = 1; s < S; s++)
+#pragma unroll
+        for (int j = 0; j < RB; j++) { v[0][j].x += v[s][j].x; v[0][j].y += v[s][j].y; v[0][j].z += v[s][j].z; v[0][j].w += v[s][j].w; }
+#pragma unroll
+      for (int j = 0; j < RB; j++) {
+        const int r = rb + 8 * j, gr = row_c + r;
+        if (r >= r1) continue;                                 // uniform over the warp
+        float4 o = v[0][j];
+        if (EPI == WIDE_RESID) {
+          float sq = 0.0f;
+          if (fok) {
+            o.x += xin[j].x; o.y += xin[j].y; o.z += xin[j].z; o.w += xin[j].w;
+            const size_t xi = (size_t)gr * p.O[0] + fo;
+            *(float4 *)(p.xres + xi) = o;
+            *(uint2 *)(p.hb + xi) = pack4(make_float4(o.x * gn.x, o.y * gn.y, o.z * gn.z, o.w * gn.w));
+            if (p.tap_mask) {
+              const uint2 tb = pack4(o);
+#pragma unroll
+              for (int s = 0; s < 3; s++)
+                if ((p.tap_mask >> s) & 1) *(uint2 *)(p.taps + (size_t)gr * 3 * p.O[0] + (size_t)s * p.O[0] + fo) = tb;
+            }
+            sq = (o.x * o.x + o.y * o.y) + (o.z * o.z + o.w * o.w);
+          }
+          for (int off = 16; off > 0; off >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, off);
+          if (lane == 0 && fok) p.ssq_out[(size_t)(fo >> 7) * p.ssq_ld + gr] = sq;
+        } else if (EPI == WIDE_QKV) {
+          const float sc = inv_s[r];
+          const int sl = slot_s[r], sq = seq_s[r];
+          o.x *= sc; o.y *= sc; o.z *= sc; o.w *= sc;
+          float4 w;                                            // the partner features (i ^ 64): lane ^ 16
+          w.x = __shfl_xor_sync(0xffffffffu, o.x, 16); w.y = __shfl_xor_sync(0xffffffffu, o.y, 16);
+          w.z = __shfl_xor_sync(0xffffffffu, o.z, 16); w.w = __shfl_xor_sync(0xffffffffu, o.w, 16);
+          if (!fok) continue;
+          if (kind < 2) {
+            const float4 c0 = *(const float4 *)(p.cs + (size_t)gr * 64 + (lane & 15) * 4), c1 = *(const float4 *)(p.cs + (size_t)gr * 64 + (lane & 15) * 4 + 2);
+            if (lane < 16) o = make_float4(o.x * c0.x - w.x * c0.y, o.y * c0.z - w.y * c0.w, o.z * c1.x - w.z * c1.y, o.w * c1.z - w.w * c1.w);
+            else o = make_float4(o.x * c0.x + w.x * c0.y, o.y * c0.z + w.y * c0.w, o.z * c1.x + w.z * c1.y, o.w * c1.z + w.w * c1.w);
+          }
+          if (kind == 0) {
+            if (sq < 0) o = make_float4(0.f, 0.f, 0.f, 0.f);   // padding row
+            *(uint2 *)(p.q + ((size_t)gr * p.H + tm) * 128 + lane * 4) = pack4(o);
+          } else if (sl >= 0) {
+            *(uint2 *)((kind == 1 ? p.kp : p.vp) + ((size_t)sl + (size_t)tm * p.page_size) * 128 + lane * 4) = pack4(o);
+          }
+        } else if (fok) {                                      // WIDE_F32
+          const float sc = inv_s[r];
+          *(float4 *)(p.out_f32 + (size_t)gr * p.ldo + fo) = make_float4(o.x * sc, o.y * sc, o.z * sc, o.w * sc);
+        }
+      }
+    }
+  }
+  if (*abort_flag && threadIdx.x == 0 && xr == 0)              // no bulk copy may still be landing when the cluster exits
+    for (int i = *n_consumed; i < *n_issued; i++) mbar_wait(&full[i % W_STAGES], (uint32_t)((i / W_STAGES) & 1));
+  cluster_sync_all();                                          // peers may still be reading this CTA's accumulator
+  if (warp == WS_EPI_WARPS + 1) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(256) : "memory");
+  if (p.stamp && threadIdx.x == 0) atomicMin(p.stamp + 1, ~global_ns());
+}
+
+// ------------------------------------------------------------------------------------------------
+// Gate/up GEMM with tiles of a chosen width: 2 x fpt accumulator columns (gate, up) per CTA pair instead of 2 x 128.  The
+// 112 tiles of the 8B shapes are 1.5 waves of 74 pairs at one row tile, i.e. two; 69 tiles of 208 features are one, a k-block
+// then costs 832 tensor cycles instead of 2 x 512 and the activations are read 69 times instead of 112.  Two accumulators of
+// this width fill the tensor memory, so the epilogue is not hidden by a next tile: taken only where the waves say so
+// (plan_swiglu).  A thread of the epilogue owns a row and writes 16 features = one 32-byte sector at a time.
+constexpr int WG_MAX_FPT = 256;
+__global__ void __launch_bounds__(WS_THREADS, 1) gemm_wide_swiglu_kernel(const __grid_constant__ WideParams p) {
+  extern __shared__ unsigned char smem_raw[];
+  unsigned char *ring = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  const int fpt = p.fpt, b_bytes = fpt / 2 * 128, stage = W_A_BYTES + 2 * b_bytes, stages = p.stages;
+  uint64_t *full = (uint64_t *)(ring + stages * stage);
+  uint64_t *empty = full + 8, *tfull = empty + 8, *tempty = tfull + 1;
+  uint32_t *tmem_slot = (uint32_t *)(tempty + 1);
+  volatile uint32_t *abort_flag = tmem_slot + 1;
+  volatile int *n_issued = (volatile int *)(tmem_slot + 2), *n_consumed = (volatile int *)(tmem_slot + 3);
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  uint32_t crank;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(crank));
+  const int xr = (int)(crank & 1u);
+  const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
+  const int ntiles = p.m_tiles * p.n_tiles, KB = p.KB;
+
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < stages; i++) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
+    mbar_init(tfull, 1);
+    mbar_init(tempty, 2 * WS_EPI_WARPS);
+    *abort_flag = 0;
+    *n_issued = 0; *n_consumed = 0;
+    if (crank != (blockIdx.x & 1u)) { *abort_flag = 1; set_status(p.status, ST_TIMEOUT, 264, blockIdx.x, (int)crank); }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == WS_EPI_WARPS + 1) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(512) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  cluster_sync_all();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem_base = *tmem_slot;
+  pdl_trigger();
+
+  if (warp == WS_EPI_WARPS) {
+    // ---- producer: own rows, and the own half of the tile's gate and up features
+    const uint64_t pol = l2_policy_evict_first();
+    int issued = 0, st = 0;
+    uint32_t ph = 1;
+    bool ok = !*abort_flag, first = true;
+    for (int t = pair; t < ntiles && ok; t += n_pairs) {
+      const int mt = t % p.m_tiles, nt = t / p.m_tiles;
+      const int wrow = nt * fpt + xr * (fpt / 2), xrow = mt * WIDE_ROWS + xr * W_HALF;
+      int kb = 0;
+      if (first) {
+        first = false;
+        const int npre = KB < stages ? KB : stages;
+        if (elect_one())
+          for (int i = 0; i < npre; i++) {
+            const uint32_t fb = mapa_u32(smem_u32(&full[i]), 0u);
+            if (xr == 0) mbar_expect_tx(&full[i], 2 * stage);
+            tma_load_2d_pair_hint(ring + i * stage + W_A_BYTES, &p.map_w[0], i * TILE_K, wrow, fb, pol);
+            tma_load_2d_pair_hint(ring + i * stage + W_A_BYTES + b_bytes, &p.map_w[1], i * TILE_K, wrow, fb, pol);
+          }
+        __syncwarp();
+        pdl_wait();
+        if (elect_one())
+          for (int i = 0; i < npre; i++) tma_load_2d_pair(ring + i * stage, &p.map_x, i * TILE_K, xrow, mapa_u32(smem_u32(&full[i]), 0u));
+        __syncwarp();
+        kb = npre; issued = npre;
+        if (npre == stages) ph = 0; else st = npre;
+      }
+      for (; kb < KB; kb++) {
+        if (!mbar_wait_warp(&empty[st], ph)) { *abort_flag = 1; set_status(p.status, ST_TIMEOUT, 260, blockIdx.x, t); ok = false; break; }
+        if (elect_one()) {
+          unsigned char *a = ring + st * stage;
+          const uint32_t fb = mapa_u32(smem_u32(&full[st]), 0u);
+          if (xr == 0) mbar_expect_tx(&full[st], 2 * stage);
+          const int kx = kb * TILE_K;
+          tma_load_2d_pair_hint(a + W_A_BYTES, &p.map_w[0], kx, wrow, fb, pol);
+          tma_load_2d_pair_hint(a + W_A_BYTES + b_bytes, &p.map_w[1], kx, wrow, fb, pol);
+          tma_load_2d_pair(a, &p.map_x, kx, xrow, fb);
+        }
+        __syncwarp();
+        issued++;
+        if (++st == stages) { st = 0; ph ^= 1u; }
+      }
+    }
+    if (first) pdl_wait();
+    if (lane == 0) *n_issued = issued;
+  } else if (warp == WS_EPI_WARPS + 1) {
+    pdl_wait();
+    if (xr == 0 && !*abort_flag) {
+      const uint32_t idesc = umma_idesc_m(fpt, 256);
+      const uint64_t desc0 = umma_desc_sw128(smem_u32(ring));
+      int consumed = 0, st = 0, it = 0;
+      uint32_t ph = 0, ready = 0;
+      bool ok = true;
+      for (int t = pair; t < ntiles && ok; t += n_pairs, it++) {
+        if (it > 0) {
+          const bool w = mbar_wait_cluster(tempty, (uint32_t)((it - 1) & 1));
+          if (!__all_sync(0xffffffffu, w)) { *abort_flag = 1; set_status(p.status, ST_TIMEOUT, 261, blockIdx.x, t); break; }
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        }
+        for (int kb = 0; kb < KB; kb++) {
+          if (!ready && !mbar_wait_warp(&full[st], ph)) { *abort_flag = 1; set_status(p.status, ST_TIMEOUT, 262, blockIdx.x, t); ok = false; break; }
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const uint64_t da = desc0 + (uint64_t)((st * stage) >> 4), dg = da + (W_A_BYTES >> 4), du = dg + (uint64_t)(b_bytes >> 4);
+          int nst = st + 1;
+          uint32_t nph = ph;
+          if (nst == stages) { nst = 0; nph ^= 1u; }
+          if (elect_one()) {
+#pragma unroll
+            for (int j = 0; j < TILE_K / UMMA_K; j++) {
+              umma_bf16_pair(tmem_base, da + 2 * j, dg + 2 * j, idesc, (kb | j) ? 1u : 0u);
+              umma_bf16_pair(tmem_base + 256, da + 2 * j, du + 2 * j, idesc, (kb | j) ? 1u : 0u);
+            }
+            umma_commit_pair(&empty[st], 0u);
+            if (kb == KB - 1) umma_commit_pair(tfull, 0u);
+          }
+          __syncwarp();
+          consumed++;
+          ready = mbar_test_warp(&full[nst], nph) ? 1u : 0u;
+          st = nst; ph = nph;
+        }
+      }
+      if (lane == 0) *n_consumed = consumed;
+    }
+  } else {
+    pdl_wait();
+    if (p.stamp && threadIdx.x == 0) atomicMin(p.stamp, global_ns());
+    const int quarter = warp & 3, part = warp >> 2;
+    int it = 0;
+    for (int t = pair; t < ntiles; t += n_pairs, it++) {
+      const int mt = t % p.m_tiles, nt = t / p.m_tiles;
+      const int row = mt * WIDE_ROWS + xr * W_HALF + quarter * 32 + lane;
+      const float inv = row < p.rows ? row_scale(p, row) : 1.0f;
+      const bool ok = mbar_wait_warp(tfull, (uint32_t)(it & 1));
+      if (!ok || *abort_flag) {
+        if (!ok && lane == 0) { *abort_flag = 1; set_status(p.status, ST_TIMEOUT, 263, blockIdx.x, t); }
+        break;
+      }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t ta = tmem_base + ((uint32_t)(quarter * 32) << 16);
+#pragma unroll 1
+      for (int c = part; c < fpt / 16; c += 4) {                 // the four warps of a quarter take alternate runs of 16 features
+        uint32_t g[16], u[16], w[8];
+        tmem_ld16(ta + c * 16, g);
+        tmem_ld16(ta + 256 + c * 16, u);
+#pragma unroll
+        for (int e = 0; e < 8; e++) {
+          float r[2];
+#pragma unroll
+          for (int z = 0; z < 2; z++) {
+            const float gv = __uint_as_float(g[2 * e + z]) * inv, uv = __uint_as_float(u[2 * e + z]) * inv;
+            r[z] = (gv / (1.0f + expf(-gv))) * uv;
+          }
+          w[e] = pack2(r[0], r[1]);
+        }
+        const int f = nt * fpt + c * 16;
+        bf16 *dst = p.act + (size_t)row * p.O[0] + f;
+        if (row < p.rows && f < p.O[0]) *(uint4 *)dst = make_uint4(w[0], w[1], w[2], w[3]);
+        if (row < p.rows && f + 8 < p.O[0]) *(uint4 *)(dst + 8) = make_uint4(w[4], w[5], w[6], w[7]);
+      }
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive_cluster(mapa_u32(smem_u32(tempty), 0u));
+    }
+  }
+  __syncthreads();
+  if (*abort_flag && threadIdx.x == 0 && xr == 0)
+    for (int i = *n_consumed; i < *n_issued; i++) mbar_wait(&full[i % stages], (uint32_t)((i / stages) & 1));
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  cluster_sync_all();
+  if (warp == WS_EPI_WARPS + 1) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512) : "memory");
+  if (p.stamp && threadIdx.x == 0) atomicMin(p.stamp + 1, ~global_ns());
 }
 
 int n_tiles_of(WideEpi epi, const int *O, int nw) {
@@ -462,11 +960,96 @@ int launch_wide(const WideParams &p, bool pdl, cudaStream_t s) {
   return cudaLaunchKernelEx(&cfg, gemm_wide_kernel<EPI>, p) == cudaSuccess ? 0 : -6;
 }
 
+template <int EPI, int S>
+int launch_split_inst(const WideParams &p, bool pdl, cudaStream_t s) {
+  static SmemLimit limit;
+  if (!limit.ensure(gemm_wide_split_kernel<EPI, S>, WS_SMEM)) return -6;
+  if (!launch_allowed()) return 0;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(2 * S * p.m_tiles * p.n_tiles, 1, 1);
+  cfg.blockDim = dim3(WS_THREADS, 1, 1);
+  cfg.dynamicSmemBytes = WS_SMEM;
+  cfg.stream = s;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = 2 * S; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = pdl ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, gemm_wide_split_kernel<EPI, S>, p) == cudaSuccess ? 0 : -6;
+}
+template <int EPI>
+int launch_split(const WideParams &p, int S, bool pdl, cudaStream_t s) {
+  switch (S) {
+    case 2: return launch_split_inst<EPI, 2>(p, pdl, s);
+    case 3: return launch_split_inst<EPI, 3>(p, pdl, s);
+    default: return launch_split_inst<EPI, 4>(p, pdl, s);
+  }
+}
+
+int launch_swiglu(WideParams &p, bool pdl, cudaStream_t s) {
+  const int stage = W_A_BYTES + p.fpt * 128;
+  p.stages = std::min(8, (W_SMEM - W_CTRL - 1024) / stage);
+  static SmemLimit limit;
+  if (!limit.ensure(gemm_wide_swiglu_kernel, W_SMEM)) return -6;
+  if (!launch_allowed()) return 0;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(2 * std::min(W_PAIRS, p.m_tiles * p.n_tiles), 1, 1);
+  cfg.blockDim = dim3(WS_THREADS, 1, 1);
+  cfg.dynamicSmemBytes = p.stages * stage + W_CTRL + 1024;
+  cfg.stream = s;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = 2; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = pdl ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, gemm_wide_swiglu_kernel, p) == cudaSuccess ? 0 : -6;
+}
+
+// Measured at 168 to 256 rows in the replayed step of the 8B shapes (weight-streaming kernel -> this one): QKV 26.7 -> 18.3 us, O 18.5 ->
+// 17.8, down 33.4 -> 33 (168 rows); 31.7 -> 18.9, 22 -> 17.9, 38 -> 33 (240 rows); LM head 276 -> 180.
+// Clusters of 2 S CTAs (one CTA per SM) that are resident at once: a cluster lives inside one GPC, whose SM counts the
+// driver reports as 33, 22 and 15 clusters of 4, 6 and 8 on this chip.
+constexpr int W_MAX_SPLIT = 4;
+constexpr int W_FIT[W_MAX_SPLIT + 1] = {0, W_PAIRS, 33, 22, 15};
+// What a launch costs beside its k-blocks, in k-blocks: the epilogue of the last tile (persistent kernel), or parking,
+// cluster barrier, reduction and epilogue (split kernel)
+constexpr int W_COST_TAIL = 12, W_COST_SPLIT = 18;
+// K slices of a launch and its cost
+long long plan_split(WideEpi epi, int tiles, int KB, int *S) {
+  long long best = (long long)((tiles + W_PAIRS - 1) / W_PAIRS) * KB + W_COST_TAIL;
+  *S = 1;
+  if (epi != WIDE_RESID && epi != WIDE_QKV && epi != WIDE_F32) return best;
+  for (int sk = 2; sk <= W_MAX_SPLIT; sk++) {
+    if (KB / sk < 4) break;
+    const long long c = (long long)((tiles + W_FIT[sk] - 1) / W_FIT[sk]) * ((KB + sk - 1) / sk + W_COST_SPLIT);
+    if (c < best) { best = c; *S = sk; }
+  }
+  return best;
+}
+
+// Gate/up: features per tile of the launch (0: the persistent kernel with 128) and its cost
+long long plan_swiglu(int F, int KB, int m_tiles, int *fpt) {
+  const int t128 = (F + 127) / 128 * m_tiles;
+  long long best = (long long)((t128 + W_PAIRS - 1) / W_PAIRS) * KB + W_COST_TAIL;
+  *fpt = 0;
+  for (int f = 64; f <= WG_MAX_FPT; f += 16) {       // N of an M = 256 MMA is a multiple of 16
+    const int tiles = (F + f - 1) / f * m_tiles;
+    const long long c = (long long)((tiles + W_PAIRS - 1) / W_PAIRS) * ((long long)KB * f / 128 + W_COST_TAIL * f / 128);
+    if (c < best) { best = c; *fpt = f; }
+  }
+  return best;
+}
+
 }  // namespace
 
 long long wide_gemm_cost(WideEpi epi, const int *O, int nw, int I, int row_tiles) {
-  const long long tiles = (long long)n_tiles_of(epi, O, nw) * row_tiles;
-  return (tiles + W_PAIRS - 1) / W_PAIRS * ((I + TILE_K - 1) / TILE_K);
+  int S;
+  if (epi == WIDE_SWIGLU) return plan_swiglu(O[0], (I + TILE_K - 1) / TILE_K, row_tiles, &S);
+  return plan_split(epi, n_tiles_of(epi, O, nw) * row_tiles, (I + TILE_K - 1) / TILE_K, &S);
 }
 
 int wide_gemm_launch(TmaMaps *g, WideEpi epi, const WideGemmArgs &a, cudaStream_t s) {
@@ -475,7 +1058,7 @@ int wide_gemm_launch(TmaMaps *g, WideEpi epi, const WideGemmArgs &a, cudaStream_
   WideParams p;
   memset(&p, 0, sizeof p);
   for (int j = 0; j < a.nw; j++) {
-    if (!a.w[j] || ((uintptr_t)a.w[j] & 15) || a.O[j] < 8 || (a.O[j] % 8)) return -1;
+    if (!a.w[j] || ((uintptr_t)a.w[j] & 15) || a.O[j] < 1 || (epi != WIDE_ARGMAX && (a.O[j] % 8))) return -1;
     const CUtensorMap *mw = tma_maps_get(g, a.w[j], a.O[j], a.I, W_HALF);
     if (!mw) return -6;
     p.map_w[j] = *mw;
@@ -492,10 +1075,35 @@ int wide_gemm_launch(TmaMaps *g, WideEpi epi, const WideGemmArgs &a, cudaStream_
   p.ssq_in = a.ssq_in; p.ssq_in_tiles = a.ssq_in_tiles; p.ssq_ld = a.ssq_ld; p.inv_k_in = 1.0f / (float)a.k_in; p.eps = a.eps;
   p.xres = a.xres; p.gain = a.gain; p.hb = a.hb; p.ssq_out = a.ssq_out; p.taps = a.taps; p.tap_mask = a.taps ? a.tap_mask : 0; p.resid_add = a.resid_add;
   p.cs = a.cs; p.slot = a.slot; p.q = a.q; p.kp = (bf16 *)a.pool.k; p.vp = (bf16 *)a.pool.v; p.H = a.H; p.page_size = a.page_size;
-  p.act = a.act; p.out_b = a.out_b; p.ldo = a.ldo; p.status = a.status;
+  p.seq = a.seq; p.kvpos = a.kvpos; p.pm = a.pm; p.G = a.G;
+  p.act = a.act; p.out_b = a.out_b; p.ldo = a.ldo; p.out_f32 = a.out_f32; p.status = a.status; p.stamp = a.stamp;
+  p.best_val = a.best_val; p.best_idx = a.best_idx; p.best_ld = a.best_ld;
+  if (epi == WIDE_SWIGLU) {
+    plan_swiglu(a.O[0], p.KB, p.m_tiles, &p.fpt);
+    if (p.fpt) {
+      for (int j = 0; j < 2; j++) {
+        const CUtensorMap *mw = tma_maps_get(g, a.w[j], a.O[j], a.I, p.fpt / 2);
+        if (!mw) return -6;
+        p.map_w[j] = *mw;
+      }
+      p.n_tiles = (a.O[0] + p.fpt - 1) / p.fpt;
+      return launch_swiglu(p, a.pdl, s);
+    }
+  }
+  int S = 1;
+  plan_split(epi, p.m_tiles * p.n_tiles, p.KB, &S);
+  if (S > 1) {
+    switch (epi) {
+      case WIDE_RESID: return launch_split<WIDE_RESID>(p, S, a.pdl, s);
+      case WIDE_QKV: return launch_split<WIDE_QKV>(p, S, a.pdl, s);
+      default: return launch_split<WIDE_F32>(p, S, a.pdl, s);
+    }
+  }
   switch (epi) {
     case WIDE_RESID: return launch_wide<WIDE_RESID>(p, a.pdl, s);
     case WIDE_QKV: return launch_wide<WIDE_QKV>(p, a.pdl, s);
+    case WIDE_F32: return launch_wide<WIDE_F32>(p, a.pdl, s);
+    case WIDE_ARGMAX: return launch_wide<WIDE_ARGMAX>(p, a.pdl, s);
     case WIDE_SWIGLU: return launch_wide<WIDE_SWIGLU>(p, a.pdl, s);
     default: return launch_wide<WIDE_BF16>(p, a.pdl, s);
   }

@@ -8,7 +8,9 @@ enum WideEpi {
   WIDE_RESID = 0,    // x[r][o] (+)= acc; hb = bf16(x * gain[o]); per-128-feature sums of squares; optional taps
   WIDE_QKV = 1,      // scale, rotate q and k by the row's position, store q, write K/V into the paged cache (head_dim 128)
   WIDE_SWIGLU = 2,   // two weights (gate, up): act = bf16(silu(scale*g) * scale*u)
-  WIDE_BF16 = 3      // out_b[r][o] = bf16(acc)
+  WIDE_BF16 = 3,     // out_b[r][o] = bf16(acc)
+  WIDE_F32 = 4,      // out_f32[r][o] = scale * acc
+  WIDE_ARGMAX = 5    // per (128 features, row) best (value, index); optional fp32 logits (scale * acc)
 };
 
 struct WideGemmArgs {
@@ -33,6 +35,8 @@ struct WideGemmArgs {
   // WIDE_QKV: w = {wq, wk, wv}, or {wk, wv} when only the cache is to be written (nw = 2)
   const float2 *cs = nullptr;   // [rows][64] (cos, sin)
   const int32_t *slot = nullptr;   // [rows] cache row page * G * page_size + offset of the row's K/V; -1: none is written
+  const int32_t *seq = nullptr, *kvpos = nullptr;   // without `slot`: the row's sequence (-1: padding, q = 0) and cache position
+  PageMap pm = {nullptr, 0, 0, 0};
   bf16 *q = nullptr;            // [rows][H][128]
   KvPool pool = {nullptr, nullptr};
   int H = 0, G = 0, page_size = 0;
@@ -41,13 +45,20 @@ struct WideGemmArgs {
   // WIDE_BF16
   bf16 *out_b = nullptr;
   int ldo = 0;
+  // WIDE_F32, the logits of WIDE_ARGMAX (may be null there)
+  float *out_f32 = nullptr;     // row pitch ldo
+  // WIDE_ARGMAX
+  float *best_val = nullptr;    // [ceil(O/128)][best_ld]
+  int32_t *best_idx = nullptr;
+  int best_ld = 0;
   // launch
   int32_t *status = nullptr;
   bool pdl = false;
+  unsigned long long *stamp = nullptr;   // profiling aid (see KernelStamp)
 };
 
 constexpr int WIDE_ROWS = 256;      // token rows per tile
-// waves of the launch on this chip times its k-blocks (64 elements): what the launch's time goes with
+// what the launch's time goes with, in k-blocks (64 elements of the contraction, 0.27 us) of a tile
 long long wide_gemm_cost(WideEpi epi, const int *O, int nw, int I, int row_tiles);
 // Returns 0 or a negative code (-1: the shape does not fit).
 int wide_gemm_launch(TmaMaps *g, WideEpi epi, const WideGemmArgs &a, cudaStream_t s);
