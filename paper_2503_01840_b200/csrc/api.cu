@@ -333,7 +333,7 @@ extern "C" int spec_init(spec_ctx **out, const spec_target_weights *tw, const sp
     }
   }
   c->fused = c->fg != nullptr;
-  c->tree_fused = c->fused && draft_tree_step_smem(c->dtiles, c->K) > 0;
+  c->tree_fused = c->fused && draft_tree_step_fits(c->dtiles, c->K);
   if (c->fg && !(c->hd <= 128 && (c->hd & (c->hd - 1)) == 0)) {
     int rc = fail(nullptr, SPEC_ERR_UNSUPPORTED, "spec_init: the bf16 tensor-core path takes a power-of-two head_dim <= 128 (got %d)", c->hd);
     tma_maps_destroy(c->fg);
@@ -1439,7 +1439,7 @@ extern "C" int spec_gemm_topk(const void *x, const void *w, int32_t rows, int32_
   if (!x || !w || !out_idx || !out_lp || !scratch) return SPEC_ERR_NULL;
   if (rows < 1 || O < 1 || I < 1 || K < 1 || K > O) return SPEC_ERR_INVALID_CFG;
   const int tiles = (O + 127) / 128;
-  if (!draft_tree_step_smem(tiles, K)) return SPEC_ERR_UNSUPPORTED;
+  if (!draft_tree_step_fits(tiles, K)) return SPEC_ERR_UNSUPPORTED;
   static TmaMaps *g = nullptr;
   if (!g) {
     std::string why;

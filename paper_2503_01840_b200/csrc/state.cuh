@@ -39,7 +39,7 @@ void launch_prep_extend(SeqState st, TreeBufs tb, RowMeta m, int B, int need_pos
 void launch_expand(SeqState st, TreeBufs tb, RowMeta m, const int32_t *d2t, int pass, int B, cudaStream_t s);
 // One launch between two draft passes (merge of the LM head's per-tile candidates, expansion, the next pass's row
 // metadata, FC2 input and RoPE angles); returns -1 when the shape does not fit (tiles > 256, K > 15 or too many candidates).
-size_t draft_tree_step_smem(int tiles, int K);
+bool draft_tree_step_fits(int tiles, int K);
 int draft_tree_cand_ld(int tiles);      // row pitch (in tiles) of the candidate arrays: tiles rounded up to a multiple of 4
 int launch_draft_tree_step(SeqState st, TreeBufs tb, RowMeta m, const int32_t *d2t, int pass, const float *cand_val,
                            const int32_t *cand_idx, const float *cand_max, const float *cand_sum, int tiles, int ld, const float *x,

@@ -6,7 +6,7 @@
 
 namespace spec {
 
-size_t draft_tree_step_smem(int tiles, int K);
+bool draft_tree_step_fits(int tiles, int K);
 int draft_tree_cand_ld(int tiles);
 
 // ---------------------------------------------------------------- block argmax helpers
@@ -456,24 +456,18 @@ void launch_expand(SeqState st, TreeBufs tb, RowMeta m, const int32_t *d2t, int 
 
 // One warp merges the per-tile candidates of one row (the draft LM head's epilogue left, per 128-logit tile, the tile
 // maximum, the sum of exp relative to it and the tile's K best logits, best first): the row's log-sum-exp and its K best
-// (value desc, index asc) as log-probabilities.  Layout: candidates [row][ld][K], statistics [row][ld], ld a multiple of
-// 4 and the arrays 16-byte aligned, so a row is fetched with 16-byte asynchronous copies that are all in flight at once.
-// stage_v / stage_i: ld * K floats / ints of 16-byte aligned scratch owned by the warp; tiles <= 256, K <= 15.
+// (value desc, index asc) as log-probabilities.  Layout: candidates [row][ld][K], statistics [row][ld]; tiles <= 256, K <= 15.
+//
+// Only the K tiles with the best heads can hold one of the K best candidates: every candidate of another tile comes behind
+// its own head, hence behind K better heads (tiles hold ascending index ranges, so the order of equal heads is the order of
+// the tiles).  So the warp first picks K tiles from the statistics it has in registers anyway and then fetches those K * K
+// candidates, one tile per lane, instead of staging all tiles' (20 KB per row, 200 KB per CTA) and walking their heads: the
+// merge of 10 rows of 250 tiles took 13 of the launch's 18 us.
 __device__ __forceinline__ void merge_tile_candidates(const float *__restrict__ cand_val, const int32_t *__restrict__ cand_idx,
                                                       const float *__restrict__ cand_max, const float *__restrict__ cand_sum,
-                                                      int tiles, int ld, int row, int K, float *stage_v, int32_t *stage_i,
-                                                      int32_t *out_id, float *out_lp) {
+                                                      int tiles, int ld, int row, int K, int32_t *out_id, float *out_lp) {
   const int lane = threadIdx.x & 31;
-  const int nvec = ld * K / 4;                           // ld % 4 == 0
-  const float4 *gv = (const float4 *)(cand_val + (size_t)row * ld * K);
-  const int4 *gi = (const int4 *)(cand_idx + (size_t)row * ld * K);
-  for (int e = lane; e < nvec; e += 32) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(stage_v + 4 * e)), "l"(gv + e) : "memory");
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(stage_i + 4 * e)), "l"(gi + e) : "memory");
-  }
-  asm volatile("cp.async.commit_group;" ::: "memory");
-  // the tile statistics meanwhile: at most 8 tiles per lane, all loads issued before the first use
-  float pm[8], ps[8];
+  float pm[8], ps[8];                                    // at most 8 tiles per lane, all loads issued before the first use
 #pragma unroll
   for (int j = 0; j < 8; j++) {
     const int t = lane + 32 * j;
@@ -484,31 +478,47 @@ __device__ __forceinline__ void merge_tile_candidates(const float *__restrict__ 
 #pragma unroll
   for (int j = 0; j < 8; j++) mx = fmaxf(mx, pm[j]);
   for (int off = 16; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-  float sum = 0.0f;                                      // lane l adds its tiles in tile order, then a fixed shuffle tree
+  // ---- the K best tiles, (head desc, tile asc): lane c keeps the c-th
+  const int nsel = K < tiles ? K : tiles;
+  unsigned key[8];
+#pragma unroll
+  for (int j = 0; j < 8; j++) key[j] = lane + 32 * j < tiles ? ordered_key(pm[j]) : 0u;      // keys of values are >= 1
+  int sel = 0;
+  for (int c = 0; c < nsel; c++) {
+    unsigned bk = 0u, wk;
+    int bt = -1;
+#pragma unroll
+    for (int j = 0; j < 8; j++)
+      if (key[j] > bk) { bk = key[j]; bt = lane + 32 * j; }
+    const int w = warp_best(bk, bt, &wk);
+    if (lane == c) sel = w;
+#pragma unroll
+    for (int j = 0; j < 8; j++)
+      if (lane + 32 * j == w) key[j] = 0u;
+  }
+  // ---- lane c holds the c-th tile's candidates, best first: only their heads compete, and the winner's list moves up
+  unsigned ck[15];
+  int ci[15];
+#pragma unroll
+  for (int i = 0; i < 15; i++) {
+    const bool have = lane < nsel && i < K;
+    const size_t at = ((size_t)row * ld + sel) * K + i;
+    ci[i] = have ? cand_idx[at] : -1;
+    ck[i] = have ? ordered_key(cand_val[at]) : 0u;
+  }
+  // the log-sum-exp while they are on their way: a lane adds its tiles in tile order, then a fixed shuffle tree
+  float sum = 0.0f;
 #pragma unroll
   for (int j = 0; j < 8; j++) sum += (lane + 32 * j < tiles) ? ps[j] * expf(pm[j] - mx) : 0.0f;
   for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
   const float lse = logf(sum);
-  asm volatile("cp.async.wait_group 0;" ::: "memory");
-  __syncwarp();
-  // a tile's candidates are stored best first: only its current head can be the next winner.  hp = head position of
-  // each of this lane's (at most 8) tiles, four bits each.
-  unsigned hp = 0;
   for (int c = 0; c < K; c++) {
-    float bv = 0.0f;
-    int bi = -1, bj = 0;
-#pragma unroll
-    for (int j = 0; j < 8; j++) {
-      const int t = lane + 32 * j, h = (hp >> (4 * j)) & 15;
-      if (t < tiles && h < K) {
-        const int ci = stage_i[t * K + h];
-        const float cv = stage_v[t * K + h];
-        if (ci >= 0 && (bi < 0 || before(cv, ci, bv, bi))) { bv = cv; bi = ci; bj = j; }
-      }
-    }
     unsigned wk;
-    const int wi = warp_best(ordered_key(bv), bi, &wk);  // two redux instructions instead of a shuffle tree
-    if (wi >= 0 && wi == bi) hp += 1u << (4 * bj);       // indices are unique: exactly one lane owns the winner
+    const int wi = warp_best(ck[0], ci[0], &wk);         // two redux instructions instead of a shuffle tree
+    const bool won = wi >= 0 && ci[0] == wi;             // indices are unique: one lane at most
+#pragma unroll
+    for (int i = 0; i < 14; i++) { ck[i] = won ? ck[i + 1] : ck[i]; ci[i] = won ? ci[i + 1] : ci[i]; }
+    if (won) ci[14] = -1;
     if (lane == 0) { out_id[c] = wi < 0 ? 0 : wi; out_lp[c] = wi < 0 ? 0.0f : (key_value(wk) - mx) - lse; }
   }
   __syncwarp();
@@ -520,20 +530,14 @@ __global__ void __launch_bounds__(256) merge_candidates_kernel(const float *cand
                                                                int32_t *__restrict__ idx, float *__restrict__ lp) {
   pdl_wait();
   pdl_trigger();
-  extern __shared__ __align__(16) unsigned char smraw[];
   const int warp = threadIdx.x >> 5, row = blockIdx.x * 8 + warp;
   if (row >= rows) return;
-  float *stage_v = (float *)smraw + (size_t)warp * 2 * ld * K;
-  merge_tile_candidates(cand_val, cand_idx, cand_max, cand_sum, tiles, ld, row, K, stage_v, (int32_t *)(stage_v + ld * K),
-                        idx + (size_t)row * K, lp + (size_t)row * K);
+  merge_tile_candidates(cand_val, cand_idx, cand_max, cand_sum, tiles, ld, row, K, idx + (size_t)row * K, lp + (size_t)row * K);
 }
 int launch_merge_candidates(const float *cand_val, const int32_t *cand_idx, const float *cand_max, const float *cand_sum, int tiles,
                             int ld, int rows, int K, int32_t *idx, float *lp, cudaStream_t s) {
-  const size_t smem = draft_tree_step_smem(tiles, K);
-  if (!smem || ld != draft_tree_cand_ld(tiles)) return -1;
-  static SmemLimit limit;
-  if (smem > 48 * 1024 && !limit.ensure(merge_candidates_kernel, (int)smem)) return -6;
-  launch_k(merge_candidates_kernel, dim3((rows + 7) / 8), dim3(256), smem, s, cand_val, cand_idx, cand_max, cand_sum, tiles, ld, rows, K, idx, lp);
+  if (!draft_tree_step_fits(tiles, K) || ld != draft_tree_cand_ld(tiles)) return -1;
+  launch_k(merge_candidates_kernel, dim3((rows + 7) / 8), dim3(256), 0, s, cand_val, cand_idx, cand_max, cand_sum, tiles, ld, rows, K, idx, lp);
   return 0;
 }
 
@@ -558,7 +562,8 @@ struct TreeStepArgs {
 };
 
 constexpr int TREE_WARPS = 10;   // one warp per row of a top-10 level
-__global__ void __launch_bounds__(TREE_WARPS * 32) draft_tree_step_kernel(const TreeStepArgs a) {
+constexpr int TREE_ANGLE_WARPS = 2, TREE_THREADS = (TREE_WARPS + TREE_ANGLE_WARPS) * 32;
+__global__ void __launch_bounds__(TREE_THREADS) draft_tree_step_kernel(const TreeStepArgs a) {
   pdl_wait();
   pdl_trigger();
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -567,19 +572,16 @@ __global__ void __launch_bounds__(TREE_WARPS * 32) draft_tree_step_kernel(const 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nrows = (pass == 1) ? 1 : K;                 // rows of this sequence in the pass that just ran
   const int nchild = nrows * K;
-  // shared memory: per-warp candidate staging, then the expansion's small arrays
-  const int ncand = a.ld * K;
-  float *stage_v = (float *)smraw + (size_t)warp * 2 * ncand;      // [ld][K] values, then indices
-  int32_t *stage_i = (int32_t *)(stage_v + ncand);
-  unsigned char *tail = smraw + (size_t)TREE_WARPS * 2 * ncand * 4;
-  float *tk_lp = (float *)tail;                          // [nrows][K]
+  const int nchild4 = (nchild + 3) & ~3;
+  float *cscore = (float *)smraw;                        // [nchild], padded to whole float4s with -inf
+  float *tk_lp = cscore + ((K * K + 3) & ~3);            // [nrows][K]
   int32_t *tk_id = (int32_t *)(tk_lp + K * K);           // [nrows][K] draft ids
-  float *cscore = (float *)(tk_id + K * K);              // [nchild]
-  int32_t *ctok = (int32_t *)(cscore + K * K);           // [nchild] target ids
+  int32_t *ctok = tk_id + K * K;                         // [nchild] target ids
   int32_t *newf = ctok + K * K;                          // [K] child index (within the level) of the new frontier
   int32_t *par_u = newf + K;                             // [K] pool index of the node each row of this pass processed
   float *par_sc = (float *)(par_u + K);                  // [K] its score
-  const int active = a.st.active[b], n = a.st.n[b], last_row = a.st.last_row[b];
+  const int active = a.st.active[b], n = a.st.n[b];
+  const int src1 = a.st.last_row[b];                     // pass 1: the row that holds the last pending entry's outputs
   const size_t pb = (size_t)b * (tb.pool + 1);
   const int base = (pass == 1) ? 0 : K + (pass - 2) * K * K;       // pool index of child 0 is base + 1
   const bool writer = blockIdx.y == 0;
@@ -599,11 +601,19 @@ __global__ void __launch_bounds__(TREE_WARPS * 32) draft_tree_step_kernel(const 
     par_u[threadIdx.x] = u;
     par_sc[threadIdx.x] = tb.pool_score[pb + u];
   }
+  // ---- the RoPE angles of the next pass (one position for all rows; double precision, rounded once): two warps of their
+  // own, while the others merge
+  if (warp >= TREE_WARPS && pass < D) {
+    for (int i = threadIdx.x - TREE_WARPS * 32; i < a.half; i += TREE_ANGLE_WARPS * 32) {
+      double sn, cs_;
+      sincos((double)(n + pass - 1) * a.inv_freq[i], &sn, &cs_);
+      for (int rr = blockIdx.y; rr < K; rr += gridDim.y) a.cs[(size_t)(b * K + rr) * a.half + i] = make_float2((float)cs_, (float)sn);
+    }
+  }
   // ---- 1. per row: log-sum-exp over the tiles and the K best of the tiles' candidates (value desc, index asc)
-  for (int r = warp; r < nrows; r += TREE_WARPS) {
-    const int row = (pass == 1) ? last_row : b * K + r;
-    merge_tile_candidates(a.cand_val, a.cand_idx, a.cand_max, a.cand_sum, a.tiles, a.ld, row, K, stage_v, stage_i, tk_id + r * K,
-                          tk_lp + r * K);
+  for (int r = warp; warp < TREE_WARPS && r < nrows; r += TREE_WARPS) {
+    const int row = (pass == 1) ? src1 : b * K + r;
+    merge_tile_candidates(a.cand_val, a.cand_idx, a.cand_max, a.cand_sum, a.tiles, a.ld, row, K, tk_id + r * K, tk_lp + r * K);
   }
   __syncthreads();
   if (writer) {   // kept for inspection: the top-K of this pass in the layout of the per-row kernels
@@ -629,13 +639,18 @@ __global__ void __launch_bounds__(TREE_WARPS * 32) draft_tree_step_kernel(const 
       tb.pool_score[pb + ci] = sc;
     }
   }
+  if ((int)threadIdx.x < nchild4 - nchild) cscore[nchild + threadIdx.x] = -INFINITY;
   __syncthreads();
   if (pass >= D) return;
   // ---- 3. next frontier: the K best children of the level, (score desc, pool index asc)
   for (int c = threadIdx.x; c < nchild; c += blockDim.x) {
     const float s = cscore[c];
     int rank = 0;
-    for (int j = 0; j < nchild; j++) rank += (cscore[j] > s || (cscore[j] == s && j < c)) ? 1 : 0;
+#pragma unroll 4
+    for (int j = 0; j < nchild4; j += 4) {               // the padding never comes before a child
+      const float4 o = *(const float4 *)(cscore + j);
+      rank += (o.x > s || (o.x == s && j < c)) + (o.y > s || (o.y == s && j + 1 < c)) + (o.z > s || (o.z == s && j + 2 < c)) + (o.w > s || (o.w == s && j + 3 < c));
+    }
     if (rank < K) newf[rank] = c;
   }
   __syncthreads();
@@ -655,7 +670,7 @@ __global__ void __launch_bounds__(TREE_WARPS * 32) draft_tree_step_kernel(const 
       if (slot < 64) lo |= 1ull << slot; else hi |= 1ull << (slot - 64);
       tb.front_cur[b * K + rr] = ci;
       tb.frontier[((size_t)b * D + pass) * K + rr] = ci;
-      tb.feat_row[row] = (pass == 1) ? last_row : b * K + pr;
+      tb.feat_row[row] = (pass == 1) ? src1 : b * K + pr;
       a.m.seq[row] = b;
       a.m.pos[row] = n + pass - 1;
       a.m.kvpos[row] = n + slot;
@@ -666,107 +681,122 @@ __global__ void __launch_bounds__(TREE_WARPS * 32) draft_tree_step_kernel(const 
       a.m.tok[row] = ctok[c];
     }
   }
-  // ---- 4. inputs of the next pass: FC2 input [bf16(feature of the parent's row) ; embedding of the node's token] and
-  // the RoPE angles of its position (double precision, rounded once), split over the CTAs of the sequence
+  // ---- 4. inputs of the next pass: FC2 input [bf16(feature of the parent's row) ; embedding of the node's token], split
+  // over the CTAs of the sequence
   const int k = a.k, vpr = 2 * k / 8;                      // 8-element vectors per row (hidden % 8 == 0)
-  for (int e = blockIdx.y * blockDim.x + threadIdx.x; e < K * vpr; e += gridDim.y * blockDim.x) {
-    const int rr = e / vpr, i = (e % vpr) * 8;
-    const int c = newf[rr];
-    uint4 out;
-    if (i < k) {
-      const int fr = (pass == 1) ? last_row : b * K + c / K;
-      const float4 lo = *(const float4 *)(a.x + (size_t)fr * k + i), hi = *(const float4 *)(a.x + (size_t)fr * k + i + 4);
-      __nv_bfloat162 p0 = __floats2bfloat162_rn(lo.x, lo.y), p1 = __floats2bfloat162_rn(lo.z, lo.w);
-      __nv_bfloat162 p2 = __floats2bfloat162_rn(hi.x, hi.y), p3 = __floats2bfloat162_rn(hi.z, hi.w);
-      out = make_uint4(*(uint32_t *)&p0, *(uint32_t *)&p1, *(uint32_t *)&p2, *(uint32_t *)&p3);
-    } else {
-      out = *(const uint4 *)(a.embed + (size_t)ctok[c] * k + (i - k));
+  const int stride = gridDim.y * blockDim.x, total = K * vpr;
+  constexpr int NV = 4;                                    // vectors of a thread whose loads are in flight together
+  for (int e0 = blockIdx.y * blockDim.x + threadIdx.x; e0 < total; e0 += NV * stride) {
+    uint4 v[NV][2];                                        // eight floats of the feature, or eight bf16 of the embedding
+#pragma unroll
+    for (int q = 0; q < NV; q++) {
+      const int e = e0 + q * stride;
+      if (e < total) {
+        const int rr = e / vpr, i = (e % vpr) * 8, c = newf[rr];
+        if (i < k) {
+          const int fr = (pass == 1) ? src1 : b * K + c / K;
+          v[q][0] = *(const uint4 *)(a.x + (size_t)fr * k + i); v[q][1] = *(const uint4 *)(a.x + (size_t)fr * k + i + 4);
+        } else {
+          v[q][0] = *(const uint4 *)(a.embed + (size_t)ctok[c] * k + (i - k));
+        }
+      }
     }
-    *(uint4 *)(a.cat + ((size_t)(b * K + rr)) * 2 * k + i) = out;
-  }
-  const int nang = K * a.half;
-  for (int e = blockIdx.y * blockDim.x + threadIdx.x; e < nang; e += gridDim.y * blockDim.x) {
-    const int rr = e / a.half, i = e % a.half;
-    double sn, cs_;
-    sincos((double)(n + pass - 1) * a.inv_freq[i], &sn, &cs_);
-    a.cs[(size_t)(b * K + rr) * a.half + i] = make_float2((float)cs_, (float)sn);
+#pragma unroll
+    for (int q = 0; q < NV; q++) {
+      const int e = e0 + q * stride;
+      if (e < total) {
+        const int rr = e / vpr, i = (e % vpr) * 8;
+        uint4 out = v[q][0];
+        if (i < k) {
+          __nv_bfloat162 p0 = __floats2bfloat162_rn(__uint_as_float(v[q][0].x), __uint_as_float(v[q][0].y)), p1 = __floats2bfloat162_rn(__uint_as_float(v[q][0].z), __uint_as_float(v[q][0].w));
+          __nv_bfloat162 p2 = __floats2bfloat162_rn(__uint_as_float(v[q][1].x), __uint_as_float(v[q][1].y)), p3 = __floats2bfloat162_rn(__uint_as_float(v[q][1].z), __uint_as_float(v[q][1].w));
+          out = make_uint4(*(uint32_t *)&p0, *(uint32_t *)&p1, *(uint32_t *)&p2, *(uint32_t *)&p3);
+        }
+        *(uint4 *)(a.cat + ((size_t)(b * K + rr)) * 2 * k + i) = out;
+      }
+    }
   }
 }
 
-// shared memory the launch needs; 0 when the shape does not fit the kernel (the caller then uses the separate kernels)
+// Shapes the kernel takes (the others use the separate kernels): at most eight tiles per lane, at most 220 KB of candidates
+// for the ten rows of a level.
 int draft_tree_cand_ld(int tiles) { return (tiles + 3) & ~3; }
-size_t draft_tree_step_smem(int tiles, int K) {
-  if (tiles > 256 || K > 15) return 0;
-  const size_t need = (size_t)TREE_WARPS * 2 * draft_tree_cand_ld(tiles) * K * 4 + (size_t)K * K * 16 + (size_t)K * 12 + 64;
-  return need <= 220 * 1024 ? need : 0;
+bool draft_tree_step_fits(int tiles, int K) {
+  if (tiles > 256 || K > 15) return false;
+  return (size_t)TREE_WARPS * 2 * draft_tree_cand_ld(tiles) * K * 4 + (size_t)K * K * 16 + (size_t)K * 12 + 64 <= 220 * 1024;
 }
 int launch_draft_tree_step(SeqState st, TreeBufs tb, RowMeta m, const int32_t *d2t, int pass, const float *cand_val,
                            const int32_t *cand_idx, const float *cand_max, const float *cand_sum, int tiles, int ld, const float *x,
                            const bf16 *embed, bf16 *cat, int k, const double *inv_freq, float2 *cs, int half, int B, cudaStream_t s) {
-  const size_t smem = draft_tree_step_smem(tiles, tb.K);
-  if (!smem || ld != draft_tree_cand_ld(tiles) || (k % 8)) return -1;
-  static SmemLimit limit;
-  if (smem > 48 * 1024 && !limit.ensure(draft_tree_step_kernel, (int)smem)) return -6;
+  if (!draft_tree_step_fits(tiles, tb.K) || ld != draft_tree_cand_ld(tiles) || (k % 8)) return -1;
+  const size_t smem = (size_t)((tb.K * tb.K + 3) & ~3) * 4 + (size_t)tb.K * tb.K * 12 + (size_t)tb.K * 12;
   TreeStepArgs a{st, tb, m, d2t, pass, cand_val, cand_max, cand_sum, cand_idx, tiles, ld, x, embed, cat, k, inv_freq, cs, half};
   const int Z = B >= 16 ? 1 : 8;        // CTAs per sequence that share the next pass's input assembly
-  launch_k(draft_tree_step_kernel, dim3(B, Z), dim3(TREE_WARPS * 32), smem, s, a);
+  launch_k(draft_tree_step_kernel, dim3(B, Z), dim3(TREE_THREADS), smem, s, a);
   return 0;
 }
 
 // ---------------------------------------------------------------- pruning + tree assembly
 // Keeps the M = min(N-1, pool) best candidates (score desc, pool index asc), numbers them in pool
 // order after the root and emits parents, depths, ancestor-or-self bit masks and the verify rows.
-__global__ void __launch_bounds__(256) rerank_kernel(SeqState st, TreeBufs tb, RowMeta m) {
+// One thread per pool entry (pool + 1 <= 1024): rank counting over four candidates per shared-memory load, numbering by
+// warp ballots (with 256 threads, scalar loads and a counting loop per kept candidate: 17 us on the step's critical path).
+__global__ void __launch_bounds__(1024) rerank_kernel(SeqState st, TreeBufs tb, RowMeta m) {
   pdl_wait();
   pdl_trigger();
-  extern __shared__ unsigned char smraw[];
-  int b = blockIdx.x, pool = tb.pool, N = tb.N;
-  float *sc = (float *)smraw;                       // [pool+1]
-  int32_t *node_of = (int32_t *)(sc + pool + 1);    // [pool+1], -1 = dropped
+  extern __shared__ __align__(16) unsigned char smraw[];
+  __shared__ int warp_kept[32];
+  const int b = blockIdx.x, pool = tb.pool, N = tb.N, pool4 = (pool + 3) & ~3;
+  float *sc = (float *)smraw;                       // [pool4]: candidate i at i - 1, padded with -inf
+  int32_t *node_of = (int32_t *)(sc + pool4);       // [pool+1], -1 = dropped
   int32_t *par = node_of + pool + 1;                // [pool+1]
-  int M = (N - 1 < pool) ? N - 1 : pool;
-  size_t pb = (size_t)b * (pool + 1);
-  int n = st.n[b];
-  bool act = st.active[b] != 0;
-  for (int i = threadIdx.x; i <= pool; i += blockDim.x) { sc[i] = tb.pool_score[pb + i]; par[i] = tb.pool_parent[pb + i]; }
+  const int M = (N - 1 < pool) ? N - 1 : pool;
+  const size_t pb = (size_t)b * (pool + 1);
+  const int n = st.n[b];
+  const bool act = st.active[b] != 0;
+  const int i = threadIdx.x;
+  float score = 0.0f;
+  int parent = 0, depth = 0, tok = 0;
+  if (i <= pool) {
+    score = tb.pool_score[pb + i]; parent = tb.pool_parent[pb + i]; depth = tb.pool_depth[pb + i]; tok = tb.pool_tok[pb + i];
+    if (i > 0) sc[i - 1] = score;
+    par[i] = parent;
+  }
+  if (i < pool4 - pool) sc[pool + i] = -INFINITY;
   __syncthreads();
-  for (int i = threadIdx.x; i <= pool; i += blockDim.x) {
-    if (i == 0) { node_of[0] = 0; continue; }
-    float s = sc[i];
+  bool kept = false;
+  if (i >= 1 && i <= pool) {
+    const int c = i - 1;
     int rank = 0;
-    for (int j = 1; j <= pool; j++) rank += (sc[j] > s || (sc[j] == s && j < i)) ? 1 : 0;
-    node_of[i] = (rank < M) ? 1 : -1;
-  }
-  __syncthreads();
-  // number the kept candidates in pool order
-  int mine[4];   // pool <= 1024 with 256 threads -> up to 4 candidates each (checked on the host)
-  int cnt = 0;
-  for (int i = threadIdx.x; i <= pool; i += blockDim.x) {
-    int idx = -1;
-    if (i == 0) idx = 0;
-    else if (node_of[i] > 0) {
-      idx = 1;
-      for (int j = 1; j < i; j++) idx += (node_of[j] > 0) ? 1 : 0;
+#pragma unroll 4
+    for (int j = 0; j < pool4; j += 4) {            // the padding never comes before a candidate
+      const float4 o = *(const float4 *)(sc + j);
+      rank += (o.x > score || (o.x == score && j < c)) + (o.y > score || (o.y == score && j + 1 < c)) +
+              (o.z > score || (o.z == score && j + 2 < c)) + (o.w > score || (o.w == score && j + 3 < c));
     }
-    mine[cnt++] = idx;
+    kept = rank < M;
   }
+  // number the kept candidates in pool order, after the root
+  const unsigned ballot = __ballot_sync(0xffffffffu, kept);
+  if ((i & 31) == 0) warp_kept[i >> 5] = __popc(ballot);
   __syncthreads();
-  cnt = 0;
-  for (int i = threadIdx.x; i <= pool; i += blockDim.x) node_of[i] = mine[cnt++];
+  int ni = i == 0 ? 0 : -1;
+  if (kept) {
+    ni = 1 + __popc(ballot & ((1u << (i & 31)) - 1u));
+    for (int w = 0; w < (i >> 5); w++) ni += warp_kept[w];
+  }
+  if (i <= pool) node_of[i] = ni;
   __syncthreads();
-  if (threadIdx.x == 0) tb.nn[b] = act ? M + 1 : 0;
-  for (int i = threadIdx.x; i <= pool; i += blockDim.x) {
-    int ni = node_of[i];
-    if (ni < 0) continue;
+  if (i == 0) tb.nn[b] = act ? M + 1 : 0;
+  if (ni >= 0 && ni < N) {
     uint64_t mask = 0;
     for (int v = i, it = 0; v >= 0 && v <= pool && it < 64; v = par[v], it++) mask |= 1ull << (node_of[v] & 63);
-    size_t t = (size_t)b * N + ni;
-    int depth = tb.pool_depth[pb + i];
-    tb.tok[t] = tb.pool_tok[pb + i];
-    tb.parent[t] = (i == 0) ? -1 : node_of[par[i]];
+    const size_t t = (size_t)b * N + ni;
+    tb.tok[t] = tok;
+    tb.parent[t] = (i == 0) ? -1 : node_of[parent];
     tb.depth[t] = depth;
     tb.poolidx[t] = i;
-    tb.score[t] = sc[i];
+    tb.score[t] = score;
     tb.mask[t] = mask;
     m.seq[t] = act ? b : -1;
     m.pos[t] = act ? n + depth : 0;
@@ -775,18 +805,18 @@ __global__ void __launch_bounds__(256) rerank_kernel(SeqState st, TreeBufs tb, R
     m.tail_base[t] = act ? n : 0;
     m.mask_lo[t] = mask;
     m.mask_hi[t] = 0ull;
-    m.tok[t] = act ? tb.pool_tok[pb + i] : 0;
+    m.tok[t] = act ? tok : 0;
   }
   // rows beyond the tree (only when pool < N-1) are padding
-  for (int i = M + 1 + threadIdx.x; i < N; i += blockDim.x) {
-    size_t t = (size_t)b * N + i;
+  for (int r = M + 1 + threadIdx.x; r < N; r += blockDim.x) {
+    const size_t t = (size_t)b * N + r;
     m.seq[t] = -1; m.pos[t] = 0; m.kvpos[t] = 0; m.ctx[t] = 0; m.tail_base[t] = 0;
     m.mask_lo[t] = 0; m.mask_hi[t] = 0; m.tok[t] = 0;
   }
 }
 void launch_rerank(SeqState st, TreeBufs tb, RowMeta m, int B, cudaStream_t s) {
-  size_t smem = (size_t)(tb.pool + 1) * 12 + 16;
-  launch_k(rerank_kernel, dim3(B), dim3(256), smem, s, st, tb, m);
+  const size_t smem = (size_t)((tb.pool + 3) & ~3) * 4 + (size_t)(tb.pool + 1) * 8;
+  launch_k(rerank_kernel, dim3(B), dim3((tb.pool + 1 + 31) / 32 * 32), smem, s, st, tb, m);
 }
 
 // Tree of the root alone (plain autoregressive decoding on the same kernels): one row per sequence.
