@@ -26,12 +26,12 @@ thread_local int tl_launch_budget = -1;
 void launch_logsoftmax_topk_rows(const float *logits, const int32_t *src_row, int rows, int n, int K, int32_t *idx,
                                  float *lp, cudaStream_t s);
 
-// dst row b*dst_stride_rows <- src row src_row[b] (fp32, `width` columns); rows with src_row < 0 are skipped
+// dst row b*dst_stride_rows <- src row src_row[b] (fp32, `width` columns; src_row null: row b); rows with src_row < 0 are skipped
 __global__ void gather_rows_kernel(const float *__restrict__ src, const int32_t *__restrict__ src_row,
                                    float *__restrict__ dst, int width, int dst_stride_rows) {
   pdl_wait();
   pdl_trigger();
-  int b = blockIdx.x, sr = src_row[b];
+  int b = blockIdx.x, sr = src_row ? src_row[b] : b;
   if (sr < 0) return;
   for (int i = threadIdx.x; i < width; i += blockDim.x)
     dst[(size_t)b * dst_stride_rows * width + i] = src[(size_t)sr * width + i];
@@ -476,15 +476,19 @@ template <typename T> struct Sched {
     tick();
   }
   // residual-producing GEMM: x (+)= in . w^T, h = bf16(x * gain), ssq, optional taps
-  void fgemm_resid(const void *in, int I, const void *w, int rows, bool add, const void *gain, int tap_mask) {
+  void fgemm_resid(const void *in, int I, const void *w, int rows, bool add, const void *gain, int tap_mask, float *xres = nullptr) {
     FusedGemmArgs a = fargs(in, rows, I);
     a.w[0] = (const bf16 *)w; a.O[0] = c->k; a.nw = 1;
-    a.xres = c->x; a.gain = (const bf16 *)gain; a.hb = (bf16 *)c->h; a.ssq_out = c->ssq; a.ssq_ld = c->Ralloc;
+    a.xres = xres ? xres : c->x; a.gain = (const bf16 *)gain; a.hb = (bf16 *)c->h; a.ssq_out = c->ssq; a.ssq_ld = c->Ralloc;
     a.taps = (bf16 *)c->node_taps; a.tap_mask = tap_mask; a.resid_add = add ? 1 : 0;
     fgemm(EPI_RESID, a);
   }
   void block_fused(const LayerW &w, KvPool pool, int rows, int tail_len, const void *next_gain, int tap_mask) {
-    int k = c->k, qd = c->H * c->hd, kvd = c->G * c->hd, F = c->F;
+    qkv_attn_fused(w, pool, rows, tail_len);
+    block_tail_fused(w, c->ao, rows, next_gain, tap_mask, c->x);
+  }
+  void qkv_attn_fused(const LayerW &w, KvPool pool, int rows, int tail_len) {
+    int k = c->k, qd = c->H * c->hd, kvd = c->G * c->hd;
     FusedGemmArgs a = fargs(c->h, rows, k);
     a.w[0] = (const bf16 *)w.wq; a.w[1] = (const bf16 *)w.wk; a.w[2] = (const bf16 *)w.wv;
     a.O[0] = qd; a.O[1] = kvd; a.O[2] = kvd; a.nw = 3;
@@ -494,13 +498,17 @@ template <typename T> struct Sched {
     a.H = c->H; a.G = c->G; a.hd = c->hd;
     fgemm(EPI_QKV, a);
     attention(pool, rows, tail_len);
-    fgemm_resid(c->ao, qd, w.wo, rows, true, w.mlp_norm, 0);
-    FusedGemmArgs g = fargs(c->h, rows, k);
-    g.w[0] = (const bf16 *)w.w_gate; g.w[1] = (const bf16 *)w.w_up; g.O[0] = F; g.O[1] = F; g.nw = 2;
+  }
+  // what follows the attention of a layer: O projection and MLP on `rows` rows whose attention outputs are in ao and whose
+  // residual stream is xres
+  void block_tail_fused(const LayerW &w, const void *ao, int rows, const void *next_gain, int tap_mask, float *xres) {
+    fgemm_resid(ao, c->H * c->hd, w.wo, rows, true, w.mlp_norm, 0, xres);
+    FusedGemmArgs g = fargs(c->h, rows, c->k);
+    g.w[0] = (const bf16 *)w.w_gate; g.w[1] = (const bf16 *)w.w_up; g.O[0] = c->F; g.O[1] = c->F; g.nw = 2;
     with_norm_scale(g);
     g.act = (bf16 *)c->act;
     fgemm(EPI_SWIGLU, g);
-    fgemm_resid(c->act, F, w.w_down, rows, true, next_gain, tap_mask);
+    fgemm_resid(c->act, c->F, w.w_down, rows, true, next_gain, tap_mask, xres);
   }
   void target_forward_fused(int rows, int tail_len, bool want_logits) {
     mark(SPEC_PROF_MISC); launch_rope_table(c->meta.pos, rows, c->hd / 2, c->inv_freq, c->cs, s); tick();
@@ -531,8 +539,9 @@ template <typename T> struct Sched {
     c->np_proj = 1; c->ps_proj = 0;
   }
   // prebuilt: the launch that closed the previous draft pass already wrote this pass's FC2 input and RoPE angles
+  // pending: the step's pass over the pending entries
   void draft_forward_fused(const float *feat, int nparts, size_t fstride, const int32_t *src_row, int rows, int tail_len,
-                           bool prebuilt = false) {
+                           bool prebuilt = false, bool pending = false) {
     if (!prebuilt) {
       mark(SPEC_PROF_MISC); launch_rope_table(c->meta.pos, rows, c->hd / 2, c->inv_freq, c->cs, s); tick();
       mark(SPEC_PROF_MISC);
@@ -540,8 +549,21 @@ template <typename T> struct Sched {
       tick();
     }
     fgemm_resid(c->cat, 2 * c->k, c->fc2, rows, false, c->dl.attn_norm, 0);
+    if (pending && extend_compact()) {
+      // Only the last entry of each sequence is used beyond its K/V, so what follows the attention runs on B rows
+      // (residual in c->proj, attention output in c->q, both free by now).
+      qkv_attn_fused(c->dl, c->pools[c->L], rows, tail_len);
+      mark(SPEC_PROF_TREE);
+      launch_gather_pending(c->st.last_row, c->x, c->proj, c->k, (const bf16 *)c->ao, (bf16 *)c->q, c->H * c->hd, c->B, s); tick();
+      block_tail_fused(c->dl, c->q, c->B, c->dfinal_norm, 0, c->proj);
+      return;
+    }
     block_fused(c->dl, c->pools[c->L], rows, tail_len, c->dfinal_norm, 0);
   }
+  // Worth a gather launch (2-3 us) when B rows take a narrower GEMM tile than B * (D + 1): 256 -> 64 rows is 297 -> 159 us
+  // for the four GEMMs of the 8B shapes, 28 -> 4 rows 132 -> 117 us.
+  static int tile_class(int rows) { return rows <= 16 ? 0 : rows <= 64 ? 1 : rows <= 128 ? 2 : 3; }
+  bool extend_compact() const { return c->tree_fused && tile_class(c->B) < tile_class(c->Te); }
   void draft_logits_fused(int rows) {
     FusedGemmArgs a = fargs(c->h, rows, c->k);
     a.w[0] = (const bf16 *)c->dlm_head; a.O[0] = c->Vd; a.nw = 1;
@@ -562,8 +584,10 @@ template <typename T> struct Sched {
   }
   void tree_step(int pass) {
     mark(SPEC_PROF_TREE);
+    const bool compact = pass == 1 && extend_compact();
     int rc = launch_draft_tree_step(c->st, c->tb, c->meta, c->d2t, pass, c->cand_val, c->cand_idx, c->cand_max, c->cand_sum, c->dtiles,
-                                    draft_tree_cand_ld(c->dtiles), c->x, (const bf16 *)c->embed, (bf16 *)c->cat, c->k, c->inv_freq, c->cs, c->hd / 2, c->B, s);
+                                    draft_tree_cand_ld(c->dtiles), compact ? c->proj : c->x, (const bf16 *)c->embed, (bf16 *)c->cat, c->k, c->inv_freq, c->cs,
+                                    c->hd / 2, c->B, compact, s);
     if (rc && !c->sched_err) c->sched_err = rc;
     tick();
   }
@@ -651,8 +675,8 @@ template <typename T> struct Sched {
 
   // draft head on the rows of c->meta: cat = [feat ; e(tok)], FC2, decoder block, final norm (-> h)
   void draft_forward(const float *feat, int nparts, size_t fstride, const int32_t *src_row, int rows, int tail_len,
-                     bool prebuilt = false) {
-    if (c->fused) return draft_forward_fused(feat, nparts, fstride, src_row, rows, tail_len, prebuilt);
+                     bool prebuilt = false, bool pending = false) {
+    if (c->fused) return draft_forward_fused(feat, nparts, fstride, src_row, rows, tail_len, prebuilt, pending);
     mark(SPEC_PROF_MISC); launch_rope_table(c->meta.pos, rows, c->hd / 2, c->inv_freq, c->cs, s); tick();
     mark(SPEC_PROF_MISC); launch_build_cat<T>(feat, nparts, fstride, src_row, (const T *)c->embed, c->meta.tok, c->meta.seq, (T *)c->cat, rows, c->k, s);
     tick();
@@ -675,8 +699,10 @@ template <typename T> struct Sched {
     size_t lo = (size_t)(pass - 1) * c->Td;
     mark(SPEC_PROF_MISC);
     if (first) {
-      launch_gather_rows(c->logits, c->st.last_row, c->cap_logits + lo * c->Vd, c->B, c->Vd, c->K, s);
-      launch_gather_rows(c->x, c->st.last_row, c->cap_a + lo * c->k, c->B, c->k, c->K, s);
+      const bool compact = c->fused && extend_compact();
+      const int32_t *rows_of = compact ? nullptr : c->st.last_row;
+      launch_gather_rows(c->logits, rows_of, c->cap_logits + lo * c->Vd, c->B, c->Vd, c->K, s);
+      launch_gather_rows(compact ? c->proj : c->x, rows_of, c->cap_a + lo * c->k, c->B, c->k, c->K, s);
     } else if (tl_launch_budget != 0) {
       cudaMemcpyAsync(c->cap_logits + lo * c->Vd, c->logits, (size_t)rows * c->Vd * 4, cudaMemcpyDeviceToDevice, s);
       cudaMemcpyAsync(c->cap_a + lo * c->k, c->x, (size_t)rows * c->k * 4, cudaMemcpyDeviceToDevice, s);
@@ -798,14 +824,7 @@ template <typename T> struct Sched {
   // the first tokens of all sequences, from the rows the passes gathered
   void prefill_finish() {
     if (last_layer_on_last_rows()) {
-      const LayerW &lw = c->tl[c->L - 1];
-      fgemm_resid(c->ao, c->H * c->hd, lw.wo, c->B, true, lw.mlp_norm, 0);
-      FusedGemmArgs g = fargs(c->h, c->B, c->k);
-      g.w[0] = (const bf16 *)lw.w_gate; g.w[1] = (const bf16 *)lw.w_up; g.O[0] = c->F; g.O[1] = c->F; g.nw = 2;
-      with_norm_scale(g);
-      g.act = (bf16 *)c->act;
-      fgemm(EPI_SWIGLU, g);
-      fgemm_resid(c->act, c->F, lw.w_down, c->B, true, c->final_norm, 0);
+      block_tail_fused(c->tl[c->L - 1], c->ao, c->B, c->final_norm, 0, c->x);
     } else {
       launch_residual_norm(c->x, (const bf16 *)c->final_norm, (bf16 *)c->h, c->ssq, c->B, c->k, c->Ralloc, s); tick();
     }
@@ -824,9 +843,10 @@ template <typename T> struct Sched {
       mark(SPEC_PROF_TREE); launch_prep_extend(c->st, c->tb, c->meta, c->B, c->need_pos, c->status, s); tick();
       c->cur_rps = c->Pmax;
       fuse(c->pend_taps, c->Te);
-      draft_forward(c->proj, c->np_proj, c->ps_proj, nullptr, c->Te, c->Pmax);
+      draft_forward(c->proj, c->np_proj, c->ps_proj, nullptr, c->Te, c->Pmax, false, true);
       if (c->tree_fused) {
-        draft_logits_topk(c->Te, c->st.last_row, c->B);
+        if (extend_compact()) draft_logits_topk(c->B, nullptr, 0);
+        else draft_logits_topk(c->Te, c->st.last_row, c->B);
         capture(1, c->Te, true);
         tree_step(1);
       } else {

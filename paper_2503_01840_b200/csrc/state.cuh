@@ -43,10 +43,13 @@ bool draft_tree_step_fits(int tiles, int K);
 int draft_tree_cand_ld(int tiles);      // row pitch (in tiles) of the candidate arrays: tiles rounded up to a multiple of 4
 int launch_draft_tree_step(SeqState st, TreeBufs tb, RowMeta m, const int32_t *d2t, int pass, const float *cand_val,
                            const int32_t *cand_idx, const float *cand_max, const float *cand_sum, int tiles, int ld, const float *x,
-                           const bf16 *embed, bf16 *cat, int k, const double *inv_freq, float2 *cs, int half, int B, cudaStream_t s);
+                           const bf16 *embed, bf16 *cat, int k, const double *inv_freq, float2 *cs, int half, int B,
+                           bool compact /* pass 1: sequence b's row is b, not last_row[b] */, cudaStream_t s);
 // the merge of per-tile candidates alone: idx / lp [rows][K]; -1 when the shape does not fit
 int launch_merge_candidates(const float *cand_val, const int32_t *cand_idx, const float *cand_max, const float *cand_sum, int tiles,
                             int ld, int rows, int K, int32_t *idx, float *lp, cudaStream_t s);
+// row b <- row last_row[b] of the residual stream (fp32, k) and of the attention output (bf16, qd); zeros where last_row < 0
+void launch_gather_pending(const int32_t *last_row, const float *x, float *cx, int k, const bf16 *ao, bf16 *cao, int qd, int B, cudaStream_t s);
 void launch_rerank(SeqState st, TreeBufs tb, RowMeta m, int B, cudaStream_t s);
 void launch_plain_tree(SeqState st, TreeBufs tb, RowMeta m, int B, cudaStream_t s);
 void launch_accept(SeqState st, TreeBufs tb, int B, int rows_per_seq, cudaStream_t s);

@@ -559,6 +559,7 @@ struct TreeStepArgs {
   const float *cand_val, *cand_max, *cand_sum; const int32_t *cand_idx; int tiles, ld;   // [rows][ld][K], [rows][ld]
   const float *x; const bf16 *embed; bf16 *cat; int k;                                    // next pass's FC2 input
   const double *inv_freq; float2 *cs; int half;                                           // next pass's RoPE angles
+  int compact;                    // pass 1: candidates and features are in row b (else in row last_row[b])
 };
 
 constexpr int TREE_WARPS = 10;   // one warp per row of a top-10 level
@@ -581,7 +582,7 @@ __global__ void __launch_bounds__(TREE_THREADS) draft_tree_step_kernel(const Tre
   int32_t *par_u = newf + K;                             // [K] pool index of the node each row of this pass processed
   float *par_sc = (float *)(par_u + K);                  // [K] its score
   const int active = a.st.active[b], n = a.st.n[b];
-  const int src1 = a.st.last_row[b];                     // pass 1: the row that holds the last pending entry's outputs
+  const int src1 = a.compact ? b : a.st.last_row[b];     // pass 1: the row that holds the last pending entry's outputs
   const size_t pb = (size_t)b * (tb.pool + 1);
   const int base = (pass == 1) ? 0 : K + (pass - 2) * K * K;       // pool index of child 0 is base + 1
   const bool writer = blockIdx.y == 0;
@@ -727,13 +728,27 @@ bool draft_tree_step_fits(int tiles, int K) {
 }
 int launch_draft_tree_step(SeqState st, TreeBufs tb, RowMeta m, const int32_t *d2t, int pass, const float *cand_val,
                            const int32_t *cand_idx, const float *cand_max, const float *cand_sum, int tiles, int ld, const float *x,
-                           const bf16 *embed, bf16 *cat, int k, const double *inv_freq, float2 *cs, int half, int B, cudaStream_t s) {
+                           const bf16 *embed, bf16 *cat, int k, const double *inv_freq, float2 *cs, int half, int B, bool compact, cudaStream_t s) {
   if (!draft_tree_step_fits(tiles, tb.K) || ld != draft_tree_cand_ld(tiles) || (k % 8)) return -1;
   const size_t smem = (size_t)((tb.K * tb.K + 3) & ~3) * 4 + (size_t)tb.K * tb.K * 12 + (size_t)tb.K * 12;
-  TreeStepArgs a{st, tb, m, d2t, pass, cand_val, cand_max, cand_sum, cand_idx, tiles, ld, x, embed, cat, k, inv_freq, cs, half};
+  TreeStepArgs a{st, tb, m, d2t, pass, cand_val, cand_max, cand_sum, cand_idx, tiles, ld, x, embed, cat, k, inv_freq, cs, half, compact ? 1 : 0};
   const int Z = B >= 16 ? 1 : 8;        // CTAs per sequence that share the next pass's input assembly
   launch_k(draft_tree_step_kernel, dim3(B, Z), dim3(TREE_THREADS), smem, s, a);
   return 0;
+}
+
+// ---------------------------------------------------------------- the last pending entries of a batch, side by side
+__global__ void __launch_bounds__(256) gather_pending_kernel(const int32_t *__restrict__ last_row, const uint4 *__restrict__ x, uint4 *__restrict__ cx,
+                                                             int x_vecs, const uint4 *__restrict__ ao, uint4 *__restrict__ cao, int ao_vecs) {
+  pdl_wait();
+  pdl_trigger();
+  const int b = blockIdx.x, r = last_row[b];
+  const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+  for (int i = threadIdx.x + blockIdx.y * blockDim.x; i < x_vecs; i += gridDim.y * blockDim.x) cx[(size_t)b * x_vecs + i] = r >= 0 ? x[(size_t)r * x_vecs + i] : zero;
+  for (int i = threadIdx.x + blockIdx.y * blockDim.x; i < ao_vecs; i += gridDim.y * blockDim.x) cao[(size_t)b * ao_vecs + i] = r >= 0 ? ao[(size_t)r * ao_vecs + i] : zero;
+}
+void launch_gather_pending(const int32_t *last_row, const float *x, float *cx, int k, const bf16 *ao, bf16 *cao, int qd, int B, cudaStream_t s) {
+  launch_k(gather_pending_kernel, dim3(B, 4), dim3(256), 0, s, last_row, (const uint4 *)x, (uint4 *)cx, k / 4, (const uint4 *)ao, (uint4 *)cao, qd / 8);
 }
 
 // ---------------------------------------------------------------- pruning + tree assembly

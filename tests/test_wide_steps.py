@@ -1,4 +1,5 @@
-"""Steps whose passes have 129 to 256 rows (the row-major GEMM kernel, split over K slices or not) against the CPU oracle."""
+"""Steps whose passes have 129 to 256 rows (the row-major GEMM kernel, split over K slices or not), and batches whose pass
+over the pending entries goes on with one row per sequence, against the CPU oracle."""
 import pytest
 
 import parity
@@ -23,3 +24,13 @@ def test_wide_verify_passes_vs_oracle(cfg, batch, nodes, sampled):
     prompts = [p.numpy() for p in synth.make_prompts(cfg)]
     st, _ = parity.run_trajectory(cfg, tw, dw, prompts, n_steps=3, tol=2e-2, tap_tol=3e-2, sampling=(0.8, 7) if sampled else None)
     assert st.passes == 3 * cfg.tree_depth * batch and st.verify_compared == 3 * batch, st
+
+
+@pytest.mark.parametrize("batch,depth", [(4, 4), (17, 3), (40, 3), (64, 3)])
+def test_pending_pass_goes_on_with_one_row_per_sequence(batch, depth):
+    """20 -> 4, 68 -> 17, 160 -> 40 and 256 -> 64 rows after the attention of the first draft pass."""
+    cfg = W4.replace(name=f"chain-b{batch}", batch=batch, tree_depth=depth, tree_topk=1, tree_nodes=depth + 1, prompt_lo=5, prompt_hi=40)
+    tw, dw = synth.make_target_weights(cfg), synth.make_draft_weights(cfg)
+    prompts = [p.numpy() for p in synth.make_prompts(cfg)]
+    st, _ = parity.run_trajectory(cfg, tw, dw, prompts, n_steps=3, tol=2e-2, tap_tol=3e-2)
+    assert st.passes == 3 * depth * batch and st.verify_compared == 3 * batch, st
