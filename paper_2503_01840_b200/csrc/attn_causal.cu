@@ -7,15 +7,23 @@
 //
 //  * a CTA owns TWO query tiles of 128 positions that share every K and V tile: two heads of the same KV head (even
 //    groups, same positions, so both tiles have the same key range), or two consecutive blocks of positions (odd groups);
-//  * S = Q K^T of a tile goes to 128 columns of tensor memory; the tile's softmax warpgroup (thread = query row) reads it,
-//    writes P (bf16) over the first 64 of these columns, and O += P V takes P straight from tensor memory.  While one
-//    warpgroup is in its softmax the tensor pipe works for the other tile: P V of step j, then S of step j + 1;
-//  * the P V of step j is issued before the S of step j + 1, so seeing S complete also means that O is up to date: a row
-//    whose reference maximum moves (by more than 2^8, rare after the first steps) rescales its O without a further wait;
-//  * only the tiles that cross the diagonal are masked.
+//  * the scores of a query tile are taken 64 keys at a time into two alternating buffers of tensor memory.  The tile's
+//    softmax warpgroup (thread = query row) reads a buffer, writes P (bf16) over it, and O += P V takes P straight from
+//    tensor memory; behind each P V the scores two steps ahead go into the buffer it freed.  So the scores of the next step
+//    are ready when a warpgroup comes for them, and no contraction lies on its path from one softmax to the next;
+//  * each tile has an MMA-issuing warp of its own (one warp for both spent 1200 of 2230 cycles per 64-key step on waits,
+//    commits and issue while the softmax waited for it);
+//  * a row whose reference maximum moves (by more than 2^8 in the exponent, rare after the first steps) waits for its last
+//    P V and rescales its O; no other step waits for one;
+//  * only the steps that cross the diagonal are masked;
+//  * the diagonal entries of training-time test come through the same K / V ring as further tiles (row = position), whose
+//    dot products the softmax threads take from shared memory.
 //
-// Measured (one B200, T = 8192, 32 / 8 heads, 3 diagonal entries per row): 0.67 ms = 826 TFLOP/s of causal flops; with one
-// 128-row tile per CTA, P in shared memory, partial results through memory and a merge kernel: 1.27 ms.
+// Measured (one B200, T = 8192, 32 / 8 heads, 3 diagonal entries per row): 0.55 ms = 1000 TFLOP/s of causal flops (0.50 ms
+// without diagonal entries).  With one 128-key score buffer per tile and one issuer: 0.67 ms; the same with an issuer per
+// tile and P V in two halves: 0.59 ms; two 64-key buffers and one issuer: 0.68 ms.  A 64-key step takes 1600 cycles: shared
+// memory delivers the operands of its MMAs and takes in the next tiles in 1250 (128 x 64 x 16 MMAs read 6 KB per 32 tensor
+// cycles), the exponentials take 1024.
 //
 // Every wait is bounded; a time-out is recorded in the status words and the CTA winds down.
 #include <math.h>
@@ -38,13 +46,13 @@ using tc::mbar_wait;
 using tc::mbar_wait_warp;
 using tc::smem_u32;
 
-constexpr int CA_HD = 128, CA_T = CAUSAL_TILE;
+constexpr int CA_HD = 128, CA_T = CAUSAL_TILE, CA_KS = 64;      // keys per softmax step
 constexpr int CA_TILE = CA_T * CA_HD * 2;          // 32 KB: a Q, K or V tile
 constexpr int CA_HALF = CA_T * 128;                // 16 KB: 64 of the 128 dimensions of a tile
 constexpr int CA_STAGES = 2;                       // K tiles and V tiles in flight (each)
 constexpr int CA_CTRL = 256;
 constexpr int CA_SMEM = (2 + 2 * CA_STAGES) * CA_TILE + CA_CTRL + 1024;
-// Two softmax warpgroups and one with the TMA warp and the MMA warp.  384 threads start with 168 registers each (64512 in
+// Two softmax warpgroups and one with the TMA warp and the MMA warps.  384 threads start with 168 registers each (64512 in
 // all); the softmax holds a row's 128 scores, so its 256 threads take 208 and the other 128 go down to 88 (64512 again).
 constexpr int CA_THREADS = 384, CA_REGS_SOFTMAX = 208, CA_REGS_ISSUE = 88;
 static_assert(256 * CA_REGS_SOFTMAX + 128 * CA_REGS_ISSUE <= CA_THREADS * 168, "register shares must fit what the block is launched with");
@@ -57,15 +65,16 @@ struct CausalParams {
   const CausalBlock *blocks;
   const bf16 *kd, *vd;
   float *lse;
-  int narrow;                      // out / kd / vd are only 8-byte aligned
+  int narrow;                      // out / kd / vd are only 8-byte aligned: the diagonal entries are read row by row instead
   int32_t *status;
 };
 
-__device__ __forceinline__ uint4 ld_row16(const bf16 *p, int narrow) {
-  if (!narrow) return *(const uint4 *)p;
+// eight elements of a row that starts on an 8-byte boundary
+__device__ __forceinline__ uint4 ld_row8(const bf16 *p) {
   const uint2 a = *(const uint2 *)p, b = *(const uint2 *)(p + 4);
   return make_uint4(a.x, a.y, b.x, b.y);
 }
+__device__ __forceinline__ void mbar_arrive(uint64_t *bar) { asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory"); }
 __device__ __forceinline__ float ex2(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -78,6 +87,11 @@ __device__ __forceinline__ uint32_t pack2(float lo, float hi) {
 __device__ __forceinline__ void load_3d(void *dst, const CUtensorMap *map, int c0, int c1, int c2, uint64_t *bar) {
   asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];" ::"r"(smem_u32(dst)),
                "l"(map), "r"(smem_u32(bar)), "r"(c0), "r"(c1), "r"(c2)
+               : "memory");
+}
+__device__ __forceinline__ void load_4d(void *dst, const CUtensorMap *map, int c0, int c1, int c2, int c3, uint64_t *bar) {
+  asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];" ::"r"(smem_u32(dst)),
+               "l"(map), "r"(smem_u32(bar)), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
                : "memory");
 }
 // D += A B with A (128 x 16 bf16, two elements per column) in tensor memory
@@ -118,14 +132,15 @@ __device__ __forceinline__ float2 bf2(uint32_t u) { return __bfloat1622float2(*(
 // DIAG: the diagonal keys of training-time test are folded in (J may be 0) and the log-normaliser is written
 template <bool DIAG>
 __global__ void __launch_bounds__(CA_THREADS, 1) attn_causal_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
-                                                           const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CausalParams p) {
+                                                           const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_kd,
+                                                           const __grid_constant__ CUtensorMap map_vd, const __grid_constant__ CausalParams p) {
   pdl_trigger();
   pdl_wait();
   extern __shared__ unsigned char smem_raw[];
   unsigned char *sQ = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);   // two tiles [hd half][128 rows][128 B]
   unsigned char *sK = sQ + 2 * CA_TILE, *sV = sK + CA_STAGES * CA_TILE;
   uint64_t *kfull = (uint64_t *)(sV + CA_STAGES * CA_TILE), *kempty = kfull + CA_STAGES, *vfull = kempty + CA_STAGES, *vempty = vfull + CA_STAGES;
-  uint64_t *q_bar = vempty + CA_STAGES, *s_bar = q_bar + 1, *p_bar = s_bar + 2, *o_bar = p_bar + 2;     // the last three: one per tile
+  uint64_t *q_bar = vempty + CA_STAGES, *s_bar = q_bar + 1, *p_bar = s_bar + 4, *o_bar = p_bar + 4;     // s, p: [tile][buffer]; o: [tile]
   uint32_t *tmem_slot = (uint32_t *)(o_bar + 2);
   volatile uint32_t *abort_flag = tmem_slot + 1;
   volatile int *n_filled = (volatile int *)(tmem_slot + 2);     // [0] K tiles, [1] V tiles requested
@@ -144,16 +159,19 @@ __global__ void __launch_bounds__(CA_THREADS, 1) attn_causal_kernel(const __grid
   }
   const int head0 = two_heads ? 2 * blockIdx.x : blockIdx.x;
   const int g = head0 / grp;
-  // tile t of the CTA: rows, first position, key tiles
+  // tile t of the CTA: rows, first position, 64-key steps
   const int rows_0 = min(nrows, CA_T), rows_1 = two_heads ? rows_0 : max(0, nrows - CA_T);
   const int off_1 = two_heads ? 0 : CA_T;
-  const int n0 = (pos0 + rows_0 + CA_T - 1) / CA_T, n1 = rows_1 > 0 ? (pos0 + off_1 + rows_1 + CA_T - 1) / CA_T : 0;
-  const int n = max(n0, n1);
+  const int n0 = (pos0 + rows_0 + CA_KS - 1) / CA_KS, n1 = rows_1 > 0 ? (pos0 + off_1 + rows_1 + CA_KS - 1) / CA_KS : 0;
+  const int n = max(n0, n1), nkt = (n + 1) / 2;     // steps, 128-key tiles
+  const bool diag_ring = DIAG && p.J > 0 && !p.narrow;
+  const int nb = two_heads ? 1 : 2;                 // ring tiles per diagonal step: both query tiles' rows, or one each
 
   if (threadIdx.x == 0) {
-    for (int i = 0; i < CA_STAGES; i++) { mbar_init(&kfull[i], 1); mbar_init(&kempty[i], 1); mbar_init(&vfull[i], 1); mbar_init(&vempty[i], 1); }
+    for (int i = 0; i < CA_STAGES; i++) { mbar_init(&kfull[i], 1); mbar_init(&kempty[i], 2); mbar_init(&vfull[i], 1); mbar_init(&vempty[i], 2); }
     mbar_init(q_bar, 1);
-    for (int i = 0; i < 2; i++) { mbar_init(&s_bar[i], 1); mbar_init(&p_bar[i], 128); mbar_init(&o_bar[i], 1); }
+    for (int i = 0; i < 4; i++) { mbar_init(&s_bar[i], 1); mbar_init(&p_bar[i], 128); }
+    for (int i = 0; i < 2; i++) mbar_init(&o_bar[i], 1);
     *abort_flag = 0;
     n_filled[0] = n_filled[1] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -165,7 +183,7 @@ __global__ void __launch_bounds__(CA_THREADS, 1) attn_causal_kernel(const __grid
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem_base = *tmem_slot;            // S / P of tile t at column 128 t, O at 256 + 128 t
+  const uint32_t tmem_base = *tmem_slot;            // S / P of tile t, buffer u at column 128 t + 64 u, O at 256 + 128 t
 
   if (warp >= 8) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(CA_REGS_ISSUE));
@@ -189,88 +207,105 @@ __global__ void __launch_bounds__(CA_THREADS, 1) attn_causal_kernel(const __grid
         if (page < 0 || page >= p.pm.num_pages) page = fallback;
         return (page * p.G + g) * ps;
       };
-      int cur = page_of(0);
-      for (int j = 0; j < n; j++) {
-        const int nxt = j + 1 < n ? page_of(j + 1) : 0;
+      // one ring tile: wait for its stage, then request it (whole warp; the elected lane issues)
+      auto fill = [&](int kv, int j, auto issue) {
         const int st = j % CA_STAGES;
-        const uint32_t ph = (uint32_t)((j / CA_STAGES) & 1);
+        uint64_t *fb = kv ? &vfull[st] : &kfull[st], *eb = kv ? &vempty[st] : &kempty[st];
+        if (!mbar_wait_warp(eb, (uint32_t)((j / CA_STAGES) & 1) ^ 1u)) {
+          *abort_flag = 1;
+          if (p.status) set_status(p.status, ST_TIMEOUT, 430 + kv, blockIdx.y, j);
+        } else if (elect_one()) {
+          mbar_expect_tx(fb, CA_TILE);
+          issue((kv ? sV : sK) + st * CA_TILE, fb);
+          n_filled[kv] = j + 1;
+        }
+        __syncwarp();
+        return !*abort_flag;
+      };
+      int cur = page_of(0);
+      bool ok = true;
+      for (int j = 0; j < nkt && ok; j++) {
+        const int nxt = j + 1 < nkt ? page_of(j + 1) : 0;
         int row[8];
 #pragma unroll
         for (int i = 0; i < 8; i++) row[i] = __shfl_sync(0xffffffffu, cur, i);
 #pragma unroll
-        for (int kv = 0; kv < 2; kv++) {
-          uint64_t *fb = kv ? &vfull[st] : &kfull[st], *eb = kv ? &vempty[st] : &kempty[st];
-          if (!mbar_wait_warp(eb, ph ^ 1u)) { *abort_flag = 1; if (p.status) set_status(p.status, ST_TIMEOUT, 430 + kv, blockIdx.y, j); break; }
-          if (elect_one()) {
-            unsigned char *d = (kv ? sV : sK) + st * CA_TILE;
-            mbar_expect_tx(fb, CA_TILE);
+        for (int kv = 0; kv < 2; kv++)
+          ok = ok && fill(kv, j, [&](unsigned char *d, uint64_t *fb) {
 #pragma unroll
-            for (int i = 0; i < 8; i++) {
-              if (i >= ppt) break;
+                 for (int i = 0; i < 8; i++) {
+                   if (i >= ppt) break;
 #pragma unroll
-              for (int h = 0; h < 2; h++) load_3d(d + h * CA_HALF + i * ps * 128, kv ? &map_v : &map_k, 0, row[i], h, fb);
-            }
-            n_filled[kv] = j + 1;
-          }
-          __syncwarp();
-        }
-        if (*abort_flag) break;
+                   for (int h = 0; h < 2; h++) load_3d(d + h * CA_HALF + i * ps * 128, kv ? &map_v : &map_k, 0, row[i], h, fb);
+                 }
+               });
         cur = nxt;
       }
-    } else if (warp == 9) {
-      // ================================================================ MMA warp
-      constexpr uint32_t idesc_s = tc::umma_idesc(CA_T);                    // both operands K-major, N = 128 keys
+      if (DIAG && diag_ring) {
+        // the diagonal steps' entries: the first of both rings, then all keys (their dot products come first), then the values
+        auto entry = [&](int kv, int e) {
+          return fill(kv, nkt + e, [&](unsigned char *d, uint64_t *fb) {
+#pragma unroll
+            for (int h = 0; h < 2; h++) load_4d(d + h * CA_HALF, kv ? &map_vd : &map_kd, 64 * h, g, row0 + (e % nb) * CA_T, e / nb, fb);
+          });
+        };
+        const int total = p.J * nb, pre = min(total, CA_STAGES);
+        for (int e = 0; e < pre; e++) ok = ok && entry(0, e) && entry(1, e);
+        for (int e = pre; e < total; e++) ok = ok && entry(0, e);
+        for (int e = pre; e < total; e++) ok = ok && entry(1, e);
+      }
+    } else if (warp <= 10) {
+      // ================================================================ MMA warps: one per query tile
+      // Both release every K and V tile, also those their own query tile has no keys in: they wait for it to land like the
+      // other one.
+      const int t = warp - 9, nt = t ? n1 : n0;
+      constexpr uint32_t idesc_s = tc::umma_idesc(CA_KS);                   // both operands K-major, N = 64 keys
       constexpr uint32_t idesc_o = tc::umma_idesc(CA_HD) | (1u << 16);      // B (the V tile) MN-major, N = 128 dimensions
-      const uint64_t dq = tc::umma_desc_sw128(smem_u32(sQ)), dk = tc::umma_desc_sw128(smem_u32(sK));
+      const uint64_t dq = tc::umma_desc_sw128(smem_u32(sQ + t * CA_TILE)), dk = tc::umma_desc_sw128(smem_u32(sK));
       const uint64_t dv = desc_mn(smem_u32(sV), CA_HALF);
-      auto issue_s = [&](int t, int st) {
+      const uint32_t ts = tmem_base + t * 128, to = tmem_base + 256 + t * 128;
+      // step i: half i % 2 of key tile i / 2, buffer i % 2
+      auto part = [&](int i) { return (uint64_t)((((i >> 1) % CA_STAGES) * CA_TILE + (i & 1) * (CA_KS * 128)) >> 4); };
+      auto issue_s = [&](int i) {
+        const uint64_t kd = dk + part(i);
 #pragma unroll
         for (int kk = 0; kk < 8; kk++) {
           const uint64_t o = (uint64_t)(((kk >> 2) * CA_HALF + (kk & 3) * 32) >> 4);
-          tc::umma_bf16(tmem_base + t * 128, dq + (uint64_t)((t * CA_TILE) >> 4) + o, dk + (uint64_t)((st * CA_TILE) >> 4) + o, idesc_s, kk ? 1u : 0u);
+          tc::umma_bf16(ts + (i & 1) * CA_KS, dq + o, kd + o, idesc_s, kk ? 1u : 0u);
         }
-        tc::umma_commit(&s_bar[t]);
+        tc::umma_commit(&s_bar[t * 2 + (i & 1)]);
       };
       bool ok = mbar_wait_warp(q_bar, 0) && mbar_wait_warp(&kfull[0], 0);
-      if (!ok) { *abort_flag = 1; if (p.status) set_status(p.status, ST_TIMEOUT, 432, blockIdx.y, 0); }
+      if (!ok) { *abort_flag = 1; if (p.status) set_status(p.status, ST_TIMEOUT, 432, blockIdx.y, t); }
       if (ok) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         if (elect_one()) {
-          issue_s(0, 0);
-          if (n1 > 0) issue_s(1, 0);
+          for (int i = 0; i < 2; i++)
+            if (i < nt) issue_s(i);
           tc::umma_commit(&kempty[0]);
         }
         __syncwarp();
-        for (int j = 0; j < n && ok; j++) {
-          const int st = j % CA_STAGES, st1 = (j + 1) % CA_STAGES;
-          bool have_v = false, have_k = false;
-#pragma unroll
-          for (int t = 0; t < 2; t++) {
-            const int nt = t ? n1 : n0;
-            if (j >= nt) continue;
-            ok = mbar_wait_warp(&p_bar[t], (uint32_t)(j & 1));
-            if (ok && !have_v) { ok = mbar_wait_warp(&vfull[st], (uint32_t)((j / CA_STAGES) & 1)); have_v = true; }
-            if (!ok || *abort_flag) { ok = false; *abort_flag = 1; if (p.status) set_status(p.status, ST_TIMEOUT, 433, blockIdx.y, j); break; }
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            if (elect_one()) {
-#pragma unroll
-              for (int kk = 0; kk < 8; kk++)         // 16 keys: 8 columns of P, 16 rows of V
-                umma_ts(tmem_base + 256 + t * 128, tmem_base + t * 128 + kk * 8, dv + (uint64_t)((st * CA_TILE + kk * 16 * 128) >> 4), idesc_o, (j | kk) ? 1u : 0u);
-              if (j + 1 == nt) tc::umma_commit(&o_bar[t]);
-            }
-            __syncwarp();
-            if (j + 1 < nt) {
-              if (!have_k) { ok = mbar_wait_warp(&kfull[st1], (uint32_t)(((j + 1) / CA_STAGES) & 1)); have_k = true; }
-              if (!ok) { *abort_flag = 1; if (p.status) set_status(p.status, ST_TIMEOUT, 434, blockIdx.y, j); break; }
-              asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-              if (elect_one()) issue_s(t, st1);
-              __syncwarp();
-            }
+        for (int i = 0; i < n; i++) {
+          const int st = (i >> 1) % CA_STAGES, st2 = ((i + 2) >> 1) % CA_STAGES;
+          if (!(i & 1)) {                              // a new V tile, and the K tile of the scores that follow it
+            ok = mbar_wait_warp(&vfull[st], (uint32_t)(((i >> 1) / CA_STAGES) & 1));
+            if (ok && i + 2 < n) ok = mbar_wait_warp(&kfull[st2], (uint32_t)((((i + 2) >> 1) / CA_STAGES) & 1));
           }
-          if (!ok) break;
+          if (ok && i < nt) ok = mbar_wait_warp(&p_bar[t * 2 + (i & 1)], (uint32_t)((i >> 1) & 1));
+          if (!ok) { *abort_flag = 1; if (p.status) set_status(p.status, ST_TIMEOUT, 433, blockIdx.y, i); break; }
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           if (elect_one()) {
-            tc::umma_commit(&vempty[st]);
-            if (j + 1 < n) tc::umma_commit(&kempty[st1]);
+            if (i < nt) {
+              const uint64_t vd = dv + part(i);
+#pragma unroll
+              for (int kk = 0; kk < 4; kk++)           // 16 keys: 8 columns of P, 16 rows of V
+                umma_ts(to, ts + (i & 1) * CA_KS + kk * 8, vd + (uint64_t)((kk * 16 * 128) >> 4), idesc_o, (i | kk) ? 1u : 0u);
+              tc::umma_commit(&o_bar[t]);
+            }
+            if (i + 2 < nt) issue_s(i + 2);
+            // the tiles whose last use has been issued
+            if ((i & 1) || i == n - 1) tc::umma_commit(&vempty[st]);
+            if (i + 2 < n && ((i & 1) || i + 2 == n - 1)) tc::umma_commit(&kempty[st2]);
           }
           __syncwarp();
         }
@@ -288,34 +323,38 @@ __global__ void __launch_bounds__(CA_THREADS, 1) attn_causal_kernel(const __grid
     const float sc = rsqrtf((float)CA_HD) * 1.4426950408889634f;                     // softmax scale folded into exp2
     float mx = -INFINITY, l = 0.0f;
     bool alive = true;
-    for (int j = 0; j < nt; j++) {
-      bool ok = mbar_wait_warp(&s_bar[t], (uint32_t)(j & 1));
-      if (!ok || *abort_flag) { if (lane == 0) { *abort_flag = 1; if (p.status) set_status(p.status, ST_TIMEOUT, 435, blockIdx.y, j); } alive = false; break; }
+    for (int i = 0; i < nt; i++) {
+      bool ok = mbar_wait_warp(&s_bar[t * 2 + (i & 1)], (uint32_t)((i >> 1) & 1));
+      if (!ok || *abort_flag) { if (lane == 0) { *abort_flag = 1; if (p.status) set_status(p.status, ST_TIMEOUT, 435, blockIdx.y, i); } alive = false; break; }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      float s[CA_T];
-#pragma unroll
-      for (int c = 0; c < 4; c++) tmem_ld32(my_s + c * 32, s + c * 32);
+      const uint32_t sb = my_s + (uint32_t)((i & 1) * CA_KS);
+      float s[CA_KS];
+      tmem_ld32(sb, s);
+      tmem_ld32(sb + 32, s + 32);
       tmem_ld_wait();
-      const int k0 = j * CA_T;
-      if (k0 + CA_T - 1 > pos - (int)(threadIdx.x & 31)) {       // uniform over the warp: its first row does not see the whole tile
-        const int lim = pos - k0;                                // keys 0..lim of the tile
+      const int k0 = i * CA_KS;
+      if (k0 + CA_KS - 1 > pos - lane) {                         // uniform over the warp: its first row does not see the whole step
+        const int lim = pos - k0;                                // keys 0..lim of the step
 #pragma unroll
-        for (int e = 0; e < CA_T; e++) s[e] = e <= lim ? s[e] : -INFINITY;
+        for (int e = 0; e < CA_KS; e++) s[e] = e <= lim ? s[e] : -INFINITY;
       }
       float m4[4] = {s[0], s[1], s[2], s[3]};
 #pragma unroll
-      for (int e = 4; e < CA_T; e += 4) {
+      for (int e = 4; e < CA_KS; e += 4) {
 #pragma unroll
         for (int z = 0; z < 4; z++) m4[z] = fmaxf(m4[z], s[e + z]);
       }
       const float tm = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
-      // the reference maximum moves only when the tile's exceeds it by more than 2^8 in the exponent
+      // the reference maximum moves only when the step's exceeds it by more than 2^8 in the exponent
       float f = 1.0f;
       if (tm > mx && (mx == -INFINITY || (tm - mx) * sc > 8.0f)) {
         f = (mx == -INFINITY) ? 1.0f : ex2((mx - tm) * sc);
         mx = tm;
       }
-      if (j > 0 && __any_sync(0xffffffffu, f != 1.0f)) {         // S of this step is complete, hence the P V of the last one
+      if (i > 0 && __any_sync(0xffffffffu, f != 1.0f)) {         // the P V of the last step must be complete before O is rescaled
+        ok = mbar_wait_warp(&o_bar[t], (uint32_t)((i - 1) & 1));
+        if (!ok) { if (lane == 0) { *abort_flag = 1; if (p.status) set_status(p.status, ST_TIMEOUT, 438, blockIdx.y, i); } alive = false; break; }
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll 1
         for (int c = 0; c < 4; c++) {
           float o[32];
@@ -326,97 +365,142 @@ __global__ void __launch_bounds__(CA_THREADS, 1) attn_causal_kernel(const __grid
           tmem_st32(my_o + c * 32, (uint32_t *)o);
         }
       }
-      const float nb = (mx == -INFINITY) ? 0.0f : mx * sc;
+      const float nb_ = (mx == -INFINITY) ? 0.0f : mx * sc;
       float rs[4] = {0.f, 0.f, 0.f, 0.f};
+      uint32_t pk[32];
 #pragma unroll
-      for (int c = 0; c < 2; c++) {
-        uint32_t pk[32];
-#pragma unroll
-        for (int e = 0; e < 32; e++) {
-          const float p0 = ex2(fmaf(s[c * 64 + 2 * e], sc, -nb)), p1 = ex2(fmaf(s[c * 64 + 2 * e + 1], sc, -nb));
-          rs[(2 * e) & 3] += p0; rs[(2 * e + 1) & 3] += p1;
-          pk[e] = pack2(p0, p1);
-        }
-        tmem_st32(my_s + c * 32, pk);
+      for (int e = 0; e < 32; e++) {
+        const float p0 = ex2(fmaf(s[2 * e], sc, -nb_)), p1 = ex2(fmaf(s[2 * e + 1], sc, -nb_));
+        rs[(2 * e) & 3] += p0; rs[(2 * e + 1) & 3] += p1;
+        pk[e] = pack2(p0, p1);
       }
+      tmem_st32(sb, pk);
       l = l * f + ((rs[0] + rs[1]) + (rs[2] + rs[3]));
       tmem_st_wait();
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&p_bar[t])) : "memory");
+      mbar_arrive(&p_bar[t * 2 + (i & 1)]);
     }
     if (alive && nt > 0) {
-      bool ok = mbar_wait_warp(&o_bar[t], 0);
+      // the scores of the last step only tell that the P V two steps earlier is complete: one phase after the other
+      bool ok = nt < 2 || mbar_wait_warp(&o_bar[t], (uint32_t)((nt - 2) & 1));
+      ok = ok && mbar_wait_warp(&o_bar[t], (uint32_t)((nt - 1) & 1));
       if (!ok || *abort_flag) { if (lane == 0) { *abort_flag = 1; if (p.status) set_status(p.status, ST_TIMEOUT, 436, blockIdx.y, nt); } alive = false; }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     }
-    if (alive && nt > 0) {
-      unsigned char *qt = sQ + t * CA_TILE;                      // this row's 16-byte chunk c: half c / 8, row lr, chunk (c % 8) ^ (lr % 8)
-      auto chunk = [&](int r, int c) { return (uint4 *)(qt + (c >> 3) * CA_HALF + r * 128 + (((c & 7) ^ (r & 7)) << 4)); };
-      const bool rv = lr < nr;
-      float fo = 1.0f, wd[CA_MAX_DIAG];
-      size_t doff = 0;
-      if (DIAG) {
-        doff = ((size_t)(rv ? trow + lr : 0) * p.G + g) * CA_HD;
-        const size_t dstep = (size_t)p.T * p.G * CA_HD;
-        float d[CA_MAX_DIAG];
+    unsigned char *qt = sQ + t * CA_TILE;                        // this row's 16-byte chunk c: half c / 8, row lr, chunk (c % 8) ^ (lr % 8)
+    auto chunk = [](unsigned char *tile, int r, int c) { return (uint4 *)(tile + (c >> 3) * CA_HALF + r * 128 + (((c & 7) ^ (r & 7)) << 4)); };
+    const bool rv = lr < nr;
+    float fo = 1.0f, wd[CA_MAX_DIAG];
+    size_t doff = 0;
+    const size_t dstep = (size_t)p.T * p.G * CA_HD;
+    if (DIAG) {
+      doff = ((size_t)(rv ? trow + lr : 0) * p.G + g) * CA_HD;
+      float d[CA_MAX_DIAG];
 #pragma unroll
-        for (int s = 0; s < CA_MAX_DIAG; s++) d[s] = 0.0f;
-        if (p.J > 0) {
-#pragma unroll 2
-          for (int c = 0; c < 16; c++) {
-            const uint4 qv = *chunk(lr, c);
-            const float2 q0 = bf2(qv.x), q1 = bf2(qv.y), q2 = bf2(qv.z), q3 = bf2(qv.w);
-#pragma unroll
-            for (int s = 0; s < CA_MAX_DIAG; s++)
-              if (s < p.J) {
-                const uint4 kv = ld_row16(p.kd + s * dstep + doff + c * 8, p.narrow);
-                const float2 k0 = bf2(kv.x), k1 = bf2(kv.y), k2 = bf2(kv.z), k3 = bf2(kv.w);
-                d[s] += ((q0.x * k0.x + q0.y * k0.y) + (q1.x * k1.x + q1.y * k1.y)) + ((q2.x * k2.x + q2.y * k2.y) + (q3.x * k3.x + q3.y * k3.y));
-              }
-          }
-        }
-        float M = mx;
+      for (int s = 0; s < CA_MAX_DIAG; s++) d[s] = 0.0f;
+      auto dot8 = [](const uint4 &a, const uint4 &b) {
+        const float2 a0 = bf2(a.x), a1 = bf2(a.y), a2 = bf2(a.z), a3 = bf2(a.w), b0 = bf2(b.x), b1 = bf2(b.y), b2 = bf2(b.z), b3 = bf2(b.w);
+        return ((a0.x * b0.x + a0.y * b0.y) + (a1.x * b1.x + a1.y * b1.y)) + ((a2.x * b2.x + a2.y * b2.y) + (a3.x * b3.x + a3.y * b3.y));
+      };
+      if (diag_ring) {
 #pragma unroll
         for (int s = 0; s < CA_MAX_DIAG; s++)
-          if (s < p.J) M = fmaxf(M, d[s]);
-        fo = ex2((mx - M) * sc);
-        l *= fo;
+          if (s < p.J) {
+            const int j = nkt + s * nb + (two_heads ? 0 : t), st = j % CA_STAGES;
+            const bool ok = mbar_wait_warp(&kfull[st], (uint32_t)((j / CA_STAGES) & 1));
+            if (!ok) { if (lane == 0) { *abort_flag = 1; if (p.status) set_status(p.status, ST_TIMEOUT, 439, blockIdx.y, s); } alive = false; }
+            if (alive) {
+#pragma unroll 4
+              for (int c = 0; c < 16; c++) d[s] += dot8(*chunk(qt, lr, c), *chunk(sK + st * CA_TILE, lr, c));
+            }
+            asm volatile("bar.sync 1, 256;" ::: "memory");       // both tiles' threads are done with the step's ring tiles
+            if ((threadIdx.x & 127) == 0)                        // one arrival per query tile, as from the MMA warps
+              for (int tb = 0; tb < nb; tb++) mbar_arrive(&kempty[(nkt + s * nb + tb) % CA_STAGES]);
+          }
+      } else if (p.J > 0 && alive && nt > 0) {
+#pragma unroll 2
+        for (int c = 0; c < 16; c++) {
+          const uint4 qv = *chunk(qt, lr, c);
 #pragma unroll
-        for (int s = 0; s < CA_MAX_DIAG; s++) {
-          wd[s] = s < p.J ? exp2f((d[s] - M) * sc) : 0.0f;
-          l += wd[s];
+          for (int s = 0; s < CA_MAX_DIAG; s++)
+            if (s < p.J) d[s] += dot8(qv, ld_row8(p.kd + s * dstep + doff + c * 8));
         }
-        if (p.lse && rv) p.lse[(size_t)(trow + lr) * p.H + head] = logf(l) + M * rsqrtf((float)CA_HD);
       }
-      const float inv = l > 0.0f ? 1.0f / l : 0.0f;
-      __syncwarp();                                              // every lane has read its q row: the tile becomes the output staging
+      float M = mx;
+#pragma unroll
+      for (int s = 0; s < CA_MAX_DIAG; s++)
+        if (s < p.J) M = fmaxf(M, d[s]);
+      fo = ex2((mx - M) * sc);
+      l *= fo;
+#pragma unroll
+      for (int s = 0; s < CA_MAX_DIAG; s++) {
+        wd[s] = s < p.J ? exp2f((d[s] - M) * sc) : 0.0f;
+        l += wd[s];
+      }
+      if (p.lse && rv && alive && nt > 0) p.lse[(size_t)(trow + lr) * p.H + head] = logf(l) + M * rsqrtf((float)CA_HD);
+    }
+    const float inv = l > 0.0f ? 1.0f / l : 0.0f;
+    __syncwarp();                                                // every lane has read its q row: the tile becomes the output staging
+    auto add8 = [](float *o, float w, const uint4 &v) {
+      const float2 v0 = bf2(v.x), v1 = bf2(v.y), v2 = bf2(v.z), v3 = bf2(v.w);
+      o[0] += w * v0.x; o[1] += w * v0.y; o[2] += w * v1.x; o[3] += w * v1.y; o[4] += w * v2.x; o[5] += w * v2.y; o[6] += w * v3.x; o[7] += w * v3.y;
+    };
+    auto put32 = [&](int c, const float *o) {
+#pragma unroll
+      for (int u = 0; u < 4; u++)
+        *chunk(qt, lr, c * 4 + u) = make_uint4(pack2(o[u * 8] * inv, o[u * 8 + 1] * inv), pack2(o[u * 8 + 2] * inv, o[u * 8 + 3] * inv),
+                                               pack2(o[u * 8 + 4] * inv, o[u * 8 + 5] * inv), pack2(o[u * 8 + 6] * inv, o[u * 8 + 7] * inv));
+    };
+    if (DIAG && diag_ring) {
+      float o[CA_HD];                                            // the whole row in registers: every step's values pass by once
+      if (alive && nt > 0) {
+#pragma unroll
+        for (int c = 0; c < 4; c++) tmem_ld32(my_o + c * 32, o + c * 32);
+        tmem_ld_wait();
+#pragma unroll
+        for (int e = 0; e < CA_HD; e++) o[e] *= fo;
+      }
+#pragma unroll 1
+      for (int s = 0; s < p.J; s++) {
+        const int j = nkt + s * nb + (two_heads ? 0 : t), st = j % CA_STAGES;
+        const bool ok = mbar_wait_warp(&vfull[st], (uint32_t)((j / CA_STAGES) & 1));
+        if (!ok) { if (lane == 0) { *abort_flag = 1; if (p.status) set_status(p.status, ST_TIMEOUT, 440, blockIdx.y, s); } alive = false; }
+        if (alive && nt > 0) {
+          float w = 0.0f;
+#pragma unroll
+          for (int z = 0; z < CA_MAX_DIAG; z++) w = z == s ? wd[z] : w;
+#pragma unroll
+          for (int c = 0; c < 16; c++) add8(o + c * 8, w, *chunk(sV + st * CA_TILE, lr, c));
+        }
+        asm volatile("bar.sync 1, 256;" ::: "memory");
+        if ((threadIdx.x & 127) == 0)
+          for (int tb = 0; tb < nb; tb++) mbar_arrive(&vempty[(nkt + s * nb + tb) % CA_STAGES]);
+      }
+      if (alive && nt > 0) {
+#pragma unroll
+        for (int c = 0; c < 4; c++) put32(c, o + c * 32);
+      }
+    } else if (alive && nt > 0) {
 #pragma unroll 1
       for (int c = 0; c < 4; c++) {
         float o[32];
         tmem_ld32(my_o + c * 32, o);
         tmem_ld_wait();
         if (DIAG) {
-          const size_t dstep = (size_t)p.T * p.G * CA_HD;
 #pragma unroll
           for (int e = 0; e < 32; e++) o[e] *= fo;
 #pragma unroll
           for (int s = 0; s < CA_MAX_DIAG; s++)
             if (s < p.J) {
 #pragma unroll
-              for (int u = 0; u < 4; u++) {
-                const uint4 vv = ld_row16(p.vd + s * dstep + doff + c * 32 + u * 8, p.narrow);
-                const float2 v0 = bf2(vv.x), v1 = bf2(vv.y), v2 = bf2(vv.z), v3 = bf2(vv.w);
-                o[u * 8 + 0] += wd[s] * v0.x; o[u * 8 + 1] += wd[s] * v0.y; o[u * 8 + 2] += wd[s] * v1.x; o[u * 8 + 3] += wd[s] * v1.y;
-                o[u * 8 + 4] += wd[s] * v2.x; o[u * 8 + 5] += wd[s] * v2.y; o[u * 8 + 6] += wd[s] * v3.x; o[u * 8 + 7] += wd[s] * v3.y;
-              }
+              for (int u = 0; u < 4; u++) add8(o + u * 8, wd[s], ld_row8(p.vd + s * dstep + doff + c * 32 + u * 8));
             }
         }
-#pragma unroll
-        for (int u = 0; u < 4; u++)
-          *chunk(lr, c * 4 + u) = make_uint4(pack2(o[u * 8] * inv, o[u * 8 + 1] * inv), pack2(o[u * 8 + 2] * inv, o[u * 8 + 3] * inv),
-                                             pack2(o[u * 8 + 4] * inv, o[u * 8 + 5] * inv), pack2(o[u * 8 + 6] * inv, o[u * 8 + 7] * inv));
+        put32(c, o);
       }
-      __syncwarp();
+    }
+    __syncwarp();
+    if (alive && nt > 0) {
       // a warp's 32 rows, two whole rows (256 bytes each) per instruction
       const int rw = (warp & 3) * 32;
 #pragma unroll 4
@@ -424,7 +508,7 @@ __global__ void __launch_bounds__(CA_THREADS, 1) attn_causal_kernel(const __grid
         const int r = rw + 2 * i + (lane >> 4), c = lane & 15;
         if (r < nr) {
           bf16 *dst = p.out + ((size_t)(trow + r) * p.H + head) * CA_HD + c * 8;
-          const uint4 v = *chunk(r, c);
+          const uint4 v = *chunk(qt, r, c);
           if (DIAG && p.narrow) { *(uint2 *)dst = make_uint2(v.x, v.y); *(uint2 *)(dst + 4) = make_uint2(v.z, v.w); }
           else *(uint4 *)dst = v;
         }
@@ -449,12 +533,15 @@ int launch_causal_attn(const CausalArgs &a, cudaStream_t s) {
   if (a.J > CA_MAX_DIAG || a.H % a.G) return -1;
   const int grp = a.H / a.G;
   const CUtensorMap *mk = kv_map(a.pool.k, a.pm.num_pages, a.G, a.pm.page_size, CA_HD, 1), *mv = kv_map(a.pool.v, a.pm.num_pages, a.G, a.pm.page_size, CA_HD, 1);
-  CUtensorMap mq;
+  CUtensorMap mq, mkd, mvd;
+  memset(&mkd, 0, sizeof mkd);
+  memset(&mvd, 0, sizeof mvd);
   if (!mk || !mv || !q_map(&mq, a.q, a.q_rows, a.H, CA_T)) return -6;
   CausalParams p;
   memset(&p, 0, sizeof p);
   p.pm = a.pm; p.out = a.out; p.H = a.H; p.G = a.G; p.T = a.T; p.J = a.J; p.blocks = a.blocks; p.kd = a.kd; p.vd = a.vd; p.lse = a.lse;
   p.narrow = (((uintptr_t)a.out | (uintptr_t)a.kd | (uintptr_t)a.vd) & 15) ? 1 : 0;
+  if (a.J > 0 && !p.narrow && (!diag_map(&mkd, a.kd, a.J, a.T, a.G, CA_T) || !diag_map(&mvd, a.vd, a.J, a.T, a.G, CA_T))) return -6;
   p.status = a.status;
   const int br = causal_block_rows(grp);
   dim3 grid(grp % 2 == 0 ? a.H / 2 : a.H, a.blocks ? a.n_blocks : (a.T + br - 1) / br);
@@ -462,10 +549,10 @@ int launch_causal_attn(const CausalArgs &a, cudaStream_t s) {
   const bool diag = !a.blocks;
   if (diag) {
     if (!limit[1].ensure(attn_causal_kernel<true>, CA_SMEM)) return -6;
-    launch_k(attn_causal_kernel<true>, grid, dim3(CA_THREADS), (size_t)CA_SMEM, s, mq, *mk, *mv, p);
+    launch_k(attn_causal_kernel<true>, grid, dim3(CA_THREADS), (size_t)CA_SMEM, s, mq, *mk, *mv, mkd, mvd, p);
   } else {
     if (!limit[0].ensure(attn_causal_kernel<false>, CA_SMEM)) return -6;
-    launch_k(attn_causal_kernel<false>, grid, dim3(CA_THREADS), (size_t)CA_SMEM, s, mq, *mk, *mv, p);
+    launch_k(attn_causal_kernel<false>, grid, dim3(CA_THREADS), (size_t)CA_SMEM, s, mq, *mk, *mv, mkd, mvd, p);
   }
   return 0;
 }

@@ -1289,6 +1289,17 @@ bool q_map(CUtensorMap *out, const void *q, int rows, int H, int box_rows) {
                 CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+bool diag_map(CUtensorMap *out, const void *kd, int J, int T, int G, int box_rows) {
+  EncodeFn encode = encode_fn();
+  if (!encode) return false;
+  cuuint64_t dims[4] = {128, (cuuint64_t)G, (cuuint64_t)T, (cuuint64_t)J};
+  cuuint64_t strides[3] = {256, (cuuint64_t)G * 256, (cuuint64_t)T * G * 256};
+  cuuint32_t box[4] = {64, 1, (cuuint32_t)box_rows, 1};
+  cuuint32_t estr[4] = {1, 1, 1, 1};
+  return encode(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, (void *)kd, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 namespace {
 template <int HD>
 int launch_tma_small(AttnParams &p, dim3 grid, const CUtensorMap *mk, const CUtensorMap *mv, int32_t *status, cudaStream_t s) {

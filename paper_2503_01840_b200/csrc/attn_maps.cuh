@@ -13,5 +13,8 @@ const CUtensorMap *kv_map(const void *pool, int num_pages, int G, int ps, int hd
 // q [rows][H][128] as {128 elements, H heads, rows}: one box = 64 elements of `box_rows` rows of one head, 128-byte
 // swizzle.  Not cached (the pointer may be a caller's); false if refused.
 bool q_map(CUtensorMap *out, const void *q, int rows, int H, int box_rows);
+// kd / vd [J][T][G][128] as {128 elements, G heads, T positions, J steps}: one box = 64 elements of `box_rows` positions of
+// one head and step, 128-byte swizzle.  Not cached; false if refused.
+bool diag_map(CUtensorMap *out, const void *kd, int J, int T, int G, int box_rows);
 
 }  // namespace spec
