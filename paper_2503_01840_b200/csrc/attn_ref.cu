@@ -88,8 +88,25 @@ __global__ void __launch_bounds__(128) attn_ref_kernel(const T *__restrict__ q, 
   __syncthreads();
   sum = red[0] + red[1] + red[2] + red[3];
   const float inv = 1.0f / sum;
+  const int n_dim = hd >> 2;
+  if (n_dim > 128) {                                      // more groups of four dimensions than threads: a thread takes several, over all keys
+    for (int dim = threadIdx.x; dim < n_dim; dim += 128) {
+      float4 acc = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll 4
+      for (int j = 0; j < nk; j++) {
+        const float p = sc[j];
+        if (p == 0.0f) continue;
+        const int pos = j < ctx ? j : tb + (j - ctx);
+        const float4 a = load4<VEC>(Vp + kv_offset(pm, seq, pos, g, G, hd) + dim * 4);
+        acc.x = fmaf(p, a.x, acc.x); acc.y = fmaf(p, a.y, acc.y); acc.z = fmaf(p, a.z, acc.z); acc.w = fmaf(p, a.w, acc.w);
+      }
+      o[dim * 4] = from_f32<T>(acc.x * inv); o[dim * 4 + 1] = from_f32<T>(acc.y * inv);
+      o[dim * 4 + 2] = from_f32<T>(acc.z * inv); o[dim * 4 + 3] = from_f32<T>(acc.w * inv);
+    }
+    return;
+  }
   // values: thread = (four dimensions, every n_grp-th key)
-  const int n_dim = hd >> 2, n_grp = 128 / n_dim, dim = threadIdx.x % n_dim, grp = threadIdx.x / n_dim;
+  const int n_grp = 128 / n_dim, dim = threadIdx.x % n_dim, grp = threadIdx.x / n_dim;
   float4 acc = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
   if (grp < n_grp) {
 #pragma unroll 4

@@ -54,3 +54,21 @@ def test_fp32_attention_vs_fp64(H, G, hd, ctx, tail, ps):
         p = np.exp(s - s.max(1, keepdims=True))
         ref = (p / p.sum(1, keepdims=True)) @ vd[:, h // (H // G)]
         assert np.abs(out[:, h].cpu().double().numpy() - ref).max() < 5e-6          # scores of order 1 .. 3 in fp32, sums of ~200 terms
+
+
+@pytest.mark.parametrize("dtype,tol", [(torch.float32, 5e-6), (torch.bfloat16, 2e-2)])
+@pytest.mark.parametrize("hd", [512, 528, 576, 1040])
+def test_plain_attention_wide_heads_vs_fp64(hd, dtype, tol):
+    """Head dimensions around and above four times the threads of a CTA, where a thread owns several groups of dimensions."""
+    rows, H, G, ctx, tail, ps = 3, 2, 1, 37, 3, 16
+    g = torch.Generator().manual_seed(hd)
+    pages = (ctx + tail + ps - 1) // ps
+    q, kp, vp = (torch.randn(*s, generator=g).to(dtype) for s in ((rows, H, hd), (pages, G, ps, hd), (pages, G, ps, hd)))
+    full = lambda c: torch.full((rows,), c, dtype=torch.int32, device="cuda")
+    lo, hi = torch.full((rows,), 7, dtype=torch.int64, device="cuda"), torch.zeros(rows, dtype=torch.int64, device="cuda")
+    table = torch.arange(pages, dtype=torch.int32, device="cuda").view(1, -1)
+    out = sb.attention(q.cuda(), kp.cuda(), vp.cuda(), table, ps, full(0), full(ctx), full(ctx), lo, hi, tail, G, ctx + tail, impl=1)
+    k, v = (t.double()[:, 0].reshape(pages * ps, hd)[: ctx + tail] for t in (kp, vp))
+    ref = torch.softmax(q.double() @ k.T / hd ** 0.5, -1) @ v
+    # fp32: scores of order 1 .. 3 and sums of 40 terms; bf16: one rounding of outputs of order 1
+    assert (out.cpu().double() - ref).abs().max() < tol
