@@ -471,7 +471,10 @@ template <typename T> struct Sched {
   void fgemm(FusedEpi epi, FusedGemmArgs a) {
     prof_mark(SPEC_PROF_GEMM);
     a.stamp = next_stamp(SPEC_PROF_GEMM);
-    int rc = row_major(epi, a) ? wide_gemm_launch(c->fg, wide_epi(epi), widened(a), s) : fused_gemm_launch(c->fg, epi, a, s);
+    const WideGemmArgs w = widened(a);
+    // (draft logits of a vocabulary that is no multiple of eight stay on the weight-streaming kernel)
+    const bool wide = row_major(epi, a) && wide_gemm_supported(wide_epi(epi), w);
+    int rc = wide ? wide_gemm_launch(c->fg, wide_epi(epi), w, s) : fused_gemm_launch(c->fg, epi, a, s);
     if (rc && !c->sched_err) c->sched_err = rc;
     tick();
   }

@@ -1052,13 +1052,20 @@ long long wide_gemm_cost(WideEpi epi, const int *O, int nw, int I, int row_tiles
   return plan_split(epi, n_tiles_of(epi, O, nw) * row_tiles, (I + TILE_K - 1) / TILE_K, &S);
 }
 
+// The epilogues store four or eight features at a time (only the argmax one's logits are stored one by one).
+bool wide_gemm_supported(WideEpi epi, const WideGemmArgs &a) {
+  if (a.rows < 1 || a.rows > a.x_rows || a.I < 8 || (a.I % 8) || ((uintptr_t)a.x & 15)) return false;
+  if (a.nw < 1 || a.nw > 3 || (epi == WIDE_SWIGLU && (a.nw != 2 || a.O[0] != a.O[1])) || (epi == WIDE_QKV && a.nw < 2)) return false;
+  for (int j = 0; j < a.nw; j++)
+    if (!a.w[j] || ((uintptr_t)a.w[j] & 15) || a.O[j] < 1 || (epi != WIDE_ARGMAX && (a.O[j] % 8))) return false;
+  return epi != WIDE_F32 || ((a.ldo % 4) == 0 && ((uintptr_t)a.out_f32 & 15) == 0);
+}
+
 int wide_gemm_launch(TmaMaps *g, WideEpi epi, const WideGemmArgs &a, cudaStream_t s) {
-  if (!g || a.rows < 1 || a.rows > a.x_rows || a.I < 8 || (a.I % 8) || ((uintptr_t)a.x & 15)) return -1;
-  if (a.nw < 1 || a.nw > 3 || (epi == WIDE_SWIGLU && (a.nw != 2 || a.O[0] != a.O[1])) || (epi == WIDE_QKV && a.nw < 2)) return -1;
+  if (!g || !wide_gemm_supported(epi, a)) return -1;
   WideParams p;
   memset(&p, 0, sizeof p);
   for (int j = 0; j < a.nw; j++) {
-    if (!a.w[j] || ((uintptr_t)a.w[j] & 15) || a.O[j] < 1 || (epi != WIDE_ARGMAX && (a.O[j] % 8))) return -1;
     const CUtensorMap *mw = tma_maps_get(g, a.w[j], a.O[j], a.I, W_HALF);
     if (!mw) return -6;
     p.map_w[j] = *mw;

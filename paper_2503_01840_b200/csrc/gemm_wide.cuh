@@ -60,7 +60,9 @@ struct WideGemmArgs {
 constexpr int WIDE_ROWS = 256;      // token rows per tile
 // what the launch's time goes with, in k-blocks (64 elements of the contraction, 0.27 us) of a tile
 long long wide_gemm_cost(WideEpi epi, const int *O, int nw, int I, int row_tiles);
-// Returns 0 or a negative code (-1: the shape does not fit).
+// whether a launch takes these widths and alignments
+bool wide_gemm_supported(WideEpi epi, const WideGemmArgs &a);
+// Returns 0 or a negative code (-1: not supported).
 int wide_gemm_launch(TmaMaps *g, WideEpi epi, const WideGemmArgs &a, cudaStream_t s);
 
 }  // namespace spec

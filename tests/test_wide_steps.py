@@ -34,3 +34,15 @@ def test_pending_pass_goes_on_with_one_row_per_sequence(batch, depth):
     prompts = [p.numpy() for p in synth.make_prompts(cfg)]
     st, _ = parity.run_trajectory(cfg, tw, dw, prompts, n_steps=3, tol=2e-2, tap_tol=3e-2)
     assert st.passes == 3 * depth * batch and st.verify_compared == 3 * batch, st
+
+
+@pytest.mark.parametrize("batch,draft_vocab", [(9, 1003), (9, 1008), (16, 1002)])
+def test_unfused_draft_logits_of_wide_passes(batch, draft_vocab):
+    """Sixteen candidates per node: the draft logits are written out (144 and 256 rows), for vocabularies that are and are
+    not a multiple of eight."""
+    cfg = W4.replace(name=f"k16-b{batch}-v{draft_vocab}", batch=batch, draft_vocab=draft_vocab, tree_depth=2, tree_topk=16, tree_nodes=16,
+                     prompt_lo=5, prompt_hi=40)
+    tw, dw = synth.make_target_weights(cfg), synth.make_draft_weights(cfg)
+    prompts = [p.numpy() for p in synth.make_prompts(cfg)]
+    st, _ = parity.run_trajectory(cfg, tw, dw, prompts, n_steps=2, tol=2e-2, tap_tol=3e-2)
+    assert st.passes == 2 * 2 * batch and st.verify_compared == 2 * batch, st
