@@ -53,7 +53,7 @@ struct alignas(64) WideParams {
   int O[3];
   int kind0;                     // WIDE_QKV: what w0 is (0 q, 1 k)
   const float *ssq_in; int ssq_in_tiles, ssq_ld; float inv_k_in, eps;
-  float *xres; const bf16 *gain; bf16 *hb; float *ssq_out; bf16 *taps; int tap_mask, resid_add;
+  float *xres; const bf16 *gain; int gain_vec; bf16 *hb; float *ssq_out; bf16 *taps; int tap_mask, resid_add;
   const float2 *cs; const int32_t *slot, *seq, *kvpos; PageMap pm; bf16 *q; bf16 *kp, *vp; int H, G, page_size;
   bf16 *act;
   bf16 *out_b; int ldo;
@@ -81,6 +81,15 @@ __device__ __forceinline__ float row_scale(const WideParams &p, int row) {
 #pragma unroll 8
   for (int u = 0; u < p.ssq_in_tiles; u++) ss += p.ssq_in[(size_t)u * p.ssq_ld + row];
   return 1.0f / sqrtf(ss * p.inv_k_in + p.eps);
+}
+
+// norm gains of features f .. f + 3; they are the caller's, who owes them no alignment beyond their own two bytes
+__device__ __forceinline__ float4 load_gain(const WideParams &p, int f) {
+  const bf16 *g = p.gain + f;
+  if (!p.gain_vec) return make_float4(to_f32(g[0]), to_f32(g[1]), to_f32(g[2]), to_f32(g[3]));
+  const uint2 u = *(const uint2 *)g;
+  const float2 g01 = __bfloat1622float2(*(const __nv_bfloat162 *)&u.x), g23 = __bfloat1622float2(*(const __nv_bfloat162 *)&u.y);
+  return make_float4(g01.x, g01.y, g23.x, g23.y);
 }
 
 __device__ __forceinline__ void cluster_sync_all() {
@@ -336,11 +345,7 @@ __global__ void __launch_bounds__(W_THREADS, 1) gemm_wide_kernel(const __grid_co
               }
             }
             float4 gn = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (fok) {
-              const uint2 g = *(const uint2 *)(p.gain + f);
-              const float2 g01 = __bfloat1622float2(*(const __nv_bfloat162 *)&g.x), g23 = __bfloat1622float2(*(const __nv_bfloat162 *)&g.y);
-              gn = make_float4(g01.x, g01.y, g23.x, g23.y);
-            }
+            if (fok) gn = load_gain(p, f);
 #pragma unroll
             for (int i = 0; i < 8; i++) {
               const int gr = row_w + i * 4 + sub;
@@ -675,11 +680,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1) gemm_wide_split_kernel(const __
     const int kind = mi + p.kind0;
     const bool fok = good && (EPI == WIDE_QKV ? tm * 128 < p.O[mi] : fo < p.O[0]);
     float4 gn = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (EPI == WIDE_RESID && fok) {
-      const uint2 g = *(const uint2 *)(p.gain + fo);
-      const float2 g01 = __bfloat1622float2(*(const __nv_bfloat162 *)&g.x), g23 = __bfloat1622float2(*(const __nv_bfloat162 *)&g.y);
-      gn = make_float4(g01.x, g01.y, g23.x, g23.y);
-    }
+    if (EPI == WIDE_RESID && fok) gn = load_gain(p, fo);
     constexpr int RB = S == 3 ? 6 : 4;                         // rows in flight per warp: a full tile's share in one or two batches
     for (int rb = r0 + sub; rb < r1; rb += 8 * RB) {
       float4 xin[RB];
@@ -1080,7 +1081,7 @@ int wide_gemm_launch(TmaMaps *g, WideEpi epi, const WideGemmArgs &a, cudaStream_
   p.h1 = a.nw > 2 ? p.h0 + (a.O[1] + 127) / 128 : 1 << 30;
   p.kind0 = a.nw == 3 ? 0 : 1;
   p.ssq_in = a.ssq_in; p.ssq_in_tiles = a.ssq_in_tiles; p.ssq_ld = a.ssq_ld; p.inv_k_in = 1.0f / (float)a.k_in; p.eps = a.eps;
-  p.xres = a.xres; p.gain = a.gain; p.hb = a.hb; p.ssq_out = a.ssq_out; p.taps = a.taps; p.tap_mask = a.taps ? a.tap_mask : 0; p.resid_add = a.resid_add;
+  p.xres = a.xres; p.gain = a.gain; p.gain_vec = ((uintptr_t)a.gain & 7) == 0; p.hb = a.hb; p.ssq_out = a.ssq_out; p.taps = a.taps; p.tap_mask = a.taps ? a.tap_mask : 0; p.resid_add = a.resid_add;
   p.cs = a.cs; p.slot = a.slot; p.q = a.q; p.kp = (bf16 *)a.pool.k; p.vp = (bf16 *)a.pool.v; p.H = a.H; p.page_size = a.page_size;
   p.seq = a.seq; p.kvpos = a.kvpos; p.pm = a.pm; p.G = a.G;
   p.act = a.act; p.out_b = a.out_b; p.ldo = a.ldo; p.out_f32 = a.out_f32; p.status = a.status; p.stamp = a.stamp;

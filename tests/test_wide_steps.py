@@ -1,8 +1,11 @@
 """Steps whose passes have 129 to 256 rows (the row-major GEMM kernel, split over K slices or not), and batches whose pass
 over the pending entries goes on with one row per sequence, against the CPU oracle."""
+import numpy as np
 import pytest
+import torch
 
 import parity
+from paper_2503_01840_b200 import binding as sb
 from paper_2503_01840_b200 import synth
 
 pytestmark = pytest.mark.gpu
@@ -46,3 +49,37 @@ def test_unfused_draft_logits_of_wide_passes(batch, draft_vocab):
     prompts = [p.numpy() for p in synth.make_prompts(cfg)]
     st, _ = parity.run_trajectory(cfg, tw, dw, prompts, n_steps=2, tol=2e-2, tap_tol=3e-2)
     assert st.passes == 2 * 2 * batch and st.verify_compared == 2 * batch, st
+
+
+def _off_grid(weights):
+    """The same weights with every norm vector one element (two bytes) behind an 8-byte boundary."""
+    def move(t):
+        buf = torch.empty(t.numel() + 4, dtype=t.dtype, device=t.device)
+        buf[1 : 1 + t.numel()] = t
+        return buf[1 : 1 + t.numel()]
+
+    out = {n: move(t) if n.endswith("norm") else t for n, t in weights.items()}
+    if "layers" in out:
+        out["layers"] = [_off_grid(layer) for layer in out["layers"]]
+    return out
+
+
+@pytest.mark.parametrize("cfg,batch,prompt", [
+    (W4, 4, 150),                                                                       # 256-row steps and a prefill, split over K
+    (W4.replace(name="W4-wide", hidden=4096, n_heads=32, n_kv_heads=8, ffn=1024), 1, 1300),   # 96 tiles: the persistent kernel
+], ids=lambda v: getattr(v, "name", str(v)))
+def test_norm_weights_need_no_alignment(cfg, batch, prompt):
+    """Norm gains off an 8-byte boundary give the bits that aligned ones give."""
+    cfg = cfg.replace(batch=batch, tree_nodes=64)
+    tw, dw = synth.make_target_weights(cfg, device="cuda"), synth.make_draft_weights(cfg, device="cuda")
+    rng = np.random.default_rng(3)
+    prompts = [rng.integers(0, cfg.vocab, prompt).astype(np.int32) for _ in range(batch)]
+    seen = []
+    for t, d in ((tw, dw), (_off_grid(tw), _off_grid(dw))):
+        dec = sb.SpecDecoder(cfg, t, d, batch=batch, max_ctx=prompt + 200)
+        got = [dec.prefill(prompts, 16)]
+        got += [x for _ in range(2) for x in dec.step()]
+        got += [dec.debug(sb.DBG_NODE_HIDDEN, b) for b in range(batch)] + list(dec.read_kv(0, -1, prompt - 2))
+        seen.append(got)
+        dec.close()
+    assert all(np.array_equal(x, y) for x, y in zip(*seen)) and np.isfinite(seen[0][-1]).all()
