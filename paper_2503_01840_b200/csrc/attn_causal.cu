@@ -430,7 +430,7 @@ __global__ void __launch_bounds__(CA_THREADS, 1) attn_causal_kernel(const __grid
 #pragma unroll
       for (int s = 0; s < CA_MAX_DIAG; s++)
         if (s < p.J) M = fmaxf(M, d[s]);
-      fo = ex2((mx - M) * sc);
+      fo = mx == -INFINITY ? 0.0f : ex2((mx - M) * sc);          // every causal score -inf: the row has no causal part
       l *= fo;
 #pragma unroll
       for (int s = 0; s < CA_MAX_DIAG; s++) {

@@ -40,3 +40,20 @@ def test_causal_kernel_edges_vs_oracle(T, H, G, J, ps, shift):
     # outputs of order 1: bf16 output and bf16 probabilities, 2^-9 each; the statistics are fp32
     assert np.abs(out.float().cpu().numpy() - o_out).max() < 2e-2
     assert np.abs(lse.cpu().numpy() - o_lse).max() < 1e-4
+
+
+@pytest.mark.parametrize("T,H,G", [(130, 4, 1), (200, 2, 2)])
+def test_rows_whose_scores_are_all_minus_infinity(T, H, G):
+    """An infinite query component against keys that are all negative there: the row's output is 0 and its normaliser -inf;
+    the other rows are what they are without it."""
+    g = torch.Generator().manual_seed(T)
+    q, k, v = (torch.randn(*s, generator=g).to(torch.bfloat16).cuda() for s in ((T, H, 128), (-(-T // 16), G, 16, 128), (-(-T // 16), G, 16, 128)))
+    k[..., 5] = -1.0 - k[..., 5].abs()
+    table = torch.arange(k.shape[0], dtype=torch.int32, device="cuda")
+    out, lse = sb.ttt_attention(q, k, v, table, None, None, want_lse=True)
+    bad = torch.zeros(T, H, dtype=torch.bool, device="cuda")
+    for r, h in ((0, 0), (70, 1), (T - 1, H - 1)):
+        q[r, h, 5], bad[r, h] = float("inf"), True
+    out2, lse2 = sb.ttt_attention(q, k, v, table, None, None, want_lse=True)
+    assert (out2[bad] == 0).all() and (lse2[bad] == -float("inf")).all()
+    assert torch.equal(out2[~bad], out[~bad]) and torch.equal(lse2[~bad], lse[~bad]) and torch.isfinite(lse).all()
