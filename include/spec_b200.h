@@ -305,6 +305,10 @@ int spec_ttt_attention(const void *q, const void *k_pool, const void *v_pool, co
                        int32_t page_size, const void *k_diag, const void *v_diag, int32_t n_steps, void *out, float *lse,
                        int32_t T, int32_t n_heads, int32_t n_kv_heads, int32_t head_dim, void *scratch, void *stream);
 
+/* Test hook for the calling thread's causal attention launches (prefill and training-time test): 0 = off, 1 = the warps that
+ * wait for the last contraction of a tile come tens of microseconds late.  Results do not depend on it. */
+int spec_debug_causal(int32_t mode);
+
 /* Per-row log-softmax + top-K (value desc, index asc) over fp32 logits [rows][n]: the expansion
  * step of the dynamic tree (Section 2.2; Appendix A "nodes during the expansion phase").  K <= 16.
  * out_idx int32 [rows][K], out_lp float [rows][K].  scratch: device buffer of

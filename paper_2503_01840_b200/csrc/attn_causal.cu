@@ -37,6 +37,8 @@
 
 namespace spec {
 
+thread_local int tl_causal_test = CAUSAL_TEST_OFF;
+
 namespace {
 
 using tc::elect_one;
@@ -67,6 +69,7 @@ struct CausalParams {
   float *lse;
   int narrow;                      // out / kd / vd are only 8-byte aligned: the diagonal entries are read row by row instead
   int32_t *status;
+  int test;                        // test hook, see CausalTest
 };
 
 // eight elements of a row that starts on an 8-byte boundary
@@ -140,8 +143,8 @@ __global__ void __launch_bounds__(CA_THREADS, 1) attn_causal_kernel(const __grid
   unsigned char *sQ = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);   // two tiles [hd half][128 rows][128 B]
   unsigned char *sK = sQ + 2 * CA_TILE, *sV = sK + CA_STAGES * CA_TILE;
   uint64_t *kfull = (uint64_t *)(sV + CA_STAGES * CA_TILE), *kempty = kfull + CA_STAGES, *vfull = kempty + CA_STAGES, *vempty = vfull + CA_STAGES;
-  uint64_t *q_bar = vempty + CA_STAGES, *s_bar = q_bar + 1, *p_bar = s_bar + 4, *o_bar = p_bar + 4;     // s, p: [tile][buffer]; o: [tile]
-  uint32_t *tmem_slot = (uint32_t *)(o_bar + 2);
+  uint64_t *q_bar = vempty + CA_STAGES, *s_bar = q_bar + 1, *p_bar = s_bar + 4, *o_bar = p_bar + 4, *d_bar = o_bar + 2;     // s, p: [tile][buffer]; o, d: [tile]
+  uint32_t *tmem_slot = (uint32_t *)(d_bar + 2);
   volatile uint32_t *abort_flag = tmem_slot + 1;
   volatile int *n_filled = (volatile int *)(tmem_slot + 2);     // [0] K tiles, [1] V tiles requested
 
@@ -171,7 +174,7 @@ __global__ void __launch_bounds__(CA_THREADS, 1) attn_causal_kernel(const __grid
     for (int i = 0; i < CA_STAGES; i++) { mbar_init(&kfull[i], 1); mbar_init(&kempty[i], 2); mbar_init(&vfull[i], 1); mbar_init(&vempty[i], 2); }
     mbar_init(q_bar, 1);
     for (int i = 0; i < 4; i++) { mbar_init(&s_bar[i], 1); mbar_init(&p_bar[i], 128); }
-    for (int i = 0; i < 2; i++) mbar_init(&o_bar[i], 1);
+    for (int i = 0; i < 2; i++) { mbar_init(&o_bar[i], 1); mbar_init(&d_bar[i], 1); }
     *abort_flag = 0;
     n_filled[0] = n_filled[1] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -301,6 +304,7 @@ __global__ void __launch_bounds__(CA_THREADS, 1) attn_causal_kernel(const __grid
               for (int kk = 0; kk < 4; kk++)           // 16 keys: 8 columns of P, 16 rows of V
                 umma_ts(to, ts + (i & 1) * CA_KS + kk * 8, vd + (uint64_t)((kk * 16 * 128) >> 4), idesc_o, (i | kk) ? 1u : 0u);
               tc::umma_commit(&o_bar[t]);
+              if (i == nt - 1) tc::umma_commit(&d_bar[t]);
             }
             if (i + 2 < nt) issue_s(i + 2);
             // the tiles whose last use has been issued
@@ -381,9 +385,11 @@ __global__ void __launch_bounds__(CA_THREADS, 1) attn_causal_kernel(const __grid
       mbar_arrive(&p_bar[t * 2 + (i & 1)]);
     }
     if (alive && nt > 0) {
-      // the scores of the last step only tell that the P V two steps earlier is complete: one phase after the other
-      bool ok = nt < 2 || mbar_wait_warp(&o_bar[t], (uint32_t)((nt - 2) & 1));
-      ok = ok && mbar_wait_warp(&o_bar[t], (uint32_t)((nt - 1) & 1));
+      // All P V of the tile.  A barrier of its own: the scores of the last step only tell that the P V two steps earlier is
+      // complete, so o_bar can be up to two phases behind, and a warp that comes late finds it two phases further, where
+      // its parity says the same.
+      if (p.test == CAUSAL_TEST_LATE) __nanosleep(50000);
+      const bool ok = mbar_wait_warp(&d_bar[t], 0);
       if (!ok || *abort_flag) { if (lane == 0) { *abort_flag = 1; if (p.status) set_status(p.status, ST_TIMEOUT, 436, blockIdx.y, nt); } alive = false; }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     }
@@ -543,6 +549,7 @@ int launch_causal_attn(const CausalArgs &a, cudaStream_t s) {
   p.narrow = (((uintptr_t)a.out | (uintptr_t)a.kd | (uintptr_t)a.vd) & 15) ? 1 : 0;
   if (a.J > 0 && !p.narrow && (!diag_map(&mkd, a.kd, a.J, a.T, a.G, CA_T) || !diag_map(&mvd, a.vd, a.J, a.T, a.G, CA_T))) return -6;
   p.status = a.status;
+  p.test = tl_causal_test;
   const int br = causal_block_rows(grp);
   dim3 grid(grp % 2 == 0 ? a.H / 2 : a.H, a.blocks ? a.n_blocks : (a.T + br - 1) / br);
   static SmemLimit limit[2];
@@ -571,6 +578,12 @@ int launch_causal_attn(const CausalArgs &a, cudaStream_t s) {
 extern "C" size_t spec_ttt_attention_scratch_bytes(int32_t T, int32_t n_heads, int32_t n_kv_heads, int32_t head_dim) {
   if (T < 1 || n_heads < 1 || n_kv_heads < 1 || n_heads % n_kv_heads || head_dim != 128) return 0;
   return 256;
+}
+
+extern "C" int spec_debug_causal(int32_t mode) {
+  if (mode < spec::CAUSAL_TEST_OFF || mode > spec::CAUSAL_TEST_LATE) return SPEC_ERR_INVALID_CFG;
+  spec::tl_causal_test = mode;
+  return SPEC_OK;
 }
 
 extern "C" int spec_ttt_attention(const void *q, const void *k_pool, const void *v_pool, const int32_t *page_table,

@@ -34,6 +34,11 @@ struct CausalArgs {
   float *lse = nullptr;
   int32_t *status = nullptr;
 };
+// Test hook of the calling thread's launches.  LATE: the softmax warps pause for tens of microseconds before they wait for
+// the last contraction of their tile, which is complete long before they look.
+enum CausalTest { CAUSAL_TEST_OFF = 0, CAUSAL_TEST_LATE = 1 };
+extern thread_local int tl_causal_test;
+
 // Returns 0 or a negative code.
 int launch_causal_attn(const CausalArgs &a, cudaStream_t s);
 

@@ -57,3 +57,23 @@ def test_rows_whose_scores_are_all_minus_infinity(T, H, G):
     out2, lse2 = sb.ttt_attention(q, k, v, table, None, None, want_lse=True)
     assert (out2[bad] == 0).all() and (lse2[bad] == -float("inf")).all()
     assert torch.equal(out2[~bad], out[~bad]) and torch.equal(lse2[~bad], lse[~bad]) and torch.isfinite(lse).all()
+
+
+@pytest.mark.parametrize("T,H,G,J", [(40, 2, 1, 0), (128, 4, 1, 2), (300, 2, 2, 1), (513, 4, 4, 0)])
+def test_softmax_warps_that_come_late(T, H, G, J):
+    """Warps that look for a tile's last contraction long after it completed (one to nine key steps per tile) find it
+    complete, and the outputs are the same bits."""
+    g = torch.Generator().manual_seed(T)
+    pages = -(-T // 16)
+    q, k, v = (torch.randn(*s, generator=g).to(torch.bfloat16).cuda() for s in ((T, H, 128), (pages, G, 16, 128), (pages, G, 16, 128)))
+    kd, vd = (torch.randn(J, T, G, 128, generator=g).to(torch.bfloat16).cuda() for _ in range(2)) if J else (None, None)
+    table = torch.arange(pages, dtype=torch.int32, device="cuda")
+    run = lambda: sb.ttt_attention(q, k, v, table, kd, vd, want_lse=True)
+    out, lse = run()
+    sb.lib().spec_debug_causal(1)
+    try:
+        late, late_lse = run()
+        torch.cuda.synchronize()
+    finally:
+        sb.lib().spec_debug_causal(0)
+    assert torch.isfinite(lse).all() and torch.equal(out, late) and torch.equal(lse, late_lse)
