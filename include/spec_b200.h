@@ -296,7 +296,8 @@ int spec_attention_static(const void *q, const void *k_pool, const void *v_pool,
  * [num_pages][n_kv_heads][page_size][128] bf16 with page_table int32 [pages_per_seq] (position p lives in page
  * page_table[p / page_size]); page_size 16, 32 or 64.  k_diag / v_diag: bf16 [n_steps][T][n_kv_heads][128], the keys and
  * values each simulated step produced at every position (may be NULL when n_steps is 0: plain causal attention);
- * n_steps <= 8.  lse: optional float [T * n_heads], the natural-log normaliser of every row (what a backward pass needs).
+ * n_steps <= 8.  Nothing synchronises: rows that a device wait that ran out kept from being computed hold NaN (as does their
+ * lse).  lse: optional float [T * n_heads], the natural-log normaliser of every row (what a backward pass needs).
  * scratch: spec_ttt_attention_scratch_bytes(...) bytes of device memory (not written any more).  head_dim must be 128
  * (SPEC_ERR_UNSUPPORTED otherwise).  One launch of the causal tcgen05 kernel, which the prefill runs as well; the backward
  * pass is not part of this library. */
@@ -306,7 +307,9 @@ int spec_ttt_attention(const void *q, const void *k_pool, const void *v_pool, co
                        int32_t T, int32_t n_heads, int32_t n_kv_heads, int32_t head_dim, void *scratch, void *stream);
 
 /* Test hook for the calling thread's causal attention launches (prefill and training-time test): 0 = off, 1 = the warps that
- * wait for the last contraction of a tile come tens of microseconds late.  Results do not depend on it. */
+ * wait for the last contraction of a tile come tens of microseconds late (results do not depend on it), 2 = one CTA never
+ * receives its queries and its bounded waits run out: a prefill returns SPEC_ERR_DEVICE_STATUS, training-time test gives NaN
+ * in that CTA's rows. */
 int spec_debug_causal(int32_t mode);
 
 /* Per-row log-softmax + top-K (value desc, index asc) over fp32 logits [rows][n]: the expansion

@@ -25,7 +25,8 @@
 // memory delivers the operands of its MMAs and takes in the next tiles in 1250 (128 x 64 x 16 MMAs read 6 KB per 32 tensor
 // cycles), the exponentials take 1024.
 //
-// Every wait is bounded; a time-out is recorded in the status words and the CTA winds down.
+// Every wait is bounded.  On a time-out the CTA winds down; a prefill's status words record it, and training-time test, which
+// has none, gets NaN in the rows (and normalisers) it could not finish.
 #include <math.h>
 #include <string.h>
 
@@ -70,6 +71,7 @@ struct CausalParams {
   int narrow;                      // out / kd / vd are only 8-byte aligned: the diagonal entries are read row by row instead
   int32_t *status;
   int test;                        // test hook, see CausalTest
+  uint32_t spin;                   // polls before a wait gives up
 };
 
 // eight elements of a row that starts on an 8-byte boundary
@@ -195,8 +197,10 @@ __global__ void __launch_bounds__(CA_THREADS, 1) attn_causal_kernel(const __grid
       const int ps = p.pm.page_size, ppt = CA_T / ps;          // pages per key tile: 8, 4 or 2
       const int32_t *tbl = p.pm.table + (size_t)seq * p.pm.pages_per_seq;
       const int fallback = tbl[0];                             // keys past the last page are masked; they still need a valid source
+      const bool hold = p.test == CAUSAL_TEST_WITHHOLD && blockIdx.x == 0 && blockIdx.y == 0;
       if (elect_one()) {
         mbar_expect_tx(q_bar, 2 * CA_TILE);
+        if (!hold)
 #pragma unroll
         for (int t = 0; t < 2; t++)
 #pragma unroll
@@ -214,7 +218,7 @@ __global__ void __launch_bounds__(CA_THREADS, 1) attn_causal_kernel(const __grid
       auto fill = [&](int kv, int j, auto issue) {
         const int st = j % CA_STAGES;
         uint64_t *fb = kv ? &vfull[st] : &kfull[st], *eb = kv ? &vempty[st] : &kempty[st];
-        if (!mbar_wait_warp(eb, (uint32_t)((j / CA_STAGES) & 1) ^ 1u)) {
+        if (!mbar_wait_warp(eb, (uint32_t)((j / CA_STAGES) & 1) ^ 1u, p.spin)) {
           *abort_flag = 1;
           if (p.status) set_status(p.status, ST_TIMEOUT, 430 + kv, blockIdx.y, j);
         } else if (elect_one()) {
@@ -223,7 +227,7 @@ __global__ void __launch_bounds__(CA_THREADS, 1) attn_causal_kernel(const __grid
           n_filled[kv] = j + 1;
         }
         __syncwarp();
-        return !*abort_flag;
+        return !__any_sync(0xffffffffu, *abort_flag != 0);      // one answer for the warp, whoever gives up meanwhile
       };
       int cur = page_of(0);
       bool ok = true;
@@ -278,7 +282,7 @@ __global__ void __launch_bounds__(CA_THREADS, 1) attn_causal_kernel(const __grid
         }
         tc::umma_commit(&s_bar[t * 2 + (i & 1)]);
       };
-      bool ok = mbar_wait_warp(q_bar, 0) && mbar_wait_warp(&kfull[0], 0);
+      bool ok = mbar_wait_warp(q_bar, 0, p.spin) && mbar_wait_warp(&kfull[0], 0, p.spin);
       if (!ok) { *abort_flag = 1; if (p.status) set_status(p.status, ST_TIMEOUT, 432, blockIdx.y, t); }
       if (ok) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -291,10 +295,10 @@ __global__ void __launch_bounds__(CA_THREADS, 1) attn_causal_kernel(const __grid
         for (int i = 0; i < n; i++) {
           const int st = (i >> 1) % CA_STAGES, st2 = ((i + 2) >> 1) % CA_STAGES;
           if (!(i & 1)) {                              // a new V tile, and the K tile of the scores that follow it
-            ok = mbar_wait_warp(&vfull[st], (uint32_t)(((i >> 1) / CA_STAGES) & 1));
-            if (ok && i + 2 < n) ok = mbar_wait_warp(&kfull[st2], (uint32_t)((((i + 2) >> 1) / CA_STAGES) & 1));
+            ok = mbar_wait_warp(&vfull[st], (uint32_t)(((i >> 1) / CA_STAGES) & 1), p.spin);
+            if (ok && i + 2 < n) ok = mbar_wait_warp(&kfull[st2], (uint32_t)((((i + 2) >> 1) / CA_STAGES) & 1), p.spin);
           }
-          if (ok && i < nt) ok = mbar_wait_warp(&p_bar[t * 2 + (i & 1)], (uint32_t)((i >> 1) & 1));
+          if (ok && i < nt) ok = mbar_wait_warp(&p_bar[t * 2 + (i & 1)], (uint32_t)((i >> 1) & 1), p.spin);
           if (!ok) { *abort_flag = 1; if (p.status) set_status(p.status, ST_TIMEOUT, 433, blockIdx.y, i); break; }
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           if (elect_one()) {
@@ -328,8 +332,9 @@ __global__ void __launch_bounds__(CA_THREADS, 1) attn_causal_kernel(const __grid
     float mx = -INFINITY, l = 0.0f;
     bool alive = true;
     for (int i = 0; i < nt; i++) {
-      bool ok = mbar_wait_warp(&s_bar[t * 2 + (i & 1)], (uint32_t)((i >> 1) & 1));
-      if (!ok || *abort_flag) { if (lane == 0) { *abort_flag = 1; if (p.status) set_status(p.status, ST_TIMEOUT, 435, blockIdx.y, i); } alive = false; break; }
+      bool ok = mbar_wait_warp(&s_bar[t * 2 + (i & 1)], (uint32_t)((i >> 1) & 1), p.spin);
+      ok = __all_sync(0xffffffffu, ok && !*abort_flag);
+      if (!ok) { if (lane == 0) { *abort_flag = 1; if (p.status) set_status(p.status, ST_TIMEOUT, 435, blockIdx.y, i); } alive = false; break; }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t sb = my_s + (uint32_t)((i & 1) * CA_KS);
       float s[CA_KS];
@@ -356,7 +361,7 @@ __global__ void __launch_bounds__(CA_THREADS, 1) attn_causal_kernel(const __grid
         mx = tm;
       }
       if (i > 0 && __any_sync(0xffffffffu, f != 1.0f)) {         // the P V of the last step must be complete before O is rescaled
-        ok = mbar_wait_warp(&o_bar[t], (uint32_t)((i - 1) & 1));
+        ok = mbar_wait_warp(&o_bar[t], (uint32_t)((i - 1) & 1), p.spin);
         if (!ok) { if (lane == 0) { *abort_flag = 1; if (p.status) set_status(p.status, ST_TIMEOUT, 438, blockIdx.y, i); } alive = false; break; }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll 1
@@ -389,8 +394,8 @@ __global__ void __launch_bounds__(CA_THREADS, 1) attn_causal_kernel(const __grid
       // complete, so o_bar can be up to two phases behind, and a warp that comes late finds it two phases further, where
       // its parity says the same.
       if (p.test == CAUSAL_TEST_LATE) __nanosleep(50000);
-      const bool ok = mbar_wait_warp(&d_bar[t], 0);
-      if (!ok || *abort_flag) { if (lane == 0) { *abort_flag = 1; if (p.status) set_status(p.status, ST_TIMEOUT, 436, blockIdx.y, nt); } alive = false; }
+      const bool ok = __all_sync(0xffffffffu, mbar_wait_warp(&d_bar[t], 0, p.spin) && !*abort_flag);
+      if (!ok) { if (lane == 0) { *abort_flag = 1; if (p.status) set_status(p.status, ST_TIMEOUT, 436, blockIdx.y, nt); } alive = false; }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     }
     unsigned char *qt = sQ + t * CA_TILE;                        // this row's 16-byte chunk c: half c / 8, row lr, chunk (c % 8) ^ (lr % 8)
@@ -413,7 +418,7 @@ __global__ void __launch_bounds__(CA_THREADS, 1) attn_causal_kernel(const __grid
         for (int s = 0; s < CA_MAX_DIAG; s++)
           if (s < p.J) {
             const int j = nkt + s * nb + (two_heads ? 0 : t), st = j % CA_STAGES;
-            const bool ok = mbar_wait_warp(&kfull[st], (uint32_t)((j / CA_STAGES) & 1));
+            const bool ok = mbar_wait_warp(&kfull[st], (uint32_t)((j / CA_STAGES) & 1), p.spin);
             if (!ok) { if (lane == 0) { *abort_flag = 1; if (p.status) set_status(p.status, ST_TIMEOUT, 439, blockIdx.y, s); } alive = false; }
             if (alive) {
 #pragma unroll 4
@@ -469,7 +474,7 @@ __global__ void __launch_bounds__(CA_THREADS, 1) attn_causal_kernel(const __grid
 #pragma unroll 1
       for (int s = 0; s < p.J; s++) {
         const int j = nkt + s * nb + (two_heads ? 0 : t), st = j % CA_STAGES;
-        const bool ok = mbar_wait_warp(&vfull[st], (uint32_t)((j / CA_STAGES) & 1));
+        const bool ok = mbar_wait_warp(&vfull[st], (uint32_t)((j / CA_STAGES) & 1), p.spin);
         if (!ok) { if (lane == 0) { *abort_flag = 1; if (p.status) set_status(p.status, ST_TIMEOUT, 440, blockIdx.y, s); } alive = false; }
         if (alive && nt > 0) {
           float w = 0.0f;
@@ -506,7 +511,9 @@ __global__ void __launch_bounds__(CA_THREADS, 1) attn_causal_kernel(const __grid
       }
     }
     __syncwarp();
-    if (alive && nt > 0) {
+    // A warp that gave up: where there are no status words to say so, its rows are NaN, never what the buffer held before.
+    if (nt > 0 && (alive || !p.status)) {
+      if (DIAG && !alive && p.lse && rv) p.lse[(size_t)(trow + lr) * p.H + head] = __int_as_float(0x7fffffff);
       // a warp's 32 rows, two whole rows (256 bytes each) per instruction
       const int rw = (warp & 3) * 32;
 #pragma unroll 4
@@ -514,7 +521,7 @@ __global__ void __launch_bounds__(CA_THREADS, 1) attn_causal_kernel(const __grid
         const int r = rw + 2 * i + (lane >> 4), c = lane & 15;
         if (r < nr) {
           bf16 *dst = p.out + ((size_t)(trow + r) * p.H + head) * CA_HD + c * 8;
-          const uint4 v = *chunk(qt, r, c);
+          const uint4 v = alive ? *chunk(qt, r, c) : make_uint4(~0u, ~0u, ~0u, ~0u);
           if (DIAG && p.narrow) { *(uint2 *)dst = make_uint2(v.x, v.y); *(uint2 *)(dst + 4) = make_uint2(v.z, v.w); }
           else *(uint4 *)dst = v;
         }
@@ -524,9 +531,9 @@ __global__ void __launch_bounds__(CA_THREADS, 1) attn_causal_kernel(const __grid
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (*abort_flag && threadIdx.x == 0) {            // no copy may still be landing when the CTA exits
-    mbar_wait(q_bar, 0);
+    mbar_wait(q_bar, 0, p.spin);
     for (int kv = 0; kv < 2; kv++)
-      for (int j = max(0, n_filled[kv] - CA_STAGES); j < n_filled[kv]; j++) mbar_wait(kv ? &vfull[j % CA_STAGES] : &kfull[j % CA_STAGES], (uint32_t)((j / CA_STAGES) & 1));
+      for (int j = max(0, n_filled[kv] - CA_STAGES); j < n_filled[kv]; j++) mbar_wait(kv ? &vfull[j % CA_STAGES] : &kfull[j % CA_STAGES], (uint32_t)((j / CA_STAGES) & 1), p.spin);
   }
   if (warp == 9) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512) : "memory");
 }
@@ -550,6 +557,7 @@ int launch_causal_attn(const CausalArgs &a, cudaStream_t s) {
   if (a.J > 0 && !p.narrow && (!diag_map(&mkd, a.kd, a.J, a.T, a.G, CA_T) || !diag_map(&mvd, a.vd, a.J, a.T, a.G, CA_T))) return -6;
   p.status = a.status;
   p.test = tl_causal_test;
+  p.spin = p.test == CAUSAL_TEST_WITHHOLD ? 2000u : tc::SPIN_LIMIT;
   const int br = causal_block_rows(grp);
   dim3 grid(grp % 2 == 0 ? a.H / 2 : a.H, a.blocks ? a.n_blocks : (a.T + br - 1) / br);
   static SmemLimit limit[2];
@@ -581,7 +589,7 @@ extern "C" size_t spec_ttt_attention_scratch_bytes(int32_t T, int32_t n_heads, i
 }
 
 extern "C" int spec_debug_causal(int32_t mode) {
-  if (mode < spec::CAUSAL_TEST_OFF || mode > spec::CAUSAL_TEST_LATE) return SPEC_ERR_INVALID_CFG;
+  if (mode < spec::CAUSAL_TEST_OFF || mode > spec::CAUSAL_TEST_WITHHOLD) return SPEC_ERR_INVALID_CFG;
   spec::tl_causal_test = mode;
   return SPEC_OK;
 }

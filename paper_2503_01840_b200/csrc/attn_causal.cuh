@@ -35,8 +35,9 @@ struct CausalArgs {
   int32_t *status = nullptr;
 };
 // Test hook of the calling thread's launches.  LATE: the softmax warps pause for tens of microseconds before they wait for
-// the last contraction of their tile, which is complete long before they look.
-enum CausalTest { CAUSAL_TEST_OFF = 0, CAUSAL_TEST_LATE = 1 };
+// the last contraction of their tile, which is complete long before they look.  WITHHOLD: the first CTA never receives its
+// queries and gives up after 2000 polls.
+enum CausalTest { CAUSAL_TEST_OFF = 0, CAUSAL_TEST_LATE = 1, CAUSAL_TEST_WITHHOLD = 2 };
 extern thread_local int tl_causal_test;
 
 // Returns 0 or a negative code.

@@ -3,8 +3,10 @@ import numpy as np
 import pytest
 import torch
 
+import parity
 import pyoracle as po
 from paper_2503_01840_b200 import binding as sb
+from paper_2503_01840_b200 import synth
 
 pytestmark = pytest.mark.gpu
 
@@ -77,3 +79,49 @@ def test_softmax_warps_that_come_late(T, H, G, J):
     finally:
         sb.lib().spec_debug_causal(0)
     assert torch.isfinite(lse).all() and torch.equal(out, late) and torch.equal(lse, late_lse)
+
+
+@pytest.mark.parametrize("T,H,G,J", [(130, 4, 1, 0), (300, 8, 2, 3), (513, 4, 4, 2)])
+def test_training_time_test_wait_that_runs_out_gives_nan(T, H, G, J):
+    """The first CTA never receives its queries (test hook): its rows, those of the last positions of its heads, are NaN, all
+    others are untouched, and the next call is whole."""
+    g = torch.Generator().manual_seed(T)
+    pages = -(-T // 16)
+    q, k, v = (torch.randn(*s, generator=g).to(torch.bfloat16).cuda() for s in ((T, H, 128), (pages, G, 16, 128), (pages, G, 16, 128)))
+    kd, vd = (torch.randn(J, T, G, 128, generator=g).to(torch.bfloat16).cuda() for _ in range(2)) if J else (None, None)
+    table = torch.arange(pages, dtype=torch.int32, device="cuda")
+    run = lambda: sb.ttt_attention(q, k, v, table, kd, vd, want_lse=True)
+    out, lse = run()
+    sb.lib().spec_debug_causal(2)
+    try:
+        lost, lost_lse = run()
+        torch.cuda.synchronize()
+    finally:
+        sb.lib().spec_debug_causal(0)
+    block, heads = (128, 2) if (H // G) % 2 == 0 else (256, 1)
+    gone = torch.zeros(T, H, dtype=torch.bool, device="cuda")
+    gone[(T - 1) // block * block :, :heads] = True
+    assert torch.isnan(lost[gone]).all() and torch.isnan(lost_lse[gone]).all()
+    assert torch.equal(lost[~gone], out[~gone]) and torch.equal(lost_lse[~gone], lse[~gone])
+    again, again_lse = run()
+    assert torch.equal(again, out) and torch.equal(again_lse, lse)
+
+
+def test_prefill_wait_that_runs_out_is_reported():
+    """The same in a prefill: it returns SPEC_ERR_DEVICE_STATUS with the site of the wait, and the next one is whole."""
+    cfg = synth.ModelCfg("wait", "bf16", 2, 512, 8, 2, 128, 1408, 2048, 1024, (0, 0, 1), 5e5, batch=2, tree_depth=2, tree_topk=4, tree_nodes=12, seed=9)
+    tw, dw = parity.to_dev(synth.make_target_weights(cfg)), parity.to_dev(synth.make_draft_weights(cfg))
+    rng = np.random.default_rng(1)
+    prompts = [rng.integers(0, cfg.vocab, n).astype(np.int32) for n in (300, 77)]
+    dec = sb.SpecDecoder(cfg, tw, dw, batch=2, max_ctx=400)
+    first = dec.prefill(prompts, 8)
+    steps = dec.step()
+    sb.lib().spec_debug_causal(2)
+    try:
+        with pytest.raises(sb.SpecError) as e:
+            dec.prefill(prompts, 8)
+    finally:
+        sb.lib().spec_debug_causal(0)
+    assert e.value.code == -7 and "site 43" in str(e.value), str(e.value)
+    assert np.array_equal(dec.prefill(prompts, 8), first) and all(np.array_equal(a, b) for a, b in zip(dec.step(), steps))
+    dec.close()
