@@ -249,17 +249,16 @@ __global__ void __launch_bounds__(CA_THREADS, 1) attn_causal_kernel(const __grid
         cur = nxt;
       }
       if (DIAG && diag_ring) {
-        // the diagonal steps' entries: the first of both rings, then all keys (their dot products come first), then the values
-        auto entry = [&](int kv, int e) {
-          return fill(kv, nkt + e, [&](unsigned char *d, uint64_t *fb) {
+        // The diagonal steps' entries: all keys (their dot products come first), then all values, by turns through the two
+        // rings, so that all four stages are in flight in either phase (see diag_entry)
+        const int total = p.J * nb;
+        for (int e = 0; e < 2 * total && ok; e++) {
+          const int x = e < total ? e : e - total;
+          ok = fill(e & 1, nkt + (e >> 1), [&](unsigned char *d, uint64_t *fb) {
 #pragma unroll
-            for (int h = 0; h < 2; h++) load_4d(d + h * CA_HALF, kv ? &map_vd : &map_kd, 64 * h, g, row0 + (e % nb) * CA_T, e / nb, fb);
+            for (int h = 0; h < 2; h++) load_4d(d + h * CA_HALF, e < total ? &map_kd : &map_vd, 64 * h, g, row0 + (x % nb) * CA_T, x / nb, fb);
           });
-        };
-        const int total = p.J * nb, pre = min(total, CA_STAGES);
-        for (int e = 0; e < pre; e++) ok = ok && entry(0, e) && entry(1, e);
-        for (int e = pre; e < total; e++) ok = ok && entry(0, e);
-        for (int e = pre; e < total; e++) ok = ok && entry(1, e);
+        }
       }
     } else if (warp <= 10) {
       // ================================================================ MMA warps: one per query tile
@@ -404,6 +403,27 @@ __global__ void __launch_bounds__(CA_THREADS, 1) attn_causal_kernel(const __grid
     float fo = 1.0f, wd[CA_MAX_DIAG];
     size_t doff = 0;
     const size_t dstep = (size_t)p.T * p.G * CA_HD;
+    // Diagonal entry e of this CTA sits in ring e % 2, place nkt + e / 2.  The two query tiles share an entry where they are
+    // two heads, and take alternate ones (one ring each) where they are two blocks of positions.  Both tiles have to be
+    // through with their keys first: a wait for place j of a ring means something only when the use of its stage before that
+    // (place j - 2, maybe keys of the other tile alone) has landed.
+    // With keys in one ring, values in the other and both tiles in step after every entry, an entry took the latency of a load
+    // (1.5 us).  With few heads that is on the critical path: 4 heads, 7 steps, T = 2048 63 us then, 57 now; T = 512 39, 33.
+    if (DIAG && diag_ring) asm volatile("bar.sync 3, 256;" ::: "memory");
+    auto diag_wait = [&](int e) -> unsigned char * {
+      const int st = (nkt + (e >> 1)) % CA_STAGES;
+      const bool ok = mbar_wait_warp((e & 1) ? &vfull[st] : &kfull[st], (uint32_t)(((nkt + (e >> 1)) / CA_STAGES) & 1), p.spin);
+      if (!ok) { if (lane == 0) { *abort_flag = 1; if (p.status) set_status(p.status, ST_TIMEOUT, 439, blockIdx.y, e); } alive = false; }
+      return ((e & 1) ? sV : sK) + st * CA_TILE;
+    };
+    auto diag_done = [&](int e) {                                // the tile's threads are done with it: its place may be filled again
+      asm volatile("bar.sync %0, 128;" ::"r"(1 + t) : "memory");
+      if (lr == 0) {                                             // two arrivals per place, as from the MMA warps
+        uint64_t *eb = (e & 1) ? &vempty[(nkt + (e >> 1)) % CA_STAGES] : &kempty[(nkt + (e >> 1)) % CA_STAGES];
+        mbar_arrive(eb);
+        if (!two_heads) mbar_arrive(eb);
+      }
+    };
     if (DIAG) {
       doff = ((size_t)(rv ? trow + lr : 0) * p.G + g) * CA_HD;
       float d[CA_MAX_DIAG];
@@ -417,16 +437,13 @@ __global__ void __launch_bounds__(CA_THREADS, 1) attn_causal_kernel(const __grid
 #pragma unroll
         for (int s = 0; s < CA_MAX_DIAG; s++)
           if (s < p.J) {
-            const int j = nkt + s * nb + (two_heads ? 0 : t), st = j % CA_STAGES;
-            const bool ok = mbar_wait_warp(&kfull[st], (uint32_t)((j / CA_STAGES) & 1), p.spin);
-            if (!ok) { if (lane == 0) { *abort_flag = 1; if (p.status) set_status(p.status, ST_TIMEOUT, 439, blockIdx.y, s); } alive = false; }
+            const int e = two_heads ? s : 2 * s + t;
+            unsigned char *kt = diag_wait(e);
             if (alive) {
 #pragma unroll 4
-              for (int c = 0; c < 16; c++) d[s] += dot8(*chunk(qt, lr, c), *chunk(sK + st * CA_TILE, lr, c));
+              for (int c = 0; c < 16; c++) d[s] += dot8(*chunk(qt, lr, c), *chunk(kt, lr, c));
             }
-            asm volatile("bar.sync 1, 256;" ::: "memory");       // both tiles' threads are done with the step's ring tiles
-            if ((threadIdx.x & 127) == 0)                        // one arrival per query tile, as from the MMA warps
-              for (int tb = 0; tb < nb; tb++) mbar_arrive(&kempty[(nkt + s * nb + tb) % CA_STAGES]);
+            diag_done(e);
           }
       } else if (p.J > 0 && alive && nt > 0) {
 #pragma unroll 2
@@ -473,19 +490,16 @@ __global__ void __launch_bounds__(CA_THREADS, 1) attn_causal_kernel(const __grid
       }
 #pragma unroll 1
       for (int s = 0; s < p.J; s++) {
-        const int j = nkt + s * nb + (two_heads ? 0 : t), st = j % CA_STAGES;
-        const bool ok = mbar_wait_warp(&vfull[st], (uint32_t)((j / CA_STAGES) & 1), p.spin);
-        if (!ok) { if (lane == 0) { *abort_flag = 1; if (p.status) set_status(p.status, ST_TIMEOUT, 440, blockIdx.y, s); } alive = false; }
+        const int e = p.J * nb + (two_heads ? s : 2 * s + t);
+        unsigned char *vt = diag_wait(e);
         if (alive && nt > 0) {
           float w = 0.0f;
 #pragma unroll
           for (int z = 0; z < CA_MAX_DIAG; z++) w = z == s ? wd[z] : w;
 #pragma unroll
-          for (int c = 0; c < 16; c++) add8(o + c * 8, w, *chunk(sV + st * CA_TILE, lr, c));
+          for (int c = 0; c < 16; c++) add8(o + c * 8, w, *chunk(vt, lr, c));
         }
-        asm volatile("bar.sync 1, 256;" ::: "memory");
-        if ((threadIdx.x & 127) == 0)
-          for (int tb = 0; tb < nb; tb++) mbar_arrive(&vempty[(nkt + s * nb + tb) % CA_STAGES]);
+        diag_done(e);
       }
       if (alive && nt > 0) {
 #pragma unroll

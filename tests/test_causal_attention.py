@@ -11,7 +11,8 @@ from paper_2503_01840_b200 import synth
 pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("T,H,G,J,ps,shift", [(1, 8, 2, 2, 16, 0), (127, 2, 2, 1, 32, 0), (256, 6, 2, 0, 64, 0), (257, 4, 4, 3, 16, 0),
-                                              (385, 3, 1, 2, 16, 0), (384, 8, 2, 3, 64, 0), (200, 4, 2, 3, 16, 4), (130, 3, 3, 8, 32, 4)])
+                                              (385, 3, 1, 2, 16, 0), (384, 8, 2, 3, 64, 0), (200, 4, 2, 3, 16, 4), (130, 3, 3, 8, 32, 4),
+                                              (100, 4, 4, 7, 16, 0), (320, 2, 2, 8, 32, 0), (700, 1, 1, 5, 64, 0), (200, 4, 1, 5, 16, 0), (129, 4, 2, 1, 16, 0)])
 def test_causal_kernel_edges_vs_oracle(T, H, G, J, ps, shift):
     """One position, whole and ragged tiles, both ways of pairing query tiles, the three page sizes, and diagonal entries
     that start on an 8-byte boundary only (shift elements into their allocation)."""
