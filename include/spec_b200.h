@@ -202,7 +202,10 @@ enum spec_debug_what {
   /* SPEC_FLAG_STAMPS: per stamped launch of the last step, in launch order, uint64 [n][2] = {earliest time a CTA of the
    * launch had its inputs ready (after its programmatic-dependent-launch wait), latest time a CTA left}, nanoseconds
    * of the GPU's global timer; and the launch's profile class, int32 [n] */
-  SPEC_DBG_STAMPS = 120, SPEC_DBG_STAMP_CLASS
+  SPEC_DBG_STAMPS = 120, SPEC_DBG_STAMP_CLASS,
+  /* rows of the passes the last prefill ran, in order, int32 [passes] (the prompts' positions lie one behind the other in them);
+   * empty where the prompts ran one by one */
+  SPEC_DBG_PREFILL_PASSES
 };
 /* Copies up to `bytes` of item `what` of sequence `seq` (last step) to host_dst; returns bytes
  * available (>= 0) or a negative status. */

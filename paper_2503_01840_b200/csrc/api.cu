@@ -107,6 +107,7 @@ struct spec_ctx {
   size_t attn_scratch_bytes;
   char *wide_base;             // the step's own buffers, free during a prefill (see WideBufs)
   size_t wide_bytes;
+  std::vector<int32_t> pass_rows;   // of the last packed prefill (SPEC_DBG_PREFILL_PASSES)
   // partial-sum bookkeeping of the plain (fp32 / debug) schedule: its GEMMs write one slice
   int np_proj = 1, np_qkv = 1, np_gu = 1;
   size_t ps_proj = 0, ps_qkv = 0, ps_gu = 0;
@@ -959,6 +960,7 @@ constexpr int WIDE_MAX_TILES = 16;       // row tiles (256 rows) of a pass: the 
 constexpr int WIDE_LAYER_COST = 64;      // what a layer's launches cost beside their waves, in k-blocks (0.27 us each)
 static int prefill_packed(spec_ctx *c, const int32_t *lens, size_t total, int32_t *root_host, bool &done) {
   done = false;
+  c->pass_rows.clear();
   const spec_cfg &g = c->cfg;
   if (!c->fused || !causal_attn_supported(c->hd, g.page_size) || (g.flags & (SPEC_FLAG_REF_ATTN | SPEC_FLAG_NO_TMA_ATTN))) return SPEC_OK;
   if (total > (size_t)1 << 30) return SPEC_OK;
@@ -1013,6 +1015,7 @@ static int prefill_packed(spec_ctx *c, const int32_t *lens, size_t total, int32_
     // the attention CTAs are issued longest key range first
     std::stable_sort(blocks.begin() + ps.blk0, blocks.end(), [](const CausalBlock &x, const CausalBlock &y) { return x.pos0 + x.nrows > y.pos0 + y.nrows; });
     passes.push_back(ps);
+    c->pass_rows.push_back(ps.rows);
   }
   if (blocks.size() > max_blocks || passes[0].rows > cap * WIDE_ROWS) return fail(c, SPEC_ERR_STATE, "spec_prefill: pass plan out of bounds");
   cudaStream_t s = c->stream;
@@ -1370,6 +1373,11 @@ extern "C" int64_t spec_debug_read(spec_ctx *c, int32_t what, int32_t seq, void 
     case SPEC_DBG_STAMP_CLASS: {
       size_t avail = c->stamp_cls.size() * sizeof(int32_t);
       if (dst && bytes) memcpy(dst, c->stamp_cls.data(), std::min(avail, bytes));
+      return (int64_t)avail;
+    }
+    case SPEC_DBG_PREFILL_PASSES: {
+      size_t avail = c->pass_rows.size() * sizeof(int32_t);
+      if (dst && bytes) memcpy(dst, c->pass_rows.data(), std::min(avail, bytes));
       return (int64_t)avail;
     }
     case SPEC_DBG_RAW_LOGITS: return copy_out(c, c->logits, (size_t)c->Ralloc * c->Vd, dst, bytes);

@@ -35,11 +35,14 @@ def test_packed_prefill_vs_oracle(cfg, lens):
     assert st.passes == cfg.tree_depth * len(lens) and st.verify_compared == len(lens), st
     dec = sb.SpecDecoder(cfg, parity.to_dev(tw), parity.to_dev(dw), batch=len(lens), max_ctx=max(lens) + 64, page_shuffle_seed=6)
     dec.prefill(prompts, 8)
+    passes = dec.debug(sb.DBG_PREFILL_PASSES)
+    assert passes.sum() == sum(lens) and (len(passes) > 1) == (sum(lens) > 4000), passes
+    cuts = np.cumsum(passes)[:-1].tolist()
     for b, n in enumerate(lens):
         orc = po.Oracle(cfg, tw, dw, n + 64)
         orc.prefill(prompts[b])
         edges = {0, 1, 63, 64, 127, 128, 129, 255, 256, 257, n // 2, n - 3, n - 2, n - 1}
-        edges |= {e - sum(lens[:b]) + d for e in (4096,) for d in (-1, 0, 1)}          # around a pass boundary
+        edges |= {e - sum(lens[:b]) + d for e in cuts for d in (-1, 0, 1)}             # around every pass boundary
         for pos in sorted(e for e in edges if 0 <= e < n):
             for layer in range(cfg.n_layers):
                 gk, gv = dec.read_kv(b, layer, pos)
