@@ -217,17 +217,24 @@ int spec_debug_read_kv(spec_ctx *ctx, int32_t seq, int32_t layer, int32_t pos, f
  * Each launches on `stream` and does not synchronise.  dtype as spec_dtype. */
 
 /* out[r][o] = sum_i x[r][i] * w[o][i]; x [rows][in] dtype, w [out][in] dtype, out fp32 [rows][ldo]
- * (first `out` columns).  impl 0: the step's tcgen05/TMEM kernel with the library's own plan (bf16 only; the shape
- * limits of spec_gemm_fused), 1: plain CUDA-core kernel. */
+ * (first `out` columns).  impl 0: spec_gemm_fused with the library's own plan (bf16 only, its shape limits), 1: plain CUDA-core kernel. */
 int spec_gemm(int32_t dtype, int32_t impl, const void *x, const void *w, float *out_f32, int32_t rows, int32_t out,
               int32_t in, int32_t ldo, void *stream);
 
-/* The same contraction on the kernel the step uses (Section 3.1's FC, projection and LM-head layers are
- * all of this form): bf16, tcgen05/TMEM, split-K reduced across a thread-block cluster through
+/* The same contraction on the kernel that passes of up to 128 rows use (Section 3.1's FC, projection and LM-head layers are
+ * all of this form; see spec_gemm_wide for more rows): bf16, tcgen05/TMEM, split-K reduced across a thread-block cluster through
  * distributed shared memory, no scratch.  rows <= 256, in % 8 == 0, 16-byte aligned x and w.
  * split: K slices (= cluster size, 1..8), stages: TMA pipeline depth; 0 lets the library choose. */
 int spec_gemm_fused(const void *x, const void *w, float *out_f32, int32_t rows, int32_t out, int32_t in, int32_t ldo,
                     int32_t split, int32_t stages, void *stream);
+
+/* The row-major kernels of passes of more than 128 rows (prefill, steps of 129 to 256 rows; gate/up from 193 rows on), without
+ * the passes' epilogues: out fp32 [rows][ldo] = x . w^T, or with w_up the gate/up form, out bf16 [rows][out] (ldo == out) as in
+ * spec_gemm_swiglu.  Any number of rows; in % 8 == 0, out % 8 == 0, ldo % 4 == 0, 16-byte aligned pointers.  form: 0 lets the library
+ * choose; else K slices (1..4, at most one per 64 of `in`), or for gate/up the features per tile (a multiple of 16 in 64..256, 1 = the
+ * persistent kernel with 128).  used (host, may be NULL) receives the form that ran. */
+int spec_gemm_wide(const void *x, const void *w, const void *w_up, void *out, int32_t rows, int32_t out_features, int32_t in, int32_t ldo,
+                   int32_t form, int32_t *used, void *stream);
 
 /* The draft LM head followed by log-softmax and top-K (Section 2.2: the draft tree is expanded by the draft model's
  * confidence; Appendix A: nodes per expansion), on the kernels the step uses, without ever writing the logits: the
@@ -241,7 +248,7 @@ int spec_gemm_topk(const void *x, const void *w, int32_t rows, int32_t out, int3
                    float *out_lp, void *scratch, void *stream);
 
 /* Gate/up half of the decoder layer's MLP (the draft layer and every target layer are LLaMA-style decoder layers,
- * Section 3.1), on the kernel the step uses: act[r][f] = bf16(silu(g) * u), g = sum_i x[r][i] * w_gate[f][i], u likewise
+ * Section 3.1), on the kernel that passes of up to 192 rows use: act[r][f] = bf16(silu(g) * u), g = sum_i x[r][i] * w_gate[f][i], u likewise
  * with w_up, both accumulated in fp32 (a cluster holds the gate and the up tile of the same 128 features and their K
  * slices).  x [rows][in] bf16, w_gate / w_up [F][in] bf16, act [rows][F] bf16, all device pointers, 16-byte aligned;
  * rows <= 256, in % 8 == 0.  Returns SPEC_OK or a negative code; nothing is allocated. */

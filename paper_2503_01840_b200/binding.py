@@ -58,7 +58,7 @@ class _Cfg(C.Structure):
 
 EXPORTS = ("spec_workspace_bytes", "spec_init", "spec_prefill", "spec_step", "spec_step_async", "spec_step_sampled", "spec_plain_step",
            "spec_lengths", "spec_profile_step", "spec_tune", "spec_launches_per_step", "spec_step_bytes", "spec_free", "spec_last_error",
-           "spec_debug_read", "spec_debug_read_kv", "spec_gemm", "spec_gemm_fused", "spec_gemm_swiglu", "spec_gemm_topk_scratch_bytes", "spec_gemm_topk", "spec_ttt_attention_scratch_bytes", "spec_ttt_attention",
+           "spec_debug_read", "spec_debug_read_kv", "spec_gemm", "spec_gemm_fused", "spec_gemm_swiglu", "spec_gemm_wide", "spec_gemm_topk_scratch_bytes", "spec_gemm_topk", "spec_ttt_attention_scratch_bytes", "spec_ttt_attention",
            "spec_debug_causal", "spec_topk_scratch_bytes", "spec_attn_scratch_bytes",
            "spec_attention", "spec_attention_static", "spec_attention_static_capacity", "spec_logsoftmax_topk", "spec_argmax")
 
@@ -111,6 +111,7 @@ def lib():
     L.spec_ttt_attention_scratch_bytes.restype = sz
     L.spec_ttt_attention.argtypes = [vp, vp, vp, vp, i32, i32, vp, vp, i32, vp, vp, i32, i32, i32, i32, vp, vp]
     L.spec_debug_causal.argtypes = [i32]
+    L.spec_gemm_wide.argtypes = [vp, vp, vp, vp, i32, i32, i32, i32, i32, C.POINTER(i32), vp]
     L.spec_topk_scratch_bytes.argtypes = [i32, i32, i32]
     L.spec_topk_scratch_bytes.restype = sz
     L.spec_logsoftmax_topk.argtypes = [vp, i32, i32, i32, vp, vp, vp, vp]
@@ -427,6 +428,21 @@ def gemm_swiglu(x: torch.Tensor, w_gate: torch.Tensor, w_up: torch.Tensor) -> to
     if rc:
         raise SpecError(rc, "spec_gemm_swiglu")
     return act
+
+
+def gemm_wide(x: torch.Tensor, w: torch.Tensor, w_up: Optional[torch.Tensor] = None, form: int = 0):
+    """(out, form that ran): x . w^T in fp32, or bf16(silu(x . w^T) * (x . w_up^T)), on the row-major kernels of wide passes."""
+    rows, I = x.shape
+    O = w.shape[0]
+    ws = [w] if w_up is None else [w, w_up]
+    assert all(t.is_contiguous() and t.dtype == torch.bfloat16 and t.shape[1] == I for t in [x, *ws]) and ws[-1].shape[0] == O
+    out = torch.empty(rows, O, dtype=torch.float32 if w_up is None else torch.bfloat16, device=x.device)
+    used = C.c_int32(0)
+    rc = lib().spec_gemm_wide(x.data_ptr(), w.data_ptr(), None if w_up is None else w_up.data_ptr(), out.data_ptr(), rows, O, I, O, form,
+                              C.byref(used), _stream_ptr(None))
+    if rc:
+        raise SpecError(rc, "spec_gemm_wide")
+    return out, used.value
 
 
 def logsoftmax_topk(logits: torch.Tensor, K: int, two_stage: bool = True):

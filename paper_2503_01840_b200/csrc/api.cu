@@ -1459,6 +1459,29 @@ extern "C" int spec_gemm_swiglu(const void *x, const void *w_gate, const void *w
   return cudaGetLastError() == cudaSuccess ? SPEC_OK : SPEC_ERR_CUDA;
 }
 
+extern "C" int spec_gemm_wide(const void *x, const void *w, const void *w_up, void *out, int32_t rows, int32_t O, int32_t I, int32_t ldo,
+                              int32_t form, int32_t *used, void *stream) {
+  if (!x || !w || !out) return SPEC_ERR_NULL;
+  if (rows < 1 || O < 1 || I < 1 || ldo < O || form < 0) return SPEC_ERR_INVALID_CFG;
+  static TmaMaps *g = nullptr;
+  if (!g) {
+    std::string why;
+    g = tma_maps_create(why);
+    if (!g) return SPEC_ERR_CUDA;
+  }
+  WideGemmArgs a;
+  a.x = (const bf16 *)x; a.rows = a.x_rows = rows; a.I = I; a.w[0] = (const bf16 *)w; a.O[0] = O;
+  if (w_up) { a.w[1] = (const bf16 *)w_up; a.O[1] = O; a.nw = 2; a.act = (bf16 *)out; }
+  else { a.out_f32 = (float *)out; a.ldo = ldo; }
+  a.form = form; a.used = used;
+  const WideEpi epi = w_up ? WIDE_SWIGLU : WIDE_F32;
+  if (!wide_gemm_supported(epi, a) || (w_up && (ldo != O || ((uintptr_t)out & 15)))) return SPEC_ERR_UNSUPPORTED;
+  int rc = wide_gemm_launch(g, epi, a, (cudaStream_t)stream);
+  tma_maps_forget(g);
+  if (rc) return rc == -1 ? SPEC_ERR_INVALID_CFG : SPEC_ERR_CUDA;
+  return cudaGetLastError() == cudaSuccess ? SPEC_OK : SPEC_ERR_CUDA;
+}
+
 extern "C" size_t spec_gemm_topk_scratch_bytes(int32_t rows, int32_t out, int32_t K) {
   if (rows < 1 || out < 1 || K < 1) return 0;
   const size_t tiles = ((size_t)out + 127) / 128;

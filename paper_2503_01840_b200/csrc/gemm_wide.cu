@@ -1059,6 +1059,11 @@ bool wide_gemm_supported(WideEpi epi, const WideGemmArgs &a) {
   if (a.nw < 1 || a.nw > 3 || (epi == WIDE_SWIGLU && (a.nw != 2 || a.O[0] != a.O[1])) || (epi == WIDE_QKV && a.nw < 2)) return false;
   for (int j = 0; j < a.nw; j++)
     if (!a.w[j] || ((uintptr_t)a.w[j] & 15) || a.O[j] < 1 || (epi != WIDE_ARGMAX && (a.O[j] % 8))) return false;
+  if (a.form && a.form != 1) {
+    if (epi == WIDE_SWIGLU ? a.form < 64 || a.form > WG_MAX_FPT || (a.form % 16) : a.form < 1 || a.form > W_MAX_SPLIT || a.form > (a.I + TILE_K - 1) / TILE_K)
+      return false;
+    if (epi == WIDE_BF16 || epi == WIDE_ARGMAX) return false;
+  }
   return epi != WIDE_F32 || ((a.ldo % 4) == 0 && ((uintptr_t)a.out_f32 & 15) == 0);
 }
 
@@ -1088,6 +1093,8 @@ int wide_gemm_launch(TmaMaps *g, WideEpi epi, const WideGemmArgs &a, cudaStream_
   p.best_val = a.best_val; p.best_idx = a.best_idx; p.best_ld = a.best_ld;
   if (epi == WIDE_SWIGLU) {
     plan_swiglu(a.O[0], p.KB, p.m_tiles, &p.fpt);
+    if (a.form) p.fpt = a.form == 1 ? 0 : a.form;
+    if (a.used) *a.used = p.fpt ? p.fpt : 1;
     if (p.fpt) {
       for (int j = 0; j < 2; j++) {
         const CUtensorMap *mw = tma_maps_get(g, a.w[j], a.O[j], a.I, p.fpt / 2);
@@ -1100,6 +1107,10 @@ int wide_gemm_launch(TmaMaps *g, WideEpi epi, const WideGemmArgs &a, cudaStream_
   }
   int S = 1;
   plan_split(epi, p.m_tiles * p.n_tiles, p.KB, &S);
+  if (epi != WIDE_SWIGLU) {
+    if (a.form) S = a.form;
+    if (a.used) *a.used = S;
+  }
   if (S > 1) {
     switch (epi) {
       case WIDE_RESID: return launch_split<WIDE_RESID>(p, S, a.pdl, s);

@@ -51,6 +51,10 @@ struct WideGemmArgs {
   float *best_val = nullptr;    // [ceil(O/128)][best_ld]
   int32_t *best_idx = nullptr;
   int best_ld = 0;
+  // Form of the kernel, 0: the plan's choice.  WIDE_SWIGLU: features per tile (a multiple of 16 in 64..256), else K slices
+  // (1..4, for the epilogues that split; 1 also selects the persistent gate/up kernel).  `used` receives what ran.
+  int form = 0;
+  int *used = nullptr;
   // launch
   int32_t *status = nullptr;
   bool pdl = false;

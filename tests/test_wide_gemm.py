@@ -1,0 +1,61 @@
+"""The row-major GEMM kernels of wide passes one by one, in every form, at the edges of their tiles, against the CPU oracle."""
+import numpy as np
+import pytest
+import torch
+
+import pyoracle as po
+from paper_2503_01840_b200 import binding as sb
+
+pytestmark = pytest.mark.gpu
+
+
+def _rand(seed, *shapes):
+    g = torch.Generator().manual_seed(seed)
+    return [(torch.randn(*s, generator=g) / (1 if i == 0 else s[1] ** 0.5)).to(torch.bfloat16) for i, s in enumerate(shapes)]
+
+
+def _same(a, b):
+    return torch.equal(a.view(torch.int16 if a.dtype == torch.bfloat16 else torch.int32), b.view(torch.int16 if b.dtype == torch.bfloat16 else torch.int32))
+
+
+@pytest.mark.parametrize("form", [1, 2, 3, 4])
+@pytest.mark.parametrize("rows,O,I", [(1, 8, 264), (127, 136, 256), (128, 256, 320), (129, 248, 1000), (255, 512, 776), (256, 264, 4096), (257, 1024, 512),
+                                      (600, 504, 1160)])
+def test_row_major_gemm_vs_oracle(rows, O, I, form):
+    """One to three row tiles, whole and ragged feature tiles and contractions, one to four K slices (uneven ones too)."""
+    x, w = _rand(rows + O + I, (rows, I), (O, I))
+    out, used = sb.gemm_wide(x.cuda(), w.cuda(), form=form)
+    assert used == form
+    ref = po.linear(w, x.float().numpy())
+    # outputs of order 1 from exact products: fp32 sums of up to 4096 of them, in any order
+    assert np.abs(out.cpu().numpy() - ref).max() < 1e-4
+    assert _same(out, sb.gemm_wide(x.cuda(), w.cuda(), form=form)[0]), "the sum over the slices must be deterministic"
+
+
+@pytest.mark.parametrize("form", [1, 64, 80, 128, 208, 256])
+@pytest.mark.parametrize("rows,F,I", [(1, 8, 64), (128, 208, 320), (129, 1000, 264), (256, 416, 1024), (300, 520, 512), (513, 264, 136)])
+def test_row_major_gate_up_vs_oracle(rows, F, I, form):
+    """Tiles of 64 to 256 features per pair and the persistent kernel with 128, whole and ragged."""
+    x, wg, wu = _rand(rows + F + I, (rows, I), (F, I), (F, I))
+    out, used = sb.gemm_wide(x.cuda(), wg.cuda(), wu.cuda(), form=form)
+    assert used == form
+    xf = x.float().numpy()
+    ref = po.swiglu(po.linear(wg, xf), po.linear(wu, xf))
+    err = np.abs(out.float().cpu().numpy() - ref) - 2.0 ** -8 * np.abs(ref)          # one bf16 rounding of the result
+    assert err.max() < 1e-4, err.max()
+    assert _same(out, sb.gemm_wide(x.cuda(), wg.cuda(), wu.cuda(), form=form)[0])
+
+
+@pytest.mark.parametrize("rows,O,I,up,want", [(256, 4096, 4096, False, 3), (256, 4096, 14336, False, 3), (2048, 4096, 4096, False, 1), (256, 512, 1160, False, 4),
+                                              (256, 6144, 4096, False, 2), (256, 14336, 4096, True, 208), (3072, 14336, 4096, True, 1)])
+def test_the_plan_takes_several_forms(rows, O, I, up, want):
+    """The widths of the 8B-shaped layers run in the form with the fewest waves, and every form of the plan occurs among them."""
+    x, w = (torch.zeros(n, I, dtype=torch.bfloat16, device="cuda") for n in (rows, O))
+    assert sb.gemm_wide(x, w, w if up else None)[1] == want
+
+
+@pytest.mark.parametrize("rows,O,I,form", [(200, 100, 256, 0), (200, 128, 252, 0), (200, 128, 64, 2), (200, 128, 256, 5), (200, 128, 512, -1)])
+def test_unsupported_shapes_are_refused(rows, O, I, form):
+    x, w = (torch.zeros(n, I, dtype=torch.bfloat16, device="cuda") for n in (rows, O))
+    with pytest.raises(sb.SpecError):
+        sb.gemm_wide(x, w, form=form)
