@@ -322,6 +322,11 @@ int spec_ttt_attention(const void *q, const void *k_pool, const void *v_pool, co
  * in that CTA's rows. */
 int spec_debug_causal(int32_t mode);
 
+/* Test hook for the calling thread's launches of the row-major GEMM: 0 = off; 1 the persistent kernel, 2 the one split over K, 3
+ * the gate/up one with tiles of a chosen width: one CTA never receives its first activation tile, its bounded waits run out and the
+ * prefill returns SPEC_ERR_DEVICE_STATUS. */
+int spec_debug_wide_gemm(int32_t kernel);
+
 /* Per-row log-softmax + top-K (value desc, index asc) over fp32 logits [rows][n]: the expansion
  * step of the dynamic tree (Section 2.2; Appendix A "nodes during the expansion phase").  K <= 16.
  * out_idx int32 [rows][K], out_lp float [rows][K].  scratch: device buffer of

@@ -59,7 +59,7 @@ class _Cfg(C.Structure):
 EXPORTS = ("spec_workspace_bytes", "spec_init", "spec_prefill", "spec_step", "spec_step_async", "spec_step_sampled", "spec_plain_step",
            "spec_lengths", "spec_profile_step", "spec_tune", "spec_launches_per_step", "spec_step_bytes", "spec_free", "spec_last_error",
            "spec_debug_read", "spec_debug_read_kv", "spec_gemm", "spec_gemm_fused", "spec_gemm_swiglu", "spec_gemm_wide", "spec_gemm_topk_scratch_bytes", "spec_gemm_topk", "spec_ttt_attention_scratch_bytes", "spec_ttt_attention",
-           "spec_debug_causal", "spec_topk_scratch_bytes", "spec_attn_scratch_bytes",
+           "spec_debug_causal", "spec_debug_wide_gemm", "spec_topk_scratch_bytes", "spec_attn_scratch_bytes",
            "spec_attention", "spec_attention_static", "spec_attention_static_capacity", "spec_logsoftmax_topk", "spec_argmax")
 
 
@@ -111,6 +111,7 @@ def lib():
     L.spec_ttt_attention_scratch_bytes.restype = sz
     L.spec_ttt_attention.argtypes = [vp, vp, vp, vp, i32, i32, vp, vp, i32, vp, vp, i32, i32, i32, i32, vp, vp]
     L.spec_debug_causal.argtypes = [i32]
+    L.spec_debug_wide_gemm.argtypes = [i32]
     L.spec_gemm_wide.argtypes = [vp, vp, vp, vp, i32, i32, i32, i32, i32, C.POINTER(i32), vp]
     L.spec_topk_scratch_bytes.argtypes = [i32, i32, i32]
     L.spec_topk_scratch_bytes.restype = sz

@@ -15,10 +15,10 @@ template <typename T> __device__ __forceinline__ T from_f32(float v);
 template <> __device__ __forceinline__ float from_f32<float>(float v) { return v; }
 template <> __device__ __forceinline__ bf16 from_f32<bf16>(float v) { return __float2bfloat16_rn(v); }
 
-// Device status words: [0] error code (0 = fine), [1] where, [2..3] detail.
+// Device status words: [0] error code (0 = fine), [1] where, [2..3] detail.  The single-kernel entry points have none (null).
 enum { ST_OK = 0, ST_CAPACITY = 1, ST_BOUNDS = 2, ST_TIMEOUT = 3 };
 __device__ __forceinline__ void set_status(int32_t *st, int code, int where, int a = 0, int b = 0) {
-  if (atomicCAS(st, 0, code) == 0) { st[1] = where; st[2] = a; st[3] = b; }
+  if (st && atomicCAS(st, 0, code) == 0) { st[1] = where; st[2] = a; st[3] = b; }
 }
 
 // "a before b" in (value desc, index asc) order: the tie-break of every argmax / top-k of the step

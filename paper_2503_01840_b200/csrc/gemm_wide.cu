@@ -19,7 +19,7 @@
 // rows on the weight-streaming kernel): 64 prompts of 64..768 tokens, 8 layers of the 8B shapes, 24 chain steps 306 -> 156 ms;
 // 56 prompts of 16..96 tokens, 16 layers 268 -> 104 ms; 16384 tokens, 32 layers 535 -> 292 ms.
 //
-// Every mbarrier wait is bounded; on a time-out the CTA records it, stops, waits (bounded) for the copies in flight, keeps
+// Every mbarrier wait is bounded and answers a warp as one; on a time-out the CTA records it, stops, waits (bounded) for the copies in flight, keeps
 // its cluster barriers and frees its tensor memory.
 #include <cuda.h>
 #include <string.h>
@@ -30,6 +30,8 @@
 #include "tcgen05_ptx.cuh"
 
 namespace spec {
+
+thread_local int tl_wide_test = WIDE_TEST_OFF;
 
 namespace {
 
@@ -62,6 +64,8 @@ struct alignas(64) WideParams {
   int fpt, stages;               // gate/up kernel with tiles of a chosen width: features per tile, ring stages
   int32_t *status;
   unsigned long long *stamp;
+  int hold;                      // test hook: block 0 leaves out the activations of its first k-block
+  uint32_t spin;                 // polls before a wait gives up
 };
 
 // cache row of a row's K/V (-1: none); seq: the row's sequence, negative for padding (1 where the caller gave slots: a real row)
@@ -100,9 +104,9 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint32_t addr) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
 }
 // bounded wait for arrivals that come from both CTAs of the pair (cluster-scope acquire)
-__device__ __forceinline__ bool mbar_wait_cluster(uint64_t *bar, uint32_t parity) {
+__device__ __forceinline__ bool mbar_wait_cluster(uint64_t *bar, uint32_t parity, uint32_t limit) {
   const uint32_t addr = smem_u32(bar);
-  for (uint32_t it = 0; it < SPIN_LIMIT; it++) {
+  for (uint32_t it = 0; it < limit; it++) {
     uint32_t ok;
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
@@ -191,7 +195,7 @@ __global__ void __launch_bounds__(W_THREADS, 1) gemm_wide_kernel(const __grid_co
     const uint64_t pol = l2_policy_evict_first();
     int issued = 0, st = 0;
     uint32_t ph = 1;                             // a stage's first use needs no wait: the preceding phase counts as complete
-    bool ok = !*abort_flag, first = true;
+    bool ok = !__any_sync(0xffffffffu, *abort_flag != 0), first = true;
     for (int t = pair; t < ntiles && ok; t += n_pairs) {
       const int mt = t % p.m_tiles, nt = t / p.m_tiles;
       int mi = 0, tm = nt;
@@ -216,13 +220,13 @@ __global__ void __launch_bounds__(W_THREADS, 1) gemm_wide_kernel(const __grid_co
         __syncwarp();
         pdl_wait();
         if (elect_one())
-          for (int i = 0; i < npre; i++) tma_load_2d_pair(ring + i * W_STAGE, &p.map_x, i * TILE_K, xrow, mapa_u32(smem_u32(&full[i]), 0u));
+          for (int i = p.hold && blockIdx.x == 0 ? 1 : 0; i < npre; i++) tma_load_2d_pair(ring + i * W_STAGE, &p.map_x, i * TILE_K, xrow, mapa_u32(smem_u32(&full[i]), 0u));
         __syncwarp();
         kb = npre; issued = npre;
         if (npre == W_STAGES) ph = 0; else st = npre;
       }
       for (; kb < KB; kb++) {
-        if (!mbar_wait_warp(&empty[st], ph)) { *abort_flag = 1; set_status(p.status, ST_TIMEOUT, 240, blockIdx.x, t); ok = false; break; }
+        if (!mbar_wait_warp(&empty[st], ph, p.spin)) { *abort_flag = 1; set_status(p.status, ST_TIMEOUT, 240, blockIdx.x, t); ok = false; break; }
         if (elect_one()) {
           unsigned char *a = ring + st * W_STAGE;
           const uint32_t fb = mapa_u32(smem_u32(&full[st]), 0u);
@@ -241,7 +245,7 @@ __global__ void __launch_bounds__(W_THREADS, 1) gemm_wide_kernel(const __grid_co
   } else if (warp == W_EPI_WARPS + 1) {
     // ================================================================ MMA issuer (even CTA only)
     pdl_wait();
-    if (xr == 0 && !*abort_flag) {
+    if (xr == 0 && !__any_sync(0xffffffffu, *abort_flag != 0)) {
       constexpr uint32_t idesc = umma_idesc_m(256, 256);
       const uint64_t desc0 = umma_desc_sw128(smem_u32(ring));
       int consumed = 0, st = 0, it = 0;
@@ -250,13 +254,13 @@ __global__ void __launch_bounds__(W_THREADS, 1) gemm_wide_kernel(const __grid_co
       for (int t = pair; t < ntiles && ok; t += n_pairs, it++) {
         const int acc = it & 1, use = it >> 1;
         if (use > 0) {                           // both CTAs' epilogues have emptied this accumulator
-          const bool w = mbar_wait_cluster(&tempty[acc], (uint32_t)((use - 1) & 1));
+          const bool w = mbar_wait_cluster(&tempty[acc], (uint32_t)((use - 1) & 1), p.spin);
           if (!__all_sync(0xffffffffu, w)) { *abort_flag = 1; set_status(p.status, ST_TIMEOUT, 241, blockIdx.x, t); break; }
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         }
         const uint32_t d = tmem_base + (uint32_t)(acc * 256);
         for (int kb = 0; kb < KB; kb++) {
-          if (!ready && !mbar_wait_warp(&full[st], ph)) { *abort_flag = 1; set_status(p.status, ST_TIMEOUT, 242, blockIdx.x, t); ok = false; break; }
+          if (!ready && !mbar_wait_warp(&full[st], ph, p.spin)) { *abort_flag = 1; set_status(p.status, ST_TIMEOUT, 242, blockIdx.x, t); ok = false; break; }
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           const uint64_t da = desc0 + (uint64_t)((st * W_STAGE) >> 4), db = da + (W_A_BYTES >> 4);
           int nst = st + 1;
@@ -303,9 +307,9 @@ __global__ void __launch_bounds__(W_THREADS, 1) gemm_wide_kernel(const __grid_co
           xin[i] = (gr < p.rows && f < p.O[0]) ? *(const float4 *)(p.xres + (size_t)gr * p.O[0] + f) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
       }
-      bool ok = mbar_wait_warp(&tfull[acc], (uint32_t)(use & 1));
-      if (!ok || *abort_flag) {
-        if (!ok && lane == 0) { *abort_flag = 1; set_status(p.status, ST_TIMEOUT, 243, blockIdx.x, t); }
+      const bool ok = __all_sync(0xffffffffu, mbar_wait_warp(&tfull[acc], (uint32_t)(use & 1), p.spin) && !*abort_flag);
+      if (!ok) {
+        if (lane == 0) { *abort_flag = 1; set_status(p.status, ST_TIMEOUT, 243, blockIdx.x, t); }
         break;
       }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -499,7 +503,7 @@ __global__ void __launch_bounds__(W_THREADS, 1) gemm_wide_kernel(const __grid_co
   __syncthreads();
   if (*abort_flag && threadIdx.x == 0 && xr == 0) {
     // no bulk copy may still be landing when the pair exits (the even CTA's barriers count both CTAs' bytes)
-    for (int i = *n_consumed; i < *n_issued; i++) mbar_wait(&full[i % W_STAGES], (uint32_t)((i / W_STAGES) & 1));
+    for (int i = *n_consumed; i < *n_issued; i++) mbar_wait(&full[i % W_STAGES], (uint32_t)((i / W_STAGES) & 1), p.spin);
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   cluster_sync_all();
@@ -574,7 +578,8 @@ __global__ void __launch_bounds__(WS_THREADS, 1) gemm_wide_split_kernel(const __
     else if (tm >= p.h0) { mi = 1; tm -= p.h0; }
     const CUtensorMap *mw = &p.map_w[mi];
     const uint64_t pol = l2_policy_evict_first();
-    const int npre = *abort_flag ? 0 : nkb < W_STAGES ? nkb : W_STAGES;
+    const bool dead = __any_sync(0xffffffffu, *abort_flag != 0), hold = p.hold && blockIdx.x == 0;      // hold: test hook
+    const int npre = dead ? 0 : nkb < W_STAGES ? nkb : W_STAGES;
     if (elect_one())
       for (int i = 0; i < npre; i++) {
         if (xr == 0) mbar_expect_tx(&full[i], 2 * W_STAGE);
@@ -584,14 +589,14 @@ __global__ void __launch_bounds__(WS_THREADS, 1) gemm_wide_split_kernel(const __
     pdl_wait();
     if (elect_one()) {
       if (p.stamp) atomicMin(p.stamp, global_ns());
-      for (int i = 0; i < npre; i++) tma_load_2d_pair(ring + i * W_STAGE, &p.map_x, (kb0 + i) * TILE_K, row_c, mapa_u32(smem_u32(&full[i]), lead));
+      for (int i = hold ? 1 : 0; i < npre; i++) tma_load_2d_pair(ring + i * W_STAGE, &p.map_x, (kb0 + i) * TILE_K, row_c, mapa_u32(smem_u32(&full[i]), lead));
     }
     __syncwarp();
     int i = npre, st = 0;
     uint32_t ph = 0;
-    if (!*abort_flag)
+    if (!dead)
       for (; i < nkb; i++) {
-        if (!mbar_wait_warp(&empty[st], ph)) { *abort_flag = 1; set_status(p.status, ST_TIMEOUT, 250, blockIdx.x, i); break; }
+        if (!mbar_wait_warp(&empty[st], ph, p.spin)) { *abort_flag = 1; set_status(p.status, ST_TIMEOUT, 250, blockIdx.x, i); break; }
         if (elect_one()) {
           unsigned char *a = ring + st * W_STAGE;
           const uint32_t fb = mapa_u32(smem_u32(&full[st]), lead);
@@ -606,7 +611,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1) gemm_wide_split_kernel(const __
     if (lane == 0) *n_issued = i;
   } else if (warp == WS_EPI_WARPS + 1) {
     pdl_wait();
-    if (xr == 0 && !*abort_flag) {
+    if (xr == 0 && !__any_sync(0xffffffffu, *abort_flag != 0)) {
       constexpr uint32_t idesc = umma_idesc_m(256, 256);
       uint32_t partner_base;
       asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(partner_base) : "r"(mapa_u32(smem_u32(tmem_slot), crank | 1u)) : "memory");
@@ -616,7 +621,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1) gemm_wide_split_kernel(const __
       int i = 0, st = 0;
       uint32_t ph = 0, ready = 0;
       for (; ok && i < nkb; i++) {
-        if (!ready && !mbar_wait_warp(&full[st], ph)) { *abort_flag = 1; set_status(p.status, ST_TIMEOUT, 251, blockIdx.x, i); ok = false; break; }
+        if (!ready && !mbar_wait_warp(&full[st], ph, p.spin)) { *abort_flag = 1; set_status(p.status, ST_TIMEOUT, 251, blockIdx.x, i); ok = false; break; }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const uint64_t da = desc0 + (uint64_t)((st * W_STAGE) >> 4), db = da + (W_A_BYTES >> 4);
         int nst = st + 1;
@@ -646,9 +651,9 @@ __global__ void __launch_bounds__(WS_THREADS, 1) gemm_wide_split_kernel(const __
       }
     }
     // ---- accumulator -> shared memory: [half][row][128 floats], 16-byte chunks swizzled by the row
-    const bool ok = mbar_wait_warp(acc_bar, 0) && !*abort_flag;
+    const bool ok = __all_sync(0xffffffffu, mbar_wait_warp(acc_bar, 0, p.spin) && !*abort_flag);
     if (!ok) {
-      if (lane == 0 && !*abort_flag) set_status(p.status, ST_TIMEOUT, 252, blockIdx.x, slice);
+      if (lane == 0) set_status(p.status, ST_TIMEOUT, 252, blockIdx.x, slice);
       *abort_flag = 1;
     } else {
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -751,7 +756,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1) gemm_wide_split_kernel(const __
     }
   }
   if (*abort_flag && threadIdx.x == 0 && xr == 0)              // no bulk copy may still be landing when the cluster exits
-    for (int i = *n_consumed; i < *n_issued; i++) mbar_wait(&full[i % W_STAGES], (uint32_t)((i / W_STAGES) & 1));
+    for (int i = *n_consumed; i < *n_issued; i++) mbar_wait(&full[i % W_STAGES], (uint32_t)((i / W_STAGES) & 1), p.spin);
   cluster_sync_all();                                          // peers may still be reading this CTA's accumulator
   if (warp == WS_EPI_WARPS + 1) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(256) : "memory");
   if (p.stamp && threadIdx.x == 0) atomicMin(p.stamp + 1, ~global_ns());
@@ -805,7 +810,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1) gemm_wide_swiglu_kernel(const _
     const uint64_t pol = l2_policy_evict_first();
     int issued = 0, st = 0;
     uint32_t ph = 1;
-    bool ok = !*abort_flag, first = true;
+    bool ok = !__any_sync(0xffffffffu, *abort_flag != 0), first = true;
     for (int t = pair; t < ntiles && ok; t += n_pairs) {
       const int mt = t % p.m_tiles, nt = t / p.m_tiles;
       const int wrow = nt * fpt + xr * (fpt / 2), xrow = mt * WIDE_ROWS + xr * W_HALF;
@@ -823,13 +828,13 @@ __global__ void __launch_bounds__(WS_THREADS, 1) gemm_wide_swiglu_kernel(const _
         __syncwarp();
         pdl_wait();
         if (elect_one())
-          for (int i = 0; i < npre; i++) tma_load_2d_pair(ring + i * stage, &p.map_x, i * TILE_K, xrow, mapa_u32(smem_u32(&full[i]), 0u));
+          for (int i = p.hold && blockIdx.x == 0 ? 1 : 0; i < npre; i++) tma_load_2d_pair(ring + i * stage, &p.map_x, i * TILE_K, xrow, mapa_u32(smem_u32(&full[i]), 0u));
         __syncwarp();
         kb = npre; issued = npre;
         if (npre == stages) ph = 0; else st = npre;
       }
       for (; kb < KB; kb++) {
-        if (!mbar_wait_warp(&empty[st], ph)) { *abort_flag = 1; set_status(p.status, ST_TIMEOUT, 260, blockIdx.x, t); ok = false; break; }
+        if (!mbar_wait_warp(&empty[st], ph, p.spin)) { *abort_flag = 1; set_status(p.status, ST_TIMEOUT, 260, blockIdx.x, t); ok = false; break; }
         if (elect_one()) {
           unsigned char *a = ring + st * stage;
           const uint32_t fb = mapa_u32(smem_u32(&full[st]), 0u);
@@ -848,7 +853,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1) gemm_wide_swiglu_kernel(const _
     if (lane == 0) *n_issued = issued;
   } else if (warp == WS_EPI_WARPS + 1) {
     pdl_wait();
-    if (xr == 0 && !*abort_flag) {
+    if (xr == 0 && !__any_sync(0xffffffffu, *abort_flag != 0)) {
       const uint32_t idesc = umma_idesc_m(fpt, 256);
       const uint64_t desc0 = umma_desc_sw128(smem_u32(ring));
       int consumed = 0, st = 0, it = 0;
@@ -856,12 +861,12 @@ __global__ void __launch_bounds__(WS_THREADS, 1) gemm_wide_swiglu_kernel(const _
       bool ok = true;
       for (int t = pair; t < ntiles && ok; t += n_pairs, it++) {
         if (it > 0) {
-          const bool w = mbar_wait_cluster(tempty, (uint32_t)((it - 1) & 1));
+          const bool w = mbar_wait_cluster(tempty, (uint32_t)((it - 1) & 1), p.spin);
           if (!__all_sync(0xffffffffu, w)) { *abort_flag = 1; set_status(p.status, ST_TIMEOUT, 261, blockIdx.x, t); break; }
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         }
         for (int kb = 0; kb < KB; kb++) {
-          if (!ready && !mbar_wait_warp(&full[st], ph)) { *abort_flag = 1; set_status(p.status, ST_TIMEOUT, 262, blockIdx.x, t); ok = false; break; }
+          if (!ready && !mbar_wait_warp(&full[st], ph, p.spin)) { *abort_flag = 1; set_status(p.status, ST_TIMEOUT, 262, blockIdx.x, t); ok = false; break; }
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           const uint64_t da = desc0 + (uint64_t)((st * stage) >> 4), dg = da + (W_A_BYTES >> 4), du = dg + (uint64_t)(b_bytes >> 4);
           int nst = st + 1;
@@ -893,9 +898,9 @@ __global__ void __launch_bounds__(WS_THREADS, 1) gemm_wide_swiglu_kernel(const _
       const int mt = t % p.m_tiles, nt = t / p.m_tiles;
       const int row = mt * WIDE_ROWS + xr * W_HALF + quarter * 32 + lane;
       const float inv = row < p.rows ? row_scale(p, row) : 1.0f;
-      const bool ok = mbar_wait_warp(tfull, (uint32_t)(it & 1));
-      if (!ok || *abort_flag) {
-        if (!ok && lane == 0) { *abort_flag = 1; set_status(p.status, ST_TIMEOUT, 263, blockIdx.x, t); }
+      const bool ok = __all_sync(0xffffffffu, mbar_wait_warp(tfull, (uint32_t)(it & 1), p.spin) && !*abort_flag);
+      if (!ok) {
+        if (lane == 0) { *abort_flag = 1; set_status(p.status, ST_TIMEOUT, 263, blockIdx.x, t); }
         break;
       }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -927,7 +932,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1) gemm_wide_swiglu_kernel(const _
   }
   __syncthreads();
   if (*abort_flag && threadIdx.x == 0 && xr == 0)
-    for (int i = *n_consumed; i < *n_issued; i++) mbar_wait(&full[i % stages], (uint32_t)((i / stages) & 1));
+    for (int i = *n_consumed; i < *n_issued; i++) mbar_wait(&full[i % stages], (uint32_t)((i / stages) & 1), p.spin);
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   cluster_sync_all();
   if (warp == WS_EPI_WARPS + 1) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512) : "memory");
@@ -941,8 +946,14 @@ int n_tiles_of(WideEpi epi, const int *O, int nw) {
   return (h + 1) / 2;
 }
 
+void set_test(WideParams &p, WideTest kernel) {
+  p.hold = tl_wide_test == kernel;
+  p.spin = p.hold ? 2000u : SPIN_LIMIT;
+}
+
 template <int EPI>
-int launch_wide(const WideParams &p, bool pdl, cudaStream_t s) {
+int launch_wide(WideParams &p, bool pdl, cudaStream_t s) {
+  set_test(p, WIDE_TEST_PERSISTENT);
   static SmemLimit limit;
   if (!limit.ensure(gemm_wide_kernel<EPI>, W_SMEM)) return -6;
   if (!launch_allowed()) return 0;
@@ -962,7 +973,8 @@ int launch_wide(const WideParams &p, bool pdl, cudaStream_t s) {
 }
 
 template <int EPI, int S>
-int launch_split_inst(const WideParams &p, bool pdl, cudaStream_t s) {
+int launch_split_inst(WideParams &p, bool pdl, cudaStream_t s) {
+  set_test(p, WIDE_TEST_SPLIT);
   static SmemLimit limit;
   if (!limit.ensure(gemm_wide_split_kernel<EPI, S>, WS_SMEM)) return -6;
   if (!launch_allowed()) return 0;
@@ -981,7 +993,7 @@ int launch_split_inst(const WideParams &p, bool pdl, cudaStream_t s) {
   return cudaLaunchKernelEx(&cfg, gemm_wide_split_kernel<EPI, S>, p) == cudaSuccess ? 0 : -6;
 }
 template <int EPI>
-int launch_split(const WideParams &p, int S, bool pdl, cudaStream_t s) {
+int launch_split(WideParams &p, int S, bool pdl, cudaStream_t s) {
   switch (S) {
     case 2: return launch_split_inst<EPI, 2>(p, pdl, s);
     case 3: return launch_split_inst<EPI, 3>(p, pdl, s);
@@ -990,6 +1002,7 @@ int launch_split(const WideParams &p, int S, bool pdl, cudaStream_t s) {
 }
 
 int launch_swiglu(WideParams &p, bool pdl, cudaStream_t s) {
+  set_test(p, WIDE_TEST_GATE_UP);
   const int stage = W_A_BYTES + p.fpt * 128;
   p.stages = std::min(8, (W_SMEM - W_CTRL - 1024) / stage);
   static SmemLimit limit;
@@ -1129,3 +1142,9 @@ int wide_gemm_launch(TmaMaps *g, WideEpi epi, const WideGemmArgs &a, cudaStream_
 }
 
 }  // namespace spec
+
+extern "C" int spec_debug_wide_gemm(int32_t kernel) {
+  if (kernel < spec::WIDE_TEST_OFF || kernel > spec::WIDE_TEST_GATE_UP) return -1;
+  spec::tl_wide_test = kernel;
+  return 0;
+}

@@ -61,6 +61,11 @@ struct WideGemmArgs {
   unsigned long long *stamp = nullptr;   // profiling aid (see KernelStamp)
 };
 
+// Test hook of the calling thread's launches: in launches of one of the three kernels the first CTA never receives its first
+// activation tile, and the waits of the launch give up after 2000 polls.
+enum WideTest { WIDE_TEST_OFF = 0, WIDE_TEST_PERSISTENT = 1, WIDE_TEST_SPLIT = 2, WIDE_TEST_GATE_UP = 3 };
+extern thread_local int tl_wide_test;
+
 constexpr int WIDE_ROWS = 256;      // token rows per tile
 // what the launch's time goes with, in k-blocks (64 elements of the contraction, 0.27 us) of a tile
 long long wide_gemm_cost(WideEpi epi, const int *O, int nw, int I, int row_tiles);

@@ -51,6 +51,32 @@ def test_unfused_draft_logits_of_wide_passes(batch, draft_vocab):
     assert st.passes == 2 * 2 * batch and st.verify_compared == 2 * batch, st
 
 
+@pytest.mark.parametrize("kernel,hidden,prompt", [(1, 4096, 1300), (2, 512, 150), (3, 512, 150)])
+def test_row_major_wait_that_runs_out_is_reported(kernel, hidden, prompt):
+    """One CTA of each row-major kernel never receives its first activation tile (test hook): its bounded waits run out, the
+    CTAs of its cluster wind down, and the prefill returns the site of the wait.  A fresh decoder works afterwards."""
+    cfg = W4.replace(name="wait", hidden=hidden, n_heads=hidden // 128, n_kv_heads=max(2, hidden // 512), ffn=1024 if hidden == 4096 else 1408,
+                     batch=1 if hidden == 4096 else 4, tree_nodes=64)
+    tw, dw = synth.make_target_weights(cfg, device="cuda"), synth.make_draft_weights(cfg, device="cuda")
+    rng = np.random.default_rng(4)
+    prompts = [rng.integers(0, cfg.vocab, prompt).astype(np.int32) for _ in range(cfg.batch)]
+    seen = []
+    for hook in (0, kernel, 0):
+        dec = sb.SpecDecoder(cfg, tw, dw, batch=cfg.batch, max_ctx=prompt + 200)
+        sb.lib().spec_debug_wide_gemm(hook)
+        try:
+            if not hook:
+                seen.append([dec.prefill(prompts, 16), *dec.step()])
+                continue
+            with pytest.raises(sb.SpecError) as e:
+                dec.prefill(prompts, 16)
+            assert e.value.code == -7 and f"site {23 + kernel}" in str(e.value), str(e.value)
+        finally:
+            sb.lib().spec_debug_wide_gemm(0)
+            dec.close()
+    assert all(np.array_equal(a, b) for a, b in zip(*seen))
+
+
 def _off_grid(weights):
     """The same weights with every norm vector one element (two bytes) behind an 8-byte boundary."""
     def move(t):
