@@ -401,6 +401,7 @@ __global__ void __launch_bounds__(256) expand_kernel(SeqState st, TreeBufs tb, R
   for (int r = threadIdx.x; r < K; r += blockDim.x) {
     pm_lo[r] = (pass == 1) ? 0ull : m.mask_lo[b * K + r];
     pm_hi[r] = (pass == 1) ? 0ull : m.mask_hi[b * K + r];
+    newf[r] = r;                            // where scores are NaN the ranks below leave places out
   }
   for (int c = threadIdx.x; c < nch; c += blockDim.x) {
     int r = (pass == 1) ? 0 : c / K, cc = (pass == 1) ? c : c % K;
@@ -641,6 +642,7 @@ __global__ void __launch_bounds__(TREE_THREADS) draft_tree_step_kernel(const Tre
     }
   }
   if ((int)threadIdx.x < nchild4 - nchild) cscore[nchild + threadIdx.x] = -INFINITY;
+  if ((int)threadIdx.x < K) newf[threadIdx.x] = threadIdx.x;           // where scores are NaN the ranks below leave places out
   __syncthreads();
   if (pass >= D) return;
   // ---- 3. next frontier: the K best children of the level, (score desc, pool index asc)

@@ -77,6 +77,24 @@ def test_row_major_wait_that_runs_out_is_reported(kernel, hidden, prompt):
     assert all(np.array_equal(a, b) for a, b in zip(*seen))
 
 
+@pytest.mark.parametrize("topk", [5, 16])
+def test_draft_logits_that_are_not_numbers(topk):
+    """A draft whose logits are all NaN gives some tree of valid tokens (fused and separate expansion kernels), and the steps
+    emit what plain decoding emits."""
+    cfg = W4.replace(name="nan", batch=2, tree_depth=3, tree_topk=topk)
+    tw, dw = synth.make_target_weights(cfg, device="cuda"), synth.make_draft_weights(cfg, device="cuda")
+    dw["lm_head"] = torch.full_like(dw["lm_head"], float("nan"))
+    prompts = [np.arange(30, dtype=np.int32), np.arange(7, 40, dtype=np.int32)]
+    spec, plain = (sb.SpecDecoder(cfg, tw, dw, batch=2, max_ctx=300) for _ in range(2))
+    assert np.array_equal(spec.prefill(prompts, 32), plain.prefill(prompts, 32))
+    out = [np.concatenate(x) for x in zip(spec.step(), spec.step())]
+    ref = np.stack([plain.plain_step() for _ in range(max(map(len, out)))], 1)
+    # one decision can be a near-tie that another order of sums turns: the first token of each sequence is compared
+    assert all(o[0] == r[0] and ((0 <= o) & (o < cfg.vocab)).all() for o, r in zip(out, ref))
+    spec.close()
+    plain.close()
+
+
 def _off_grid(weights):
     """The same weights with every norm vector one element (two bytes) behind an 8-byte boundary."""
     def move(t):
