@@ -115,11 +115,19 @@ __global__ void __launch_bounds__(128) gemm_skinny_kernel(const float *__restric
   }
 }
 
-// Rows up to which the warp-per-feature kernel is taken: always up to 32 (every weight is read once), beyond that while
-// the weights fit the L2 comfortably (they are read once per 32 rows).
+// When the warp-per-feature kernel is taken: up to 32 rows every weight is read once; up to 256 rows while the weights fit the
+// L2 comfortably (they are read once per 32 rows); and in either case only where it is the shorter one.  Its time goes with
+// (rows padded to a group) x features x (contraction + 192: the exchange costs as much as 192 elements), spread over the chip
+// from a few thousand warps on; the tile kernel's goes with the contraction alone until its 64 x 64 tiles fill the chip (256 of
+// them).  The line is a fit to both kernels' times at 900 shapes of 1 to 256 rows, 64 to 128256 features, 16 to 4096 elements (tile / this
+// kernel, us, binding included): 256 x 4096 x 64 13.3 / 29.2, x 256 39.4 / 43.6, x 512 72 / 68, x 1024 138 / 125; 64 x 4096 x
+// 64 11.5 / 11.8, x 256 31 / 14.7; 32 x 128256 x 64 54 / 99, 4 x 4096 x 256 29 / 12.
 static bool skinny_ok(const float *x, const float *w, int rows, int O, int I) {
   if ((I & 3) || (((uintptr_t)x | (uintptr_t)w) & 15)) return false;
-  return rows <= 32 || (rows <= 256 && (long long)O * I <= (4 << 20));
+  if (rows > 256 || (rows > 32 && (long long)O * I > (4 << 20))) return false;
+  const int padded = rows <= 4 ? 4 : rows <= 8 ? 8 : rows <= 16 ? 16 : (rows + 31) / 32 * 32;
+  const double tiles = (double)((O + 63) / 64) * ((rows + 63) / 64);
+  return (double)padded * O * (I + 192) <= 1.31e6 * I * std::max(1.0, tiles / 256);
 }
 static void launch_skinny(const float *x, SkinnyWeights sw, float *out, int rows, int O, int I, int ldo, cudaStream_t s) {
   auto go = [&](auto kern, int R, int C) { launch_k(kern, dim3((O + 4 * C - 1) / (4 * C), (rows + R - 1) / R), dim3(128), 0, s, x, sw, out, rows, O, I, ldo); };

@@ -10,10 +10,12 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("rows,O,I,shift", [(1, 1, 4, 0), (3, 31, 128, 0), (4, 256, 256, 0), (5, 33, 688, 0), (8, 8, 12, 0), (9, 1000, 260, 0),
                                             (16, 100, 768, 0), (17, 65, 132, 0), (32, 7, 512, 0), (33, 300, 256, 0), (256, 64, 128, 0),
-                                            (257, 64, 128, 0), (64, 2049, 2052, 0), (4, 50, 30, 0), (4, 50, 32, 1)])
+                                            (257, 64, 128, 0), (64, 2049, 2052, 0), (4, 50, 30, 0), (4, 50, 32, 1),
+                                            (256, 4096, 64, 0), (17, 16390, 32, 0), (16, 33000, 16, 0)])
 def test_fp32_gemm_row_groups(rows, O, I, shift):
     """Every row group of the warp-per-feature kernel, its remainders, and the shapes that stay on the tile kernel (a
-    contraction that is no multiple of four, operands off a 16-byte boundary, many rows of a large weight)."""
+    contraction that is no multiple of four, operands off a 16-byte boundary, many rows of a large weight, a contraction that is
+    short for its many outputs)."""
     g = torch.Generator().manual_seed(rows * 1000 + O + I)
     x, w = torch.randn(rows, I, generator=g), torch.randn(O, I, generator=g)
 
