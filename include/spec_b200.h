@@ -242,7 +242,8 @@ int spec_gemm_wide(const void *x, const void *w, const void *w_up, void *out, in
  * best logits, and a merge kernel turns them into each row's K best ids (value descending, lower id first on ties) and
  * their log-probabilities.  x [rows][in] bf16, w [out][in] bf16, out_idx int32 [rows][K], out_lp float [rows][K];
  * scratch: spec_gemm_topk_scratch_bytes(rows, out, K) bytes of device memory.  rows <= 256, in % 8 == 0, K <= 15,
- * out <= 32768 and out / 128 * K <= 3200 (SPEC_ERR_UNSUPPORTED otherwise). */
+ * out <= 32768 and, with t = out / 128 rounded up to a multiple of 4, 80 t K + 16 K K + 12 K <= 225216 (SPEC_ERR_UNSUPPORTED
+ * otherwise). */
 size_t spec_gemm_topk_scratch_bytes(int32_t rows, int32_t out, int32_t K);
 int spec_gemm_topk(const void *x, const void *w, int32_t rows, int32_t out, int32_t in, int32_t K, int32_t *out_idx,
                    float *out_lp, void *scratch, void *stream);

@@ -721,8 +721,9 @@ __global__ void __launch_bounds__(TREE_THREADS) draft_tree_step_kernel(const Tre
   }
 }
 
-// Shapes the kernel takes (the others use the separate kernels): at most eight tiles per lane, at most 220 KB of candidates
-// for the ten rows of a level.
+// Shapes the kernel takes (the others use the separate kernels): at most eight tiles per lane and 15 candidates per tile in
+// registers.  The kernel itself has no other limit.  The product of the two is the line between the calls that spec_gemm_topk
+// takes and refuses; it dates from a form that staged the candidates of a level's ten rows in 220 KB of shared memory.
 int draft_tree_cand_ld(int tiles) { return (tiles + 3) & ~3; }
 bool draft_tree_step_fits(int tiles, int K) {
   if (tiles > 256 || K > 15) return false;
