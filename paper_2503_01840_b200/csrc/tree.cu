@@ -469,9 +469,11 @@ __device__ __forceinline__ void merge_tile_candidates(const float *__restrict__ 
                                                       int tiles, int ld, int row, int K, int32_t *out_id, float *out_lp) {
   const int lane = threadIdx.x & 31;
   float pm[8], ps[8];                                    // at most 8 tiles per lane, all loads issued before the first use
+  int head[8];                                           // K = 1: the tiles' best are all the candidates there are (one load less to wait for)
 #pragma unroll
   for (int j = 0; j < 8; j++) {
     const int t = lane + 32 * j;
+    head[j] = (K == 1 && t < tiles) ? cand_idx[(size_t)row * ld + t] : -1;
     pm[j] = t < tiles ? cand_max[(size_t)row * ld + t] : -INFINITY;
     ps[j] = t < tiles ? cand_sum[(size_t)row * ld + t] : 0.0f;
   }
@@ -479,33 +481,41 @@ __device__ __forceinline__ void merge_tile_candidates(const float *__restrict__ 
 #pragma unroll
   for (int j = 0; j < 8; j++) mx = fmaxf(mx, pm[j]);
   for (int off = 16; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-  // ---- the K best tiles, (head desc, tile asc): lane c keeps the c-th
-  const int nsel = K < tiles ? K : tiles;
   unsigned key[8];
 #pragma unroll
   for (int j = 0; j < 8; j++) key[j] = lane + 32 * j < tiles ? ordered_key(pm[j]) : 0u;      // keys of values are >= 1
-  int sel = 0;
-  for (int c = 0; c < nsel; c++) {
-    unsigned bk = 0u, wk;
-    int bt = -1;
-#pragma unroll
-    for (int j = 0; j < 8; j++)
-      if (key[j] > bk) { bk = key[j]; bt = lane + 32 * j; }
-    const int w = warp_best(bk, bt, &wk);
-    if (lane == c) sel = w;
-#pragma unroll
-    for (int j = 0; j < 8; j++)
-      if (lane + 32 * j == w) key[j] = 0u;
-  }
-  // ---- lane c holds the c-th tile's candidates, best first: only their heads compete, and the winner's list moves up
   unsigned ck[15];
   int ci[15];
+  if (K == 1) {                                          // each lane's best head, by (value desc, tile asc)
 #pragma unroll
-  for (int i = 0; i < 15; i++) {
-    const bool have = lane < nsel && i < K;
-    const size_t at = ((size_t)row * ld + sel) * K + i;
-    ci[i] = have ? cand_idx[at] : -1;
-    ck[i] = have ? ordered_key(cand_val[at]) : 0u;
+    for (int i = 0; i < 15; i++) { ck[i] = 0u; ci[i] = -1; }
+#pragma unroll
+    for (int j = 0; j < 8; j++)
+      if (head[j] >= 0 && key[j] > ck[0]) { ck[0] = key[j]; ci[0] = head[j]; }
+  } else {
+    // ---- the K best tiles, (head desc, tile asc): lane c keeps the c-th
+    const int nsel = K < tiles ? K : tiles;
+    int sel = 0;
+    for (int c = 0; c < nsel; c++) {
+      unsigned bk = 0u, wk;
+      int bt = -1;
+#pragma unroll
+      for (int j = 0; j < 8; j++)
+        if (key[j] > bk) { bk = key[j]; bt = lane + 32 * j; }
+      const int w = warp_best(bk, bt, &wk);
+      if (lane == c) sel = w;
+#pragma unroll
+      for (int j = 0; j < 8; j++)
+        if (lane + 32 * j == w) key[j] = 0u;
+    }
+    // ---- lane c holds the c-th tile's candidates, best first: only their heads compete, and the winner's list moves up
+#pragma unroll
+    for (int i = 0; i < 15; i++) {
+      const bool have = lane < nsel && i < K;
+      const size_t at = ((size_t)row * ld + sel) * K + i;
+      ci[i] = have ? cand_idx[at] : -1;
+      ck[i] = have ? ordered_key(cand_val[at]) : 0u;
+    }
   }
   // the log-sum-exp while they are on their way: a lane adds its tiles in tile order, then a fixed shuffle tree
   float sum = 0.0f;
