@@ -451,7 +451,9 @@ template <typename T> struct Sched {
   }
   // From 129 rows on (up to 256: batches, and whole trees at a small batch) a weight byte meets more flops than the
   // weight-streaming kernel's tiles feed the tensor pipe with: it re-reads the 32 KB activation k-block for every 128
-  // features and spends as long in its 256-row epilogues as in its loops.  These passes take the row-major kernel.
+  // features and spends as long in its 256-row epilogues as in its loops.  These passes take the row-major kernel.  Alone (8B
+  // shapes, launches from a graph without the passes' epilogues, weight-streaming / row-major, us): QKV 23.4 / 19.2 at 144 rows, 30.9 / 20.0
+  // at 256; O 16.2 / 17.5, 19.5 / 18.5; down 30.8 / 32.6, 34.9 / 34.3; gate/up 56.7 / 57.8 at 192 and 58.9 / 53.9 at 256.
   bool row_major(FusedEpi epi, const FusedGemmArgs &a) const {
     return a.rows > (epi == EPI_SWIGLU ? 192 : 128) && !a.withhold && !fused_gemm_pairs() && epi != EPI_TOPK && (epi != EPI_QKV || a.hd == 128);
   }
@@ -564,8 +566,9 @@ template <typename T> struct Sched {
     }
     block_fused(c->dl, c->pools[c->L], rows, tail_len, c->dfinal_norm, 0);
   }
-  // Worth a gather launch (2-3 us) when B rows take a narrower GEMM tile than B * (D + 1): 256 -> 64 rows is 297 -> 159 us
-  // for the four GEMMs of the 8B shapes, 28 -> 4 rows 132 -> 117 us.
+  // Worth a gather launch (2-3 us) when B rows take a narrower GEMM tile than B * (D + 1): the four GEMMs of the 8B shapes (O,
+  // gate/up, down, draft LM head; launches from a graph, without the passes' epilogues) take 214 us for 256 rows, 148 for 64, 135
+  // for 28 and 122 for 4.
   static int tile_class(int rows) { return rows <= 16 ? 0 : rows <= 64 ? 1 : rows <= 128 ? 2 : 3; }
   bool extend_compact() const { return c->tree_fused && tile_class(c->B) < tile_class(c->Te); }
   void draft_logits_fused(int rows) {

@@ -1025,8 +1025,9 @@ int launch_swiglu(WideParams &p, bool pdl, cudaStream_t s) {
 
 // Measured at 168 to 256 rows in the replayed step of the 8B shapes (weight-streaming kernel -> this one): QKV 26.7 -> 18.3 us, O 18.5 ->
 // 17.8, down 33.4 -> 33 (168 rows); 31.7 -> 18.9, 22 -> 17.9, 38 -> 33 (240 rows); LM head 276 -> 180.
-// Clusters of 2 S CTAs (one CTA per SM) that are resident at once: a cluster lives inside one GPC, whose SM counts the
-// driver reports as 33, 22 and 15 clusters of 4, 6 and 8 on this chip.
+// Whole requests with 129, 144 and 160 rows a step (4 layers, 12 steps, their prefill included): 32.1 -> 26.4 ms, 31.8 -> 26.4, 36.4 -> 28.8.
+// Clusters of 2 S CTAs (one CTA per SM) that are resident at once: a cluster lives inside one GPC, and this chip's GPCs hold
+// 33, 22 and 15 clusters of 4, 6 and 8.  Constants: on a chip cut otherwise the plan may take one wave for two, no result changes.
 constexpr int W_MAX_SPLIT = 4;
 constexpr int W_FIT[W_MAX_SPLIT + 1] = {0, W_PAIRS, 33, 22, 15};
 // What a launch costs beside its k-blocks, in k-blocks: the epilogue of the last tile (persistent kernel), or parking,

@@ -568,9 +568,8 @@ def test_lm_head_topk_epilogue_and_merge_bit_exact(O, K):
 
 @pytest.mark.parametrize("T,H,G,J", [(300, 8, 2, 3), (128, 4, 4, 0), (517, 32, 8, 1), (70, 8, 2, 8)])
 def test_ttt_attention_vs_oracle(T, H, G, J):
-    """Training-time-test attention (Section 3.2): dense causal part on the tensor-core tile kernel over 128-position
-    blocks (several blocks and a ragged last one), diagonal entries of J simulated steps as dot products, shuffled pages;
-    sampled positions (all block boundaries among them) x every head against the oracle's definition: outputs within the
+    """Training-time-test attention (Section 3.2) on the causal tensor-core kernel: several blocks of positions and a ragged
+    last one, diagonal entries of J simulated steps as dot products, shuffled pages; sampled positions (all block boundaries among them) x every head against the oracle's definition: outputs within the
     bf16 tolerance 2e-2, log-normalisers within 2e-2."""
     hd, ps = 128, 16
     g = torch.Generator().manual_seed(T * 7 + J)
@@ -600,7 +599,8 @@ def test_ttt_attention_vs_oracle(T, H, G, J):
 
 @pytest.mark.parametrize("rows,O,I,split", [(256, 512, 512, 2), (200, 4096, 4096, 0), (129, 768, 1024, 1), (256, 1024, 4096, 4)])
 def test_gemm_cta_pairs_bit_equal(rows, O, I, split):
-    """256-row GEMM tiles as CTA pairs (one M = 256 MMA over two CTAs, each loading half of the activation rows) against
+    """256-row tiles of the weight-streaming GEMM (an optional mode; passes of more than 128 rows run the row-major kernel
+    otherwise) as CTA pairs (one M = 256 MMA over two CTAs, each loading half of the activation rows) against
     the single-CTA kernel: the same products are added in the same order, so the results must be bit-identical; and
     against a float64 matmul within the bf16-input tolerance."""
     g = torch.Generator().manual_seed(rows + O + I)
@@ -623,7 +623,7 @@ def test_gemm_cta_pairs_bit_equal(rows, O, I, split):
 
 @pytest.mark.parametrize("rows,F,I", [(256, 512, 512), (200, 1024, 4096), (129, 1792, 1024), (256, 384, 1024)])
 def test_gate_up_cta_pairs_bit_equal(rows, F, I):
-    """The 256-row gate/up kernel as CTA pairs (the default) against single CTAs: bit-identical activations, and both
+    """The 256-row gate/up kernel (passes of 129 to 192 rows) as CTA pairs (the default) against single CTAs: bit-identical activations, and both
     within bf16 rounding of SiLU(x Wg^T) * (x Wu^T) computed in float64."""
     g = torch.Generator().manual_seed(rows + F + I)
     x = torch.randn(rows, I, generator=g).to(torch.bfloat16).cuda()
