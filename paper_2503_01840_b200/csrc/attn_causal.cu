@@ -13,17 +13,17 @@
 //    are ready when a warpgroup comes for them, and no contraction lies on its path from one softmax to the next;
 //  * each tile has an MMA-issuing warp of its own (one warp for both spent 1200 of 2230 cycles per 64-key step on waits,
 //    commits and issue while the softmax waited for it);
-//  * a row whose reference maximum moves (by more than 2^8 in the exponent, rare after the first steps) waits for its last
-//    P V and rescales its O; no other step waits for one;
+//  * a row whose reference maximum moves (see CA_EARLY; rare after the first steps) waits for its last P V and rescales its O;
+//    no other step waits for one;
 //  * only the steps that cross the diagonal are masked;
-//  * the diagonal entries of training-time test come through the same K / V ring as further tiles (row = position), whose
+//  * the diagonal entries of training-time test come through the K and V rings as further tiles (row = position), whose
 //    dot products the softmax threads take from shared memory.
 //
-// Measured (one B200, T = 8192, 32 / 8 heads, 3 diagonal entries per row): 0.55 ms = 1000 TFLOP/s of causal flops (0.50 ms
-// without diagonal entries).  With one 128-key score buffer per tile and one issuer: 0.67 ms; the same with an issuer per
-// tile and P V in two halves: 0.59 ms; two 64-key buffers and one issuer: 0.68 ms.  A 64-key step takes 1600 cycles: shared
-// memory delivers the operands of its MMAs and takes in the next tiles in 1250 (128 x 64 x 16 MMAs read 6 KB per 32 tensor
-// cycles), the exponentials take 1024.
+// Measured (one B200, T = 8192, 32 / 8 heads, 3 diagonal entries per row): 0.54 ms = 1020 TFLOP/s of causal flops (0.50 ms
+// without diagonal entries) called in a row on the same inputs, 0.62 ms on inputs that change from call to call.  Earlier forms,
+// in a row: one 128-key score buffer per tile and one issuer 0.67 ms; the same with an issuer per tile and P V in two halves
+// 0.59; two 64-key buffers and one issuer 0.68.  A 64-key step takes 1600 cycles: shared memory delivers the operands of its
+// MMAs and takes in the next tiles in 1250 (128 x 64 x 16 MMAs read 6 KB per 32 tensor cycles), the exponentials take 1024.
 //
 // Every wait is bounded.  On a time-out the CTA winds down; a prefill's status words record it, and training-time test, which
 // has none, gets NaN in the rows (and normalisers) it could not finish.
@@ -60,15 +60,17 @@ constexpr int CA_SMEM = (2 + 2 * CA_STAGES) * CA_TILE + CA_CTRL + 1024;
 constexpr int CA_THREADS = 384, CA_REGS_SOFTMAX = 208, CA_REGS_ISSUE = 88;
 static_assert(256 * CA_REGS_SOFTMAX + 128 * CA_REGS_ISSUE <= CA_THREADS * 168, "register shares must fit what the block is launched with");
 constexpr int CA_MAX_DIAG = 8;
-// How closely a row's reference maximum follows its maximum.  P is bf16, so the error of an output comes from the row's largest
-// probabilities; it is least when those lie at or just below 1, i.e. when the reference is the maximum.  The prefill moves the
-// reference by jumps beyond 2^CA_FAR only (each costs a rescaled O; the error of a layer's activations hides the difference).
-// Training-time test follows jumps beyond 2^CA_NEAR while the maximum settles, in a row's first CA_EARLY steps.  Sequences of
-// at most CA_BRIEF positions have few and therefore large probabilities: they follow closely throughout and divide by the sum
-// of the rounded ones, which O sums, so that the rounding of a large one partly cancels (a kernel of its own: the second sum costs 5 to
-// 8 % wherever it stands).  Relative error against fp64 in 1e-3 (the bf16 output alone is 1.66) and time: T = 8192, 32 / 8 heads, 3
-// diagonal entries: jumps of 2^8 only 2.175, 551 us; this 2.141, 552; 2^1 throughout 2.123, 588; rounded sum and 2^0.5 in the
-// first 8 steps 2.125, 582.  T = 256, 16 / 16 heads: jumps of 2^8 only 1.958, 2^0.5 1.927, with the rounded sum 1.903; T = 512, 32 / 8 heads, 3 entries 2.073 (26 us) and 2.011 (29).
+// How closely a row's reference maximum follows its maximum.  P is bf16, so the error of an output comes from the row's
+// largest probabilities; it is least when those lie at or just below 1, i.e. when the reference is the maximum.  The prefill
+// moves the reference by jumps beyond 2^CA_FAR only (each costs a rescaled O; the rounding of a layer's activations hides the
+// difference).  Training-time test follows jumps beyond 2^CA_NEAR while the maximum settles, in a row's first CA_EARLY steps.
+// Sequences of at most CA_BRIEF positions have few and therefore large probabilities: they follow closely throughout and
+// divide by the sum of the rounded ones, which O sums, so that the rounding of a large one partly cancels (a kernel of its own:
+// the second sum costs 5 to 8 % wherever it stands).
+// Relative error against fp64 in 1e-3 (the bf16 output alone is 1.66) and time.  T = 8192, 32 / 8 heads, 3 diagonal entries:
+// jumps of 2^8 only 2.175, 551 us; this 2.141, 539; 2^1 throughout 2.123, 588; rounded sum and 2^0.5 in the first 8 steps 2.125,
+// 582.  T = 512, 32 / 8 heads, 3 entries: 2^8 only 2.073, 26 us; 2^0.5 in the first 4 steps 2.034, 26; this 2.011, 29.  T = 256,
+// 16 / 16 heads: 1.958, 1.927 and 1.903, 19 us each.
 constexpr int CA_EARLY = 4, CA_BRIEF = 512;
 constexpr float CA_NEAR = 0.5f, CA_FAR = 8.0f;
 
@@ -368,12 +370,14 @@ __global__ void __launch_bounds__(CA_THREADS, 1) attn_causal_kernel(const __grid
       // the warp's other rows then move along)
       const float jump = DIAG && (BRIEF || i < CA_EARLY) ? CA_NEAR : CA_FAR;
       float f = 1.0f;
-      const bool over = tm > mx && (tm - mx) * sc > jump;
-      if (DIAG ? __any_sync(0xffffffffu, over) && tm > mx : over) {
+      bool move = (tm - mx) * sc > jump;
+      if (DIAG) move = __any_sync(0xffffffffu, move);
+      if (move && tm > mx) {
         f = (mx == -INFINITY) ? 1.0f : ex2((mx - tm) * sc);
         mx = tm;
       }
-      if (i > 0 && __any_sync(0xffffffffu, f != 1.0f)) {         // the P V of the last step must be complete before O is rescaled
+      if (!DIAG) move = __any_sync(0xffffffffu, f != 1.0f);
+      if (i > 0 && move) {                                       // the P V of the last step must be complete before O is rescaled
         ok = mbar_wait_warp(&o_bar[t], (uint32_t)((i - 1) & 1), p.spin);
         if (!ok) { if (lane == 0) { *abort_flag = 1; if (p.status) set_status(p.status, ST_TIMEOUT, 438, blockIdx.y, i); } alive = false; break; }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
