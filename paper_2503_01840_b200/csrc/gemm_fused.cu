@@ -55,7 +55,7 @@ struct alignas(64) FusedParams {
   float *out_f32; int ldo;
   float *xres; const bf16 *gain; bf16 *hb; float *ssq_out; bf16 *taps; int tap_mask, resid_add;
   const float2 *cs; RowMeta m; bf16 *q; KvPool pool; PageMap pm; int H, G, hd;
-  bf16 *act;
+  bf16 *act; int act_vec;                  // act_vec: pairs of features may be stored as one word
   float *best_val; int32_t *best_idx; int best_ld;
   int topk; float *cand_val, *cand_max, *cand_sum; int32_t *cand_idx; int cand_ld; const int32_t *want_rows; int n_want;
   int32_t *status;
@@ -119,6 +119,13 @@ __device__ __forceinline__ float4 sum_peers4(uint32_t local_addr, int s0, int n,
 // separate cluster members), the two accumulators sit side by side in tensor memory, and the cluster holds only the
 // Sk K slices.
 //
+// MIX (EPI_SWIGLU only): one 128-row weight tile made of 64 gate features and the 64 up features of the same range, the whole
+// contraction in one CTA.  It takes the place of PAIR with two K slices: the same number of CTAs, but no cluster, no parked
+// partial sums and no exchange through distributed shared memory, which cost 5 us of a launch at 60 rows (the launch is bound by
+// the weight stream, and what comes after the last k-block is not hidden by it).  8B shapes, inside the replayed step: 46.6 ->
+// 41.7 us at 60 rows, 38.0 -> 34.5 at 10, 43.8 -> 40.2 at 40; 13B shapes at 50 rows 52.6 -> 47.3; C2 step 4.950 -> 4.775 ms.  The
+// activation k-block is read once per 64 features instead of 128 (1.5 bytes from L2 per weight byte at 60 rows against 1.25).
+//
 // DUO (256-row tiles; EPI_F32 / EPI_RESID / EPI_QKV): two neighbouring feature tiles run as a CTA pair (cta_group::2).
 // Each CTA streams its own weight tile but only HALF of the activation k-block (128 of the 256 rows); the even CTA issues
 // one M = 256 MMA per k-step that reads both CTAs' shared memory, and each CTA's tensor memory receives the accumulator
@@ -130,12 +137,14 @@ __device__ __forceinline__ float4 sum_peers4(uint32_t local_addr, int s0, int n,
 // as long as its main loop).
 constexpr int fused_threads(int nt, int epi) { return (nt == 256 && (epi == EPI_F32 || epi == EPI_RESID || epi == EPI_QKV)) ? 256 : 128; }
 
-template <int NT, int EPI, bool PAIR = false, bool DUO = false>
+template <int NT, int EPI, bool PAIR = false, bool DUO = false, bool MIX = false>
 __global__ void __launch_bounds__(fused_threads(NT, EPI)) gemm_fused_kernel(const __grid_constant__ FusedParams p) {
   constexpr int THREADS = fused_threads(NT, EPI), NH = THREADS / 128;
   static_assert(!PAIR || EPI == EPI_SWIGLU, "two weight tiles per CTA exist for the gate/up epilogue only");
+  static_assert(!MIX || (EPI == EPI_SWIGLU && !PAIR && !DUO), "tiles of 64 gate and 64 up features exist for the gate/up epilogue only");
   static_assert(!DUO || (NT == 256 && !PAIR && (EPI == EPI_F32 || EPI == EPI_RESID || EPI == EPI_QKV)), "CTA pairs serve the 256-row tiles");
   constexpr int A_TILES = PAIR ? 2 : 1;
+  constexpr int F_TILE = MIX ? TILE_M / 2 : TILE_M;            // output features of a tile
   constexpr int B_BYTES = (DUO ? NT / 2 : NT) * TILE_K * 2;
   constexpr int STAGE = A_TILES * A_BYTES + B_BYTES;
   constexpr int TMEM_COLS = (A_TILES * NT < 32) ? 32 : A_TILES * NT;
@@ -158,12 +167,12 @@ __global__ void __launch_bounds__(fused_threads(NT, EPI)) gemm_fused_kernel(cons
   const uint32_t crank = (S > 1 || DUO) ? cluster_rank() : 0u;
   const int xr = DUO ? (int)(crank & 1u) : 0;                 // DUO: position in the CTA pair (0 issues the MMAs)
   const int slice = DUO ? (int)(crank >> 1) : (int)crank;     // K slice = rank among the CTAs that share this feature tile
-  const int ksl = (EPI == EPI_SWIGLU && !PAIR) ? slice % Sk : slice;   // K slice
+  const int ksl = (EPI == EPI_SWIGLU && !PAIR && !MIX) ? slice % Sk : slice;   // K slice
   const int kb0 = (int)(((long long)ksl * p.KB) / Sk), kb1 = (int)(((long long)(ksl + 1) * p.KB) / Sk);
   const int nkb = kb1 - kb0;
   int mi = 0, tm = blockIdx.x;                   // weight index and tile within that weight
   if (EPI == EPI_SWIGLU) {
-    mi = PAIR ? 0 : slice / Sk;                  // ranks [0,Sk) stream the gate tile, [Sk,2Sk) the up tile
+    mi = PAIR || MIX ? 0 : slice / Sk;                  // ranks [0,Sk) stream the gate tile, [Sk,2Sk) the up tile
   } else {
     if (tm >= p.tiles1) { mi = 2; tm -= p.tiles1; }
     else if (tm >= p.tiles0) { mi = 1; tm -= p.tiles0; }
@@ -246,7 +255,8 @@ __global__ void __launch_bounds__(fused_threads(NT, EPI)) gemm_fused_kernel(cons
       for (int i = 0; i < npre; i++) {
         unsigned char *a = tiles + i * STAGE;
         mbar_expect_tx(&full[i], STAGE);
-        tma_load_2d_hint(a, mw0, (kb0 + i) * TILE_K, tm * TILE_M, &full[i], pol);
+        tma_load_2d_hint(a, mw0, (kb0 + i) * TILE_K, tm * F_TILE, &full[i], pol);
+        if (MIX) tma_load_2d_hint(a + A_BYTES / 2, &p.map_w[1], (kb0 + i) * TILE_K, tm * F_TILE, &full[i], pol);
         if (PAIR) tma_load_2d_hint(a + A_BYTES, &p.map_w[1], (kb0 + i) * TILE_K, tm * TILE_M, &full[i], pol);
       }
     __syncwarp();
@@ -264,7 +274,8 @@ __global__ void __launch_bounds__(fused_threads(NT, EPI)) gemm_fused_kernel(cons
       if (elect_one()) {
         unsigned char *a = tiles + st * STAGE;
         mbar_expect_tx(&full[st], STAGE);
-        tma_load_2d_hint(a, mw0, (kb0 + i) * TILE_K, tm * TILE_M, &full[st], pol);
+        tma_load_2d_hint(a, mw0, (kb0 + i) * TILE_K, tm * F_TILE, &full[st], pol);
+        if (MIX) tma_load_2d_hint(a + A_BYTES / 2, &p.map_w[1], (kb0 + i) * TILE_K, tm * F_TILE, &full[st], pol);
         if (PAIR) tma_load_2d_hint(a + A_BYTES, &p.map_w[1], (kb0 + i) * TILE_K, tm * TILE_M, &full[st], pol);
         tma_load_2d(a + A_TILES * A_BYTES, &p.map_x, (kb0 + i) * TILE_K, 0, &full[st]);
       }
@@ -503,6 +514,22 @@ __global__ void __launch_bounds__(fused_threads(NT, EPI)) gemm_fused_kernel(cons
           }
         }
       }
+    } else if (MIX) {
+      // red[row] = 64 gate values, then the 64 up values of the same features: a warp takes a row, a lane two features
+      const int o2 = tm * F_TILE + 2 * lane;
+      if (good && o2 < p.O[0])
+#pragma unroll 4
+        for (int r = warp; r < nrow; r += 4) {
+          const float sc = inv_s[c0 + r];
+          const float2 g = *(const float2 *)&red[r * TILE_M + 2 * lane], u = *(const float2 *)&red[r * TILE_M + TILE_M / 2 + 2 * lane];
+          const float g0 = g.x * sc, g1 = g.y * sc, a0 = (g0 / (1.0f + expf(-g0))) * (u.x * sc), a1 = (g1 / (1.0f + expf(-g1))) * (u.y * sc);
+          bf16 *dst = p.act + (size_t)(c0 + r) * p.O[0] + o2;
+          if (p.act_vec) *(__nv_bfloat162 *)dst = __floats2bfloat162_rn(a0, a1);
+          else {
+            dst[0] = __float2bfloat16_rn(a0);
+            if (o2 + 1 < p.O[0]) dst[1] = __float2bfloat16_rn(a1);
+          }
+        }
     } else if (EPI == EPI_SWIGLU) {
       for (int r = r0; r < r1; r++) {
         const int row = c0 + r;
@@ -876,7 +903,7 @@ constexpr int NUM_SMS = 148;
 constexpr int SMEM_ONE = 200 * 1024;      // ring budget with one CTA per SM
 constexpr int SMEM_TWO = 104 * 1024;      // ring budget that lets two CTAs share an SM
 
-struct Plan { int nt, tiles, S, Sk, stages, smem, ctrl_off, KB, chunk; bool pair, duo; };
+struct Plan { int nt, tiles, S, Sk, stages, smem, ctrl_off, KB, chunk; bool pair, duo, mix; };
 
 // K slices per feature tile.  An SM streams at a capped rate whether one or two CTAs feed it, so the time
 // of a launch goes with (CTAs on the busiest SM) x (k-blocks per CTA + a fixed cost per CTA); two CTAs per SM
@@ -896,8 +923,13 @@ Plan make_plan(FusedEpi epi, const FusedGemmArgs &a, bool force_two = false, boo
   pl.tiles = fused_gemm_tiles(epi, a);
   // gate/up below 256 rows: gate and up tile in ONE CTA (256 rows: the pair kernel without K split)
   pl.pair = epi == EPI_SWIGLU && pl.nt <= 128;
+  // Where pairs of whole tiles would be split in two over K (89 to 148 of them), tiles of 64 + 64 features give as many CTAs
+  // without a cluster.  With fewer pairs (more K slices) the halved tiles alone would leave SMs idle; with more, one slice per
+  // pair already fills the chip and reads the activations half as often (70B shapes: 224 pairs).
+  pl.mix = pl.pair && a.split == 0 && a.stages == 0 && (g_target_ctas + pl.tiles / 2) / pl.tiles == 2;
+  if (pl.mix) { pl.pair = false; pl.tiles = (a.O[0] + TILE_M / 2 - 1) / (TILE_M / 2); }
   const int stage = (pl.pair ? 2 : 1) * A_BYTES + (duo ? pl.nt / 2 : pl.nt) * TILE_K * 2;
-  const int wmul = (epi == EPI_SWIGLU && !pl.pair) ? 2 : 1;   // cluster members per K slice
+  const int wmul = (epi == EPI_SWIGLU && !pl.pair && !pl.mix) ? 2 : 1;   // cluster members per K slice
   const int smax = MAX_CLUSTER / (duo ? 2 : wmul);
   const bool wide = duo || SMEM_TWO / stage < (pl.pair ? 2 : 3);     // 256-row tiles: the ring of one CTA takes the SM
   const bool one_per_sm = wide && !force_two;
@@ -923,6 +955,7 @@ Plan make_plan(FusedEpi epi, const FusedGemmArgs &a, bool force_two = false, boo
       Sk = up;
     }
   }
+  if (pl.mix) Sk = 1;
   if (a.split > 0) Sk = std::max(1, std::min(std::min(a.split, smax), pl.KB));
   pl.Sk = Sk;
   pl.S = Sk * wmul;
@@ -949,10 +982,10 @@ Plan make_plan(FusedEpi epi, const FusedGemmArgs &a, bool force_two = false, boo
   return pl;
 }
 
-template <int NT, int EPI, bool PAIR = false, bool DUO = false>
+template <int NT, int EPI, bool PAIR = false, bool DUO = false, bool MIX = false>
 int launch_inst(const FusedParams &p, const Plan &pl, bool pdl, cudaStream_t s) {
   static SmemLimit limit;
-  if (!limit.ensure(gemm_fused_kernel<NT, EPI, PAIR, DUO>, pl.smem)) return -6;
+  if (!limit.ensure(gemm_fused_kernel<NT, EPI, PAIR, DUO, MIX>, pl.smem)) return -6;
   if (pl.S * (DUO ? 2 : 1) > 8 || (DUO && (pl.tiles & 1))) return -1;   // portable cluster sizes only; pairs need an even tile count
   if (!launch_allowed()) return 0;
   cudaLaunchConfig_t cfg = {};
@@ -974,7 +1007,7 @@ int launch_inst(const FusedParams &p, const Plan &pl, bool pdl, cudaStream_t s) 
   }
   cfg.attrs = at;
   cfg.numAttrs = na;
-  return cudaLaunchKernelEx(&cfg, gemm_fused_kernel<NT, EPI, PAIR, DUO>, p) == cudaSuccess ? 0 : -6;
+  return cudaLaunchKernelEx(&cfg, gemm_fused_kernel<NT, EPI, PAIR, DUO, MIX>, p) == cudaSuccess ? 0 : -6;
 }
 
 // clusters of the plan's shape that can be resident at once (0: unknown)
@@ -1015,6 +1048,13 @@ int launch_epi(const FusedParams &p, const Plan &pl, bool pdl, cudaStream_t s) {
     case 64: return launch_inst<64, EPI>(p, pl, pdl, s);
     case 128: return launch_inst<128, EPI>(p, pl, pdl, s);
     default: return launch_inst<256, EPI>(p, pl, pdl, s);
+  }
+}
+int launch_swiglu_mix(const FusedParams &p, const Plan &pl, bool pdl, cudaStream_t s) {
+  switch (pl.nt) {
+    case 16: return launch_inst<16, EPI_SWIGLU, false, false, true>(p, pl, pdl, s);
+    case 64: return launch_inst<64, EPI_SWIGLU, false, false, true>(p, pl, pdl, s);
+    default: return launch_inst<128, EPI_SWIGLU, false, false, true>(p, pl, pdl, s);
   }
 }
 int launch_swiglu_pair(const FusedParams &p, const Plan &pl, bool pdl, cudaStream_t s) {
@@ -1071,7 +1111,7 @@ int fused_gemm_launch(TmaMaps *g, FusedEpi epi, const FusedGemmArgs &a, cudaStre
   FusedParams p;
   memset(&p, 0, sizeof p);
   for (int j = 0; j < a.nw; j++) {
-    const CUtensorMap *mw = tma_maps_get(g, a.w[j], a.O[j], a.I, TILE_M);
+    const CUtensorMap *mw = tma_maps_get(g, a.w[j], a.O[j], a.I, pl.mix ? TILE_M / 2 : TILE_M);
     if (!mw) return -6;
     p.map_w[j] = *mw;
     p.O[j] = a.O[j];
@@ -1087,7 +1127,7 @@ int fused_gemm_launch(TmaMaps *g, FusedEpi epi, const FusedGemmArgs &a, cudaStre
   p.xres = a.xres; p.gain = a.gain; p.hb = a.hb; p.ssq_out = a.ssq_out; p.taps = a.tap_mask ? a.taps : nullptr;
   p.tap_mask = a.taps ? a.tap_mask : 0; p.resid_add = a.resid_add;
   p.cs = a.cs; p.m = a.m; p.q = a.q; p.pool = a.pool; p.pm = a.pm; p.H = a.H; p.G = a.G; p.hd = a.hd;
-  p.act = a.act;
+  p.act = a.act; p.act_vec = (a.O[0] & 1) == 0 && ((uintptr_t)a.act & 3) == 0;
   p.best_val = a.best_val; p.best_idx = a.best_idx; p.best_ld = a.best_ld;
   p.topk = a.topk; p.cand_val = a.cand_val; p.cand_max = a.cand_max; p.cand_sum = a.cand_sum; p.cand_idx = a.cand_idx;
   p.cand_ld = a.cand_ld; p.want_rows = a.want_rows; p.n_want = a.n_want;
@@ -1145,7 +1185,7 @@ int fused_gemm_launch(TmaMaps *g, FusedEpi epi, const FusedGemmArgs &a, cudaStre
     case EPI_F32: return launch_epi<EPI_F32>(p, pl, a.pdl, s);
     case EPI_RESID: return launch_epi<EPI_RESID>(p, pl, a.pdl, s);
     case EPI_QKV: return launch_epi<EPI_QKV>(p, pl, a.pdl, s);
-    case EPI_SWIGLU: return pl.pair ? launch_swiglu_pair(p, pl, a.pdl, s) : launch_epi<EPI_SWIGLU>(p, pl, a.pdl, s);
+    case EPI_SWIGLU: return pl.mix ? launch_swiglu_mix(p, pl, a.pdl, s) : pl.pair ? launch_swiglu_pair(p, pl, a.pdl, s) : launch_epi<EPI_SWIGLU>(p, pl, a.pdl, s);
     case EPI_TOPK: return launch_epi<EPI_TOPK>(p, pl, a.pdl, s);
     default: return launch_epi<EPI_ARGMAX>(p, pl, a.pdl, s);
   }
