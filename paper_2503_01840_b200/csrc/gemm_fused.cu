@@ -154,11 +154,14 @@ __device__ __forceinline__ void arrived(const float4 (&v)[N]) {
 // per weight byte drops from 3 x to 2 x, which is what bounds the loop at this width.  The cluster is (2, S): x = the
 // pair, y = the K slices; the reduction runs over the members with the same x.
 // Threads per CTA: 128; the 256-row tiles run 256, so that two threads share a feature when the accumulator is dumped and twice
-// as many warps take rows afterwards (the epilogue of a 256-row tile is as long as its main loop).
-constexpr int fused_threads(int nt, int epi) { return (nt == 256 && (epi == EPI_F32 || epi == EPI_RESID || epi == EPI_QKV)) ? 256 : 128; }
+// as many warps take rows afterwards (the epilogue of a 256-row tile is as long as its main loop).  So do the top-K and the gate/up
+// epilogues from 64-row tiles on, whose arithmetic per value (selection, exponential and division) is long enough to share:
+// top-K at 40 rows 70 -> 66 us, gate/up at 60 rows 41.5 -> 40.7.  They need two CTAs per SM as the others do, hence the bound on
+// registers (without it top-K at 40 rows takes 82 us, the 70B gate/up 208 us instead of 147).
+constexpr int fused_threads(int nt, int epi) { return ((epi == EPI_TOPK || epi == EPI_SWIGLU) && nt >= 64) || (nt == 256 && (epi == EPI_F32 || epi == EPI_RESID || epi == EPI_QKV)) ? 256 : 128; }
 
 template <int NT, int EPI, bool PAIR = false, bool DUO = false, bool MIX = false>
-__global__ void __launch_bounds__(fused_threads(NT, EPI)) gemm_fused_kernel(const __grid_constant__ FusedParams p) {
+__global__ void __launch_bounds__(fused_threads(NT, EPI), EPI == EPI_TOPK || EPI == EPI_SWIGLU ? 2 : 1) gemm_fused_kernel(const __grid_constant__ FusedParams p) {
   constexpr int THREADS = fused_threads(NT, EPI), NH = THREADS / 128;
   static_assert((EPI == EPI_SWIGLU) == (PAIR || MIX), "two weight tiles per CTA exist for the gate/up epilogue only");
   static_assert(!MIX || (EPI == EPI_SWIGLU && !PAIR && !DUO), "tiles of 64 gate and 64 up features exist for the gate/up epilogue only");
@@ -558,11 +561,11 @@ __global__ void __launch_bounds__(fused_threads(NT, EPI)) gemm_fused_kernel(cons
       // red[row] = 64 gate values, then the 64 up values of the same features: a warp takes four rows at a time, a lane two features
       const int o2 = tm * F_TILE + 2 * lane;
       if (good)
-        for (int rb = warp; rb < nrow; rb += 16) {
+        for (int rb = warp; rb < nrow; rb += 4 * NW) {
           float2 g[4], u[4];
 #pragma unroll
           for (int j = 0; j < 4; j++) {
-            const int r = min(rb + 4 * j, nrow - 1);
+            const int r = min(rb + NW * j, nrow - 1);
             const float sc = inv_s[c0 + r];
             g[j] = *(const float2 *)&red[r * TILE_M + 2 * lane]; u[j] = *(const float2 *)&red[r * TILE_M + TILE_M / 2 + 2 * lane];
             g[j].x *= sc; g[j].y *= sc; u[j].x *= sc; u[j].y *= sc;
@@ -571,7 +574,7 @@ __global__ void __launch_bounds__(fused_threads(NT, EPI)) gemm_fused_kernel(cons
           for (int j = 0; j < 4; j++) { g[j].x = silu_mul(g[j].x, u[j].x); g[j].y = silu_mul(g[j].y, u[j].y); }
 #pragma unroll
           for (int j = 0; j < 4; j++) {
-            const int r = rb + 4 * j;
+            const int r = rb + NW * j;
             bf16 *dst = p.act + (size_t)(c0 + r) * p.O[0] + o2;
             if (r >= nrow || o2 >= p.O[0]) continue;
             if (p.vec) *(__nv_bfloat162 *)dst = __floats2bfloat162_rn(g[j].x, g[j].y);
@@ -595,94 +598,122 @@ __global__ void __launch_bounds__(fused_threads(NT, EPI)) gemm_fused_kernel(cons
       }
       unsigned char *want = (unsigned char *)wpart;                // [256]: rows that need candidates (a list made by an earlier kernel)
       if (p.want_rows) {
-        for (int t = threadIdx.x; t < 256; t += 128) want[t] = 0;
+        for (int t = threadIdx.x; t < 256; t += THREADS) want[t] = 0;
         __syncthreads();
-        for (int t = threadIdx.x; t < p.n_want; t += 128) { const int wr = p.want_rows[t]; if (wr >= 0 && wr < 256) want[wr] = 1; }
+        for (int t = threadIdx.x; t < p.n_want; t += THREADS) { const int wr = p.want_rows[t]; if (wr >= 0 && wr < 256) want[wr] = 1; }
         __syncthreads();
       }
       if (good && p.out_f32 && o < p.O[0])
-        for (int r = r0; r < r1; r++) p.out_f32[(size_t)(c0 + r) * p.ldo + o] = src[(r - r0) * TILE_M + f] * inv_s[c0 + r];
-      // One warp takes four rows at a time: four independent dependency chains (a CTA has only four warps, nothing else hides
-      // the latencies).  Lane l holds features l, l+32, l+64, l+96 of the tile as order-preserving keys.  The K-th largest of the
-      // 32 lane maxima bounds the tile's K-th best value from below, and few values reach it (K to about 1.5 K): those are
-      // collected and ranked by counting, so that the K results leave in one store.  Launch with K = 10, 32000 x 4096, against
-      // picking the best K times by a warp-wide reduction: 49.3 -> 44.9 us at 10 rows, 74.5 -> 59 us at 40 rows.
+        for (int r = r0 + hw; r < r1; r += NH) p.out_f32[(size_t)(c0 + r) * p.ldo + o] = src[(r - r0) * TILE_M + f] * inv_s[c0 + r];
+      // One warp takes four rows at a time: four independent dependency chains in straight-line code (a CTA has only four warps,
+      // nothing else hides the latencies).  Lane l holds features l, l+32, l+64, l+96 of the tile as order-preserving keys.  The
+      // K-th largest of the 32 lane maxima bounds the tile's K-th best value from below, and few values reach it (K to about
+      // 1.5 K): those are collected and ranked by counting, so that the K results leave in one store.  In the
+      // replayed step, 32000 x 4096, against picking the best K times by a warp-wide reduction: K = 10 49.3 -> 44.4 us at 10 rows,
+      // 76.7 -> 54.7 at 40; K = 1 60.0 -> 50.5 at 64 rows (one exchange for the four rows' sums).
       const int K = p.topk;
       unsigned *sk = (unsigned *)(sumb + (S > 1 ? per : 0) * TILE_M) + warp * 4 * 96;   // per row of the batch: [32] lane maxima, [32] (key, id)
-      for (int rb = r0 + warp; rb < r1; rb += 16) {
+      const int nv = min(4, max(0, (p.O[0] - tm * TILE_M - lane + 31) / 32));          // features of this lane that exist
+      for (int rb = r0 + warp; rb < r1; rb += 4 * NW) {
         unsigned key[4][4], lm[4];
-        int nv[4];                               // features of this lane that exist
         bool act[4];
-        size_t slot[4];
+        float mx[4], sum[4];
 #pragma unroll
         for (int q = 0; q < 4; q++) {
-          const int r = rb + 4 * q, row = c0 + r;
+          const int r = rb + NW * q, row = c0 + r;
           const int rs = r < r1 ? r : r0;                                  // a row that exists (results are masked)
           act[q] = good && r < r1 && (!p.want_rows || want[row < 256 ? row : 255]);     // uniform over the warp
-          slot[q] = (size_t)row * p.cand_ld * K + (size_t)blockIdx.x * K;
           const float sc = inv_s[c0 + rs];
           float v[4];
-          float mx = -INFINITY;
-          nv[q] = min(4, max(0, (p.O[0] - tm * TILE_M - lane + 31) / 32));
+#pragma unroll
+          for (int j2 = 0; j2 < 4; j2++) v[j2] = j2 < nv ? src[(rs - r0) * TILE_M + lane + 32 * j2] * sc : -INFINITY;
+          mx[q] = key_value(__reduce_max_sync(0xffffffffu, ordered_key(fmaxf(fmaxf(v[0], v[1]), fmaxf(v[2], v[3])))));   // NaN: ignored
+          sum[q] = 0.0f;
           lm[q] = 0u;
 #pragma unroll
           for (int j2 = 0; j2 < 4; j2++) {
-            v[j2] = j2 < nv[q] ? src[(rs - r0) * TILE_M + lane + 32 * j2] * sc : -INFINITY;
             key[q][j2] = ordered_key(v[j2]);
-            mx = fmaxf(mx, v[j2]);
-            if (j2 < nv[q]) lm[q] = max(lm[q], key[q][j2]);
+            if (j2 < nv) { lm[q] = max(lm[q], key[q][j2]); sum[q] += expf(v[j2] - mx[q]); }
           }
-          for (int off = 16; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-          float sum = 0.0f;
-#pragma unroll
-          for (int j2 = 0; j2 < 4; j2++) sum += j2 < nv[q] ? expf(v[j2] - mx) : 0.0f;
-          for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+        }
+        // sums over the lanes, the four rows in one exchange: afterwards lanes 8 q .. hold row q
+        {
+          const bool u1 = lane & 16, u2 = lane & 8;
+          const float a = (u1 ? sum[2] : sum[0]) + __shfl_xor_sync(0xffffffffu, u1 ? sum[0] : sum[2], 16);
+          const float b = (u1 ? sum[3] : sum[1]) + __shfl_xor_sync(0xffffffffu, u1 ? sum[1] : sum[3], 16);
+          float t = (u2 ? b : a) + __shfl_xor_sync(0xffffffffu, u2 ? a : b, 8);
+          for (int off = 4; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
           // row-major: all candidates / statistics of a row are contiguous, so that the merge fetches a row in one go
-          if (act[q] && lane == 0) { p.cand_max[(size_t)row * p.cand_ld + blockIdx.x] = mx; p.cand_sum[(size_t)row * p.cand_ld + blockIdx.x] = sum; }
+          const int q = lane >> 3;
+          if ((lane & 7) == 0 && (q == 0 ? act[0] : q == 1 ? act[1] : q == 2 ? act[2] : act[3])) {
+            const size_t at = (size_t)(c0 + rb + NW * q) * p.cand_ld + blockIdx.x;
+            p.cand_max[at] = q == 0 ? mx[0] : q == 1 ? mx[1] : q == 2 ? mx[2] : mx[3];
+            p.cand_sum[at] = t;
+          }
+        }
+        const size_t slot0 = ((size_t)(c0 + rb) * p.cand_ld + blockIdx.x) * K, slot4 = (size_t)NW * p.cand_ld * K;     // slot of row q: slot0 + q slot4
+        if (K == 1) {                            // the maximum itself
+#pragma unroll
+          for (int q = 0; q < 4; q++) {
+            const unsigned m = __reduce_max_sync(0xffffffffu, lm[q]);
+            int id = -1;
+#pragma unroll
+            for (int j2 = 3; j2 >= 0; j2--)
+              if (j2 < nv && key[q][j2] == m) id = tm * TILE_M + lane + 32 * j2;
+            const unsigned w = __reduce_min_sync(0xffffffffu, (unsigned)id);
+            if (act[q] && lane == 0) { p.cand_val[slot0 + q * slot4] = key_value(m); p.cand_idx[slot0 + q * slot4] = (int)w; }
+          }
+          continue;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
           sk[q * 96 + lane] = lm[q];
+          *(uint2 *)&sk[q * 96 + 32 + 2 * lane] = make_uint2(0u, 0x7fffffffu);     // an entry that ranks behind every value
         }
         __syncwarp();
-        // place of the lane's maximum among the lanes' (ties: lower lane first; lanes without a feature are the highest lanes, so
-        // they come last; with fewer than K lanes that have one, each of them has one value and all are candidates)
-        int place[4] = {0, 0, 0, 0};
+        int above[4] = {0, 0, 0, 0};             // lane maxima larger than the lane's own
 #pragma unroll
         for (int i = 0; i < 8; i++)
 #pragma unroll
           for (int q = 0; q < 4; q++) {
             const uint4 w = *(const uint4 *)&sk[q * 96 + 4 * i];
-            place[q] += (w.x > lm[q] || (w.x == lm[q] && 4 * i < lane)) + (w.y > lm[q] || (w.y == lm[q] && 4 * i + 1 < lane)) +
-                        (w.z > lm[q] || (w.z == lm[q] && 4 * i + 2 < lane)) + (w.w > lm[q] || (w.w == lm[q] && 4 * i + 3 < lane));
+            above[q] += (w.x > lm[q]) + (w.y > lm[q]) + (w.z > lm[q]) + (w.w > lm[q]);
           }
         int cnt[4];
 #pragma unroll
         for (int q = 0; q < 4; q++) {
-          const unsigned bound = __reduce_min_sync(0xffffffffu, place[q] < K && nv[q] > 0 ? lm[q] : 0xffffffffu);
+          // (with fewer than K lanes that have a feature each of them has one, and all are candidates)
+          const unsigned bound = __reduce_min_sync(0xffffffffu, above[q] < K && nv > 0 ? lm[q] : 0xffffffffu);
           cnt[q] = 0;
-          unsigned *cand = sk + q * 96 + 32;
 #pragma unroll
           for (int j2 = 0; j2 < 4; j2++) {
-            const bool in = j2 < nv[q] && key[q][j2] >= bound;
+            const bool in = j2 < nv && key[q][j2] >= bound;
             const unsigned m = __ballot_sync(0xffffffffu, in);
             const int at = cnt[q] + __popc(m & ((1u << lane) - 1u));
-            if (in && at < 32) { cand[2 * at] = key[q][j2]; cand[2 * at + 1] = (unsigned)(tm * TILE_M + lane + 32 * j2); }
+            if (in && at < 32) *(uint2 *)&sk[q * 96 + 32 + 2 * at] = make_uint2(key[q][j2], (unsigned)(tm * TILE_M + lane + 32 * j2));
             cnt[q] += __popc(m);
           }
         }
         __syncwarp();
+        const int most = min(32, max(max(cnt[0], cnt[1]), max(cnt[2], cnt[3])));
+        uint2 me[4];
+        int rank[4] = {0, 0, 0, 0};
+#pragma unroll
+        for (int q = 0; q < 4; q++) me[q] = *(const uint2 *)&sk[q * 96 + 32 + 2 * lane];
+#pragma unroll 4
+        for (int i = 0; i < most; i++)
+#pragma unroll
+          for (int q = 0; q < 4; q++) {
+            const uint2 w = *(const uint2 *)&sk[q * 96 + 32 + 2 * i];
+            rank[q] += w.x > me[q].x || (w.x == me[q].x && w.y < me[q].y);
+          }
 #pragma unroll
         for (int q = 0; q < 4; q++) {
           if (!act[q]) continue;                 // uniform over the warp
+          const size_t slot = slot0 + q * slot4;
           if (cnt[q] <= 32) {
-            const uint2 *cand = (const uint2 *)(sk + q * 96 + 32);
-            const uint2 me = cand[min(lane, max(cnt[q], 1) - 1)];
-            int rank = 0;
-#pragma unroll 4
-            for (int i = 0; i < cnt[q]; i++) {
-              const uint2 w = cand[i];
-              rank += w.x > me.x || (w.x == me.x && w.y < me.y);
-            }
-            if (lane < cnt[q] && rank < K) { p.cand_val[slot[q] + rank] = key_value(me.x); p.cand_idx[slot[q] + rank] = (int)me.y; }
-            if (lane >= cnt[q] && lane < K) { p.cand_val[slot[q] + lane] = 0.0f; p.cand_idx[slot[q] + lane] = -1; }       // tile exhausted
+            if (lane < cnt[q] && rank[q] < K) { p.cand_val[slot + rank[q]] = key_value(me[q].x); p.cand_idx[slot + rank[q]] = (int)me[q].y; }
+            if (lane >= cnt[q] && lane < K) { p.cand_val[slot + lane] = 0.0f; p.cand_idx[slot + lane] = -1; }       // tile exhausted
           } else {                               // many equal values: the best of what is left, K times
             unsigned taken = 0u;
             for (int c = 0; c < K; c++) {
@@ -690,14 +721,14 @@ __global__ void __launch_bounds__(fused_threads(NT, EPI)) gemm_fused_kernel(cons
               int bi = -1;
 #pragma unroll
               for (int j2 = 0; j2 < 4; j2++) {
-                const bool better = j2 < nv[q] && !(taken >> j2 & 1u) && (bi < 0 || key[q][j2] > bk);      // equal: the lower feature stays
+                const bool better = j2 < nv && !(taken >> j2 & 1u) && (bi < 0 || key[q][j2] > bk);      // equal: the lower feature stays
                 bk = better ? key[q][j2] : bk;
                 bi = better ? tm * TILE_M + lane + 32 * j2 : bi;
               }
               unsigned wk;
               const int wi = warp_best(bk, bi, &wk);
               if (wi >= 0 && bi == wi) taken |= 1u << ((wi - tm * TILE_M) >> 5);
-              if (lane == 0) { p.cand_val[slot[q] + c] = wi < 0 ? 0.0f : key_value(wk); p.cand_idx[slot[q] + c] = wi; }
+              if (lane == 0) { p.cand_val[slot + c] = wi < 0 ? 0.0f : key_value(wk); p.cand_idx[slot + c] = wi; }
             }
           }
         }
@@ -1002,7 +1033,7 @@ __global__ void __launch_bounds__(PAIR_THREADS) gemm_swiglu_pair_kernel(const __
 // ---------------------------------------------------------------------------------------------- host side
 int pick_nt(int rows) { return rows <= 16 ? 16 : rows <= 64 ? 64 : rows <= 128 ? 128 : 256; }
 
-constexpr int TOPK_BYTES = 4 * 4 * 96 * 4;   // EPI_TOPK: selection scratch of four warps
+constexpr int TOPK_BYTES = 8 * 4 * 96 * 4;   // EPI_TOPK: selection scratch of up to eight warps
 constexpr int NUM_SMS = 148;
 constexpr int SMEM_ONE = 200 * 1024;      // ring budget with one CTA per SM
 constexpr int SMEM_TWO = 104 * 1024;      // ring budget that lets two CTAs share an SM
