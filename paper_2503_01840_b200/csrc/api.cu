@@ -614,7 +614,7 @@ template <typename T> struct Sched {
         for (int b = 0; b < c->B; b++) hint = std::max(hint, c->n_upper[b]);
       tick(launch_attn_fast((const bf16 *)c->q, pool, pm, c->meta, tail_len, (bf16 *)c->ao, rows, c->H, c->G, c->hd,
                             c->cur_rps, hint, c->attn_scratch, s, !(c->cfg.flags & SPEC_FLAG_NO_TMA_ATTN), c->status,
-                            c->st.order, c->B, next_stamp(SPEC_PROF_ATTN)));
+                            c->st.order, c->B, next_stamp(SPEC_PROF_ATTN), c->ctx_hint < 0));
     } else {
       launch_attn_ref<T>((const T *)c->q, pool, pm, c->meta, tail_len, (T *)c->ao, rows, c->H, c->G, c->hd,
                          c->cfg.max_ctx + tail_len, s);

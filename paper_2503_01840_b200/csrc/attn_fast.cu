@@ -85,6 +85,7 @@ struct AttnParams {
   PageMap pm;
   RowMeta m;
   int tail_len, rows, H, G, rps, nsplit;
+  int ctx_ready;    // the context's K/V were complete before the previous kernel of the stream started: read before the wait
   bf16 *out;
   float *part_o;    // [nsplit][rows*H][hd]
   float *part_ml;   // [nsplit][rows*H][2]
@@ -343,12 +344,15 @@ __device__ __forceinline__ void tile_pages(int (&pg)[4], const int32_t *tbl, int
   for (int j = 0; j < 4; j++) pg[j] = (j < ppt && first + j < pages_per_seq) ? tbl[first + j] : -1;
 }
 
+// What these kernels do before the wait for the QKV launch: the row metadata, the page table and the key tiles that hold nothing
+// but context (launch_attn_fast says when that is allowed).  After the wait only the queries and the tail tiles are left; the chain
+// metadata -> page -> K/V tile, and Q behind a look at its row's sequence, used to take 4.2 us of it.  Replayed step, 8B shapes
+// (with the merge of the splits): verify pass of 60 rows 14.9 -> 13.5 us, draft pass 8.9 -> 7.0; four sequences of 60 rows 28.8 ->
+// 26.3; 13B shapes (multi-head attention) 13.4 -> 11.5.
 template <int HD, int STAGES>
 __global__ void __launch_bounds__(288) attn_tma_kernel(const __grid_constant__ CUtensorMap map_k,
                                                        const __grid_constant__ CUtensorMap map_v, AttnParams p, int32_t *status) {
   pdl_trigger();   // the next kernel may start staging its weights; it still waits for this grid to complete
-  pdl_wait();
-  KernelStamp stamp_guard(p.stamp);
   constexpr int ROWB = HD * 2, CPR = HD / 8;
   constexpr int NKS = HD / 16;
   constexpr int TILEB = KT * ROWB;                     // bytes of one K (or V) tile
@@ -372,22 +376,31 @@ __global__ void __launch_bounds__(288) attn_tma_kernel(const __grid_constant__ C
     const int s = p.m.seq[row0 + i], cx = p.m.ctx[row0 + i];   // both loads in flight together
     if (s >= 0) { seq = s; ctx = cx; break; }
   }
-  const int nkeys = (seq >= 0) ? ctx + p.tail_len : 0;
+  const int nkeys = (seq >= 0) ? ctx + p.tail_len : 0, ctx_early = p.ctx_ready ? ctx : 0;
   const int ntiles = (nkeys + KT - 1) / KT;
   const int t_begin = (int)(((long long)blockIdx.y * ntiles) / p.nsplit);
   const int t_end = (int)(((long long)(blockIdx.y + 1) * ntiles) / p.nsplit);
 
+  KernelStamp stamp_guard(p.stamp, false);
   // consumer warps that own at least one query row; the others leave after the Q phase
   const int nactive = (M - m0 >= MT) ? 8 : (M - m0 + 15) / 16;
   // The producer warp sets up the barriers and starts the first K/V copies while the consumer warps fetch Q: the
   // page-table look-up and the copies overlap the Q round trip.  Named barrier 1 (288 threads): the producer only
   // arrives, the consumers wait there for the barrier set-up and for each other's part of the Q tile.
+  // rows owned by this thread: rA = quad row, rB = rA + 8 (within the warp's 16 rows)
+  const int mA = m0 + warp * 16 + (lane >> 2), mB = mA + 8;
+  uint64_t loA = 0, hiA = 0, loB = 0, hiB = 0;
+  bool vA = false, vB = false;
   if (warp < 8) {
+    if (mA < M) { int r = row0 + mA / grp; vA = p.m.seq[r] >= 0; loA = p.m.mask_lo[r]; hiA = p.m.mask_hi[r]; }
+    if (mB < M) { int r = row0 + mB / grp; vB = p.m.seq[r] >= 0; loB = p.m.mask_lo[r]; hiB = p.m.mask_hi[r]; }
+    pdl_wait();
+    if (p.stamp && threadIdx.x == 0) atomicMin(p.stamp, global_ns());
+    // (a padding row's scores are masked whatever its query holds)
     for (int id = threadIdx.x; id < MT * CPR; id += 256) {
       int lr = id / CPR, c = id % CPR, mrow = m0 + lr;
       bool v = mrow < M;
       int i = v ? mrow / grp : 0, hq = v ? mrow % grp : 0;
-      v = v && p.m.seq[row0 + i] >= 0;
       const bf16 *src = p.q + ((size_t)(row0 + i) * p.H + g * grp + hq) * HD + c * 8;
       cp_async16(smem_u32(sQ + swz<ROWB>(lr, c)), src, v);
     }
@@ -409,10 +422,12 @@ __global__ void __launch_bounds__(288) attn_tma_kernel(const __grid_constant__ C
       const int fallback = tbl[0];                     // keys past the last page are masked; they still need a valid source
       const int ppt = KT / ps;                         // pages per tile
       int cur[4], nxt[4] = {-1, -1, -1, -1};
+      bool waited = false;
       if (t_begin < t_end) tile_pages(cur, tbl, p.pm.pages_per_seq, t_begin, ps);
       for (int t = t_begin; t < t_end; t++) {
         const int i = t - t_begin, st = i % STAGES;
         if (t + 1 < t_end) tile_pages(nxt, tbl, p.pm.pages_per_seq, t + 1, ps);
+        if (!waited && (i == STAGES - 1 || (t + 1) * KT > ctx_early)) { pdl_wait(); waited = true; }
         if (i == STAGES - 1 && !mbar_wait_warp(q_bar, 0)) { if (status) set_status(status, ST_TIMEOUT, 400, blockIdx.z, t); break; }
         if (i >= STAGES && !mbar_wait_warp(&empty[st], (uint32_t)(((i / STAGES) - 1) & 1))) { if (status) set_status(status, ST_TIMEOUT, 401, blockIdx.z, t); break; }
         if (elect_one()) {
@@ -433,6 +448,7 @@ __global__ void __launch_bounds__(288) attn_tma_kernel(const __grid_constant__ C
         for (int pg = 0; pg < 4; pg++) cur[pg] = nxt[pg];
       }
     }
+    pdl_wait();
     return;
   }
 
@@ -451,14 +467,6 @@ __global__ void __launch_bounds__(288) attn_tma_kernel(const __grid_constant__ C
   auto koff = [&](int kr, int c) -> uint32_t {
     return (uint32_t)((kr >> psh) * psb + (c >> 3) * (ps * 128) + (kr & (ps - 1)) * 128 + (((c & 7) ^ (kr & 7)) << 4));
   };
-  const int tb = ctx;                                   // tail keys follow the context
-  (void)tb;
-  // rows owned by this thread: rA = quad row, rB = rA + 8 (within the warp's 16 rows)
-  const int mA = m0 + warp * 16 + (lane >> 2), mB = mA + 8;
-  uint64_t loA = 0, hiA = 0, loB = 0, hiB = 0;
-  bool vA = false, vB = false;
-  if (mA < M) { int r = row0 + mA / grp; vA = p.m.seq[r] >= 0; if (vA) { loA = p.m.mask_lo[r]; hiA = p.m.mask_hi[r]; } }
-  if (mB < M) { int r = row0 + mB / grp; vB = p.m.seq[r] >= 0; if (vB) { loB = p.m.mask_lo[r]; hiB = p.m.mask_hi[r]; } }
   clip_tail(loA, hiA, p.tail_len);
   clip_tail(loB, hiB, p.tail_len);
 
@@ -640,8 +648,7 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&v)[16
 __global__ void __launch_bounds__(UM_THREADS, 1) attn_umma_kernel(const __grid_constant__ CUtensorMap map_k,
                                                         const __grid_constant__ CUtensorMap map_v, AttnParams p, int32_t *status) {
   pdl_trigger();   // the next kernel may start staging its weights; it still waits for this grid to complete
-  pdl_wait();
-  KernelStamp stamp_guard(p.stamp);
+  KernelStamp stamp_guard(p.stamp, false);
   constexpr int HD = UM_HD;
   extern __shared__ __align__(1024) unsigned char sm[];
   unsigned char *sQ = sm;                                   // [2 halves][128 rows][128 B]
@@ -668,19 +675,55 @@ __global__ void __launch_bounds__(UM_THREADS, 1) attn_umma_kernel(const __grid_c
     int s = p.m.seq[row0 + i];
     if (s >= 0) { seq = s; ctx = p.m.ctx[row0 + i]; break; }
   }
-  const int nkeys = (seq >= 0) ? ctx + p.tail_len : 0;
+  const int nkeys = (seq >= 0) ? ctx + p.tail_len : 0, ctx_early = p.ctx_ready ? ctx : 0;
   const int ntiles = (nkeys + KT - 1) / KT;
   const int t_begin = (int)(((long long)blockIdx.y * ntiles) / p.nsplit);
   const int t_end = (int)(((long long)(blockIdx.y + 1) * ntiles) / p.nsplit);
   const int ntl = t_end - t_begin;
 
-  if (threadIdx.x == 0) {
+  if (warp == 8 && lane == 0) {
     for (int i = 0; i < UM_STAGES; i++) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
     mbar_init(&s_bar[0], 1);
     mbar_init(&s_bar[1], 1);
     for (int i = 0; i < 2; i++) { mbar_init(&p_bar[i], 128); mbar_init(&o_bar[i], 1); }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  // ---- producer state (warp 8): the copies of key tiles that hold nothing but context start here, before the wait for the
+  // previous kernel and before the block's first barrier
+  const int32_t *tbl = p.pm.table + (size_t)(seq >= 0 ? seq : 0) * p.pm.pages_per_seq;
+  const int ppt = KT / ps;                             // pages per tile
+  int cur[4] = {-1, -1, -1, -1}, nxt[4] = {-1, -1, -1, -1}, fallback = 0, i_load = 0;
+  auto load_tile = [&](int i) {                        // converged warp; page ids of tile i in cur
+    if (i + 1 < ntl) tile_pages(nxt, tbl, p.pm.pages_per_seq, t_begin + i + 1, ps);
+    if (elect_one()) {
+      const int st = i % UM_STAGES;
+      unsigned char *kb = ring + st * 2 * UM_TILE, *vb = kb + UM_TILE;
+      mbar_expect_tx(&full[st], 2 * UM_TILE);
+#pragma unroll
+      for (int pg = 0; pg < 4; pg++) {
+        if (pg >= ppt) break;
+        int page = cur[pg];
+        if (page < 0 || page >= p.pm.num_pages) page = fallback;
+        const int row = (page * p.G + g) * ps;
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+          tma_load_3d(kb + h * UM_HALF + pg * ps * 128, &map_k, 0, row, h, &full[st]);
+          tma_load_3d(vb + h * UM_HALF + pg * ps * 128, &map_v, 0, row, h, &full[st]);
+        }
+      }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int pg = 0; pg < 4; pg++) cur[pg] = nxt[pg];
+  };
+  if (warp == 8) {
+    __syncwarp();
+    if (seq >= 0 && ntl > 0) {
+      fallback = tbl[0];                               // keys past the last page are masked; they still need a valid source
+      tile_pages(cur, tbl, p.pm.pages_per_seq, t_begin, ps);
+      for (; i_load < ntl && i_load < UM_STAGES && (t_begin + i_load + 1) * KT <= ctx_early; i_load++) load_tile(i_load);
+    }
   }
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(UM_TMEM_COLS) : "memory");
@@ -701,6 +744,8 @@ __global__ void __launch_bounds__(UM_THREADS, 1) attn_umma_kernel(const __grid_c
     if (rvalid) { mlo = p.m.mask_lo[row0 + qi]; mhi = p.m.mask_hi[row0 + qi]; }
     else { mlo = ~0ull; mhi = ~0ull; }                         // a padding row attends every tail key (zeroed at the end)
     clip_tail(mlo, mhi, p.tail_len);
+    pdl_wait();
+    if (p.stamp && threadIdx.x == 0) atomicMin(p.stamp, global_ns());
     const uint4 *src = (const uint4 *)(p.q + ((size_t)(row0 + qi) * p.H + g * grp + qh) * HD);
 #pragma unroll
     for (int cc = 0; cc < 8; cc++) {                        // each of the row's two threads copies one half of it
@@ -718,42 +763,17 @@ __global__ void __launch_bounds__(UM_THREADS, 1) attn_umma_kernel(const __grid_c
 
   if (warp == 8) {
     // ================================================================ producer
-    if (seq >= 0) {     // the whole warp walks the loop, the elected lane issues the copies
-      const int32_t *tbl = p.pm.table + (size_t)seq * p.pm.pages_per_seq;
-      const int fallback = tbl[0];                     // keys past the last page are masked; they still need a valid source
-      const int ppt = KT / ps;                         // pages per tile
-      int cur[4], nxt[4] = {-1, -1, -1, -1};
-      if (ntl > 0) tile_pages(cur, tbl, p.pm.pages_per_seq, t_begin, ps);
-      for (int i = 0; i < ntl; i++) {
-        const int t = t_begin + i, st = i % UM_STAGES;
-        if (i + 1 < ntl) tile_pages(nxt, tbl, p.pm.pages_per_seq, t + 1, ps);
-        if (i >= UM_STAGES && !mbar_wait_warp(&empty[st], (uint32_t)(((i / UM_STAGES) - 1) & 1))) {
+    pdl_wait();
+    if (seq >= 0)       // the whole warp walks the loop, the elected lane issues the copies
+      for (; i_load < ntl; i_load++) {
+        if (i_load >= UM_STAGES && !mbar_wait_warp(&empty[i_load % UM_STAGES], (uint32_t)(((i_load / UM_STAGES) - 1) & 1))) {
           *abort_flag = 1;
-          if (status) set_status(status, ST_TIMEOUT, 420, blockIdx.z, t);
+          if (status) set_status(status, ST_TIMEOUT, 420, blockIdx.z, t_begin + i_load);
           break;
         }
         if (*abort_flag) break;
-        if (elect_one()) {
-          unsigned char *kb = ring + st * 2 * UM_TILE, *vb = kb + UM_TILE;
-          mbar_expect_tx(&full[st], 2 * UM_TILE);
-#pragma unroll
-          for (int pg = 0; pg < 4; pg++) {
-            if (pg >= ppt) break;
-            int page = cur[pg];
-            if (page < 0 || page >= p.pm.num_pages) page = fallback;
-            const int row = (page * p.G + g) * ps;
-#pragma unroll
-            for (int h = 0; h < 2; h++) {
-              tma_load_3d(kb + h * UM_HALF + pg * ps * 128, &map_k, 0, row, h, &full[st]);
-              tma_load_3d(vb + h * UM_HALF + pg * ps * 128, &map_v, 0, row, h, &full[st]);
-            }
-          }
-        }
-        __syncwarp();
-#pragma unroll
-        for (int pg = 0; pg < 4; pg++) cur[pg] = nxt[pg];
+        load_tile(i_load);
       }
-    }
   } else if (warp == 9) {
     // ================================================================ MMA issuer
     if (ntl > 0) {      // the whole warp walks the loop, the elected lane issues the MMAs and commits
@@ -952,12 +972,14 @@ __global__ void __launch_bounds__(UM_THREADS, 1) attn_umma_kernel(const __grid_c
 // group) and single-token decoding.  One 16-row tile would leave seven of eight row-parallel warps idle, so here
 // the four consumer warps share the rows and split the KEYS of every 64-key tile (16 keys each); each keeps its own
 // online-softmax state and the four states are merged through shared memory at the end.
+// At batch this kernel streams the cache, and a stage is only refilled when its tile has been consumed, so the time per tile
+// counts: context tiles take no masks, O is rescaled only when a maximum moved, 2^x is the special-function unit's; three CTAs
+// share an SM (hence the bound on registers).  64 chains of 256..2048 tokens: 81.7 -> 73.1 us a layer; 56 chains 68.9 -> 59.7.
 template <int HD, int STAGES>
-__global__ void __launch_bounds__(160) attn_tma_small_kernel(const __grid_constant__ CUtensorMap map_k,
+__global__ void __launch_bounds__(160, HD == 128 ? 3 : 1) attn_tma_small_kernel(const __grid_constant__ CUtensorMap map_k,
                                                              const __grid_constant__ CUtensorMap map_v, AttnParams p, int32_t *status) {
   pdl_trigger();   // the next kernel may start staging its weights; it still waits for this grid to complete
-  pdl_wait();
-  KernelStamp stamp_guard(p.stamp);
+  KernelStamp stamp_guard(p.stamp, false);
   constexpr int ROWB = HD * 2, CPR = HD / 8;
   constexpr int NKS = HD / 16;
   constexpr int TILEB = KT * ROWB;
@@ -979,20 +1001,62 @@ __global__ void __launch_bounds__(160) attn_tma_small_kernel(const __grid_consta
     int s = p.m.seq[row0 + i];
     if (s >= 0) { seq = s; ctx = p.m.ctx[row0 + i]; break; }
   }
-  const int nkeys = (seq >= 0) ? ctx + p.tail_len : 0;
+  const int nkeys = (seq >= 0) ? ctx + p.tail_len : 0, ctx_early = p.ctx_ready ? ctx : 0;
   const int ntiles = (nkeys + KT - 1) / KT;
   const int t_begin = (int)(((long long)blockIdx.y * ntiles) / p.nsplit);
   const int t_end = (int)(((long long)(blockIdx.y + 1) * ntiles) / p.nsplit);
 
-  if (threadIdx.x == 0) {
-    for (int i = 0; i < STAGES; i++) { mbar_init(&full[i], 1); mbar_init(&empty[i], NW); }
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  // ---- producer state (warp NW): the copies of key tiles that hold nothing but context start here, before the wait for the
+  // previous kernel and before the block's first barrier
+  const int32_t *tbl = p.pm.table + (size_t)(seq >= 0 ? seq : 0) * p.pm.pages_per_seq;
+  const int ppt = KT / ps;                             // pages per tile
+  int cur[4] = {-1, -1, -1, -1}, nxt[4] = {-1, -1, -1, -1}, fallback = 0, t_load = t_begin;
+  auto load_tile = [&](int t) {                        // converged warp; page ids of tile t in cur
+    const int st = (t - t_begin) % STAGES;
+    if (t + 1 < t_end) tile_pages(nxt, tbl, p.pm.pages_per_seq, t + 1, ps);
+    if (elect_one()) {
+      unsigned char *kb = sm + st * 2 * TILEB, *vb = kb + TILEB;
+      mbar_expect_tx(&full[st], 2 * TILEB);
+#pragma unroll
+      for (int pg = 0; pg < 4; pg++) {
+        if (pg >= ppt) break;
+        int page = cur[pg];
+        if (page < 0 || page >= p.pm.num_pages) page = fallback;
+        const int row = (page * p.G + g) * ps;
+        tma_load_3d(kb + pg * ps * ROWB, &map_k, 0, row, 0, &full[st]);
+        tma_load_3d(vb + pg * ps * ROWB, &map_v, 0, row, 0, &full[st]);
+      }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int pg = 0; pg < 4; pg++) cur[pg] = nxt[pg];
+  };
+  if (warp == NW) {
+    if (lane == 0) {
+      for (int i = 0; i < STAGES; i++) { mbar_init(&full[i], 1); mbar_init(&empty[i], NW); }
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncwarp();
+    if (seq >= 0 && t_begin < t_end) {
+      fallback = tbl[0];                               // keys past the last page are masked; they still need a valid source
+      tile_pages(cur, tbl, p.pm.pages_per_seq, t_begin, ps);
+      for (; t_load < t_end && t_load < t_begin + STAGES && (t_load + 1) * KT <= ctx_early; t_load++) load_tile(t_load);
+    }
   }
+  const int mA = lane >> 2, mB = mA + 8;
+  uint64_t loA = 0, hiA = 0, loB = 0, hiB = 0;
+  bool vA = false, vB = false;
+  if (warp < NW) {
+    if (mA < M) { int r = row0 + mA / grp; vA = p.m.seq[r] >= 0; loA = p.m.mask_lo[r]; hiA = p.m.mask_hi[r]; }
+    if (mB < M) { int r = row0 + mB / grp; vB = p.m.seq[r] >= 0; loB = p.m.mask_lo[r]; hiB = p.m.mask_hi[r]; }
+  }
+  pdl_wait();
+  if (p.stamp && threadIdx.x == 0) atomicMin(p.stamp, global_ns());
+  // (a padding row's scores are masked whatever its query holds)
   for (int id = threadIdx.x; id < 16 * CPR; id += 160) {
     int lr = id / CPR, c = id % CPR;
     bool v = lr < M;
     int i = v ? lr / grp : 0, hq = v ? lr % grp : 0;
-    v = v && p.m.seq[row0 + i] >= 0;
     const bf16 *src = p.q + ((size_t)(row0 + i) * p.H + g * grp + hq) * HD + c * 8;
     cp_async16(smem_u32(sQ + swz<ROWB>(lr, c)), src, v);
   }
@@ -1001,34 +1065,12 @@ __global__ void __launch_bounds__(160) attn_tma_small_kernel(const __grid_consta
   __syncthreads();
 
   if (warp == NW) {
-    if (seq >= 0) {     // the whole warp walks the loop, the elected lane issues the copies
-      const int32_t *tbl = p.pm.table + (size_t)seq * p.pm.pages_per_seq;
-      const int fallback = tbl[0];
-      const int ppt = KT / ps;
-      int cur[4], nxt[4] = {-1, -1, -1, -1};
-      if (t_begin < t_end) tile_pages(cur, tbl, p.pm.pages_per_seq, t_begin, ps);
-      for (int t = t_begin; t < t_end; t++) {
-        const int i = t - t_begin, st = i % STAGES;
-        if (t + 1 < t_end) tile_pages(nxt, tbl, p.pm.pages_per_seq, t + 1, ps);
-        if (i >= STAGES && !mbar_wait_warp(&empty[st], (uint32_t)(((i / STAGES) - 1) & 1))) { if (status) set_status(status, ST_TIMEOUT, 411, blockIdx.z, t); break; }
-        if (elect_one()) {
-          unsigned char *kb = sm + st * 2 * TILEB, *vb = kb + TILEB;
-          mbar_expect_tx(&full[st], 2 * TILEB);
-#pragma unroll
-          for (int pg = 0; pg < 4; pg++) {
-            if (pg >= ppt) break;
-            int page = cur[pg];
-            if (page < 0 || page >= p.pm.num_pages) page = fallback;
-            const int row = (page * p.G + g) * ps;
-            tma_load_3d(kb + pg * ps * ROWB, &map_k, 0, row, 0, &full[st]);
-            tma_load_3d(vb + pg * ps * ROWB, &map_v, 0, row, 0, &full[st]);
-          }
-        }
-        __syncwarp();
-#pragma unroll
-        for (int pg = 0; pg < 4; pg++) cur[pg] = nxt[pg];
+    if (seq >= 0)       // the whole warp walks the loop, the elected lane issues the copies
+      for (; t_load < t_end; t_load++) {
+        const int i = t_load - t_begin;
+        if (i >= STAGES && !mbar_wait_warp(&empty[i % STAGES], (uint32_t)(((i / STAGES) - 1) & 1))) { if (status) set_status(status, ST_TIMEOUT, 411, blockIdx.z, t_load); break; }
+        load_tile(t_load);
       }
-    }
   } else {
     // ---- consumers: all four warps hold the same 16-row Q tile
     uint32_t qf[NKS][4];
@@ -1041,11 +1083,8 @@ __global__ void __launch_bounds__(160) attn_tma_small_kernel(const __grid_consta
     auto koff = [&](int kr, int c) -> uint32_t {
       return (uint32_t)((kr >> psh) * psb + (c >> 3) * (ps * 128) + (kr & (ps - 1)) * 128 + (((c & 7) ^ (kr & 7)) << 4));
     };
-    const int mA = lane >> 2, mB = mA + 8;
-    uint64_t loA = 0, hiA = 0, loB = 0, hiB = 0;
-    bool vA = false, vB = false;
-    if (mA < M) { int r = row0 + mA / grp; vA = p.m.seq[r] >= 0; if (vA) { loA = p.m.mask_lo[r]; hiA = p.m.mask_hi[r]; } }
-    if (mB < M) { int r = row0 + mB / grp; vB = p.m.seq[r] >= 0; if (vB) { loB = p.m.mask_lo[r]; hiB = p.m.mask_hi[r]; } }
+    clip_tail(loA, hiA, p.tail_len);
+    clip_tail(loB, hiB, p.tail_len);
     float o[HD / 8][4];
 #pragma unroll
     for (int n = 0; n < HD / 8; n++) { o[n][0] = o[n][1] = o[n][2] = o[n][3] = 0.0f; }
@@ -1067,34 +1106,30 @@ __global__ void __launch_bounds__(160) attn_tma_small_kernel(const __grid_consta
         mma_bf16(s[0], qf[ks], b0, b1);
         mma_bf16(s[1], qf[ks], b2, b3);
       }
-      float tmA = -INFINITY, tmB = -INFINITY;
+      // Rows without a query run the loop like the others and are dropped at the end, so that context tiles need no mask.
+      if (t * KT + KT > ctx) {
+        // one allow word per row for the tile, shifted so that this lane's keys sit at bits 8 n + e
+        const uint32_t wA = (uint32_t)(tile_allow(loA, hiA, ctx, t * KT) >> (k0w + (lane & 3) * 2)), wB = (uint32_t)(tile_allow(loB, hiB, ctx, t * KT) >> (k0w + (lane & 3) * 2));
 #pragma unroll
-      for (int n = 0; n < 2; n++) {
+        for (int n = 0; n < 2; n++)
 #pragma unroll
-        for (int e = 0; e < 2; e++) {
-          int key = t * KT + k0w + n * 8 + (lane & 3) * 2 + e;
-          bool in_ctx = key < ctx;
-          int tt = key - ctx;
-          bool in_tail = !in_ctx && tt < p.tail_len;
-          bool okA = vA && (in_ctx || (in_tail && ((tt < 64 ? (loA >> tt) : (hiA >> (tt - 64))) & 1ull)));
-          bool okB = vB && (in_ctx || (in_tail && ((tt < 64 ? (loB >> tt) : (hiB >> (tt - 64))) & 1ull)));
-          s[n][e] = okA ? s[n][e] : -INFINITY;
-          s[n][2 + e] = okB ? s[n][2 + e] : -INFINITY;
-          tmA = fmaxf(tmA, s[n][e]);
-          tmB = fmaxf(tmB, s[n][2 + e]);
-        }
+          for (int e = 0; e < 2; e++) {
+            s[n][e] = (wA >> (8 * n + e)) & 1u ? s[n][e] : -INFINITY;
+            s[n][2 + e] = (wB >> (8 * n + e)) & 1u ? s[n][2 + e] : -INFINITY;
+          }
       }
+      float tmA = fmaxf(fmaxf(s[0][0], s[0][1]), fmaxf(s[1][0], s[1][1])), tmB = fmaxf(fmaxf(s[0][2], s[0][3]), fmaxf(s[1][2], s[1][3]));
       tmA = fmaxf(tmA, __shfl_xor_sync(0xffffffffu, tmA, 1)); tmA = fmaxf(tmA, __shfl_xor_sync(0xffffffffu, tmA, 2));
       tmB = fmaxf(tmB, __shfl_xor_sync(0xffffffffu, tmB, 1)); tmB = fmaxf(tmB, __shfl_xor_sync(0xffffffffu, tmB, 2));
       float nmA = fmaxf(mxA, tmA), nmB = fmaxf(mxB, tmB);
-      float fA = (nmA == -INFINITY) ? 1.0f : exp2f((mxA - nmA) * sc), fB = (nmB == -INFINITY) ? 1.0f : exp2f((mxB - nmB) * sc);
+      float fA = (nmA == -INFINITY) ? 1.0f : ex2_approx((mxA - nmA) * sc), fB = (nmB == -INFINITY) ? 1.0f : ex2_approx((mxB - nmB) * sc);
       float baseA = (nmA == -INFINITY) ? 0.0f : nmA, baseB = (nmB == -INFINITY) ? 0.0f : nmB;
       float rsA = 0.0f, rsB = 0.0f;
       uint32_t pf[4];
 #pragma unroll
       for (int n = 0; n < 2; n++) {
-        float p0 = exp2f((s[n][0] - baseA) * sc), p1 = exp2f((s[n][1] - baseA) * sc);
-        float p2 = exp2f((s[n][2] - baseB) * sc), p3 = exp2f((s[n][3] - baseB) * sc);
+        float p0 = ex2_approx((s[n][0] - baseA) * sc), p1 = ex2_approx((s[n][1] - baseA) * sc);
+        float p2 = ex2_approx((s[n][2] - baseB) * sc), p3 = ex2_approx((s[n][3] - baseB) * sc);
         rsA += p0 + p1; rsB += p2 + p3;
         pf[n * 2] = pack_bf16(p0, p1);
         pf[n * 2 + 1] = pack_bf16(p2, p3);
@@ -1103,8 +1138,10 @@ __global__ void __launch_bounds__(160) attn_tma_small_kernel(const __grid_consta
       rsB += __shfl_xor_sync(0xffffffffu, rsB, 1); rsB += __shfl_xor_sync(0xffffffffu, rsB, 2);
       lA = lA * fA + rsA; lB = lB * fB + rsB;
       mxA = nmA; mxB = nmB;
+      if (__any_sync(0xffffffffu, fA != 1.0f || fB != 1.0f)) {
 #pragma unroll
-      for (int n = 0; n < HD / 8; n++) { o[n][0] *= fA; o[n][1] *= fA; o[n][2] *= fB; o[n][3] *= fB; }
+        for (int n = 0; n < HD / 8; n++) { o[n][0] *= fA; o[n][1] *= fA; o[n][2] *= fB; o[n][3] *= fB; }
+      }
 #pragma unroll
       for (int d2 = 0; d2 < HD / 16; d2++) {
         uint32_t b0, b1, b2, b3;
@@ -1116,6 +1153,8 @@ __global__ void __launch_bounds__(160) attn_tma_small_kernel(const __grid_consta
       __syncwarp();
       if (lane == 0) mbar_arrive(&empty[st]);
     }
+    if (!vA) { mxA = -INFINITY; lA = 0.0f; }
+    if (!vB) { mxB = -INFINITY; lB = 0.0f; }
     // ---- merge the four key subsets: every warp parks (o, max, sum) in shared memory
     float *so = (float *)sm;                            // [NW][16][HD]: the ring is free once every warp has left the loop
     float *sml = so + NW * 16 * HD;                     // [NW][16][2]
@@ -1343,7 +1382,7 @@ void attn_fast_override_umma(int v) { tl_attn_umma = v; }
 
 int launch_attn_fast(const bf16 *q, KvPool pool, PageMap pm, RowMeta m, int tail_len, bf16 *out, int rows, int H, int G,
                      int hd, int rps, int ctx_hint, void *scratch, cudaStream_t s, bool contiguous_tail, int32_t *status,
-                     const int32_t *order, int order_len, unsigned long long *stamp) {
+                     const int32_t *order, int order_len, unsigned long long *stamp, bool ctx_ready) {
   if (rps < 1 || rows % rps) rps = 1;
   int seqs = rows / rps, grp = H / G;
   int mtiles = (rps * grp + MT - 1) / MT;
@@ -1355,6 +1394,7 @@ int launch_attn_fast(const bf16 *q, KvPool pool, PageMap pm, RowMeta m, int tail
   p.part_o = (float *)scratch;
   p.order = (order && order_len == seqs) ? order : nullptr;
   p.stamp = stamp;
+  p.ctx_ready = ctx_ready ? 1 : 0;
   p.part_ml = p.part_o ? p.part_o + (size_t)MAX_SPLITS * rows * H * hd : nullptr;
   dim3 grid(mtiles, nsplit, seqs * G);
   // TMA-staged kernel when the tail follows the context and a page is a whole number of 128-byte-swizzle boxes

@@ -244,7 +244,9 @@ __global__ void __launch_bounds__(fused_threads(NT, EPI), EPI == EPI_TOPK || EPI
   if (DUO) cluster_sync_all(); else __syncthreads();   // pairs: the partner's barriers must exist before anything signals them
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem_base = *tmem_slot;
-  pdl_trigger();
+  // EPI_QKV lets its dependents start only once it is past its own wait: whatever earlier kernels of the stream wrote is then
+  // complete, and the attention kernel that follows reads it (row metadata, page table, cached context) before it waits itself.
+  if (EPI != EPI_QKV) pdl_trigger();
 
   if (DUO && *abort_flag) {
     pdl_wait();            // wrong cluster layout: nothing is loaded or issued; the epilogue below writes nothing
@@ -260,6 +262,7 @@ __global__ void __launch_bounds__(fused_threads(NT, EPI), EPI == EPI_TOPK || EPI
       }
     __syncwarp();
     pdl_wait();
+    if (EPI == EPI_QKV) pdl_trigger();
     if (elect_one()) {
       if (p.stamp) atomicMin(p.stamp, global_ns());
       for (int i = 0; i < npre; i++)
@@ -286,6 +289,7 @@ __global__ void __launch_bounds__(fused_threads(NT, EPI), EPI == EPI_TOPK || EPI
     // ---- producer warp (all lanes walk the loop, the elected lane issues); the ring already holds weight tiles
     const CUtensorMap *mw0 = &p.map_w[mi];
     pdl_wait();
+    if (EPI == EPI_QKV) pdl_trigger();
     if (elect_one()) {
       if (p.stamp) atomicMin(p.stamp, global_ns());
       const bool hold = p.withhold && blockIdx.x == 0 && blockIdx.y == 0;     // test hook: the first stage never completes
@@ -310,6 +314,7 @@ __global__ void __launch_bounds__(fused_threads(NT, EPI), EPI == EPI_TOPK || EPI
     if (lane == 0) *n_issued = i;
   } else {
     pdl_wait();
+    if (EPI == EPI_QKV) pdl_trigger();
     if (DUO && warp == 1) {
       // ---- MMA issuer of a CTA pair (even CTA only): M = 256 over both CTAs' weight tiles, N = both activation halves
       if (xr == 0) {

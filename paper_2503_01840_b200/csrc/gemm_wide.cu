@@ -188,7 +188,7 @@ __global__ void __launch_bounds__(W_THREADS, 1) gemm_wide_kernel(const __grid_co
   cluster_sync_all();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem_base = *tmem_slot;        // 512 columns: the whole tensor memory, so both CTAs start at column 0
-  pdl_trigger();
+  if (EPI != WIDE_QKV) pdl_trigger();            // WIDE_QKV: after the wait, see gemm_fused_kernel
 
   if (warp == W_EPI_WARPS) {
     // ================================================================ producer (converged warp, the elected lane issues)
@@ -219,6 +219,7 @@ __global__ void __launch_bounds__(W_THREADS, 1) gemm_wide_kernel(const __grid_co
           }
         __syncwarp();
         pdl_wait();
+        if (EPI == WIDE_QKV) pdl_trigger();
         if (elect_one())
           for (int i = p.hold && blockIdx.x == 0 ? 1 : 0; i < npre; i++) tma_load_2d_pair(ring + i * W_STAGE, &p.map_x, i * TILE_K, xrow, mapa_u32(smem_u32(&full[i]), 0u));
         __syncwarp();
@@ -245,6 +246,7 @@ __global__ void __launch_bounds__(W_THREADS, 1) gemm_wide_kernel(const __grid_co
   } else if (warp == W_EPI_WARPS + 1) {
     // ================================================================ MMA issuer (even CTA only)
     pdl_wait();
+    if (EPI == WIDE_QKV) pdl_trigger();
     if (xr == 0 && !__any_sync(0xffffffffu, *abort_flag != 0)) {
       constexpr uint32_t idesc = umma_idesc_m(256, 256);
       const uint64_t desc0 = umma_desc_sw128(smem_u32(ring));
@@ -283,6 +285,7 @@ __global__ void __launch_bounds__(W_THREADS, 1) gemm_wide_kernel(const __grid_co
   } else {
     // ================================================================ epilogue: thread = token row, warp / 4 = half tile
     pdl_wait();
+    if (EPI == WIDE_QKV) pdl_trigger();
     if (p.stamp && threadIdx.x == 0) atomicMin(p.stamp, global_ns());
     unsigned char *stg = stg_all + warp * W_STG;
     const int quarter = warp & 3, half = warp >> 2;
@@ -569,7 +572,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1) gemm_wide_split_kernel(const __
   cluster_sync_all();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem_base = *tmem_slot;
-  pdl_trigger();
+  if (EPI != WIDE_QKV) pdl_trigger();            // WIDE_QKV: after the wait, see gemm_fused_kernel
 
   if (warp == WS_EPI_WARPS) {
     // ---- producer: own rows and own half of the features; all bytes are counted on the even CTA's barrier
@@ -587,6 +590,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1) gemm_wide_split_kernel(const __
       }
     __syncwarp();
     pdl_wait();
+    if (EPI == WIDE_QKV) pdl_trigger();
     if (elect_one()) {
       if (p.stamp) atomicMin(p.stamp, global_ns());
       for (int i = hold ? 1 : 0; i < npre; i++) tma_load_2d_pair(ring + i * W_STAGE, &p.map_x, (kb0 + i) * TILE_K, row_c, mapa_u32(smem_u32(&full[i]), lead));
@@ -611,6 +615,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1) gemm_wide_split_kernel(const __
     if (lane == 0) *n_issued = i;
   } else if (warp == WS_EPI_WARPS + 1) {
     pdl_wait();
+    if (EPI == WIDE_QKV) pdl_trigger();
     if (xr == 0 && !__any_sync(0xffffffffu, *abort_flag != 0)) {
       constexpr uint32_t idesc = umma_idesc_m(256, 256);
       uint32_t partner_base;
@@ -642,6 +647,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1) gemm_wide_split_kernel(const __
     }
   } else {
     pdl_wait();
+    if (EPI == WIDE_QKV) pdl_trigger();
     if ((int)threadIdx.x < nrow) {                             // per-row values of this CTA's rows
       inv_s[threadIdx.x] = row_scale(p, row_c + threadIdx.x);
       if (EPI == WIDE_QKV) {
