@@ -1258,13 +1258,15 @@ __global__ void __launch_bounds__(256) attn_combine_kernel(const float *__restri
 
 int g_attn_target_ctas = 148;
 
-int pick_splits(int seqs, int G, int mtiles, int max_ctx_tiles, int target = 0) {
-  int base = seqs * G * mtiles;
-  int want = (target > 0 ? target : g_attn_target_ctas) / base;                             // the kernels run one CTA per SM (register-bound): never more CTAs than one wave
-  if (want < 1) want = 1;
-  int s = want < max_ctx_tiles ? want : max_ctx_tiles;
-  if (s > MAX_SPLITS) s = MAX_SPLITS;
-  return s < 1 ? 1 : s;
+// Key splits: as many as one wave of CTAs allows (the kernels run one CTA per SM, they are register-bound), but no more than
+// give the busiest CTA its number of tiles: further splits only add partial results to merge.  One tile more than the hint is
+// counted, because the context grows while a captured step is replayed.  8B verify pass at 572..660 keys (9 or 10 tiles): 9 splits
+// (one or two tiles a CTA) 13.5 us, 5 splits (two) 12.5.
+int pick_splits(int seqs, int G, int mtiles, int ntiles) {
+  const int n = ntiles + 1;
+  int s = std::min(std::max(1, g_attn_target_ctas / (seqs * G * mtiles)), std::min(n, MAX_SPLITS));
+  const int per = (n + s - 1) / s;
+  return (n + per - 1) / per;
 }
 
 }  // namespace
@@ -1352,8 +1354,9 @@ int launch_tma_small(AttnParams &p, dim3 grid, const CUtensorMap *mk, const CUte
   return 0;
 }
 
-int g_attn_umma = 2;            // tcgen05 kernel for the tree passes: 0 off, 1 on, 2 on when a CTA gets at least UM_MIN_TILES key tiles
-constexpr int UM_MIN_TILES = 3; // below that the pass is launch- and latency-bound and the mma.sync kernel's shorter prologue wins
+int g_attn_umma = 2;            // tcgen05 kernel for the tree passes: 0 off, 1 on, 2 on when the busiest CTA gets at least UM_MIN_TILES key tiles
+// 8B verify pass, mma.sync / tcgen05 kernel: two tiles 12.5 / 12.5 us, three 14.6 / 13.6; with 40 query rows (draft) two tiles 8.8 / 9.0
+constexpr int UM_MIN_TILES = 3;
 thread_local int tl_attn_umma = -1;   // per-call override (-1: none)
 
 int launch_umma(AttnParams &p, dim3 grid, const CUtensorMap *mk, const CUtensorMap *mv, int32_t *status, cudaStream_t s) {
@@ -1380,14 +1383,21 @@ void attn_fast_set_target_ctas(int n) { g_attn_target_ctas = n; }
 void attn_fast_set_umma(int mode) { g_attn_umma = mode; }
 void attn_fast_override_umma(int v) { tl_attn_umma = v; }
 
+int attn_fast_plan(int rows, int H, int G, int hd, int rps, int ctx_hint, int tail_len) {
+  if (rps < 1 || rows % rps) rps = 1;
+  const int grp = H / G, mtiles = (rps * grp + MT - 1) / MT, ntiles = std::max(1, (ctx_hint + tail_len + KT - 1) / KT);
+  const int nsplit = pick_splits(rows / rps, G, mtiles, ntiles);
+  const int um_mode = tl_attn_umma >= 0 ? tl_attn_umma : g_attn_umma;
+  const bool umma = hd == 128 && rps * grp > 16 && (um_mode == 1 || (um_mode == 2 && ntiles + 1 > (UM_MIN_TILES - 1) * nsplit));
+  return nsplit << 1 | (umma ? 1 : 0);
+}
+
 int launch_attn_fast(const bf16 *q, KvPool pool, PageMap pm, RowMeta m, int tail_len, bf16 *out, int rows, int H, int G,
                      int hd, int rps, int ctx_hint, void *scratch, cudaStream_t s, bool contiguous_tail, int32_t *status,
                      const int32_t *order, int order_len, unsigned long long *stamp, bool ctx_ready) {
   if (rps < 1 || rows % rps) rps = 1;
-  int seqs = rows / rps, grp = H / G;
-  int mtiles = (rps * grp + MT - 1) / MT;
-  int ntiles_hint = (ctx_hint + tail_len + KT - 1) / KT;
-  int nsplit = scratch ? pick_splits(seqs, G, mtiles, ntiles_hint < 1 ? 1 : ntiles_hint) : 1;
+  const int seqs = rows / rps, grp = H / G, mtiles = (rps * grp + MT - 1) / MT;
+  const int plan = attn_fast_plan(rows, H, G, hd, rps, ctx_hint, tail_len), nsplit = scratch ? plan >> 1 : 1;
   AttnParams p;
   p.q = q; p.kpool = (const bf16 *)pool.k; p.vpool = (const bf16 *)pool.v; p.pm = pm; p.m = m; p.tail_len = tail_len;
   p.rows = rows; p.H = H; p.G = G; p.rps = rps; p.nsplit = nsplit; p.out = out;
@@ -1400,8 +1410,7 @@ int launch_attn_fast(const bf16 *q, KvPool pool, PageMap pm, RowMeta m, int tail
   // TMA-staged kernel when the tail follows the context and a page is a whole number of 128-byte-swizzle boxes
   const int ps = pm.page_size;
   if (contiguous_tail && (ps == 16 || ps == 32 || ps == 64) && (hd == 64 || hd == 128)) {
-    const int um_mode = tl_attn_umma >= 0 ? tl_attn_umma : g_attn_umma;
-    const bool umma = hd == 128 && rps * grp > 16 && (um_mode == 1 || (um_mode == 2 && ntiles_hint >= UM_MIN_TILES * nsplit));
+    const bool umma = plan & 1;
     const CUtensorMap *mk = kv_map(pool.k, pm.num_pages, G, ps, hd, umma ? 1 : 0), *mv = kv_map(pool.v, pm.num_pages, G, ps, hd, umma ? 1 : 0);
     if (mk && mv) {
       int rc = umma ? launch_umma(p, grid, mk, mv, status, s) : hd == 128 ? launch_tma<128>(p, grid, mk, mv, status, s) : launch_tma<64>(p, grid, mk, mv, status, s);
