@@ -6,6 +6,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <atomic>
 #include <string>
 #include <vector>
 
@@ -50,6 +51,17 @@ struct LayerW {
   const void *attn_norm, *wq, *wk, *wv, *wo, *mlp_norm, *w_gate, *w_up, *w_down;
 };
 
+// Sequence state of freshly read prompts: st.n_prev holds their lengths, y their first tokens.
+__global__ void prefill_state_kernel(SeqState st, const int32_t *__restrict__ y, int32_t *__restrict__ pend_tok, int B, int Pmax) {
+  pdl_wait();
+  pdl_trigger();
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < B * Pmax; i += gridDim.x * blockDim.x) {
+    const int b = i / Pmax, root = y[b];
+    pend_tok[i] = i % Pmax == 0 ? root : 0;
+    if (i % Pmax == 0) { st.n[b] = st.n_prev[b]; st.P[b] = 1; st.root[b] = root; }
+  }
+}
+
 // Bump allocator over the caller's workspace; with base == nullptr it only measures.
 struct Carver {
   char *base;
@@ -62,6 +74,12 @@ struct Carver {
     return p;
   }
   void *take_bytes(size_t n) { return take<char>(n); }
+};
+
+// what a captured step depends on besides the context's own buffers (see step_plan)
+struct StepPlan {
+  int epoch = -1, extend = 0, tree = 0, verify = 0;
+  bool operator==(const StepPlan &o) const { return epoch == o.epoch && extend == o.extend && tree == o.tree && verify == o.verify; }
 };
 
 struct spec_ctx {
@@ -85,6 +103,10 @@ struct spec_ctx {
   SeqState st;
   TreeBufs tb;
   int32_t *status;
+  // What a call returns lies in one run of the workspace and comes to the host in one copy into pinned memory: [B * Pmax] emitted
+  // ids, [B] counts, [B] lengths, [B] root tokens, [8] status words.
+  int32_t *res = nullptr, *res_host = nullptr;
+  float *u_host = nullptr;     // pinned staging of u_dev
   float *cap_logits, *cap_a;   // capture buffers (SPEC_FLAG_CAPTURE)
   // fused bf16 path: GEMM epilogues do the norm / RoPE / activation / residual / argmax work
   bool fused = false;
@@ -117,6 +139,7 @@ struct spec_ctx {
   bool prefilled = false, draft_stale = false;
   cudaGraphExec_t graph = nullptr;
   cudaGraphExec_t graph_sampled = nullptr;   // the same step with the stochastic acceptance kernel
+  StepPlan graph_plan[2];                    // of graph, graph_sampled
   int launches = 0, launches_graph = 0, launches_graph_sampled = 0;
   bool sampled = false;        // the step being scheduled ends with the stochastic acceptance
   float *u_dev = nullptr;      // [B][2N] uniforms of the sampled step, then 1 / temperature
@@ -215,8 +238,10 @@ static size_t carve(spec_ctx *c, void *base) {
   }
   c->pools_dev = cv.take<KvPool>(c->L + 1);
   c->page_table = cv.take<int32_t>((size_t)B * c->pps);
-  c->st.n = cv.take<int32_t>(B); c->st.n_prev = cv.take<int32_t>(B); c->st.P = cv.take<int32_t>(B);
-  c->st.root = cv.take<int32_t>(B); c->st.cap = cv.take<int32_t>(B); c->st.last_row = cv.take<int32_t>(B);
+  c->res = cv.take<int32_t>((size_t)B * (c->Pmax + 3) + 8);
+  c->tb.out_ids = c->res; c->tb.out_cnt = c->res + (size_t)B * c->Pmax;
+  c->st.n = c->tb.out_cnt + B; c->st.root = c->st.n + B; c->status = c->st.root + B;
+  c->st.n_prev = cv.take<int32_t>(B); c->st.P = cv.take<int32_t>(B); c->st.cap = cv.take<int32_t>(B); c->st.last_row = cv.take<int32_t>(B);
   c->st.active = cv.take<int32_t>(B);
   c->st.order = cv.take<int32_t>(B);
   TreeBufs &t = c->tb;
@@ -232,11 +257,9 @@ static size_t carve(spec_ctx *c, void *base) {
   t.tok = cv.take<int32_t>(ne); t.parent = cv.take<int32_t>(ne); t.depth = cv.take<int32_t>(ne);
   t.poolidx = cv.take<int32_t>(ne); t.score = cv.take<float>(ne); t.mask = cv.take<uint64_t>(ne);
   t.nn = cv.take<int32_t>(B); t.y = cv.take<int32_t>(ne);
-  t.path = cv.take<int32_t>((size_t)B * c->Pmax); t.out_ids = cv.take<int32_t>((size_t)B * c->Pmax);
-  t.out_cnt = cv.take<int32_t>(B); t.pend_tok = cv.take<int32_t>((size_t)B * c->Pmax);
+  t.path = cv.take<int32_t>((size_t)B * c->Pmax); t.pend_tok = cv.take<int32_t>((size_t)B * c->Pmax);
   c->u_dev = cv.take<float>((size_t)B * 2 * c->N + 1);
   c->prompt_dev = cv.take<int32_t>((size_t)B * g.max_ctx + 1);
-  c->status = cv.take<int32_t>(8);
   if (g.flags & SPEC_FLAG_CAPTURE) {
     c->cap_logits = cv.take<float>((size_t)c->D * c->Td * c->Vd);
     c->cap_a = cv.take<float>((size_t)c->D * c->Td * k);
@@ -277,6 +300,7 @@ extern "C" size_t spec_workspace_bytes(const spec_cfg *cfg) {
 
 extern "C" const char *spec_last_error(const spec_ctx *ctx) { return ctx ? ctx->err : g_init_err; }
 
+extern "C" int spec_free(spec_ctx *c);
 extern "C" int spec_init(spec_ctx **out, const spec_target_weights *tw, const spec_draft_weights *dw, const spec_cfg *cfg) {
   if (out) *out = nullptr;
   if (!out || !tw || !dw || !cfg) return fail(nullptr, SPEC_ERR_NULL, "spec_init: NULL argument");
@@ -322,6 +346,12 @@ extern "C" int spec_init(spec_ctx **out, const spec_target_weights *tw, const sp
     delete c;
     return rc;
   }
+  if (cudaMallocHost((void **)&c->res_host, ((size_t)c->B * (c->Pmax + 3) + 8) * sizeof(int32_t)) != cudaSuccess ||
+      cudaMallocHost((void **)&c->u_host, ((size_t)c->B * 2 * c->N + 1) * sizeof(float)) != cudaSuccess) {
+    cudaGetLastError();
+    spec_free(c);
+    return fail(nullptr, SPEC_ERR_CUDA, "spec_init: no pinned host memory");
+  }
   c->n_upper.assign(c->B, 0); c->cap_host.assign(c->B, 0); c->n_pages_host.assign(c->B, 0);
   c->page_table_host.assign((size_t)c->B * c->pps, 0);
   if (cfg->dtype == SPEC_BF16 && !((cfg->flags & SPEC_FLAG_REF_GEMM))) {
@@ -329,7 +359,7 @@ extern "C" int spec_init(spec_ctx **out, const spec_target_weights *tw, const sp
     c->fg = tma_maps_create(why);
     if (!c->fg) {
       int rc = fail(nullptr, SPEC_ERR_CUDA, "spec_init: tcgen05 GEMM set-up failed: %s", why.c_str());
-      delete c;
+      spec_free(c);
       return rc;
     }
   }
@@ -337,14 +367,12 @@ extern "C" int spec_init(spec_ctx **out, const spec_target_weights *tw, const sp
   c->tree_fused = c->fused && draft_tree_step_fits(c->dtiles, c->K);
   if (c->fg && !(c->hd <= 128 && (c->hd & (c->hd - 1)) == 0)) {
     int rc = fail(nullptr, SPEC_ERR_UNSUPPORTED, "spec_init: the bf16 tensor-core path takes a power-of-two head_dim <= 128 (got %d)", c->hd);
-    tma_maps_destroy(c->fg);
-    delete c;
+    spec_free(c);
     return rc;
   }
   if (c->fg && c->R > 256) {
     int rc = fail(nullptr, SPEC_ERR_UNSUPPORTED, "spec_init: %d rows per pass exceed the 256 the tensor-core GEMM takes", c->R);
-    tma_maps_destroy(c->fg);
-    delete c;
+    spec_free(c);
     return rc;
   }
   *out = c;
@@ -357,6 +385,8 @@ extern "C" int spec_free(spec_ctx *c) {
   if (c->graph_sampled) cudaGraphExecDestroy(c->graph_sampled);
   if (c->fg) tma_maps_destroy(c->fg);
   for (cudaEvent_t e : c->prof_ev) cudaEventDestroy(e);
+  if (c->res_host) cudaFreeHost(c->res_host);
+  if (c->u_host) cudaFreeHost(c->u_host);
   delete c;
   return SPEC_OK;
 }
@@ -898,10 +928,12 @@ template <typename T> struct Sched {
 // hazard note: draft_forward for tree passes reads c->x (previous pass) in build_cat before FC2 + the
 // block's first add_norm overwrite it; everything is ordered on one stream.
 
-static int read_status(spec_ctx *c) {
-  int32_t st[4] = {0, 0, 0, 0};
-  CUDA_TRY(c, cudaMemcpyAsync(st, c->status, sizeof st, cudaMemcpyDeviceToHost, c->stream));
+// Waits for the stream and brings the results run to c->res_host; reports (and clears) what the kernels left in the status words.
+static int fetch_results(spec_ctx *c) {
+  const size_t n = (size_t)c->B * (c->Pmax + 3) + 8;
+  CUDA_TRY(c, cudaMemcpyAsync(c->res_host, c->res, n * sizeof(int32_t), cudaMemcpyDeviceToHost, c->stream));
   CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+  const int32_t *st = c->res_host + (c->status - c->res);
   if (st[0] != 0) {
     cudaMemsetAsync(c->status, 0, 16, c->stream);
     int code = st[0] == ST_CAPACITY ? SPEC_ERR_CAPACITY : SPEC_ERR_DEVICE_STATUS;
@@ -909,10 +941,21 @@ static int read_status(spec_ctx *c) {
   }
   return SPEC_OK;
 }
+// the end of a step: its outputs and the committed lengths
+static int finish_step(spec_ctx *c, int32_t *out_ids, int32_t *out_counts) {
+  const int rc = fetch_results(c);
+  if (rc && rc != SPEC_ERR_CAPACITY && rc != SPEC_ERR_DEVICE_STATUS) return rc;      // no results came
+  if (out_ids) memcpy(out_ids, c->res_host, (size_t)c->B * c->Pmax * sizeof(int32_t));
+  if (out_counts) memcpy(out_counts, c->res_host + (size_t)c->B * c->Pmax, c->B * sizeof(int32_t));
+  if (rc) return rc;
+  const int32_t *n = c->res_host + (c->st.n - c->res);
+  c->n_upper.assign(n, n + c->B);
+  return SPEC_OK;
+}
 
 // ---- prefill, one prompt after the other in passes of PREFILL_CHUNK rows: the fp32 model, head dimensions other than 128
 // and the page sizes without tensor maps
-template <typename T> static int prefill_blocks(spec_ctx *c, const int32_t *lens, int32_t *root_host) {
+template <typename T> static int prefill_blocks(spec_ctx *c, const int32_t *lens) {
   cudaStream_t s = c->stream;
   Sched<T> sc(c);
   const int B = c->B;
@@ -940,7 +983,7 @@ template <typename T> static int prefill_blocks(spec_ctx *c, const int32_t *lens
         CUDA_TRY(c, cudaMemcpyAsync((char *)c->pend_taps + (size_t)b * c->Pmax * 3 * c->k * c->esz,
                                     (char *)c->node_taps + (size_t)(nv - 1) * 3 * c->k * c->esz, (size_t)3 * c->k * c->esz,
                                     cudaMemcpyDeviceToDevice, s));
-        CUDA_TRY(c, cudaMemcpyAsync(&root_host[b], c->tb.y + (nv - 1), 4, cudaMemcpyDeviceToHost, s));
+        CUDA_TRY(c, cudaMemcpyAsync(c->st.root + b, c->tb.y + (nv - 1), 4, cudaMemcpyDeviceToDevice, s));
       }
       int nd = last ? nv - 1 : nv;        // draft entries j use token j+1; the last position waits for the root
       if (nd > 0) {
@@ -949,7 +992,6 @@ template <typename T> static int prefill_blocks(spec_ctx *c, const int32_t *lens
         sc.draft_forward(c->proj, c->np_proj, c->ps_proj, nullptr, CH, PREFILL_BLOCK);
       }
     }
-    CUDA_TRY(c, cudaStreamSynchronize(s));
     c->ctx_hint = -1;
     off += n;
   }
@@ -961,7 +1003,7 @@ template <typename T> static int prefill_blocks(spec_ctx *c, const int32_t *lens
 // GEMMs run at the tensor pipe's rate (64 prompts of 64..768 tokens: 26.6k rows are 9 passes instead of 132).
 constexpr int WIDE_MAX_TILES = 16;       // row tiles (256 rows) of a pass: the waves of a launch are full enough by then
 constexpr int WIDE_LAYER_COST = 64;      // what a layer's launches cost beside their waves, in k-blocks (0.27 us each)
-static int prefill_packed(spec_ctx *c, const int32_t *lens, size_t total, int32_t *root_host, bool &done) {
+static int prefill_packed(spec_ctx *c, const int32_t *lens, size_t total, bool &done) {
   done = false;
   c->pass_rows.clear();
   const spec_cfg &g = c->cfg;
@@ -1032,10 +1074,32 @@ static int prefill_packed(spec_ctx *c, const int32_t *lens, size_t total, int32_
   }
   CUDA_TRY(c, cudaGetLastError());
   if (c->sched_err) return fail(c, SPEC_ERR_CUDA, "a prefill launch was rejected (code %d)", c->sched_err);
-  CUDA_TRY(c, cudaMemcpyAsync(root_host, c->tb.y, B * 4, cudaMemcpyDeviceToHost, s));
-  CUDA_TRY(c, cudaStreamSynchronize(s));
   done = true;
   return SPEC_OK;
+}
+
+// A captured step is made of the context's own buffers; all that changes with the prompts is how the attention passes split
+// their keys.  It is kept from one request to the next while that, and the process-wide knobs, are what they were at capture
+// (capture and instantiation take 0.3 to 1 ms).
+static std::atomic<int> g_tune_epoch{0};
+static StepPlan step_plan(const spec_ctx *c) {
+  StepPlan p;
+  p.epoch = g_tune_epoch.load();
+  if (!c->fused) return p;                 // the plain schedule's attention takes no plan
+  int hint = 0;
+  for (int b = 0; b < c->B; b++) hint = std::max(hint, c->n_upper[b]);
+  p.extend = attn_fast_plan(c->Te, c->H, c->G, c->hd, c->Pmax, hint, c->Pmax);
+  p.tree = attn_fast_plan(c->Td, c->H, c->G, c->hd, c->K, hint, c->tail_tree);
+  p.verify = attn_fast_plan(c->Tv, c->H, c->G, c->hd, c->N, hint, c->N);
+  return p;
+}
+static void drop_graph(cudaGraphExec_t &g) {
+  if (g) { cudaGraphExecDestroy(g); g = nullptr; }
+}
+static void drop_stale_graphs(spec_ctx *c) {
+  const StepPlan p = step_plan(c);
+  if (c->stamps || !(c->graph_plan[0] == p)) drop_graph(c->graph);          // (stamps: the list of stamped launches is made at capture)
+  if (c->stamps || !(c->graph_plan[1] == p)) drop_graph(c->graph_sampled);
 }
 
 template <typename T> static int do_prefill(spec_ctx *c, const int32_t *ids, const int32_t *lens, int32_t reserve, int32_t *first) {
@@ -1068,8 +1132,7 @@ template <typename T> static int do_prefill(spec_ctx *c, const int32_t *ids, con
   }
   c->cap_host = cap;
   CUDA_TRY(c, cudaMemcpyAsync(c->page_table, c->page_table_host.data(), c->page_table_host.size() * 4, cudaMemcpyHostToDevice, s));
-  CUDA_TRY(c, cudaMemcpyAsync(c->st.cap, cap.data(), B * 4, cudaMemcpyHostToDevice, s));
-  CUDA_TRY(c, cudaStreamSynchronize(s));
+  CUDA_TRY(c, cudaMemcpyAsync(c->st.cap, cap.data(), B * 4, cudaMemcpyHostToDevice, s));       // (pageable: taken over before the call returns)
 
   size_t total_ids = 0;
   for (int b = 0; b < B; b++) {
@@ -1081,25 +1144,21 @@ template <typename T> static int do_prefill(spec_ctx *c, const int32_t *ids, con
   // the prompts go to the device once; the row metadata of each pass is then built by a small kernel, so the host never
   // waits inside the loop over passes
   CUDA_TRY(c, cudaMemcpyAsync(c->prompt_dev, ids, total_ids * 4, cudaMemcpyHostToDevice, s));
-  std::vector<int32_t> n_host(lens, lens + B), P_host(B, 1), root_host(B);
+  CUDA_TRY(c, cudaMemcpyAsync(c->st.n_prev, lens, B * 4, cudaMemcpyHostToDevice, s));
   bool packed = false;
-  if (int rc = prefill_packed(c, lens, total_ids, root_host.data(), packed)) return rc;
+  if (int rc = prefill_packed(c, lens, total_ids, packed)) return rc;
   if (!packed)
-    if (int rc = prefill_blocks<T>(c, lens, root_host.data())) return rc;
-  CUDA_TRY(c, cudaMemcpyAsync(c->st.n, n_host.data(), B * 4, cudaMemcpyHostToDevice, s));
-  CUDA_TRY(c, cudaMemcpyAsync(c->st.n_prev, n_host.data(), B * 4, cudaMemcpyHostToDevice, s));
-  CUDA_TRY(c, cudaMemcpyAsync(c->st.P, P_host.data(), B * 4, cudaMemcpyHostToDevice, s));
-  CUDA_TRY(c, cudaMemcpyAsync(c->st.root, root_host.data(), B * 4, cudaMemcpyHostToDevice, s));
-  std::vector<int32_t> pt((size_t)B * c->Pmax, 0);
-  for (int b = 0; b < B; b++) pt[(size_t)b * c->Pmax] = root_host[b];
-  CUDA_TRY(c, cudaMemcpyAsync(c->tb.pend_tok, pt.data(), pt.size() * 4, cudaMemcpyHostToDevice, s));
-  CUDA_TRY(c, cudaStreamSynchronize(s));
-  for (int b = 0; b < B; b++) { c->n_upper[b] = n_host[b]; first[b] = root_host[b]; }
+    if (int rc = prefill_blocks<T>(c, lens)) return rc;
+  prefill_state_kernel<<<std::min(16, (B * c->Pmax + 127) / 128), 128, 0, s>>>(c->st, packed ? c->tb.y : c->st.root, c->tb.pend_tok, B, c->Pmax);
+  CUDA_TRY(c, cudaGetLastError());
+  const int rc = fetch_results(c);
+  if (rc && rc != SPEC_ERR_CAPACITY && rc != SPEC_ERR_DEVICE_STATUS) return rc;
+  const int32_t *root = c->res_host + (c->st.root - c->res);
+  for (int b = 0; b < B; b++) { c->n_upper[b] = lens[b]; first[b] = root[b]; }
   c->prefilled = true;
   c->draft_stale = false;
-  if (c->graph) { cudaGraphExecDestroy(c->graph); c->graph = nullptr; }
-  if (c->graph_sampled) { cudaGraphExecDestroy(c->graph_sampled); c->graph_sampled = nullptr; }
-  return read_status(c);
+  drop_stale_graphs(c);
+  return rc;
 }
 
 extern "C" int spec_prefill(spec_ctx *c, const int32_t *ids, const int32_t *lens, int32_t reserve, int32_t *first) {
@@ -1131,6 +1190,7 @@ static int launch_step(spec_ctx *c, bool plain) {
     cudaGraphDestroy(gr);
     if (e != cudaSuccess) { graph = nullptr; return fail(c, SPEC_ERR_CUDA, "graph instantiate: %s", cudaGetErrorString(e)); }
     launches_graph = c->launches;
+    c->graph_plan[c->sampled ? 1 : 0] = step_plan(c);
   }
   c->launches = launches_graph;
   CUDA_TRY(c, cudaGraphLaunch(graph, c->stream));
@@ -1170,10 +1230,7 @@ extern "C" int spec_step(spec_ctx *c, int32_t *out_ids, int32_t *out_counts) {
   if (!c) return SPEC_ERR_NULL;
   if (!out_ids || !out_counts) return fail(c, SPEC_ERR_NULL, "spec_step: NULL output");
   if (int rc = spec_step_async(c, nullptr, nullptr)) return rc;
-  CUDA_TRY(c, cudaMemcpyAsync(out_ids, c->tb.out_ids, (size_t)c->B * c->Pmax * 4, cudaMemcpyDeviceToHost, c->stream));
-  CUDA_TRY(c, cudaMemcpyAsync(out_counts, c->tb.out_cnt, (size_t)c->B * 4, cudaMemcpyDeviceToHost, c->stream));
-  if (int rc = read_status(c)) return rc;
-  return sync_lengths(c);
+  return finish_step(c, out_ids, out_counts);
 }
 
 extern "C" int spec_step_sampled(spec_ctx *c, float temperature, const float *u, int32_t *out_ids, int32_t *out_counts) {
@@ -1183,19 +1240,15 @@ extern "C" int spec_step_sampled(spec_ctx *c, float temperature, const float *u,
   if (c->draft_stale) return fail(c, SPEC_ERR_STATE, "spec_step_sampled after spec_plain_step: the draft cache is stale, prefill again");
   if (int rc = check_capacity(c, c->Pmax, "spec_step_sampled")) return rc;
   const size_t nu = (size_t)c->B * 2 * c->N;
-  const float inv_t = 1.0f / temperature;
-  CUDA_TRY(c, cudaMemcpyAsync(c->u_dev, u, nu * sizeof(float), cudaMemcpyHostToDevice, c->stream));
-  CUDA_TRY(c, cudaMemcpyAsync(c->u_dev + nu, &inv_t, sizeof(float), cudaMemcpyHostToDevice, c->stream));
-  CUDA_TRY(c, cudaStreamSynchronize(c->stream));           // inv_t lives on this stack frame
+  memcpy(c->u_host, u, nu * sizeof(float));
+  c->u_host[nu] = 1.0f / temperature;
+  CUDA_TRY(c, cudaMemcpyAsync(c->u_dev, c->u_host, (nu + 1) * sizeof(float), cudaMemcpyHostToDevice, c->stream));
   c->sampled = true;
   int rc = launch_step(c, false);
   c->sampled = false;
-  if (rc) return rc;
+  if (rc) { cudaStreamSynchronize(c->stream); return rc; }     // the staging buffer is the next call's
   for (int b = 0; b < c->B; b++) c->n_upper[b] += c->Pmax;
-  CUDA_TRY(c, cudaMemcpyAsync(out_ids, c->tb.out_ids, (size_t)c->B * c->Pmax * 4, cudaMemcpyDeviceToHost, c->stream));
-  CUDA_TRY(c, cudaMemcpyAsync(out_counts, c->tb.out_cnt, (size_t)c->B * 4, cudaMemcpyDeviceToHost, c->stream));
-  if (int rc2 = read_status(c)) return rc2;
-  return sync_lengths(c);
+  return finish_step(c, out_ids, out_counts);
 }
 
 extern "C" int spec_plain_step(spec_ctx *c, int32_t *out_ids) {
@@ -1204,11 +1257,9 @@ extern "C" int spec_plain_step(spec_ctx *c, int32_t *out_ids) {
   if (int rc = check_capacity(c, 1, "spec_plain_step")) return rc;
   c->draft_stale = true;
   if (int rc = launch_step(c, true)) return rc;
-  std::vector<int32_t> ids((size_t)c->B * c->Pmax);
-  CUDA_TRY(c, cudaMemcpyAsync(ids.data(), c->tb.out_ids, ids.size() * 4, cudaMemcpyDeviceToHost, c->stream));
-  if (int rc = read_status(c)) return rc;
-  for (int b = 0; b < c->B; b++) out_ids[b] = ids[(size_t)b * c->Pmax];
-  return sync_lengths(c);
+  if (int rc = finish_step(c, nullptr, nullptr)) return rc;
+  for (int b = 0; b < c->B; b++) out_ids[b] = c->res_host[(size_t)b * c->Pmax];
+  return SPEC_OK;
 }
 
 extern "C" int spec_lengths(spec_ctx *c, int32_t *lens) {
@@ -1230,7 +1281,7 @@ extern "C" int spec_profile_step(spec_ctx *c, float *class_ms, int32_t *class_la
   c->prof = false;
   for (int b = 0; b < c->B; b++) c->n_upper[b] += c->Pmax;
   CUDA_TRY(c, cudaGetLastError());
-  if (int rc = read_status(c)) return rc;
+  if (int rc = fetch_results(c)) return rc;
   for (int i = 0; i + 1 < c->prof_n; i++) {
     float ms = 0.0f;
     CUDA_TRY(c, cudaEventElapsedTime(&ms, c->prof_ev[i], c->prof_ev[i + 1]));
@@ -1245,6 +1296,7 @@ extern "C" int spec_tune(spec_ctx *c, int32_t what, int32_t value) {
     if (what != SPEC_TUNE_GEMM_PAIRS) return SPEC_ERR_NULL;
     if (value < 0 || value > 3) return SPEC_ERR_INVALID_CFG;
     fused_gemm_set_pairs(value);
+    g_tune_epoch++;
     return SPEC_OK;
   }
   if (what == SPEC_TUNE_ATTN_CTAS) {
@@ -1267,8 +1319,10 @@ extern "C" int spec_tune(spec_ctx *c, int32_t what, int32_t value) {
   } else {
     return fail(c, SPEC_ERR_INVALID_CFG, "spec_tune: unknown knob %d", what);
   }
-  if (c->graph) { cudaStreamSynchronize(c->stream); cudaGraphExecDestroy(c->graph); c->graph = nullptr; }   // re-capture with the new plan
-  if (c->graph_sampled) { cudaStreamSynchronize(c->stream); cudaGraphExecDestroy(c->graph_sampled); c->graph_sampled = nullptr; }
+  g_tune_epoch++;                                  // every other context captures again with its next request
+  cudaStreamSynchronize(c->stream);
+  drop_graph(c->graph);
+  drop_graph(c->graph_sampled);
   return SPEC_OK;
 }
 
