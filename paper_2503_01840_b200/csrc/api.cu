@@ -93,6 +93,7 @@ struct spec_ctx {
   const int32_t *d2t;
   // device buffers
   float *x, *proj, *qkv, *gu, *logits;
+  float *x_alt = nullptr;      // fp32 schedule: the residual stream alternates between x and this
   void *h, *q, *ao, *act, *cat, *node_taps, *pend_taps;
   float2 *cs;
   double *inv_freq;
@@ -217,6 +218,7 @@ static size_t carve(spec_ctx *c, void *base) {
   Carver cv(base);
   c->x = cv.take<float>((size_t)R * k);
   c->proj = cv.take<float>((size_t)R * k);
+  c->x_alt = e == 4 ? cv.take<float>((size_t)R * k) : nullptr;
   if (g.flags & SPEC_FLAG_CAPTURE) c->logits = cv.take<float>((size_t)R * std::max(c->V, c->Vd));
   c->h = cv.take_bytes((size_t)R * k * e);
   c->q = cv.take_bytes((size_t)R * qd * e);
@@ -678,6 +680,61 @@ template <typename T> struct Sched {
     gemm(c->act, w.w_down, c->proj, rows, k, F, k, 0, c->np_proj);
   }
 
+  // ---- fp32 model, few rows: the norms, RoPE, cache writes and activations ride on the GEMMs (launch_norm_*); five launches a
+  // layer instead of nine.  Weights or row counts those kernels are not for take the schedule above.
+  bool norm_fused(int rows) const {
+    if (sizeof(T) != 4 || (c->hd & 1)) return false;
+    auto layer_ok = [&](const LayerW &w) {
+      const float *qkv[3] = {(const float *)w.wq, (const float *)w.wk, (const float *)w.wv}, *gu[2] = {(const float *)w.w_gate, (const float *)w.w_up};
+      return gemm_norm_ok(qkv, 3, (const float *)w.attn_norm, rows, (c->H + 2 * c->G) * c->hd, c->k) &&
+             gemm_norm_ok(gu, 2, (const float *)w.mlp_norm, rows, 2 * c->F, c->k);
+    };
+    for (const LayerW &w : c->tl)
+      if (!layer_ok(w)) return false;
+    return layer_ok(c->dl);
+  }
+  float *x_now = nullptr;        // where the residual stream is
+  float *x_other() const { return x_now == c->x ? c->x_alt : c->x; }
+  // the layer up to its attention; add: the partial result still to be added to x_now; set: the stream is that result
+  void block_qkv32(const LayerW &w, KvPool pool, int rows, bool add, bool set, int tap_mask) {
+    const PageMap pm{c->page_table, c->pps, c->cfg.page_size, c->cfg.num_pages};
+    float *next = set ? c->x : add ? x_other() : nullptr;
+    mark(SPEC_PROF_GEMM);
+    launch_norm_qkv(set ? c->proj : x_now, add ? c->proj : nullptr, next, (float *)c->node_taps, tap_mask, (const float *)w.attn_norm, c->cfg.rms_eps,
+                    (const float *)w.wq, (const float *)w.wk, (const float *)w.wv, c->cs, c->meta, (float *)c->q, pool, pm, rows, c->H, c->G, c->hd, c->k,
+                    c->status, s);
+    tick();
+    if (next) x_now = next;
+  }
+  void block32(const LayerW &w, KvPool pool, int rows, int tail_len, bool add, bool set, int tap_mask) {
+    block_qkv32(w, pool, rows, add, set, tap_mask);
+    attention(pool, rows, tail_len);
+    gemm(c->ao, w.wo, c->proj, rows, c->k, c->H * c->hd, c->k, 0, 1);
+    float *next = x_other();
+    mark(SPEC_PROF_GEMM);
+    launch_norm_swiglu(x_now, c->proj, next, (const float *)w.mlp_norm, c->cfg.rms_eps, (const float *)w.w_gate, (const float *)w.w_up, (float *)c->act, rows,
+                       c->F, c->k, s);
+    tick();
+    x_now = next;
+    gemm(c->act, w.w_down, c->proj, rows, c->k, c->F, c->k, 0, 1);
+  }
+  // the closing norm (the stream, which a block leaves in x_alt, ends in c->x) and, where its GEMM is one of these too, the
+  // head behind it
+  void close32(const void *gain, int tap_mask, const void *head, int O, float *logits, int rows) {
+    const float *w[1] = {(const float *)head};
+    if (head && gemm_norm_ok(w, 1, (const float *)gain, rows, O, c->k)) {
+      mark(SPEC_PROF_GEMM);
+      launch_norm_gemm(x_now, c->proj, c->x, (float *)c->node_taps, tap_mask, (const float *)gain, c->cfg.rms_eps, w[0], logits, rows, O, c->k, s);
+      tick();
+      return;
+    }
+    cudaMemcpyAsync(c->x, x_now, (size_t)rows * c->k * 4, cudaMemcpyDeviceToDevice, s);
+    mark(SPEC_PROF_NORM);
+    launch_add_norm<float>(c->x, c->proj, 1, 0, 2, (float *)c->node_taps, tap_mask, (const float *)gain, c->cfg.rms_eps, (float *)c->h, nullptr, rows, rows, c->k, s);
+    tick();
+    if (head) gemm(c->h, head, logits, rows, O, c->k, O, 0, 1);
+  }
+
   int tap_mask_of(int layer) const {
     int m = 0;
     for (int i = 0; i < 3; i++) m |= (c->cfg.fuse_layers[i] == layer) ? (1 << i) : 0;
@@ -688,6 +745,21 @@ template <typename T> struct Sched {
   // plain schedule can leave the others out)
   void target_forward(int rows, int tail_len, bool want_logits, int only_row = -1) {
     if (c->fused) return target_forward_fused(rows, tail_len, want_logits);
+    if (norm_fused(rows)) {
+      mark(SPEC_PROF_MISC);
+      launch_rope_embed(c->meta.pos, c->inv_freq, c->cs, c->hd / 2, (const float *)c->embed, c->meta.tok, c->x, rows, c->k, s);
+      tick();
+      x_now = c->x;
+      for (int l = 0; l < c->L; l++) block32(c->tl[l], c->pools[l], rows, tail_len, l > 0, false, l == 0 ? 0 : tap_mask_of(l - 1));
+      const bool all = want_logits && only_row < 0;
+      close32(c->final_norm, tap_mask_of(c->L - 1), all ? c->lm_head : nullptr, c->V, c->logits, rows);
+      if (want_logits && !all) gemm((const T *)c->h + (size_t)only_row * c->k, c->lm_head, c->logits + (size_t)only_row * c->V, 1, c->V, c->k, c->V, 0, 1);
+      if (want_logits) {
+        const int r0 = all ? 0 : only_row;
+        mark(SPEC_PROF_ARGMAX); launch_argmax(c->logits + (size_t)r0 * c->V, all ? rows : 1, c->V, c->tb.y + r0, s); tick();
+      }
+      return;
+    }
     mark(SPEC_PROF_MISC); launch_rope_table(c->meta.pos, rows, c->hd / 2, c->inv_freq, c->cs, s); tick();
     mark(SPEC_PROF_MISC); launch_embed<T>((const T *)c->embed, c->meta.tok, c->x, rows, c->k, s); tick();
     for (int l = 0; l < c->L; l++)
@@ -711,9 +783,25 @@ template <typename T> struct Sched {
   }
 
   // draft head on the rows of c->meta: cat = [feat ; e(tok)], FC2, decoder block, final norm (-> h)
+  // logits: the draft LM head follows (draft_logits), which the fp32 schedule runs with the closing norm
   void draft_forward(const float *feat, int nparts, size_t fstride, const int32_t *src_row, int rows, int tail_len,
-                     bool prebuilt = false, bool pending = false) {
+                     bool prebuilt = false, bool pending = false, bool logits = false) {
     if (c->fused) return draft_forward_fused(feat, nparts, fstride, src_row, rows, tail_len, prebuilt, pending);
+    head_done = false;
+    if (nparts == 1 && norm_fused(rows)) {
+      mark(SPEC_PROF_MISC);
+      launch_rope_cat(c->meta.pos, c->inv_freq, c->cs, c->hd / 2, feat, src_row, (const float *)c->embed, c->meta.tok, c->meta.seq, (float *)c->cat, rows, c->k, s);
+      tick();
+      gemm(c->cat, c->fc2, c->proj, rows, c->k, 2 * c->k, c->k, 0, 1);
+      if (!logits) {               // prefill: of the draft layer only the cached K/V are used
+        block_qkv32(c->dl, c->pools[c->L], rows, false, true, 0);
+        return;
+      }
+      block32(c->dl, c->pools[c->L], rows, tail_len, false, true, 0);
+      close32(c->dfinal_norm, 0, c->dlm_head, c->Vd, c->logits, rows);
+      head_done = true;
+      return;
+    }
     mark(SPEC_PROF_MISC); launch_rope_table(c->meta.pos, rows, c->hd / 2, c->inv_freq, c->cs, s); tick();
     mark(SPEC_PROF_MISC); launch_build_cat<T>(feat, nparts, fstride, src_row, (const T *)c->embed, c->meta.tok, c->meta.seq, (T *)c->cat, rows, c->k, s);
     tick();
@@ -725,8 +813,10 @@ template <typename T> struct Sched {
     tick();
   }
 
+  bool head_done = false;        // the draft LM head ran with the closing norm
   void draft_logits(int rows) {
     if (c->fused) return draft_logits_fused(rows);
+    if (head_done) return;
     gemm(c->h, c->dlm_head, c->logits, rows, c->Vd, c->k, c->Vd, 0, 1);
   }
 
@@ -880,7 +970,7 @@ template <typename T> struct Sched {
       mark(SPEC_PROF_TREE); launch_prep_extend(c->st, c->tb, c->meta, c->B, c->need_pos, c->status, s); tick();
       c->cur_rps = c->Pmax;
       fuse(c->pend_taps, c->Te);
-      draft_forward(c->proj, c->np_proj, c->ps_proj, nullptr, c->Te, c->Pmax, false, true);
+      draft_forward(c->proj, c->np_proj, c->ps_proj, nullptr, c->Te, c->Pmax, false, true, true);
       if (c->tree_fused) {
         if (extend_compact()) draft_logits_topk(c->B, nullptr, 0);
         else draft_logits_topk(c->Te, c->st.last_row, c->B);
@@ -894,7 +984,7 @@ template <typename T> struct Sched {
       }
       for (int p = 2; p <= c->D; p++) {
         c->cur_rps = c->K;
-        draft_forward(c->x, 1, 0, c->tb.feat_row, c->Td, c->tail_tree, c->tree_fused);
+        draft_forward(c->x, 1, 0, c->tb.feat_row, c->Td, c->tail_tree, c->tree_fused, false, true);
         if (c->tree_fused) {
           draft_logits_topk(c->Td, nullptr, 0);
           capture(p, c->Td, false);

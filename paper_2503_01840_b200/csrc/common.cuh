@@ -170,6 +170,11 @@ void launch_gather_last(const int2 *fin, int nfin, const bf16 *taps, bf16 *pend_
 void launch_embed_half(const bf16 *embed, const int32_t *tok, bf16 *cat, int rows, int k, cudaStream_t s);
 void launch_residual_norm(const float *x, const bf16 *gain, bf16 *hb, float *ssq, int rows, int k, int ssq_ld, cudaStream_t s);
 
+// RoPE table and what a pass of the fp32 model starts from in one launch: x = E[tok], or cat = [feat[src_row] ; E[tok]]
+void launch_rope_embed(const int32_t *pos, const double *inv_freq, float2 *cs, int half, const float *embed, const int32_t *tok, float *x, int rows,
+                       int k, cudaStream_t s);
+void launch_rope_cat(const int32_t *pos, const double *inv_freq, float2 *cs, int half, const float *feat, const int32_t *src_row, const float *embed,
+                     const int32_t *tok, const int32_t *seq, float *cat, int rows, int k, cudaStream_t s);
 void launch_rope_table(const int32_t *pos, int rows, int half, const double *inv_freq, float2 *cs, cudaStream_t s);
 
 // qkv partial sums [nparts][rows][(H+2G)hd] fp32 -> q (T, [rows][H][hd], rotated) and K/V written into the
@@ -194,6 +199,18 @@ template <> void launch_gemm_ref<bf16>(const bf16 *x, const bf16 *w, float *out,
 // nw (2 or 3) weights that share the input, their outputs side by side in `out`; returns the number of kernels launched
 template <typename T>
 int launch_gemm_ref_cat(const T *x, const T *const (&w)[3], const int (&O)[3], int nw, float *out, int rows, int I, int ldo, cudaStream_t s);
+
+// fp32 model, few rows: RMSNorm of x + add (which is stored to x_out, and to the taps) in front of a GEMM,
+// with the plain result, RoPE + cache write, or SiLU(gate) * up behind it.  gemm_norm_ok: shapes and alignments it is taken for (O: all
+// features of the launch).  x_out must not be x.
+bool gemm_norm_ok(const float *const *w, int nw, const float *gain, int rows, int O, int I);
+void launch_norm_gemm(const float *x, const float *add, float *x_out, float *taps, int tap_mask, const float *gain, float eps, const float *w, float *out,
+                      int rows, int O, int I, cudaStream_t s);
+void launch_norm_swiglu(const float *x, const float *add, float *x_out, const float *gain, float eps, const float *w_gate, const float *w_up, float *act,
+                        int rows, int F, int I, cudaStream_t s);
+void launch_norm_qkv(const float *x, const float *add, float *x_out, float *taps, int tap_mask, const float *gain, float eps, const float *wq,
+                     const float *wk, const float *wv, const float2 *cs, RowMeta m, float *q, KvPool pool, PageMap pm, int rows, int H, int G, int hd,
+                     int I, int32_t *status, cudaStream_t s);
 
 // ---------------------------------------------------------------- launchers (attn_ref.cu)
 template <typename T>

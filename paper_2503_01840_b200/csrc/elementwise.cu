@@ -127,6 +127,46 @@ void launch_rope_table(const int32_t *pos, int rows, int half, const double *inv
   launch_k(rope_table_kernel, dim3((n + 255) / 256), dim3(256), 0, s, pos, rows, half, inv_freq, cs);
 }
 
+__device__ __forceinline__ void rope_row(int pos, const double *inv_freq, float2 *cs, int half) {
+  for (int i = threadIdx.x; i < half; i += blockDim.x) {
+    double sn, c;
+    sincos((double)pos * inv_freq[i], &sn, &c);
+    cs[i] = make_float2((float)c, (float)sn);
+  }
+}
+__global__ void rope_embed_kernel(const int32_t *__restrict__ pos, const double *__restrict__ inv_freq, float2 *__restrict__ cs, int half,
+                                  const float *__restrict__ embed, const int32_t *__restrict__ tok, float *__restrict__ x, int k) {
+  pdl_wait();
+  pdl_trigger();
+  const int r = blockIdx.x;
+  const float *e = embed + (size_t)tok[r] * k;
+  for (int i = threadIdx.x; i < k; i += blockDim.x) x[(size_t)r * k + i] = e[i];
+  rope_row(pos[r], inv_freq, cs + (size_t)r * half, half);
+}
+void launch_rope_embed(const int32_t *pos, const double *inv_freq, float2 *cs, int half, const float *embed, const int32_t *tok, float *x, int rows,
+                       int k, cudaStream_t s) {
+  launch_k(rope_embed_kernel, dim3(rows), dim3(256), 0, s, pos, inv_freq, cs, half, embed, tok, x, k);
+}
+__global__ void rope_cat_kernel(const int32_t *__restrict__ pos, const double *__restrict__ inv_freq, float2 *__restrict__ cs, int half,
+                                const float *__restrict__ feat, const int32_t *__restrict__ src_row, const float *__restrict__ embed,
+                                const int32_t *__restrict__ tok, const int32_t *__restrict__ seq, float *__restrict__ cat, int k) {
+  pdl_wait();
+  pdl_trigger();
+  const int r = blockIdx.x;
+  const bool valid = seq[r] >= 0;
+  const int sr = !valid ? 0 : src_row ? src_row[r] : r, t = valid ? tok[r] : 0;
+  float *c = cat + (size_t)r * 2 * k;
+  for (int i = threadIdx.x; i < k; i += blockDim.x) {
+    c[i] = valid ? feat[(size_t)sr * k + i] : 0.0f;
+    c[k + i] = valid ? embed[(size_t)t * k + i] : 0.0f;
+  }
+  rope_row(pos[r], inv_freq, cs + (size_t)r * half, half);
+}
+void launch_rope_cat(const int32_t *pos, const double *inv_freq, float2 *cs, int half, const float *feat, const int32_t *src_row, const float *embed,
+                     const int32_t *tok, const int32_t *seq, float *cat, int rows, int k, cudaStream_t s) {
+  launch_k(rope_cat_kernel, dim3(rows), dim3(256), 0, s, pos, inv_freq, cs, half, feat, src_row, embed, tok, seq, cat, k);
+}
+
 // ---------------------------------------------------------------- row metadata of one prefill pass
 // Row r < nvalid is prompt position start + r of sequence b, fed with toks[r]; a pass is made of blocks of `block`
 // positions: the rows of a block are each other's tail keys (causal through the two-word masks), everything before the

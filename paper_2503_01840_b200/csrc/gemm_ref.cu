@@ -115,6 +115,142 @@ __global__ void __launch_bounds__(128) gemm_skinny_kernel(const float *__restric
   }
 }
 
+// The same kernel with what surrounds it in a decoder layer: RMSNorm on the way in (the pending partial result is added to the
+// residual stream, the norm's factor is applied to the finished sums, the sum of squares comes out of the same loop) and RoPE
+// with the cache write, or SiLU(gate) * up, on the way out.  A warp's features come in pairs (rotation partners j and j + hd / 2
+// of a head, gate and up), which end in neighbouring lanes.  The new residual row goes to a buffer of its own (the last block of a
+// row group does nothing else): other blocks still read the old one.  A step of the tiny model is a chain of dependent launches of 2 to
+// 3 us each, so what counts is their number: five a layer instead of nine,
+// 48 a step instead of 76: a request of ten steps 3.06 -> 2.76 ms.  (With a branch per row around the added partial result, and the cache
+// slot looked up in front of the loop, it was 3.34: every load must be on its way before the first is used.)
+struct NormIn {
+  const float *x, *add;        // [rows][I]; add may be null
+  float *x_out, *taps;         // x + add (may be null: unchanged); feature taps [rows][3 I], slots by tap_mask
+  int tap_mask;
+  const float *gain;
+  float eps;
+};
+enum { NOUT_PLAIN = 0, NOUT_QKV = 1, NOUT_SWIGLU = 2 };
+struct NormOut {
+  float *out; int ldo;                                   // NOUT_PLAIN; NOUT_SWIGLU: act [rows][pairs]
+  const float2 *cs; RowMeta m; float *q, *kp, *vp; PageMap pm; int H, G, hd; int32_t *status;   // NOUT_QKV
+};
+template <int R, int C, int OUT, bool ADD>
+__global__ void __launch_bounds__(128) gemm_norm_kernel(NormIn in, SkinnyWeights sw, NormOut no, int rows, int O, int I) {
+  pdl_wait();
+  pdl_trigger();
+  constexpr int NV = R * C, P = C / 2;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int r0 = blockIdx.y * R;
+  const int u0 = (blockIdx.x * 4 + warp) * (OUT == NOUT_PLAIN ? C : P), units = OUT == NOUT_PLAIN ? O : O / 2;    // features, or pairs of features
+  if (blockIdx.x + 1 == gridDim.x) {                   // the new residual rows and the taps: the last block of the row group
+    if (in.x_out || in.tap_mask)
+      for (int i = threadIdx.x; i < min(R, rows - r0) * (I / 4); i += 128) {
+        const int r = r0 + i / (I / 4), k = i % (I / 4) * 4;
+        const size_t at = (size_t)r * I + k;
+        float4 a = *(const float4 *)(in.x + at);
+        if (ADD) { const float4 b = *(const float4 *)(in.add + at); a.x += b.x; a.y += b.y; a.z += b.z; a.w += b.w; }
+        if (in.x_out) *(float4 *)(in.x_out + at) = a;
+#pragma unroll
+        for (int s = 0; s < 3; s++)
+          if ((in.tap_mask >> s) & 1) *(float4 *)(in.taps + (size_t)r * 3 * I + (size_t)s * I + k) = a;
+      }
+    return;
+  }
+  if (u0 >= units) return;
+  const int half = OUT == NOUT_QKV ? no.hd >> 1 : 1;
+  const float *wr[C];
+#pragma unroll
+  for (int c = 0; c < C; c++) {
+    const int u = min(u0 + (OUT == NOUT_PLAIN ? c : c % P), units - 1);           // past the end: repeats the last (not stored)
+    const int o = OUT == NOUT_PLAIN ? u : OUT == NOUT_QKV ? u / half * no.hd + u % half + (c >= P ? half : 0) : u + (c >= P ? units : 0);
+    wr[c] = o < sw.o1 ? sw.w0 + (size_t)o * I : o < sw.o2 ? sw.w1 + (size_t)(o - sw.o1) * I : sw.w2 + (size_t)(o - sw.o2) * I;
+  }
+  // where this lane's value goes: row rl of the group, feature (or pair member) lane % C; 64 values: row = lane, both members
+  const int rl = NV == 32 ? lane / C : lane, c_own = NV == 32 ? lane % C : 0;
+  const int row = r0 + rl, unit = u0 + (OUT == NOUT_PLAIN ? c_own : c_own % P);
+  const bool mine = row < rows && unit < units;
+  float2 cs = make_float2(1.0f, 0.0f);
+  int head = 0, seq = -1, kvpos = 0;
+  if (OUT == NOUT_QKV && mine) {                       // not used before the sums are there
+    head = unit / half;
+    seq = no.m.seq[row];
+    kvpos = no.m.kvpos[row];
+    if (head < no.H + no.G) cs = no.cs[(size_t)row * half + unit % half];
+  }
+  float v[NV], sq[R];
+#pragma unroll
+  for (int e = 0; e < NV; e++) v[e] = 0.0f;
+#pragma unroll
+  for (int r = 0; r < R; r++) sq[r] = 0.0f;
+#pragma unroll 1
+  for (int k = lane * 4; k < I; k += 128) {           // I % 4 == 0
+    float4 w[C];
+#pragma unroll
+    for (int c = 0; c < C; c++) w[c] = *(const float4 *)(wr[c] + k);
+    const float4 g = *(const float4 *)(in.gain + k);
+#pragma unroll
+    for (int r = 0; r < R; r++) {
+      const size_t at = (size_t)min(r0 + r, rows - 1) * I + k;
+      float4 a = *(const float4 *)(in.x + at);
+      if (ADD) { const float4 b = *(const float4 *)(in.add + at); a.x += b.x; a.y += b.y; a.z += b.z; a.w += b.w; }
+      sq[r] = fmaf(a.x, a.x, fmaf(a.y, a.y, fmaf(a.z, a.z, fmaf(a.w, a.w, sq[r]))));
+      a.x *= g.x; a.y *= g.y; a.z *= g.z; a.w *= g.w;
+#pragma unroll
+      for (int c = 0; c < C; c++) v[r * C + c] = fmaf(a.x, w[c].x, fmaf(a.y, w[c].y, fmaf(a.z, w[c].z, fmaf(a.w, w[c].w, v[r * C + c]))));
+    }
+  }
+  int page = -1;                                       // cache page of the row, on its way during the exchange
+  const bool in_cache = OUT == NOUT_QKV && mine && seq >= 0 && head >= no.H;
+  if (in_cache) {
+    if (kvpos < 0 || kvpos / no.pm.page_size >= no.pm.pages_per_seq) { set_status(no.status, ST_BOUNDS, 1, row, kvpos); page = -2; }
+    else page = no.pm.table[(size_t)seq * no.pm.pages_per_seq + kvpos / no.pm.page_size];
+  }
+  // halving exchange of the sums (cf. gemm_skinny_kernel), and of the squares down to the lane's own row
+#pragma unroll
+  for (int step = 0; step < 5; step++) {
+    const int off = 16 >> step, hv = NV >> (step + 1), hr = R >> (step + 1);
+    const bool up = lane & off;
+#pragma unroll
+    for (int i = 0; i < hv; i++) {
+      const float keep = up ? v[i + hv] : v[i], send = up ? v[i] : v[i + hv];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+    }
+    if (hr >= 1) {
+#pragma unroll
+      for (int i = 0; i < hr; i++) {
+        const float keep = up ? sq[i + hr] : sq[i], send = up ? sq[i] : sq[i + hr];
+        sq[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+      }
+    } else sq[0] += __shfl_xor_sync(0xffffffffu, sq[0], off);
+  }
+  const float inv = 1.0f / sqrtf(sq[0] / (float)I + in.eps);
+  if (OUT == NOUT_PLAIN) {
+#pragma unroll
+    for (int i = 0; i < NV / 32; i++)
+      if (row < rows && u0 + c_own + i < units) no.out[(size_t)row * no.ldo + u0 + c_own + i] = v[i] * inv;
+    return;
+  }
+  // a: first member of the pair (feature j, gate), b: second (j + hd / 2, up)
+  const float own = v[0] * inv, other = NV == 32 ? __shfl_xor_sync(0xffffffffu, own, P) : v[NV / 32 - 1] * inv;
+  const bool second = NV == 32 && c_own >= P;
+  const float a = second ? other : own, b = second ? own : other;
+  if (mine && OUT == NOUT_SWIGLU && !second) no.out[(size_t)row * units + unit] = (a / (1.0f + expf(-a))) * b;
+  if (OUT == NOUT_SWIGLU || !mine) return;
+  const int j = unit % half;
+  float *kv = nullptr;
+  if (in_cache && page != -2) {
+    if (page < 0 || page >= no.pm.num_pages) set_status(no.status, ST_BOUNDS, 2, row, page);
+    else kv = (head < no.H + no.G ? no.kp : no.vp) + (((size_t)page * no.G + (head - no.H) % no.G) * no.pm.page_size + kvpos % no.pm.page_size) * no.hd;
+  }
+  float *dst = head < no.H ? no.q + ((size_t)row * no.H + head) * no.hd : kv;
+  if (!dst) return;
+  float oa = a * cs.x - b * cs.y, ob = b * cs.x + a * cs.y;
+  if (head < no.H && seq < 0) oa = ob = 0.0f;           // padding row
+  if (!second) dst[j] = oa;
+  if (second || NV != 32) dst[j + half] = ob;
+}
+
 // When the warp-per-feature kernel is taken: up to 32 rows every weight is read once; up to 256 rows while the weights fit the
 // L2 comfortably (they are read once per 32 rows); and in either case only where it is the shorter one.  Its time goes with
 // (rows padded to a group) x features x (contraction + 192: the exchange costs as much as 192 elements), spread over the chip
@@ -135,6 +271,40 @@ static void launch_skinny(const float *x, SkinnyWeights sw, float *out, int rows
   else if (rows <= 8) go(gemm_skinny_kernel<8, 4>, 8, 4);
   else if (rows <= 16) go(gemm_skinny_kernel<16, 2>, 16, 2);
   else go(gemm_skinny_kernel<32, 2>, 32, 2);
+}
+
+template <int OUT>
+static void launch_norm(const NormIn &in, const SkinnyWeights &sw, const NormOut &no, int rows, int O, int I, cudaStream_t s) {
+  auto go = [&](auto kern, int R, int C) { launch_k(kern, dim3((O + 4 * C - 1) / (4 * C) + 1, (rows + R - 1) / R), dim3(128), 0, s, in, sw, no, rows, O, I); };
+  auto pick = [&](auto k4, auto k8, auto k16, auto k32) {
+    if (rows <= 4) go(k4, 4, 8);
+    else if (rows <= 8) go(k8, 8, 4);
+    else if (rows <= 16) go(k16, 16, 2);
+    else go(k32, 32, 2);
+  };
+  if (in.add) pick(gemm_norm_kernel<4, 8, OUT, true>, gemm_norm_kernel<8, 4, OUT, true>, gemm_norm_kernel<16, 2, OUT, true>, gemm_norm_kernel<32, 2, OUT, true>);
+  else pick(gemm_norm_kernel<4, 8, OUT, false>, gemm_norm_kernel<8, 4, OUT, false>, gemm_norm_kernel<16, 2, OUT, false>, gemm_norm_kernel<32, 2, OUT, false>);
+}
+bool gemm_norm_ok(const float *const *w, int nw, const float *gain, int rows, int O, int I) {
+  if ((uintptr_t)gain & 15) return false;
+  for (int j = 0; j < nw; j++)
+    if (!skinny_ok(nullptr, w[j], rows, O, I)) return false;
+  return true;
+}
+void launch_norm_gemm(const float *x, const float *add, float *x_out, float *taps, int tap_mask, const float *gain, float eps, const float *w, float *out,
+                      int rows, int O, int I, cudaStream_t s) {
+  launch_norm<NOUT_PLAIN>(NormIn{x, add, x_out, taps, tap_mask, gain, eps}, SkinnyWeights{w, w, w, O, O}, NormOut{out, O}, rows, O, I, s);
+}
+void launch_norm_swiglu(const float *x, const float *add, float *x_out, const float *gain, float eps, const float *w_gate, const float *w_up, float *act,
+                        int rows, int F, int I, cudaStream_t s) {
+  launch_norm<NOUT_SWIGLU>(NormIn{x, add, x_out, nullptr, 0, gain, eps}, SkinnyWeights{w_gate, w_up, w_up, F, 2 * F}, NormOut{act, F}, rows, 2 * F, I, s);
+}
+void launch_norm_qkv(const float *x, const float *add, float *x_out, float *taps, int tap_mask, const float *gain, float eps, const float *wq,
+                     const float *wk, const float *wv, const float2 *cs, RowMeta m, float *q, KvPool pool, PageMap pm, int rows, int H, int G, int hd,
+                     int I, int32_t *status, cudaStream_t s) {
+  const int o1 = H * hd, o2 = o1 + G * hd;
+  launch_norm<NOUT_QKV>(NormIn{x, add, x_out, taps, tap_mask, gain, eps}, SkinnyWeights{wq, wk, wv, o1, o2},
+                        NormOut{nullptr, 0, cs, m, q, (float *)pool.k, (float *)pool.v, pm, H, G, hd, status}, rows, o2 + G * hd, I, s);
 }
 
 template <typename T>

@@ -1,0 +1,54 @@
+"""The fp32 model's schedule with norms, RoPE, cache writes and activations on the GEMMs: every row group of those kernels (4, 8, 16,
+32 rows and several groups), head dimensions and feature counts off the warps' shares, padding rows, taps, against the CPU oracle;
+weights off a 16-byte boundary stay on the plain schedule and agree with it."""
+import numpy as np
+import pytest
+
+import parity
+from paper_2503_01840_b200 import binding as sb
+from paper_2503_01840_b200 import synth
+
+pytestmark = pytest.mark.gpu
+
+BASE = synth.ModelCfg("F", "fp32", 3, 72, 3, 1, 48, 200, 131, 77, (0, 1, 2), 5e5, tree_depth=3, tree_topk=2, tree_nodes=7, seed=23)
+
+
+@pytest.mark.parametrize("kw,batch", [
+    (dict(), 1),                                                       # 4, 2 and 7 rows
+    (dict(tree_topk=4, tree_nodes=16), 1),                             # 16 rows
+    (dict(n_heads=4, n_kv_heads=2, head_dim=16, ffn=136, tree_topk=5, tree_nodes=29), 1),     # 29 rows
+    (dict(tree_depth=2, tree_topk=3, tree_nodes=11), 3),               # 9, 9 and 33 rows: a second group of one row
+    (dict(hidden=256, n_heads=2, n_kv_heads=2, head_dim=80, ffn=688, tree_depth=4, tree_nodes=12), 5),   # 25, 10 and 60 rows
+], ids=str)
+def test_fp32_schedule_vs_oracle(kw, batch):
+    cfg = BASE.replace(batch=batch, prompt_lo=5, prompt_hi=70, prompt_len=37, **kw)
+    tw, dw = synth.make_target_weights(cfg), synth.make_draft_weights(cfg)
+    prompts = [p.numpy() for p in synth.make_prompts(cfg)]
+    st, _ = parity.run_trajectory(cfg, tw, dw, prompts, n_steps=4, tol=1e-4)
+    assert st.passes == 4 * cfg.tree_depth * batch and st.verify_compared == 4 * batch, st
+
+
+def test_fp32_unaligned_norm_weights():
+    """Norm gains off a 16-byte boundary take the plain schedule; both are fp32 sums of the same products."""
+    import torch
+    cfg = BASE.replace(hidden=256, n_heads=4, n_kv_heads=2, head_dim=64, tree_nodes=12)
+    tw, dw = synth.make_target_weights(cfg, device="cuda"), synth.make_draft_weights(cfg, device="cuda")
+
+    def shifted(t):
+        buf = torch.empty(t.numel() + 1, device="cuda")
+        buf[1:].copy_(t.view(-1))
+        return buf[1:].view(t.shape)
+
+    def off_grid(w):
+        return {k: [off_grid(x) for x in v] if isinstance(v, list) else shifted(v) if "norm" in k else v for k, v in w.items()}
+
+    prompt, hidden = [np.arange(40, dtype=np.int32) % cfg.vocab], []
+    for t, d in ((tw, dw), (off_grid(tw), off_grid(dw))):
+        dec = sb.SpecDecoder(cfg, t, d, batch=1, max_ctx=160)
+        dec.prefill(prompt, 16)
+        dec.step()
+        hidden.append((dec.debug(sb.DBG_TREE_TOK), dec.debug(sb.DBG_NODE_HIDDEN)))
+        dec.close()
+    assert np.array_equal(hidden[0][0], hidden[1][0])
+    a, b = hidden[0][1].astype(np.float64), hidden[1][1].astype(np.float64)
+    assert np.abs(a - b).max() <= 2e-5 * np.sqrt((b * b).mean())         # sums of up to 400 products, three layers deep
