@@ -67,14 +67,17 @@ __global__ void __launch_bounds__(256) gemm_ref_kernel(const T *__restrict__ x, 
 // Several weights that share the input run in one launch (q, k, v; gate, up): feature o belongs to w0 below o1, to w1 below
 // o2, else to w2.
 struct SkinnyWeights { const float *w0, *w1, *w2; int o1, o2; };
-template <int R, int C>
+// KS: the block's four warps take the same features and a quarter of the contraction each (added up through shared memory): a
+// warp then walks 128 elements of every 512 instead of all.  Taken from 384 elements on (three dependent steps of loads) while the
+// blocks, four times as many, are resident together (8 a SM).  Tiny request of ten steps 2.76 -> 2.48 ms.
+template <int R, int C, bool KS>
 __global__ void __launch_bounds__(128) gemm_skinny_kernel(const float *__restrict__ x, SkinnyWeights sw, float *__restrict__ out, int rows,
                                                           int O, int I, int ldo) {
   pdl_wait();
   pdl_trigger();
   constexpr int NV = R * C;
   const int lane = threadIdx.x & 31;
-  const int o0 = (blockIdx.x * 4 + (threadIdx.x >> 5)) * C, r0 = blockIdx.y * R;
+  const int warp = threadIdx.x >> 5, o0 = (KS ? blockIdx.x : blockIdx.x * 4 + warp) * C, r0 = blockIdx.y * R;
   if (o0 >= O) return;
   const float *wr[C];
 #pragma unroll
@@ -86,7 +89,7 @@ __global__ void __launch_bounds__(128) gemm_skinny_kernel(const float *__restric
 #pragma unroll
   for (int e = 0; e < NV; e++) v[e] = 0.0f;
 #pragma unroll 2
-  for (int k = lane * 4; k < I; k += 128) {           // I % 4 == 0
+  for (int k = (KS ? warp * 128 : 0) + lane * 4; k < I; k += KS ? 512 : 128) {        // I % 4 == 0
     float4 w[C];
 #pragma unroll
     for (int c = 0; c < C; c++) w[c] = *(const float4 *)(wr[c] + k);
@@ -106,6 +109,19 @@ __global__ void __launch_bounds__(128) gemm_skinny_kernel(const float *__restric
     for (int i = 0; i < half; i++) {
       const float keep = up ? v[i + half] : v[i], send = up ? v[i] : v[i + half];
       v[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+    }
+  }
+  if constexpr (KS) {
+    __shared__ float part[3][NV];
+    if (warp)
+#pragma unroll
+      for (int i = 0; i < NV / 32; i++) part[warp - 1][lane * (NV / 32) + i] = v[i];
+    __syncthreads();
+    if (warp) return;
+#pragma unroll
+    for (int i = 0; i < NV / 32; i++) {
+      const int e = lane * (NV / 32) + i;
+      v[i] = (v[i] + part[0][e]) + (part[1][e] + part[2][e]);
     }
   }
 #pragma unroll
@@ -266,11 +282,15 @@ static bool skinny_ok(const float *x, const float *w, int rows, int O, int I) {
   return (double)padded * O * (I + 192) <= 1.31e6 * I * std::max(1.0, tiles / 256);
 }
 static void launch_skinny(const float *x, SkinnyWeights sw, float *out, int rows, int O, int I, int ldo, cudaStream_t s) {
-  auto go = [&](auto kern, int R, int C) { launch_k(kern, dim3((O + 4 * C - 1) / (4 * C), (rows + R - 1) / R), dim3(128), 0, s, x, sw, out, rows, O, I, ldo); };
-  if (rows <= 4) go(gemm_skinny_kernel<4, 8>, 4, 8);
-  else if (rows <= 8) go(gemm_skinny_kernel<8, 4>, 8, 4);
-  else if (rows <= 16) go(gemm_skinny_kernel<16, 2>, 16, 2);
-  else go(gemm_skinny_kernel<32, 2>, 32, 2);
+  auto go = [&](auto kern, auto split, int R, int C) {
+    const int groups = (rows + R - 1) / R;
+    if (I >= 384 && (O + C - 1) / C * groups <= 1184) launch_k(split, dim3((O + C - 1) / C, groups), dim3(128), 0, s, x, sw, out, rows, O, I, ldo);
+    else launch_k(kern, dim3((O + 4 * C - 1) / (4 * C), groups), dim3(128), 0, s, x, sw, out, rows, O, I, ldo);
+  };
+  if (rows <= 4) go(gemm_skinny_kernel<4, 8, false>, gemm_skinny_kernel<4, 8, true>, 4, 8);
+  else if (rows <= 8) go(gemm_skinny_kernel<8, 4, false>, gemm_skinny_kernel<8, 4, true>, 8, 4);
+  else if (rows <= 16) go(gemm_skinny_kernel<16, 2, false>, gemm_skinny_kernel<16, 2, true>, 16, 2);
+  else go(gemm_skinny_kernel<32, 2, false>, gemm_skinny_kernel<32, 2, true>, 32, 2);
 }
 
 template <int OUT>

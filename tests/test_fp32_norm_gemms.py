@@ -52,3 +52,17 @@ def test_fp32_unaligned_norm_weights():
     assert np.array_equal(hidden[0][0], hidden[1][0])
     a, b = hidden[0][1].astype(np.float64), hidden[1][1].astype(np.float64)
     assert np.abs(a - b).max() <= 2e-5 * np.sqrt((b * b).mean())         # sums of up to 400 products, three layers deep
+
+
+@pytest.mark.parametrize("rows", [1, 4, 5, 16, 17, 33])
+@pytest.mark.parametrize("O,I", [(33, 380), (33, 384), (250, 388), (2, 516), (70, 1028), (1184, 640), (4744, 512)])
+def test_fp32_gemm_contraction_over_warps(rows, O, I):
+    """Contractions around the length from which a block's warps share them, remainders of the 512 elements they take at a time,
+    and feature counts on both sides of the blocks that are resident together."""
+    import torch
+    g = torch.Generator().manual_seed(rows + O + I)
+    x, w = torch.randn(rows, I, generator=g), torch.randn(O, I, generator=g)
+    out = sb.gemm(x.cuda(), w.cuda(), impl=1).cpu().double().numpy()
+    xd, wd = x.double().numpy(), w.double().numpy()
+    bound = 2.0 ** -23 * (8 + I / 32) * (np.abs(xd) @ np.abs(wd).T)     # lane sums of up to I / 32 products, then eight exchanges
+    assert (np.abs(out - xd @ wd.T) <= bound + 1e-30).all()
