@@ -694,8 +694,8 @@ __global__ void __launch_bounds__(UM_THREADS, 1) attn_umma_kernel(const __grid_c
   const int32_t *tbl = p.pm.table + (size_t)(seq >= 0 ? seq : 0) * p.pm.pages_per_seq;
   const int ppt = KT / ps;                             // pages per tile
   int cur[4] = {-1, -1, -1, -1}, nxt[4] = {-1, -1, -1, -1}, fallback = 0, i_load = 0;
+  auto next_pages = [&](int i) { if (i + 1 < ntl) tile_pages(nxt, tbl, p.pm.pages_per_seq, t_begin + i + 1, ps); };    // before the wait for a free stage
   auto load_tile = [&](int i) {                        // converged warp; page ids of tile i in cur
-    if (i + 1 < ntl) tile_pages(nxt, tbl, p.pm.pages_per_seq, t_begin + i + 1, ps);
     if (elect_one()) {
       const int st = i % UM_STAGES;
       unsigned char *kb = ring + st * 2 * UM_TILE, *vb = kb + UM_TILE;
@@ -722,7 +722,7 @@ __global__ void __launch_bounds__(UM_THREADS, 1) attn_umma_kernel(const __grid_c
     if (seq >= 0 && ntl > 0) {
       fallback = tbl[0];                               // keys past the last page are masked; they still need a valid source
       tile_pages(cur, tbl, p.pm.pages_per_seq, t_begin, ps);
-      for (; i_load < ntl && i_load < UM_STAGES && (t_begin + i_load + 1) * KT <= ctx_early; i_load++) load_tile(i_load);
+      for (; i_load < ntl && i_load < UM_STAGES && (t_begin + i_load + 1) * KT <= ctx_early; i_load++) { next_pages(i_load); load_tile(i_load); }
     }
   }
   if (warp == 0) {
@@ -766,6 +766,7 @@ __global__ void __launch_bounds__(UM_THREADS, 1) attn_umma_kernel(const __grid_c
     pdl_wait();
     if (seq >= 0)       // the whole warp walks the loop, the elected lane issues the copies
       for (; i_load < ntl; i_load++) {
+        next_pages(i_load);
         if (i_load >= UM_STAGES && !mbar_wait_warp(&empty[i_load % UM_STAGES], (uint32_t)(((i_load / UM_STAGES) - 1) & 1))) {
           *abort_flag = 1;
           if (status) set_status(status, ST_TIMEOUT, 420, blockIdx.z, t_begin + i_load);
@@ -1016,9 +1017,10 @@ __global__ void __launch_bounds__(160, HD == 128 ? 3 : 1) attn_tma_small_kernel(
   const int32_t *tbl = p.pm.table + (size_t)(seq >= 0 ? seq : 0) * p.pm.pages_per_seq;
   const int ppt = KT / ps;                             // pages per tile
   int cur[4] = {-1, -1, -1, -1}, nxt[4] = {-1, -1, -1, -1}, fallback = 0, t_load = t_begin;
+  // the next tile's page ids are asked for before the wait for a free stage: behind it they would hold up the copy after this one
+  auto next_pages = [&](int t) { if (t + 1 < t_end) tile_pages(nxt, tbl, p.pm.pages_per_seq, t + 1, ps); };
   auto load_tile = [&](int t) {                        // converged warp; page ids of tile t in cur
     const int st = (t - t_begin) % STAGES;
-    if (t + 1 < t_end) tile_pages(nxt, tbl, p.pm.pages_per_seq, t + 1, ps);
     if (elect_one()) {
       unsigned char *kb = sm + st * 2 * TILEB, *vb = kb + TILEB;
       mbar_expect_tx(&full[st], 2 * TILEB);
@@ -1045,7 +1047,7 @@ __global__ void __launch_bounds__(160, HD == 128 ? 3 : 1) attn_tma_small_kernel(
     if (seq >= 0 && t_begin < t_end) {
       fallback = tbl[0];                               // keys past the last page are masked; they still need a valid source
       tile_pages(cur, tbl, p.pm.pages_per_seq, t_begin, ps);
-      for (; t_load < t_end && t_load < t_begin + STAGES && (t_load + 1) * KT <= ctx_early; t_load++) load_tile(t_load);
+      for (; t_load < t_end && t_load < t_begin + STAGES && (t_load + 1) * KT <= ctx_early; t_load++) { next_pages(t_load); load_tile(t_load); }
     }
   }
   const int mA = lane >> 2, mB = mA + 8;
@@ -1073,6 +1075,7 @@ __global__ void __launch_bounds__(160, HD == 128 ? 3 : 1) attn_tma_small_kernel(
     if (seq >= 0)       // the whole warp walks the loop, the elected lane issues the copies
       for (; t_load < t_end; t_load++) {
         const int i = t_load - t_begin;
+        next_pages(t_load);
         if (i >= STAGES && !mbar_wait_warp(&empty[i % STAGES], (uint32_t)(((i / STAGES) - 1) & 1))) { if (status) set_status(status, ST_TIMEOUT, 411, blockIdx.z, t_load); break; }
         load_tile(t_load);
       }
