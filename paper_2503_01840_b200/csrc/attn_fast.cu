@@ -979,8 +979,9 @@ __global__ void __launch_bounds__(UM_THREADS, 1) attn_umma_kernel(const __grid_c
 // the four consumer warps share the rows and split the KEYS of every 64-key tile (16 keys each); each keeps its own
 // online-softmax state and the four states are merged through shared memory at the end.
 // At batch this kernel streams the cache, and a stage is only refilled when its tile has been consumed, so the time per tile
-// counts: context tiles take no masks, O is rescaled only when a maximum moved, 2^x is the special-function unit's; three CTAs
-// share an SM (hence the bound on registers).  64 chains of 256..2048 tokens: 81.7 -> 73.1 us a layer; 56 chains 68.9 -> 59.7.
+// counts: context tiles take no masks, O is rescaled only when a maximum moved; three CTAs share an SM (hence the bound on
+// registers).  64 chains of 256..2048 tokens: 81.7 -> 73.1 us a layer; 56 chains 68.9 -> 59.7.  2^x is exp2f throughout: a factor
+// below 2^-126 still counts where the values it meets are large, and the merges below and in attn_combine_kernel use it too.
 template <int HD, int STAGES>
 __global__ void __launch_bounds__(160, HD == 128 ? 3 : 1) attn_tma_small_kernel(const __grid_constant__ CUtensorMap map_k,
                                                              const __grid_constant__ CUtensorMap map_v, AttnParams p, int32_t *status) {
@@ -1130,14 +1131,14 @@ __global__ void __launch_bounds__(160, HD == 128 ? 3 : 1) attn_tma_small_kernel(
       tmA = fmaxf(tmA, __shfl_xor_sync(0xffffffffu, tmA, 1)); tmA = fmaxf(tmA, __shfl_xor_sync(0xffffffffu, tmA, 2));
       tmB = fmaxf(tmB, __shfl_xor_sync(0xffffffffu, tmB, 1)); tmB = fmaxf(tmB, __shfl_xor_sync(0xffffffffu, tmB, 2));
       float nmA = fmaxf(mxA, tmA), nmB = fmaxf(mxB, tmB);
-      float fA = (nmA == -INFINITY) ? 1.0f : ex2_approx((mxA - nmA) * sc), fB = (nmB == -INFINITY) ? 1.0f : ex2_approx((mxB - nmB) * sc);
+      float fA = (nmA == -INFINITY) ? 1.0f : exp2f((mxA - nmA) * sc), fB = (nmB == -INFINITY) ? 1.0f : exp2f((mxB - nmB) * sc);
       float baseA = (nmA == -INFINITY) ? 0.0f : nmA, baseB = (nmB == -INFINITY) ? 0.0f : nmB;
       float rsA = 0.0f, rsB = 0.0f;
       uint32_t pf[4];
 #pragma unroll
       for (int n = 0; n < 2; n++) {
-        float p0 = ex2_approx((s[n][0] - baseA) * sc), p1 = ex2_approx((s[n][1] - baseA) * sc);
-        float p2 = ex2_approx((s[n][2] - baseB) * sc), p3 = ex2_approx((s[n][3] - baseB) * sc);
+        float p0 = exp2f((s[n][0] - baseA) * sc), p1 = exp2f((s[n][1] - baseA) * sc);
+        float p2 = exp2f((s[n][2] - baseB) * sc), p3 = exp2f((s[n][3] - baseB) * sc);
         rsA += p0 + p1; rsB += p2 + p3;
         pf[n * 2] = pack_bf16(p0, p1);
         pf[n * 2 + 1] = pack_bf16(p2, p3);
