@@ -979,11 +979,14 @@ __global__ void __launch_bounds__(UM_THREADS, 1) attn_umma_kernel(const __grid_c
 // the four consumer warps share the rows and split the KEYS of every 64-key tile (16 keys each); each keeps its own
 // online-softmax state and the four states are merged through shared memory at the end.
 // At batch this kernel streams the cache, and a stage is only refilled when its tile has been consumed, so the time per tile
-// counts: context tiles take no masks, O is rescaled only when a maximum moved; three CTAs share an SM (hence the bound on
-// registers).  64 chains of 256..2048 tokens: 81.7 -> 73.1 us a layer; 56 chains 68.9 -> 59.7.  2^x is exp2f throughout: a factor
-// below 2^-126 still counts where the values it meets are large, and the merges below and in attn_combine_kernel use it too.
+// counts: context tiles take no masks, O is rescaled only when a maximum moved.  2^x is exp2f throughout: a factor below 2^-126
+// still counts where the values it meets are large, and the merges below and in attn_combine_kernel use it too.
+// The bound of two CTAs per SM keeps it at 166 registers (unbounded it takes 176, of which a quarter of the register file holds two
+// warps: one CTA per SM).  Three CTAs fit at 128 registers with spills, and lose at every batch but the largest: verify pass of
+// n chains of four rows, 256..2048 tokens, 8B shapes in the replayed step, us a layer with three / two CTAs per SM: n = 8 29.9 / 23.3,
+// 16 45.8 / 34.3, 32 48.4 / 39.1, 48 55.2 / 47.8, 64 63.6 / 64.0; 56 chains of three rows 57.7 / 55.3; draft passes of 64 rows 58.4 / 54.0.
 template <int HD, int STAGES>
-__global__ void __launch_bounds__(160, HD == 128 ? 3 : 1) attn_tma_small_kernel(const __grid_constant__ CUtensorMap map_k,
+__global__ void __launch_bounds__(160, HD == 128 ? 2 : 1) attn_tma_small_kernel(const __grid_constant__ CUtensorMap map_k,
                                                              const __grid_constant__ CUtensorMap map_v, AttnParams p, int32_t *status) {
   pdl_trigger();   // the next kernel may start staging its weights; it still waits for this grid to complete
   KernelStamp stamp_guard(p.stamp, false);
@@ -1353,7 +1356,7 @@ bool diag_map(CUtensorMap *out, const void *kd, int J, int T, int G, int box_row
 namespace {
 template <int HD>
 int launch_tma_small(AttnParams &p, dim3 grid, const CUtensorMap *mk, const CUtensorMap *mv, int32_t *status, cudaStream_t s) {
-  // two stages at head_dim 128 (68 KB): three CTAs share an SM and hide each other's prologue and merge, and the next
+  // two stages at head_dim 128 (68 KB): the CTAs that share an SM hide each other's prologue and merge, and the next
   // GEMM's CTAs find room to stage their weights early (C3 step -2.9 % against three stages)
   constexpr int STAGES = HD == 128 ? 2 : 4;
   const int smem = STAGES * 2 * KT * HD * 2 + 256 + 16 * HD * 2;   // ring (reused by the final merge) + barriers + Q tile

@@ -1,4 +1,5 @@
-"""The attention kernel of few query rows per KV head (chain drafts, single-token decoding): factors at the end of the fp32 range."""
+"""The attention kernel of few query rows per KV head (chain drafts, single-token decoding) against fp64: numbers of sequences that
+leave the chip idle or fill it several times, ragged contexts, factors at the end of the fp32 range."""
 import math
 
 import pytest
@@ -30,3 +31,32 @@ def test_rescaling_by_small_factors(new_key):
     # the result is rounded to bf16: 8 significant bits, half a unit is up to 2^-8 of the value; the smallest factor, 2^-138.7, has
     # 11 bits, and its exponent is off by some 2^-15
     assert float((out - ref).abs().max()) <= (2.0 ** -8 + 2.0 ** -11 + 2.0 ** -14) * ref
+
+
+@pytest.mark.parametrize("hd,grp", [(128, 1), (128, 4), (128, 16), (64, 4)])
+@pytest.mark.parametrize("n", [1, 5, 20, 70])
+def test_ragged_sequences_vs_fp64(n, hd, grp):
+    from paper_2503_01840_b200 import binding as sb
+    G, ps, tail = 8, 16, 3
+    H = G * grp
+    g = torch.Generator(device="cuda").manual_seed(n * grp + hd)
+
+    def rand(*s):
+        return torch.randn(*s, generator=g, device="cuda").to(torch.bfloat16)
+
+    ctx = torch.randint(0, 400, (n,), generator=g, device="cuda", dtype=torch.int32)
+    ctx[0] = 399
+    pps = 26
+    q, kp, vp = rand(n, H, hd) * 2, rand(n * pps, G, ps, hd), rand(n * pps, G, ps, hd)
+    table = torch.randperm(n * pps, generator=g, device="cuda").to(torch.int32).view(n, pps)
+    lo = torch.randint(0, 8, (n,), generator=g, device="cuda") | 1                    # tail keys in sight
+    out = sb.attention(q, kp, vp, table, ps, torch.arange(n, dtype=torch.int32, device="cuda"), ctx, ctx, lo, torch.zeros_like(lo), tail, G,
+                       400, impl=2).double()
+    for b in range(n):
+        c = int(ctx[b])
+        seen = torch.tensor(list(range(c)) + [c + t for t in range(tail) if int(lo[b]) >> t & 1], device="cuda")
+        K, V = (p[table[b].long()].permute(1, 0, 2, 3).reshape(G, pps * ps, hd)[:, seen].double() for p in (kp, vp))
+        p = (torch.einsum("gch,gnh->gcn", q[b].double().view(G, grp, hd), K) * hd ** -0.5).softmax(-1)
+        ref, mag = (torch.einsum("gcn,gnh->gch", p, x).reshape(H, hd) for x in (V, V.abs()))
+        # the probabilities and the result are rounded to bf16 (8 significant bits), everything else is fp32
+        assert bool(((out[b] - ref).abs() <= 2.0 ** -8 * 1.01 * (mag + ref.abs()) + 1e-5).all()), b
