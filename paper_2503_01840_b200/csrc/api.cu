@@ -485,11 +485,9 @@ template <typename T> struct Sched {
   // weight-streaming kernel's tiles feed the tensor pipe with: it re-reads the 32 KB activation k-block for every 128
   // features and spends as long in its 256-row epilogues as in its loops.  These passes take the row-major kernel.  Alone (8B
   // shapes, launches from a graph without the passes' epilogues, weight-streaming / row-major, us): QKV 23.4 / 19.2 at 144 rows, 30.9 / 20.0
-  // at 256; O 16.2 / 17.5, 19.5 / 18.5; down 30.8 / 32.6, 34.9 / 34.3; gate/up 56.7 / 57.8 at 192 and 58.9 / 53.9 at 256.  In the replayed
-  // step, with the epilogues' real inputs and at the clock a batch leaves, gate/up is the faster one from 129 rows on too: 69.0 / 66.7 at 144
-  // rows, 69.0 / 66.0 at 168.
+  // at 256; O 16.2 / 17.5, 19.5 / 18.5; down 30.8 / 32.6, 34.9 / 34.3; gate/up 56.7 / 57.8 at 192 and 58.9 / 53.9 at 256.
   bool row_major(FusedEpi epi, const FusedGemmArgs &a) const {
-    return a.rows > 128 && !a.withhold && !fused_gemm_pairs() && epi != EPI_TOPK && (epi != EPI_QKV || a.hd == 128);
+    return a.rows > (epi == EPI_SWIGLU ? 192 : 128) && !a.withhold && !fused_gemm_pairs() && epi != EPI_TOPK && (epi != EPI_QKV || a.hd == 128);
   }
   static WideEpi wide_epi(FusedEpi e) {
     return e == EPI_RESID ? WIDE_RESID : e == EPI_QKV ? WIDE_QKV : e == EPI_SWIGLU ? WIDE_SWIGLU : e == EPI_ARGMAX ? WIDE_ARGMAX : WIDE_F32;
