@@ -229,7 +229,7 @@ int spec_gemm(int32_t dtype, int32_t impl, const void *x, const void *w, float *
 int spec_gemm_fused(const void *x, const void *w, float *out_f32, int32_t rows, int32_t out, int32_t in, int32_t ldo,
                     int32_t split, int32_t stages, void *stream);
 
-/* The row-major kernels of passes of more than 128 rows (prefill, steps of 129 to 256 rows), without
+/* The row-major kernels of passes of more than 128 rows (prefill, steps of 129 to 256 rows; gate/up from 193 rows on), without
  * the passes' epilogues: out fp32 [rows][ldo] = x . w^T, or with w_up the gate/up form, out bf16 [rows][out] (ldo == out) as in
  * spec_gemm_swiglu.  Any number of rows; in % 8 == 0, out % 8 == 0, ldo % 4 == 0, 16-byte aligned pointers.  form: 0 lets the library
  * choose; else K slices (1..4, at most one per 64 of `in`), or for gate/up the features per tile (a multiple of 16 in 64..256, 1 = the
