@@ -698,8 +698,8 @@ template <typename T> struct Sched {
   }
   float *x_now = nullptr;        // where the residual stream is
   float *x_other() const { return x_now == c->x ? c->x_alt : c->x; }
-  // the layer up to its attention; add: the partial result still to be added to x_now; set: the stream is that result
-  void block_qkv32(const LayerW &w, KvPool pool, int rows, bool add, bool set, int tap_mask) {
+  // add: the partial result still to be added to x_now; set: the stream is that result
+  void block32(const LayerW &w, KvPool pool, int rows, int tail_len, bool add, bool set, int tap_mask) {
     const PageMap pm{c->page_table, c->pps, c->cfg.page_size, c->cfg.num_pages};
     float *next = set ? c->x : add ? x_other() : nullptr;
     mark(SPEC_PROF_GEMM);
@@ -708,12 +708,9 @@ template <typename T> struct Sched {
                     c->status, s);
     tick();
     if (next) x_now = next;
-  }
-  void block32(const LayerW &w, KvPool pool, int rows, int tail_len, bool add, bool set, int tap_mask) {
-    block_qkv32(w, pool, rows, add, set, tap_mask);
     attention(pool, rows, tail_len);
     gemm(c->ao, w.wo, c->proj, rows, c->k, c->H * c->hd, c->k, 0, 1);
-    float *next = x_other();
+    next = x_other();
     mark(SPEC_PROF_GEMM);
     launch_norm_swiglu(x_now, c->proj, next, (const float *)w.mlp_norm, c->cfg.rms_eps, (const float *)w.w_gate, (const float *)w.w_up, (float *)c->act, rows,
                        c->F, c->k, s);
@@ -786,9 +783,8 @@ template <typename T> struct Sched {
   }
 
   // draft head on the rows of c->meta: cat = [feat ; e(tok)], FC2, decoder block, final norm (-> h)
-  // logits: the draft LM head follows (draft_logits), which the fp32 schedule runs with the closing norm
   void draft_forward(const float *feat, int nparts, size_t fstride, const int32_t *src_row, int rows, int tail_len,
-                     bool prebuilt = false, bool pending = false, bool logits = false) {
+                     bool prebuilt = false, bool pending = false) {
     if (c->fused) return draft_forward_fused(feat, nparts, fstride, src_row, rows, tail_len, prebuilt, pending);
     head_done = false;
     if (nparts == 1 && norm_fused(rows)) {
@@ -796,10 +792,6 @@ template <typename T> struct Sched {
       launch_rope_cat(c->meta.pos, c->inv_freq, c->cs, c->hd / 2, feat, src_row, (const float *)c->embed, c->meta.tok, c->meta.seq, (float *)c->cat, rows, c->k, s);
       tick();
       gemm(c->cat, c->fc2, c->proj, rows, c->k, 2 * c->k, c->k, 0, 1);
-      if (!logits) {               // prefill: of the draft layer only the cached K/V are used
-        block_qkv32(c->dl, c->pools[c->L], rows, false, true, 0);
-        return;
-      }
       block32(c->dl, c->pools[c->L], rows, tail_len, false, true, 0);
       close32(c->dfinal_norm, 0, c->dlm_head, c->Vd, c->logits, rows);
       head_done = true;
@@ -973,7 +965,7 @@ template <typename T> struct Sched {
       mark(SPEC_PROF_TREE); launch_prep_extend(c->st, c->tb, c->meta, c->B, c->need_pos, c->status, s); tick();
       c->cur_rps = c->Pmax;
       fuse(c->pend_taps, c->Te);
-      draft_forward(c->proj, c->np_proj, c->ps_proj, nullptr, c->Te, c->Pmax, false, true, true);
+      draft_forward(c->proj, c->np_proj, c->ps_proj, nullptr, c->Te, c->Pmax, false, true);
       if (c->tree_fused) {
         if (extend_compact()) draft_logits_topk(c->B, nullptr, 0);
         else draft_logits_topk(c->Te, c->st.last_row, c->B);
@@ -987,7 +979,7 @@ template <typename T> struct Sched {
       }
       for (int p = 2; p <= c->D; p++) {
         c->cur_rps = c->K;
-        draft_forward(c->x, 1, 0, c->tb.feat_row, c->Td, c->tail_tree, c->tree_fused, false, true);
+        draft_forward(c->x, 1, 0, c->tb.feat_row, c->Td, c->tail_tree, c->tree_fused);
         if (c->tree_fused) {
           draft_logits_topk(c->Td, nullptr, 0);
           capture(p, c->Td, false);

@@ -134,9 +134,9 @@ __global__ void __launch_bounds__(128) gemm_skinny_kernel(const float *__restric
 // The same kernel with what surrounds it in a decoder layer: RMSNorm on the way in (the pending partial result is added to the
 // residual stream, the norm's factor is applied to the finished sums, the sum of squares comes out of the same loop) and RoPE
 // with the cache write, or SiLU(gate) * up, on the way out.  A warp's features come in pairs (rotation partners j and j + hd / 2
-// of a head, gate and up), which end in neighbouring lanes.  The new residual row goes to a buffer of its own (the last block of a
-// row group does nothing else): other blocks still read the old one.  A step of the tiny model is a chain of dependent launches of 2 to
-// 3 us each, so what counts is their number: five a layer instead of nine,
+// of a head, gate and up), which end in neighbouring lanes.  The new residual rows go to a buffer of their own (the last block does
+// nothing else): other blocks still read the old one.  A step of the tiny model is a chain of dependent launches of 4 to
+// 5 us each, so what counts is their number: five a layer instead of nine,
 // 48 a step instead of 76: a request of ten steps 3.06 -> 2.76 ms.  (With a branch per row around the added partial result, and the cache
 // slot looked up in front of the loop, it was 3.34: every load must be on its way before the first is used.)
 struct NormIn {
@@ -156,13 +156,13 @@ __global__ void __launch_bounds__(128) gemm_norm_kernel(NormIn in, SkinnyWeights
   pdl_wait();
   pdl_trigger();
   constexpr int NV = R * C, P = C / 2;
+  static_assert(NV == 32, "every lane ends with one value");
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int r0 = blockIdx.y * R;
   const int u0 = (blockIdx.x * 4 + warp) * (OUT == NOUT_PLAIN ? C : P), units = OUT == NOUT_PLAIN ? O : O / 2;    // features, or pairs of features
-  if (blockIdx.x + 1 == gridDim.x) {                   // the new residual rows and the taps: the last block of the row group
+  if (blockIdx.x + 1 == gridDim.x) {                   // the new residual rows and the taps: the last block
     if (in.x_out || in.tap_mask)
-      for (int i = threadIdx.x; i < min(R, rows - r0) * (I / 4); i += 128) {
-        const int r = r0 + i / (I / 4), k = i % (I / 4) * 4;
+      for (int i = threadIdx.x; i < rows * (I / 4); i += 128) {
+        const int r = i / (I / 4), k = i % (I / 4) * 4;
         const size_t at = (size_t)r * I + k;
         float4 a = *(const float4 *)(in.x + at);
         if (ADD) { const float4 b = *(const float4 *)(in.add + at); a.x += b.x; a.y += b.y; a.z += b.z; a.w += b.w; }
@@ -182,9 +182,8 @@ __global__ void __launch_bounds__(128) gemm_norm_kernel(NormIn in, SkinnyWeights
     const int o = OUT == NOUT_PLAIN ? u : OUT == NOUT_QKV ? u / half * no.hd + u % half + (c >= P ? half : 0) : u + (c >= P ? units : 0);
     wr[c] = o < sw.o1 ? sw.w0 + (size_t)o * I : o < sw.o2 ? sw.w1 + (size_t)(o - sw.o1) * I : sw.w2 + (size_t)(o - sw.o2) * I;
   }
-  // where this lane's value goes: row rl of the group, feature (or pair member) lane % C; 64 values: row = lane, both members
-  const int rl = NV == 32 ? lane / C : lane, c_own = NV == 32 ? lane % C : 0;
-  const int row = r0 + rl, unit = u0 + (OUT == NOUT_PLAIN ? c_own : c_own % P);
+  // where this lane's value goes: row lane / C, feature (or pair member) lane % C
+  const int row = lane / C, c_own = lane % C, unit = u0 + (OUT == NOUT_PLAIN ? c_own : c_own % P);
   const bool mine = row < rows && unit < units;
   float2 cs = make_float2(1.0f, 0.0f);
   int head = 0, seq = -1, kvpos = 0;
@@ -207,7 +206,7 @@ __global__ void __launch_bounds__(128) gemm_norm_kernel(NormIn in, SkinnyWeights
     const float4 g = *(const float4 *)(in.gain + k);
 #pragma unroll
     for (int r = 0; r < R; r++) {
-      const size_t at = (size_t)min(r0 + r, rows - 1) * I + k;
+      const size_t at = (size_t)min(r, rows - 1) * I + k;
       float4 a = *(const float4 *)(in.x + at);
       if (ADD) { const float4 b = *(const float4 *)(in.add + at); a.x += b.x; a.y += b.y; a.z += b.z; a.w += b.w; }
       sq[r] = fmaf(a.x, a.x, fmaf(a.y, a.y, fmaf(a.z, a.z, fmaf(a.w, a.w, sq[r]))));
@@ -242,14 +241,12 @@ __global__ void __launch_bounds__(128) gemm_norm_kernel(NormIn in, SkinnyWeights
   }
   const float inv = 1.0f / sqrtf(sq[0] / (float)I + in.eps);
   if (OUT == NOUT_PLAIN) {
-#pragma unroll
-    for (int i = 0; i < NV / 32; i++)
-      if (row < rows && u0 + c_own + i < units) no.out[(size_t)row * no.ldo + u0 + c_own + i] = v[i] * inv;
+    if (mine) no.out[(size_t)row * no.ldo + unit] = v[0] * inv;
     return;
   }
   // a: first member of the pair (feature j, gate), b: second (j + hd / 2, up)
-  const float own = v[0] * inv, other = NV == 32 ? __shfl_xor_sync(0xffffffffu, own, P) : v[NV / 32 - 1] * inv;
-  const bool second = NV == 32 && c_own >= P;
+  const float own = v[0] * inv, other = __shfl_xor_sync(0xffffffffu, own, P);
+  const bool second = c_own >= P;
   const float a = second ? other : own, b = second ? own : other;
   if (mine && OUT == NOUT_SWIGLU && !second) no.out[(size_t)row * units + unit] = (a / (1.0f + expf(-a))) * b;
   if (OUT == NOUT_SWIGLU || !mine) return;
@@ -263,8 +260,7 @@ __global__ void __launch_bounds__(128) gemm_norm_kernel(NormIn in, SkinnyWeights
   if (!dst) return;
   float oa = a * cs.x - b * cs.y, ob = b * cs.x + a * cs.y;
   if (head < no.H && seq < 0) oa = ob = 0.0f;           // padding row
-  if (!second) dst[j] = oa;
-  if (second || NV != 32) dst[j + half] = ob;
+  dst[second ? j + half : j] = second ? ob : oa;
 }
 
 // When the warp-per-feature kernel is taken: up to 32 rows every weight is read once; up to 256 rows while the weights fit the
@@ -295,18 +291,17 @@ static void launch_skinny(const float *x, SkinnyWeights sw, float *out, int rows
 
 template <int OUT>
 static void launch_norm(const NormIn &in, const SkinnyWeights &sw, const NormOut &no, int rows, int O, int I, cudaStream_t s) {
-  auto go = [&](auto kern, int R, int C) { launch_k(kern, dim3((O + 4 * C - 1) / (4 * C) + 1, (rows + R - 1) / R), dim3(128), 0, s, in, sw, no, rows, O, I); };
-  auto pick = [&](auto k4, auto k8, auto k16, auto k32) {
-    if (rows <= 4) go(k4, 4, 8);
-    else if (rows <= 8) go(k8, 8, 4);
-    else if (rows <= 16) go(k16, 16, 2);
-    else go(k32, 32, 2);
-  };
-  if (in.add) pick(gemm_norm_kernel<4, 8, OUT, true>, gemm_norm_kernel<8, 4, OUT, true>, gemm_norm_kernel<16, 2, OUT, true>, gemm_norm_kernel<32, 2, OUT, true>);
-  else pick(gemm_norm_kernel<4, 8, OUT, false>, gemm_norm_kernel<8, 4, OUT, false>, gemm_norm_kernel<16, 2, OUT, false>, gemm_norm_kernel<32, 2, OUT, false>);
+  auto go = [&](auto kern, int C) { launch_k(kern, dim3((O + 4 * C - 1) / (4 * C) + 1), dim3(128), 0, s, in, sw, no, rows, O, I); };
+  auto pick = [&](auto k4, auto k8, auto k16) { if (rows <= 4) go(k4, 8); else if (rows <= 8) go(k8, 4); else go(k16, 2); };
+  if (in.add) pick(gemm_norm_kernel<4, 8, OUT, true>, gemm_norm_kernel<8, 4, OUT, true>, gemm_norm_kernel<16, 2, OUT, true>);
+  else pick(gemm_norm_kernel<4, 8, OUT, false>, gemm_norm_kernel<8, 4, OUT, false>, gemm_norm_kernel<16, 2, OUT, false>);
 }
+// Every warp norms all rows for its own two to eight features, so what the launches saved cost grows with rows x contraction.  Steps
+// of fp32 models of four layers, separate kernels / these, us: 8 rows 302 / 239 at hidden 256, 317 / 283 at 512, 472 / 436 at 1024, 2239 /
+// 2183 at 4096; 16 rows 254 / 250 at 64, 297 / 290 at 256, 324 / 338 at 320, 326 / 349 at 512, 608 / 681 at 1024; 24 rows 264 / 286 at
+// hidden 64 already, 32 rows 372 / 584 at 512, 4910 / 12690 at 4096.
 bool gemm_norm_ok(const float *const *w, int nw, const float *gain, int rows, int O, int I) {
-  if ((uintptr_t)gain & 15) return false;
+  if (((uintptr_t)gain & 15) || rows > (I <= 256 ? 16 : 8)) return false;
   for (int j = 0; j < nw; j++)
     if (!skinny_ok(nullptr, w[j], rows, O, I)) return false;
   return true;

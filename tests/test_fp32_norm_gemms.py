@@ -1,6 +1,6 @@
-"""The fp32 model's schedule with norms, RoPE, cache writes and activations on the GEMMs: every row group of those kernels (4, 8, 16,
-32 rows and several groups), head dimensions and feature counts off the warps' shares, padding rows, taps, against the CPU oracle;
-weights off a 16-byte boundary stay on the plain schedule and agree with it."""
+"""The fp32 model's schedule with norms, RoPE, cache writes and activations on the GEMMs: every form of those kernels (4, 8, 16
+rows), steps whose passes have more rows than they take, head dimensions and feature counts off the warps' shares, padding rows,
+taps, against the CPU oracle; the rows they are taken for; weights off a 16-byte boundary stay on the plain schedule and agree with it."""
 import numpy as np
 import pytest
 
@@ -16,9 +16,9 @@ BASE = synth.ModelCfg("F", "fp32", 3, 72, 3, 1, 48, 200, 131, 77, (0, 1, 2), 5e5
 @pytest.mark.parametrize("kw,batch", [
     (dict(), 1),                                                       # 4, 2 and 7 rows
     (dict(tree_topk=4, tree_nodes=16), 1),                             # 16 rows
-    (dict(n_heads=4, n_kv_heads=2, head_dim=16, ffn=136, tree_topk=5, tree_nodes=29), 1),     # 29 rows
-    (dict(tree_depth=2, tree_topk=3, tree_nodes=11), 3),               # 9, 9 and 33 rows: a second group of one row
-    (dict(hidden=256, n_heads=2, n_kv_heads=2, head_dim=80, ffn=688, tree_depth=4, tree_nodes=12), 5),   # 25, 10 and 60 rows
+    (dict(n_heads=4, n_kv_heads=2, head_dim=16, ffn=136, tree_topk=5, tree_nodes=29), 1),     # 4 and 5 rows, 29 on the plain schedule
+    (dict(tree_depth=2, tree_topk=3, tree_nodes=11), 3),               # 9 and 9 rows, 33 on the plain schedule
+    (dict(hidden=256, n_heads=2, n_kv_heads=2, head_dim=80, ffn=688, tree_depth=4, tree_nodes=12), 5),   # 10 rows, 25 and 60 on the plain schedule
 ], ids=str)
 def test_fp32_schedule_vs_oracle(kw, batch):
     cfg = BASE.replace(batch=batch, prompt_lo=5, prompt_hi=70, prompt_len=37, **kw)
@@ -26,6 +26,24 @@ def test_fp32_schedule_vs_oracle(kw, batch):
     prompts = [p.numpy() for p in synth.make_prompts(cfg)]
     st, _ = parity.run_trajectory(cfg, tw, dw, prompts, n_steps=4, tol=1e-4)
     assert st.passes == 4 * cfg.tree_depth * batch and st.verify_compared == 4 * batch, st
+
+
+@pytest.mark.parametrize("hidden,most", [(64, 16), (256, 16), (264, 8), (1024, 8)])
+def test_fp32_rows_the_schedule_is_taken_for(hidden, most):
+    """Up to 16 rows at short contractions, up to 8 at others: seen by the launches of a step whose draft passes have few rows."""
+    def launches(rows):
+        cfg = BASE.replace(hidden=hidden, tree_depth=6, tree_topk=4, tree_nodes=rows)
+        tw, dw = synth.make_target_weights(cfg, device="cuda"), synth.make_draft_weights(cfg, device="cuda")
+        dec = sb.SpecDecoder(cfg, tw, dw, batch=1, max_ctx=64)
+        dec.prefill([np.arange(20, dtype=np.int32)], 10)
+        dec.step()
+        n = dec.launches_per_step()
+        dec.close()
+        return n
+
+    few = launches(3)
+    assert launches(most) == few
+    assert launches(most + 1) > few
 
 
 def test_fp32_unaligned_norm_weights():
