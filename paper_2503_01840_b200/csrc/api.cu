@@ -424,6 +424,11 @@ static size_t wide_carve(const spec_ctx *c, WideBufs &w, void *base, int rows, s
 }
 
 // ------------------------------------------------------------------------------------------ schedule
+// the attention of a pass runs on the tensor-core kernels, whose launches launch_attn_fast plans by the context's length
+static bool attn_is_fast(const spec_ctx *c) {
+  return c->cfg.dtype == SPEC_BF16 && !(c->cfg.flags & SPEC_FLAG_REF_ATTN) && attn_fast_supported(c->hd, c->H / c->G);
+}
+
 template <typename T> struct Sched {
   spec_ctx *c;
   cudaStream_t s;
@@ -642,8 +647,7 @@ template <typename T> struct Sched {
   void attention(KvPool pool, int rows, int tail_len) {
     mark(SPEC_PROF_ATTN);
     PageMap pm{c->page_table, c->pps, c->cfg.page_size, c->cfg.num_pages};
-    bool fast = c->cfg.dtype == SPEC_BF16 && !(c->cfg.flags & SPEC_FLAG_REF_ATTN) && attn_fast_supported(c->hd, c->H / c->G);
-    if (fast) {
+    if (attn_is_fast(c)) {
       int hint = std::max(0, c->ctx_hint);
       if (c->ctx_hint < 0)
         for (int b = 0; b < c->B; b++) hint = std::max(hint, c->n_upper[b]);
@@ -1170,7 +1174,7 @@ static std::atomic<int> g_tune_epoch{0};
 static StepPlan step_plan(const spec_ctx *c) {
   StepPlan p;
   p.epoch = g_tune_epoch.load();
-  if (!c->fused) return p;                 // the plain schedule's attention takes no plan
+  if (!attn_is_fast(c)) return p;          // the plain attention kernel takes no plan
   int hint = 0;
   for (int b = 0; b < c->B; b++) hint = std::max(hint, c->n_upper[b]);
   p.extend = attn_fast_plan(c->Te, c->H, c->G, c->hd, c->Pmax, hint, c->Pmax);

@@ -8,6 +8,16 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("dtype,batch", [("fp32", 1), ("fp32", 2), ("bf16", 1), ("bf16", 3)])
 def test_requests_in_a_row_equal_fresh_contexts(dtype, batch):
+    _requests_in_a_row(dtype, batch, 0)
+
+
+@pytest.mark.parametrize("flags", ["FLAG_REF_GEMM", "FLAG_REF_ATTN", "FLAG_NO_TMA_ATTN", "FLAG_NO_PDL"])
+def test_requests_in_a_row_on_other_kernels(flags):
+    from paper_2503_01840_b200 import binding as sb
+    _requests_in_a_row("bf16", 2, getattr(sb, flags))
+
+
+def _requests_in_a_row(dtype, batch, flags):
     from paper_2503_01840_b200 import binding as sb
     from paper_2503_01840_b200 import synth
     cfg = synth.ModelCfg("R", dtype, 2, 256, 4, 2, 64 if dtype == "fp32" else 128, 688, 2048, 1000, (0, 1, 1), 5e5, tree_depth=4, tree_topk=4, tree_nodes=20, seed=17).replace(batch=batch)
@@ -24,9 +34,9 @@ def test_requests_in_a_row_equal_fresh_contexts(dtype, batch):
         hidden = [] if mode == "plain" else [dec.debug(sb.DBG_NODE_HIDDEN, b) for b in range(batch)]      # (a plain pass has one row per sequence)
         return got + [dec.lengths()] + hidden
 
-    one = sb.SpecDecoder(cfg, tw, dw, batch=batch, max_ctx=800)
+    one = sb.SpecDecoder(cfg, tw, dw, batch=batch, max_ctx=800, flags=flags)
     for n, mode in requests:
-        fresh = sb.SpecDecoder(cfg, tw, dw, batch=batch, max_ctx=800)
+        fresh = sb.SpecDecoder(cfg, tw, dw, batch=batch, max_ctx=800, flags=flags)
         a, b = serve(one, n, mode), serve(fresh, n, mode)
         fresh.close()
         assert len(a) == len(b) and all(np.array_equal(x, y) for x, y in zip(a, b)), (n, mode)
