@@ -1190,14 +1190,16 @@ int launch_swiglu_mix(const FusedParams &p, const Plan &pl, bool pdl, cudaStream
   switch (pl.nt) {
     case 16: return launch_inst<16, EPI_SWIGLU, false, false, true>(p, pl, pdl, s);
     case 64: return launch_inst<64, EPI_SWIGLU, false, false, true>(p, pl, pdl, s);
-    default: return launch_inst<128, EPI_SWIGLU, false, false, true>(p, pl, pdl, s);
+    case 128: return launch_inst<128, EPI_SWIGLU, false, false, true>(p, pl, pdl, s);
+    default: return -1;                // the pair kernel's
   }
 }
 int launch_swiglu_pair(const FusedParams &p, const Plan &pl, bool pdl, cudaStream_t s) {
   switch (pl.nt) {
     case 16: return launch_inst<16, EPI_SWIGLU, true>(p, pl, pdl, s);
     case 64: return launch_inst<64, EPI_SWIGLU, true>(p, pl, pdl, s);
-    default: return launch_inst<128, EPI_SWIGLU, true>(p, pl, pdl, s);
+    case 128: return launch_inst<128, EPI_SWIGLU, true>(p, pl, pdl, s);
+    default: return -1;                // the pair kernel's
   }
 }
 
@@ -1223,7 +1225,8 @@ bool fused_gemm_supported(FusedEpi epi, const FusedGemmArgs &a) {
   if (a.nw != need) return false;
   for (int j = 0; j < a.nw; j++)
     if (!a.w[j] || ((uintptr_t)a.w[j] & 15) || a.O[j] < 1) return false;
-  if (epi == EPI_SWIGLU && a.O[0] != a.O[1]) return false;
+  // gate/up beyond 128 rows is the pair kernel's, which has one slice and a ring of its own
+  if (epi == EPI_SWIGLU && (a.O[0] != a.O[1] || (a.rows > 128 && (a.split || a.stages)))) return false;
   if (epi == EPI_RESID && (a.O[0] & 7)) return false;
   if (epi == EPI_TOPK && (a.topk < 1 || a.topk > 16 || !a.cand_val || !a.cand_idx || !a.cand_max || !a.cand_sum || a.cand_ld < (a.O[0] + TILE_M - 1) / TILE_M)) return false;
   if (epi == EPI_QKV) {
@@ -1274,7 +1277,7 @@ int fused_gemm_launch(TmaMaps *g, FusedEpi epi, const FusedGemmArgs &a, cudaStre
   p.stamp = a.stamp;
   p.spin = a.spin_limit ? a.spin_limit : SPIN_LIMIT;
   p.withhold = a.withhold ? 1 : 0;
-  if (epi == EPI_SWIGLU && pl.nt == 256 && a.split == 0 && a.stages == 0) {
+  if (epi == EPI_SWIGLU && pl.nt == 256) {
     // wide rows: one CTA per (gate tile, up tile) pair sharing the activation tiles; optionally two such CTAs as a
     // CTA pair that also share the activation k-block (each loads half of the rows)
     const bool duo2 = g_pairs_swiglu && (p.tiles0 % 2) == 0;

@@ -1,0 +1,51 @@
+"""Host rules of the kernels that no entry point shows, asked of the built library by a small program (no GPU: nothing is launched)."""
+import os
+import subprocess
+
+import pytest
+
+from paper_2503_01840_b200 import binding as sb
+from paper_2503_01840_b200 import build
+
+ASK = r"""
+#include <cstdio>
+#include <cstdlib>
+#include "gemm_fused.cuh"
+using namespace spec;
+int main(int, char **v) {                       // epilogue, rows, split, stages
+  static char mem[64];
+  FusedGemmArgs a;
+  const FusedEpi epi = (FusedEpi)atoi(v[1]);
+  a.x = (const bf16 *)(((uintptr_t)mem + 15) & ~(uintptr_t)15);
+  a.w[0] = a.w[1] = a.x;
+  a.O[0] = a.O[1] = 512; a.I = 512; a.nw = epi == EPI_SWIGLU ? 2 : 1;
+  a.rows = atoi(v[2]); a.split = atoi(v[3]); a.stages = atoi(v[4]);
+  printf("%d", fused_gemm_supported(epi, a) ? 1 : 0);
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def ask(tmp_path_factory):
+    d = tmp_path_factory.mktemp("rules")
+    src, exe = d / "ask.cu", d / "ask"
+    src.write_text(ASK)
+    lib = sb.library_path()
+    sb.lib()
+    subprocess.run([build.NVCC, "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-I", build.CSRC, str(src), lib, "-o", str(exe),
+                    "-Xlinker", "-rpath", "-Xlinker", os.path.dirname(lib)], check=True, capture_output=True)
+    return lambda *args: int(subprocess.run([str(exe), *map(str, args)], check=True, capture_output=True).stdout)
+
+
+F32, SWIGLU = 0, 3
+
+
+@pytest.mark.parametrize("rows,split,stages,taken", [
+    (128, 0, 0, 1), (128, 2, 0, 1), (128, 0, 3, 1), (256, 0, 0, 1), (129, 0, 0, 1),
+    (129, 2, 0, 0), (129, 0, 3, 0), (256, 1, 0, 0), (256, 4, 4, 0),
+])
+def test_gate_up_plans_are_for_up_to_128_rows(ask, rows, split, stages, taken):
+    """A forced K split or ring depth exists for gate/up up to 128 rows only: beyond, the tile kernel would read 256-row activation
+    boxes into stages of 128 rows."""
+    assert ask(SWIGLU, rows, split, stages) == taken
+    assert ask(F32, rows, split, stages) == 1
