@@ -87,7 +87,7 @@ def _kernel_bodies():
         if not fn.endswith(".cu"):
             continue
         s = open(os.path.join(csrc, fn)).read()
-        for m in re.finditer(r"__global__\s+void\s+(?:__launch_bounds__\([^)]*\)\s*)?(\w+)\s*\(", s):
+        for m in re.finditer(r"__global__\s+void\s+(?:__launch_bounds__\((?:[^()]|\([^()]*\))*\)\s*)?(\w+)\s*\(", s):
             i = s.index("{", m.end())
             depth, j = 0, i
             while True:
@@ -102,7 +102,8 @@ def test_every_step_kernel_orders_itself_behind_its_predecessor():
     """Kernels of a step are launched with programmatic dependent launch: a kernel may start before its predecessor
     has finished, and its successor waits only for IT.  A kernel without griddepcontrol.wait would let its successor
     overtake the kernel before it (the first QKV GEMM reading a RoPE table that is still being written), so every
-    kernel the scheduler launches with the attribute must wait, and must do so before it touches global memory."""
+    kernel the scheduler launches with the attribute must wait, and must do so before it touches what a kernel of the step
+    wrote.  The GEMMs read weights before it, the attention kernels what the next test names."""
     never_pdl = {"gemm_tcgen05_kernel", "reduce_slices_kernel"}      # launched without the attribute
     seen = 0
     for fn, name, body in _kernel_bodies():
@@ -118,3 +119,36 @@ def test_every_step_kernel_orders_itself_behind_its_predecessor():
             head = body[: body.index("pdl_wait()")]
             head = "\n".join(l for l in head.split("\n") if "__shared__" not in l)
             assert "[" not in head and "->" not in head, f"{fn}: {name} touches memory before pdl_wait()"
+
+
+def test_attention_reads_ahead_only_behind_launches_that_wait_first():
+    """The attention kernels of attn_fast.cu read row metadata, the page table and cached context before their wait.  That holds only
+    while the launch in front lets its dependents start after its own wait (everything before it is complete then), and while
+    nothing that launch writes is read early."""
+    bodies = {name: body for _, name, body in _kernel_bodies()}
+    early = [n for n in ("attn_tma_kernel", "attn_umma_kernel", "attn_tma_small_kernel") if "p.m.seq" in bodies[n][: bodies[n].index("pdl_wait()")]]
+    assert len(early) == 3, early
+    for name in early:
+        head = bodies[name][: bodies[name].index("pdl_wait()")]
+        for written_in_front in ("p.q ", "p.q+", "p.out", "part_o", "part_ml"):
+            assert written_in_front not in head, f"{name} touches {written_in_front} before its wait"
+        assert "p.ctx_ready ? ctx : 0" in head and "ctx_early" in bodies[name], name
+    # the launches in front of an attention launch
+    for name, epi in (("gemm_fused_kernel", "EPI_QKV"), ("gemm_wide_kernel", "WIDE_QKV"), ("gemm_wide_split_kernel", "WIDE_QKV")):
+        lines = [l.strip() for l in bodies[name].split("\n")]
+        at = [i for i, l in enumerate(lines) if "pdl_trigger()" in l]
+        for i in at:
+            if lines[i].startswith(f"if (EPI != {epi}) pdl_trigger();"):
+                continue
+            assert lines[i].startswith(f"if (EPI == {epi}) pdl_trigger();") and lines[i - 1] == "pdl_wait();", f"{name}: {lines[i]}"
+        assert len(at) >= 3, name
+    body = bodies["rope_kv_kernel"]
+    assert body.index("pdl_wait()") < body.index("pdl_trigger()")
+    # and nothing is launched between the two
+    api = open(os.path.join(ROOT, "paper_2503_01840_b200", "csrc", "api.cu")).read()
+    calls = [m.start() for m in re.finditer(r"\n\s+attention\(pool, rows, tail_len\);", api)]
+    assert len(calls) == 3
+    for c in calls:
+        before = [m for m in re.finditer(r"(\w+)(?:<T>)?\(", api[:c]) if m.group(1) in ("fgemm", "wgemm", "gemm", "gemm_cat") or m.group(1).startswith("launch_")]
+        last = before[-1]
+        assert last.group(1) in ("launch_rope_kv", "launch_norm_qkv") or api[last.end():].startswith("EPI_QKV"), last.group(1)
