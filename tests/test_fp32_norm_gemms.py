@@ -72,6 +72,34 @@ def test_fp32_unaligned_norm_weights():
     assert np.abs(a - b).max() <= 2e-5 * np.sqrt((b * b).mean())         # sums of up to 400 products, three layers deep
 
 
+def test_fp32_heads_off_the_schedule():
+    """LM heads off a 16-byte boundary run behind a closing norm of their own, which takes the residual stream from where the last
+    layer left it (a copy inside the captured step)."""
+    import torch
+    cfg = BASE.replace(hidden=256, n_heads=4, n_kv_heads=2, head_dim=64, tree_nodes=12)
+    tw, dw = synth.make_target_weights(cfg, device="cuda"), synth.make_draft_weights(cfg, device="cuda")
+
+    def shifted(t):
+        buf = torch.empty(t.numel() + 1, device="cuda")
+        buf[1:].copy_(t.view(-1))
+        return buf[1:].view(t.shape)
+
+    tws, dws = dict(tw, lm_head=shifted(tw["lm_head"])), dict(dw, lm_head=shifted(dw["lm_head"]))
+    prompt, seen = [np.arange(40, dtype=np.int32) % cfg.vocab], []
+    for t, d, flags in ((tw, dw, 0), (tws, dws, 0), (tws, dws, sb.FLAG_NO_GRAPH)):
+        dec = sb.SpecDecoder(cfg, t, d, batch=1, max_ctx=160, flags=flags)
+        dec.prefill(prompt, 16)
+        ids = np.concatenate([dec.step()[0] for _ in range(3)])
+        seen.append((ids, dec.debug(sb.DBG_TREE_TOK), dec.debug(sb.DBG_NODE_HIDDEN), dec.debug(sb.DBG_TARGET_LOGITS)))
+        dec.close()
+    assert all(np.array_equal(x, y) for x, y in zip(seen[1], seen[2]))
+    for a, b in zip(seen[0][:2], seen[1][:2]):
+        assert np.array_equal(a, b)
+    for a, b in zip(seen[0][2:], seen[1][2:]):
+        a, b = a.astype(np.float64), b.astype(np.float64)
+        assert np.abs(a - b).max() <= 2e-5 * np.sqrt((b * b).mean())     # sums of up to 400 products, three layers deep
+
+
 @pytest.mark.parametrize("rows", [1, 4, 5, 16, 17, 33])
 @pytest.mark.parametrize("O,I", [(33, 380), (33, 384), (250, 388), (2, 516), (70, 1028), (1184, 640), (4744, 512)])
 def test_fp32_gemm_contraction_over_warps(rows, O, I):
