@@ -662,8 +662,9 @@ template <typename T> struct Sched {
   }
 
   // One decoder block on `rows` rows described by c->meta.  first_mode: how the residual stream is
-  // formed from the pending partial sums (0 keep, 1 set, 2 add); tap_mask: taps of the previous block.
-  void block(const LayerW &w, KvPool pool, int rows, int tail_len, int first_mode, int tap_mask) {
+  // formed from the pending partial sums (0 keep, 1 set, 2 add); tap_mask: taps of the previous block; kv_only: no further than the
+  // cached K/V.
+  void block(const LayerW &w, KvPool pool, int rows, int tail_len, int first_mode, int tap_mask, bool kv_only = false) {
     int k = c->k, qd = c->H * c->hd, kvd = c->G * c->hd, qkvd = qd + 2 * kvd, F = c->F;
     PageMap pm{c->page_table, c->pps, c->cfg.page_size, c->cfg.num_pages};
     mark(SPEC_PROF_NORM); launch_add_norm<T>(c->x, c->proj, c->np_proj, c->ps_proj, first_mode, (T *)c->node_taps, tap_mask, (const T *)w.attn_norm,
@@ -673,6 +674,7 @@ template <typename T> struct Sched {
     gemm_cat(c->h, w.wq, qd, w.wk, kvd, w.wv, kvd, 3, c->qkv, rows, k, qkvd);
     mark(SPEC_PROF_ROPE_KV); launch_rope_kv<T>(c->qkv, c->np_qkv, c->ps_qkv, c->cs, c->meta, (T *)c->q, pool, pm, rows, c->H, c->G, c->hd, c->status, s);
     tick();
+    if (kv_only) return;
     attention(pool, rows, tail_len);
     c->np_proj = pick(k, qd, 1); c->ps_proj = pstride(k);
     gemm(c->ao, w.wo, c->proj, rows, k, qd, k, 0, c->np_proj);
@@ -787,8 +789,9 @@ template <typename T> struct Sched {
   }
 
   // draft head on the rows of c->meta: cat = [feat ; e(tok)], FC2, decoder block, final norm (-> h)
+  // kv_only (fp32): a prefill uses nothing of the draft layer but its cached K/V
   void draft_forward(const float *feat, int nparts, size_t fstride, const int32_t *src_row, int rows, int tail_len,
-                     bool prebuilt = false, bool pending = false) {
+                     bool prebuilt = false, bool pending = false, bool kv_only = false) {
     if (c->fused) return draft_forward_fused(feat, nparts, fstride, src_row, rows, tail_len, prebuilt, pending);
     head_done = false;
     if (nparts == 1 && norm_fused(rows)) {
@@ -806,7 +809,8 @@ template <typename T> struct Sched {
     tick();
     c->np_proj = pick(c->k, 2 * c->k, 1); c->ps_proj = pstride(c->k);
     gemm(c->cat, c->fc2, c->proj, rows, c->k, 2 * c->k, c->k, 0, c->np_proj);
-    block(c->dl, c->pools[c->L], rows, tail_len, 1, 0);
+    block(c->dl, c->pools[c->L], rows, tail_len, 1, 0, kv_only);
+    if (kv_only) return;
     mark(SPEC_PROF_NORM); launch_add_norm<T>(c->x, c->proj, c->np_proj, c->ps_proj, 2, (T *)nullptr, 0, (const T *)c->dfinal_norm, c->cfg.rms_eps,
                        (T *)c->h, nullptr, rows, rows, c->k, s);
     tick();
@@ -1078,7 +1082,7 @@ template <typename T> static int prefill_blocks(spec_ctx *c, const int32_t *lens
       if (nd > 0) {
         sc.fuse(c->node_taps, CH);
         CUDA_TRY(c, upload_meta(nd, b, start, c->prompt_dev + off + start + 1));
-        sc.draft_forward(c->proj, c->np_proj, c->ps_proj, nullptr, CH, PREFILL_BLOCK);
+        sc.draft_forward(c->proj, c->np_proj, c->ps_proj, nullptr, CH, PREFILL_BLOCK, false, false, c->cfg.dtype == SPEC_F32);
       }
     }
     c->ctx_hint = -1;
