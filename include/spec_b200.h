@@ -197,7 +197,8 @@ enum spec_debug_what {
   SPEC_DBG_PATH,             /* int32 [count]            */
   SPEC_DBG_STATUS,           /* int32 [4] device status words */
   SPEC_DBG_PAGE_TABLE,       /* int32 [pages of seq]     */
-  /* raw activation buffers of the last pass as floats, all allocated rows (debugging) */
+  /* raw activation buffers of the last pass as floats, all allocated rows (debugging); a buffer that the kernels of the last pass
+   * did not need holds what an earlier pass left (RAW_H: fp32 passes whose norms ride on the GEMMs) */
   SPEC_DBG_RAW_X = 100, SPEC_DBG_RAW_H, SPEC_DBG_RAW_Q, SPEC_DBG_RAW_AO, SPEC_DBG_RAW_ACT, SPEC_DBG_RAW_CAT,
   SPEC_DBG_RAW_SSQ, SPEC_DBG_RAW_LOGITS,
   /* SPEC_FLAG_STAMPS: per stamped launch of the last step, in launch order, uint64 [n][2] = {earliest time a CTA of the
@@ -251,8 +252,7 @@ int spec_gemm_topk(const void *x, const void *w, int32_t rows, int32_t out, int3
 
 /* Gate/up half of the decoder layer's MLP (the draft layer and every target layer are LLaMA-style decoder layers,
  * Section 3.1), on the kernel that passes of up to 192 rows use: act[r][f] = bf16(silu(g) * u), g = sum_i x[r][i] * w_gate[f][i], u likewise
- * with w_up, both accumulated in fp32 (a cluster holds the gate and the up tile of the same 128 features and their K
- * slices).  x [rows][in] bf16, w_gate / w_up [F][in] bf16, act [rows][F] bf16, all device pointers, 16-byte aligned;
+ * with w_up, both accumulated in fp32 (a CTA holds the gate and the up features of the same range).  x [rows][in] bf16, w_gate / w_up [F][in] bf16, act [rows][F] bf16, all device pointers, 16-byte aligned;
  * rows <= 256, in % 8 == 0.  Returns SPEC_OK or a negative code; nothing is allocated. */
 int spec_gemm_swiglu(const void *x, const void *w_gate, const void *w_up, void *act, int32_t rows, int32_t F, int32_t in,
                      void *stream);

@@ -594,9 +594,10 @@ __global__ void __launch_bounds__(288) attn_tma_kernel(const __grid_constant__ C
 //   O += P V  : A = P (bf16, written to shared memory by the softmax threads), B = the V tile read MN-major (the keys
 //               are the contraction dimension and the slow axis of the tile), accumulator = 128 columns that stay in
 //               tensor memory for the whole key range.
-// Thread r of the four softmax warps owns query row r = tensor-memory lane r: its row maximum and row sum need no
-// shuffles.  When a row maximum grows, the warp rescales its 32 rows of O in tensor memory (rare once the maximum has
-// settled).  Warp 4 is the TMA producer, warp 5 issues the MMAs.  Same masks, statistics and partial-result format as
+// Two warpgroups take the key tiles in turn, each with statistics and an O of its own, merged at the end.  Thread r of a group's
+// four warps owns query row r = tensor-memory lane r: its row maximum and row sum need no shuffles.  When a row maximum grows, the
+// warp rescales its 32 rows of O in tensor memory (rare once the maximum has
+// settled).  Warp 8 is the TMA producer, warp 9 issues the MMAs.  Same masks, statistics and partial-result format as
 // the kernels above.  Every wait is bounded; a timeout is recorded in the status words and the CTA winds down.
 constexpr int UM_STAGES = 5;
 constexpr int UM_S = 4;                            // score buffers: tile i uses buffer i % 4, its scores are computed up to three tiles ahead
@@ -1270,10 +1271,12 @@ __global__ void __launch_bounds__(256) attn_combine_kernel(const float *__restri
 
 int g_attn_target_ctas = 148;
 
-// Key splits: as many as one wave of CTAs allows (the kernels run one CTA per SM, they are register-bound), but no more than
-// give the busiest CTA its number of tiles: further splits only add partial results to merge.  One tile more than the hint is
-// counted, because the context grows while a captured step is replayed.  8B verify pass at 572..660 keys (9 or 10 tiles): 9 splits
-// (one or two tiles a CTA) 13.5 us, 5 splits (two) 12.5.
+// Key splits: as many as one wave of CTAs allows (the row-parallel and the tcgen05 kernel run one CTA per SM, they are
+// register-bound), but no more than give the busiest CTA its number of tiles: further splits only add partial results to merge.
+// One tile more than the hint is counted, because the context grows while a captured step is replayed.  8B verify pass at 572..660
+// keys (9 or 10 tiles): 9 splits (one or two tiles a CTA) 13.5 us, 5 splits (two) 12.5.  The key-parallel kernel, of which an SM holds
+// two, is planned by the same number; with 296 instead of 148 its verify pass takes (us a layer) 16.8 instead of 14.4 with two chains of
+// 256..2048 tokens, 15.3 instead of 16.7 with four, 18.9 instead of 23.6 with eight.
 int pick_splits(int seqs, int G, int mtiles, int ntiles) {
   const int n = ntiles + 1;
   int s = std::min(std::max(1, g_attn_target_ctas / (seqs * G * mtiles)), std::min(n, MAX_SPLITS));

@@ -610,8 +610,8 @@ __global__ void __launch_bounds__(fused_threads(NT, EPI), EPI == EPI_TOPK || EPI
       }
       if (good && p.out_f32 && o < p.O[0])
         for (int r = r0 + hw; r < r1; r += NH) p.out_f32[(size_t)(c0 + r) * p.ldo + o] = src[(r - r0) * TILE_M + f] * inv_s[c0 + r];
-      // One warp takes four rows at a time: four independent dependency chains in straight-line code (a CTA has only four warps,
-      // nothing else hides the latencies).  Lane l holds features l, l+32, l+64, l+96 of the tile as order-preserving keys.  The
+      // One warp takes four rows at a time: four independent dependency chains in straight-line code (a CTA has four warps,
+      // eight from 64-row tiles on: nothing else hides the latencies).  Lane l holds features l, l+32, l+64, l+96 of the tile as order-preserving keys.  The
       // K-th largest of the 32 lane maxima bounds the tile's K-th best value from below, and few values reach it (K to about
       // 1.5 K): those are collected and ranked by counting, so that the K results leave in one store.  In the
       // replayed step, 32000 x 4096, against picking the best K times by a warp-wide reduction: K = 10 49.3 -> 44.4 us at 10 rows,
