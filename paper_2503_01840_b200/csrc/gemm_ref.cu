@@ -69,7 +69,8 @@ __global__ void __launch_bounds__(256) gemm_ref_kernel(const T *__restrict__ x, 
 struct SkinnyWeights { const float *w0, *w1, *w2; int o1, o2; };
 // KS: the block's four warps take the same features and a quarter of the contraction each (added up through shared memory): a
 // warp then walks 128 elements of every 512 instead of all.  Taken from 384 elements on (three dependent steps of loads) while the
-// blocks, four times as many, are resident together (8 a SM).  Tiny request of ten steps 2.76 -> 2.48 ms.
+// blocks, four times as many, are resident together, and where they take two or three waves from the length on at which the shorter
+// walk is worth them (launch_skinny).  Tiny request of ten steps 2.76 -> 2.48 ms.
 template <int R, int C, bool KS>
 __global__ void __launch_bounds__(128) gemm_skinny_kernel(const float *__restrict__ x, SkinnyWeights sw, float *__restrict__ out, int rows,
                                                           int O, int I, int ldo) {
@@ -278,15 +279,21 @@ static bool skinny_ok(const float *x, const float *w, int rows, int O, int I) {
   return (double)padded * O * (I + 192) <= 1.31e6 * I * std::max(1.0, tiles / 256);
 }
 static void launch_skinny(const float *x, SkinnyWeights sw, float *out, int rows, int O, int I, int ldo, cudaStream_t s) {
-  auto go = [&](auto kern, auto split, int R, int C) {
-    const int groups = (rows + R - 1) / R;
-    if (I >= 384 && (O + C - 1) / C * groups <= 1184) launch_k(split, dim3((O + C - 1) / C, groups), dim3(128), 0, s, x, sw, out, rows, O, I, ldo);
+  // resident: blocks of the form that the chip holds (by registers); two, three: contraction from which KS may take as many waves of
+  // them.  Whole / shared contraction, us: 4 rows x 2048 x 384 (256 blocks) 3.1 / 2.5, x 4096 (512) x 512 3.8 / 3.9, x 1024 5.6 / 4.8, x 8192
+  // (1024) x 1024 6.4 / 6.8; 8 rows x 4096 (1024) x 384 3.9 / 4.0, x 512 5.0 / 4.4; 16 rows x 1024 (512) x 384 3.7 / 3.3, x 2048 (1024) x 384
+  // 4.1 / 4.7, x 512 5.3 / 4.8; 32 rows x 1024 (512) x 384 4.2 / 4.5, x 512 5.2 / 4.8, x 2048 (1024) x 1024 10.7 / 11.9; 64 rows x 688 (688)
+  // x 768 8.5 / 8.8, x 1024 10.5 / 10.0.
+  auto go = [&](auto kern, auto split, int R, int C, int resident, int two, int three) {
+    const int groups = (rows + R - 1) / R, blocks = (O + C - 1) / C * groups, waves = (blocks + resident - 1) / resident;
+    if (blocks <= 1184 && I >= (waves == 1 ? 384 : waves == 2 ? two : waves == 3 ? three : I + 1))
+      launch_k(split, dim3((O + C - 1) / C, groups), dim3(128), 0, s, x, sw, out, rows, O, I, ldo);
     else launch_k(kern, dim3((O + 4 * C - 1) / (4 * C), groups), dim3(128), 0, s, x, sw, out, rows, O, I, ldo);
   };
-  if (rows <= 4) go(gemm_skinny_kernel<4, 8, false>, gemm_skinny_kernel<4, 8, true>, 4, 8);
-  else if (rows <= 8) go(gemm_skinny_kernel<8, 4, false>, gemm_skinny_kernel<8, 4, true>, 8, 4);
-  else if (rows <= 16) go(gemm_skinny_kernel<16, 2, false>, gemm_skinny_kernel<16, 2, true>, 16, 2);
-  else go(gemm_skinny_kernel<32, 2, false>, gemm_skinny_kernel<32, 2, true>, 32, 2);
+  if (rows <= 4) go(gemm_skinny_kernel<4, 8, false>, gemm_skinny_kernel<4, 8, true>, 4, 8, 444, 1024, 1536);
+  else if (rows <= 8) go(gemm_skinny_kernel<8, 4, false>, gemm_skinny_kernel<8, 4, true>, 8, 4, 592, 512, 512);
+  else if (rows <= 16) go(gemm_skinny_kernel<16, 2, false>, gemm_skinny_kernel<16, 2, true>, 16, 2, 444, 384, 512);
+  else go(gemm_skinny_kernel<32, 2, false>, gemm_skinny_kernel<32, 2, true>, 32, 2, 296, 512, 1024);
 }
 
 template <int OUT>

@@ -105,6 +105,18 @@ def test_fp32_heads_off_the_schedule():
 def test_fp32_gemm_contraction_over_warps(rows, O, I):
     """Contractions around the length from which a block's warps share them, remainders of the 512 elements they take at a time,
     and feature counts on both sides of the blocks that are resident together."""
+    _gemm_vs_fp64(rows, O, I)
+
+
+@pytest.mark.parametrize("rows,O,I", [(4, 3552, 388), (4, 3560, 1020), (4, 3560, 1024), (4, 7112, 1532), (4, 7112, 1536), (7, 2372, 508), (7, 2372, 512),
+                                      (13, 890, 388), (13, 1778, 508), (13, 1778, 512), (30, 592, 388), (30, 594, 508), (30, 594, 512), (30, 1186, 1020),
+                                      (30, 1186, 1024), (30, 1778, 1028)])
+def test_fp32_gemm_blocks_around_waves(rows, O, I):
+    """Feature counts on both sides of one, two and three waves of each form, contractions on both sides of where they are taken."""
+    _gemm_vs_fp64(rows, O, I)
+
+
+def _gemm_vs_fp64(rows, O, I):
     import torch
     g = torch.Generator().manual_seed(rows + O + I)
     x, w = torch.randn(rows, I, generator=g), torch.randn(O, I, generator=g)
