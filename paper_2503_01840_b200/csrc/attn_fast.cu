@@ -1273,12 +1273,12 @@ int g_attn_target_ctas = 148;
 
 // Key splits: as many as one wave of CTAs allows (the row-parallel and the tcgen05 kernel run one CTA per SM, they are
 // register-bound), but no more than give the busiest CTA its number of tiles: further splits only add partial results to merge.
-// One tile more than the hint is counted, because the context grows while a captured step is replayed.  8B verify pass at 572..660
+// A captured step counts one tile more than the hint (grows), because the context grows while it is replayed; a launch whose hint is
+// its length does not (one row at 764 keys: 12 splits 9.8 us, a 13th without a tile 10.7).  8B verify pass at 572..660
 // keys (9 or 10 tiles): 9 splits (one or two tiles a CTA) 13.5 us, 5 splits (two) 12.5.  The key-parallel kernel, of which an SM holds
 // two, is planned by the same number; with 296 instead of 148 its verify pass takes (us a layer) 16.8 instead of 14.4 with two chains of
 // 256..2048 tokens, 15.3 instead of 16.7 with four, 18.9 instead of 23.6 with eight.
-int pick_splits(int seqs, int G, int mtiles, int ntiles) {
-  const int n = ntiles + 1;
+int pick_splits(int seqs, int G, int mtiles, int n) {
   int s = std::min(std::max(1, g_attn_target_ctas / (seqs * G * mtiles)), std::min(n, MAX_SPLITS));
   const int per = (n + s - 1) / s;
   return (n + per - 1) / per;
@@ -1398,12 +1398,12 @@ void attn_fast_set_target_ctas(int n) { g_attn_target_ctas = n; }
 void attn_fast_set_umma(int mode) { g_attn_umma = mode; }
 void attn_fast_override_umma(int v) { tl_attn_umma = v; }
 
-int attn_fast_plan(int rows, int H, int G, int hd, int rps, int ctx_hint, int tail_len) {
+int attn_fast_plan(int rows, int H, int G, int hd, int rps, int ctx_hint, int tail_len, bool grows) {
   if (rps < 1 || rows % rps) rps = 1;
-  const int grp = H / G, mtiles = (rps * grp + MT - 1) / MT, ntiles = std::max(1, (ctx_hint + tail_len + KT - 1) / KT);
+  const int grp = H / G, mtiles = (rps * grp + MT - 1) / MT, ntiles = std::max(1, (ctx_hint + tail_len + KT - 1) / KT) + (grows ? 1 : 0);
   const int nsplit = pick_splits(rows / rps, G, mtiles, ntiles);
   const int um_mode = tl_attn_umma >= 0 ? tl_attn_umma : g_attn_umma;
-  const bool umma = hd == 128 && rps * grp > 16 && (um_mode == 1 || (um_mode == 2 && ntiles + 1 > (UM_MIN_TILES - 1) * nsplit));
+  const bool umma = hd == 128 && rps * grp > 16 && (um_mode == 1 || (um_mode == 2 && ntiles > (UM_MIN_TILES - 1) * nsplit));
   return nsplit << 1 | (umma ? 1 : 0);
 }
 
@@ -1412,7 +1412,7 @@ int launch_attn_fast(const bf16 *q, KvPool pool, PageMap pm, RowMeta m, int tail
                      const int32_t *order, int order_len, unsigned long long *stamp, bool ctx_ready) {
   if (rps < 1 || rows % rps) rps = 1;
   const int seqs = rows / rps, grp = H / G, mtiles = (rps * grp + MT - 1) / MT;
-  const int plan = attn_fast_plan(rows, H, G, hd, rps, ctx_hint, tail_len), nsplit = scratch ? plan >> 1 : 1;
+  const int plan = attn_fast_plan(rows, H, G, hd, rps, ctx_hint, tail_len, ctx_ready), nsplit = scratch ? plan >> 1 : 1;
   AttnParams p;
   p.q = q; p.kpool = (const bf16 *)pool.k; p.vpool = (const bf16 *)pool.v; p.pm = pm; p.m = m; p.tail_len = tail_len;
   p.rows = rows; p.H = H; p.G = G; p.rps = rps; p.nsplit = nsplit; p.out = out;

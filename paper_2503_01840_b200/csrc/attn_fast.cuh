@@ -21,10 +21,11 @@ int launch_attn_fast(const bf16 *q, KvPool pool, PageMap pm, RowMeta m, int tail
 // Under programmatic dependent launch the row metadata, `order` and the page table are read before the wait for the previous
 // kernel: that kernel must let its dependents start only after its own wait (the QKV GEMM does), so that whatever the kernels
 // before it wrote is complete.  ctx_ready: the same holds for the K/V of the context positions (not in a prefill pass, where
-// a block's context may have been written by the pass's own QKV launch).
+// a block's context may have been written by the pass's own QKV launch).  It also says that the launch is a step's, whose context may
+// have grown beyond the hint by the time it is replayed (grows below).
 // What launch_attn_fast chooses by sizes and hint alone: key splits << 1 | tcgen05 kernel.  Two passes with equal plans are
 // recorded as equal launches.
-int attn_fast_plan(int rows, int H, int G, int hd, int rps, int ctx_hint, int tail_len);
+int attn_fast_plan(int rows, int H, int G, int hd, int rps, int ctx_hint, int tail_len, bool grows);
 // Drops the cached K/V tensor maps (pools of one-shot callers come and go).
 void attn_fast_forget_maps();
 // CTAs an attention launch aims at when it splits the keys (process-wide; default 148 = one wave)

@@ -10,9 +10,11 @@ from paper_2503_01840_b200 import build
 ASK = r"""
 #include <cstdio>
 #include <cstdlib>
+#include "attn_fast.cuh"
 #include "gemm_fused.cuh"
 using namespace spec;
-int main(int, char **v) {                       // epilogue, rows, split, stages
+int main(int n, char **v) {                     // epilogue, rows, split, stages; or rows, rows per sequence, context, tail, grows (32 heads, 8 KV heads)
+  if (n == 6) { printf("%d", attn_fast_plan(atoi(v[1]), 32, 8, 128, atoi(v[2]), atoi(v[3]), atoi(v[4]), atoi(v[5]) != 0) >> 1); return 0; }
   static char mem[64];
   FusedGemmArgs a;
   const FusedEpi epi = (FusedEpi)atoi(v[1]);
@@ -49,3 +51,17 @@ def test_gate_up_plans_are_for_up_to_128_rows(ask, rows, split, stages, taken):
     boxes into stages of 128 rows."""
     assert ask(SWIGLU, rows, split, stages) == taken
     assert ask(F32, rows, split, stages) == 1
+
+
+@pytest.mark.parametrize("rows,rps,ctx,tail,now,growing", [
+    (1, 1, 700, 64, 12, 13),        # 18 splits would fit: as many as key tiles
+    (1, 1, 10, 1, 1, 2),
+    (60, 60, 10, 60, 2, 3),
+    (60, 60, 512, 60, 9, 5),        # 9 fit: 9 tiles, one each; 10 tiles, two each
+    (60, 60, 580, 60, 5, 6),        # 10 tiles; 11
+    (256, 4, 2000, 4, 1, 1),
+])
+def test_key_splits_of_a_launch_and_of_a_step_that_grows(ask, rows, rps, ctx, tail, now, growing):
+    """No split without a key tile where the hint is the length; a captured step has one tile to grow by."""
+    assert ask(rows, rps, ctx, tail, 0) == now
+    assert ask(rows, rps, ctx, tail, 1) == growing

@@ -25,8 +25,8 @@ def test_tree_attention_tiles_vs_fp64(rows, ctx):
     vis[:, 0] = True
     lo = torch.tensor([sum(1 << t for t in range(tail) if vis[r, t]) for r in range(rows)], dtype=torch.int64, device="cuda")
     full = lambda c: torch.full((rows,), c, dtype=torch.int32, device="cuda")
-    # a hint of one position: two key splits whatever the context is
-    out = sb.attention(q, kp, vp, table, ps, full(0), full(ctx), full(ctx), lo, torch.zeros_like(lo), tail, G, 1, impl=3).double()
+    # a hint of one tile beside the tail's: two key splits whatever the context is
+    out = sb.attention(q, kp, vp, table, ps, full(0), full(ctx), full(ctx), lo, torch.zeros_like(lo), tail, G, 64, impl=3).double()
     K, V = (p[table[0].long()].permute(1, 0, 2, 3).reshape(G, pages * ps, hd)[:, :n].double() for p in (kp, vp))
     s = torch.einsum("rgch,gnh->rgcn", q.double().view(rows, G, H // G, hd), K) * hd ** -0.5
     mask = torch.cat([torch.ones(rows, ctx, dtype=torch.bool, device="cuda"), vis], 1)
