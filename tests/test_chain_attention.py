@@ -60,3 +60,31 @@ def test_ragged_sequences_vs_fp64(n, hd, grp):
         ref, mag = (torch.einsum("gcn,gnh->gch", p, x).reshape(H, hd) for x in (V, V.abs()))
         # the probabilities and the result are rounded to bf16 (8 significant bits), everything else is fp32
         assert bool(((out[b] - ref).abs() <= 2.0 ** -8 * 1.01 * (mag + ref.abs()) + 1e-5).all()), b
+
+
+@pytest.mark.parametrize("hd,grp,n", [(128, 4, 1), (128, 5, 3), (128, 16, 40), (64, 4, 2)])
+def test_output_and_scratch_off_the_vector_alignment(hd, grp, n):
+    """Results and partial results leave in vector stores where the caller's pointers allow it, else value by value: the same bits.
+    (The scratch owes its statistics 8 bytes.)  Splits of one tile and of several, one split, 4 to 16 query rows."""
+    from paper_2503_01840_b200 import binding as sb
+    G, ps, ctx, pps = 2, 16, 700, 46
+    H = G * grp
+    g = torch.Generator(device="cuda").manual_seed(7)
+    q, kp, vp = (torch.randn(*s, generator=g, device="cuda").to(torch.bfloat16) for s in ((n, H, hd), (n * pps, G, ps, hd), (n * pps, G, ps, hd)))
+    table = torch.arange(n * pps, device="cuda", dtype=torch.int32).view(n, pps)
+    seq = torch.arange(n, device="cuda", dtype=torch.int32)
+    c = torch.full((n,), ctx, device="cuda", dtype=torch.int32)
+    lo, hi = torch.ones(n, device="cuda", dtype=torch.int64), torch.zeros(n, device="cuda", dtype=torch.int64)
+    need = sb.lib().spec_attn_scratch_bytes(n, H, hd, ctx)
+    got = []
+    for out_off, scratch_off in ((0, 0), (1, 0), (2, 8), (4, 8)):
+        out = torch.zeros(n * H * hd + 8, device="cuda", dtype=torch.bfloat16)
+        scratch = torch.empty(need + 16, device="cuda", dtype=torch.uint8)
+        rc = sb.lib().spec_attention(1, 2, q.data_ptr(), kp.data_ptr(), vp.data_ptr(), table.data_ptr(), pps, ps, seq.data_ptr(), c.data_ptr(), c.data_ptr(),
+                                     lo.data_ptr(), hi.data_ptr(), 1, out.data_ptr() + 2 * out_off, n, H, G, hd, ctx, scratch.data_ptr() + scratch_off,
+                                     torch.cuda.current_stream().cuda_stream)
+        assert rc == 0
+        torch.cuda.synchronize()
+        assert not out[:out_off].any() and not out[out_off + n * H * hd:].any()
+        got.append(out[out_off:out_off + n * H * hd])
+    assert all(torch.equal(got[0], o) for o in got[1:])
