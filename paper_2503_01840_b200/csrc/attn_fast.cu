@@ -1240,33 +1240,42 @@ __global__ void __launch_bounds__(160, HD == 128 ? 2 : 1) attn_tma_small_kernel(
   }
 }
 
-// merge the splits: out = sum_s 2^((m_s - M) c) O_s / sum_s 2^((m_s - M) c) l_s.  One warp per (row, head): lanes first
-// fetch the (max, sum) pairs of all splits at once, then every lane adds up its HD/32 output dimensions with the
-// loads of eight splits in flight.
-template <int HD>
-__global__ void __launch_bounds__(256) attn_combine_kernel(const float *__restrict__ part_o, const float *__restrict__ part_ml, int nsplit,
-                                                           int nrh, bf16 *__restrict__ out, unsigned long long *stamp) {
+// merge the splits: out = sum_s 2^((m_s - M) c) O_s / sum_s 2^((m_s - M) c) l_s.  One warp per (row, head): a lane owns HD / 32
+// neighbouring output dimensions and the statistics of one split.  The launch moves little and is a chain of latencies, so the
+// statistics and the partial rows of up to NB splits are requested together, in 16-byte loads: 18 are all that one wave of CTAs
+// makes of eight KV heads, and up to six splits take fewer registers and fewer steps.  Attention and merge called in a row (8B shapes,
+// us; before: 12 splits at a time in 4-byte loads): draft pass, 18 splits 28.3 -> 23.4, 17 splits 17.7 -> 13.6, 11 splits 8.2 -> 7.4;
+// verify pass, 6 splits 13.6 -> 12.2, 9 splits 22.5 -> 21.9.  In the replayed step the GEMM behind it hides part of that: draft pass
+// at 6k 16.6 -> 15.4, 70B shapes at 1k 16.0 -> 13.4, their verify pass 19.1 -> 16.2.
+constexpr int COMBINE_WARPS = 4;
+template <int HD, int NB>
+__global__ void __launch_bounds__(32 * COMBINE_WARPS) attn_combine_kernel(const float *__restrict__ part_o, const float *__restrict__ part_ml, int nsplit,
+                                                           int nrh, bf16 *__restrict__ out, int vec, unsigned long long *stamp) {
   pdl_trigger();   // the next kernel may start staging its weights; it still waits for this grid to complete
   pdl_wait();
   KernelStamp stamp_guard(stamp, false);
   constexpr int DPL = HD / 32;                              // dimensions per lane
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int rh = blockIdx.x * 8 + warp;
+  const int rh = blockIdx.x * COMBINE_WARPS + warp;
   if (rh >= nrh) return;
   const float sc = rsqrtf((float)HD) * 1.4426950408889634f;
   float m = -INFINITY, ls = 0.0f;                           // lane s holds split s (nsplit <= 32)
   float2 ml = make_float2(-INFINITY, 0.0f);
   if (lane < nsplit) ml = *(const float2 *)(part_ml + ((size_t)lane * nrh + rh) * 2);
-  constexpr int NB = 12;                                    // partial rows in flight per lane
-  // the first NB partial rows are requested together with the statistics: one round trip instead of two
+  const float *src = part_o + (size_t)rh * HD + lane * DPL;
+  const size_t pitch = (size_t)nrh * HD;
   float v[NB][DPL];
+  auto fetch = [&](int s0) {
 #pragma unroll
-  for (int s = 0; s < NB; s++)
-    if (s < nsplit) {
-      const float *src = part_o + ((size_t)s * nrh + rh) * HD + lane * DPL;
+    for (int s = 0; s < NB; s++)
+      if (s0 + s < nsplit) {
+        if (vec) load_vec<DPL>(v[s], src + (s0 + s) * pitch);
+        else
 #pragma unroll
-      for (int e = 0; e < DPL; e++) v[s][e] = src[e];
-    }
+          for (int e = 0; e < DPL; e++) v[s][e] = src[(s0 + s) * pitch + e];
+      }
+  };
+  fetch(0);
   m = ml.x; ls = ml.y;
   float M = m;
   for (int off = 16; off > 0; off >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, off));
@@ -1277,15 +1286,7 @@ __global__ void __launch_bounds__(256) attn_combine_kernel(const float *__restri
 #pragma unroll
   for (int e = 0; e < DPL; e++) acc[e] = 0.0f;
   for (int s0 = 0; s0 < nsplit; s0 += NB) {
-    if (s0 > 0) {
-#pragma unroll
-      for (int s = 0; s < NB; s++)
-        if (s0 + s < nsplit) {
-          const float *src = part_o + ((size_t)(s0 + s) * nrh + rh) * HD + lane * DPL;
-#pragma unroll
-          for (int e = 0; e < DPL; e++) v[s][e] = src[e];
-        }
-    }
+    if (s0 > 0) fetch(s0);
 #pragma unroll
     for (int s = 0; s < NB; s++) {
       const float ws = __shfl_sync(0xffffffffu, w, (s0 + s) & 31);
@@ -1297,7 +1298,8 @@ __global__ void __launch_bounds__(256) attn_combine_kernel(const float *__restri
   }
   const float inv = l > 0.0f ? 1.0f / l : 0.0f;
 #pragma unroll
-  for (int e = 0; e < DPL; e++) out[(size_t)rh * HD + lane * DPL + e] = __float2bfloat16_rn(acc[e] * inv);
+  for (int e = 0; e < DPL; e++) acc[e] *= inv;
+  store_bf16<DPL>(out + (size_t)rh * HD + lane * DPL, acc, vec);
 }
 
 int g_attn_target_ctas = 148;
@@ -1413,6 +1415,13 @@ int launch_umma(AttnParams &p, dim3 grid, const CUtensorMap *mk, const CUtensorM
 }
 
 template <int HD>
+void launch_combine(const AttnParams &p, cudaStream_t s) {
+  const int nrh = p.rows * p.H;
+  launch_k(p.nsplit <= 6 ? attn_combine_kernel<HD, 6> : attn_combine_kernel<HD, 18>, dim3((nrh + COMBINE_WARPS - 1) / COMBINE_WARPS), dim3(32 * COMBINE_WARPS),
+           0, s, (const float *)p.part_o, (const float *)p.part_ml, p.nsplit, nrh, p.out, p.vec, p.stamp);
+}
+
+template <int HD>
 int launch_tma(AttnParams &p, dim3 grid, const CUtensorMap *mk, const CUtensorMap *mv, int32_t *status, cudaStream_t s) {
   if (p.rps * (p.H / p.G) <= 16) return launch_tma_small<HD>(p, grid, mk, mv, status, s);
   constexpr int STAGES = HD == 128 ? 3 : 4;
@@ -1463,8 +1472,7 @@ int launch_attn_fast(const bf16 *q, KvPool pool, PageMap pm, RowMeta m, int tail
       int rc = umma ? launch_umma(p, grid, mk, mv, status, s) : hd == 128 ? launch_tma<128>(p, grid, mk, mv, status, s) : launch_tma<64>(p, grid, mk, mv, status, s);
       if (rc == 0) {
         if (nsplit > 1) {
-          if (hd == 128) launch_k(attn_combine_kernel<128>, dim3((rows * H + 7) / 8), dim3(256), 0, s, p.part_o, p.part_ml, nsplit, rows * H, out, p.stamp);
-          else launch_k(attn_combine_kernel<64>, dim3((rows * H + 7) / 8), dim3(256), 0, s, p.part_o, p.part_ml, nsplit, rows * H, out, p.stamp);
+          if (hd == 128) launch_combine<128>(p, s); else launch_combine<64>(p, s);
         }
         return nsplit > 1 ? 2 : 1;
       }
@@ -1476,11 +1484,11 @@ int launch_attn_fast(const bf16 *q, KvPool pool, PageMap pm, RowMeta m, int tail
   if (hd == 128) {
     if (!limit[1].ensure(attn_mma_kernel<128>, (int)smem)) return -1;
     launch_k(attn_mma_kernel<128>, grid, dim3(256), smem, s, p);
-    if (nsplit > 1) launch_k(attn_combine_kernel<128>, dim3((rows * H + 7) / 8), dim3(256), 0, s, p.part_o, p.part_ml, nsplit, rows * H, out, p.stamp);
+    if (nsplit > 1) launch_combine<128>(p, s);
   } else {
     if (!limit[0].ensure(attn_mma_kernel<64>, (int)smem)) return -1;
     launch_k(attn_mma_kernel<64>, grid, dim3(256), smem, s, p);
-    if (nsplit > 1) launch_k(attn_combine_kernel<64>, dim3((rows * H + 7) / 8), dim3(256), 0, s, p.part_o, p.part_ml, nsplit, rows * H, out, p.stamp);
+    if (nsplit > 1) launch_combine<64>(p, s);
   }
   return nsplit > 1 ? 2 : 1;
 }

@@ -88,3 +88,21 @@ def test_output_and_scratch_off_the_vector_alignment(hd, grp, n):
         assert not out[:out_off].any() and not out[out_off + n * H * hd:].any()
         got.append(out[out_off:out_off + n * H * hd])
     assert all(torch.equal(got[0], o) for o in got[1:])
+
+
+@pytest.mark.parametrize("tiles", [2, 6, 7, 18, 19, 32, 40])
+@pytest.mark.parametrize("hd", [64, 128])
+def test_merge_of_many_splits(hd, tiles):
+    """One KV head: as many key splits as tiles, up to 32.  Around the numbers the merge takes in one go (6 and 18)."""
+    from paper_2503_01840_b200 import binding as sb
+    H, G, ps, ctx = 5, 1, 16, 64 * tiles - 1
+    pps = 4 * tiles + 1
+    g = torch.Generator(device="cuda").manual_seed(tiles)
+    q, kp, vp = (torch.randn(*s, generator=g, device="cuda").to(torch.bfloat16) for s in ((1, H, hd), (pps, G, ps, hd), (pps, G, ps, hd)))
+    table = torch.randperm(pps, generator=g, device="cuda").to(torch.int32).view(1, pps)
+    c, lo = torch.full((1,), ctx, device="cuda", dtype=torch.int32), torch.ones(1, device="cuda", dtype=torch.int64)
+    out = sb.attention(q, kp, vp, table, ps, torch.zeros(1, device="cuda", dtype=torch.int32), c, c, lo, torch.zeros_like(lo), 1, G, ctx, impl=2).double()
+    K, V = (p[table[0].long()].reshape(pps * ps, hd)[: ctx + 1].double() for p in (kp, vp))
+    p = (q[0].double() @ K.T * hd ** -0.5).softmax(-1)
+    ref, mag = p @ V, p @ V.abs()
+    assert bool(((out[0] - ref).abs() <= 2.0 ** -8 * 1.01 * (mag + ref.abs()) + 1e-5).all())       # as above
