@@ -628,8 +628,9 @@ constexpr int UM_TILE = KT * UM_HD * 2;            // 16 KB: the K (or the V) ti
 constexpr int UM_HALF = KT * 128;                  // 8 KB: one 64-element half of head_dim for 64 keys
 constexpr int UM_Q_BYTES = MT * UM_HD * 2;         // 32 KB
 constexpr int UM_P_BYTES = MT * KT * 2;            // 16 KB
-constexpr int UM_XCHG_BYTES = 2 * MT * 4;          // row statistics handed from softmax warpgroup 1 to warpgroup 0
-constexpr int UM_SMEM = UM_Q_BYTES + 2 * UM_P_BYTES + UM_STAGES * 2 * UM_TILE + 256 + UM_XCHG_BYTES;
+constexpr int UM_SMEM = UM_Q_BYTES + 2 * UM_P_BYTES + UM_STAGES * 2 * UM_TILE + 256;
+constexpr int UM_OUT_PITCH = 64 + 4;               // floats between the rows a warp stages for its stores (16-byte accesses without conflicts)
+static_assert(8 * 32 * UM_OUT_PITCH * 4 <= UM_STAGES * 2 * UM_TILE, "the ring holds the staged output");
 constexpr int UM_THREADS = 320;                    // two softmax warpgroups, the TMA producer warp, the MMA warp
 constexpr uint32_t UM_TMEM_COLS = 512;             // score buffers: columns 0..255, O of the two warpgroups: columns 256..511
 
@@ -661,6 +662,18 @@ __device__ __forceinline__ void tmem_ld64(uint32_t taddr, float (&v)[64]) {
       : "r"(taddr));
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
+  uint32_t *u = (uint32_t *)v;
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+      : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3]), "=r"(u[4]), "=r"(u[5]), "=r"(u[6]), "=r"(u[7]), "=r"(u[8]), "=r"(u[9]), "=r"(u[10]),
+        "=r"(u[11]), "=r"(u[12]), "=r"(u[13]), "=r"(u[14]), "=r"(u[15]), "=r"(u[16]), "=r"(u[17]), "=r"(u[18]), "=r"(u[19]), "=r"(u[20]),
+        "=r"(u[21]), "=r"(u[22]), "=r"(u[23]), "=r"(u[24]), "=r"(u[25]), "=r"(u[26]), "=r"(u[27]), "=r"(u[28]), "=r"(u[29]), "=r"(u[30]),
+        "=r"(u[31])
+      : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
 __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&v)[16]) {
   asm volatile(
       "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};" ::"r"(taddr),
@@ -683,7 +696,6 @@ __global__ void __launch_bounds__(UM_THREADS, 1) attn_umma_kernel(const __grid_c
   uint64_t *s_bar = empty + UM_STAGES, *p_bar = s_bar + UM_S, *o_bar = p_bar + 2;    // s_bar one per score buffer, the others one per warpgroup
   uint32_t *tmem_slot = (uint32_t *)(o_bar + 2);
   volatile uint32_t *abort_flag = tmem_slot + 1;
-  float *xchg = (float *)(sm + UM_SMEM - UM_XCHG_BYTES);    // [2][128]: reference maximum and sum of warpgroup 1's rows
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int grp = p.H / p.G;
@@ -696,8 +708,8 @@ __global__ void __launch_bounds__(UM_THREADS, 1) attn_umma_kernel(const __grid_c
   const int ps = p.pm.page_size;
   int seq = -1, ctx = 0;
   for (int i = 0; i < p.rps; i++) {
-    int s = p.m.seq[row0 + i];
-    if (s >= 0) { seq = s; ctx = p.m.ctx[row0 + i]; break; }
+    const int s = p.m.seq[row0 + i], cx = p.m.ctx[row0 + i];   // both loads in flight together
+    if (s >= 0) { seq = s; ctx = cx; break; }
   }
   const int nkeys = (seq >= 0) ? ctx + p.tail_len : 0, ctx_early = p.ctx_ready ? ctx : 0;
   const int ntiles = (nkeys + KT - 1) / KT;
@@ -767,14 +779,28 @@ __global__ void __launch_bounds__(UM_THREADS, 1) attn_umma_kernel(const __grid_c
     if (rvalid) { mlo = p.m.mask_lo[row0 + qi]; mhi = p.m.mask_hi[row0 + qi]; }
     else { mlo = ~0ull; mhi = ~0ull; }                         // a padding row attends every tail key (zeroed at the end)
     clip_tail(mlo, mhi, p.tail_len);
+    // A warp copies 16 rows, half a warp one of them at a time (a thread per row reads 32 rows of 16 bytes in each instruction: 2 us
+    // from the wait to the last row instead of 1).  A padding row's query may be anything: the row is dropped at the end.
+    int qoff[8];
+    {
+      const int mr = m0 + warp * 16 + (lane >> 4);
+      int i = mr / grp, hq = mr - i * grp;
+#pragma unroll
+      for (int it = 0; it < 8; it++) {
+        qoff[it] = mr + 2 * it < M ? ((row0 + i) * p.H + g * grp + hq) * (HD / 8) + (lane & 15) : -1;
+        hq += 2;
+        while (hq >= grp) { hq -= grp; i++; }
+      }
+    }
     pdl_wait();
     if (p.stamp && threadIdx.x == 0) atomicMin(p.stamp, global_ns());
-    const uint4 *src = (const uint4 *)(p.q + ((size_t)(row0 + qi) * p.H + g * grp + qh) * HD);
+    uint4 qv[8];
 #pragma unroll
-    for (int cc = 0; cc < 8; cc++) {                        // each of the row's two threads copies one half of it
-      const int c = wg * 8 + cc;
-      uint4 v = rvalid ? src[c] : make_uint4(0u, 0u, 0u, 0u);
-      *(uint4 *)(sQ + (c >> 3) * (MT * 128) + lr * 128 + (((c & 7) ^ (lr & 7)) << 4)) = v;
+    for (int it = 0; it < 8; it++) qv[it] = qoff[it] >= 0 ? ((const uint4 *)p.q)[qoff[it]] : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+    for (int it = 0; it < 8; it++) {
+      const int r = warp * 16 + it * 2 + (lane >> 4), c = lane & 15;
+      *(uint4 *)(sQ + (c >> 3) * (MT * 128) + r * 128 + (((c & 7) ^ (r & 7)) << 4)) = qv[it];
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
@@ -941,51 +967,57 @@ __global__ void __launch_bounds__(UM_THREADS, 1) attn_umma_kernel(const __grid_c
       if (!ok) { if (lane == 0) { *abort_flag = 1; if (status) set_status(status, ST_TIMEOUT, 426, blockIdx.z, t_end); } alive = false; }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     }
-    // ---- merge of the two streams: group 1 hands over its rows' statistics, group 0 reads both O accumulators.
-    // Every softmax thread reaches this barrier exactly once, whether or not its group gave up.
-    if (wg == 1) { xchg[lr] = mx; xchg[128 + lr] = l; }
+    // ---- merge of the two streams: each group shows the other its rows' statistics, then takes 64 of the 128 output dimensions of
+    // both O accumulators.  Every softmax thread reaches this barrier exactly once, whether or not its group gave up.
+    // (The statistics lie in the groups' own P tiles, whose last P V is complete.)
+    ((float2 *)my_p)[lr] = make_float2(mx, l);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     asm volatile("bar.sync 1, 256;" ::: "memory");
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const bool has1 = ntl > 1;                                   // group 1 accumulated something
-    // ---- write: final (one split) or partial
-    if (wg == 0 && alive) {
-      const float m1 = has1 ? xchg[lr] : -INFINITY, l1 = has1 ? xchg[128 + lr] : 0.0f;
-      const float mm = fmaxf(mx, m1);
-      const float f0 = (mx == -INFINITY) ? 0.0f : ex2_approx((mx - mm) * sc), f1 = (m1 == -INFINITY) ? 0.0f : ex2_approx((m1 - mm) * sc);
-      l = l * f0 + l1 * f1;
+    // ---- write: final (one split) or partial.  The ring is free (both groups have seen their last P V complete): every warp turns
+    // its 32 rows there, so that they leave in whole runs of 128 or 256 bytes (a thread per row stored 16 bytes to each of 32 rows
+    // at a time, and one group alone: 2.7 us of the CTA; now 1).  32 columns at a time: with 64 the kernel takes 148 registers instead
+    // of 125, and then a warp of the merge kernel no longer fits beside three of this one's (draft pass at 16k +1.5 us).
+    // With the coalesced queries, in the replayed step (us a layer): verify pass at 6k 21.7 -> 19.7, at 16k 37.1 -> 35.4, four
+    // sequences 27.2 -> 25.3, 70B shapes at 1k 16.5 -> 14.2.
+    if (alive) {
+      const float2 st0 = ((const float2 *)sP)[lr], st1 = ((const float2 *)(sP + UM_P_BYTES))[lr];
+      const float m0s = st0.x, l0 = st0.y, m1 = has1 ? st1.x : -INFINITY, l1 = has1 ? st1.y : 0.0f;
+      const float mm = fmaxf(m0s, m1);
+      const float f0 = (m0s == -INFINITY) ? 0.0f : ex2_approx((m0s - mm) * sc), f1 = (m1 == -INFINITY) ? 0.0f : ex2_approx((m1 - mm) * sc);
+      l = l0 * f0 + l1 * f1;
       mx = mm;
       const int r = row0 + qi, h = g * grp + qh;
       if (!rvalid) { l = 0.0f; mx = -INFINITY; }              // padding row: an empty partial, a zero output
-      const float inv = l > 0.0f ? 1.0f / l : 0.0f;
-      const size_t idx = (size_t)blockIdx.y * p.rows * p.H + (size_t)r * p.H + h;
+      const float inv = p.nsplit > 1 ? 1.0f : l > 0.0f ? 1.0f / l : 0.0f;
+      const int row_id = mrow < M ? r * p.H + h : -1;
+      if (__any_sync(0xffffffffu, row_id >= 0)) {              // the warp has rows
+        const bool use0 = ntl > 0 && rvalid && f0 != 0.0f, use1 = has1 && rvalid && f1 != 0.0f;
+        float *mine = (float *)ring + warp * 32 * UM_OUT_PITCH;
 #pragma unroll 1
-      for (int c = 0; c < HD / 16; c++) {
-        uint32_t v[16], w1[16];
-        if (ntl > 0) tc::tmem_ld16(tmem_o + lane_base + c * 16, v);              // the whole warp takes part
-        if (has1) tc::tmem_ld16(tmem_o + lane_base + HD + c * 16, w1);
+        for (int c = 0; c < 64; c += 32) {
+          float o0[32], o1[32];
+          if (ntl > 0) tmem_ld32(tmem_o + lane_base + (uint32_t)(wg * 64 + c), o0);              // the whole warp takes part
+          if (has1) tmem_ld32(tmem_o + lane_base + (uint32_t)(HD + wg * 64 + c), o1);
 #pragma unroll
-        for (int e = 0; e < 16; e++) {
-          float o0 = (ntl > 0 && rvalid && f0 != 0.0f) ? __uint_as_float(v[e]) * f0 : 0.0f;
-          float o1 = (has1 && rvalid && f1 != 0.0f) ? __uint_as_float(w1[e]) * f1 : 0.0f;
-          v[e] = __float_as_uint(o0 + o1);
+          for (int e = 0; e < 32; e++) o0[e] = ((use0 ? o0[e] * f0 : 0.0f) + (use1 ? o1[e] * f1 : 0.0f)) * inv;
+#pragma unroll
+          for (int e = 0; e < 32; e += 4) *(float4 *)(mine + lane * UM_OUT_PITCH + c + e) = make_float4(o0[e], o0[e + 1], o0[e + 2], o0[e + 3]);
         }
-        if (mrow < M) {
-          if (p.nsplit == 1) {
-            uint32_t w[8];
-#pragma unroll
-            for (int e = 0; e < 8; e++) w[e] = pack_bf16(__uint_as_float(v[2 * e]) * inv, __uint_as_float(v[2 * e + 1]) * inv);
-            uint4 *dst = (uint4 *)(p.out + ((size_t)r * p.H + h) * HD + c * 16);
-            dst[0] = make_uint4(w[0], w[1], w[2], w[3]);
-            dst[1] = make_uint4(w[4], w[5], w[6], w[7]);
-          } else {
-            uint4 *dst = (uint4 *)(p.part_o + idx * HD + c * 16);
-#pragma unroll
-            for (int e = 0; e < 4; e++) dst[e] = make_uint4(v[4 * e], v[4 * e + 1], v[4 * e + 2], v[4 * e + 3]);
-          }
+        __syncwarp();
+        const size_t split0 = (size_t)blockIdx.y * p.rows * p.H;
+#pragma unroll 4
+        for (int it = 0; it < 16; it++) {                         // two rows at a time, 16 bytes a lane
+          const int rr = it * 2 + (lane >> 4), id = __shfl_sync(0xffffffffu, row_id, rr);
+          if (id < 0) continue;
+          float t[4];
+          load_vec<4>(t, mine + rr * UM_OUT_PITCH + 4 * (lane & 15));
+          if (p.nsplit == 1) store_bf16<4>(p.out + (size_t)id * HD + wg * 64 + 4 * (lane & 15), t, p.vec);
+          else store_f32<4>(p.part_o + (split0 + id) * HD + wg * 64 + 4 * (lane & 15), t, p.vec);
         }
+        if (wg == 0 && row_id >= 0 && p.nsplit > 1) *(float2 *)(p.part_ml + (split0 + row_id) * 2) = make_float2(mx, l);
       }
-      if (mrow < M && p.nsplit > 1) { p.part_ml[idx * 2] = mx; p.part_ml[idx * 2 + 1] = l; }
     }
   }
 
@@ -1031,8 +1063,8 @@ __global__ void __launch_bounds__(160, HD == 128 ? 2 : 1) attn_tma_small_kernel(
   const int ps = p.pm.page_size;
   int seq = -1, ctx = 0;
   for (int i = 0; i < p.rps; i++) {
-    int s = p.m.seq[row0 + i];
-    if (s >= 0) { seq = s; ctx = p.m.ctx[row0 + i]; break; }
+    const int s = p.m.seq[row0 + i], cx = p.m.ctx[row0 + i];   // both loads in flight together
+    if (s >= 0) { seq = s; ctx = cx; break; }
   }
   const int nkeys = (seq >= 0) ? ctx + p.tail_len : 0, ctx_early = p.ctx_ready ? ctx : 0;
   const int ntiles = (nkeys + KT - 1) / KT;
