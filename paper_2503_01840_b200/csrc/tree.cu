@@ -462,12 +462,19 @@ void launch_expand(SeqState st, TreeBufs tb, RowMeta m, const int32_t *d2t, int 
 // Only the K tiles with the best heads can hold one of the K best candidates: every candidate of another tile comes behind
 // its own head, hence behind K better heads (tiles hold ascending index ranges, so the order of equal heads is the order of
 // the tiles).  So the warp first picks K tiles from the statistics it has in registers anyway and then fetches those K * K
-// candidates, one tile per lane, instead of staging all tiles' (20 KB per row, 200 KB per CTA) and walking their heads: the
-// merge of 10 rows of 250 tiles took 13 of the launch's 18 us.
+// candidates, one tile per lane.  Both selections bound the K-th best from below (by the K-th largest lane maximum, by the least
+// of the K heads), collect the few entries that reach the bound and rank them by counting; with more than 32 of them (many equal
+// values), or fewer than K lists, the best is picked K times by warp-wide reductions.
+// tgt (may be null): d2t, whose values for the winners go to out_tok; they are asked for before the ranking.
+constexpr int MERGE_SCRATCH = 32 + 64 + 16;              // words of shared memory a warp needs: lane maxima, (key, id) entries, tiles
 __device__ __forceinline__ void merge_tile_candidates(const float *__restrict__ cand_val, const int32_t *__restrict__ cand_idx,
                                                       const float *__restrict__ cand_max, const float *__restrict__ cand_sum,
-                                                      int tiles, int ld, int row, int K, int32_t *out_id, float *out_lp) {
+                                                      int tiles, int ld, int row, int K, int32_t *out_id, float *out_lp,
+                                                      const int32_t *__restrict__ tgt, int32_t *out_tok, unsigned *scratch) {
   const int lane = threadIdx.x & 31;
+  unsigned *s_max = scratch;
+  uint2 *s_ent = (uint2 *)(scratch + 32);
+  int *s_sel = (int *)(scratch + 96);
   float pm[8], ps[8];                                    // at most 8 tiles per lane, all loads issued before the first use
   int head[8];                                           // K = 1: the tiles' best are all the candidates there are (one load less to wait for)
 #pragma unroll
@@ -484,8 +491,23 @@ __device__ __forceinline__ void merge_tile_candidates(const float *__restrict__ 
   unsigned key[8];
 #pragma unroll
   for (int j = 0; j < 8; j++) key[j] = lane + 32 * j < tiles ? ordered_key(pm[j]) : 0u;      // keys of values are >= 1
+  // entries (key >= bound) of this lane join the list, in any order; returns how many the warp has (those past 32 are not stored)
+  int cnt = 0;
+  auto collect = [&](bool in, unsigned k, int id) {
+    const unsigned m = __ballot_sync(0xffffffffu, in);
+    const int at = cnt + __popc(m & ((1u << lane) - 1u));
+    if (in && at < 32) s_ent[at] = make_uint2(k, (unsigned)id);
+    cnt += __popc(m);
+  };
+  auto rank_of = [&](uint2 me) {                         // (key desc, id asc) among the cnt <= 32 entries
+    int rank = 0;
+#pragma unroll 4
+    for (int i = 0; i < cnt; i++) { const uint2 w = s_ent[i]; rank += w.x > me.x || (w.x == me.x && w.y < me.y); }
+    return rank;
+  };
   unsigned ck[15];
   int ci[15];
+  const int nsel = K < tiles ? K : tiles;
   if (K == 1) {                                          // each lane's best head, by (value desc, tile asc)
 #pragma unroll
     for (int i = 0; i < 15; i++) { ck[i] = 0u; ci[i] = -1; }
@@ -494,21 +516,42 @@ __device__ __forceinline__ void merge_tile_candidates(const float *__restrict__ 
       if (head[j] >= 0 && key[j] > ck[0]) { ck[0] = key[j]; ci[0] = head[j]; }
   } else {
     // ---- the K best tiles, (head desc, tile asc): lane c keeps the c-th
-    const int nsel = K < tiles ? K : tiles;
+    unsigned lm = 0u;
+#pragma unroll
+    for (int j = 0; j < 8; j++) lm = max(lm, key[j]);
+    s_max[lane] = lm;
+    __syncwarp();
+    int above = 0;                                       // lanes with a larger maximum
+#pragma unroll
+    for (int i = 0; i < 32; i += 4) { const uint4 w = *(const uint4 *)(s_max + i); above += (w.x > lm) + (w.y > lm) + (w.z > lm) + (w.w > lm); }
+    const unsigned bound = __reduce_min_sync(0xffffffffu, above < K && lm > 0u ? lm : 0xffffffffu);
+#pragma unroll
+    for (int j = 0; j < 8; j++) collect(key[j] >= bound, key[j], lane + 32 * j);
+    __syncwarp();
     int sel = 0;
-    for (int c = 0; c < nsel; c++) {
-      unsigned bk = 0u, wk;
-      int bt = -1;
+    if (cnt <= 32) {
+      if (lane < cnt) {
+        const uint2 me = s_ent[lane];
+        const int rank = rank_of(me);
+        if (rank < nsel) s_sel[rank] = (int)me.y;
+      }
+      __syncwarp();
+      if (lane < nsel) sel = s_sel[lane];
+    } else {
+      for (int c = 0; c < nsel; c++) {
+        unsigned bk = 0u, wk;
+        int bt = -1;
 #pragma unroll
-      for (int j = 0; j < 8; j++)
-        if (key[j] > bk) { bk = key[j]; bt = lane + 32 * j; }
-      const int w = warp_best(bk, bt, &wk);
-      if (lane == c) sel = w;
+        for (int j = 0; j < 8; j++)
+          if (key[j] > bk) { bk = key[j]; bt = lane + 32 * j; }
+        const int w = warp_best(bk, bt, &wk);
+        if (lane == c) sel = w;
 #pragma unroll
-      for (int j = 0; j < 8; j++)
-        if (lane + 32 * j == w) key[j] = 0u;
+        for (int j = 0; j < 8; j++)
+          if (lane + 32 * j == w) key[j] = 0u;
+      }
     }
-    // ---- lane c holds the c-th tile's candidates, best first: only their heads compete, and the winner's list moves up
+    // ---- lane c holds the c-th tile's candidates, best first
 #pragma unroll
     for (int i = 0; i < 15; i++) {
       const bool have = lane < nsel && i < K;
@@ -523,14 +566,43 @@ __device__ __forceinline__ void merge_tile_candidates(const float *__restrict__ 
   for (int j = 0; j < 8; j++) sum += (lane + 32 * j < tiles) ? ps[j] * expf(pm[j] - mx) : 0.0f;
   for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
   const float lse = logf(sum);
-  for (int c = 0; c < K; c++) {
-    unsigned wk;
-    const int wi = warp_best(ck[0], ci[0], &wk);         // two redux instructions instead of a shuffle tree
-    const bool won = wi >= 0 && ci[0] == wi;             // indices are unique: one lane at most
+  // ---- the K best of the lists
+  cnt = 33;
+  if (K > 1 && nsel == K) {
+    __syncwarp();                                        // the tiles' entries have been read
+    cnt = 0;
+    const unsigned bound = __reduce_min_sync(0xffffffffu, lane < K ? ck[0] : 0xffffffffu);      // K heads reach it
 #pragma unroll
-    for (int i = 0; i < 14; i++) { ck[i] = won ? ck[i + 1] : ck[i]; ci[i] = won ? ci[i + 1] : ci[i]; }
-    if (won) ci[14] = -1;
-    if (lane == 0) { out_id[c] = wi < 0 ? 0 : wi; out_lp[c] = wi < 0 ? 0.0f : (key_value(wk) - mx) - lse; }
+    for (int i = 0; i < 15; i++)
+      if (i < K) collect(ci[i] >= 0 && ck[i] >= bound, ck[i], ci[i]);
+    __syncwarp();
+  }
+  if (cnt >= K && cnt <= 32) {
+    if (lane < cnt) {
+      const uint2 me = s_ent[lane];
+      const int tok = tgt ? tgt[me.y] : 0;
+      const int rank = rank_of(me);
+      if (rank < K) {
+        out_id[rank] = (int)me.y;
+        out_lp[rank] = (key_value(me.x) - mx) - lse;
+        if (tgt) out_tok[rank] = tok;
+      }
+    }
+  } else {
+    // only the lists' heads compete, and the winner's list moves up
+    for (int c = 0; c < K; c++) {
+      unsigned wk;
+      const int wi = warp_best(ck[0], ci[0], &wk);       // two redux instructions instead of a shuffle tree
+      const bool won = wi >= 0 && ci[0] == wi;           // indices are unique: one lane at most
+#pragma unroll
+      for (int i = 0; i < 14; i++) { ck[i] = won ? ck[i + 1] : ck[i]; ci[i] = won ? ci[i + 1] : ci[i]; }
+      if (won) ci[14] = -1;
+      if (lane == 0) {
+        out_id[c] = wi < 0 ? 0 : wi;
+        out_lp[c] = wi < 0 ? 0.0f : (key_value(wk) - mx) - lse;
+        if (tgt) out_tok[c] = tgt[wi < 0 ? 0 : wi];
+      }
+    }
   }
   __syncwarp();
 }
@@ -541,9 +613,10 @@ __global__ void __launch_bounds__(256) merge_candidates_kernel(const float *cand
                                                                int32_t *__restrict__ idx, float *__restrict__ lp) {
   pdl_wait();
   pdl_trigger();
+  __shared__ __align__(16) unsigned scratch[8][MERGE_SCRATCH];
   const int warp = threadIdx.x >> 5, row = blockIdx.x * 8 + warp;
   if (row >= rows) return;
-  merge_tile_candidates(cand_val, cand_idx, cand_max, cand_sum, tiles, ld, row, K, idx + (size_t)row * K, lp + (size_t)row * K);
+  merge_tile_candidates(cand_val, cand_idx, cand_max, cand_sum, tiles, ld, row, K, idx + (size_t)row * K, lp + (size_t)row * K, nullptr, nullptr, scratch[warp]);
 }
 int launch_merge_candidates(const float *cand_val, const int32_t *cand_idx, const float *cand_max, const float *cand_sum, int tiles,
                             int ld, int rows, int K, int32_t *idx, float *lp, cudaStream_t s) {
@@ -585,18 +658,46 @@ __global__ void __launch_bounds__(TREE_THREADS) draft_tree_step_kernel(const Tre
   const int nrows = (pass == 1) ? 1 : K;                 // rows of this sequence in the pass that just ran
   const int nchild = nrows * K;
   const int nchild4 = (nchild + 3) & ~3;
-  float *cscore = (float *)smraw;                        // [nchild], padded to whole float4s with -inf
+  unsigned *scratch = (unsigned *)smraw;                 // [TREE_WARPS][MERGE_SCRATCH]
+  uint64_t *par_mask = (uint64_t *)(scratch + TREE_WARPS * MERGE_SCRATCH);   // [K][2] ancestor masks of this pass's rows
+  float *cscore = (float *)(par_mask + 2 * K);           // [nchild], padded to whole float4s with -inf
   float *tk_lp = cscore + ((K * K + 3) & ~3);            // [nrows][K]
   int32_t *tk_id = (int32_t *)(tk_lp + K * K);           // [nrows][K] draft ids
   int32_t *ctok = tk_id + K * K;                         // [nchild] target ids
   int32_t *newf = ctok + K * K;                          // [K] child index (within the level) of the new frontier
   int32_t *par_u = newf + K;                             // [K] pool index of the node each row of this pass processed
   float *par_sc = (float *)(par_u + K);                  // [K] its score
+  // What follows is a chain of round trips to L2 that nothing hides; everything that does not depend on another load is asked for
+  // at once: the sequence's state, the parents and their masks, the tiles' statistics.
   const int active = a.st.active[b], n = a.st.n[b];
-  const int src1 = a.compact ? b : a.st.last_row[b];     // pass 1: the row that holds the last pending entry's outputs
+  const int src1 = pass > 1 || a.compact ? b : a.st.last_row[b];     // pass 1: the row that holds the last pending entry's outputs
   const size_t pb = (size_t)b * (tb.pool + 1);
   const int base = (pass == 1) ? 0 : K + (pass - 2) * K * K;       // pool index of child 0 is base + 1
   const bool writer = blockIdx.y == 0;
+  // the parents of this pass's rows (two dependent loads)
+  if ((int)threadIdx.x < nrows) {
+    const int u = (pass == 1) ? 0 : tb.frontier[((size_t)b * D + pass - 1) * K + threadIdx.x];
+    const bool masks = writer && pass > 1;                // the writer replaces them below, and it alone reads them
+    const uint64_t lo = masks ? a.m.mask_lo[b * K + threadIdx.x] : 0ull, hi = masks ? a.m.mask_hi[b * K + threadIdx.x] : 0ull;
+    par_u[threadIdx.x] = u;
+    par_sc[threadIdx.x] = tb.pool_score[pb + u];
+    par_mask[2 * threadIdx.x] = lo; par_mask[2 * threadIdx.x + 1] = hi;
+  }
+  // ---- the RoPE angles of the next pass (one position for all rows; double precision, rounded once): two warps of their
+  // own, while the others merge
+  if (warp >= TREE_WARPS && pass < D && active) {
+    for (int i = threadIdx.x - TREE_WARPS * 32; i < a.half; i += TREE_ANGLE_WARPS * 32) {
+      double sn, cs_;
+      sincos((double)(n + pass - 1) * a.inv_freq[i], &sn, &cs_);
+      for (int rr = blockIdx.y; rr < K; rr += gridDim.y) a.cs[(size_t)(b * K + rr) * a.half + i] = make_float2((float)cs_, (float)sn);
+    }
+  }
+  // ---- 1. per row: log-sum-exp over the tiles and the K best of the tiles' candidates (value desc, index asc).  (The rows of a
+  // skipped sequence hold candidates too, of padding or of an earlier step; they are dropped below.)
+  for (int r = warp; warp < TREE_WARPS && r < nrows; r += TREE_WARPS) {
+    const int row = (pass == 1) ? max(src1, 0) : b * K + r;
+    merge_tile_candidates(a.cand_val, a.cand_idx, a.cand_max, a.cand_sum, a.tiles, a.ld, row, K, tk_id + r * K, tk_lp + r * K, a.d2t, ctok + r * K, scratch + warp * MERGE_SCRATCH);
+  }
   if (!active) {   // skipped sequence: its rows of the next pass are padding
     if (pass < D) {
       if (writer)
@@ -607,54 +708,29 @@ __global__ void __launch_bounds__(TREE_THREADS) draft_tree_step_kernel(const Tre
     }
     return;
   }
-  // the parents of this pass's rows (two dependent loads) are fetched while the candidates are on their way
-  if ((int)threadIdx.x < nrows) {
-    const int u = (pass == 1) ? 0 : tb.frontier[((size_t)b * D + pass - 1) * K + threadIdx.x];
-    par_u[threadIdx.x] = u;
-    par_sc[threadIdx.x] = tb.pool_score[pb + u];
-  }
-  // ---- the RoPE angles of the next pass (one position for all rows; double precision, rounded once): two warps of their
-  // own, while the others merge
-  if (warp >= TREE_WARPS && pass < D) {
-    for (int i = threadIdx.x - TREE_WARPS * 32; i < a.half; i += TREE_ANGLE_WARPS * 32) {
-      double sn, cs_;
-      sincos((double)(n + pass - 1) * a.inv_freq[i], &sn, &cs_);
-      for (int rr = blockIdx.y; rr < K; rr += gridDim.y) a.cs[(size_t)(b * K + rr) * a.half + i] = make_float2((float)cs_, (float)sn);
-    }
-  }
-  // ---- 1. per row: log-sum-exp over the tiles and the K best of the tiles' candidates (value desc, index asc)
-  for (int r = warp; warp < TREE_WARPS && r < nrows; r += TREE_WARPS) {
-    const int row = (pass == 1) ? src1 : b * K + r;
-    merge_tile_candidates(a.cand_val, a.cand_idx, a.cand_max, a.cand_sum, a.tiles, a.ld, row, K, tk_id + r * K, tk_lp + r * K);
-  }
   __syncthreads();
-  if (writer) {   // kept for inspection: the top-K of this pass in the layout of the per-row kernels
-    for (int i = threadIdx.x; i < nchild; i += blockDim.x) {
-      const int row = (pass == 1) ? b : b * K + i / K;
-      tb.tk_idx[(size_t)row * K + i % K] = tk_id[i];
-      tb.tk_lp[(size_t)row * K + i % K] = tk_lp[i];
-    }
-  }
   // ---- 2. children join the pool with cumulative scores
   for (int c = threadIdx.x; c < nchild; c += blockDim.x) {
     const int r = c / K;
     const int u = par_u[r];                                // the node row r processed
     const float sc = par_sc[r] + tk_lp[c];
-    const int tokid = a.d2t[tk_id[c]];
     cscore[c] = sc;
-    ctok[c] = tokid;
     if (writer) {
       const int ci = base + c + 1;
-      tb.pool_tok[pb + ci] = tokid;
+      tb.pool_tok[pb + ci] = ctok[c];
       tb.pool_parent[pb + ci] = u;
       tb.pool_depth[pb + ci] = pass;
       tb.pool_score[pb + ci] = sc;
+      // kept for inspection: the top-K of this pass in the layout of the per-row kernels
+      const int row = (pass == 1) ? b : b * K + r;
+      tb.tk_idx[(size_t)row * K + c - r * K] = tk_id[c];
+      tb.tk_lp[(size_t)row * K + c - r * K] = tk_lp[c];
     }
   }
+  if (pass >= D) return;
   if ((int)threadIdx.x < nchild4 - nchild) cscore[nchild + threadIdx.x] = -INFINITY;
   if ((int)threadIdx.x < K) newf[threadIdx.x] = threadIdx.x;           // where scores are NaN the ranks below leave places out
   __syncthreads();
-  if (pass >= D) return;
   // ---- 3. next frontier: the K best children of the level, (score desc, pool index asc)
   for (int c = threadIdx.x; c < nchild; c += blockDim.x) {
     const float s = cscore[c];
@@ -667,32 +743,23 @@ __global__ void __launch_bounds__(TREE_THREADS) draft_tree_step_kernel(const Tre
     if (rank < K) newf[rank] = c;
   }
   __syncthreads();
-  {
-    // the parents' masks are read by every writing thread before any row of the next pass is written
-    const int rr = threadIdx.x;
-    const bool mine = writer && rr < K;
-    const int c = mine ? newf[rr] : 0;
+  if (writer && (int)threadIdx.x < K) {
+    const int rr = threadIdx.x, c = newf[rr];
     const int pr = c / K;                                  // parent's row in the pass that just ran (0 in pass 1)
-    uint64_t lo = 0ull, hi = 0ull;
-    if (mine && pass > 1) { lo = a.m.mask_lo[b * K + pr]; hi = a.m.mask_hi[b * K + pr]; }
-    __syncthreads();
-    if (mine) {
-      const int ci = base + c + 1;
-      const int row = b * K + rr;
-      const int slot = (pass - 1) * K + rr;
-      if (slot < 64) lo |= 1ull << slot; else hi |= 1ull << (slot - 64);
-      tb.front_cur[b * K + rr] = ci;
-      tb.frontier[((size_t)b * D + pass) * K + rr] = ci;
-      tb.feat_row[row] = (pass == 1) ? src1 : b * K + pr;
-      a.m.seq[row] = b;
-      a.m.pos[row] = n + pass - 1;
-      a.m.kvpos[row] = n + slot;
-      a.m.ctx[row] = n;
-      a.m.tail_base[row] = n;
-      a.m.mask_lo[row] = lo;
-      a.m.mask_hi[row] = hi;
-      a.m.tok[row] = ctok[c];
-    }
+    const int ci = base + c + 1, row = b * K + rr, slot = (pass - 1) * K + rr;
+    uint64_t lo = par_mask[2 * pr], hi = par_mask[2 * pr + 1];
+    if (slot < 64) lo |= 1ull << slot; else hi |= 1ull << (slot - 64);
+    tb.front_cur[b * K + rr] = ci;
+    tb.frontier[((size_t)b * D + pass) * K + rr] = ci;
+    tb.feat_row[row] = (pass == 1) ? src1 : b * K + pr;
+    a.m.seq[row] = b;
+    a.m.pos[row] = n + pass - 1;
+    a.m.kvpos[row] = n + slot;
+    a.m.ctx[row] = n;
+    a.m.tail_base[row] = n;
+    a.m.mask_lo[row] = lo;
+    a.m.mask_hi[row] = hi;
+    a.m.tok[row] = ctok[c];
   }
   // ---- 4. inputs of the next pass: FC2 input [bf16(feature of the parent's row) ; embedding of the node's token], split
   // over the CTAs of the sequence
@@ -743,7 +810,7 @@ int launch_draft_tree_step(SeqState st, TreeBufs tb, RowMeta m, const int32_t *d
                            const int32_t *cand_idx, const float *cand_max, const float *cand_sum, int tiles, int ld, const float *x,
                            const bf16 *embed, bf16 *cat, int k, const double *inv_freq, float2 *cs, int half, int B, bool compact, cudaStream_t s) {
   if (!draft_tree_step_fits(tiles, tb.K) || ld != draft_tree_cand_ld(tiles) || (k % 8)) return -1;
-  const size_t smem = (size_t)((tb.K * tb.K + 3) & ~3) * 4 + (size_t)tb.K * tb.K * 12 + (size_t)tb.K * 12;
+  const size_t smem = (size_t)TREE_WARPS * MERGE_SCRATCH * 4 + (size_t)tb.K * 16 + (size_t)((tb.K * tb.K + 3) & ~3) * 4 + (size_t)tb.K * tb.K * 12 + (size_t)tb.K * 12;
   TreeStepArgs a{st, tb, m, d2t, pass, cand_val, cand_max, cand_sum, cand_idx, tiles, ld, x, embed, cat, k, inv_freq, cs, half, compact ? 1 : 0};
   const int Z = B >= 16 ? 1 : 8;        // CTAs per sequence that share the next pass's input assembly
   launch_k(draft_tree_step_kernel, dim3(B, Z), dim3(TREE_THREADS), smem, s, a);
