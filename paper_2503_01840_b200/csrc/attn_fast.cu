@@ -1434,9 +1434,12 @@ int launch_tma_small(AttnParams &p, dim3 grid, const CUtensorMap *mk, const CUte
   return 0;
 }
 
-int g_attn_umma = 2;            // tcgen05 kernel for the tree passes: 0 off, 1 on, 2 on when the busiest CTA gets at least UM_MIN_TILES key tiles
-// 8B verify pass, mma.sync / tcgen05 kernel: two tiles 12.5 / 12.5 us, three 14.6 / 13.6; with 40 query rows (draft) two tiles 8.8 / 9.0
-constexpr int UM_MIN_TILES = 3;
+int g_attn_umma = 2;            // tcgen05 kernel for the tree passes: 0 off, 1 on, 2 on when the busiest CTA gets at least um_min_tiles key tiles
+// The mma.sync kernel takes 2 us a tile whatever the rows, the tcgen05 kernel has two tiles in work at once but starts and ends later.
+// Replayed step, attention and merge, mma.sync / tcgen05 (us): 240 query rows per KV head (8B verify pass), one tile a CTA 10.9 / 11.5 at
+// 400 tokens, 12.1 / 10.9 at 250; two tiles 13.8 / 10.5 at 512, 14.9 / 12.0 at 1000.  40 rows (draft pass): one tile 7.4 / 9.3, two
+// 9.8 / 10.1 at 1500 tokens; three 14.6 / 13.6.
+int um_min_tiles(int query_rows) { return query_rows > 64 ? 2 : 3; }
 thread_local int tl_attn_umma = -1;   // per-call override (-1: none)
 
 int launch_umma(AttnParams &p, dim3 grid, const CUtensorMap *mk, const CUtensorMap *mv, int32_t *status, cudaStream_t s) {
@@ -1475,7 +1478,7 @@ int attn_fast_plan(int rows, int H, int G, int hd, int rps, int ctx_hint, int ta
   const int grp = H / G, mtiles = (rps * grp + MT - 1) / MT, ntiles = std::max(1, (ctx_hint + tail_len + KT - 1) / KT) + (grows ? 1 : 0);
   const int nsplit = pick_splits(rows / rps, G, mtiles, ntiles);
   const int um_mode = tl_attn_umma >= 0 ? tl_attn_umma : g_attn_umma;
-  const bool umma = hd == 128 && rps * grp > 16 && (um_mode == 1 || (um_mode == 2 && ntiles > (UM_MIN_TILES - 1) * nsplit));
+  const bool umma = hd == 128 && rps * grp > 16 && (um_mode == 1 || (um_mode == 2 && ntiles > (um_min_tiles(rps * grp) - 1) * nsplit));
   return nsplit << 1 | (umma ? 1 : 0);
 }
 
