@@ -1181,9 +1181,10 @@ static StepPlan step_plan(const spec_ctx *c) {
   if (!attn_is_fast(c)) return p;          // the plain attention kernel takes no plan
   int hint = 0;
   for (int b = 0; b < c->B; b++) hint = std::max(hint, c->n_upper[b]);
-  p.extend = attn_fast_plan(c->Te, c->H, c->G, c->hd, c->Pmax, hint, c->Pmax, true);
-  p.tree = attn_fast_plan(c->Td, c->H, c->G, c->hd, c->K, hint, c->tail_tree, true);
-  p.verify = attn_fast_plan(c->Tv, c->H, c->G, c->hd, c->N, hint, c->N, true);
+  const bool tma = attn_takes_tma(c->cfg.page_size, c->hd, !(c->cfg.flags & SPEC_FLAG_NO_TMA_ATTN));
+  p.extend = attn_fast_plan(c->Te, c->H, c->G, c->hd, c->Pmax, hint, c->Pmax, true, tma);
+  p.tree = attn_fast_plan(c->Td, c->H, c->G, c->hd, c->K, hint, c->tail_tree, true, tma);
+  p.verify = attn_fast_plan(c->Tv, c->H, c->G, c->hd, c->N, hint, c->N, true, tma);
   return p;
 }
 static void drop_graph(cudaGraphExec_t &g) {

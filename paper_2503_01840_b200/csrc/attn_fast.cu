@@ -1340,11 +1340,16 @@ int g_attn_target_ctas = 148;
 // register-bound), but no more than give the busiest CTA its number of tiles: further splits only add partial results to merge.
 // A captured step counts one tile more than the hint (grows), because the context grows while it is replayed; a launch whose hint is
 // its length does not (one row at 764 keys: 12 splits 9.8 us, a 13th without a tile 10.7).  8B verify pass at 572..660
-// keys (9 or 10 tiles): 9 splits (one or two tiles a CTA) 13.5 us, 5 splits (two) 12.5.  The key-parallel kernel, of which an SM holds
-// two, is planned by the same number; with 296 instead of 148 its verify pass takes (us a layer) 16.8 instead of 14.4 with two chains of
-// 256..2048 tokens, 15.3 instead of 16.7 with four, 18.9 instead of 23.6 with eight.
-int pick_splits(int seqs, int G, int mtiles, int n) {
-  int s = std::min(std::max(1, g_attn_target_ctas / (seqs * G * mtiles)), std::min(n, MAX_SPLITS));
+// keys (9 or 10 tiles): 9 splits (one or two tiles a CTA) 13.5 us, 5 splits (two) 12.5.
+// two_per_sm: the key-parallel kernel, of which an SM holds two; it is split for two waves' worth of CTAs as long as they keep two tiles
+// each (one tile each gains nothing: six chains of 30..200 tokens 6.7 us with 3 splits, 7.6 with 5).  Replayed step, 8B shapes, chains of
+// four rows, 64..1400 tokens, verify pass with 148 / 296 CTAs (us a layer): 4 chains 9.7 / 9.2, 6 11.7 / 10.4, 12 22.5 / 13.1, 16 of up
+// to 1000 17.7 / 13.7, 18 23.0 / 16.8.
+int pick_splits(int seqs, int G, int mtiles, int n, bool two_per_sm) {
+  const int units = seqs * G * mtiles;
+  int s = std::max(1, g_attn_target_ctas / units);
+  if (two_per_sm) s = std::max(s, std::min(2 * g_attn_target_ctas / units, n / 2));
+  s = std::min(s, std::min(n, MAX_SPLITS));
   const int per = (n + s - 1) / s;
   return (n + per - 1) / per;
 }
@@ -1473,10 +1478,14 @@ void attn_fast_set_target_ctas(int n) { g_attn_target_ctas = n; }
 void attn_fast_set_umma(int mode) { g_attn_umma = mode; }
 void attn_fast_override_umma(int v) { tl_attn_umma = v; }
 
-int attn_fast_plan(int rows, int H, int G, int hd, int rps, int ctx_hint, int tail_len, bool grows) {
+bool attn_takes_tma(int page_size, int hd, bool contiguous_tail) {
+  return contiguous_tail && (page_size == 16 || page_size == 32 || page_size == 64) && (hd == 64 || hd == 128);
+}
+
+int attn_fast_plan(int rows, int H, int G, int hd, int rps, int ctx_hint, int tail_len, bool grows, bool tma) {
   if (rps < 1 || rows % rps) rps = 1;
   const int grp = H / G, mtiles = (rps * grp + MT - 1) / MT, ntiles = std::max(1, (ctx_hint + tail_len + KT - 1) / KT) + (grows ? 1 : 0);
-  const int nsplit = pick_splits(rows / rps, G, mtiles, ntiles);
+  const int nsplit = pick_splits(rows / rps, G, mtiles, ntiles, tma && rps * grp <= 16);
   const int um_mode = tl_attn_umma >= 0 ? tl_attn_umma : g_attn_umma;
   const bool umma = hd == 128 && rps * grp > 16 && (um_mode == 1 || (um_mode == 2 && ntiles > (um_min_tiles(rps * grp) - 1) * nsplit));
   return nsplit << 1 | (umma ? 1 : 0);
@@ -1487,7 +1496,8 @@ int launch_attn_fast(const bf16 *q, KvPool pool, PageMap pm, RowMeta m, int tail
                      const int32_t *order, int order_len, unsigned long long *stamp, bool ctx_ready) {
   if (rps < 1 || rows % rps) rps = 1;
   const int seqs = rows / rps, grp = H / G, mtiles = (rps * grp + MT - 1) / MT;
-  const int plan = attn_fast_plan(rows, H, G, hd, rps, ctx_hint, tail_len, ctx_ready), nsplit = scratch ? plan >> 1 : 1;
+  const bool tma = attn_takes_tma(pm.page_size, hd, contiguous_tail);
+  const int plan = attn_fast_plan(rows, H, G, hd, rps, ctx_hint, tail_len, ctx_ready, tma), nsplit = scratch ? plan >> 1 : 1;
   AttnParams p;
   p.q = q; p.kpool = (const bf16 *)pool.k; p.vpool = (const bf16 *)pool.v; p.pm = pm; p.m = m; p.tail_len = tail_len;
   p.rows = rows; p.H = H; p.G = G; p.rps = rps; p.nsplit = nsplit; p.out = out;
@@ -1500,7 +1510,7 @@ int launch_attn_fast(const bf16 *q, KvPool pool, PageMap pm, RowMeta m, int tail
   dim3 grid(mtiles, nsplit, seqs * G);
   // TMA-staged kernel when the tail follows the context and a page is a whole number of 128-byte-swizzle boxes
   const int ps = pm.page_size;
-  if (contiguous_tail && (ps == 16 || ps == 32 || ps == 64) && (hd == 64 || hd == 128)) {
+  if (tma) {
     const bool umma = plan & 1;
     const CUtensorMap *mk = kv_map(pool.k, pm.num_pages, G, ps, hd, umma ? 1 : 0), *mv = kv_map(pool.v, pm.num_pages, G, ps, hd, umma ? 1 : 0);
     if (mk && mv) {

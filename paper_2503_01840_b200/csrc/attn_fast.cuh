@@ -23,9 +23,11 @@ int launch_attn_fast(const bf16 *q, KvPool pool, PageMap pm, RowMeta m, int tail
 // before it wrote is complete.  ctx_ready: the same holds for the K/V of the context positions (not in a prefill pass, where
 // a block's context may have been written by the pass's own QKV launch).  It also says that the launch is a step's, whose context may
 // have grown beyond the hint by the time it is replayed (grows below).
+// Whether the TMA-staged kernels take a launch (the others are for one CTA per SM).
+bool attn_takes_tma(int page_size, int head_dim, bool contiguous_tail);
 // What launch_attn_fast chooses by sizes and hint alone: key splits << 1 | tcgen05 kernel.  Two passes with equal plans are
-// recorded as equal launches.
-int attn_fast_plan(int rows, int H, int G, int hd, int rps, int ctx_hint, int tail_len, bool grows);
+// recorded as equal launches.  tma: attn_takes_tma of the launch.
+int attn_fast_plan(int rows, int H, int G, int hd, int rps, int ctx_hint, int tail_len, bool grows, bool tma = true);
 // Drops the cached K/V tensor maps (pools of one-shot callers come and go).
 void attn_fast_forget_maps();
 // CTAs an attention launch aims at when it splits the keys (process-wide; default 148 = one wave)
