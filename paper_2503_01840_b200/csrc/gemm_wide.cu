@@ -51,6 +51,7 @@ constexpr int W_PAIRS = 74;                               // 148 SMs
 struct alignas(64) WideParams {
   CUtensorMap map_x, map_w[3];
   int rows, KB, m_tiles, n_tiles;
+  int half;                      // rows of a CTA: 128, or with one row tile half of the rows there are (split kernel)
   int h0, h1;                    // half tiles [0,h0) belong to w0, [h0,h1) to w1, the rest to w2
   int O[3];
   int kind0;                     // WIDE_QKV: what w0 is (0 q, 1 k)
@@ -533,7 +534,8 @@ __device__ __forceinline__ float4 ld_peer4(uint32_t local_addr, uint32_t rank) {
   return v;
 }
 
-template <int EPI, int S>
+// FEW: at most 96 rows per CTA
+template <int EPI, int S, bool FEW>
 __global__ void __launch_bounds__(WS_THREADS, 1) gemm_wide_split_kernel(const __grid_constant__ WideParams p) {
   extern __shared__ unsigned char smem_raw[];
   unsigned char *ring = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -553,8 +555,9 @@ __global__ void __launch_bounds__(WS_THREADS, 1) gemm_wide_split_kernel(const __
   const uint32_t lead = crank & ~1u;
   const int t = blockIdx.x / (2 * S), mt = t % p.m_tiles, nt = t / p.m_tiles;
   const int kb0 = (int)(((long long)slice * p.KB) / S), kb1 = (int)(((long long)(slice + 1) * p.KB) / S), nkb = kb1 - kb0;
-  const int row_c = mt * WIDE_ROWS + xr * W_HALF;              // first row of this CTA
-  const int nrow = min(max(p.rows - row_c, 0), W_HALF);
+  const int row_c = mt * WIDE_ROWS + xr * p.half;              // first row of this CTA
+  const int nrow = min(max(p.rows - row_c, 0), p.half);
+  const uint32_t fill = 2u * (uint32_t)(p.half * TILE_K * 2 + W_A_BYTES);      // bytes of a stage, both CTAs
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < W_STAGES; i++) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
@@ -585,7 +588,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1) gemm_wide_split_kernel(const __
     const int npre = dead ? 0 : nkb < W_STAGES ? nkb : W_STAGES;
     if (elect_one())
       for (int i = 0; i < npre; i++) {
-        if (xr == 0) mbar_expect_tx(&full[i], 2 * W_STAGE);
+        if (xr == 0) mbar_expect_tx(&full[i], fill);
         tma_load_2d_pair_hint(ring + i * W_STAGE + W_A_BYTES, mw, (kb0 + i) * TILE_K, tm * W_HALF, mapa_u32(smem_u32(&full[i]), lead), pol);
       }
     __syncwarp();
@@ -604,7 +607,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1) gemm_wide_split_kernel(const __
         if (elect_one()) {
           unsigned char *a = ring + st * W_STAGE;
           const uint32_t fb = mapa_u32(smem_u32(&full[st]), lead);
-          if (xr == 0) mbar_expect_tx(&full[st], 2 * W_STAGE);
+          if (xr == 0) mbar_expect_tx(&full[st], fill);
           const int kx = (kb0 + i) * TILE_K;
           tma_load_2d_pair_hint(a + W_A_BYTES, mw, kx, tm * W_HALF, fb, pol);
           tma_load_2d_pair(a, &p.map_x, kx, row_c, fb);
@@ -661,7 +664,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1) gemm_wide_split_kernel(const __
     if (!ok) {
       if (lane == 0) set_status(p.status, ST_TIMEOUT, 252, blockIdx.x, slice);
       *abort_flag = 1;
-    } else {
+    } else if ((warp & 3) * 32 < nrow) {
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const int r = (warp & 3) * 32 + lane, half = warp >> 3, c0 = (warp >> 2 & 1) * 2;      // four warps per quarter: 64 columns each
       unsigned char *dst = ring + (half * W_HALF + r) * 512;
@@ -692,7 +695,8 @@ __global__ void __launch_bounds__(WS_THREADS, 1) gemm_wide_split_kernel(const __
     const bool fok = good && (EPI == WIDE_QKV ? tm * 128 < p.O[mi] : fo < p.O[0]);
     float4 gn = make_float4(0.f, 0.f, 0.f, 0.f);
     if (EPI == WIDE_RESID && fok) gn = load_gain(p, fo);
-    constexpr int RB = S == 3 ? 6 : 4;                         // rows in flight per warp: a full tile's share in one or two batches
+    // rows in flight per warp: a share in one batch (two with two slices), of 128 rows or of at most 96
+    constexpr int RB = FEW ? (S == 3 ? 4 : 3) : S == 3 ? 6 : 4;
     for (int rb = r0 + sub; rb < r1; rb += 8 * RB) {
       float4 xin[RB];
 #pragma unroll
@@ -978,11 +982,11 @@ int launch_wide(WideParams &p, bool pdl, cudaStream_t s) {
   return cudaLaunchKernelEx(&cfg, gemm_wide_kernel<EPI>, p) == cudaSuccess ? 0 : -6;
 }
 
-template <int EPI, int S>
+template <int EPI, int S, bool FEW>
 int launch_split_inst(WideParams &p, bool pdl, cudaStream_t s) {
   set_test(p, WIDE_TEST_SPLIT);
   static SmemLimit limit;
-  if (!limit.ensure(gemm_wide_split_kernel<EPI, S>, WS_SMEM)) return -6;
+  if (!limit.ensure(gemm_wide_split_kernel<EPI, S, FEW>, WS_SMEM)) return -6;
   if (!launch_allowed()) return 0;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(2 * S * p.m_tiles * p.n_tiles, 1, 1);
@@ -996,14 +1000,15 @@ int launch_split_inst(WideParams &p, bool pdl, cudaStream_t s) {
   at[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = pdl ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, gemm_wide_split_kernel<EPI, S>, p) == cudaSuccess ? 0 : -6;
+  return cudaLaunchKernelEx(&cfg, gemm_wide_split_kernel<EPI, S, FEW>, p) == cudaSuccess ? 0 : -6;
 }
 template <int EPI>
 int launch_split(WideParams &p, int S, bool pdl, cudaStream_t s) {
+  const bool few = p.half <= 96;
   switch (S) {
-    case 2: return launch_split_inst<EPI, 2>(p, pdl, s);
-    case 3: return launch_split_inst<EPI, 3>(p, pdl, s);
-    default: return launch_split_inst<EPI, 4>(p, pdl, s);
+    case 2: return few ? launch_split_inst<EPI, 2, true>(p, pdl, s) : launch_split_inst<EPI, 2, false>(p, pdl, s);
+    case 3: return few ? launch_split_inst<EPI, 3, true>(p, pdl, s) : launch_split_inst<EPI, 3, false>(p, pdl, s);
+    default: return few ? launch_split_inst<EPI, 4, true>(p, pdl, s) : launch_split_inst<EPI, 4, false>(p, pdl, s);
   }
 }
 
@@ -1097,11 +1102,9 @@ int wide_gemm_launch(TmaMaps *g, WideEpi epi, const WideGemmArgs &a, cudaStream_
     p.map_w[j] = *mw;
     p.O[j] = a.O[j];
   }
-  const CUtensorMap *mx = tma_maps_get(g, a.x, a.x_rows, a.I, W_HALF);
-  if (!mx) return -6;
-  p.map_x = *mx;
   p.rows = a.rows; p.KB = (a.I + TILE_K - 1) / TILE_K;
   p.m_tiles = (a.rows + WIDE_ROWS - 1) / WIDE_ROWS; p.n_tiles = n_tiles_of(epi, a.O, a.nw);
+  p.half = W_HALF;
   p.h0 = a.nw > 1 ? (a.O[0] + 127) / 128 : 1 << 30;
   p.h1 = a.nw > 2 ? p.h0 + (a.O[1] + 127) / 128 : 1 << 30;
   p.kind0 = a.nw == 3 ? 0 : 1;
@@ -1111,10 +1114,25 @@ int wide_gemm_launch(TmaMaps *g, WideEpi epi, const WideGemmArgs &a, cudaStream_
   p.seq = a.seq; p.kvpos = a.kvpos; p.pm = a.pm; p.G = a.G;
   p.act = a.act; p.out_b = a.out_b; p.ldo = a.ldo; p.out_f32 = a.out_f32; p.status = a.status; p.stamp = a.stamp;
   p.best_val = a.best_val; p.best_idx = a.best_idx; p.best_ld = a.best_ld;
+  int S = 1;
   if (epi == WIDE_SWIGLU) {
     plan_swiglu(a.O[0], p.KB, p.m_tiles, &p.fpt);
     if (a.form) p.fpt = a.form == 1 ? 0 : a.form;
     if (a.used) *a.used = p.fpt ? p.fpt : 1;
+  } else {
+    plan_split(epi, p.m_tiles * p.n_tiles, p.KB, &S);
+    if (a.form) S = a.form;
+    if (a.used) *a.used = S;
+  }
+  // One row tile of the split kernel is shared evenly: with 168 rows each CTA of a pair fetches, parks and adds up 88 or 80 of them
+  // instead of 128 or 40 (in whole groups of eight, as the operand lies in shared memory).  Replayed step, 8B shapes (us, before -> now):
+  // 132 rows QKV 19.6 -> 17.7, O 17.4 -> 15.3, down 32.9 -> 31.0; 168 rows 19.6 -> 18.1, 18.6 -> 16.3, 34.5 -> 31.9; 192 rows 20.5 -> 18.7,
+  // 18.3 -> 16.1, 34.8 -> 32.4; 240 rows the same.
+  if (p.m_tiles == 1 && S > 1) p.half = std::min(W_HALF, ((a.rows + 1) / 2 + 7) & ~7);
+  const CUtensorMap *mx = tma_maps_get(g, a.x, a.x_rows, a.I, p.half);
+  if (!mx) return -6;
+  p.map_x = *mx;
+  if (epi == WIDE_SWIGLU) {
     if (p.fpt) {
       for (int j = 0; j < 2; j++) {
         const CUtensorMap *mw = tma_maps_get(g, a.w[j], a.O[j], a.I, p.fpt / 2);
@@ -1124,12 +1142,6 @@ int wide_gemm_launch(TmaMaps *g, WideEpi epi, const WideGemmArgs &a, cudaStream_
       p.n_tiles = (a.O[0] + p.fpt - 1) / p.fpt;
       return launch_swiglu(p, a.pdl, s);
     }
-  }
-  int S = 1;
-  plan_split(epi, p.m_tiles * p.n_tiles, p.KB, &S);
-  if (epi != WIDE_SWIGLU) {
-    if (a.form) S = a.form;
-    if (a.used) *a.used = S;
   }
   if (S > 1) {
     switch (epi) {

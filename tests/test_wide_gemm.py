@@ -59,3 +59,16 @@ def test_unsupported_shapes_are_refused(rows, O, I, form):
     x, w = (torch.zeros(n, I, dtype=torch.bfloat16, device="cuda") for n in (rows, O))
     with pytest.raises(sb.SpecError):
         sb.gemm_wide(x, w, form=form)
+
+
+ROWS = [8, 9, 16, 130, 152, 185, 192, 193, 208, 240]          # one row tile shared evenly by the CTAs of a pair, in whole groups of eight rows
+
+
+@pytest.mark.parametrize("form", [2, 3, 4])
+@pytest.mark.parametrize("rows", ROWS)
+def test_one_row_tile_shared_evenly_vs_oracle(rows, form):
+    x, w = _rand(rows, (rows, 1160), (264, 1160))
+    out, used = sb.gemm_wide(x.cuda(), w.cuda(), form=form)
+    assert used == form
+    # outputs of order 1 from exact products: fp32 sums of 1160 of them, in any order
+    assert np.abs(out.cpu().numpy() - po.linear(w, x.float().numpy())).max() < 1e-4
