@@ -490,12 +490,11 @@ template <typename T> struct Sched {
   // weight-streaming kernel's tiles feed the tensor pipe with: it re-reads the 32 KB activation k-block for every 128
   // features and spends as long in its 256-row epilogues as in its loops.  These passes take the row-major kernel.  Alone (8B
   // shapes, launches from a graph without the passes' epilogues, weight-streaming / row-major, us): QKV 23.4 / 19.2 at 144 rows, 30.9 / 20.0
-  // at 256; O 16.2 / 17.5, 19.5 / 18.5; down 30.8 / 32.6, 34.9 / 34.3; gate/up 56.7 / 57.8 at 192 and 58.9 / 53.9 at 256.
-  // Gate/up takes it from 193 rows on.  In the replayed step, at the full clock (us): 13B shapes at 150 rows 62.8 / 75.7, 70B shapes at
-  // 180 rows 204.8 / 219.9, 8B shapes at 180 rows 53.5 / 54.9; only at the clock a long batch of the 8B shapes leaves (1.4 GHz) is it
-  // the other way round, 72.5 / 70 at 168 rows.
+  // at 256; O 16.2 / 17.5, 19.5 / 18.5; down 30.8 / 32.6, 34.9 / 34.3.  Gate/up in the replayed step (weight-streaming pair kernel /
+  // row-major, us): 8B shapes 132 rows 47.6 / 48.8, 160 49.6 / 49.3, 192 50.9 / 49.2, 208 54.7 / 49.5, 240 54.6 / 49.4, 256 58.3 / 49.1; 13B shapes
+  // 150 rows 56.3 / 54.2, 250 67.0 / 55.1; 70B shapes 180 rows 192 / 184, 240 220 / 187.
   bool row_major(FusedEpi epi, const FusedGemmArgs &a) const {
-    return a.rows > (epi == EPI_SWIGLU ? 192 : 128) && !a.withhold && !fused_gemm_pairs() && epi != EPI_TOPK && (epi != EPI_QKV || a.hd == 128);
+    return a.rows > 128 && !a.withhold && !fused_gemm_pairs() && epi != EPI_TOPK && (epi != EPI_QKV || a.hd == 128);
   }
   static WideEpi wide_epi(FusedEpi e) {
     return e == EPI_RESID ? WIDE_RESID : e == EPI_QKV ? WIDE_QKV : e == EPI_SWIGLU ? WIDE_SWIGLU : e == EPI_ARGMAX ? WIDE_ARGMAX : WIDE_F32;

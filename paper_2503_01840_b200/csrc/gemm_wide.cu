@@ -51,7 +51,7 @@ constexpr int W_PAIRS = 74;                               // 148 SMs
 struct alignas(64) WideParams {
   CUtensorMap map_x, map_w[3];
   int rows, KB, m_tiles, n_tiles;
-  int half;                      // rows of a CTA: 128, or with one row tile half of the rows there are (split kernel)
+  int half;                      // rows of a CTA: 128, or with one row tile half of the rows there are (split and gate/up kernel)
   int h0, h1;                    // half tiles [0,h0) belong to w0, [h0,h1) to w1, the rest to w2
   int O[3];
   int kind0;                     // WIDE_QKV: what w0 is (0 q, 1 k)
@@ -389,6 +389,7 @@ __global__ void __launch_bounds__(W_THREADS, 1) gemm_wide_kernel(const __grid_co
         const int f0 = nt * 128 + half * 64;
 #pragma unroll
         for (int c = 0; c < 2; c++) {
+          if (!any_row) break;                                   // uniform over the warp
           uint32_t g[32], u[32];
           tmem_ld32(ta + half * 64 + c * 32, g);
           tmem_ld32(ta + 128 + half * 64 + c * 32, u);
@@ -400,7 +401,8 @@ __global__ void __launch_bounds__(W_THREADS, 1) gemm_wide_kernel(const __grid_co
               float r[2];
 #pragma unroll
               for (int z = 0; z < 2; z++) {
-                const float gv = __uint_as_float(g[8 * j + 2 * e + z]) * inv, uv = __uint_as_float(u[8 * j + 2 * e + z]) * inv;
+                // (a lane without a row divides 1: see gemm_wide_swiglu_kernel)
+                const float gv = row < p.rows ? __uint_as_float(g[8 * j + 2 * e + z]) * inv : 1.0f, uv = __uint_as_float(u[8 * j + 2 * e + z]) * inv;
                 r[z] = (gv / (1.0f + expf(-gv))) * uv;
               }
               w[e] = pack2(r[0], r[1]);
@@ -795,6 +797,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1) gemm_wide_swiglu_kernel(const _
   const int xr = (int)(crank & 1u);
   const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
   const int ntiles = p.m_tiles * p.n_tiles, KB = p.KB;
+  const uint32_t fill = 2u * (uint32_t)(p.half * TILE_K * 2 + 2 * b_bytes);    // bytes of a stage, both CTAs
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < stages; i++) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
@@ -823,7 +826,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1) gemm_wide_swiglu_kernel(const _
     bool ok = !__any_sync(0xffffffffu, *abort_flag != 0), first = true;
     for (int t = pair; t < ntiles && ok; t += n_pairs) {
       const int mt = t % p.m_tiles, nt = t / p.m_tiles;
-      const int wrow = nt * fpt + xr * (fpt / 2), xrow = mt * WIDE_ROWS + xr * W_HALF;
+      const int wrow = nt * fpt + xr * (fpt / 2), xrow = mt * WIDE_ROWS + xr * p.half;
       int kb = 0;
       if (first) {
         first = false;
@@ -831,7 +834,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1) gemm_wide_swiglu_kernel(const _
         if (elect_one())
           for (int i = 0; i < npre; i++) {
             const uint32_t fb = mapa_u32(smem_u32(&full[i]), 0u);
-            if (xr == 0) mbar_expect_tx(&full[i], 2 * stage);
+            if (xr == 0) mbar_expect_tx(&full[i], fill);
             tma_load_2d_pair_hint(ring + i * stage + W_A_BYTES, &p.map_w[0], i * TILE_K, wrow, fb, pol);
             tma_load_2d_pair_hint(ring + i * stage + W_A_BYTES + b_bytes, &p.map_w[1], i * TILE_K, wrow, fb, pol);
           }
@@ -848,7 +851,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1) gemm_wide_swiglu_kernel(const _
         if (elect_one()) {
           unsigned char *a = ring + st * stage;
           const uint32_t fb = mapa_u32(smem_u32(&full[st]), 0u);
-          if (xr == 0) mbar_expect_tx(&full[st], 2 * stage);
+          if (xr == 0) mbar_expect_tx(&full[st], fill);
           const int kx = kb * TILE_K;
           tma_load_2d_pair_hint(a + W_A_BYTES, &p.map_w[0], kx, wrow, fb, pol);
           tma_load_2d_pair_hint(a + W_A_BYTES + b_bytes, &p.map_w[1], kx, wrow, fb, pol);
@@ -906,8 +909,9 @@ __global__ void __launch_bounds__(WS_THREADS, 1) gemm_wide_swiglu_kernel(const _
     int it = 0;
     for (int t = pair; t < ntiles; t += n_pairs, it++) {
       const int mt = t % p.m_tiles, nt = t / p.m_tiles;
-      const int row = mt * WIDE_ROWS + xr * W_HALF + quarter * 32 + lane;
-      const float inv = row < p.rows ? row_scale(p, row) : 1.0f;
+      const int lr = quarter * 32 + lane, row = mt * WIDE_ROWS + xr * p.half + lr;
+      const bool mine = lr < p.half && row < p.rows;             // the other lanes' accumulators hold zeros or anything
+      const float inv = mine ? row_scale(p, row) : 1.0f;
       const bool ok = __all_sync(0xffffffffu, mbar_wait_warp(tfull, (uint32_t)(it & 1), p.spin) && !*abort_flag);
       if (!ok) {
         if (lane == 0) { *abort_flag = 1; set_status(p.status, ST_TIMEOUT, 263, blockIdx.x, t); }
@@ -915,8 +919,9 @@ __global__ void __launch_bounds__(WS_THREADS, 1) gemm_wide_swiglu_kernel(const _
       }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t ta = tmem_base + ((uint32_t)(quarter * 32) << 16);
+      const int runs = __any_sync(0xffffffffu, mine) ? fpt / 16 : 0;
 #pragma unroll 1
-      for (int c = part; c < fpt / 16; c += 4) {                 // the four warps of a quarter take alternate runs of 16 features
+      for (int c = part; c < runs; c += 4) {                 // the four warps of a quarter take alternate runs of 16 features
         uint32_t g[16], u[16], w[8];
         tmem_ld16(ta + c * 16, g);
         tmem_ld16(ta + 256 + c * 16, u);
@@ -925,15 +930,16 @@ __global__ void __launch_bounds__(WS_THREADS, 1) gemm_wide_swiglu_kernel(const _
           float r[2];
 #pragma unroll
           for (int z = 0; z < 2; z++) {
-            const float gv = __uint_as_float(g[2 * e + z]) * inv, uv = __uint_as_float(u[2 * e + z]) * inv;
+            // (A lane without a row divides 1: zeros and the like send the whole warp through the division's slow path, 8 us of a launch.)
+            const float gv = mine ? __uint_as_float(g[2 * e + z]) * inv : 1.0f, uv = __uint_as_float(u[2 * e + z]) * inv;
             r[z] = (gv / (1.0f + expf(-gv))) * uv;
           }
           w[e] = pack2(r[0], r[1]);
         }
         const int f = nt * fpt + c * 16;
         bf16 *dst = p.act + (size_t)row * p.O[0] + f;
-        if (row < p.rows && f < p.O[0]) *(uint4 *)dst = make_uint4(w[0], w[1], w[2], w[3]);
-        if (row < p.rows && f + 8 < p.O[0]) *(uint4 *)(dst + 8) = make_uint4(w[4], w[5], w[6], w[7]);
+        if (mine && f < p.O[0]) *(uint4 *)dst = make_uint4(w[0], w[1], w[2], w[3]);
+        if (mine && f + 8 < p.O[0]) *(uint4 *)(dst + 8) = make_uint4(w[4], w[5], w[6], w[7]);
       }
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
@@ -1057,14 +1063,20 @@ long long plan_split(WideEpi epi, int tiles, int KB, int *S) {
   return best;
 }
 
-// Gate/up: features per tile of the launch (0: the persistent kernel with 128) and its cost
+// Gate/up: features per tile of the launch (0: the persistent kernel with 128) and its cost.  A k-block of a tile fetches 128 rows of
+// activations and f of weights per CTA, and that fill bounds it: its time goes with 96 + f, not with f, so narrow tiles cost more than their
+// share.  Row-major kernel alone at 168 rows, own choice of the older estimate (f / 128) / of this one (us): F 14336 57.6 / 57.6, 13824 x
+// 5120 83.2 / 62.1, 13824 x 4096 71.4 / 53.2, 11008 57.7 / 47.0, 16384 64.1 / 61.8, 28672 x 8192 227.8 / 198.4.  The persistent kernel hides its
+// epilogues; with one row tile its waves are bound by the fill too (a third on top: F 14336 68, 18432 x 6144 96 against 95 with 256).  512 rows,
+// older choice / this one: F 14336 80: 132.7 / persistent: 103.8, 11008 80: 106.8 / 82.4; 768 rows 11008 64: 155.9 / 108.3.
 long long plan_swiglu(int F, int KB, int m_tiles, int *fpt) {
   const int t128 = (F + 127) / 128 * m_tiles;
   long long best = (long long)((t128 + W_PAIRS - 1) / W_PAIRS) * KB + W_COST_TAIL;
+  if (m_tiles == 1) best = best * 4 / 3;
   *fpt = 0;
   for (int f = 64; f <= WG_MAX_FPT; f += 16) {       // N of an M = 256 MMA is a multiple of 16
     const int tiles = (F + f - 1) / f * m_tiles;
-    const long long c = (long long)((tiles + W_PAIRS - 1) / W_PAIRS) * ((long long)KB * f / 128 + W_COST_TAIL * f / 128);
+    const long long c = (long long)((tiles + W_PAIRS - 1) / W_PAIRS) * ((long long)KB * (96 + f) / 160 + W_COST_TAIL * f / 128);
     if (c < best) { best = c; *fpt = f; }
   }
   return best;
@@ -1124,11 +1136,11 @@ int wide_gemm_launch(TmaMaps *g, WideEpi epi, const WideGemmArgs &a, cudaStream_
     if (a.form) S = a.form;
     if (a.used) *a.used = S;
   }
-  // One row tile of the split kernel is shared evenly: with 168 rows each CTA of a pair fetches, parks and adds up 88 or 80 of them
+  // One row tile of the split and the gate/up kernel is shared evenly: with 168 rows each CTA of a pair fetches, parks and adds up 88 or 80 of them
   // instead of 128 or 40 (in whole groups of eight, as the operand lies in shared memory).  Replayed step, 8B shapes (us, before -> now):
   // 132 rows QKV 19.6 -> 17.7, O 17.4 -> 15.3, down 32.9 -> 31.0; 168 rows 19.6 -> 18.1, 18.6 -> 16.3, 34.5 -> 31.9; 192 rows 20.5 -> 18.7,
   // 18.3 -> 16.1, 34.8 -> 32.4; 240 rows the same.
-  if (p.m_tiles == 1 && S > 1) p.half = std::min(W_HALF, ((a.rows + 1) / 2 + 7) & ~7);
+  if (p.m_tiles == 1 && (S > 1 || p.fpt)) p.half = std::min(W_HALF, ((a.rows + 1) / 2 + 7) & ~7);
   const CUtensorMap *mx = tma_maps_get(g, a.x, a.x_rows, a.I, p.half);
   if (!mx) return -6;
   p.map_x = *mx;

@@ -72,3 +72,28 @@ def test_one_row_tile_shared_evenly_vs_oracle(rows, form):
     assert used == form
     # outputs of order 1 from exact products: fp32 sums of 1160 of them, in any order
     assert np.abs(out.cpu().numpy() - po.linear(w, x.float().numpy())).max() < 1e-4
+
+
+@pytest.mark.parametrize("form", [1, 64, 208])
+@pytest.mark.parametrize("rows", ROWS + [300])
+def test_gate_up_of_a_shared_row_tile_vs_oracle(rows, form):
+    """Some rows of zeros and some whose gates leave the exponential's range among them."""
+    x, wg, wu = _rand(rows + 1, (rows, 320), (424, 320), (424, 320))
+    x[3], x[rows - 1] = 0.0, 300.0
+    out, used = sb.gemm_wide(x.cuda(), wg.cuda(), wu.cuda(), form=form)
+    assert used == form
+    xf = x.float().numpy()
+    with np.errstate(over="ignore"):
+        g, u = po.linear(wg, xf), po.linear(wu, xf)
+        ref = po.swiglu(g, u)
+    # one bf16 rounding of the result, and fp32 sums of 320 products whose size the last row's values raise to 300
+    mag = 1e-4 * np.maximum(1.0, np.abs(xf).max(1, keepdims=True)) * np.maximum(1.0, np.abs(u))
+    assert (np.abs(out.float().cpu().numpy() - ref) - 2.0 ** -8 * np.abs(ref) - mag).max() < 0
+
+
+@pytest.mark.parametrize("F,I,want", [(14336, 4096, 208), (13824, 5120, 192), (11008, 4096, 160), (28672, 8192, 208)])
+def test_gate_up_widths_of_one_row_tile(F, I, want):
+    """One wave (or two) of the fewest features per tile, not several waves of narrow ones; from two row tiles on the persistent kernel."""
+    x, w = (torch.zeros(n, I, dtype=torch.bfloat16, device="cuda") for n in (512, F))
+    assert sb.gemm_wide(x[:168].contiguous(), w, w)[1] == want
+    assert sb.gemm_wide(x, w, w)[1] == 1
