@@ -48,6 +48,7 @@ struct alignas(64) FusedParams {
   CUtensorMap map_x;
   int tiles0, tiles1;          // tile index ranges of the weights: [0,tiles0) w0, [tiles0,tiles1) w1, rest w2
   int O[3];
+  int nrt;                                 // gemm_swiglu_pair_kernel: rows of its MMAs, the rows there are in whole 16s
   int rows, KB, S, stages, ctrl_off;       // S = K slices = cluster size (CTA pairs: half of it)
   int chunk;                               // rows per epilogue round
   const float *ssq_in; int ssq_in_tiles, ssq_ld; float inv_k_in, eps;
@@ -797,8 +798,7 @@ __global__ void __launch_bounds__(fused_threads(NT, EPI), EPI == EPI_TOPK || EPI
 constexpr int PAIR_THREADS = 512, PAIR_GROUPS = PAIR_THREADS / 128;
 template <int NT, bool DUO = false>
 __global__ void __launch_bounds__(PAIR_THREADS) gemm_swiglu_pair_kernel(const __grid_constant__ FusedParams p) {
-  constexpr int B_BYTES = (DUO ? NT / 2 : NT) * TILE_K * 2;
-  constexpr int STAGE = 2 * A_BYTES + B_BYTES;
+  const int xrows = DUO ? p.nrt / 2 : p.nrt, STAGE = 2 * A_BYTES + xrows * TILE_K * 2;     // activation rows of this CTA, bytes of a stage
   constexpr int TMEM_COLS = 2 * NT;
   static_assert(TMEM_COLS <= 512, "two accumulators must fit the tensor memory");
   extern __shared__ unsigned char smem_raw[];
@@ -862,7 +862,7 @@ __global__ void __launch_bounds__(PAIR_THREADS) gemm_swiglu_pair_kernel(const __
     if (elect_one()) {
       if (p.stamp) atomicMin(p.stamp, global_ns());
       for (int i = 0; i < npre; i++)
-        tma_load_2d_pair(tiles + i * STAGE + 2 * A_BYTES, &p.map_x, i * TILE_K, xr * (NT / 2), mapa_u32(smem_u32(&full[i]), 0u));
+        tma_load_2d_pair(tiles + i * STAGE + 2 * A_BYTES, &p.map_x, i * TILE_K, xr * xrows, mapa_u32(smem_u32(&full[i]), 0u));
     }
     __syncwarp();
     int i = npre, st = 0;
@@ -875,7 +875,7 @@ __global__ void __launch_bounds__(PAIR_THREADS) gemm_swiglu_pair_kernel(const __
         if (xr == 0) mbar_expect_tx(&full[st], 2 * STAGE);
         tma_load_2d_pair_hint(a, &p.map_w[0], i * TILE_K, tm * TILE_M, fb, pol);
         tma_load_2d_pair_hint(a + A_BYTES, &p.map_w[1], i * TILE_K, tm * TILE_M, fb, pol);
-        tma_load_2d_pair(a + 2 * A_BYTES, &p.map_x, i * TILE_K, xr * (NT / 2), fb);
+        tma_load_2d_pair(a + 2 * A_BYTES, &p.map_x, i * TILE_K, xr * xrows, fb);
       }
       __syncwarp();
       if (++st == stages) { st = 0; ph ^= 1u; }
@@ -919,7 +919,7 @@ __global__ void __launch_bounds__(PAIR_THREADS) gemm_swiglu_pair_kernel(const __
     if (DUO && warp == 1) {
       // ---- MMA issuer warp of a CTA pair (even CTA only): M = 256 over both CTAs' gate tiles, then both up tiles
       if (xr == 0) {
-        constexpr uint32_t idesc = umma_idesc_m(NT, 2 * TILE_M);
+        const uint32_t idesc = umma_idesc_m(p.nrt, 2 * TILE_M);
         const uint32_t partner_base = ld_peer_u32(smem_u32(tmem_slot), 1u);
         if (partner_base != tmem_base) { *abort_flag = 1; set_status(p.status, ST_TIMEOUT, 226, blockIdx.x, (int)partner_base); }
         const uint64_t desc0 = umma_desc_sw128(smem_u32(tiles));
@@ -951,7 +951,7 @@ __global__ void __launch_bounds__(PAIR_THREADS) gemm_swiglu_pair_kernel(const __
       }
     } else if (!DUO && warp == 1) {
       // ---- MMA issuer warp (the elected lane issues): gate accumulator at column 0, up accumulator at column NT
-      constexpr uint32_t idesc = umma_idesc(NT);
+      const uint32_t idesc = umma_idesc(p.nrt);
       const uint64_t desc0 = umma_desc_sw128(smem_u32(tiles));
       int i = 0, st = 0;
       uint32_t ph = 0, ready = 0;
@@ -1002,10 +1002,10 @@ __global__ void __launch_bounds__(PAIR_THREADS) gemm_swiglu_pair_kernel(const __
 
   // ---- epilogue: thread = feature f (tensor-memory lane), 16 rows (columns) of both accumulators at a time
   const int o = tm * TILE_M + (threadIdx.x & (TILE_M - 1));
-  const int hw = threadIdx.x >> 7;               // which share of the rows (accumulator columns) this thread converts
+  const int hw = threadIdx.x >> 7;               // which share of the rows (accumulator columns) this thread converts: every fourth 16
   if (good) {
 #pragma unroll 1
-    for (int cc = hw * (NT / PAIR_GROUPS); cc < p.rows && cc < (hw + 1) * (NT / PAIR_GROUPS); cc += 16) {
+    for (int cc = hw * 16; cc < p.rows; cc += PAIR_GROUPS * 16) {
       uint32_t g[16], u[16];
       tmem_ld16(tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)cc, g);
       tmem_ld16(tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(NT + cc), u);
@@ -1281,12 +1281,11 @@ int fused_gemm_launch(TmaMaps *g, FusedEpi epi, const FusedGemmArgs &a, cudaStre
     // wide rows: one CTA per (gate tile, up tile) pair sharing the activation tiles; optionally two such CTAs as a
     // CTA pair that also share the activation k-block (each loads half of the rows)
     const bool duo2 = g_pairs_swiglu && (p.tiles0 % 2) == 0;
-    const int stage2 = 2 * A_BYTES + (duo2 ? 128 : 256) * TILE_K * 2;
-    if (duo2) {
-      const CUtensorMap *mxh = tma_maps_get(g, a.x, a.rows, a.I, 128);
-      if (!mxh) return -6;
-      p.map_x = *mxh;
-    }
+    p.nrt = (a.rows + 15) & ~15;                 // N of an MMA is a multiple of 16
+    const int xrows = duo2 ? p.nrt / 2 : p.nrt, stage2 = 2 * A_BYTES + xrows * TILE_K * 2;
+    const CUtensorMap *mxh = tma_maps_get(g, a.x, a.rows, a.I, xrows);
+    if (!mxh) return -6;
+    p.map_x = *mxh;
     p.stages = std::max(2, std::min(SMEM_ONE / stage2, pl.KB));
     p.S = 1;
     p.ctrl_off = (p.stages * stage2 + 1023) & ~1023;
