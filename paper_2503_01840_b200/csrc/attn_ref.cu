@@ -19,102 +19,146 @@ template <bool VEC> __device__ __forceinline__ float4 load4(const bf16 *p) {
   return make_float4(to_f32(p[0]), to_f32(p[1]), to_f32(p[2]), to_f32(p[3]));
 }
 
-// Bound by latency (a row attends tens to hundreds of keys): four threads share a key's dot product, so that a key row is
-// read in 64-byte runs with all its loads in flight, and the value pass splits the KEYS over the threads that are left
-// beside hd / 4 dimension groups instead of walking them one after the other (70 keys, 16 CTAs: 45 -> 14 us, cold).
+// Bound by latency: a row attends tens to hundreds of keys, and a launch has a few dozen CTAs.  So there are four dependent round trips
+// and no more for up to 128 keys: metadata, page ids, K and V rows together, output.  Four threads share a key's dot product (256 keys a round,
+// their page ids and then their rows requested at once), and a thread's first V_AHEAD values, whose addresses need no score, are
+// requested before the scores.  The value pass splits the keys over the threads that are left beside hd / 4 dimension groups.
+// Tiny fp32 model, replayed step with the register-resident top-K: 214 -> 189 us at 64 tokens,
+// 275 -> 213 at 250, 386 -> 253 at 600.
+constexpr int AR_THREADS = 256, V_AHEAD = 8;
 template <typename T, bool VEC>
-__global__ void __launch_bounds__(128) attn_ref_kernel(const T *__restrict__ q, KvPool pool, PageMap pm, RowMeta m,
+__global__ void __launch_bounds__(AR_THREADS) attn_ref_kernel(const T *__restrict__ q, KvPool pool, PageMap pm, RowMeta m,
                                                        int tail_len, T *__restrict__ out, int H, int G, int hd) {
   pdl_wait();
   pdl_trigger();
   extern __shared__ __align__(16) float smem[];
   float *qs = smem;            // [hd]
   float *sc = smem + hd;       // [ctx + tail_len]
-  float4 *part = (float4 *)smem;   // [128], over both once they are done with
-  __shared__ float red[4];
+  float4 *part = (float4 *)smem;   // [AR_THREADS], over both once they are done with
+  __shared__ float red[2][AR_THREADS / 32];
   const int r = blockIdx.x, h = blockIdx.y, g = h / (H / G);
-  const int seq = m.seq[r];
+  const int seq = m.seq[r], ctx = m.ctx[r], tb = m.tail_base[r];
+  const uint64_t mlo = m.mask_lo[r], mhi = m.mask_hi[r];
+  for (int i = threadIdx.x; i < hd; i += AR_THREADS) qs[i] = to_f32(q[((size_t)r * H + h) * hd + i]);
   T *o = out + ((size_t)r * H + h) * hd;
   if (seq < 0) {
-    for (int i = threadIdx.x; i < hd; i += blockDim.x) o[i] = from_f32<T>(0.0f);
+    for (int i = threadIdx.x; i < hd; i += AR_THREADS) o[i] = from_f32<T>(0.0f);
     return;
   }
-  const int ctx = m.ctx[r], tb = m.tail_base[r];
-  const uint64_t mlo = m.mask_lo[r], mhi = m.mask_hi[r];
-  const int nk = ctx + tail_len;
+  const int nk = ctx + tail_len, ps = pm.page_size, psh = (ps & (ps - 1)) == 0 ? __ffs(ps) - 1 : -1;
   const T *Kp = (const T *)pool.k, *Vp = (const T *)pool.v;
-  for (int i = threadIdx.x; i < hd; i += blockDim.x) qs[i] = to_f32(q[((size_t)r * H + h) * hd + i]);
+  const int32_t *tbl = pm.table + (size_t)seq * pm.pages_per_seq;
+  // first element of the row of a position, from its page
+  auto page_of = [&](int pos) { return tbl[psh >= 0 ? pos >> psh : pos / ps]; };
+  auto row_at = [&](int page, int pos) { return (((size_t)page * G + g) * ps + (psh >= 0 ? pos & (ps - 1) : pos % ps)) * hd; };
+  auto pos_of = [&](int j) { return j < ctx ? j : tb + (j - ctx); };
+  auto visible = [&](int j) {
+    const int t = j - ctx;
+    return j < nk && (t < 0 || (t < 64 ? ((mlo >> t) & 1ull) : ((mhi >> (t - 64)) & 1ull)));
+  };
+  const int n_dim = hd >> 2;
+  const int n_grp = n_dim <= AR_THREADS ? AR_THREADS / n_dim : 0, dim = n_grp ? threadIdx.x % n_dim : 0, grp = n_grp ? threadIdx.x / n_dim : 0;
+  const bool has_v = n_grp && grp < n_grp;               // thread = (four dimensions, every n_grp-th key)
+  // ---- page ids of the first keys and of this thread's first values, then those values
+  constexpr int KR = 4;                                  // rounds of AR_THREADS / 4 keys in flight
+  const int sub = threadIdx.x & 3, key0 = threadIdx.x >> 2;
+  int kpage[KR], vpage[V_AHEAD];
+  auto key_pages = [&](int j0) {
+#pragma unroll
+    for (int u = 0; u < KR; u++) {
+      const int j = j0 + u * (AR_THREADS / 4) + key0;
+      kpage[u] = visible(j) ? page_of(pos_of(j)) : -1;
+    }
+  };
+  key_pages(0);
+#pragma unroll
+  for (int u = 0; u < V_AHEAD; u++) {
+    const int j = grp + u * n_grp;
+    vpage[u] = has_v && visible(j) ? page_of(pos_of(j)) : -1;
+  }
+  float4 vv[V_AHEAD];
+#pragma unroll
+  for (int u = 0; u < V_AHEAD; u++) vv[u] = vpage[u] >= 0 ? load4<VEC>(Vp + row_at(vpage[u], pos_of(grp + u * n_grp)) + dim * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
   __syncthreads();
   const float scale = 1.0f / sqrtf((float)hd);
   float mx = -INFINITY;
-  const int sub = threadIdx.x & 3;
-  for (int j0 = 0; j0 < nk; j0 += 32) {                  // 32 keys per round: all four threads of a key take part
-    const int j = j0 + (threadIdx.x >> 2);
-    bool vis = j < nk;
-    int pos = j;
-    if (j >= ctx) {
-      const int t = j - ctx;
-      vis = vis && (t < 64 ? ((mlo >> t) & 1ull) : ((mhi >> (t - 64)) & 1ull));
-      pos = tb + t;
+  for (int j0 = 0; j0 < nk; j0 += KR * (AR_THREADS / 4)) {      // all four threads of a key take part
+    if (j0 > 0) key_pages(j0);
+    const T *kr[KR];
+    float d[KR];
+#pragma unroll
+    for (int u = 0; u < KR; u++) {
+      kr[u] = kpage[u] >= 0 ? Kp + row_at(kpage[u], pos_of(j0 + u * (AR_THREADS / 4) + key0)) : nullptr;
+      d[u] = 0.0f;
     }
-    float d = 0.0f;
-    if (vis) {
-      const T *kr = Kp + kv_offset(pm, seq, pos, g, G, hd);
 #pragma unroll 4
-      for (int i = sub * 4; i < hd; i += 16) {            // hd is a multiple of 16
-        const float4 a = load4<VEC>(kr + i), b = *(const float4 *)(qs + i);
-        d = fmaf(b.x, a.x, fmaf(b.y, a.y, fmaf(b.z, a.z, fmaf(b.w, a.w, d))));
-      }
+    for (int i = sub * 4; i < hd; i += 16) {              // hd is a multiple of 16
+      const float4 b = *(const float4 *)(qs + i);
+#pragma unroll
+      for (int u = 0; u < KR; u++)
+        if (kr[u]) {
+          const float4 a = load4<VEC>(kr[u] + i);
+          d[u] = fmaf(b.x, a.x, fmaf(b.y, a.y, fmaf(b.z, a.z, fmaf(b.w, a.w, d[u]))));
+        }
     }
-    d += __shfl_xor_sync(0xffffffffu, d, 1);
-    d += __shfl_xor_sync(0xffffffffu, d, 2);
-    const float s = vis ? d * scale : -INFINITY;
-    if (sub == 0 && j < nk) sc[j] = s;
-    mx = fmaxf(mx, s);
+#pragma unroll
+    for (int u = 0; u < KR; u++) {
+      const int j = j0 + u * (AR_THREADS / 4) + key0;
+      float t = d[u] + __shfl_xor_sync(0xffffffffu, d[u], 1);
+      t += __shfl_xor_sync(0xffffffffu, t, 2);
+      const float s = kpage[u] >= 0 ? t * scale : -INFINITY;
+      if (sub == 0 && j < nk) sc[j] = s;
+      mx = fmaxf(mx, s);
+    }
   }
   for (int off = 16; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
+  if ((threadIdx.x & 31) == 0) red[0][threadIdx.x >> 5] = mx;
   __syncthreads();
-  mx = fmaxf(fmaxf(red[0], red[1]), fmaxf(red[2], red[3]));
-  __syncthreads();
+  mx = red[0][0];
+#pragma unroll
+  for (int w = 1; w < AR_THREADS / 32; w++) mx = fmaxf(mx, red[0][w]);
   float sum = 0.0f;
-  for (int j = threadIdx.x; j < nk; j += blockDim.x) {
+  for (int j = threadIdx.x; j < nk; j += AR_THREADS) {
     float e = (sc[j] == -INFINITY) ? 0.0f : expf(sc[j] - mx);
     sc[j] = e;
     sum += e;
   }
   for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = sum;
+  if ((threadIdx.x & 31) == 0) red[1][threadIdx.x >> 5] = sum;
   __syncthreads();
-  sum = red[0] + red[1] + red[2] + red[3];
+  sum = red[1][0];
+#pragma unroll
+  for (int w = 1; w < AR_THREADS / 32; w++) sum += red[1][w];
   const float inv = 1.0f / sum;
-  const int n_dim = hd >> 2;
-  if (n_dim > 128) {                                      // more groups of four dimensions than threads: a thread takes several, over all keys
-    for (int dim = threadIdx.x; dim < n_dim; dim += 128) {
+  if (!n_grp) {                                           // more groups of four dimensions than threads: a thread takes several, over all keys
+    for (int dm = threadIdx.x; dm < n_dim; dm += AR_THREADS) {
       float4 acc = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
 #pragma unroll 4
       for (int j = 0; j < nk; j++) {
         const float p = sc[j];
         if (p == 0.0f) continue;
-        const int pos = j < ctx ? j : tb + (j - ctx);
-        const float4 a = load4<VEC>(Vp + kv_offset(pm, seq, pos, g, G, hd) + dim * 4);
+        const float4 a = load4<VEC>(Vp + row_at(page_of(pos_of(j)), pos_of(j)) + dm * 4);
         acc.x = fmaf(p, a.x, acc.x); acc.y = fmaf(p, a.y, acc.y); acc.z = fmaf(p, a.z, acc.z); acc.w = fmaf(p, a.w, acc.w);
       }
-      o[dim * 4] = from_f32<T>(acc.x * inv); o[dim * 4 + 1] = from_f32<T>(acc.y * inv);
-      o[dim * 4 + 2] = from_f32<T>(acc.z * inv); o[dim * 4 + 3] = from_f32<T>(acc.w * inv);
+      o[dm * 4] = from_f32<T>(acc.x * inv); o[dm * 4 + 1] = from_f32<T>(acc.y * inv);
+      o[dm * 4 + 2] = from_f32<T>(acc.z * inv); o[dm * 4 + 3] = from_f32<T>(acc.w * inv);
     }
     return;
   }
-  // values: thread = (four dimensions, every n_grp-th key)
-  const int n_grp = 128 / n_dim, dim = threadIdx.x % n_dim, grp = threadIdx.x / n_dim;
   float4 acc = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-  if (grp < n_grp) {
+  if (has_v) {
+#pragma unroll
+    for (int u = 0; u < V_AHEAD; u++) {
+      const int j = grp + u * n_grp;
+      const float p = j < nk ? sc[j] : 0.0f;
+      if (p == 0.0f) continue;                            // a hidden key counts nothing, whatever its value holds
+      acc.x = fmaf(p, vv[u].x, acc.x); acc.y = fmaf(p, vv[u].y, acc.y); acc.z = fmaf(p, vv[u].z, acc.z); acc.w = fmaf(p, vv[u].w, acc.w);
+    }
 #pragma unroll 4
-    for (int j = grp; j < nk; j += n_grp) {
+    for (int j = grp + V_AHEAD * n_grp; j < nk; j += n_grp) {
       const float p = sc[j];
       if (p == 0.0f) continue;
-      const int pos = j < ctx ? j : tb + (j - ctx);
-      const float4 a = load4<VEC>(Vp + kv_offset(pm, seq, pos, g, G, hd) + dim * 4);
+      const float4 a = load4<VEC>(Vp + row_at(page_of(pos_of(j)), pos_of(j)) + dim * 4);
       acc.x = fmaf(p, a.x, acc.x); acc.y = fmaf(p, a.y, acc.y); acc.z = fmaf(p, a.z, acc.z); acc.w = fmaf(p, a.w, acc.w);
     }
   }
@@ -133,7 +177,7 @@ __global__ void __launch_bounds__(128) attn_ref_kernel(const T *__restrict__ q, 
 
 size_t attn_ref_smem_bytes(int max_keys, int hd) {
   const size_t n = ((size_t)max_keys + hd) * sizeof(float);
-  return n < 128 * sizeof(float4) ? 128 * sizeof(float4) : n;
+  return n < AR_THREADS * sizeof(float4) ? AR_THREADS * sizeof(float4) : n;
 }
 
 template <typename T>
@@ -148,7 +192,7 @@ void launch_attn_ref(const T *q, KvPool pool, PageMap pm, RowMeta m, int tail_le
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     configured[which] = smem;
   }
-  launch_k(kern, dim3(rows, H), dim3(128), smem, s, q, pool, pm, m, tail_len, out, H, G, hd);
+  launch_k(kern, dim3(rows, H), dim3(AR_THREADS), smem, s, q, pool, pm, m, tail_len, out, H, G, hd);
 }
 template void launch_attn_ref<float>(const float *, KvPool, PageMap, RowMeta, int, float *, int, int, int, int, int,
                                      cudaStream_t);

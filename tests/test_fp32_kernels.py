@@ -74,3 +74,40 @@ def test_plain_attention_wide_heads_vs_fp64(hd, dtype, tol):
     ref = torch.softmax(q.double() @ k.T / hd ** 0.5, -1) @ v
     # fp32: scores of order 1 .. 3 and sums of 40 terms; bf16: one rounding of outputs of order 1
     assert (out.cpu().double() - ref).abs().max() < tol
+
+
+@pytest.mark.parametrize("hd,ps", [(64, 16), (48, 5)])
+@pytest.mark.parametrize("n", [1, 63, 64, 127, 128, 129, 255, 256, 257, 600])
+def test_plain_attention_key_counts_vs_fp64(n, hd, ps):
+    """Around the keys whose values are requested ahead of their scores, a round of keys, and page sizes that are no power of two."""
+    H, G = 3, 1
+    g = torch.Generator().manual_seed(n)
+    pages = (n + ps - 1) // ps
+    q, kp, vp = (torch.randn(*s, generator=g) for s in ((2, H, hd), (pages, G, ps, hd), (pages, G, ps, hd)))
+    full = lambda c: torch.full((2,), c, dtype=torch.int32, device="cuda")
+    lo, hi = torch.ones(2, dtype=torch.int64, device="cuda"), torch.zeros(2, dtype=torch.int64, device="cuda")
+    table = torch.randperm(pages, generator=g).to(torch.int32).view(1, pages)
+    out = sb.attention(q.cuda(), kp.cuda(), vp.cuda(), table.cuda(), ps, full(0), full(n - 1), full(n - 1), lo, hi, 1, G, n, impl=1).cpu().double()
+    k, v = (t[table[0].long()].double()[:, 0].reshape(pages * ps, hd)[:n] for t in (kp, vp))
+    ref = torch.softmax(q.double() @ k.T / hd ** 0.5, -1) @ v
+    assert (out - ref).abs().max() < 5e-6                   # scores of order 1 .. 3 in fp32, sums of up to 600 terms
+
+
+@pytest.mark.parametrize("K", [1, 4, 16])
+@pytest.mark.parametrize("n", [16, 17, 255, 257, 1023, 1024, 1025, 2047, 2048, 2049])
+def test_log_softmax_top_k_edges(n, K):
+    """Numbers of logits around what a thread keeps in registers, with ties, infinities and rows of equal values."""
+    g = torch.Generator().manual_seed(n + K)
+    z = torch.randn(6, n, generator=g)
+    z[1] = 0.25
+    z[2, n // 2:] = float("-inf")
+    z[3] = torch.randint(0, 3, (n,), generator=g).float()
+    idx, lp = (t.cpu() for t in sb.logsoftmax_topk(z.cuda(), K, two_stage=False))
+    for r in range(6):
+        want = sorted(range(n), key=lambda i: (-float(z[r, i]), i))[:K]
+        ref = torch.log_softmax(z[r].double(), 0)[want]
+        live = [c for c in range(K) if z[r, want[c]] > float("-inf")]
+        gaps = torch.diff(z[r][want]).abs()
+        if not bool(((gaps > 0) & (gaps < 1e-5)).any()):    # values that fp32 log-probabilities may merge
+            assert idx[r].tolist() == want, r
+        assert (lp[r][live] - ref[live]).abs().max() < 1e-5
