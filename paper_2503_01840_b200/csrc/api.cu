@@ -556,10 +556,9 @@ template <typename T> struct Sched {
     fgemm_resid(c->act, c->F, w.w_down, rows, true, next_gain, tap_mask, xres);
   }
   void target_forward_fused(int rows, int tail_len, bool want_logits) {
-    mark(SPEC_PROF_MISC); launch_rope_table(c->meta.pos, rows, c->hd / 2, c->inv_freq, c->cs, s); tick();
     mark(SPEC_PROF_MISC);
     launch_embed_norm((const bf16 *)c->embed, c->meta.tok, (const bf16 *)c->tl[0].attn_norm, c->x, (bf16 *)c->h, c->ssq, rows, c->k,
-                      c->Ralloc, s);
+                      c->Ralloc, c->meta.pos, c->inv_freq, c->cs, c->hd / 2, s);
     tick();
     for (int l = 0; l < c->L; l++)
       block_fused(c->tl[l], c->pools[l], rows, tail_len, l + 1 < c->L ? c->tl[l + 1].attn_norm : c->final_norm, tap_mask_of(l));
@@ -588,9 +587,9 @@ template <typename T> struct Sched {
   void draft_forward_fused(const float *feat, int nparts, size_t fstride, const int32_t *src_row, int rows, int tail_len,
                            bool prebuilt = false, bool pending = false) {
     if (!prebuilt) {
-      mark(SPEC_PROF_MISC); launch_rope_table(c->meta.pos, rows, c->hd / 2, c->inv_freq, c->cs, s); tick();
       mark(SPEC_PROF_MISC);
-      launch_build_cat<bf16>(feat, nparts, fstride, src_row, (const bf16 *)c->embed, c->meta.tok, c->meta.seq, (bf16 *)c->cat, rows, c->k, s);
+      launch_build_cat<bf16>(feat, nparts, fstride, src_row, (const bf16 *)c->embed, c->meta.tok, c->meta.seq, (bf16 *)c->cat, rows, c->k, c->meta.pos,
+                             c->inv_freq, c->cs, c->hd / 2, s);
       tick();
     }
     fgemm_resid(c->cat, 2 * c->k, c->fc2, rows, false, c->dl.attn_norm, 0);
@@ -803,8 +802,9 @@ template <typename T> struct Sched {
       head_done = true;
       return;
     }
-    mark(SPEC_PROF_MISC); launch_rope_table(c->meta.pos, rows, c->hd / 2, c->inv_freq, c->cs, s); tick();
-    mark(SPEC_PROF_MISC); launch_build_cat<T>(feat, nparts, fstride, src_row, (const T *)c->embed, c->meta.tok, c->meta.seq, (T *)c->cat, rows, c->k, s);
+    mark(SPEC_PROF_MISC);
+    launch_build_cat<T>(feat, nparts, fstride, src_row, (const T *)c->embed, c->meta.tok, c->meta.seq, (T *)c->cat, rows, c->k, c->meta.pos, c->inv_freq, c->cs,
+                        c->hd / 2, s);
     tick();
     c->np_proj = pick(c->k, 2 * c->k, 1); c->ps_proj = pstride(c->k);
     gemm(c->cat, c->fc2, c->proj, rows, c->k, 2 * c->k, c->k, 0, c->np_proj);
@@ -912,8 +912,9 @@ template <typename T> struct Sched {
     const PageMap pm{c->page_table, c->pps, c->cfg.page_size, c->cfg.num_pages};
     const int qd = c->H * c->hd;
     launch_pack_meta(blocks, n_blocks, c->prompt_dev, w.m, pm, c->G, c->status, s); tick();
-    launch_rope_table(w.m.pos, rows, c->hd / 2, c->inv_freq, w.cs, s); tick();
-    launch_embed_norm((const bf16 *)c->embed, w.m.tok, (const bf16 *)c->tl[0].attn_norm, w.x, w.h, w.ssq, rows, c->k, w.cap, s); tick();
+    launch_embed_norm((const bf16 *)c->embed, w.m.tok, (const bf16 *)c->tl[0].attn_norm, w.x, w.h, w.ssq, rows, c->k, w.cap, w.m.pos, c->inv_freq, w.cs,
+                      c->hd / 2, s);
+    tick();
     const bool prune = last_layer_on_last_rows();
     for (int l = 0; l < c->L; l++) {
       const LayerW &lw = c->tl[l];
@@ -939,7 +940,7 @@ template <typename T> struct Sched {
       a.w[0] = (const bf16 *)c->fc3; a.O[0] = c->k; a.nw = 1;
       a.out_f32 = c->proj; a.ldo = c->k;
       fgemm(EPI_F32, a);
-      launch_build_cat<bf16>(c->proj, 1, 0, nullptr, (const bf16 *)c->embed, w.m.tok_next, w.m.seq_d, w.cat, rows, c->k, s); tick();
+      launch_build_cat<bf16>(c->proj, 1, 0, nullptr, (const bf16 *)c->embed, w.m.tok_next, w.m.seq_d, w.cat, rows, c->k, nullptr, nullptr, nullptr, 0, s); tick();
     } else {
       launch_embed_half((const bf16 *)c->embed, w.m.tok_next, w.cat, rows, c->k, s); tick();
       WideGemmArgs a = wargs(w, w.taps, rows, 3 * c->k);

@@ -140,9 +140,9 @@ __device__ __forceinline__ size_t kv_offset(const PageMap &pm, int seq, int pos,
 template <typename T>
 void launch_embed(const T *embed, const int32_t *tok, float *x, int rows, int k, cudaStream_t s);
 
-// fused-path embedding: x = E[tok], hb = bf16(x * gain), ssq[tile][row] = per-128-feature sums of x^2
+// fused-path embedding: x = E[tok], hb = bf16(x * gain), ssq[tile][row] = per-128-feature sums of x^2; and the rows' RoPE angles
 void launch_embed_norm(const bf16 *embed, const int32_t *tok, const bf16 *gain, float *x, bf16 *hb, float *ssq, int rows,
-                       int k, int ssq_ld, cudaStream_t s);
+                       int k, int ssq_ld, const int32_t *pos, const double *inv_freq, float2 *cs, int half, cudaStream_t s);
 
 // x (+)= sum of `nparts` partial slices [nparts][rows][k]; optional taps (T, [rows][3k], slots by bitmask);
 // optional h[r] = rmsnorm(x[src_row ? src_row[r] : r]) * gain.  mode: 0 keep x, 1 x = parts, 2 x += parts.
@@ -186,10 +186,11 @@ void launch_rope_kv(const float *qkv, int nparts, size_t part_stride, const floa
 template <typename T>
 void launch_silu_mul(const float *gu, int nparts, size_t part_stride, T *act, int rows, int F, cudaStream_t s);
 
-// cat[r] = [ T(feat[src_row[r]]) ; embed[tok[r]] ], feat = sum of partial slices (fp32)
+// cat[r] = [ T(feat[src_row[r]]) ; embed[tok[r]] ], feat = sum of partial slices (fp32); with pos also the rows' RoPE angles
 template <typename T>
 void launch_build_cat(const float *feat, int nparts, size_t part_stride, const int32_t *src_row, const T *embed,
-                      const int32_t *tok, const int32_t *seq, T *cat, int rows, int k, cudaStream_t s);
+                      const int32_t *tok, const int32_t *seq, T *cat, int rows, int k, const int32_t *pos, const double *inv_freq, float2 *cs, int half,
+                      cudaStream_t s);
 
 // ---------------------------------------------------------------- launchers (gemm_ref.cu)
 template <typename T>

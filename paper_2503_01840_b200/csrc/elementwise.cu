@@ -38,6 +38,16 @@ void launch_embed(const T *embed, const int32_t *tok, float *x, int rows, int k,
 template void launch_embed<float>(const float *, const int32_t *, float *, int, int, cudaStream_t);
 template void launch_embed<bf16>(const bf16 *, const int32_t *, float *, int, int, cudaStream_t);
 
+// RoPE angles that ride on a launch over the same rows (double, rounded once): its blocks of one more slice of the grid take a row each
+struct RopeJob { const int32_t *pos; const double *inv_freq; float2 *cs; int half; };
+__device__ __forceinline__ void rope_row(int pos, const double *inv_freq, float2 *cs, int half) {
+  for (int i = threadIdx.x; i < half; i += blockDim.x) {
+    double sn, c;
+    sincos((double)pos * inv_freq[i], &sn, &c);
+    cs[i] = make_float2((float)c, (float)sn);
+  }
+}
+
 // ---------------------------------------------------------------- embedding gather feeding the fused GEMM path
 // x = E[tok] (fp32 residual stream), hb = bf16(x * gain) (input of the first QKV GEMM, which applies
 // the RMSNorm factor as a row scale), ssq[tile][row] = sum of x^2 over the tile's 128 features.
@@ -48,11 +58,13 @@ template void launch_embed<bf16>(const bf16 *, const int32_t *, float *, int, in
 template <bool VEC>
 __global__ void __launch_bounds__(256) embed_norm_kernel(const bf16 *__restrict__ embed, const int32_t *__restrict__ tok,
                                                          const bf16 *__restrict__ gain, float *__restrict__ x, bf16 *__restrict__ hb,
-                                                         float *__restrict__ ssq, int k, int ssq_ld) {
-  // The wait also orders this kernel's successors after its predecessor: the first QKV GEMM waits only for this
-  // kernel and reads the RoPE table the kernel before it wrote.
+                                                         float *__restrict__ ssq, int k, int ssq_ld, RopeJob rope) {
   pdl_wait();
   pdl_trigger();
+  if (blockIdx.y * 2048 >= (unsigned)k) {                    // the slice behind the features
+    rope_row(rope.pos[blockIdx.x], rope.inv_freq, rope.cs + (size_t)blockIdx.x * rope.half, rope.half);
+    return;
+  }
   const int r = blockIdx.x, o = (blockIdx.y * 256 + threadIdx.x) * 8, tile = o >> 7;       // k % 8 == 0: a thread's eight exist together
   float v[8], sq = 0.0f;
   if (o < k) {
@@ -80,9 +92,10 @@ __global__ void __launch_bounds__(256) embed_norm_kernel(const bf16 *__restrict_
   if ((threadIdx.x & 15) == 0 && o < k) ssq[(size_t)tile * ssq_ld + r] = sq;
 }
 void launch_embed_norm(const bf16 *embed, const int32_t *tok, const bf16 *gain, float *x, bf16 *hb, float *ssq, int rows,
-                       int k, int ssq_ld, cudaStream_t s) {
+                       int k, int ssq_ld, const int32_t *pos, const double *inv_freq, float2 *cs, int half, cudaStream_t s) {
   const bool vec = (((uintptr_t)embed | (uintptr_t)gain) & 15) == 0;
-  launch_k(vec ? embed_norm_kernel<true> : embed_norm_kernel<false>, dim3(rows, (k + 2047) / 2048), dim3(256), 0, s, embed, tok, gain, x, hb, ssq, k, ssq_ld);
+  launch_k(vec ? embed_norm_kernel<true> : embed_norm_kernel<false>, dim3(rows, (k + 2047) / 2048 + 1), dim3(256), 0, s, embed, tok, gain, x, hb, ssq, k, ssq_ld,
+           RopeJob{pos, inv_freq, cs, half});
 }
 
 // ---------------------------------------------------------------- partial-sum reduce + residual + RMSNorm (+ taps)
@@ -145,13 +158,6 @@ void launch_rope_table(const int32_t *pos, int rows, int half, const double *inv
   launch_k(rope_table_kernel, dim3((n + 255) / 256), dim3(256), 0, s, pos, rows, half, inv_freq, cs);
 }
 
-__device__ __forceinline__ void rope_row(int pos, const double *inv_freq, float2 *cs, int half) {
-  for (int i = threadIdx.x; i < half; i += blockDim.x) {
-    double sn, c;
-    sincos((double)pos * inv_freq[i], &sn, &c);
-    cs[i] = make_float2((float)c, (float)sn);
-  }
-}
 __global__ void rope_embed_kernel(const int32_t *__restrict__ pos, const double *__restrict__ inv_freq, float2 *__restrict__ cs, int half,
                                   const float *__restrict__ embed, const int32_t *__restrict__ tok, float *__restrict__ x, int k) {
   pdl_wait();
@@ -380,9 +386,13 @@ template <typename T>
 __global__ void build_cat_kernel(const float *__restrict__ feat, int nparts, size_t part_stride,
                                  const int32_t *__restrict__ src_row, const T *__restrict__ embed,
                                  const int32_t *__restrict__ tok, const int32_t *__restrict__ seq, T *__restrict__ cat,
-                                 int k) {
+                                 int k, RopeJob rope) {
   pdl_wait();
   pdl_trigger();
+  if (blockIdx.y * 256 >= (unsigned)k) {                     // the slice behind the features, where there is one
+    rope_row(rope.pos[blockIdx.x], rope.inv_freq, rope.cs + (size_t)blockIdx.x * rope.half, rope.half);
+    return;
+  }
   // one element per thread (grid.y slices of the row): every load of the launch is in flight at once
   int r = blockIdx.x;
   int i = blockIdx.y * blockDim.x + threadIdx.x;
@@ -402,12 +412,14 @@ __global__ void build_cat_kernel(const float *__restrict__ feat, int nparts, siz
 }
 template <typename T>
 void launch_build_cat(const float *feat, int nparts, size_t part_stride, const int32_t *src_row, const T *embed,
-                      const int32_t *tok, const int32_t *seq, T *cat, int rows, int k, cudaStream_t s) {
-  launch_k(build_cat_kernel<T>, dim3(rows, (k + 255) / 256), dim3(256), 0, s, feat, nparts, part_stride, src_row, embed, tok, seq, cat, k);
+                      const int32_t *tok, const int32_t *seq, T *cat, int rows, int k, const int32_t *pos, const double *inv_freq, float2 *cs, int half,
+                      cudaStream_t s) {
+  launch_k(build_cat_kernel<T>, dim3(rows, (k + 255) / 256 + (pos ? 1 : 0)), dim3(256), 0, s, feat, nparts, part_stride, src_row, embed, tok, seq, cat, k,
+           RopeJob{pos, inv_freq, cs, half});
 }
 template void launch_build_cat<float>(const float *, int, size_t, const int32_t *, const float *, const int32_t *,
-                                      const int32_t *, float *, int, int, cudaStream_t);
+                                      const int32_t *, float *, int, int, const int32_t *, const double *, float2 *, int, cudaStream_t);
 template void launch_build_cat<bf16>(const float *, int, size_t, const int32_t *, const bf16 *, const int32_t *,
-                                     const int32_t *, bf16 *, int, int, cudaStream_t);
+                                     const int32_t *, bf16 *, int, int, const int32_t *, const double *, float2 *, int, cudaStream_t);
 
 }  // namespace spec

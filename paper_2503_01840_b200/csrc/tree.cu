@@ -356,7 +356,8 @@ __global__ void __launch_bounds__(256) argmax_merge_kernel(const float *__restri
   __shared__ VI sh[32];
   int r = blockIdx.x;
   VI b{0.0f, -1};
-  for (int t = threadIdx.x; t < tiles; t += blockDim.x) {
+#pragma unroll 4
+  for (int t = threadIdx.x; t < tiles; t += blockDim.x) {    // the loads of four rounds in flight
     float v = best_val[(size_t)t * ld + r];
     int i = best_idx[(size_t)t * ld + r];
     if (i >= 0 && (b.i < 0 || before(v, i, b.v, b.i))) { b.v = v; b.i = i; }
@@ -909,11 +910,24 @@ __global__ void __launch_bounds__(1024) rerank_kernel(SeqState st, TreeBufs tb, 
   if (i >= 1 && i <= pool) {
     const int c = i - 1;
     int rank = 0;
+    // equal scores: the lower index comes first.  Only around the warp's own candidates does that take a look at the index: those
+    // before them come first if they are not smaller, those behind them if they are larger (half the instructions)
+    const int c_lo = max((i & ~31) - 1, 0) & ~3, c_hi = min(((i | 31) + 3) & ~3, pool4);      // the warp's candidates are i - 1, in whole fours
 #pragma unroll 4
-    for (int j = 0; j < pool4; j += 4) {            // the padding never comes before a candidate
+    for (int j = 0; j < c_lo; j += 4) {
+      const float4 o = *(const float4 *)(sc + j);
+      rank += (o.x >= score) + (o.y >= score) + (o.z >= score) + (o.w >= score);
+    }
+#pragma unroll 4
+    for (int j = c_lo; j < c_hi; j += 4) {          // the padding never comes before a candidate
       const float4 o = *(const float4 *)(sc + j);
       rank += (o.x > score || (o.x == score && j < c)) + (o.y > score || (o.y == score && j + 1 < c)) +
               (o.z > score || (o.z == score && j + 2 < c)) + (o.w > score || (o.w == score && j + 3 < c));
+    }
+#pragma unroll 4
+    for (int j = c_hi; j < pool4; j += 4) {
+      const float4 o = *(const float4 *)(sc + j);
+      rank += (o.x > score) + (o.y > score) + (o.z > score) + (o.w > score);
     }
     kept = rank < M;
   }
@@ -980,46 +994,43 @@ void launch_plain_tree(SeqState st, TreeBufs tb, RowMeta m, int B, cudaStream_t 
 
 // ---------------------------------------------------------------- greedy acceptance
 // Follow, from the root, the child whose token equals the target's argmax at the current node.
-__global__ void accept_kernel(SeqState st, TreeBufs tb, int rows_per_seq) {
+// A thread per node looks whether it is the one its parent goes on to; the walk is then one step of shared memory per accepted node.
+constexpr int ACCEPT_THREADS = 64;                           // nodes a tree can have
+__global__ void __launch_bounds__(ACCEPT_THREADS) accept_kernel(SeqState st, TreeBufs tb, int rows_per_seq) {
   pdl_wait();
   pdl_trigger();
-  int b = blockIdx.x;
-  int Pmax = tb.Pmax;
-  int nn = tb.nn[b];
-  // the walk is serial: the tree goes to shared memory first, so that no iteration waits for a global load
-  __shared__ int32_t tok[64], par[64], y[64];
-  for (int i = threadIdx.x; i < nn && i < 64; i += blockDim.x) {
-    tok[i] = tb.tok[(size_t)b * rows_per_seq + i];
-    par[i] = tb.parent[(size_t)b * rows_per_seq + i];
-    y[i] = tb.y[(size_t)b * rows_per_seq + i];
-  }
+  __shared__ int32_t tok[64], y[64], next[64];
+  const int b = blockIdx.x, i = threadIdx.x, Pmax = tb.Pmax;
+  const size_t row0 = (size_t)b * rows_per_seq;
+  // everything is asked for at once (rows_per_seq <= 64)
+  const int nn = tb.nn[b], active = st.active[b], n = st.n[b];
+  const bool row = i < rows_per_seq;
+  const int t = row ? tb.tok[row0 + i] : 0, p = row ? tb.parent[row0 + i] : -1, best = row ? tb.y[row0 + i] : 0;
+  tok[i] = t; y[i] = best; next[i] = 64;
   __syncthreads();
-  if (threadIdx.x != 0) return;
-  if (!st.active[b] || nn < 1) { tb.out_cnt[b] = 0; return; }
+  if (i > 0 && i < nn && row && p >= 0 && p < i && t == y[p]) atomicMin(&next[p], i);      // the first child whose token the target would emit
+  __syncthreads();
+  if (i != 0) return;
+  if (!active || nn < 1) { tb.out_cnt[b] = 0; return; }
   int cur = 0, a = 0;
   tb.path[b * Pmax] = 0;
-  while (a + 1 < Pmax) {
-    int nxt = -1;
-    for (int c = cur + 1; c < nn; c++)
-      if (par[c] == cur && tok[c] == y[cur]) { nxt = c; break; }
-    if (nxt < 0) break;
-    tb.out_ids[b * Pmax + a] = tok[nxt];
-    tb.pend_tok[b * Pmax + a] = tok[nxt];
-    cur = nxt;
+  while (a + 1 < Pmax && next[cur] < 64) {
+    cur = next[cur];
+    tb.out_ids[b * Pmax + a] = tok[cur];
+    tb.pend_tok[b * Pmax + a] = tok[cur];
     tb.path[b * Pmax + (++a)] = cur;
   }
   tb.out_ids[b * Pmax + a] = y[cur];
   tb.pend_tok[b * Pmax + a] = y[cur];
   for (int j = a + 1; j < Pmax; j++) tb.out_ids[b * Pmax + j] = -1;
   tb.out_cnt[b] = a + 1;
-  int n = st.n[b];
   st.n_prev[b] = n;
   st.n[b] = n + a + 1;
   st.P[b] = a + 1;
   st.root[b] = y[cur];
 }
 void launch_accept(SeqState st, TreeBufs tb, int B, int rows_per_seq, cudaStream_t s) {
-  launch_k(accept_kernel, dim3(B), dim3(32), 0, s, st, tb, rows_per_seq);
+  launch_k(accept_kernel, dim3(B), dim3(ACCEPT_THREADS), 0, s, st, tb, rows_per_seq);
 }
 
 // ---------------------------------------------------------------- stochastic acceptance (temperature > 0)
@@ -1278,20 +1289,28 @@ __global__ void __launch_bounds__(256) commit_kernel(SeqState st, TreeBufs tb, c
           if (mv[jj]) { *(uint4 *)(Kp + dof[jj]) = kv[jj]; *(uint4 *)(Vp + dof[jj]) = vv[jj]; }
       }
     }
-  } else {
-    // taps of the accepted nodes -> pending entries (different buffers: no ordering needed)
+  } else if (const int j = l - L; j < cnt) {
+    // taps of the j-th accepted node -> pending entry j (different buffers: no ordering needed), a block each with its loads in flight (one
+    // block for all of them took 15 us, and with it the launch)
     const int nvec = 3 * k / VEC;
-    for (int j = 0; j < cnt; j++) {
-      const uint4 *src = (const uint4 *)(node_taps + ((size_t)b * rows_per_seq + path_s[j]) * 3 * k);
-      uint4 *dst = (uint4 *)(pend_taps + ((size_t)b * Pmax + j) * 3 * k);
-      for (int e = threadIdx.x; e < nvec; e += blockDim.x) dst[e] = src[e];
+    const uint4 *__restrict__ src = (const uint4 *)(node_taps + ((size_t)b * rows_per_seq + path_s[j]) * 3 * k);
+    uint4 *__restrict__ dst = (uint4 *)(pend_taps + ((size_t)b * Pmax + j) * 3 * k);
+    constexpr int NV = 8;
+    for (int e0 = threadIdx.x; e0 < nvec; e0 += NV * blockDim.x) {
+      uint4 v[NV];
+#pragma unroll
+      for (int q = 0; q < NV; q++)
+        if (e0 + q * (int)blockDim.x < nvec) v[q] = src[e0 + q * blockDim.x];
+#pragma unroll
+      for (int q = 0; q < NV; q++)
+        if (e0 + q * (int)blockDim.x < nvec) dst[e0 + q * blockDim.x] = v[q];
     }
   }
 }
 template <typename T>
 void launch_commit(SeqState st, TreeBufs tb, const KvPool *pools, PageMap pm, const T *node_taps, T *pend_taps, int B,
                    int L, int G, int hd, int k, int rows_per_seq, cudaStream_t s) {
-  launch_k(commit_kernel<T>, dim3(B, L + 1), dim3(256), 0, s, st, tb, pools, pm, node_taps, pend_taps, L, G, hd, k, rows_per_seq);
+  launch_k(commit_kernel<T>, dim3(B, L + tb.Pmax), dim3(256), 0, s, st, tb, pools, pm, node_taps, pend_taps, L, G, hd, k, rows_per_seq);
 }
 template void launch_commit<float>(SeqState, TreeBufs, const KvPool *, PageMap, const float *, float *, int, int, int,
                                    int, int, int, cudaStream_t);
