@@ -143,6 +143,7 @@ struct spec_ctx {
   StepPlan graph_plan[2];                    // of graph, graph_sampled
   int launches = 0, launches_graph = 0, launches_graph_sampled = 0;
   bool sampled = false;        // the step being scheduled ends with the stochastic acceptance
+  float2 *mass_part = nullptr; // sampled step: masses of the verify rows' logits, by runs of ids
   float *u_dev = nullptr;      // [B][2N] uniforms of the sampled step, then 1 / temperature
   int32_t *prompt_dev = nullptr;   // [B * max_ctx] the prompts of the prefill being run, concatenated
   int sched_err = 0;
@@ -261,6 +262,7 @@ static size_t carve(spec_ctx *c, void *base) {
   t.nn = cv.take<int32_t>(B); t.y = cv.take<int32_t>(ne);
   t.path = cv.take<int32_t>((size_t)B * c->Pmax); t.pend_tok = cv.take<int32_t>((size_t)B * c->Pmax);
   c->u_dev = cv.take<float>((size_t)B * 2 * c->N + 1);
+  c->mass_part = cv.take<float2>((size_t)c->Tv * accept_mass_chunks(c->V));
   c->prompt_dev = cv.take<int32_t>((size_t)B * g.max_ctx + 1);
   if (g.flags & SPEC_FLAG_CAPTURE) {
     c->cap_logits = cv.take<float>((size_t)c->D * c->Td * c->Vd);
@@ -1006,9 +1008,8 @@ template <typename T> struct Sched {
     c->cur_rps = rps;
     target_forward(rows, rps, true);
     mark(SPEC_PROF_TREE);
-    if (c->sampled && !plain) launch_accept_sampled(c->st, c->tb, c->logits, c->V, c->u_dev, c->B, rps, s);
-    else launch_accept(c->st, c->tb, c->B, rps, s);
-    tick();
+    if (c->sampled && !plain) tick(launch_accept_sampled(c->st, c->tb, c->logits, c->V, c->u_dev, c->mass_part, c->B, rps, s));
+    else { launch_accept(c->st, c->tb, c->B, rps, s); tick(); }
     PageMap pm{c->page_table, c->pps, c->cfg.page_size, c->cfg.num_pages};
     mark(SPEC_PROF_COMMIT); launch_commit<T>(c->st, c->tb, c->pools_dev, pm, (const T *)c->node_taps, (T *)c->pend_taps, c->B, c->L, c->G, c->hd,
                      c->k, rps, s);

@@ -1042,199 +1042,232 @@ void launch_accept(SeqState st, TreeBufs tb, int B, int rows_per_seq, cudaStream
 constexpr int ACC_THREADS = 1024;
 constexpr int ACC_MAX_REJ = 64;
 
-__device__ __forceinline__ float block_reduce_max(float v, float *sh) {
-  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
-  __syncthreads();
-  float r = sh[0];
-  for (int w = 1; w < ACC_THREADS / 32; w++) r = fmaxf(r, sh[w]);
-  __syncthreads();
-  return r;
-}
-__device__ __forceinline__ float block_reduce_sum(float v, float *sh) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
-  __syncthreads();
-  float r = 0.0f;
-  for (int w = 0; w < ACC_THREADS / 32; w++) r += sh[w];      // every thread adds the 32 warp sums in the same order
-  __syncthreads();
-  return r;
-}
-
 // exp on the special-function unit (ex2.approx): every term of a row goes through the same routine, so the
 // probabilities stay consistent; its relative error (~1e-6 near the maximum) is far inside the parity slack
 __device__ __forceinline__ float acc_exp(float x) { return __expf(x); }
 
-__global__ void __launch_bounds__(ACC_THREADS) accept_sampled_kernel(SeqState st, TreeBufs tb, const float *__restrict__ logits,
-                                                                     int V, const float *__restrict__ u, int rows_per_seq) {
+// Masses of the verify rows: per run of MASS_CHUNK ids the largest logit and sum exp((z - largest) / T), [row][chunk].  The acceptance walks one
+// node after the other on one SM, which reads a row of 128256 logits in 7 us: three times a visited node, that was most of the launch.
+// Here the whole chip reads all rows once, and the walk needs a few numbers a node.  Sampled step of the 8B shapes over a greedy one, 6.2
+// nodes visited: 145 -> 65 us (of which the logits' way to memory, the uniforms' copy and the host take 40).
+constexpr int MASS_CHUNK = 8192;
+int accept_mass_chunks(int V) { return (V + MASS_CHUNK - 1) / MASS_CHUNK; }
+__global__ void __launch_bounds__(256) row_mass_kernel(const float *__restrict__ logits, int V, const float *__restrict__ inv_temp, float2 *__restrict__ part) {
   pdl_wait();
   pdl_trigger();
-  __shared__ float red[ACC_THREADS / 32];
-  __shared__ float part[ACC_THREADS / 32];
-  extern __shared__ float seg[];                           // [ceil(V / 32)] residual terms of the range that holds the drawn token
+  __shared__ float red[2][8];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int v0 = blockIdx.x * MASS_CHUNK, n = min(MASS_CHUNK, V - v0);
+  const float *z = logits + (size_t)blockIdx.y * V + v0;
+  const float inv_T = *inv_temp;
+  constexpr int PER = MASS_CHUNK / 256;
+  float v[PER];
+  if ((V & 3) == 0) {                                        // rows are then 16-byte aligned
+#pragma unroll
+    for (int j = 0; j < PER / 4; j++) {
+      const int i = 4 * (threadIdx.x + j * 256);
+      const float4 q = i < n ? *(const float4 *)(z + i) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+      v[4 * j] = q.x; v[4 * j + 1] = q.y; v[4 * j + 2] = q.z; v[4 * j + 3] = q.w;
+    }
+  } else {
+#pragma unroll
+    for (int j = 0; j < PER; j++) { const int i = threadIdx.x + j * 256; v[j] = i < n ? z[i] : -INFINITY; }
+  }
+  float m = -INFINITY;
+#pragma unroll
+  for (int j = 0; j < PER; j++) m = fmaxf(m, v[j]);
+  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if (lane == 0) red[0][warp] = m;
+  __syncthreads();
+  m = red[0][0];
+#pragma unroll
+  for (int w = 1; w < 8; w++) m = fmaxf(m, red[0][w]);
+  float sum = 0.0f;
+  if (m > -INFINITY) {
+#pragma unroll
+    for (int j = 0; j < PER; j++) sum += acc_exp((v[j] - m) * inv_T);      // exp(-inf) = 0 past the end
+  }
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  if (lane == 0) red[1][warp] = sum;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    sum = red[1][0];
+#pragma unroll
+    for (int w = 1; w < 8; w++) sum += red[1][w];
+    part[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = make_float2(m, sum);
+  }
+}
+
+__global__ void __launch_bounds__(ACC_THREADS) accept_sampled_kernel(SeqState st, TreeBufs tb, const float *__restrict__ logits,
+                                                                     int V, const float *__restrict__ u, const float2 *__restrict__ mass_part, int chunks,
+                                                                     int rows_per_seq) {
+  pdl_wait();
+  pdl_trigger();
+  constexpr int NWARP = ACC_THREADS / 32;
+  __shared__ float seg[MASS_CHUNK];                          // residual terms of the chunk that holds the drawn token
+  __shared__ float part[NWARP];
   __shared__ int32_t rej[ACC_MAX_REJ];
-  __shared__ int s_next, s_nrej, s_pick, s_owner;
+  __shared__ float rej_e[ACC_MAX_REJ];
+  __shared__ int s_cur, s_len, s_nrej, s_pick, s_owner;
   __shared__ float s_target;
-  const int b = blockIdx.x, tid = threadIdx.x;
+  __shared__ int32_t tok[64];
+  __shared__ float ub[128], zc[64], zmax_s[64], mass_s[64];
+  __shared__ unsigned long long kids[64];                    // children of a node, in node order
+  const int b = blockIdx.x, tid = threadIdx.x, wid = tid >> 5, ln = tid & 31;
   const int Pmax = tb.Pmax, N = tb.N;
-  const int nn = tb.nn[b];
+  const int nn = min(tb.nn[b], 64);
   if (!st.active[b] || nn < 1) {
     if (tid == 0) tb.out_cnt[b] = 0;
     return;
   }
-  // the tree and the uniforms go to shared memory once: the walk below is serial, and a global load per node would
-  // put an L2 round trip into every iteration
-  __shared__ int32_t tok[64], par[64];
-  __shared__ float ub[128];
-  if (tid < nn && tid < 64) { tok[tid] = tb.tok[(size_t)b * rows_per_seq + tid]; par[tid] = tb.parent[(size_t)b * rows_per_seq + tid]; }
+  if (tid < 64) kids[tid] = 0ull;
+  __syncthreads();
+  // ---- the tree, the uniforms, the nodes' masses and their tokens' logits go to shared memory at once: the walk below is serial
+  const size_t row0 = (size_t)b * rows_per_seq;
   if (tid < 2 * N && tid < 128) ub[tid] = u[(size_t)b * 2 * N + tid];
   const float inv_T = u[(size_t)gridDim.x * 2 * N];          // 1 / temperature follows the uniforms
+  if (tid < nn) {
+    const int t = tb.tok[row0 + tid], p = tb.parent[row0 + tid];
+    tok[tid] = t;
+    if (tid > 0) { zc[tid] = logits[(row0 + p) * V + t]; atomicOr(&kids[p], 1ull << tid); }
+  }
+  for (int node = wid; node < nn; node += NWARP) {           // a warp per node, a lane per chunk
+    const float2 *mp = mass_part + (row0 + node) * chunks;
+    float m = -INFINITY, sum = 0.0f;
+    for (int c = ln; c < chunks; c += 32) m = fmaxf(m, mp[c].x);
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    for (int c = ln; c < chunks; c += 32) sum += mp[c].y > 0.0f ? mp[c].y * acc_exp((mp[c].x - m) * inv_T) : 0.0f;
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (ln == 0) { zmax_s[node] = m; mass_s[node] = sum; }
+  }
   __syncthreads();
-  int cur = 0, a = 0;
-  if (tid == 0) tb.path[b * Pmax] = 0;
-  for (;;) {
-    const float *z = logits + ((size_t)b * rows_per_seq + cur) * V;
-    // one SM reads the row from L2: wide, unrolled loads keep enough requests in flight
-    const bool vec = (V & 3) == 0;                       // rows are then 16-byte aligned
-    const float4 *z4 = (const float4 *)z;
-    float m = -INFINITY;
-    if (vec) {
-#pragma unroll 4
-      for (int i = tid; i < V / 4; i += ACC_THREADS) {
-        const float4 q = z4[i];
-        m = fmaxf(m, fmaxf(fmaxf(q.x, q.y), fmaxf(q.z, q.w)));
-      }
-    } else {
-#pragma unroll 8
-      for (int v = tid; v < V; v += ACC_THREADS) m = fmaxf(m, z[v]);
-    }
-    const float zmax = block_reduce_max(m, red);
-    float sum = 0.0f;
-    if (vec) {
-#pragma unroll 4
-      for (int i = tid; i < V / 4; i += ACC_THREADS) {
-        const float4 q = z4[i];
-        sum += (acc_exp((q.x - zmax) * inv_T) + acc_exp((q.y - zmax) * inv_T)) + (acc_exp((q.z - zmax) * inv_T) + acc_exp((q.w - zmax) * inv_T));
-      }
-    } else {
-#pragma unroll 8
-      for (int v = tid; v < V; v += ACC_THREADS) sum += acc_exp((z[v] - zmax) * inv_T);
-    }
-    float mass = block_reduce_sum(sum, red);
-    // ---- the children of cur in node order, tried by one thread
-    if (tid == 0) {
-      int nxt = -1, nrej = 0;
+  // ---- the walk, by one thread: the children of the current node in node order
+  if (tid == 0) {
+    int cur = 0, a = 0, nrej;
+    tb.path[b * Pmax] = 0;
+    for (;;) {
+      int nxt = -1;
+      float mass = mass_s[cur];
+      nrej = 0;
       if (a + 1 < Pmax) {
-        for (int c = cur + 1; c < nn && nxt < 0; c++) {
-          if (par[c] != cur) continue;
-          const float e = acc_exp((z[tok[c]] - zmax) * inv_T);
+        for (unsigned long long left = kids[cur]; left && nxt < 0; left &= left - 1) {
+          const int c = __ffsll(left) - 1;
+          const float e = acc_exp((zc[c] - zmax_s[cur]) * inv_T);
           const float pc = mass > 0.0f ? e / mass : 0.0f;
           if (ub[c] < pc) nxt = c;
-          else { mass -= e; if (nrej < ACC_MAX_REJ) rej[nrej++] = tok[c]; }
+          else { mass -= e; if (nrej < ACC_MAX_REJ) { rej[nrej] = tok[c]; rej_e[nrej++] = e; } }
         }
       }
-      s_next = nxt; s_nrej = nrej;
-    }
-    __syncthreads();
-    const int nxt = s_next, nrej = s_nrej;
-    if (nxt >= 0) {
-      if (tid == 0) {
-        tb.out_ids[b * Pmax + a] = tok[nxt];
-        tb.pend_tok[b * Pmax + a] = tok[nxt];
-        tb.path[b * Pmax + a + 1] = nxt;
-      }
+      if (nxt < 0) break;
+      tb.out_ids[b * Pmax + a] = tok[nxt];
+      tb.pend_tok[b * Pmax + a] = tok[nxt];
+      tb.path[b * Pmax + a + 1] = nxt;
       cur = nxt;
       a++;
-      __syncthreads();
-      continue;
     }
-    // ---- the final token: inverse CDF over the residual, in two levels.  Warp w owns the ids [w * CW, (w + 1) * CW):
-    // its lanes read them coalesced and the warp sum goes to part[w]; one thread finds the warp whose range holds the
-    // target; that warp then walks its range 32 ids at a time with a warp prefix sum.
-    const int NWARP = ACC_THREADS / 32, wid = tid >> 5, ln = tid & 31;
-    const int CW = (V + NWARP - 1) / NWARP;
-    const int w0 = wid * CW, w1 = (w0 + CW < V) ? w0 + CW : V;
-    float loc = 0.0f;
-#pragma unroll 8
-    for (int v = w0 + ln; v < w1; v += 32) loc += acc_exp((z[v] - zmax) * inv_T);
-    for (int o = 16; o > 0; o >>= 1) loc += __shfl_xor_sync(0xffffffffu, loc, o);
-    if (ln == 0) part[wid] = loc;
-    __syncthreads();
-    if (tid == 0) {
-      for (int r = 0; r < nrej; r++) {                   // the rejected tokens leave the residual
-        const float e = acc_exp((z[rej[r]] - zmax) * inv_T);
-        const int w = rej[r] / CW;
-        part[w] = fmaxf(part[w] - e, 0.0f);
+    s_cur = cur; s_len = a; s_nrej = nrej;
+  }
+  __syncthreads();
+  const int cur = s_cur, a = s_len, nrej = s_nrej;
+  const float *z = logits + (row0 + cur) * V;
+  const float zmax = zmax_s[cur];
+  // ---- the final token: inverse CDF over the residual, in three levels.  One thread finds the chunk that holds the target, the chunk's
+  // terms go to shared memory, one thread finds the warp whose 32nd of them holds what is left of it, and that warp walks its range 32 ids at a
+  // time with a warp prefix sum.
+  for (int c = tid; c < chunks; c += ACC_THREADS) {          // masses of the chunks (at most MASS_CHUNK of them: V < 2^26), without the rejected tokens
+    const float2 mp = mass_part[(row0 + cur) * chunks + c];
+    float m = mp.y > 0.0f ? mp.y * acc_exp((mp.x - zmax) * inv_T) : 0.0f;
+    for (int r = 0; r < nrej; r++)
+      if (rej[r] / MASS_CHUNK == c) m = fmaxf(m - rej_e[r], 0.0f);
+    seg[c] = m;
+  }
+  __syncthreads();
+  if (tid == 0) {
+    float total = 0.0f;
+    for (int c = 0; c < chunks; c++) total += seg[c];
+    const float target = ub[N + cur] * total;
+    float cum = 0.0f, last_cum = 0.0f;
+    int owner = -1, last = 0;
+    for (int c = 0; c < chunks; c++) {
+      const float m = seg[c];
+      if (m > 0.0f) {
+        last = c; last_cum = cum;
+        if (cum + m > target) { owner = c; break; }
       }
-      float total = 0.0f;
-      for (int w = 0; w < NWARP; w++) total += part[w];
-      const float target = ub[N + cur] * total;
-      float cum = 0.0f;
-      int owner = -1;
-      for (int w = 0; w < NWARP; w++) {
-        if (part[w] > 0.0f && cum + part[w] > target) { owner = w; break; }
-        cum += part[w];
-      }
-      if (owner < 0) {                                   // rounding at the upper end: the last warp with mass
-        cum = total;
-        for (int w = NWARP - 1; w >= 0; w--)
-          if (part[w] > 0.0f) { owner = w; cum = total - part[w]; break; }
-      }
-      s_owner = owner; s_target = target - cum; s_pick = 0;
+      cum += m;
     }
-    __syncthreads();
-    // the owning warp's range goes to shared memory with every thread's help (one parallel, coalesced pass), so the
-    // ordered walk below reads no global memory
-    {
-      const int o0 = s_owner * CW, o1 = (o0 + CW < V) ? o0 + CW : V;
-      for (int v = o0 + tid; v < o1; v += ACC_THREADS) {
-        float e = acc_exp((z[v] - zmax) * inv_T);
-        for (int r = 0; r < nrej; r++) if (rej[r] == v) e = 0.0f;
-        seg[v - o0] = e;
+    if (owner < 0) { owner = last; cum = last_cum; }           // rounding at the upper end: the last chunk with mass
+    s_owner = owner; s_target = target - cum;
+  }
+  __syncthreads();
+  const int c0 = s_owner * MASS_CHUNK, n = min(MASS_CHUNK, V - c0);
+  const float in_chunk = s_target;
+  for (int i = tid; i < n; i += ACC_THREADS) {
+    float e = acc_exp((z[c0 + i] - zmax) * inv_T);
+    for (int r = 0; r < nrej; r++)
+      if (rej[r] == c0 + i) e = 0.0f;
+    seg[i] = e;
+  }
+  __syncthreads();
+  const int CW = (n + NWARP - 1) / NWARP, w0 = wid * CW, w1 = min(w0 + CW, n);
+  float loc = 0.0f;
+  for (int i = w0 + ln; i < w1; i += 32) loc += seg[i];
+  for (int o = 16; o > 0; o >>= 1) loc += __shfl_xor_sync(0xffffffffu, loc, o);
+  if (ln == 0) part[wid] = loc;
+  __syncthreads();
+  if (tid == 0) {
+    float cum = 0.0f, last_cum = 0.0f;
+    int owner = -1, last = 0;
+    for (int w = 0; w < NWARP; w++) {
+      if (part[w] > 0.0f) {
+        last = w; last_cum = cum;
+        if (cum + part[w] > in_chunk) { owner = w; break; }
       }
+      cum += part[w];
     }
-    __syncthreads();
-    if (wid == s_owner) {
-      const float target = s_target;
-      float cum = 0.0f;
-      int pick = -1, last = -1;
-      for (int base = w0; base < w1 && pick < 0; base += 32) {
-        const int v = base + ln;
-        const float e = v < w1 ? seg[v - w0] : 0.0f;
-        float inc = e;                                   // inclusive prefix sum over the 32 lanes
-        for (int o = 1; o < 32; o <<= 1) {
-          const float t = __shfl_up_sync(0xffffffffu, inc, o);
-          if (ln >= o) inc += t;
-        }
-        const bool hit = e > 0.0f && cum + inc > target;
-        const unsigned hits = __ballot_sync(0xffffffffu, hit), alive = __ballot_sync(0xffffffffu, e > 0.0f);
-        if (alive) last = base + 31 - __clz(alive);
-        if (hits) pick = base + __ffs(hits) - 1;
-        cum += __shfl_sync(0xffffffffu, inc, 31);
+    if (owner < 0) { owner = last; cum = last_cum; }           // rounding: the last warp with mass
+    s_owner = owner; s_target = in_chunk - cum; s_pick = 0;
+  }
+  __syncthreads();
+  if (wid == s_owner) {
+    const float target = s_target;
+    float cum = 0.0f;
+    int pick = -1, last = -1;
+    for (int base = w0; base < w1 && pick < 0; base += 32) {
+      const int i = base + ln;
+      const float e = i < w1 ? seg[i] : 0.0f;
+      float inc = e;                                         // inclusive prefix sum over the 32 lanes
+      for (int o = 1; o < 32; o <<= 1) {
+        const float t = __shfl_up_sync(0xffffffffu, inc, o);
+        if (ln >= o) inc += t;
       }
-      if (ln == 0) s_pick = pick >= 0 ? pick : (last >= 0 ? last : w0);
+      const bool hit = e > 0.0f && cum + inc > target;
+      const unsigned hits = __ballot_sync(0xffffffffu, hit), alive = __ballot_sync(0xffffffffu, e > 0.0f);
+      if (alive) last = base + 31 - __clz(alive);
+      if (hits) pick = base + __ffs(hits) - 1;
+      cum += __shfl_sync(0xffffffffu, inc, 31);
     }
-    __syncthreads();
-    if (tid == 0) {
-      const int bonus = s_pick;
-      tb.out_ids[b * Pmax + a] = bonus;
-      tb.pend_tok[b * Pmax + a] = bonus;
-      for (int j = a + 1; j < Pmax; j++) tb.out_ids[b * Pmax + j] = -1;
-      tb.out_cnt[b] = a + 1;
-      const int n = st.n[b];
-      st.n_prev[b] = n;
-      st.n[b] = n + a + 1;
-      st.P[b] = a + 1;
-      st.root[b] = bonus;
-    }
-    break;
+    if (ln == 0) s_pick = c0 + (pick >= 0 ? pick : (last >= 0 ? last : w0));
+  }
+  __syncthreads();
+  if (tid == 0) {
+    const int bonus = s_pick;
+    tb.out_ids[b * Pmax + a] = bonus;
+    tb.pend_tok[b * Pmax + a] = bonus;
+    for (int j = a + 1; j < Pmax; j++) tb.out_ids[b * Pmax + j] = -1;
+    tb.out_cnt[b] = a + 1;
+    const int n0 = st.n[b];
+    st.n_prev[b] = n0;
+    st.n[b] = n0 + a + 1;
+    st.P[b] = a + 1;
+    st.root[b] = bonus;
   }
 }
-void launch_accept_sampled(SeqState st, TreeBufs tb, const float *logits, int V, const float *u, int B, int rows_per_seq, cudaStream_t s) {
-  const size_t smem = (size_t)((V + ACC_THREADS / 32 - 1) / (ACC_THREADS / 32)) * sizeof(float);
-  static SmemLimit limit;
-  if (smem > 40 * 1024) limit.ensure(accept_sampled_kernel, (int)smem);
-  launch_k(accept_sampled_kernel, dim3(B), dim3(ACC_THREADS), smem, s, st, tb, logits, V, u, rows_per_seq);
+int launch_accept_sampled(SeqState st, TreeBufs tb, const float *logits, int V, const float *u, float2 *mass_part, int B, int rows_per_seq, cudaStream_t s) {
+  const int chunks = accept_mass_chunks(V);
+  launch_k(row_mass_kernel, dim3(chunks, B * rows_per_seq), dim3(256), 0, s, logits, V, u + (size_t)B * 2 * tb.N, mass_part);
+  launch_k(accept_sampled_kernel, dim3(B), dim3(ACC_THREADS), 0, s, st, tb, logits, V, u, (const float2 *)mass_part, chunks, rows_per_seq);
+  return 2;
 }
 
 // ---------------------------------------------------------------- commit: KV compaction + tap gather
