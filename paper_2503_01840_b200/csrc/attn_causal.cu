@@ -19,11 +19,17 @@
 //  * the diagonal entries of training-time test come through the K and V rings as further tiles (row = position), whose
 //    dot products the softmax threads take from shared memory.
 //
-// Measured (one B200, T = 8192, 32 / 8 heads, 3 diagonal entries per row): 0.54 ms = 1020 TFLOP/s of causal flops (0.50 ms
-// without diagonal entries) called in a row on the same inputs, 0.62 ms on inputs that change from call to call.  Earlier forms,
-// in a row: one 128-key score buffer per tile and one issuer 0.67 ms; the same with an issuer per tile and P V in two halves
-// 0.59; two 64-key buffers and one issuer 0.68.  A 64-key step takes 1600 cycles: shared memory delivers the operands of its
-// MMAs and takes in the next tiles in 1250 (128 x 64 x 16 MMAs read 6 KB per 32 tensor cycles), the exponentials take 1024.
+// Measured (one B200, T = 8192, 32 / 8 heads, 3 diagonal entries per row): 0.494 ms = 1110 TFLOP/s of causal flops (0.48 ms
+// without diagonal entries) called in a row on the same inputs.  Earlier forms, in a row: one 128-key score buffer per tile and
+// one issuer 0.67 ms; the same with an issuer per tile and P V in two halves 0.59; two 64-key buffers and one issuer 0.68; with
+// an issuer each 0.536.  A 64-key step of both tiles takes 1470 cycles: shared memory delivers the operands of its MMAs and takes
+// in the next tiles in 1250 (a 128 x 64 x 16 MMA reads 6 KB and takes 48 cycles, 32 with A in tensor memory), the exponentials
+// take 1024, and the two softmax warps of a scheduler, which run in step, leave the special-function unit idle for the rest of
+// theirs.  That rest was 580 cycles and is 450: one vote and one branch decide whether a reference moves, the next scores are
+// asked for before this step's P is known to be written, additions and multiply-adds go two at a time.
+// Not better (same call, ms): the two warps' exponentials by turns 0.488 to 0.498; the next step's scores loaded, and their
+// maximum taken, under this step's exponentials 0.59 to 0.62 (they come too late for it); an eighth to a third of the
+// exponentials by a polynomial on the multiply-add pipe 0.493 to 0.514; half of Q in tensor memory with one score buffer 0.575.
 //
 // Every wait is bounded.  On a time-out the CTA winds down; a prefill's status words record it, and training-time test, which
 // has none, gets NaN in the rows (and normalisers) it could not finish.
@@ -45,6 +51,7 @@ namespace {
 using tc::elect_one;
 using tc::mbar_expect_tx;
 using tc::mbar_init;
+using tc::mbar_test_warp;
 using tc::mbar_wait;
 using tc::mbar_wait_warp;
 using tc::smem_u32;
@@ -98,6 +105,18 @@ __device__ __forceinline__ float ex2(float x) {
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {      // two multiply-adds in one instruction, each rounded like fmaf
+  float2 r;
+  asm("{\n\t.reg .b64 a, b, c, d;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\tmov.b64 c, {%6, %7};\n\tfma.rn.f32x2 d, a, b, c;\n\tmov.b64 {%0, %1}, d;\n\t}"
+      : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+  return r;
+}
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+  float2 r;
+  asm("{\n\t.reg .b64 a, b, d;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\tadd.rn.f32x2 d, a, b;\n\tmov.b64 {%0, %1}, d;\n\t}"
+      : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return r;
+}
 __device__ __forceinline__ uint32_t pack2(float lo, float hi) {
   __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
   return *(uint32_t *)&v;
@@ -133,6 +152,13 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float *f) {     // no 
         "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]),
         "=r"(v[30]), "=r"(v[31])
       : "r"(taddr));
+}
+// values that a tmem_ld32 put out, from here on: nothing that uses them moves to before the wait for them
+__device__ __forceinline__ void pin32(float *f) {
+  asm volatile("" : "+f"(f[0]), "+f"(f[1]), "+f"(f[2]), "+f"(f[3]), "+f"(f[4]), "+f"(f[5]), "+f"(f[6]), "+f"(f[7]), "+f"(f[8]), "+f"(f[9]), "+f"(f[10]), "+f"(f[11]),
+                    "+f"(f[12]), "+f"(f[13]), "+f"(f[14]), "+f"(f[15]));
+  asm volatile("" : "+f"(f[16]), "+f"(f[17]), "+f"(f[18]), "+f"(f[19]), "+f"(f[20]), "+f"(f[21]), "+f"(f[22]), "+f"(f[23]), "+f"(f[24]), "+f"(f[25]), "+f"(f[26]),
+                    "+f"(f[27]), "+f"(f[28]), "+f"(f[29]), "+f"(f[30]), "+f"(f[31]));
 }
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t *v) {
@@ -188,7 +214,7 @@ __global__ void __launch_bounds__(CA_THREADS, 1) attn_causal_kernel(const __grid
   if (threadIdx.x == 0) {
     for (int i = 0; i < CA_STAGES; i++) { mbar_init(&kfull[i], 1); mbar_init(&kempty[i], 2); mbar_init(&vfull[i], 1); mbar_init(&vempty[i], 2); }
     mbar_init(q_bar, 1);
-    for (int i = 0; i < 4; i++) { mbar_init(&s_bar[i], 1); mbar_init(&p_bar[i], 128); }
+    for (int i = 0; i < 4; i++) { mbar_init(&s_bar[i], 1); mbar_init(&p_bar[i], 4); }
     for (int i = 0; i < 2; i++) { mbar_init(&o_bar[i], 1); mbar_init(&d_bar[i], 1); }
     *abort_flag = 0;
     n_filled[0] = n_filled[1] = 0;
@@ -343,16 +369,27 @@ __global__ void __launch_bounds__(CA_THREADS, 1) attn_causal_kernel(const __grid
     const float sc = rsqrtf((float)CA_HD) * 1.4426950408889634f;                     // softmax scale folded into exp2
     float mx = -INFINITY, l = 0.0f, lrnd = 0.0f;                  // sums of the probabilities and (BRIEF) of the rounded ones
     bool alive = true;
-    for (int i = 0; i < nt; i++) {
-      bool ok = mbar_wait_warp(&s_bar[t * 2 + (i & 1)], (uint32_t)((i >> 1) & 1), p.spin);
-      ok = __all_sync(0xffffffffu, ok && !*abort_flag);
-      if (!ok) { if (lane == 0) { *abort_flag = 1; if (p.status) set_status(p.status, ST_TIMEOUT, 435, blockIdx.y, i); } alive = false; break; }
+    // The scores of step i into s, once they are complete
+    float s[CA_KS];
+    auto fetch = [&](int i) {
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t sb = my_s + (uint32_t)((i & 1) * CA_KS);
-      float s[CA_KS];
-      tmem_ld32(sb, s);
-      tmem_ld32(sb + 32, s + 32);
+      tmem_ld32(my_s + (uint32_t)((i & 1) * CA_KS), s);
+      tmem_ld32(my_s + (uint32_t)((i & 1) * CA_KS + 32), s + 32);
+    };
+    auto gave_up = [&](int site, int i) {
+      if (lane == 0) { *abort_flag = 1; if (p.status) set_status(p.status, ST_TIMEOUT, site, blockIdx.y, i); }
+      alive = false;
+    };
+    auto await = [&](int i) {
+      if (mbar_wait_warp(&s_bar[t * 2 + (i & 1)], (uint32_t)((i >> 1) & 1), p.spin)) fetch(i);
+      else gave_up(435, i);
+    };
+    float nb_ = 0.0f;                                            // the reference maximum in the exponent (0 while there is none)
+    if (nt > 0) await(0);
+    for (int i = 0; i < nt && alive; i++) {
       tmem_ld_wait();
+      pin32(s);
+      pin32(s + 32);
       const int k0 = i * CA_KS;
       if (k0 + CA_KS - 1 > pos - lane) {                         // uniform over the warp: its first row does not see the whole step
         const int lim = pos - k0;                                // keys 0..lim of the step
@@ -369,52 +406,55 @@ __global__ void __launch_bounds__(CA_THREADS, 1) attn_causal_kernel(const __grid
       // the reference maximum moves when the step's exceeds it by more than this in the exponent (training-time test: those of
       // the warp's other rows then move along)
       const float jump = DIAG && (BRIEF || i < CA_EARLY) ? CA_NEAR : CA_FAR;
-      float f = 1.0f;
-      bool move = (tm - mx) * sc > jump;
-      if (DIAG) move = __any_sync(0xffffffffu, move);
-      if (move && tm > mx) {
-        f = (mx == -INFINITY) ? 1.0f : ex2((mx - tm) * sc);
-        mx = tm;
-      }
-      if (!DIAG) move = __any_sync(0xffffffffu, f != 1.0f);
-      if (i > 0 && move) {                                       // the P V of the last step must be complete before O is rescaled
-        ok = mbar_wait_warp(&o_bar[t], (uint32_t)((i - 1) & 1), p.spin);
-        if (!ok) { if (lane == 0) { *abort_flag = 1; if (p.status) set_status(p.status, ST_TIMEOUT, 438, blockIdx.y, i); } alive = false; break; }
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const bool far = (tm - mx) * sc > jump;
+      if (__any_sync(0xffffffffu, far)) {                        // rare after a row's first steps: all that a moving reference costs is in here
+        float f = 1.0f;
+        if ((DIAG || far) && tm > mx) {
+          f = (mx == -INFINITY) ? 1.0f : ex2((mx - tm) * sc);
+          mx = tm;
+          nb_ = mx * sc;
+        }
+        l *= f;
+        lrnd *= f;
+        if (i > 0 && __any_sync(0xffffffffu, f != 1.0f)) {       // the P V of the last step must be complete before O is rescaled
+          if (!mbar_wait_warp(&o_bar[t], (uint32_t)((i - 1) & 1), p.spin)) { gave_up(438, i); break; }
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll 1
-        for (int c = 0; c < 4; c++) {
-          float o[32];
-          tmem_ld32(my_o + c * 32, o);
-          tmem_ld_wait();
+          for (int c = 0; c < 4; c++) {
+            float o[32];
+            tmem_ld32(my_o + c * 32, o);
+            tmem_ld_wait();
 #pragma unroll
-          for (int e = 0; e < 32; e++) o[e] *= f;
-          tmem_st32(my_o + c * 32, (uint32_t *)o);
+            for (int e = 0; e < 32; e++) o[e] *= f;
+            tmem_st32(my_o + c * 32, (uint32_t *)o);
+          }
         }
       }
-      const float nb_ = (mx == -INFINITY) ? 0.0f : mx * sc;
-      float rs[4] = {0.f, 0.f, 0.f, 0.f};
+      float2 rs[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+      const float2 sc2 = make_float2(sc, sc), nb2 = make_float2(-nb_, -nb_);
       uint32_t pk[32];
 #pragma unroll
       for (int e = 0; e < 32; e++) {
-        const float p0 = ex2(fmaf(s[2 * e], sc, -nb_)), p1 = ex2(fmaf(s[2 * e + 1], sc, -nb_));
-        rs[(2 * e) & 3] += p0; rs[(2 * e + 1) & 3] += p1;
-        pk[e] = pack2(p0, p1);
+        const float2 x = fma2(make_float2(s[2 * e], s[2 * e + 1]), sc2, nb2), pr = make_float2(ex2(x.x), ex2(x.y));
+        rs[e & 1] = add2(rs[e & 1], pr);
+        pk[e] = pack2(pr.x, pr.y);
       }
-      tmem_st32(sb, pk);
-      l = l * f + ((rs[0] + rs[1]) + (rs[2] + rs[3]));
+      tmem_st32(my_s + (uint32_t)((i & 1) * CA_KS), pk);
+      const bool ready = i + 1 < nt && mbar_test_warp(&s_bar[t * 2 + ((i + 1) & 1)], (uint32_t)(((i + 1) >> 1) & 1));
+      if (ready) fetch(i + 1);                                   // mostly: the loads run beside the wait for the stores of P
+      l += (rs[0].x + rs[0].y) + (rs[1].x + rs[1].y);
       if (BRIEF) {
 #pragma unroll
-        for (int z = 0; z < 4; z++) rs[z] = 0.0f;
+        for (int z = 0; z < 2; z++) rs[z] = make_float2(0.f, 0.f);
 #pragma unroll
-        for (int e = 0; e < 32; e++) {
-          const float2 b = bf2(pk[e]);
-          rs[(2 * e) & 3] += b.x; rs[(2 * e + 1) & 3] += b.y;
-        }
-        lrnd = lrnd * f + ((rs[0] + rs[1]) + (rs[2] + rs[3]));
+        for (int e = 0; e < 32; e++) rs[e & 1] = add2(rs[e & 1], bf2(pk[e]));
+        lrnd += (rs[0].x + rs[0].y) + (rs[1].x + rs[1].y);
       }
       tmem_st_wait();
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      mbar_arrive(&p_bar[t * 2 + (i & 1)]);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&p_bar[t * 2 + (i & 1)]);
+      if (i + 1 < nt && !ready) await(i + 1);
     }
     if (alive && nt > 0) {
       // All P V of the tile.  A barrier of its own: the scores of the last step only tell that the P V two steps earlier is

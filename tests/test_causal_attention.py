@@ -143,3 +143,21 @@ def test_error_against_fp64(T, H, bound):
     ref = torch.einsum("htk,hkd->thd", s.softmax(-1), V)
     rel = ((out - ref).norm() / ref.norm()).item()
     assert rel < bound, rel
+
+
+@pytest.mark.parametrize("T,H,G", [(65, 2, 2), (400, 4, 1), (900, 2, 1), (901, 3, 3)])
+def test_maxima_that_rise_with_the_keys(T, H, G):
+    """Rows whose maximum rises by more than 2^8 every three 64-key steps, to the last of them, beside rows (every other one) whose
+    scores stay small: the first rescale their sums again and again, the second are what they are without them."""
+    g = torch.Generator().manual_seed(T)
+    pages = -(-T // 16)
+    q, k, v = (torch.randn(*s, generator=g).to(torch.bfloat16).cuda() for s in ((T, H, 128), (pages, G, 16, 128), (pages, G, 16, 128)))
+    q[::2, :, 3], q[1::2, :, 3] = 8.0, 0.0
+    k[..., 3] = ((torch.arange(pages * 16, device="cuda") // 64) * 4).view(pages, 1, 16).to(torch.bfloat16)      # exact: 0, 4, 8, ...
+    out, lse = sb.ttt_attention(q, k, v, torch.arange(pages, dtype=torch.int32, device="cuda"), None, None, want_lse=True)
+    K, V = (t.double().permute(1, 0, 2, 3).reshape(G, pages * 16, 128)[:, :T].repeat_interleave(H // G, 0) for t in (k, v))
+    s = torch.einsum("thd,hkd->htk", q.double(), K) / 128 ** 0.5
+    s.masked_fill_(torch.ones(T, T, dtype=torch.bool, device="cuda").triu(1), -float("inf"))
+    # outputs of order 1: bf16 output and bf16 probabilities, 2^-9 each; scores to 50, sums of fp32 terms: 50 * 2^-24 and 2^-22 an exponential
+    assert (out.double() - torch.einsum("htk,hkd->thd", s.softmax(-1), V)).abs().max() < 2e-2
+    assert (lse.double() - torch.logsumexp(s, -1).T).abs().max() < 1e-4
