@@ -251,9 +251,10 @@ int spec_gemm_topk(const void *x, const void *w, int32_t rows, int32_t out, int3
                    float *out_lp, void *scratch, void *stream);
 
 /* Gate/up half of the decoder layer's MLP (the draft layer and every target layer are LLaMA-style decoder layers,
- * Section 3.1), on the kernels that passes of up to 128 rows use, or (more rows) with a gate and an up tile per block: act[r][f] = bf16(silu(g) * u), g = sum_i x[r][i] * w_gate[f][i], u likewise
- * with w_up, both accumulated in fp32 (a CTA holds the gate and the up features of the same range).  x [rows][in] bf16, w_gate / w_up [F][in] bf16, act [rows][F] bf16, all device pointers, 16-byte aligned;
- * rows <= 256, in % 8 == 0.  Returns SPEC_OK or a negative code; nothing is allocated. */
+ * Section 3.1), on the kernels that passes of up to 128 rows use, or (more rows) with a gate and an up tile per block:
+ * act[r][f] = bf16(silu(g) * u), g = sum_i x[r][i] * w_gate[f][i], u likewise with w_up, both accumulated in fp32 (a CTA
+ * holds the gate and the up features of the same range).  x [rows][in] bf16, w_gate / w_up [F][in] bf16, act [rows][F] bf16,
+ * all device pointers, 16-byte aligned; rows <= 256, in % 8 == 0.  Returns SPEC_OK or a negative code; nothing is allocated. */
 int spec_gemm_swiglu(const void *x, const void *w_gate, const void *w_up, void *act, int32_t rows, int32_t F, int32_t in,
                      void *stream);
 
