@@ -3,6 +3,8 @@
 // stand-in for the tensor-core kernel on bf16 models.
 #include "common.cuh"
 
+#include <algorithm>
+
 namespace spec {
 
 // four consecutive elements; VEC: one 16-byte (fp32) or 8-byte (bf16) load, for rows that start on such a boundary
@@ -19,23 +21,29 @@ template <bool VEC> __device__ __forceinline__ float4 load4(const bf16 *p) {
   return make_float4(to_f32(p[0]), to_f32(p[1]), to_f32(p[2]), to_f32(p[3]));
 }
 
-// Bound by latency: a row attends tens to hundreds of keys, and a launch has a few dozen CTAs.  So there are four dependent round trips
-// and no more for up to 128 keys: metadata, page ids, K and V rows together, output.  Four threads share a key's dot product (256 keys a round,
-// their page ids and then their rows requested at once), and a thread's first V_AHEAD values, whose addresses need no score, are
-// requested before the scores.  The value pass splits the keys over the threads that are left beside hd / 4 dimension groups.
+// A launch of at most one wave is bound by latency: a row attends tens to hundreds of keys.  So there (AHEAD) are four dependent round
+// trips and no more for up to 8192 / head_dim keys: metadata, page ids, K and V rows together, output.  Four threads share a key's dot product
+// (256 keys a round, their page ids and then their rows requested at once), and a thread's first V_AHEAD values, whose addresses need no
+// score, are requested before the scores.  The value pass splits the keys over the threads that are left beside hd / 4 dimension groups.
 // Tiny fp32 model, replayed step with the register-resident top-K: 214 -> 189 us at 64 tokens,
 // 275 -> 213 at 250, 386 -> 253 at 600.
-constexpr int AR_THREADS = 256, V_AHEAD = 8;
-template <typename T, bool VEC>
-__global__ void __launch_bounds__(AR_THREADS) attn_ref_kernel(const T *__restrict__ q, KvPool pool, PageMap pm, RowMeta m,
+// That takes 128 registers and 256 threads, two CTAs an SM.  A larger grid is bound by the requests in flight on the whole chip and wants
+// the 40 registers and 128 threads of the form without reading ahead, eleven CTAs an SM.
+template <bool AHEAD> struct ArShape {
+  static constexpr int THREADS = AHEAD ? 256 : 128, KEY_ROUNDS = AHEAD ? 4 : 1, V_AHEAD = AHEAD ? 8 : 0, PER_SM = AHEAD ? 2 : 10;
+  static constexpr int STATIC_SMEM = (AHEAD ? 2 : 1) * (THREADS / 32) * (int)sizeof(float);      // red
+};
+template <typename T, bool VEC, bool AHEAD>
+__global__ void __launch_bounds__(ArShape<AHEAD>::THREADS, ArShape<AHEAD>::PER_SM) attn_ref_kernel(const T *__restrict__ q, KvPool pool, PageMap pm, RowMeta m,
                                                        int tail_len, T *__restrict__ out, int H, int G, int hd) {
+  constexpr int AR_THREADS = ArShape<AHEAD>::THREADS, V_AHEAD = ArShape<AHEAD>::V_AHEAD;
   pdl_wait();
   pdl_trigger();
   extern __shared__ __align__(16) float smem[];
   float *qs = smem;            // [hd]
   float *sc = smem + hd;       // [ctx + tail_len]
   float4 *part = (float4 *)smem;   // [AR_THREADS], over both once they are done with
-  __shared__ float red[2][AR_THREADS / 32];
+  __shared__ float red[AHEAD ? 2 : 1][AR_THREADS / 32];
   const int r = blockIdx.x, h = blockIdx.y, g = h / (H / G);
   const int seq = m.seq[r], ctx = m.ctx[r], tb = m.tail_base[r];
   const uint64_t mlo = m.mask_lo[r], mhi = m.mask_hi[r];
@@ -60,9 +68,9 @@ __global__ void __launch_bounds__(AR_THREADS) attn_ref_kernel(const T *__restric
   const int n_grp = n_dim <= AR_THREADS ? AR_THREADS / n_dim : 0, dim = n_grp ? threadIdx.x % n_dim : 0, grp = n_grp ? threadIdx.x / n_dim : 0;
   const bool has_v = n_grp && grp < n_grp;               // thread = (four dimensions, every n_grp-th key)
   // ---- page ids of the first keys and of this thread's first values, then those values
-  constexpr int KR = 4;                                  // rounds of AR_THREADS / 4 keys in flight
+  constexpr int KR = ArShape<AHEAD>::KEY_ROUNDS;         // rounds of AR_THREADS / 4 keys in flight
   const int sub = threadIdx.x & 3, key0 = threadIdx.x >> 2;
-  int kpage[KR], vpage[V_AHEAD];
+  int kpage[KR];
   auto key_pages = [&](int j0) {
 #pragma unroll
     for (int u = 0; u < KR; u++) {
@@ -71,14 +79,17 @@ __global__ void __launch_bounds__(AR_THREADS) attn_ref_kernel(const T *__restric
     }
   };
   key_pages(0);
+  float4 vv[AHEAD ? V_AHEAD : 1];
+  if constexpr (AHEAD) {
+    int vpage[V_AHEAD];
 #pragma unroll
-  for (int u = 0; u < V_AHEAD; u++) {
-    const int j = grp + u * n_grp;
-    vpage[u] = has_v && visible(j) ? page_of(pos_of(j)) : -1;
+    for (int u = 0; u < V_AHEAD; u++) {
+      const int j = grp + u * n_grp;
+      vpage[u] = has_v && visible(j) ? page_of(pos_of(j)) : -1;
+    }
+#pragma unroll
+    for (int u = 0; u < V_AHEAD; u++) vv[u] = vpage[u] >= 0 ? load4<VEC>(Vp + row_at(vpage[u], pos_of(grp + u * n_grp)) + dim * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
   }
-  float4 vv[V_AHEAD];
-#pragma unroll
-  for (int u = 0; u < V_AHEAD; u++) vv[u] = vpage[u] >= 0 ? load4<VEC>(Vp + row_at(vpage[u], pos_of(grp + u * n_grp)) + dim * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
   __syncthreads();
   const float scale = 1.0f / sqrtf((float)hd);
   float mx = -INFINITY;
@@ -117,6 +128,8 @@ __global__ void __launch_bounds__(AR_THREADS) attn_ref_kernel(const T *__restric
   mx = red[0][0];
 #pragma unroll
   for (int w = 1; w < AR_THREADS / 32; w++) mx = fmaxf(mx, red[0][w]);
+  constexpr int SUMS = AHEAD ? 1 : 0;                     // (without reading ahead the sums take the maxima's place)
+  if (!AHEAD) __syncthreads();
   float sum = 0.0f;
   for (int j = threadIdx.x; j < nk; j += AR_THREADS) {
     float e = (sc[j] == -INFINITY) ? 0.0f : expf(sc[j] - mx);
@@ -124,11 +137,11 @@ __global__ void __launch_bounds__(AR_THREADS) attn_ref_kernel(const T *__restric
     sum += e;
   }
   for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
-  if ((threadIdx.x & 31) == 0) red[1][threadIdx.x >> 5] = sum;
+  if ((threadIdx.x & 31) == 0) red[SUMS][threadIdx.x >> 5] = sum;
   __syncthreads();
-  sum = red[1][0];
+  sum = red[SUMS][0];
 #pragma unroll
-  for (int w = 1; w < AR_THREADS / 32; w++) sum += red[1][w];
+  for (int w = 1; w < AR_THREADS / 32; w++) sum += red[SUMS][w];
   const float inv = 1.0f / sum;
   if (!n_grp) {                                           // more groups of four dimensions than threads: a thread takes several, over all keys
     for (int dm = threadIdx.x; dm < n_dim; dm += AR_THREADS) {
@@ -175,24 +188,34 @@ __global__ void __launch_bounds__(AR_THREADS) attn_ref_kernel(const T *__restric
   }
 }
 
-size_t attn_ref_smem_bytes(int max_keys, int hd) {
-  const size_t n = ((size_t)max_keys + hd) * sizeof(float);
-  return n < AR_THREADS * sizeof(float4) ? AR_THREADS * sizeof(float4) : n;
+// Whether a launch reads ahead: up to one wave of that form, two CTAs an SM (registers).  Above, the form with ten CTAs an SM is faster, up to
+// 2.6 times, as long as shared memory (a score for every key that the caller allows for) holds more than three of them.  Called in a row, us,
+// reading ahead / not: fp32 hd 64, 240 CTAs 6.9 / 7.4 with 20 keys, 13.0 / 20.8 with 250, 34 / 67 with 1000; 300 CTAs 9.9 / 6.9, 20.1 / 20.6,
+// 63 / 65; 960 CTAs 18.8 / 7.9, 39.6 / 23.1, 125 / 72; bf16 hd 96, 320 CTAs 12.6 / 8.4, 30.9 / 29.2, 89 / 98; 1920 CTAs 39 / 16, 107 / 64, 312 / 218.
+// 1920 CTAs of bf16 hd 96, 250 keys of 6000 / 12000 / 16000 / 24000 allowed for: 106 / 65, 107 / 110, 107 / 134, 107 / 184.
+bool attn_ref_reads_ahead(int rows, int H, int hd, int max_keys) {
+  const size_t smem = ((size_t)max_keys + hd) * sizeof(float);
+  if (smem + ArShape<true>::STATIC_SMEM > 227 * 1024) return false;      // the last dozen keys that an SM can hold are for the smaller one
+  return (long long)rows * H <= 148 * ArShape<true>::PER_SM || 228 * 1024 / (smem + ArShape<false>::STATIC_SMEM + 1024) <= 3;
+}
+
+template <typename T, bool VEC, bool AHEAD>
+void launch_attn_ref_form(const T *q, KvPool pool, PageMap pm, RowMeta m, int tail_len, T *out, int rows, int H, int G, int hd, int max_keys, cudaStream_t s) {
+  constexpr int threads = ArShape<AHEAD>::THREADS;
+  const size_t smem = std::max(((size_t)max_keys + hd) * sizeof(float), threads * sizeof(float4));
+  static SmemLimit limit;
+  if (smem > 48 * 1024) limit.ensure(attn_ref_kernel<T, VEC, AHEAD>, (int)smem);
+  launch_k(attn_ref_kernel<T, VEC, AHEAD>, dim3(rows, H), dim3(threads), smem, s, q, pool, pm, m, tail_len, out, H, G, hd);
 }
 
 template <typename T>
 void launch_attn_ref(const T *q, KvPool pool, PageMap pm, RowMeta m, int tail_len, T *out, int rows, int H, int G,
                      int hd, int max_keys, cudaStream_t s) {
-  size_t smem = attn_ref_smem_bytes(max_keys, hd);
   const bool vec = (((uintptr_t)pool.k | (uintptr_t)pool.v) & (4 * sizeof(T) - 1)) == 0;      // rows are multiples of 16 elements
-  auto kern = vec ? attn_ref_kernel<T, true> : attn_ref_kernel<T, false>;
-  static size_t configured[4] = {0, 0, 0, 0};
-  int which = (sizeof(T) == 4 ? 0 : 1) + (vec ? 2 : 0);
-  if (smem > 48 * 1024 && smem > configured[which]) {
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    configured[which] = smem;
-  }
-  launch_k(kern, dim3(rows, H), dim3(AR_THREADS), smem, s, q, pool, pm, m, tail_len, out, H, G, hd);
+  const bool ahead = attn_ref_reads_ahead(rows, H, hd, max_keys);
+  auto launch = ahead ? (vec ? launch_attn_ref_form<T, true, true> : launch_attn_ref_form<T, false, true>)
+                      : (vec ? launch_attn_ref_form<T, true, false> : launch_attn_ref_form<T, false, false>);
+  launch(q, pool, pm, m, tail_len, out, rows, H, G, hd, max_keys, s);
 }
 template void launch_attn_ref<float>(const float *, KvPool, PageMap, RowMeta, int, float *, int, int, int, int, int,
                                      cudaStream_t);

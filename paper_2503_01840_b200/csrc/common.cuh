@@ -217,7 +217,7 @@ void launch_norm_qkv(const float *x, const float *add, float *x_out, float *taps
 template <typename T>
 void launch_attn_ref(const T *q, KvPool pool, PageMap pm, RowMeta m, int tail_len, T *out, int rows, int H, int G,
                      int hd, int max_keys, cudaStream_t s);
-size_t attn_ref_smem_bytes(int max_keys, int hd);
+bool attn_ref_reads_ahead(int rows, int H, int hd, int max_keys);      // which of its two forms takes a launch
 
 // ---------------------------------------------------------------- launchers (tree.cu)
 void launch_logsoftmax_topk(const float *logits, int rows, int n, int K, int32_t *idx, float *lp, cudaStream_t s);

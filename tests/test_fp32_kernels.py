@@ -111,3 +111,45 @@ def test_log_softmax_top_k_edges(n, K):
         if not bool(((gaps > 0) & (gaps < 1e-5)).any()):    # values that fp32 log-probabilities may merge
             assert idx[r].tolist() == want, r
         assert (lp[r][live] - ref[live]).abs().max() < 1e-5
+
+
+@pytest.mark.parametrize("hd,ps,dtype,tol", [(64, 16, torch.float32, 5e-6), (48, 5, torch.float32, 5e-6), (80, 16, torch.bfloat16, 2e-2), (528, 16, torch.float32, 5e-6)])
+@pytest.mark.parametrize("n", [1, 31, 33, 129, 600])
+@pytest.mark.parametrize("rows", [98, 99])
+def test_plain_attention_of_more_than_a_wave_vs_fp64(rows, n, hd, ps, dtype, tol):
+    """294 and 297 CTAs: the last grid that reads values ahead of their scores and the first that does not.  Rows of three sequences,
+    some of them padding, masks that hide tail keys (whose values hold anything)."""
+    H, G, tail = 3, 1, min(n, 4)
+    ctx = n - tail
+    g = torch.Generator().manual_seed(n)
+    pages = (n + ps - 1) // ps
+    q, kp, vp = (torch.randn(*s, generator=g).to(dtype) for s in ((rows, H, hd), (3 * pages, G, ps, hd), (3 * pages, G, ps, hd)))
+    table = torch.randperm(3 * pages, generator=g).to(torch.int32).view(3, pages)
+    if n > 1:                                                       # the third tail key of the last sequence is hidden from all its rows
+        vp[int(table[2, (ctx + 2) // ps]), :, (ctx + 2) % ps] = float("nan")
+    seq = (torch.arange(rows) % 4 - 1).to(torch.int32)              # -1: padding
+    full = torch.full((rows,), ctx, dtype=torch.int32)
+    lo = torch.full((rows,), 0b1011 if n > 1 else 1, dtype=torch.int64)
+    out = sb.attention(q.cuda(), kp.cuda(), vp.cuda(), table.cuda(), ps, seq.cuda(), full.cuda(), full.cuda(), lo.cuda(), torch.zeros_like(lo).cuda(), tail, G, n,
+                       impl=1).cpu().double()
+    assert not out[seq < 0].any()
+    seen = [j for j in range(n) if j < ctx or 0b1011 >> (j - ctx) & 1]
+    for s in range(3):
+        k, v = (t[table[s].long()].double()[:, 0].reshape(pages * ps, hd)[seen] for t in (kp, vp))
+        ref = torch.softmax(q[seq == s].double() @ k.T / hd ** 0.5, -1) @ v
+        assert (out[seq == s] - ref).abs().max() < tol              # scores of order 1 .. 3 in fp32, sums of up to 600 terms; bf16: the output's rounding
+
+
+@pytest.mark.parametrize("rows,short", [(1, 12), (1, 0), (300, 12), (300, 0)])
+def test_plain_attention_takes_as_many_keys_as_shared_memory_holds(rows, short):
+    """227 KB are a score per key, a query and 16 bytes: no form refuses what another takes.  (The keys a launch allows for, not those it has.)"""
+    hd, ps = 64, 16
+    most = (227 * 1024 - 16) // 4 - hd - 1 - short
+    g = torch.Generator().manual_seed(1)
+    q, kp, vp = (torch.randn(*s, generator=g) for s in ((rows, 1, hd), (2, 1, ps, hd), (2, 1, ps, hd)))
+    full = torch.full((rows,), 20, dtype=torch.int32, device="cuda")
+    lo = torch.ones(rows, dtype=torch.int64, device="cuda")
+    out = sb.attention(q.cuda(), kp.cuda(), vp.cuda(), torch.tensor([[1, 0]], dtype=torch.int32, device="cuda"), ps, torch.zeros_like(full), full, full, lo,
+                       torch.zeros_like(lo), 1, 1, most, impl=1).cpu().double()
+    k, v = (t.flip(0).double().reshape(2 * ps, hd)[:21] for t in (kp, vp))
+    assert (out[:, 0] - torch.softmax(q[:, 0].double() @ k.T / hd ** 0.5, -1) @ v).abs().max() < 5e-6

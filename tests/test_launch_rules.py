@@ -14,6 +14,7 @@ ASK = r"""
 #include "gemm_fused.cuh"
 using namespace spec;
 int main(int n, char **v) {                     // epilogue, rows, split, stages; or rows, rows per sequence, context, tail, grows (32 heads, 8 KV heads)
+  if (v[1][0] == 'a') { printf("%d", attn_ref_reads_ahead(atoi(v[2]), atoi(v[3]), atoi(v[4]), atoi(v[5])) ? 1 : 0); return 0; }      // "ahead", rows, heads, head size, keys
   if (n == 6) { printf("%d", attn_fast_plan(atoi(v[1]), 32, 8, 128, atoi(v[2]), atoi(v[3]), atoi(v[4]), atoi(v[5]) != 0) >> 1); return 0; }
   static char mem[64];
   FusedGemmArgs a;
@@ -65,3 +66,13 @@ def test_key_splits_of_a_launch_and_of_a_step_that_grows(ask, rows, rps, ctx, ta
     """No split without a key tile where the hint is the length; a captured step has one tile to grow by."""
     assert ask(rows, rps, ctx, tail, 0) == now
     assert ask(rows, rps, ctx, tail, 1) == growing
+
+
+@pytest.mark.parametrize("rows,H,hd,keys,ahead", [
+    (1, 4, 64, 100, 1), (74, 4, 64, 100, 1), (75, 4, 64, 100, 0), (240, 4, 64, 600, 0), (60, 32, 96, 2000, 0),
+    (60, 32, 96, 14000, 0), (60, 32, 96, 14700, 1),                 # four or three CTAs of the small form in an SM's 228 KB
+    (1, 1, 64, 58028, 1), (1, 1, 64, 58033, 0),                     # 227 KB
+    (262144, 64, 128, 100, 0),
+])
+def test_plain_attention_reads_ahead_in_one_wave(ask, rows, H, hd, keys, ahead):
+    assert ask("ahead", rows, H, hd, keys) == ahead
