@@ -132,7 +132,7 @@ int spec_step_async(spec_ctx *ctx, int32_t *dev_ids, int32_t *dev_counts);
  * drawn from that residual (inverse CDF over increasing ids).  The emitted tokens are distributed as plain sampling
  * from the target.  The random numbers are inputs: u host float [batch][2 * tree_nodes] in [0, 1); u[b][c] decides
  * node c of sequence b, u[b][tree_nodes + cur] draws the final token at node cur.  out_ids / out_counts as spec_step.
- * 0 < temperature <= 1e4.  Synchronises. */
+ * 0 < temperature <= 1e4; vocab <= 2^26 (SPEC_ERR_UNSUPPORTED).  Synchronises. */
 int spec_step_sampled(spec_ctx *ctx, float temperature, const float *u, int32_t *out_ids, int32_t *out_counts);
 
 /* Plain greedy decoding of the target on the same kernels (the paper's "vanilla" baseline): one target

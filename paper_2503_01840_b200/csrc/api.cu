@@ -1008,8 +1008,11 @@ template <typename T> struct Sched {
     c->cur_rps = rps;
     target_forward(rows, rps, true);
     mark(SPEC_PROF_TREE);
-    if (c->sampled && !plain) tick(launch_accept_sampled(c->st, c->tb, c->logits, c->V, c->u_dev, c->mass_part, c->B, rps, s));
-    else { launch_accept(c->st, c->tb, c->B, rps, s); tick(); }
+    if (c->sampled && !plain) {
+      const int n = launch_accept_sampled(c->st, c->tb, c->logits, c->V, c->u_dev, c->mass_part, c->B, rps, s);
+      if (n < 0 && !c->sched_err) c->sched_err = n;
+      tick(std::max(n, 0));
+    } else { launch_accept(c->st, c->tb, c->B, rps, s); tick(); }
     PageMap pm{c->page_table, c->pps, c->cfg.page_size, c->cfg.num_pages};
     mark(SPEC_PROF_COMMIT); launch_commit<T>(c->st, c->tb, c->pools_dev, pm, (const T *)c->node_taps, (T *)c->pend_taps, c->B, c->L, c->G, c->hd,
                      c->k, rps, s);
@@ -1269,7 +1272,7 @@ static int launch_step(spec_ctx *c, bool plain) {
   if (!use_graph) {
     if (c->cfg.dtype == SPEC_F32) Sched<float>(c).step(plain); else Sched<bf16>(c).step(plain);
     CUDA_TRY(c, cudaGetLastError());
-    if (c->sched_err) return fail(c, SPEC_ERR_CUDA, "a GEMM launch was rejected (code %d)", c->sched_err);
+    if (c->sched_err) return fail(c, SPEC_ERR_CUDA, "a launch was rejected (code %d)", c->sched_err);
     return SPEC_OK;
   }
   cudaGraphExec_t &graph = c->sampled ? c->graph_sampled : c->graph;
@@ -1280,7 +1283,7 @@ static int launch_step(spec_ctx *c, bool plain) {
     if (c->cfg.dtype == SPEC_F32) Sched<float>(c).step(false); else Sched<bf16>(c).step(false);
     cudaError_t e = cudaStreamEndCapture(c->stream, &gr);
     if (e != cudaSuccess) return fail(c, SPEC_ERR_CUDA, "graph capture: %s", cudaGetErrorString(e));
-    if (c->sched_err) { cudaGraphDestroy(gr); return fail(c, SPEC_ERR_CUDA, "a GEMM launch was rejected (code %d)", c->sched_err); }
+    if (c->sched_err) { cudaGraphDestroy(gr); return fail(c, SPEC_ERR_CUDA, "a launch was rejected (code %d)", c->sched_err); }
     e = cudaGraphInstantiate(&graph, gr, 0);
     cudaGraphDestroy(gr);
     if (e != cudaSuccess) { graph = nullptr; return fail(c, SPEC_ERR_CUDA, "graph instantiate: %s", cudaGetErrorString(e)); }
@@ -1332,6 +1335,7 @@ extern "C" int spec_step_sampled(spec_ctx *c, float temperature, const float *u,
   if (!c) return SPEC_ERR_NULL;
   if (!u || !out_ids || !out_counts) return fail(c, SPEC_ERR_NULL, "spec_step_sampled: NULL argument");
   if (!(temperature > 0.0f) || !(temperature <= 1e4f)) return fail(c, SPEC_ERR_INVALID_CFG, "spec_step_sampled: the temperature must be in (0, 1e4]");
+  if (!accept_sampled_takes(c->V)) return fail(c, SPEC_ERR_UNSUPPORTED, "spec_step_sampled: vocabularies of up to 2^26 ids");
   if (c->draft_stale) return fail(c, SPEC_ERR_STATE, "spec_step_sampled after spec_plain_step: the draft cache is stale, prefill again");
   if (int rc = check_capacity(c, c->Pmax, "spec_step_sampled")) return rc;
   const size_t nu = (size_t)c->B * 2 * c->N;

@@ -54,8 +54,10 @@ void launch_rerank(SeqState st, TreeBufs tb, RowMeta m, int B, cudaStream_t s);
 void launch_plain_tree(SeqState st, TreeBufs tb, RowMeta m, int B, cudaStream_t s);
 void launch_accept(SeqState st, TreeBufs tb, int B, int rows_per_seq, cudaStream_t s);
 // Stochastic acceptance: logits fp32 [B * rows_per_seq][V] of the verify pass; u = B x 2N uniforms followed by one float,
-// 1 / temperature (all device memory); mass_part [B * rows_per_seq][accept_mass_chunks(V)].  Returns the number of kernels launched.
+// 1 / temperature (all device memory); mass_part [B * rows_per_seq][accept_mass_chunks(V)].  Returns the number of kernels launched, -1
+// where a launch was rejected or V has more runs than the walk has room for.
 int accept_mass_chunks(int V);
+bool accept_sampled_takes(int V);
 int launch_accept_sampled(SeqState st, TreeBufs tb, const float *logits, int V, const float *u, float2 *mass_part, int B, int rows_per_seq,
                           cudaStream_t s);
 template <typename T>

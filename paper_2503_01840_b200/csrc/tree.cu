@@ -1051,14 +1051,16 @@ __device__ __forceinline__ float acc_exp(float x) { return __expf(x); }
 // Here the whole chip reads all rows once, and the walk needs a few numbers a node.  Sampled step of the 8B shapes over a greedy one, 6.2
 // nodes visited: 145 -> 65 us (of which the logits' way to memory, the uniforms' copy and the host take 40).
 constexpr int MASS_CHUNK = 8192;
-int accept_mass_chunks(int V) { return (V + MASS_CHUNK - 1) / MASS_CHUNK; }
+int accept_mass_chunks(int V) { return (int)(((long long)V + MASS_CHUNK - 1) / MASS_CHUNK); }
+bool accept_sampled_takes(int V) { return accept_mass_chunks(V) <= MASS_CHUNK; }      // the walk holds a row's masses in the place of a run's terms
+// grid (rows, chunks): there are up to 4096 x 64 rows, and a grid's second index ends at 65535
 __global__ void __launch_bounds__(256) row_mass_kernel(const float *__restrict__ logits, int V, const float *__restrict__ inv_temp, float2 *__restrict__ part) {
   pdl_wait();
   pdl_trigger();
   __shared__ float red[2][8];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int v0 = blockIdx.x * MASS_CHUNK, n = min(MASS_CHUNK, V - v0);
-  const float *z = logits + (size_t)blockIdx.y * V + v0;
+  const int v0 = blockIdx.y * MASS_CHUNK, n = min(MASS_CHUNK, V - v0);
+  const float *z = logits + (size_t)blockIdx.x * V + v0;
   const float inv_T = *inv_temp;
   constexpr int PER = MASS_CHUNK / 256;
   float v[PER];
@@ -1094,7 +1096,7 @@ __global__ void __launch_bounds__(256) row_mass_kernel(const float *__restrict__
     sum = red[1][0];
 #pragma unroll
     for (int w = 1; w < 8; w++) sum += red[1][w];
-    part[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = make_float2(m, sum);
+    part[(size_t)blockIdx.x * gridDim.y + blockIdx.y] = make_float2(m, sum);
   }
 }
 
@@ -1174,7 +1176,7 @@ __global__ void __launch_bounds__(ACC_THREADS) accept_sampled_kernel(SeqState st
   // ---- the final token: inverse CDF over the residual, in three levels.  One thread finds the chunk that holds the target, the chunk's
   // terms go to shared memory, one thread finds the warp whose 32nd of them holds what is left of it, and that warp walks its range 32 ids at a
   // time with a warp prefix sum.
-  for (int c = tid; c < chunks; c += ACC_THREADS) {          // masses of the chunks (at most MASS_CHUNK of them: V < 2^26), without the rejected tokens
+  for (int c = tid; c < chunks; c += ACC_THREADS) {          // masses of the chunks (at most MASS_CHUNK of them), without the rejected tokens
     const float2 mp = mass_part[(row0 + cur) * chunks + c];
     float m = mp.y > 0.0f ? mp.y * acc_exp((mp.x - zmax) * inv_T) : 0.0f;
     for (int r = 0; r < nrej; r++)
@@ -1264,9 +1266,10 @@ __global__ void __launch_bounds__(ACC_THREADS) accept_sampled_kernel(SeqState st
   }
 }
 int launch_accept_sampled(SeqState st, TreeBufs tb, const float *logits, int V, const float *u, float2 *mass_part, int B, int rows_per_seq, cudaStream_t s) {
+  if (!accept_sampled_takes(V)) return -1;
   const int chunks = accept_mass_chunks(V);
-  launch_k(row_mass_kernel, dim3(chunks, B * rows_per_seq), dim3(256), 0, s, logits, V, u + (size_t)B * 2 * tb.N, mass_part);
-  launch_k(accept_sampled_kernel, dim3(B), dim3(ACC_THREADS), 0, s, st, tb, logits, V, u, (const float2 *)mass_part, chunks, rows_per_seq);
+  if (launch_k(row_mass_kernel, dim3(B * rows_per_seq, chunks), dim3(256), 0, s, logits, V, u + (size_t)B * 2 * tb.N, mass_part) != cudaSuccess) return -1;
+  if (launch_k(accept_sampled_kernel, dim3(B), dim3(ACC_THREADS), 0, s, st, tb, logits, V, u, (const float2 *)mass_part, chunks, rows_per_seq) != cudaSuccess) return -1;
   return 2;
 }
 

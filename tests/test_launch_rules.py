@@ -12,9 +12,11 @@ ASK = r"""
 #include <cstdlib>
 #include "attn_fast.cuh"
 #include "gemm_fused.cuh"
+#include "state.cuh"
 using namespace spec;
 int main(int n, char **v) {                     // epilogue, rows, split, stages; or rows, rows per sequence, context, tail, grows (32 heads, 8 KV heads)
   if (v[1][0] == 'a') { printf("%d", attn_ref_reads_ahead(atoi(v[2]), atoi(v[3]), atoi(v[4]), atoi(v[5])) ? 1 : 0); return 0; }      // "ahead", rows, heads, head size, keys
+  if (v[1][0] == 'v') { printf("%d", accept_sampled_takes(atoi(v[2])) ? accept_mass_chunks(atoi(v[2])) : -accept_mass_chunks(atoi(v[2]))); return 0; }      // "vocabulary", ids
   if (n == 6) { printf("%d", attn_fast_plan(atoi(v[1]), 32, 8, 128, atoi(v[2]), atoi(v[3]), atoi(v[4]), atoi(v[5]) != 0) >> 1); return 0; }
   static char mem[64];
   FusedGemmArgs a;
@@ -76,3 +78,9 @@ def test_key_splits_of_a_launch_and_of_a_step_that_grows(ask, rows, rps, ctx, ta
 ])
 def test_plain_attention_reads_ahead_in_one_wave(ask, rows, H, hd, keys, ahead):
     assert ask("ahead", rows, H, hd, keys) == ahead
+
+
+@pytest.mark.parametrize("vocab,chunks", [(2, 1), (8192, 1), (8193, 2), (128256, 16), (1 << 26, 8192), ((1 << 26) + 1, -8193), (2 ** 31 - 1, -262144)])
+def test_vocabularies_of_the_stochastic_acceptance(ask, vocab, chunks):
+    """Runs of 8192 ids; one CTA's shared memory holds the masses of 8192 runs, and a larger vocabulary is refused."""
+    assert ask("vocabulary", vocab) == chunks
