@@ -1041,9 +1041,10 @@ void launch_accept(SeqState st, TreeBufs tb, int B, int rows_per_seq, cudaStream
 // has a fixed order, so a step is reproducible on this kernel.
 constexpr int ACC_THREADS = 1024;
 constexpr int ACC_MAX_REJ = 64;
+constexpr float ACC_LEAST = 1e-30f;      // of the row's mass, below which a run of ids counts as empty: its terms may be 0 one by one
 
-// exp on the special-function unit (ex2.approx): every term of a row goes through the same routine, so the
-// probabilities stay consistent; its relative error (~1e-6 near the maximum) is far inside the parity slack
+// exp on the special-function unit (ex2.approx), relative error ~1e-6 near the maximum, far inside the parity slack.  A term of a
+// row's mass is the product of two, of its distance to its run's maximum and of the run's to the row's.
 __device__ __forceinline__ float acc_exp(float x) { return __expf(x); }
 
 // Masses of the verify rows: per run of MASS_CHUNK ids the largest logit and sum exp((z - largest) / T), [row][chunk].  The acceptance walks one
@@ -1110,7 +1111,8 @@ __global__ void __launch_bounds__(ACC_THREADS) accept_sampled_kernel(SeqState st
   __shared__ float part[NWARP];
   __shared__ int32_t rej[ACC_MAX_REJ];
   __shared__ float rej_e[ACC_MAX_REJ];
-  __shared__ int s_cur, s_len, s_nrej, s_pick, s_owner;
+  __shared__ int again[ACC_MAX_REJ];                         // chunks whose residual is added up again
+  __shared__ int s_cur, s_len, s_nrej, s_pick, s_owner, s_again;
   __shared__ float s_target;
   __shared__ int32_t tok[64];
   __shared__ float ub[128], zc[64], zmax_s[64], mass_s[64];
@@ -1167,7 +1169,7 @@ __global__ void __launch_bounds__(ACC_THREADS) accept_sampled_kernel(SeqState st
       cur = nxt;
       a++;
     }
-    s_cur = cur; s_len = a; s_nrej = nrej;
+    s_cur = cur; s_len = a; s_nrej = nrej; s_again = 0;
   }
   __syncthreads();
   const int cur = s_cur, a = s_len, nrej = s_nrej;
@@ -1176,14 +1178,39 @@ __global__ void __launch_bounds__(ACC_THREADS) accept_sampled_kernel(SeqState st
   // ---- the final token: inverse CDF over the residual, in three levels.  One thread finds the chunk that holds the target, the chunk's
   // terms go to shared memory, one thread finds the warp whose 32nd of them holds what is left of it, and that warp walks its range 32 ids at a
   // time with a warp prefix sum.
+  // The residual of a chunk is its mass without the rejected tokens'.  Where they are more than half of it, the difference has lost bits,
+  // up to all of them, and what is left is added up again from its terms.
+  auto residual = [&](int id) {                              // term of an id, 0 for a rejected one
+    float e = acc_exp((z[id] - zmax) * inv_T);
+    for (int r = 0; r < nrej; r++)
+      if (rej[r] == id) e = 0.0f;
+    return e;
+  };
   for (int c = tid; c < chunks; c += ACC_THREADS) {          // masses of the chunks (at most MASS_CHUNK of them), without the rejected tokens
     const float2 mp = mass_part[(row0 + cur) * chunks + c];
-    float m = mp.y > 0.0f ? mp.y * acc_exp((mp.x - zmax) * inv_T) : 0.0f;
+    const float m = mp.y > 0.0f ? mp.y * acc_exp((mp.x - zmax) * inv_T) : 0.0f;
+    float left = m;
+    bool less = false;
     for (int r = 0; r < nrej; r++)
-      if (rej[r] / MASS_CHUNK == c) m = fmaxf(m - rej_e[r], 0.0f);
-    seg[c] = m;
+      if (rej[r] / MASS_CHUNK == c) { left -= rej_e[r]; less = true; }
+    if (less && !(left >= 0.5f * m)) again[atomicAdd(&s_again, 1)] = c;      // one per rejected token at most
+    seg[c] = left > ACC_LEAST ? left : 0.0f;
   }
   __syncthreads();
+  for (int q = 0; q < s_again; q++) {
+    const int c0 = again[q] * MASS_CHUNK, n = min(MASS_CHUNK, V - c0);
+    float loc = 0.0f;
+    for (int i = tid; i < n; i += ACC_THREADS) loc += residual(c0 + i);
+    for (int o = 16; o > 0; o >>= 1) loc += __shfl_xor_sync(0xffffffffu, loc, o);
+    if (ln == 0) part[wid] = loc;
+    __syncthreads();
+    if (tid == 0) {
+      float m = 0.0f;
+      for (int w = 0; w < NWARP; w++) m += part[w];
+      seg[again[q]] = m > ACC_LEAST ? m : 0.0f;
+    }
+    __syncthreads();
+  }
   if (tid == 0) {
     float total = 0.0f;
     for (int c = 0; c < chunks; c++) total += seg[c];
@@ -1204,12 +1231,7 @@ __global__ void __launch_bounds__(ACC_THREADS) accept_sampled_kernel(SeqState st
   __syncthreads();
   const int c0 = s_owner * MASS_CHUNK, n = min(MASS_CHUNK, V - c0);
   const float in_chunk = s_target;
-  for (int i = tid; i < n; i += ACC_THREADS) {
-    float e = acc_exp((z[c0 + i] - zmax) * inv_T);
-    for (int r = 0; r < nrej; r++)
-      if (rej[r] == c0 + i) e = 0.0f;
-    seg[i] = e;
-  }
+  for (int i = tid; i < n; i += ACC_THREADS) seg[i] = residual(c0 + i);
   __syncthreads();
   const int CW = (n + NWARP - 1) / NWARP, w0 = wid * CW, w1 = min(w0 + CW, n);
   float loc = 0.0f;
