@@ -153,7 +153,8 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float *f) {     // no 
         "=r"(v[30]), "=r"(v[31])
       : "r"(taddr));
 }
-// values that a tmem_ld32 put out, from here on: nothing that uses them moves to before the wait for them
+// values that a tmem_ld32 put out, from here on: no arithmetic on them moves to before the wait for them.  Copies may: so the paths
+// of two such loads into the same values meet only behind their waits (the compiler makes their registers the same where they meet).
 __device__ __forceinline__ void pin32(float *f) {
   asm volatile("" : "+f"(f[0]), "+f"(f[1]), "+f"(f[2]), "+f"(f[3]), "+f"(f[4]), "+f"(f[5]), "+f"(f[6]), "+f"(f[7]), "+f"(f[8]), "+f"(f[9]), "+f"(f[10]), "+f"(f[11]),
                     "+f"(f[12]), "+f"(f[13]), "+f"(f[14]), "+f"(f[15]));
@@ -371,25 +372,27 @@ __global__ void __launch_bounds__(CA_THREADS, 1) attn_causal_kernel(const __grid
     bool alive = true;
     // The scores of step i into s, once they are complete
     float s[CA_KS];
-    auto fetch = [&](int i) {
+    auto ask = [&](int i) {
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       tmem_ld32(my_s + (uint32_t)((i & 1) * CA_KS), s);
       tmem_ld32(my_s + (uint32_t)((i & 1) * CA_KS + 32), s + 32);
+    };
+    auto got = [&]() {                                           // in the same straight line as ask()
+      tmem_ld_wait();
+      pin32(s);
+      pin32(s + 32);
     };
     auto gave_up = [&](int site, int i) {
       if (lane == 0) { *abort_flag = 1; if (p.status) set_status(p.status, ST_TIMEOUT, site, blockIdx.y, i); }
       alive = false;
     };
     auto await = [&](int i) {
-      if (mbar_wait_warp(&s_bar[t * 2 + (i & 1)], (uint32_t)((i >> 1) & 1), p.spin)) fetch(i);
+      if (mbar_wait_warp(&s_bar[t * 2 + (i & 1)], (uint32_t)((i >> 1) & 1), p.spin)) { ask(i); got(); }
       else gave_up(435, i);
     };
     float nb_ = 0.0f;                                            // the reference maximum in the exponent (0 while there is none)
     if (nt > 0) await(0);
     for (int i = 0; i < nt && alive; i++) {
-      tmem_ld_wait();
-      pin32(s);
-      pin32(s + 32);
       const int k0 = i * CA_KS;
       if (k0 + CA_KS - 1 > pos - lane) {                         // uniform over the warp: its first row does not see the whole step
         const int lim = pos - k0;                                // keys 0..lim of the step
@@ -441,20 +444,28 @@ __global__ void __launch_bounds__(CA_THREADS, 1) attn_causal_kernel(const __grid
       }
       tmem_st32(my_s + (uint32_t)((i & 1) * CA_KS), pk);
       const bool ready = i + 1 < nt && mbar_test_warp(&s_bar[t * 2 + ((i + 1) & 1)], (uint32_t)(((i + 1) >> 1) & 1));
-      if (ready) fetch(i + 1);                                   // mostly: the loads run beside the wait for the stores of P
-      l += (rs[0].x + rs[0].y) + (rs[1].x + rs[1].y);
-      if (BRIEF) {
+      auto hand_over = [&]() {                                   // the sums, and P to the MMA warp once it is written
+        l += (rs[0].x + rs[0].y) + (rs[1].x + rs[1].y);
+        if (BRIEF) {
 #pragma unroll
-        for (int z = 0; z < 2; z++) rs[z] = make_float2(0.f, 0.f);
+          for (int z = 0; z < 2; z++) rs[z] = make_float2(0.f, 0.f);
 #pragma unroll
-        for (int e = 0; e < 32; e++) rs[e & 1] = add2(rs[e & 1], bf2(pk[e]));
-        lrnd += (rs[0].x + rs[0].y) + (rs[1].x + rs[1].y);
+          for (int e = 0; e < 32; e++) rs[e & 1] = add2(rs[e & 1], bf2(pk[e]));
+          lrnd += (rs[0].x + rs[0].y) + (rs[1].x + rs[1].y);
+        }
+        tmem_st_wait();
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&p_bar[t * 2 + (i & 1)]);
+      };
+      if (ready) {                                               // mostly: the loads run beside the wait for the stores of P
+        ask(i + 1);
+        hand_over();
+        got();
+      } else {
+        hand_over();
+        if (i + 1 < nt) await(i + 1);
       }
-      tmem_st_wait();
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&p_bar[t * 2 + (i & 1)]);
-      if (i + 1 < nt && !ready) await(i + 1);
     }
     if (alive && nt > 0) {
       // All P V of the tile.  A barrier of its own: the scores of the last step only tell that the P V two steps earlier is

@@ -152,3 +152,17 @@ def test_attention_reads_ahead_only_behind_launches_that_wait_first():
         before = [m for m in re.finditer(r"(\w+)(?:<T>)?\(", api[:c]) if m.group(1) in ("fgemm", "wgemm", "gemm", "gemm_cat") or m.group(1).startswith("launch_")]
         last = before[-1]
         assert last.group(1) in ("launch_rope_kv", "launch_norm_qkv") or api[last.end():].startswith("EPI_QKV"), last.group(1)
+
+
+def test_scores_in_flight_are_waited_for_before_two_loads_of_them_meet():
+    """The causal kernel asks for the next step's scores at two places.  Before tcgen05.wait::ld nothing may read them, not even a copy that
+    the compiler puts where two paths with a load each come together: every request is followed by its wait in its own straight line."""
+    bodies = {name: body for _, name, body in _kernel_bodies()}
+    body = bodies["attn_causal_kernel"]
+    asked = [m for m in re.finditer(r"\b(\w+)\(i(?: \+ 1)?\);", body) if m.group(1) == "ask"]
+    assert len(asked) == 2, "requests for scores"
+    for m in asked:
+        between = body[m.end(): body.index("got();", m.end())]
+        assert not re.search(r"[{}]|\b(if|for|while|break|ask)\b", between), between
+    wait = body[body.index("auto got = "):]
+    assert wait.index("tmem_ld_wait();") < wait.index("pin32(s);") < wait.index("pin32(s + 32);") < wait.index("};")
