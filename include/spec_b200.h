@@ -176,7 +176,7 @@ int spec_step_bytes(spec_ctx *ctx, double *bytes);
 int spec_free(spec_ctx *ctx);
 const char *spec_last_error(const spec_ctx *ctx);
 
-/* ---- inspection for parity tests (synchronises; copies to host) ----------------------------- */
+/* ---- inspection for parity tests (synchronises; copies to host): the last step, a tree of one node per sequence after a plain one */
 enum spec_debug_what {
   SPEC_DBG_TREE_TOK = 1,     /* int32 [nodes]            */
   SPEC_DBG_TREE_PARENT,      /* int32 [nodes], root -1   */

@@ -138,6 +138,7 @@ struct spec_ctx {
   std::vector<int32_t> n_upper, cap_host, n_pages_host;
   std::vector<int32_t> page_table_host;
   bool prefilled = false, draft_stale = false;
+  int seq_rows = 0;            // verify rows of a sequence in the last step, which spec_debug_read reads: tree_nodes, 1 after a plain step
   cudaGraphExec_t graph = nullptr;
   cudaGraphExec_t graph_sampled = nullptr;   // the same step with the stochastic acceptance kernel
   StepPlan graph_plan[2];                    // of graph, graph_sampled
@@ -356,6 +357,7 @@ extern "C" int spec_init(spec_ctx **out, const spec_target_weights *tw, const sp
     spec_free(c);
     return fail(nullptr, SPEC_ERR_CUDA, "spec_init: no pinned host memory");
   }
+  c->seq_rows = c->N;
   c->n_upper.assign(c->B, 0); c->cap_host.assign(c->B, 0); c->n_pages_host.assign(c->B, 0);
   c->page_table_host.assign((size_t)c->B * c->pps, 0);
   if (cfg->dtype == SPEC_BF16 && !((cfg->flags & SPEC_FLAG_REF_GEMM))) {
@@ -1255,6 +1257,7 @@ template <typename T> static int do_prefill(spec_ctx *c, const int32_t *ids, con
   for (int b = 0; b < B; b++) { c->n_upper[b] = lens[b]; first[b] = root[b]; }
   c->prefilled = true;
   c->draft_stale = false;
+  c->seq_rows = c->N;
   drop_stale_graphs(c);
   return rc;
 }
@@ -1269,6 +1272,7 @@ extern "C" int spec_prefill(spec_ctx *c, const int32_t *ids, const int32_t *lens
 static int launch_step(spec_ctx *c, bool plain) {
   bool use_graph = !(c->cfg.flags & SPEC_FLAG_NO_GRAPH) && !plain;
   c->launches = 0;
+  c->seq_rows = plain ? 1 : c->N;
   if (!use_graph) {
     if (c->cfg.dtype == SPEC_F32) Sched<float>(c).step(plain); else Sched<bf16>(c).step(plain);
     CUDA_TRY(c, cudaGetLastError());
@@ -1472,7 +1476,7 @@ extern "C" int64_t spec_debug_read(spec_ctx *c, int32_t what, int32_t seq, void 
   int32_t nn = 0, cnt = 0;
   cudaMemcpy(&nn, c->tb.nn + seq, 4, cudaMemcpyDeviceToHost);
   cudaMemcpy(&cnt, c->tb.out_cnt + seq, 4, cudaMemcpyDeviceToHost);
-  size_t t0 = (size_t)seq * c->N, p0 = (size_t)seq * (c->pool + 1);
+  size_t t0 = (size_t)seq * c->seq_rows, p0 = (size_t)seq * (c->pool + 1);
   const TreeBufs &t = c->tb;
   switch (what) {
     case SPEC_DBG_TREE_TOK: return copy_out(c, t.tok + t0, nn, dst, bytes);
