@@ -63,13 +63,21 @@ class ClockSampler:
          "clocks_event_reasons.hw_thermal_slowdown,clocks_event_reasons.sw_thermal_slowdown,clocks_event_reasons.sw_power_cap")
 
     def __init__(self, gpu_index: int):
+        """Returns once samples come in: nvidia-smi takes longer to start than a short timed region lasts."""
         self.f = tempfile.NamedTemporaryFile("w+", suffix=".csv", delete=False)
-        self.p = None
+        self.p, self.before = None, 0
         try:
-            self.p = subprocess.Popen(["nvidia-smi", f"--query-gpu={self.Q}", "--format=csv,noheader,nounits", "-lms", "100",
+            self.p = subprocess.Popen(["nvidia-smi", f"--query-gpu={self.Q}", "--format=csv,noheader,nounits", "-lms", "20",
                                        "-i", str(gpu_index)], stdout=self.f, stderr=subprocess.DEVNULL)
+            t0 = time.time()
+            while os.path.getsize(self.f.name) == 0 and self.p.poll() is None and time.time() - t0 < 5.0:
+                time.sleep(0.01)
         except Exception:
             self.p = None
+
+    def mark(self):
+        """The timed region starts here: what was sampled before does not count."""
+        self.before = os.path.getsize(self.f.name)
 
     def stop(self):
         out = {"sm_mhz": None, "sm_max_mhz": None, "reasons": [], "samples": 0}
@@ -81,7 +89,7 @@ class ClockSampler:
         except Exception:
             self.p.kill()
         self.f.flush()
-        self.f.seek(0)
+        self.f.seek(self.before)
         sm, mx, reasons = [], [], set()
         for line in self.f.read().splitlines():
             c = [x.strip() for x in line.split(",")]
@@ -279,12 +287,14 @@ def main():
     prefill_launches = dec.launches_per_step()
 
     counts = torch.zeros(max(args.steps, args.warmup + 16, 16), B, dtype=torch.int32, device=dev)
+    sampler = ClockSampler(local) if rank == 0 else None
     timed_steps(dec, args.warmup, counts)
     n_mid = dec.lengths().astype(np.float64)
     bytes_step = dec.step_bytes()
     if world > 1:
         dist.barrier()
-    sampler = ClockSampler(local) if rank == 0 else None
+    if sampler:
+        sampler.mark()
     if args.nvtx:
         torch.cuda.nvtx.range_push("timed_steps")
     ms, toks = timed_steps(dec, args.steps, counts)

@@ -166,3 +166,22 @@ def test_scores_in_flight_are_waited_for_before_two_loads_of_them_meet():
         assert not re.search(r"[{}]|\b(if|for|while|break|ask)\b", between), between
     wait = body[body.index("auto got = "):]
     assert wait.index("tmem_ld_wait();") < wait.index("pin32(s);") < wait.index("pin32(s + 32);") < wait.index("};")
+
+
+def test_clock_record_of_a_short_timed_region(tmp_path, monkeypatch):
+    """A region of 0.1 s has samples of its own, however long nvidia-smi takes to start (a stand-in for it here)."""
+    import time
+    fake = tmp_path / "nvidia-smi"
+    fake.write_text('#!/bin/bash\nsleep 0.3\necho "0, 600, 1965, 200.0, 0x1, Not Active, Not Active, Not Active, Not Active"\n'
+                    'while [ ! -e "%s" ]; do sleep 0.01; done\n'
+                    'while true; do echo "0, 1900, 1965, 900.0, 0x4, Not Active, Not Active, Not Active, Active"; sleep 0.01; done\n' % (tmp_path / "busy"))
+    fake.chmod(0o755)
+    monkeypatch.setenv("PATH", f"{tmp_path}:{os.environ['PATH']}")
+    monkeypatch.syspath_prepend(ROOT)
+    import bench
+    sampler = bench.ClockSampler(0)
+    sampler.mark()
+    (tmp_path / "busy").write_text("")
+    time.sleep(0.3)
+    out = sampler.stop()
+    assert out["samples"] >= 2 and out["sm_mhz"] == 1900 and out["sm_max_mhz"] == 1965 and out["reasons"] == ["sw_power_cap"], out
