@@ -55,8 +55,10 @@ void launch_argmax(const float *logits, int rows, int n, int32_t *idx, cudaStrea
 }
 
 // log-softmax + top-K, (value desc, index asc).  Row r reads logits row src_row[r] when given.
-// PER > 0: up to PER * 256 logits, which a thread reads once and keeps; every warp then ranks its own K best by warp-wide reductions and
-// warp 0 those of all warps by counting.  PER = 0: any number, read again for each of the K results.  1024 logits, K = 4, cold: 9.4 -> 5.6 us.
+// PER > 0: up to PER * 256 logits, which a thread reads once and keeps; every warp then ranks its own K best by warp-wide reductions, and
+// a thread per entry those of all warps by counting.  PER = 0: any number, read again for each of the K results.  Cold, PER = 0 / PER > 0: 1024
+// logits, K = 4: 9.4 / 5.6 us.  (With the keys made again for each result and all 8 K entries ranked by one warp, K = 16 took 16.6 to 17.2 us
+// at 200 logits where PER = 0 takes 15.4, and 1024 rows of 1025 logits 58 where it takes 43.)
 template <int PER>
 __global__ void __launch_bounds__(256) logsoftmax_topk_kernel(const float *__restrict__ logits, const int32_t *src_row,
                                                               int n, int K, int32_t *__restrict__ idx,
@@ -105,29 +107,29 @@ __global__ void __launch_bounds__(256) logsoftmax_topk_kernel(const float *__res
   for (int w = 0; w < 8; w++) sum += shf[1][w];
   const float lse = logf(sum);
   if (PER > 0) {
-    unsigned taken = 0u;                                   // of this thread's values
+    unsigned key[PER > 0 ? PER : 1];                       // of this thread's values that are still to be taken (keys of values are >= 1)
+#pragma unroll
+    for (int j = 0; j < PER; j++) key[j] = threadIdx.x + j * 256 < n ? ordered_key((v[j] - mx) - lse) : 0u;
     for (int c = 0; c < K; c++) {
       unsigned bk = 0u, wk;
-      int bi = -1, bj = 0;
+      int bj = -1;
 #pragma unroll
-      for (int j = 0; j < PER; j++) {
-        const int i = threadIdx.x + j * 256;
-        const unsigned k = ordered_key((v[j] - mx) - lse);
-        if (i < n && !(taken >> j & 1u) && (bi < 0 || k > bk)) { bk = k; bi = i; bj = j; }      // equal: the lower index stays
-      }
+      for (int j = 0; j < PER; j++)
+        if (key[j] > bk) { bk = key[j]; bj = j; }          // equal: the lower index stays
+      const int bi = bj < 0 ? -1 : (int)threadIdx.x + bj * 256;
       const int wi = warp_best(bk, bi, &wk);
-      if (wi >= 0 && wi == bi) taken |= 1u << bj;
+#pragma unroll
+      for (int j = 0; j < PER; j++)
+        if (wi == (int)threadIdx.x + j * 256) key[j] = 0u;
       if (lane == 0) cand[warp * K + c] = make_uint2(wk, (unsigned)wi);
     }
     __syncthreads();
-    if (warp > 0) return;
-    for (int e = lane; e < 8 * K; e += 32) {
-      const uint2 me = cand[e];
-      if ((int)me.y < 0) continue;                         // the warp has fewer than K values
-      int rank = 0;
-      for (int o = 0; o < 8 * K; o++) { const uint2 w = cand[o]; rank += (int)w.y >= 0 && (w.x > me.x || (w.x == me.x && w.y < me.y)); }
-      if (rank < K) { idx[(size_t)r * K + rank] = (int)me.y; lp[(size_t)r * K + rank] = key_value(me.x); }
-    }
+    if ((int)threadIdx.x >= 8 * K) return;                 // an entry per thread: one warp for all of them took a third of the launch at K = 16
+    const uint2 me = cand[threadIdx.x];
+    if ((int)me.y < 0) return;                             // its warp has fewer than K values
+    int rank = 0;
+    for (int o = 0; o < 8 * K; o++) { const uint2 w = cand[o]; rank += (int)w.y >= 0 && (w.x > me.x || (w.x == me.x && w.y < me.y)); }
+    if (rank < K) { idx[(size_t)r * K + rank] = (int)me.y; lp[(size_t)r * K + rank] = key_value(me.x); }
     return;
   }
   float pv = INFINITY;
