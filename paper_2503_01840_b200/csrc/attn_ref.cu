@@ -21,7 +21,7 @@ template <bool VEC> __device__ __forceinline__ float4 load4(const bf16 *p) {
   return make_float4(to_f32(p[0]), to_f32(p[1]), to_f32(p[2]), to_f32(p[3]));
 }
 
-// A launch of at most one wave is bound by latency: a row attends tens to hundreds of keys.  So there (AHEAD) are four dependent round
+// A launch of a wave or two is bound by latency: a row attends tens to hundreds of keys.  So there (AHEAD) are four dependent round
 // trips and no more for up to 8192 / head_dim keys: metadata, page ids, K and V rows together, output.  Four threads share a key's dot product
 // (256 keys a round, their page ids and then their rows requested at once), and a thread's first V_AHEAD values, whose addresses need no
 // score, are requested before the scores.  The value pass splits the keys over the threads that are left beside hd / 4 dimension groups.
@@ -188,15 +188,18 @@ __global__ void __launch_bounds__(ArShape<AHEAD>::THREADS, ArShape<AHEAD>::PER_S
   }
 }
 
-// Whether a launch reads ahead: up to one wave of that form, two CTAs an SM (registers).  Above, the form with ten CTAs an SM is faster, up to
-// 2.6 times, as long as shared memory (a score for every key that the caller allows for) holds more than three of them.  Called in a row, us,
-// reading ahead / not: fp32 hd 64, 240 CTAs 6.9 / 7.4 with 20 keys, 13.0 / 20.8 with 250, 34 / 67 with 1000; 300 CTAs 9.9 / 6.9, 20.1 / 20.6,
-// 63 / 65; 960 CTAs 18.8 / 7.9, 39.6 / 23.1, 125 / 72; bf16 hd 96, 320 CTAs 12.6 / 8.4, 30.9 / 29.2, 89 / 98; 1920 CTAs 39 / 16, 107 / 64, 312 / 218.
-// 1920 CTAs of bf16 hd 96, 250 keys of 6000 / 12000 / 16000 / 24000 allowed for: 106 / 65, 107 / 110, 107 / 134, 107 / 184.
+// Whether a launch reads ahead: up to two waves of that form, two CTAs an SM (registers).  Above, the form with ten CTAs an SM is faster, up to
+// 2.6 times, as long as shared memory (a score for every key that the caller allows for) holds more than three of them.  Called in a row on
+// the same few caches, us, reading ahead / not: fp32 hd 64, 240 CTAs 6.9 / 7.4 with 20 keys, 13.0 / 20.8 with 250, 34 / 67 with 1000; 512 CTAs 11.0 / 7.3,
+// 23.2 / 21.1, 55 / 54 with 800; 640 CTAs 15.0 / 7.3, 31.8 / 21.6, 79 / 56; 960 CTAs 18.8 / 7.9, 39.6 / 23.1, 125 / 72; bf16 hd 96, 1920 CTAs 39 / 16,
+// 107 / 64, 312 / 218.  In a step, whose weights have pushed the cache out of L2, the line lies higher, ms a step with two waves / one: hidden 1024,
+// 512 CTAs .749 / .768 at 40 tokens, .932 / .978 at 400; 576 CTAs .890 / .903, 1.075 / 1.125; three waves / two: 640 CTAs .915 / .896, 1.125 / 1.137;
+// 768 CTAs .941 / .927, 1.174 / 1.161; bf16 hd 32, 768 CTAs .471 / .439.
+// 1920 CTAs of bf16 hd 96, 250 keys of 6000 / 12000 / 16000 / 24000 allowed for: 106 / 65, 107 / 110, 107 / 134, 107 / 184 us.
 bool attn_ref_reads_ahead(int rows, int H, int hd, int max_keys) {
   const size_t smem = ((size_t)max_keys + hd) * sizeof(float);
   if (smem + ArShape<true>::STATIC_SMEM > 227 * 1024) return false;      // the last dozen keys that an SM can hold are for the smaller one
-  return (long long)rows * H <= 148 * ArShape<true>::PER_SM || 228 * 1024 / (smem + ArShape<false>::STATIC_SMEM + 1024) <= 3;
+  return (long long)rows * H <= 2 * 148 * ArShape<true>::PER_SM || 228 * 1024 / (smem + ArShape<false>::STATIC_SMEM + 1024) <= 3;
 }
 
 template <typename T, bool VEC, bool AHEAD>

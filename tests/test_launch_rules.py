@@ -71,12 +71,12 @@ def test_key_splits_of_a_launch_and_of_a_step_that_grows(ask, rows, rps, ctx, ta
 
 
 @pytest.mark.parametrize("rows,H,hd,keys,ahead", [
-    (1, 4, 64, 100, 1), (74, 4, 64, 100, 1), (75, 4, 64, 100, 0), (240, 4, 64, 600, 0), (60, 32, 96, 2000, 0),
+    (1, 4, 64, 100, 1), (148, 4, 64, 100, 1), (149, 4, 64, 100, 0), (240, 4, 64, 600, 0), (60, 32, 96, 2000, 0),
     (60, 32, 96, 14000, 0), (60, 32, 96, 14700, 1),                 # four or three CTAs of the small form in an SM's 228 KB
     (1, 1, 64, 58028, 1), (1, 1, 64, 58033, 0),                     # 227 KB
     (262144, 64, 128, 100, 0),
 ])
-def test_plain_attention_reads_ahead_in_one_wave(ask, rows, H, hd, keys, ahead):
+def test_plain_attention_reads_ahead_in_two_waves(ask, rows, H, hd, keys, ahead):
     assert ask("ahead", rows, H, hd, keys) == ahead
 
 
