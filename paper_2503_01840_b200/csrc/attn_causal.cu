@@ -25,11 +25,13 @@
 // an issuer each 0.536.  A 64-key step of both tiles takes 1470 cycles: shared memory delivers the operands of its MMAs and takes
 // in the next tiles in 1250 (a 128 x 64 x 16 MMA reads 6 KB and takes 48 cycles, 32 with A in tensor memory), the exponentials
 // take 1024, and the two softmax warps of a scheduler, which run in step, leave the special-function unit idle for the rest of
-// theirs.  That rest was 580 cycles and is 450: one vote and one branch decide whether a reference moves, the next scores are
-// asked for before this step's P is known to be written, additions and multiply-adds go two at a time.
+// theirs.  That rest was 580 cycles and is 450: one vote and one branch decide whether a reference moves, additions and multiply-adds
+// go two at a time.
 // Not better (same call, ms): the two warps' exponentials by turns 0.488 to 0.498; the next step's scores loaded, and their
 // maximum taken, under this step's exponentials 0.59 to 0.62 (they come too late for it); an eighth to a third of the
-// exponentials by a polynomial on the multiply-add pipe 0.493 to 0.514; half of Q in tensor memory with one score buffer 0.575.
+// exponentials by a polynomial on the multiply-add pipe 0.493 to 0.514; half of Q in tensor memory with one score buffer 0.575; the next
+// step's scores asked for before this step's P is known to be written 0.494 too, and 3 to 5 % slower where softmax alone is the bound (500
+// positions of 16 heads 18.7 against 17.9 us, 2500 of 16 / 4 heads 44.3 against 43.1): two loads into the same registers want copies.
 //
 // Every wait is bounded.  On a time-out the CTA winds down; a prefill's status words record it, and training-time test, which
 // has none, gets NaN in the rows (and normalisers) it could not finish.
@@ -51,7 +53,6 @@ namespace {
 using tc::elect_one;
 using tc::mbar_expect_tx;
 using tc::mbar_init;
-using tc::mbar_test_warp;
 using tc::mbar_wait;
 using tc::mbar_wait_warp;
 using tc::smem_u32;
@@ -153,8 +154,7 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float *f) {     // no 
         "=r"(v[30]), "=r"(v[31])
       : "r"(taddr));
 }
-// values that a tmem_ld32 put out, from here on: no arithmetic on them moves to before the wait for them.  Copies may: so the paths
-// of two such loads into the same values meet only behind their waits (the compiler makes their registers the same where they meet).
+// values that a tmem_ld32 put out, from here on: behind the wait for them, nothing that uses them moves to before it
 __device__ __forceinline__ void pin32(float *f) {
   asm volatile("" : "+f"(f[0]), "+f"(f[1]), "+f"(f[2]), "+f"(f[3]), "+f"(f[4]), "+f"(f[5]), "+f"(f[6]), "+f"(f[7]), "+f"(f[8]), "+f"(f[9]), "+f"(f[10]), "+f"(f[11]),
                     "+f"(f[12]), "+f"(f[13]), "+f"(f[14]), "+f"(f[15]));
@@ -370,29 +370,20 @@ __global__ void __launch_bounds__(CA_THREADS, 1) attn_causal_kernel(const __grid
     const float sc = rsqrtf((float)CA_HD) * 1.4426950408889634f;                     // softmax scale folded into exp2
     float mx = -INFINITY, l = 0.0f, lrnd = 0.0f;                  // sums of the probabilities and (BRIEF) of the rounded ones
     bool alive = true;
-    // The scores of step i into s, once they are complete
-    float s[CA_KS];
-    auto ask = [&](int i) {
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      tmem_ld32(my_s + (uint32_t)((i & 1) * CA_KS), s);
-      tmem_ld32(my_s + (uint32_t)((i & 1) * CA_KS + 32), s + 32);
-    };
-    auto got = [&]() {                                           // in the same straight line as ask()
-      tmem_ld_wait();
-      pin32(s);
-      pin32(s + 32);
-    };
     auto gave_up = [&](int site, int i) {
       if (lane == 0) { *abort_flag = 1; if (p.status) set_status(p.status, ST_TIMEOUT, site, blockIdx.y, i); }
       alive = false;
     };
-    auto await = [&](int i) {
-      if (mbar_wait_warp(&s_bar[t * 2 + (i & 1)], (uint32_t)((i >> 1) & 1), p.spin)) { ask(i); got(); }
-      else gave_up(435, i);
-    };
     float nb_ = 0.0f;                                            // the reference maximum in the exponent (0 while there is none)
-    if (nt > 0) await(0);
-    for (int i = 0; i < nt && alive; i++) {
+    for (int i = 0; i < nt; i++) {
+      if (!mbar_wait_warp(&s_bar[t * 2 + (i & 1)], (uint32_t)((i >> 1) & 1), p.spin)) { gave_up(435, i); break; }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      float s[CA_KS];
+      tmem_ld32(my_s + (uint32_t)((i & 1) * CA_KS), s);
+      tmem_ld32(my_s + (uint32_t)((i & 1) * CA_KS + 32), s + 32);
+      tmem_ld_wait();
+      pin32(s);
+      pin32(s + 32);
       const int k0 = i * CA_KS;
       if (k0 + CA_KS - 1 > pos - lane) {                         // uniform over the warp: its first row does not see the whole step
         const int lim = pos - k0;                                // keys 0..lim of the step
@@ -443,29 +434,18 @@ __global__ void __launch_bounds__(CA_THREADS, 1) attn_causal_kernel(const __grid
         pk[e] = pack2(pr.x, pr.y);
       }
       tmem_st32(my_s + (uint32_t)((i & 1) * CA_KS), pk);
-      const bool ready = i + 1 < nt && mbar_test_warp(&s_bar[t * 2 + ((i + 1) & 1)], (uint32_t)(((i + 1) >> 1) & 1));
-      auto hand_over = [&]() {                                   // the sums, and P to the MMA warp once it is written
-        l += (rs[0].x + rs[0].y) + (rs[1].x + rs[1].y);
-        if (BRIEF) {
+      l += (rs[0].x + rs[0].y) + (rs[1].x + rs[1].y);
+      if (BRIEF) {
 #pragma unroll
-          for (int z = 0; z < 2; z++) rs[z] = make_float2(0.f, 0.f);
+        for (int z = 0; z < 2; z++) rs[z] = make_float2(0.f, 0.f);
 #pragma unroll
-          for (int e = 0; e < 32; e++) rs[e & 1] = add2(rs[e & 1], bf2(pk[e]));
-          lrnd += (rs[0].x + rs[0].y) + (rs[1].x + rs[1].y);
-        }
-        tmem_st_wait();
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&p_bar[t * 2 + (i & 1)]);
-      };
-      if (ready) {                                               // mostly: the loads run beside the wait for the stores of P
-        ask(i + 1);
-        hand_over();
-        got();
-      } else {
-        hand_over();
-        if (i + 1 < nt) await(i + 1);
+        for (int e = 0; e < 32; e++) rs[e & 1] = add2(rs[e & 1], bf2(pk[e]));
+        lrnd += (rs[0].x + rs[0].y) + (rs[1].x + rs[1].y);
       }
+      tmem_st_wait();
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&p_bar[t * 2 + (i & 1)]);
     }
     if (alive && nt > 0) {
       // All P V of the tile.  A barrier of its own: the scores of the last step only tell that the P V two steps earlier is
