@@ -155,12 +155,14 @@ int spec_profile_step(spec_ctx *ctx, float *class_ms, int32_t *class_launches);
  *   SPEC_TUNE_GEMM_CTAS   CTAs a weight-streaming GEMM launch aims at (process-wide) */
 enum spec_tune_knob { SPEC_TUNE_GEMM_CTAS = 2,
                       SPEC_TUNE_DEBUG_LAUNCH_BUDGET = 3 /* debugging: run only the first n kernels of each step (-1: all) */,
-                      SPEC_TUNE_ATTN_CTAS = 4 /* CTAs an attention launch aims at when splitting keys (process-wide) */,
+                      SPEC_TUNE_ATTN_CTAS = 4 /* CTAs an attention launch aims at when splitting keys (process-wide); the key-parallel kernel (at most
+                                                  16 query rows per KV head) aims at twice the number where a CTA keeps two key tiles */,
                       SPEC_TUNE_DEBUG_WAIT_RUNS_OUT = 5 /* test hook for the bounded device waits: with a value n > 0 one CTA of the verify
                                                   pass's LM-head GEMM never receives its first activation tile and gives up after n
                                                   polls; the step then returns SPEC_ERR_DEVICE_STATUS (0 = off) */,
                       SPEC_TUNE_GEMM_PAIRS = 7 /* 256-row GEMM tiles of neighbouring feature tiles as CTA pairs (tcgen05 cta_group::2): bit 0 = the split-K
-                                                  kernel (default off: measured no faster), bit 1 = the gate/up kernel (default on); process-wide;
+                                                  kernel (default off: measured no faster), bit 1 = the gate/up kernel that spec_gemm_swiglu runs
+                                                  above 128 rows (default on); process-wide;
                                                   the one knob that may be set with a NULL ctx */,
                       SPEC_TUNE_ATTN_UMMA = 6 /* tree passes (head_dim 128): 1 = tcgen05 attention kernel, 0 = mma.sync kernel, 2 (default) = tcgen05
                                                   when every CTA gets several key tiles, i.e. long contexts (process-wide) */ };
@@ -251,8 +253,8 @@ int spec_gemm_topk(const void *x, const void *w, int32_t rows, int32_t out, int3
                    float *out_lp, void *scratch, void *stream);
 
 /* Gate/up half of the decoder layer's MLP (the draft layer and every target layer are LLaMA-style decoder layers,
- * Section 3.1), on the kernels that passes of up to 128 rows use, or (more rows) with a gate and an up tile per block:
- * act[r][f] = bf16(silu(g) * u), g = sum_i x[r][i] * w_gate[f][i], u likewise with w_up, both accumulated in fp32 (a CTA
+ * Section 3.1), on the kernels that passes of up to 128 rows use, or (more rows, where the passes take the kernels of
+ * spec_gemm_wide) with a gate and an up tile per block: act[r][f] = bf16(silu(g) * u), g = sum_i x[r][i] * w_gate[f][i], u likewise with w_up, both accumulated in fp32 (a CTA
  * holds the gate and the up features of the same range).  x [rows][in] bf16, w_gate / w_up [F][in] bf16, act [rows][F] bf16,
  * all device pointers, 16-byte aligned; rows <= 256, in % 8 == 0.  Returns SPEC_OK or a negative code; nothing is allocated. */
 int spec_gemm_swiglu(const void *x, const void *w_gate, const void *w_up, void *act, int32_t rows, int32_t F, int32_t in,

@@ -492,11 +492,16 @@ template <typename T> struct Sched {
   }
   // From 129 rows on (up to 256: batches, and whole trees at a small batch) a weight byte meets more flops than the
   // weight-streaming kernel's tiles feed the tensor pipe with: it re-reads the 32 KB activation k-block for every 128
-  // features and spends as long in its 256-row epilogues as in its loops.  These passes take the row-major kernel.  Alone (8B
-  // shapes, launches from a graph without the passes' epilogues, weight-streaming / row-major, us): QKV 23.4 / 19.2 at 144 rows, 30.9 / 20.0
-  // at 256; O 16.2 / 17.5, 19.5 / 18.5; down 30.8 / 32.6, 34.9 / 34.3.  Gate/up in the replayed step (weight-streaming pair kernel /
-  // row-major, us): 8B shapes 132 rows 47.6 / 48.8, 160 49.6 / 49.3, 192 50.9 / 49.2, 208 54.7 / 49.5, 240 54.6 / 49.4, 256 58.3 / 49.1; 13B shapes
-  // 150 rows 56.3 / 54.2, 250 67.0 / 55.1; 70B shapes 180 rows 192 / 184, 240 220 / 187.
+  // features and spends as long in its 256-row epilogues as in its loops.  These passes take the row-major kernel.  Replayed step, us a
+  // launch of a verify layer, weight-streaming / row-major kernel:
+  //   rows  QKV          O            gate/up (pair)  down         layer           rows  QKV          O            gate/up      down         layer
+  //   8B shapes                                                                    13B shapes
+  //   132   33.7 / 17.2  13.4 / 15.4  47.7 / 47.3     29.2 / 30.4  141.1 / 127.1   132   42.4 / 37.2  18.1 / 17.7  54.5 / 53.6  34.8 / 32.0  163.5 / 155.0
+  //   160   34.4 / 17.2  14.0 / 16.4  49.0 / 47.5     29.7 / 31.0  145.8 / 129.7   192   46.0 / 37.7  19.4 / 17.2  57.6 / 54.3  36.8 / 32.7  185.6 / 166.2
+  //   192   36.1 / 17.9  14.8 / 16.2  50.7 / 47.9     30.9 / 31.4  152.0 / 132.5   250   51.4 / 38.4  22.7 / 20.1  67.4 / 54.2  40.1 / 35.0  208.0 / 174.3
+  //   240   38.5 / 19.2  16.4 / 18.0  54.2 / 48.3     32.4 / 33.0  161.7 / 138.2   70B shapes
+  //   256   39.6 / 19.3  16.8 / 18.0  55.8 / 48.6     32.8 / 33.5  164.9 / 139.3   180   65.3 / 50.3  38.8 / 32.8  185 / 176    106.0 / 92.3  416 / 374
+  // (O and down of the 8B shapes alone would be 1 to 2 us shorter on the weight-streaming kernel.)
   bool row_major(FusedEpi epi, const FusedGemmArgs &a) const {
     return a.rows > 128 && !a.withhold && !fused_gemm_pairs() && epi != EPI_TOPK && (epi != EPI_QKV || a.hd == 128);
   }

@@ -897,8 +897,9 @@ __global__ void __launch_bounds__(UM_THREADS, 1) attn_umma_kernel(const __grid_c
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       float s[KT];
       tmem_ld64(tmem_s + lane_base + (uint32_t)((i % UM_S) * KT), s);
-      // Padding rows (beyond the tile's last row, or of a skipped sequence) run the loop like real rows and are
-      // zeroed at the end: their Q is zero, and a row that always took the masked path would slow its whole warp.
+      // Padding rows run the loop like real rows and are dropped at the store: a row that always took the masked path would slow
+      // its whole warp.  Those beyond the tile's last row have a Q of zero, those of a skipped sequence any Q at all (NaN and infinities too):
+      // nothing that a row computes may reach another row.
       float t4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};      // four chains instead of one of 64 steps
       if (t * KT + KT <= ctx) {
 #pragma unroll
@@ -1443,7 +1444,9 @@ int g_attn_umma = 2;            // tcgen05 kernel for the tree passes: 0 off, 1 
 // The mma.sync kernel takes 2 us a tile whatever the rows, the tcgen05 kernel has two tiles in work at once but starts and ends later.
 // Replayed step, attention and merge, mma.sync / tcgen05 (us): 240 query rows per KV head (8B verify pass), one tile a CTA 10.9 / 11.5 at
 // 400 tokens, 12.1 / 10.9 at 250; two tiles 13.8 / 10.5 at 512, 14.9 / 12.0 at 1000.  40 rows (draft pass): one tile 7.4 / 9.3, two
-// 9.8 / 10.1 at 1500 tokens; three 14.6 / 13.6.
+// 9.8 / 10.1 at 1500 tokens; three 14.6 / 13.6.  Between, two tiles: 68 rows 10.5 / 10.4 at 1300 tokens, 12.8 / 11.8 at 2000 and 12.1 / 10.1 of four
+// sequences at 450; 80 rows 10.8 / 10.5 and 13.0 / 12.1; 104 rows 11.9 / 10.8; 128 rows 12.9 / 11.3; 160 rows 11.9 / 10.3 at 600 and 13.1 / 11.8 at
+// 1000; 70B shapes, 80 rows 11.1 / 10.9, 160 rows 12.5 / 10.2.
 int um_min_tiles(int query_rows) { return query_rows > 64 ? 2 : 3; }
 thread_local int tl_attn_umma = -1;   // per-call override (-1: none)
 

@@ -30,7 +30,8 @@ bool attn_takes_tma(int page_size, int head_dim, bool contiguous_tail);
 int attn_fast_plan(int rows, int H, int G, int hd, int rps, int ctx_hint, int tail_len, bool grows, bool tma = true);
 // Drops the cached K/V tensor maps (pools of one-shot callers come and go).
 void attn_fast_forget_maps();
-// CTAs an attention launch aims at when it splits the keys (process-wide; default 148 = one wave)
+// CTAs an attention launch aims at when it splits the keys (process-wide; default 148 = one an SM; the key-parallel kernel, at most 16 query rows
+// per KV head, aims at twice the number, as long as a CTA keeps two key tiles)
 void attn_fast_set_target_ctas(int n);
 // tcgen05 kernel for passes with more than 16 query rows per (sequence, KV head) and head_dim 128 (process-wide):
 // 0 never, 1 always, 2 (default) when every CTA gets several key tiles; and a per-thread override for single calls (-1: none)

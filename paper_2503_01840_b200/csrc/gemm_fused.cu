@@ -795,6 +795,8 @@ __global__ void __launch_bounds__(fused_threads(NT, EPI), EPI == EPI_TOPK || EPI
 // k-block 48 KB instead of 64 KB per CTA, four stages instead of three).
 // PAIR_THREADS threads: several threads share a feature (tensor-memory lane) and split the rows in the epilogue, which
 // converts 2 x 256 accumulator columns per feature (with 128 threads it took a quarter of the launch).
+// It serves spec_gemm_swiglu, and passes under the pair switch of the split-K kernel: the passes' own gate/up above 128 rows is the
+// row-major kernel's (gemm_wide.cu), which is ahead at every row count (the table is beside row_major in api.cu).
 constexpr int PAIR_THREADS = 512, PAIR_GROUPS = PAIR_THREADS / 128;
 template <int NT, bool DUO = false>
 __global__ void __launch_bounds__(PAIR_THREADS) gemm_swiglu_pair_kernel(const __grid_constant__ FusedParams p) {

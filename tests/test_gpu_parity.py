@@ -623,7 +623,7 @@ def test_gemm_cta_pairs_bit_equal(rows, O, I, split):
 
 @pytest.mark.parametrize("rows,F,I", [(256, 512, 512), (200, 1024, 4096), (129, 1792, 1024), (256, 384, 1024)])
 def test_gate_up_cta_pairs_bit_equal(rows, F, I):
-    """The 256-row gate/up kernel (passes of 129 to 192 rows) as CTA pairs (the default) against single CTAs: bit-identical activations, and both
+    """The gate/up kernel that spec_gemm_swiglu runs above 128 rows (the passes take the row-major one) as CTA pairs (the default) against single CTAs: bit-identical activations, and both
     within bf16 rounding of SiLU(x Wg^T) * (x Wu^T) computed in float64."""
     g = torch.Generator().manual_seed(rows + F + I)
     x = torch.randn(rows, I, generator=g).to(torch.bfloat16).cuda()

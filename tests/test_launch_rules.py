@@ -17,6 +17,7 @@ using namespace spec;
 int main(int n, char **v) {                     // epilogue, rows, split, stages; or rows, rows per sequence, context, tail, grows (32 heads, 8 KV heads)
   if (v[1][0] == 'a') { printf("%d", attn_ref_reads_ahead(atoi(v[2]), atoi(v[3]), atoi(v[4]), atoi(v[5])) ? 1 : 0); return 0; }      // "ahead", rows, heads, head size, keys
   if (v[1][0] == 'v') { printf("%d", accept_sampled_takes(atoi(v[2])) ? accept_mass_chunks(atoi(v[2])) : -accept_mass_chunks(atoi(v[2]))); return 0; }      // "vocabulary", ids
+  if (n == 7) { printf("%d", attn_fast_plan(atoi(v[1]), 32, 8, 128, atoi(v[2]), atoi(v[3]), atoi(v[4]), atoi(v[5]) != 0, atoi(v[6]) != 0) >> 1); return 0; }      // ... and TMA
   if (n == 6) { printf("%d", attn_fast_plan(atoi(v[1]), 32, 8, 128, atoi(v[2]), atoi(v[3]), atoi(v[4]), atoi(v[5]) != 0) >> 1); return 0; }
   static char mem[64];
   FusedGemmArgs a;
@@ -84,3 +85,23 @@ def test_plain_attention_reads_ahead_in_two_waves(ask, rows, H, hd, keys, ahead)
 def test_vocabularies_of_the_stochastic_acceptance(ask, vocab, chunks):
     """Runs of 8192 ids; one CTA's shared memory holds the masses of 8192 runs, and a larger vocabulary is refused."""
     assert ask("vocabulary", vocab) == chunks
+
+
+@pytest.mark.parametrize("seqs,ctx,grows,one_cta,two_ctas", [
+    (1, 700, 0, 11, 11), (2, 700, 0, 6, 6),                          # 11 tiles: one wave of one CTA an SM already gives most of them a tile each
+    (2, 2000, 0, 8, 16), (4, 700, 0, 4, 4),                          # 32 tiles, two each; 11 tiles in 4 or in 5 splits are three each
+    (6, 700, 0, 3, 4), (6, 2000, 0, 3, 6), (6, 60, 0, 1, 1),         # no split for less than two tiles
+    (12, 700, 0, 1, 3), (12, 700, 1, 1, 3), (18, 700, 0, 1, 2), (18, 120, 1, 1, 1),
+    (36, 700, 0, 1, 1), (37, 700, 0, 1, 1), (64, 2000, 1, 1, 1),
+])
+def test_key_splits_of_chains(ask, seqs, ctx, grows, one_cta, two_ctas):
+    """Up to 16 query rows per KV head (four rows, four heads a group): the key-parallel kernel, two of whose CTAs an SM holds, is split for 296
+    CTAs as long as each keeps two tiles; without TMA another kernel takes the launch, one CTA an SM."""
+    assert ask(4 * seqs, 4, ctx, 4, grows, 0) == one_cta
+    assert ask(4 * seqs, 4, ctx, 4, grows, 1) == ask(4 * seqs, 4, ctx, 4, grows) == two_ctas
+
+
+@pytest.mark.parametrize("seqs,ctx", [(2, 700), (6, 2000), (18, 700)])
+def test_key_splits_of_trees_do_not_depend_on_tma(ask, seqs, ctx):
+    """More than 16 query rows: one CTA an SM either way."""
+    assert ask(20 * seqs, 20, ctx, 20, 0, 0) == ask(20 * seqs, 20, ctx, 20, 0, 1)
